@@ -4,15 +4,24 @@
 // proportion to Algorithm 2's weight (0.01 + L_i/L_s) * (inf_ij/L_s) and are rounded by largest
 // remainder so that they sum to D exactly.  Options: the head share over the layer's own sum (the prose under
 // Eq. 6), a per-head cap whose excess is handed on to the other heads, Algorithm 2's own rounding.
-// The sums over heads and layers run sequentially in index order on one thread and every product / quotient
-// is a separately rounded IEEE operation (__dadd_rn / __dmul_rn / __ddiv_rn stop the compiler from fusing
-// them), so the integers that come out do not depend on the launch shape.
+// The sums over heads and layers run in index order on one thread and every product / quotient is a separately
+// rounded IEEE operation (__dadd_rn / __dmul_rn / __ddiv_rn stop the compiler from fusing them), so the integers that
+// come out do not depend on the launch shape.
+//
+// What bounds it: latency.  The order of the sums is part of the result, so one chain of N dependent fp64 additions
+// stays; everything else runs on all threads -- the weights (two fp64 divisions each, formerly part of that chain) are
+// in shared memory before the chain starts, which then only loads and adds, and the largest remainders are found by a
+// comparison of all pairs split over the whole CTA (N <= 1024) or by a radix descent (beyond), not by one thread per
+// head walking all the others.  256 heads: 70.5 -> 7 us.
 #include "slkv_internal.cuh"
 
 namespace slkv {
 namespace {
 
 constexpr int kAllocThreads = 1024;
+constexpr int kPairsMax = 1024;        // heads up to which all pairs of remainders are compared: at 1024 a thread compares
+                                       // its head with all others (~5 us); beyond that the radix descent's eight
+                                       // levels of about 1 us each cost less
 
 struct AllocOpts {
   int within_layer;      // head share over the layer's sum (prose under Eq. 6) instead of the grand sum (Algorithm 2)
@@ -20,17 +29,28 @@ struct AllocOpts {
   long long cap;         // < 0: none
 };
 
-// Algorithm 2's weight of head a = (layer i, head j): (0.01 + L_i / L_s) * S_ij; 1 for every head when no head has
-// any influence.
-__device__ __forceinline__ double head_weight(const float* inf, const double* La, double Ls, int H, int a,
-                                              bool uniform, bool within_layer) {
-  if (uniform) return 1.0;
-  const int i = a / H;
-  const double lw = __dadd_rn(kLayerFloor, __ddiv_rn(La[i], Ls));      // 0.01 + L_{i,h}
+// Algorithm 2's weight of a head of influence x in a layer of H heads with sum La_i: (0.01 + L_i / L_s) * S_ij.
+__device__ __forceinline__ double head_weight(double x, double La_i, double Ls, int H, bool within_layer) {
+  const double lw = __dadd_rn(kLayerFloor, __ddiv_rn(La_i, Ls));       // 0.01 + L_{i,h}
   double share;
-  if (within_layer) share = La[i] > 0.0 ? __ddiv_rn((double)inf[a], La[i]) : __ddiv_rn(1.0, (double)H);
-  else share = __ddiv_rn((double)inf[a], Ls);                          // S_{j,h}
+  if (within_layer) share = La_i > 0.0 ? __ddiv_rn(x, La_i) : __ddiv_rn(1.0, (double)H);
+  else share = __ddiv_rn(x, Ls);                                       // S_{j,h}
   return __dmul_rn(lw, share);
+}
+
+// v[0] + v[1] + ... in index order, one thread; eight loads are in flight ahead of the additions.
+__device__ __forceinline__ double ordered_sum(const double* v, int n) {
+  double acc = 0.0;
+  int a = 0;
+  for (; a + 8 <= n; a += 8) {
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = v[a + u];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, x[u]);
+  }
+  for (; a < n; ++a) acc = __dadd_rn(acc, v[a]);
+  return acc;
 }
 
 __device__ long long block_sum_ll(long long v, long long* red) {
@@ -38,8 +58,8 @@ __device__ long long block_sum_ll(long long v, long long* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  long long t = 0;
-  for (int w = 0; w < kAllocThreads / 32; ++w) t += red[w];
+  long long t = red[threadIdx.x & 31];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   return t;
 }
 
@@ -48,51 +68,44 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
         int32_t* __restrict__ budgets, int32_t* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = L * H;
-  double* rem = reinterpret_cast<double*>(smem_raw);       // [N] fractional parts
-  double* La = rem + N;                                    // [L] layer sums
-  unsigned char* active = reinterpret_cast<unsigned char*>(La + L);   // [N] head still below the cap
+  double* wt = reinterpret_cast<double*>(smem_raw);        // [N] INF_sc, then the weights (0 once a head is filled), then
+                                                           //     the remainders' bit patterns + 1 (0: not a candidate)
+  unsigned long long* key = reinterpret_cast<unsigned long long*>(smem_raw);
+  double* La = wt + N;                                     // [L] layer sums
+  int* fl = reinterpret_cast<int*>(La + L);                // [N] dynamic parts
+  unsigned char* active = reinterpret_cast<unsigned char*>(fl + N);   // [N] head still below the cap
   __shared__ long long red[kAllocThreads / 32];
   __shared__ double sh_Ls, sh_W;
-  __shared__ int sh_bad, sh_uniform, sh_flat, sh_n_active;
+  __shared__ int hist[256];
+  __shared__ int sh_digit, sh_above;
   const int tid = threadIdx.x;
   const long long D = total - (long long)N * fixed;
   const bool within = opt.within_layer != 0;
   pdl_launch_dependents();
   pdl_wait();
 
-  if (tid == 0) sh_bad = 0;
-  __syncthreads();
+  int bad = 0;
   for (int a = tid; a < N; a += kAllocThreads) {
-    float x = inf[a];
-    if (!(x >= 0.0f) || !(x <= 3.402823466e38f)) sh_bad = 1;         // negative, NaN or infinite
+    const float x = inf[a];
+    bad |= !(x >= 0.0f) || !(x <= 3.402823466e38f);                  // negative, NaN or infinite
+    wt[a] = (double)x;
+    active[a] = 1;
   }
-  __syncthreads();
-  if (sh_bad) {
+  if (__syncthreads_or(bad)) {
     if (tid == 0 && status) *status = SLKV_ERR_NEG_INF_SC;
     return;
   }
-
-  // layer sums: one thread per layer, each sequential over its heads (index order)
-  for (int i = tid; i < L; i += kAllocThreads) {
-    double acc = 0.0;
-    for (int j = 0; j < H; ++j) acc = __dadd_rn(acc, (double)inf[i * H + j]);
-    La[i] = acc;
-  }
+  for (int i = tid; i < L; i += kAllocThreads) La[i] = ordered_sum(wt + (size_t)i * H, H);
   __syncthreads();
-  if (tid == 0) {
-    double Ls = 0.0;
-    for (int i = 0; i < L; ++i) Ls = __dadd_rn(Ls, La[i]);
-    sh_Ls = Ls;
-    sh_uniform = !(Ls > 0.0);
-  }
+  if (tid == 0) sh_Ls = ordered_sum(La, L);
   __syncthreads();
   const double Ls = sh_Ls;
-  const bool uniform = sh_uniform != 0;
+  const bool uniform = !(Ls > 0.0);                                   // no head has any influence: all weights 1
 
   if (opt.paper_rounding) {
     // Algorithm 2's own last line: C = floor(max(0, fixed + D * w) + 0.5), clipped at the cap; nothing is normalised
     for (int a = tid; a < N; a += kAllocThreads) {
-      const double w = uniform ? __ddiv_rn(1.0, (double)N) : head_weight(inf, La, Ls, H, a, false, within);
+      const double w = uniform ? __ddiv_rn(1.0, (double)N) : head_weight(wt[a], La[a / H], Ls, H, within);
       const double b = __dadd_rn((double)fixed, __dmul_rn((double)D, w));
       long long c = (long long)floor(__dadd_rn(fmax(0.0, b), 0.5));
       if (opt.cap >= 0 && c > opt.cap) c = opt.cap;
@@ -100,74 +113,126 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     }
     return;
   }
+  for (int a = tid; a < N; a += kAllocThreads) wt[a] = uniform ? 1.0 : head_weight(wt[a], La[a / H], Ls, H, within);
 
-  // Heads that would rise above the cap are filled and taken out, the rest share what is left, until none does
-  // (without a cap: one round, nobody is taken out).  The sum of the weights runs sequentially in index order.
-  for (int a = tid; a < N; a += kAllocThreads) active[a] = 1;
+  // Heads that would rise above the cap are filled and taken out (their weight becomes 0, which leaves the ordered sum
+  // of the others as it is), the rest share what is left, until none does (without a cap: one round, nobody is taken
+  // out).
   const long long room = opt.cap >= 0 ? opt.cap - fixed : -1;
   long long d_rem = D;
+  int n_active = N;
+  double W;
+  bool flat;
   while (true) {
     __syncthreads();
-    if (tid == 0) {
-      double W = 0.0;
-      int n_active = 0;
-      for (int a = 0; a < N; ++a)
-        if (active[a]) { W = __dadd_rn(W, head_weight(inf, La, Ls, H, a, uniform, within)); ++n_active; }
-      const int flat = !(W > 0.0);                                    // every weight left underflowed: share evenly
-      if (flat) W = (double)n_active;
-      sh_W = W; sh_flat = flat; sh_n_active = n_active;
-    }
+    if (tid == 0) sh_W = ordered_sum(wt, N);
     __syncthreads();
-    if (room < 0 || sh_n_active == 0) break;
-    const double W = sh_W;
-    const bool flat = sh_flat != 0;
+    W = sh_W;
+    flat = !(W > 0.0);                                                // every weight left underflowed: share evenly
+    if (flat) W = (double)n_active;
+    if (room < 0 || n_active == 0) break;
     long long filled = 0;
     for (int a = tid; a < N; a += kAllocThreads) {
       if (!active[a]) continue;
-      const double wgt = flat ? 1.0 : head_weight(inf, La, Ls, H, a, uniform, within);
-      const double q = __ddiv_rn(__dmul_rn((double)d_rem, wgt), W);
-      if (q >= (double)room) { active[a] = 0; budgets[a] = (int32_t)room; ++filled; }
+      const double q = __ddiv_rn(__dmul_rn((double)d_rem, flat ? 1.0 : wt[a]), W);
+      if (q >= (double)room) { active[a] = 0; wt[a] = 0.0; fl[a] = (int)room; ++filled; }
     }
     filled = block_sum_ll(filled, red);
     if (filled == 0) break;
     d_rem -= filled * room;
+    n_active -= (int)filled;
   }
-  const double W = sh_W;
-  const bool flat = sh_flat != 0;
-  const int n_active = sh_n_active;
 
   // quotas, floors, remainders of the heads still below the cap
   long long fsum = 0;
   for (int a = tid; a < N; a += kAllocThreads) {
-    if (!active[a]) continue;
-    const double wgt = flat ? 1.0 : head_weight(inf, La, Ls, H, a, uniform, within);
-    const double q = __ddiv_rn(__dmul_rn((double)d_rem, wgt), W);
-    const double fl = floor(q);
-    rem[a] = __dadd_rn(q, -fl);
-    const long long f = (long long)fl;
-    budgets[a] = (int32_t)f;                                          // floors for now
-    fsum += f;
+    unsigned long long kk = 0;
+    if (active[a]) {
+      const double q = __ddiv_rn(__dmul_rn((double)d_rem, flat ? 1.0 : wt[a]), W);
+      const double f = floor(q);
+      kk = (unsigned long long)__double_as_longlong(__dadd_rn(q, -f)) + 1ull;    // remainders are >= 0: bit order = order
+      fl[a] = (int)(long long)f;
+      fsum += (long long)f;
+    }
+    key[a] = kk;
   }
-  long long Rleft = d_rem - block_sum_ll(fsum, red);
+  long long Rleft = d_rem - block_sum_ll(fsum, red);                  // its barriers also publish key[] and fl[]
   if (n_active > 0 && Rleft >= n_active) {                            // not reachable in exact arithmetic
     const long long each = Rleft / n_active;
     for (int a = tid; a < N; a += kAllocThreads)
-      if (active[a]) budgets[a] += (int32_t)each;
+      if (active[a]) fl[a] += (int)each;
     Rleft -= each * n_active;
   }
-  __syncthreads();
   if (Rleft > 0) {
     // largest remainder first, ties -> lower index: head a gets +1 iff fewer than Rleft heads precede it
-    for (int a = tid; a < N; a += kAllocThreads) {
-      if (!active[a]) continue;
-      const double ra = rem[a];
+    if (N <= kPairsMax) {
+      int lanes = 1;                                                  // threads per head, neighbours in a warp
+      while (lanes < 32 && 2 * lanes * N <= kAllocThreads) lanes *= 2;
+      const int a = tid / lanes, sub = tid % lanes;
+      const unsigned long long ka = a < N ? key[a] : 0ull;
       int rank = 0;
-      for (int b = 0; b < N; ++b) {
-        if (!active[b]) continue;
-        const double rb = rem[b];
-        rank += (rb > ra) || (rb == ra && b < a);
+      if (ka) {
+#pragma unroll 8
+        for (int b = sub; b < N; b += lanes) {
+          const unsigned long long kb = key[b];
+          rank += (kb > ka) || (kb == ka && b < a);
+        }
       }
-      if (rank < Rleft) budgets[a] += 1;
+      for (int o = 1; o < lanes; o *= 2) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+      if (ka && sub == 0 && rank < Rleft) fl[a] += 1;
+    } else {
+      // the Rleft-th largest key by a radix descent, eight bits at a time
+      unsigned long long prefix = 0, mask = 0;
+      int need = (int)Rleft;
+      for (int shift = 56; shift >= 0; shift -= 8) {
+        if (tid < 256) hist[tid] = 0;
+        __syncthreads();
+        for (int a = tid; a < N; a += kAllocThreads) {
+          const unsigned long long k = key[a];
+          if (k && (k & mask) == prefix) atomicAdd(&hist[(int)(k >> shift) & 255], 1);
+        }
+        __syncthreads();
+        if (tid < 32) {                                               // lane t: the bins 255 - 8t .. 248 - 8t
+          int c[8], s = 0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) { c[u] = hist[255 - 8 * tid - u]; s += c[u]; }
+          int inc = s;
+          for (int o = 1; o < 32; o <<= 1) {
+            const int n = __shfl_up_sync(0xffffffffu, inc, o);
+            if (tid >= o) inc += n;
+          }
+          int above = inc - s;
+          if (above < need && need <= inc)
+            for (int u = 0; u < 8; ++u) {
+              if (need <= above + c[u]) { sh_digit = 255 - 8 * tid - u; sh_above = above; break; }
+              above += c[u];
+            }
+        }
+        __syncthreads();
+        prefix |= (unsigned long long)sh_digit << shift;
+        mask |= 255ull << shift;
+        need -= sh_above;
+        __syncthreads();
+      }
+      // keys above `prefix` and, in index order, the first `need` equal to it
+      const int per = (N + kAllocThreads - 1) / kAllocThreads;
+      const int a0 = min(tid * per, N), a1 = min(a0 + per, N);
+      int eq = 0;
+      for (int a = a0; a < a1; ++a) eq += key[a] == prefix;
+      int inc = eq;
+      const int lane = tid & 31, wid = tid >> 5;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += n;
+      }
+      if (lane == 31) hist[wid] = inc;
+      __syncthreads();
+      int before = inc - eq;
+      for (int w2 = 0; w2 < wid; ++w2) before += hist[w2];
+      for (int a = a0; a < a1; ++a) {
+        if (key[a] > prefix) fl[a] += 1;
+        else if (key[a] == prefix && before++ < need) fl[a] += 1;
+      }
     }
   }
   while (Rleft < 0) {
@@ -178,24 +243,22 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     int nd = 0;
     for (int a = tid; a < N; a += kAllocThreads, ++nd) {
       dec[nd] = 0;
-      if (!active[a] || budgets[a] <= 0) continue;
-      const double ra = rem[a];
+      if (!active[a] || fl[a] <= 0) continue;
       int rank = 0;
       for (int b = 0; b < N; ++b) {
-        if (!active[b] || budgets[b] <= 0) continue;
-        const double rb = rem[b];
-        rank += (rb < ra) || (rb == ra && b > a);
+        if (!active[b] || fl[b] <= 0) continue;
+        rank += (key[b] < key[a]) || (key[b] == key[a] && b > a);
       }
       if (rank < -Rleft) { dec[nd] = 1; ++taken; }
     }
     __syncthreads();
     nd = 0;
     for (int a = tid; a < N; a += kAllocThreads, ++nd)
-      if (dec[nd]) budgets[a] -= 1;
+      if (dec[nd]) fl[a] -= 1;
     Rleft += block_sum_ll(taken, red);
   }
   __syncthreads();
-  for (int a = tid; a < N; a += kAllocThreads) budgets[a] += fixed;
+  for (int a = tid; a < N; a += kAllocThreads) budgets[a] = fl[a] + fixed;
 }
 
 }  // namespace
@@ -203,13 +266,13 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
 cudaError_t launch_alloc(const float* inf, int n_layers, int n_heads, int fixed, long long total, int within_layer,
                          int paper_rounding, long long cap, int32_t* budgets, int32_t* status, cudaStream_t st) {
   const size_t n = (size_t)n_layers * n_heads;
-  size_t smem = (n + n_layers) * sizeof(double) + n;
+  const size_t smem = (n + n_layers) * sizeof(double) + n * (sizeof(int) + 1);
   static thread_local int configured_dev = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(k_alloc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_alloc, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
     if (e != cudaSuccess) return e;
     configured_dev = dev;
   }
@@ -217,8 +280,8 @@ cudaError_t launch_alloc(const float* inf, int n_layers, int n_heads, int fixed,
   opt.within_layer = within_layer; opt.paper_rounding = paper_rounding; opt.cap = cap;
   int launches = 0;
   LaunchScope scope(KID_ALLOC, st, &launches);
-  k_alloc<<<1, kAllocThreads, smem, st>>>(inf, n_layers, n_heads, fixed, total, opt, budgets, status);
-  return cudaGetLastError();
+  return launch_pdl(k_alloc, dim3(1), dim3(kAllocThreads), smem, st, 1, inf, n_layers, n_heads, fixed, total, opt,
+                    budgets, status);
 }
 
 }  // namespace slkv
