@@ -1,11 +1,14 @@
-"""ctypes binding of libslkv.so: the same entry points as include/slkv.h, argument marshalling only.
+"""Binding of libslkv.so: the same entry points as include/slkv.h, argument marshalling only.
 
 Tensors are torch tensors (device memory and streams come from torch); every step of the method runs in
 the library's kernels.  There is no fallback: if the shared library is missing, lib() raises.
+Calls that a program makes per layer go through a small C module (csrc/slkv_pycall.c) that converts tensors, lists and
+structures itself: about 1 us a call, against 8 us through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from typing import List, Optional, Sequence, Tuple
 
@@ -131,8 +134,17 @@ def lib() -> C.CDLL:
     return _lib
 
 
-def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
-    return None if t is None else t.data_ptr()
+class _EntryPoints(dict):
+    """Entry point name -> callable(stream, *args); filled on first use."""
+
+    def __missing__(self, name: str):
+        address = C.cast(getattr(lib(), name), C.c_void_p).value
+        from ._slkv_call import call
+        self[name] = fn = functools.partial(call, address)
+        return fn
+
+
+_fn = _EntryPoints()
 
 
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
@@ -143,6 +155,10 @@ def _stream(stream: Optional[torch.cuda.Stream]) -> int:
 def _cu_host(cu_seqlens: Sequence[int]):
     arr = (C.c_int32 * len(cu_seqlens))(*[int(x) for x in cu_seqlens])
     return arr
+
+
+def _cu_list(cu_seqlens: Sequence[int]):
+    return cu_seqlens if type(cu_seqlens) in (list, tuple) else [int(x) for x in cu_seqlens]
 
 
 def make_params(q_win: torch.Tensor, k: torch.Tensor, v: Optional[torch.Tensor], window: int, pool_kernel: int,
@@ -178,14 +194,14 @@ def slkv_alloc_budgets(inf_sc: torch.Tensor, fixed: int, total: int, budgets: Op
     assert inf_sc.is_cuda and inf_sc.dtype == torch.float32 and inf_sc.dim() == 2 and inf_sc.is_contiguous()
     if budgets is None:
         budgets = torch.empty(inf_sc.shape, dtype=torch.int32, device=inf_sc.device)
+    n_layers, n_heads = inf_sc.shape
     if options is not None:
-        rc = lib().slkv_alloc_budgets_ex(inf_sc.data_ptr(), inf_sc.shape[0], inf_sc.shape[1], int(fixed), int(total),
-                                         C.byref(options), budgets.data_ptr(), _ptr(status), _stream(stream))
+        rc = _fn["slkv_alloc_budgets_ex"](stream, inf_sc, n_layers, n_heads, int(fixed), int(total), options, budgets,
+                                          status)
         if rc != SLKV_OK:
             raise SlkvError(rc, "slkv_alloc_budgets_ex")
         return budgets
-    rc = lib().slkv_alloc_budgets(inf_sc.data_ptr(), inf_sc.shape[0], inf_sc.shape[1], int(fixed), int(total),
-                                  budgets.data_ptr(), _ptr(status), _stream(stream))
+    rc = _fn["slkv_alloc_budgets"](stream, inf_sc, n_layers, n_heads, int(fixed), int(total), budgets, status)
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_alloc_budgets")
     return budgets
@@ -196,17 +212,16 @@ def slkv_behavior_scores(attn: torch.Tensor, needle_idx: torch.Tensor, topk_idx:
     [n] (one list for all rows), entries < 0 are padding.  Returns (SF_sc, LG_sc, INF_sc), CUDA float32 [n_rows]."""
     assert attn.is_cuda and attn.dtype == torch.float32 and attn.dim() == 2 and attn.stride(1) == 1
     n_rows, row_len = attn.shape
-    outs = [torch.empty(n_rows, dtype=torch.float32, device=attn.device) for _ in range(3)]
-
-    def lst(t):
+    sf, lg, inf = torch.empty((3, n_rows), dtype=torch.float32, device=attn.device).unbind(0)
+    for t in (needle_idx, topk_idx):
         assert t.is_cuda and t.dtype == torch.int32 and t.is_contiguous() and t.dim() in (1, 2)
-        return t.data_ptr(), t.shape[-1], (t.shape[-1] if t.dim() == 2 else 0)
-    (np_, nn, ns), (tp, tn, ts) = lst(needle_idx), lst(topk_idx)
-    rc = lib().slkv_behavior_scores(attn.data_ptr(), n_rows, row_len, attn.stride(0), np_, nn, ns, tp, tn, ts,
-                                    outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr(), _stream(stream))
+    nn, tn = needle_idx.shape[-1], topk_idx.shape[-1]
+    rc = _fn["slkv_behavior_scores"](stream, attn, n_rows, row_len, attn.stride(0), needle_idx, nn,
+                                     nn if needle_idx.dim() == 2 else 0, topk_idx, tn, tn if topk_idx.dim() == 2 else 0,
+                                     sf, lg, inf)
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_behavior_scores")
-    return tuple(outs)
+    return sf, lg, inf
 
 
 def slkv_workspace_bytes(params: SlkvParams, cu_seqlens: Sequence[int]) -> int:
@@ -228,20 +243,19 @@ def new_workspace(params: SlkvParams, cu_seqlens: Sequence[int], device) -> torc
     return torch.empty(n, dtype=torch.uint8, device=device)
 
 
-def _lse(lse: Optional[torch.Tensor], params: SlkvParams) -> Optional[int]:
+def _lse(lse: Optional[torch.Tensor], params: SlkvParams) -> Optional[torch.Tensor]:
     if lse is None:
         return None
     assert lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
     assert lse.numel() == params.n_seqs * params.n_q_heads * params.window, "lse is [n_seqs, n_q_heads, window]"
-    return lse.data_ptr()
+    return lse
 
 
 def slkv_score(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_dev: torch.Tensor,
                cu_seqlens: Sequence[int], pooled: torch.Tensor, workspace: torch.Tensor,
                status: Optional[torch.Tensor] = None, stream=None, lse: Optional[torch.Tensor] = None) -> torch.Tensor:
-    rc = lib().slkv_score(C.byref(params), q_win.data_ptr(), k.data_ptr(), cu_dev.data_ptr(), _cu_host(cu_seqlens),
-                          _lse(lse, params), pooled.data_ptr(), _ptr(status), workspace.data_ptr(), workspace.numel(),
-                          _stream(stream))
+    rc = _fn["slkv_score"](stream, params, q_win, k, cu_dev, _cu_list(cu_seqlens), _lse(lse, params), pooled, status,
+                           workspace, workspace.numel())
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_score")
     return pooled
@@ -252,8 +266,8 @@ def slkv_row_lse(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_de
                  status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """lse_out: CUDA float32 [n_seqs, n_q_heads, window], the window rows' log-sum-exp in params.lse_units."""
     _lse(lse_out, params)
-    rc = lib().slkv_row_lse(C.byref(params), q_win.data_ptr(), k.data_ptr(), cu_dev.data_ptr(), _cu_host(cu_seqlens),
-                            lse_out.data_ptr(), _ptr(status), workspace.data_ptr(), workspace.numel(), _stream(stream))
+    rc = _fn["slkv_row_lse"](stream, params, q_win, k, cu_dev, _cu_list(cu_seqlens), lse_out, status, workspace,
+                             workspace.numel())
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_row_lse")
     return lse_out
@@ -268,9 +282,8 @@ def slkv_score_noalloc(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor,
                        stream=None, lse: Optional[torch.Tensor] = None) -> torch.Tensor:
     """slkv_score for callers that cannot allocate: the scratch is a fixed array inside the library
     (slkv_noalloc_scratch_bytes() bytes); larger shapes raise SLKV_ERR_WORKSPACE."""
-    rc = lib().slkv_score_noalloc(C.byref(params), q_win.data_ptr(), k.data_ptr(), cu_dev.data_ptr(),
-                                  _cu_host(cu_seqlens), _lse(lse, params), pooled.data_ptr(), _ptr(status),
-                                  _stream(stream))
+    rc = _fn["slkv_score_noalloc"](stream, params, q_win, k, cu_dev, _cu_list(cu_seqlens), _lse(lse, params), pooled,
+                                   status)
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_score_noalloc")
     return pooled
@@ -283,11 +296,9 @@ def slkv_noalloc_scratch_bytes() -> int:
 def slkv_compress(params: SlkvParams, q_win, k, v, cu_dev, cu_seqlens: Sequence[int], budgets, k_out, v_out,
                   offsets, kept_idx, workspace, pooled: Optional[torch.Tensor] = None,
                   status: Optional[torch.Tensor] = None, stream=None, lse: Optional[torch.Tensor] = None) -> None:
-    rc = lib().slkv_compress(C.byref(params), q_win.data_ptr(), k.data_ptr(), v.data_ptr(), cu_dev.data_ptr(),
-                             _cu_host(cu_seqlens), budgets.data_ptr(), _lse(lse, params), k_out.data_ptr(),
-                             v_out.data_ptr(),
-                             k_out.shape[0], offsets.data_ptr(), kept_idx.data_ptr(), _ptr(pooled), _ptr(status),
-                             workspace.data_ptr(), workspace.numel(), _stream(stream))
+    rc = _fn["slkv_compress"](stream, params, q_win, k, v, cu_dev, _cu_list(cu_seqlens), budgets, _lse(lse, params),
+                              k_out, v_out, k_out.size(0), offsets, kept_idx, pooled, status, workspace,
+                              workspace.numel())
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_compress")
 
@@ -297,11 +308,9 @@ def slkv_compress_overlapped(params: SlkvParams, q_win, k, v, cu_dev, cu_seqlens
                              status: Optional[torch.Tensor] = None, stream=None,
                              lse: Optional[torch.Tensor] = None) -> None:
     """slkv_compress with successive calls overlapped on the GPU; outputs are valid behind slkv_join()."""
-    rc = lib().slkv_compress_overlapped(C.byref(params), q_win.data_ptr(), k.data_ptr(), v.data_ptr(),
-                                        cu_dev.data_ptr(), _cu_host(cu_seqlens), budgets.data_ptr(),
-                                        _lse(lse, params), k_out.data_ptr(), v_out.data_ptr(), k_out.shape[0], offsets.data_ptr(),
-                                        kept_idx.data_ptr(), _ptr(pooled), _ptr(status), workspace.data_ptr(),
-                                        workspace.numel(), _stream(stream))
+    rc = _fn["slkv_compress_overlapped"](stream, params, q_win, k, v, cu_dev, _cu_list(cu_seqlens), budgets,
+                                         _lse(lse, params), k_out, v_out, k_out.size(0), offsets, kept_idx, pooled,
+                                         status, workspace, workspace.numel())
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_compress_overlapped")
 
@@ -311,7 +320,7 @@ def slkv_workspace_bytes_overlapped(params: SlkvParams, cu_seqlens: Sequence[int
 
 
 def slkv_join(stream=None) -> None:
-    rc = lib().slkv_join(_stream(stream))
+    rc = _fn["slkv_join"](stream)
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_join")
 
@@ -327,10 +336,8 @@ def slkv_compress_host(params: SlkvParams, q_win, k, v, cu_seqlens: Sequence[int
         assert not t.is_cuda and t.is_contiguous()
     assert arena.is_cuda
     rows = C.c_int64(0)
-    rc = lib().slkv_compress_host(C.byref(params), q_win.data_ptr(), k.data_ptr(), v.data_ptr(), _cu_host(cu_seqlens),
-                                  budgets.data_ptr(), k_out.data_ptr(), v_out.data_ptr(), k_out.shape[0],
-                                  offsets.data_ptr(), kept_idx.data_ptr(), C.byref(rows), arena.data_ptr(),
-                                  arena.numel(), _stream(stream))
+    rc = _fn["slkv_compress_host"](stream, params, q_win, k, v, _cu_list(cu_seqlens), budgets, k_out, v_out,
+                                   k_out.size(0), offsets, kept_idx, rows, arena, arena.numel())
     if rc != SLKV_OK:
         raise SlkvError(rc, "slkv_compress_host")
     return int(rows.value)
@@ -368,32 +375,29 @@ def _check(rc: int, what: str) -> None:
 
 def slkv_cp_merge_lse(params: SlkvParams, lse_parts: torch.Tensor, lse_out: torch.Tensor, stream=None) -> torch.Tensor:
     """lse_parts: CUDA float32 [n_parts, n_q_heads, window] (contiguous); lse_out: [1, n_q_heads, window]."""
-    _check(lib().slkv_cp_merge_lse(C.byref(params), lse_parts.data_ptr(), int(lse_parts.shape[0]), lse_out.data_ptr(),
-                                   _stream(stream)), "slkv_cp_merge_lse")
+    _check(_fn["slkv_cp_merge_lse"](stream, params, lse_parts, lse_parts.size(0), lse_out), "slkv_cp_merge_lse")
     return lse_out
 
 
 def slkv_cp_select_init(budgets: torch.Tensor, window: int, seq_len: int, prefix: torch.Tensor, need: torch.Tensor,
                         stream=None) -> None:
-    _check(lib().slkv_cp_select_init(budgets.data_ptr(), int(budgets.numel()), int(window), int(seq_len),
-                                     prefix.data_ptr(), need.data_ptr(), _stream(stream)), "slkv_cp_select_init")
+    _check(_fn["slkv_cp_select_init"](stream, budgets, budgets.numel(), int(window), int(seq_len), prefix, need),
+           "slkv_cp_select_init")
 
 
 def slkv_cp_histogram(pooled: torch.Tensor, n_kv_heads: int, row_stride: int, own_begin: int, own_count: int, level: int,
                       prefix: torch.Tensor, hist: torch.Tensor, stream=None) -> torch.Tensor:
-    _check(lib().slkv_cp_histogram(pooled.data_ptr(), int(n_kv_heads), int(row_stride), int(own_begin), int(own_count),
-                                   int(level), prefix.data_ptr(), hist.data_ptr(), _stream(stream)), "slkv_cp_histogram")
+    _check(_fn["slkv_cp_histogram"](stream, pooled, int(n_kv_heads), int(row_stride), int(own_begin), int(own_count),
+                                    int(level), prefix, hist), "slkv_cp_histogram")
     return hist
 
 
 def slkv_cp_descend(hist: torch.Tensor, level: int, prefix: torch.Tensor, need: torch.Tensor, stream=None) -> None:
-    _check(lib().slkv_cp_descend(hist.data_ptr(), int(prefix.numel()), int(level), prefix.data_ptr(), need.data_ptr(),
-                                 _stream(stream)), "slkv_cp_descend")
+    _check(_fn["slkv_cp_descend"](stream, hist, prefix.numel(), int(level), prefix, need), "slkv_cp_descend")
 
 
 def slkv_cp_local_ties(hist_local: torch.Tensor, prefix: torch.Tensor, ties: torch.Tensor, stream=None) -> torch.Tensor:
-    _check(lib().slkv_cp_local_ties(hist_local.data_ptr(), prefix.data_ptr(), int(prefix.numel()), ties.data_ptr(),
-                                    _stream(stream)), "slkv_cp_local_ties")
+    _check(_fn["slkv_cp_local_ties"](stream, hist_local, prefix, prefix.numel(), ties), "slkv_cp_local_ties")
     return ties
 
 
@@ -406,9 +410,7 @@ def slkv_cp_emit(params: SlkvParams, k: torch.Tensor, v: torch.Tensor, rows: int
                  ties_all: torch.Tensor, part: int, window_rows: int, window_pos0: int, k_out: torch.Tensor,
                  v_out: torch.Tensor, offsets: torch.Tensor, kept_idx: torch.Tensor, workspace: torch.Tensor,
                  status: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(lib().slkv_cp_emit(C.byref(params), k.data_ptr(), v.data_ptr(), int(rows), pooled.data_ptr(), int(row_stride),
-                              int(own_begin), int(own_count), int(pos0), threshold.data_ptr(), need.data_ptr(),
-                              ties_all.data_ptr(), int(ties_all.shape[0]), int(part), int(window_rows), int(window_pos0),
-                              k_out.data_ptr(), v_out.data_ptr(), int(k_out.shape[0]), offsets.data_ptr(),
-                              kept_idx.data_ptr(), _ptr(status), workspace.data_ptr(), workspace.numel(),
-                              _stream(stream)), "slkv_cp_emit")
+    _check(_fn["slkv_cp_emit"](stream, params, k, v, int(rows), pooled, int(row_stride), int(own_begin), int(own_count),
+                               int(pos0), threshold, need, ties_all, ties_all.size(0), int(part), int(window_rows),
+                               int(window_pos0), k_out, v_out, k_out.size(0), offsets, kept_idx, status, workspace,
+                               workspace.numel()), "slkv_cp_emit")

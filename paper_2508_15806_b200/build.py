@@ -1,14 +1,16 @@
-"""Builds libslkv.so (CUDA, sm_100a) next to this file:  python -m paper_2508_15806_b200.build"""
+"""Builds libslkv.so (CUDA, sm_100a) and _slkv_call.so (the Python binding's call path) next to this file:  python -m paper_2508_15806_b200.build"""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libslkv.so")
+CALL = os.path.join(HERE, "_slkv_call.so")
 SOURCES = ["slkv_api.cu", "slkv_alloc.cu", "slkv_score_simt.cu", "slkv_score_tc.cu", "slkv_score_pipe.cu", "slkv_select.cu", "slkv_select_cluster.cu", "slkv_select_cta.cu",
            "slkv_noalloc.cu", "slkv_behavior.cu", "slkv_cp.cu"]
 
@@ -21,9 +23,9 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "slkv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -58,6 +60,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("nvcc failed linking libslkv.so")
+    r = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                        "-o", CALL, os.path.join(CSRC, "slkv_pycall.c")], capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("building _slkv_call.so failed")
     return LIB
 
 
