@@ -34,7 +34,7 @@ WORKLOAD_INDEX = 2          # the 32k-context, 32-layer configuration (third of 
 TOTAL_INDEX = 1             # average budget 512 per KV head
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_per_key_row.txt")
 KERNEL_SOURCES = {"k_score_pipe": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"],
-                  "k_score_fused": ["slkv_score_tc.cu", "slkv_tc_device.cuh"]}
+                  "k_score_fused": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"]}
 
 
 def source_sha16(kernel: str):

@@ -72,7 +72,7 @@ enum { SLKV_HISTORY = 0,                              /* slkv_params.softmax_dom
 enum { SLKV_LSE_LN = 0, SLKV_LSE_LOG2 = 1 };          /* slkv_params.lse_units: natural log / base-2 log */
 enum { SLKV_PATH_AUTO = 0,                            /* slkv_params.score_path */
        SLKV_PATH_SIMT = 1,                            /*   fp32 FMA kernels (any dtype, head_dim 64/128) */
-       SLKV_PATH_TENSOR = 2 };                        /*   tcgen05 + TMA kernels (bf16, head_dim 128) */
+       SLKV_PATH_TENSOR = 2 };                        /*   tcgen05 + TMA kernels (bf16, up to 256 score rows per KV head) */
 
 /* Shapes and options shared by slkv_score / slkv_compress. Strides are in elements. */
 typedef struct slkv_params {
@@ -239,17 +239,15 @@ int slkv_compress(const slkv_params* p, const void* q_win, const void* k, const 
  *
  * The layers of a prefill are independent problems, and inside one layer the vote pass needs every key's row
  * statistics first (the softmax of Eq. 7 runs over all keys).  This entry point therefore works on several layers
- * at once: the score kernel takes a LIST of layers per launch and runs, in every CTA, the row-statistics pass of a
- * layer beside the vote pass of the layer before it; the selection and the gather of a layer run on side streams
- * of the library's own while the score kernel works on later layers.  A call queues its layer; the score kernel
- * goes out when eight layers are queued and a ninth arrives, or at slkv_join.  Consequences:
- *   - Nothing of a call needs to have been enqueued when it returns, and its outputs (k_out, v_out, offsets,
- *     kept_idx, pooled_opt, status) are NOT ordered on `stream`.  slkv_join(stream) enqueues whatever is still
+ * at once: a call queues its layer, and a list of layers goes out as three launches on `stream` -- the score kernel, in
+ * which the row-statistics pass of later layers runs between the vote passes of earlier ones, then the selections and the
+ * gathers of all layers of the list -- when sixteen layers are queued, or at slkv_join.  Consequences:
+ *   - Nothing of a call needs to have been enqueued when it returns: slkv_join(stream) enqueues whatever is still
  *     queued and makes `stream` wait for every overlapped call made so far on the current device (no host wait);
  *     consume outputs, or free / overwrite any input, output or workspace buffer -- q_win, k, v, cu_seqlens_dev
  *     and budgets included -- only behind it.  cu_seqlens_host is read during the call only.  Any other slkv_*
  *     call that uses a workspace joins by itself first.
- *   - Streams and host threads: the calls made on one stream form one sequence (queue, workspace slots, events);
+ *   - Streams and host threads: the calls made on one stream form one sequence (queue, workspace);
  *     calls made on another stream -- by another host thread or the same one -- form another, and the two do not
  *     disturb each other as long as each has its own workspace (calls on two streams that share a workspace are
  *     serialised: the later one waits for what the other stream has in flight).  A join orders its stream behind
@@ -257,18 +255,14 @@ int slkv_compress(const slkv_params* p, const void* q_win, const void* k, const 
  *     itself.  The entry points may be called from several host threads at once (one lock inside); up to eight
  *     streams per device keep a sequence each, a ninth takes over the one used longest ago once that one's
  *     stream has been made to wait for what it had in flight.
- *   - workspace must hold slkv_workspace_bytes_overlapped: votes, source-row lists and row statistics for up to
- *     eighteen layers in flight (77 MB for 8 KV heads x 32k keys; three layers' worth for shapes the list kernel
- *     does not take).  Successive calls share one workspace; a call with another shape or workspace first drains
- *     what is in flight.  q_win, k, v, budgets and the outputs of calls that may be in flight together must not
- *     alias each other's outputs.
- *   - The first call on a stream creates eighteen side streams and 54 events for it (no device memory).
- *   - The call sequence is stream-ordered and allocates nothing, so a step's calls plus the join can be captured
- *     in a CUDA graph (the side streams fork from and rejoin `stream`).
- *   - The list kernel takes bf16, head_dim 128, (n_q_heads / n_kv_heads) * window <= 128 and a multiple of 32,
- *     at most 64 sequences, segments of at most 32768 history positions, pool_kernel <= 9.  Other shapes that the
- *     one-CTA selection takes run one layer per score launch with the selection and gather on the side streams;
- *     the rest run as slkv_compress does, on `stream`, after a join.
+ *   - workspace must hold slkv_workspace_bytes_overlapped: votes, source-row lists and row statistics for the
+ *     sixteen layers of a list (one layer's worth for shapes that are not taken as lists).  Successive calls share one
+ *     workspace; a call with another shape or workspace first sends out what is queued.  q_win, k, v, budgets and the
+ *     outputs of calls that may be in flight together must not alias each other's outputs.
+ *   - The call sequence is stream-ordered and allocates nothing on the device, so a step's calls plus the join can be
+ *     captured in a CUDA graph.
+ *   - Lists take bf16 and (n_q_heads / n_kv_heads) * window <= 256, at most 64 sequences, segments the one-launch
+ *     selections take (up to 131072 history positions).  Other shapes run as slkv_compress does, on `stream`, after a join.
  * Arguments, results and error codes otherwise as slkv_compress.
  */
 int slkv_compress_overlapped(const slkv_params* p, const void* q_win, const void* k, const void* v,
@@ -403,24 +397,17 @@ int slkv_kernel_count(void);
 
 /*
  * Timeline tracing of the tensor-core score kernels (diagnostics; no counterpart in the paper).
- * With a device buffer set on the calling thread, every CTA of the two score kernels stores %globaltimer
- * nanosecond stamps into it: 64 uint64 slots per CTA, pass 1 first (n_cta * 64 entries), pass 2 after
- * it.  Slots: 0 CTA start, 1 set-up done, 2 query tile landed, 3 first key tile landed, 4 CTA end,
- * 8+2i / 9+2i start / end of the softmax arithmetic on the CTA's i-th tile (i < 28).  The score kernel of the
- * overlapped entry point (a list of layers per launch, two streams per CTA) writes: 0 CTA start, 1 / 7 stream
- * A / B past its wait for the launch before, 2 first accumulator of stream A ready, 3 first log-sum-exps of
- * stream B merged, 5 / 6 stream A / B done, 4 CTA end, 8+2j / 9+2j list entry j published by stream A / begun by
- * stream B, 60 / 61 the SM cycle counter at CTA start / end.  The buffer that is set when a launch is enqueued is
- * the one it writes (the overlapped entry point enqueues a list when it is full and one more layer has come, or at
- * a join).  The buffer must hold 2 * n_cta * 64 * 8 bytes (n_cta <= number of SMs); smaller buffers switch tracing
- * off.  NULL switches it off.
+ * With a device buffer set on the calling thread, every CTA of the score kernel stores %globaltimer nanosecond stamps
+ * into it, 64 uint64 slots per CTA: 0 CTA start, 1 past its wait for the launch before, 3 first log-sum-exps of a vote
+ * phase there, 4 CTA end, 60 / 61 the SM cycle counter at CTA start / end.  The buffer that is set when a launch is
+ * enqueued is the one it writes (the overlapped entry point enqueues a list when it is full, or at a join).  The buffer must
+ * hold n_cta * 64 * 8 bytes (n_cta <= number of SMs); smaller buffers switch tracing off.  NULL switches it off.
  */
 int slkv_trace_set_buffer(void* dev_buf, size_t bytes);
 
 /*
  * Test hook for the bounded waits (no counterpart in the paper).  Where the CTAs of a launch wait for one another
- * (the grid-wide barrier between the two passes of slkv_score / slkv_compress, the per-layer counters of the list
- * kernel behind slkv_compress_overlapped), every wait gives up after one second, sets SLKV_ERR_DEVICE_TIMEOUT in the
+ * (the counters between the two passes of the score kernel), every wait gives up after one second, sets SLKV_ERR_DEVICE_TIMEOUT in the
  * call's status word, releases what the CTA holds and returns.  With the hook armed (on != 0) the next such launch made
  * by the calling thread waits for one arrival more than there are CTAs, so that exactly this path runs: the call's
  * results are then incomplete and its status word says so; the calls after it are unaffected.  One-shot: the launch

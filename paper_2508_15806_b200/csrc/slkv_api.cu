@@ -32,7 +32,6 @@ cudaEvent_t prof_event() {
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-constexpr int kMinChunkKeys = 128;     // no score path uses smaller chunks (sizes the partial buffers)
 constexpr int kMaxWindow = 256;
 constexpr size_t kSimtSmemLimit = 192 * 1024;
 
@@ -41,10 +40,11 @@ int cuda_fail(cudaError_t e) {
   return SLKV_ERR_CUDA;
 }
 
-constexpr int kLaySlots = 2 * kPipeMaxLayers + 2;   // overlapped calls: layers in flight at once
+constexpr int kLaySlots = kListMaxLayers;      // overlapped calls: layers a launch takes
 struct Layout {
-  size_t hist_off, tile_off, vote[kLaySlots], pooled, part_m[kLaySlots], part_z[kLaySlots], flags, gather_src[kLaySlots],
-      win_m[kLaySlots], win_z[kLaySlots], total;
+  size_t hist_off, tile_off, pooled, flags, total;
+  size_t layer0, layer_bytes;                  // per-layer part: layer i's begins at layer0 + i * layer_bytes
+  size_t vote, part, gather_src, win_m, win_z; // ... with these in it
 };
 
 // Validates p and cu_seqlens_host and fills the host-known fields of `pb`.
@@ -126,10 +126,10 @@ int describe(const slkv_params* p, const int32_t* cu_host, Problem* pb) {
   return SLKV_OK;
 }
 
-// Layers an overlapped call sequence keeps in flight: many where the score kernel takes lists of layers, three
-// otherwise (one being scored, one being selected, one being gathered).
-int overlapped_slots(const Problem& pb) {
-  return tensor_path_supported(pb.p) && score_pipe_supported(pb) && pb.p.score_path != SLKV_PATH_SIMT ? kLaySlots : 3;
+// Overlapped calls are launched as lists where the tensor-core score kernel and a list selection take the shape.
+bool list_supported(const Problem& pb) {
+  return tensor_path_supported(pb.p) && pb.p.score_path != SLKV_PATH_SIMT && pb.tab.n_inline > 0 && pb.max_hist > 0 &&
+         (select_cta_supported(pb) || select_cluster_supported(pb));
 }
 
 Layout layout_of(const Problem& pb, bool overlapped = false) {
@@ -137,39 +137,26 @@ Layout layout_of(const Problem& pb, bool overlapped = false) {
   size_t o = 0;
   L.hist_off = o; o = align_up(o + (size_t)(pb.p.n_seqs + 1) * sizeof(int64_t));
   L.tile_off = o; o = align_up(o + (size_t)(pb.p.n_seqs + 1) * sizeof(int32_t));
-  // Overlapped calls keep many layers in flight (the score kernel takes a list of layers per launch, selections and
-  // gathers trail behind): each has its own votes, source-row list and per-CTA row statistics.  Ordinary calls use
-  // the first of each.
   const size_t votes = (size_t)pb.p.n_kv_heads * (size_t)pb.total_hist * sizeof(float);
-  const int n_slots = overlapped ? overlapped_slots(pb) : 1;
-  for (int i = 0; i < kLaySlots; ++i) {
-    L.vote[i] = i < n_slots ? o : L.vote[0];
-    if (i < n_slots) o = align_up(o + votes);
-  }
   L.pooled = o; o = align_up(o + votes);
-  const size_t nchunks = (size_t)(pb.max_hist + kMinChunkKeys - 1) / kMinChunkKeys + 2;
-  const size_t parts = (size_t)pb.n_seg * pb.R * nchunks * sizeof(float);
-  for (int i = 0; i < kLaySlots; ++i) {
-    L.part_m[i] = i < n_slots ? o : L.part_m[0];
-    if (i < n_slots) o = align_up(o + parts);
-    L.part_z[i] = i < n_slots ? o : L.part_z[0];
-    if (i < n_slots) o = align_up(o + parts);
-  }
   L.flags = o; o = align_up(o + 8 * sizeof(int32_t));
-  const size_t srcs = (size_t)pb.p.n_kv_heads * (size_t)pb.total_tokens * sizeof(int32_t);
-  for (int i = 0; i < kLaySlots; ++i) {
-    L.gather_src[i] = i < n_slots ? o : L.gather_src[0];
-    if (i < n_slots) o = align_up(o + srcs);
-  }
+  // Every layer of a list has its own votes, row statistics and source-row list; ordinary calls use the first.
+  L.layer0 = o;
+  size_t q = 0;
+  L.vote = q; q = align_up(q + votes);
+  // row statistics per split range (tensor-core path: see stat_view) or chunk that shares a segment
+  const size_t shares = (size_t)tensor_slot_stride(pb);
+  const size_t chunks = (size_t)(pb.max_hist + simt_chunk_keys() - 1) / simt_chunk_keys();
+  const size_t by_tensor = (size_t)pb.n_seg * ((shares * 8 + 12) * (size_t)pb.R + kMaxSplit / 8);
+  const size_t by_simt = (size_t)pb.n_seg * pb.R * chunks * 8;
+  L.part = q; q = align_up(q + (by_tensor > by_simt ? by_tensor : by_simt));
+  L.gather_src = q; q = align_up(q + (size_t)pb.p.n_kv_heads * (size_t)pb.total_tokens * sizeof(int32_t));
   // row statistics over the window keys (all-causal softmax domain): [n_seg][R] maxima and sums
   const size_t wins = (size_t)pb.n_seg * pb.R * sizeof(float);
-  for (int i = 0; i < kLaySlots; ++i) {
-    L.win_m[i] = i < n_slots ? o : L.win_m[0];
-    if (i < n_slots) o = align_up(o + wins);
-    L.win_z[i] = i < n_slots ? o : L.win_z[0];
-    if (i < n_slots) o = align_up(o + wins);
-  }
-  L.total = o;
+  L.win_m = q; q = align_up(q + wins);
+  L.win_z = q; q = align_up(q + wins);
+  L.layer_bytes = q;
+  L.total = o + q * (size_t)(overlapped && list_supported(pb) ? kLaySlots : 1);
   return L;
 }
 
@@ -184,29 +171,32 @@ int resolve_path(const Problem& pb, int* path) {
   return SLKV_OK;
 }
 
-// slot: which of the vote arrays / source-row lists / sets of row statistics (overlapped calls)
-int bind_workspace(Problem* pb, void* ws, size_t ws_bytes, int path, bool overlapped = false, int slot = 0) {
-  if (!ws) return SLKV_ERR_WORKSPACE;
-  if (reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SLKV_ERR_BAD_ALIGN;
-  Layout L = layout_of(*pb, overlapped);
-  if (ws_bytes < L.total) return SLKV_ERR_WORKSPACE;
+// slot: the layer's place in the list (overlapped calls)
+void carve(Problem* pb, const Layout& L, void* ws, int path, int slot) {
   unsigned char* b = static_cast<unsigned char*>(ws);
   pb->hist_off = reinterpret_cast<int64_t*>(b + L.hist_off);
   pb->tile_off = reinterpret_cast<int32_t*>(b + L.tile_off);
   pb->tab.tile_ptr = pb->tile_off;
   pb->tab.hist_ptr = reinterpret_cast<const long long*>(pb->hist_off);
-  pb->vote = reinterpret_cast<float*>(b + L.vote[slot]);
   pb->pooled_ws = reinterpret_cast<float*>(b + L.pooled);
-  pb->part_m = reinterpret_cast<float*>(b + L.part_m[slot]);
-  pb->part_z = reinterpret_cast<float*>(b + L.part_z[slot]);
   pb->dev_flags = reinterpret_cast<int32_t*>(b + L.flags);
-  pb->gather_src = reinterpret_cast<int32_t*>(b + L.gather_src[slot]);
-  pb->win_m = reinterpret_cast<float*>(b + L.win_m[slot]);
-  pb->win_z = reinterpret_cast<float*>(b + L.win_z[slot]);
+  unsigned char* l = b + L.layer0 + (size_t)slot * L.layer_bytes;
+  pb->vote = reinterpret_cast<float*>(l + L.vote);
+  pb->part = l + L.part;
+  pb->gather_src = reinterpret_cast<int32_t*>(l + L.gather_src);
+  pb->win_m = reinterpret_cast<float*>(l + L.win_m);
+  pb->win_z = reinterpret_cast<float*>(l + L.win_z);
   pb->chunk_keys = path == SLKV_PATH_TENSOR ? 128 : simt_chunk_keys();
   pb->n_chunks = path == SLKV_PATH_TENSOR ? tensor_slot_stride(*pb)
                                           : (pb->max_hist + pb->chunk_keys - 1) / pb->chunk_keys;
   if (pb->n_chunks < 1) pb->n_chunks = 1;
+}
+int bind_workspace(Problem* pb, void* ws, size_t ws_bytes, int path) {
+  if (!ws) return SLKV_ERR_WORKSPACE;
+  if (reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SLKV_ERR_BAD_ALIGN;
+  const Layout L = layout_of(*pb);
+  if (ws_bytes < L.total) return SLKV_ERR_WORKSPACE;
+  carve(pb, L, ws, path, 0);
   return SLKV_OK;
 }
 
@@ -227,299 +217,230 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
   int rc = enqueue_window_stats(pb, path, st, launches);
   if (rc != SLKV_OK) return rc;
   const int passes = pb.lse_opt ? 2 : 3;
-  cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes, st, launches)
+  cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes, nullptr, st, launches)
                                            : launch_score_simt(pb, passes, st, launches);
   if (e != cudaSuccess) return cuda_fail(e);
   return SLKV_OK;
 }
 
 // ---- overlapped calls ---------------------------------------------------------------------------------------
-// The selection and the gather of a layer run on side streams while the score kernels of the following layers
-// run on the caller's stream.  Where the two-layer score kernel takes the shape, a call enqueues pass 1 of its
-// own layer together with pass 2 of the layer before (which stays "pending" until the next call or a join).
-constexpr int kSlots = 2 * kPipeMaxLayers + 2;     // layers whose votes / source rows / row statistics are live at once
-constexpr int kSideStreams = 9;   // after the last launch of a list the selections of its layers run side by side
-struct PendingCall {
-  bool valid = false;
-  Problem pb;
-  TcPlan plan;
-  int slot = 0;
-  const int32_t* budgets = nullptr;
-  void* k_out = nullptr;
-  void* v_out = nullptr;
-  int64_t capacity = 0;
-  int32_t* offsets = nullptr;
-  int32_t* kept_idx = nullptr;
-  float* pooled_opt = nullptr;
-  int32_t* status = nullptr;
-  cudaStream_t st = nullptr;
-  std::vector<int32_t> cu_host;          // the call's cu_seqlens_host (the caller's copy is only valid during the call)
-};
-struct ShapeSig {                                  // calls in flight together must carve the workspace alike
-  const void* ws = nullptr;
+// A call queues its layer; a list of layers goes out as three launches on the caller's stream -- scores, selections,
+// gathers, each over all layers of the list -- when it is full or at a join.  What a list gives over single calls: the
+// statistics of one layer overlap the votes of another, 16 layers' selections fill the SMs side by side, and the host
+// makes three launches instead of 48.
+struct ListState {
+  bool open = false;             // the shape below is valid
+  slkv_params p;
+  std::vector<int32_t> cu_host;
+  const int32_t* cu_dev = nullptr;
+  void* ws = nullptr;
   size_t ws_bytes = 0;
-  int n_seqs = 0, n_kv_heads = 0, R = 0, max_hist = 0, path = 0;
-  int64_t total_hist = 0, total_tokens = 0;
-  bool operator==(const ShapeSig& o) const {
-    return ws == o.ws && ws_bytes == o.ws_bytes && n_seqs == o.n_seqs && n_kv_heads == o.n_kv_heads && R == o.R &&
-           max_hist == o.max_hist && path == o.path && total_hist == o.total_hist && total_tokens == o.total_tokens;
-  }
-};
-struct OverlapState {
-  cudaStream_t side_select[kSideStreams] = {}, side_gather[kSideStreams] = {};   // slot s uses streams s % kSideStreams
-  cudaEvent_t scored[kSlots] = {};       // recorded on the caller's stream after the vote pass of the slot's layer
-  cudaEvent_t selected[kSlots] = {};     // recorded on a selection stream after the selection
-  cudaEvent_t done[kSlots] = {};         // recorded on the gather stream after the gather
-  bool in_flight[kSlots] = {};
-  bool wait_done[kSlots] = {};           // the slot's next selection must first wait for the gather that had the slot
-  unsigned seq = 0;
-  std::vector<PendingCall> queue;        // layers whose score kernel is not launched yet (at most kPipeMaxLayers + 1)
-  PendingCall pending;                   // pass 1 launched, pass 2 not
-  std::vector<PendingCall> deferred;     // votes launched and `scored` recorded, selection and gather not enqueued yet
-  ShapeSig sig;
+  bool with_lse = false;
+  Problem pb;                    // of the shape; the per-layer pointers are set call by call
+  Layout layout;
+  ScorePlan plan;
+  int n = 0;                     // layers queued
+  ScoreLayer score[kListMaxLayers];
+  TailLayer tail[kListMaxLayers];
+  bool in_flight = false;        // lists have gone out since this stream's last join
+  cudaEvent_t event = nullptr;   // orders another stream behind this one
 };
 // One state per (device, caller's stream): calls made on different streams (by different host threads, or by one)
-// never share a queue, a slot or an event, so each stream's calls keep their own order whatever the others do.
+// never share a queue, so each stream's calls keep their own order whatever the others do.
 constexpr int kMaxDevices = 64;
 constexpr int kStatesPerDevice = 8;
 struct DeviceStates {
-  OverlapState st[kStatesPerDevice];
+  ListState st[kStatesPerDevice];
   cudaStream_t owner[kStatesPerDevice] = {};
   bool used[kStatesPerDevice] = {};
   unsigned long long last_use[kStatesPerDevice] = {};
   unsigned long long tick = 0;
 };
-DeviceStates g_overlap[kMaxDevices];
-std::mutex g_overlap_mu;
-constexpr int kSelectSmReserve = 16;              // SMs left to the selection kernels of the layers before
+DeviceStates* g_lists[kMaxDevices] = {};
+std::mutex g_lists_mu;
 
-cudaError_t flush_pending(OverlapState* os, int* launches);
-
-bool state_idle(const OverlapState& s) {
-  if (!s.queue.empty() || s.pending.valid || !s.deferred.empty()) return false;
-  for (int h = 0; h < kSlots; ++h)
-    if (s.in_flight[h]) return false;
-  return true;
+// The queued layers of a state go out on its stream (g_lists_mu held).
+cudaError_t flush_list(ListState* s, cudaStream_t owner, int* launches) {
+  if (s->n == 0) return cudaSuccess;
+  const int n = s->n;
+  s->n = 0;
+  s->in_flight = true;
+  cudaError_t e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, owner, launches);
+  if (e == cudaSuccess)
+    e = select_cta_supported(s->pb) ? launch_select_cta(s->pb, s->tail, n, owner, launches)
+                                    : launch_select_cluster(s->pb, s->tail, n, owner, launches);
+  if (e == cudaSuccess) e = launch_gather(s->pb, s->tail, n, owner, launches);
+  return e;
 }
 
-// The state of overlapped calls made on `st` on the current device (g_overlap_mu held).  All eight in use by other
-// streams: the one used longest ago is drained -- its queued layers go out and its own stream waits for what it has
-// in flight, as a join on that stream would -- and handed over.
-cudaError_t overlap_state(cudaStream_t st, OverlapState** out, int* launches) {
+// Orders `st` behind everything of a state that has gone out.
+cudaError_t order_behind(ListState* s, cudaStream_t owner, cudaStream_t st) {
+  if (!s->in_flight || owner == st) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  if (!s->event) e = cudaEventCreateWithFlags(&s->event, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(s->event, owner);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->event, 0);
+  return e;
+}
+
+cudaError_t device_states(DeviceStates** out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  DeviceStates& d = g_overlap[dev];
+  if (!g_lists[dev]) g_lists[dev] = new DeviceStates();
+  *out = g_lists[dev];
+  return cudaSuccess;
+}
+
+// The state of overlapped calls made on `st` on the current device (g_lists_mu held).  All eight in use by other
+// streams: the one used longest ago is handed over once its queued layers have gone out on its own stream.
+cudaError_t list_state(cudaStream_t st, ListState** out, DeviceStates** states, int* launches) {
+  DeviceStates* d = nullptr;
+  cudaError_t e = device_states(&d);
+  if (e != cudaSuccess) return e;
+  *states = d;
   int idx = -1;
   for (int i = 0; i < kStatesPerDevice; ++i)
-    if (d.used[i] && d.owner[i] == st) idx = i;
+    if (d->used[i] && d->owner[i] == st) idx = i;
   if (idx < 0) {
     for (int i = 0; i < kStatesPerDevice && idx < 0; ++i)
-      if (!d.used[i]) idx = i;
+      if (!d->used[i]) idx = i;
     if (idx < 0) {
       int oldest = 0, oldest_idle = -1;
       for (int i = 0; i < kStatesPerDevice; ++i) {
-        if (d.last_use[i] < d.last_use[oldest]) oldest = i;
-        if (state_idle(d.st[i]) && (oldest_idle < 0 || d.last_use[i] < d.last_use[oldest_idle])) oldest_idle = i;
+        if (d->last_use[i] < d->last_use[oldest]) oldest = i;
+        if (d->st[i].n == 0 && !d->st[i].in_flight && (oldest_idle < 0 || d->last_use[i] < d->last_use[oldest_idle])) oldest_idle = i;
       }
       idx = oldest_idle >= 0 ? oldest_idle : oldest;
-      OverlapState& v = d.st[idx];
-      e = flush_pending(&v, launches);
-      for (int h = 0; h < kSlots && e == cudaSuccess; ++h)
-        if (v.in_flight[h]) {
-          e = cudaStreamWaitEvent(d.owner[idx], v.done[h], 0);
-          v.in_flight[h] = false;
-        }
+      e = flush_list(&d->st[idx], d->owner[idx], launches);
+      // a later join on any stream must still cover these calls: the stream that takes the state over stands for them
+      if (e == cudaSuccess) e = order_behind(&d->st[idx], d->owner[idx], st);
       if (e != cudaSuccess) return e;
-      v.sig = ShapeSig();
+      d->st[idx].open = false;
     }
-    d.used[idx] = true;
-    d.owner[idx] = st;
+    d->used[idx] = true;
+    d->owner[idx] = st;
   }
-  d.last_use[idx] = ++d.tick;
-  OverlapState& s = d.st[idx];
-  if (!s.side_gather[kSideStreams - 1]) {
-    for (int i = 0; i < kSideStreams; ++i) {
-      e = cudaStreamCreateWithFlags(&s.side_select[i], cudaStreamNonBlocking);
-      if (e != cudaSuccess) return e;
-      e = cudaStreamCreateWithFlags(&s.side_gather[i], cudaStreamNonBlocking);
-      if (e != cudaSuccess) return e;
-    }
-    for (int h = 0; h < kSlots; ++h) {
-      e = cudaEventCreateWithFlags(&s.scored[h], cudaEventDisableTiming);
-      if (e != cudaSuccess) return e;
-      e = cudaEventCreateWithFlags(&s.selected[h], cudaEventDisableTiming);
-      if (e != cudaSuccess) return e;
-      e = cudaEventCreateWithFlags(&s.done[h], cudaEventDisableTiming);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  *out = &s;
+  d->last_use[idx] = ++d->tick;
+  *out = &d->st[idx];
   return cudaSuccess;
-}
-
-// Before a layer takes a slot: its vote array may still be read by the selection of the layer that had the slot,
-// its source-row list by that layer's gather.
-cudaError_t flush_deferred(OverlapState* os, int* launches);
-cudaError_t claim_slot(OverlapState* os, int slot, cudaStream_t st, int* launches) {
-  for (size_t i = 0; i < os->deferred.size(); ++i)
-    if (os->deferred[i].slot == slot) {                              // its selection is not even enqueued yet
-      cudaError_t e = flush_deferred(os, launches);
-      if (e != cudaSuccess) return e;
-      break;
-    }
-  if (!os->in_flight[slot]) return cudaSuccess;
-  os->wait_done[slot] = true;
-  return cudaStreamWaitEvent(st, os->selected[slot], 0);
-}
-
-// The votes of layer `c` are enqueued on c.st: selection on a side stream, gather on another.  While more score
-// launches follow, two selections at a time (a selection takes one SM per segment, and a score launch whose CTAs wait
-// for one another starts only when all of them fit beside what is running); `wide`: nothing follows, all side
-// streams.  `scored_recorded`: the layer's event was recorded when its votes were launched (a deferred tail).
-cudaError_t enqueue_tail(OverlapState* os, const PendingCall& c, bool beside_pipe, bool wide, int* launches,
-                         bool scored_recorded = false) {
-  const int slot = c.slot;
-  const int si = wide ? slot % kSideStreams : slot % 2;
-  cudaStream_t sel = os->side_select[si], gat = os->side_gather[si];
-  if (g_prof_on == 1) sel = gat = c.st;  // timing of every kernel: one stream, so that the event pairs do not overlap
-  cudaError_t e = scored_recorded ? cudaSuccess : cudaEventRecord(os->scored[slot], c.st);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(sel, os->scored[slot], 0);
-  if (e == cudaSuccess && os->wait_done[slot]) e = cudaStreamWaitEvent(sel, os->done[slot], 0);
-  os->wait_done[slot] = false;
-  if (e != cudaSuccess) return e;
-  e = launch_select_cta(c.pb, c.pooled_opt, c.budgets, c.offsets, c.kept_idx, c.capacity, c.status, sel, launches);
-  if (e != cudaSuccess) return e;
-  e = cudaEventRecord(os->selected[slot], sel);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(gat, os->selected[slot], 0);
-  if (e != cudaSuccess) return e;
-  // beside the two-layer score kernel an SM has registers left for one 128-thread gather CTA
-  e = launch_gather(c.pb, c.offsets, c.kept_idx, c.k_out, c.v_out, c.capacity, gat, launches,
-                    beside_pipe ? 128 : 256);
-  if (e != cudaSuccess) return e;
-  e = cudaEventRecord(os->done[slot], gat);
-  if (e != cudaSuccess) return e;
-  os->in_flight[slot] = true;
-  return cudaSuccess;
-}
-
-// Selections and gathers that were held back until the score launch after theirs had gone out: the score kernel is
-// then ahead of them in the order the device takes its work in and has its SMs first, and they fill the SMs it leaves.
-cudaError_t flush_deferred(OverlapState* os, int* launches) {
-  cudaError_t e = cudaSuccess;
-  for (size_t i = 0; i < os->deferred.size() && e == cudaSuccess; ++i)
-    e = enqueue_tail(os, os->deferred[i], true, true, launches, true);
-  os->deferred.clear();
-  return e;
-}
-
-// Launches the score kernel for the first n queued layers (pass 1) together with pass 2 of the pending layer and of
-// all but the last of them -- of all of them when `finish` is set -- then the selections and gathers of the
-// layers whose votes that gives.
-cudaError_t launch_queue(OverlapState* os, int n, bool finish, int* launches) {
-  if (n > (int)os->queue.size()) n = (int)os->queue.size();
-  if (n == 0 && !(finish && os->pending.valid)) return cudaSuccess;
-  if (n == 1 && finish && !os->pending.valid) {
-    // a single layer and nothing to pair it with: both passes in the single-layer kernel
-    const PendingCall& c = os->queue[0];
-    cudaError_t e1 = launch_score_tensor(c.pb, c.cu_host.data(), c.status, c.pb.lse_opt ? 2 : 3, c.st, launches);
-    if (e1 == cudaSuccess) e1 = flush_deferred(os, launches);
-    if (e1 == cudaSuccess) e1 = enqueue_tail(os, c, false, true, launches);
-    os->queue.clear();
-    return e1;
-  }
-  const TcPlan* plans[kPipeMaxLayers];
-  for (int i = 0; i < n; ++i) plans[i] = &os->queue[i].plan;
-  cudaStream_t st = n > 0 ? os->queue[0].st : os->pending.st;
-  // layers that came with their row statistics need the vote pass only (a queue holds one kind: see compress_impl)
-  const bool votes_only = n > 0 && os->queue[0].pb.lse_opt != nullptr;
-  const bool more_follow = !finish;                  // a full list went out because one more layer has come
-  if (votes_only) finish = true;
-  cudaError_t e = launch_score_pipe(os->pending.valid ? &os->pending.plan : nullptr, plans, n, finish, votes_only, st,
-                                    launches);
-  if (votes_only && more_follow) {
-    // An ordinary launch takes the SMs that are free when it starts: selections that became ready at the same moment
-    // would take a third of them for their 26 µs.  So this launch's selections and gathers are held back until the
-    // next score launch is out (or a join), and the ones held back at the launch before go out now, behind this one.
-    for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaEventRecord(os->scored[os->queue[i].slot], st);
-    if (e == cudaSuccess) e = flush_deferred(os, launches);
-    for (int i = 0; i < n && e == cudaSuccess; ++i) os->deferred.push_back(os->queue[i]);
-    os->queue.erase(os->queue.begin(), os->queue.begin() + n);
-    return e;
-  }
-  if (e == cudaSuccess) e = flush_deferred(os, launches);
-  if (e == cudaSuccess && os->pending.valid) e = enqueue_tail(os, os->pending, true, finish, launches);
-  os->pending.valid = false;
-  const int n_voted = finish ? n : n - 1;
-  for (int i = 0; i < n_voted && e == cudaSuccess; ++i) e = enqueue_tail(os, os->queue[i], true, finish, launches);
-  if (!finish && n > 0) os->pending = os->queue[n - 1];
-  os->queue.erase(os->queue.begin(), os->queue.begin() + n);
-  return e;
-}
-cudaError_t flush_pending(OverlapState* os, int* launches) {
-  cudaError_t e = cudaSuccess;
-  while (!os->queue.empty() && (int)os->queue.size() > kPipeMaxLayers && e == cudaSuccess)
-    e = launch_queue(os, kPipeMaxLayers, false, launches);
-  if (e == cudaSuccess) e = launch_queue(os, (int)os->queue.size(), true, launches);
-  if (e == cudaSuccess) e = flush_deferred(os, launches);
-  return e;
 }
 
 // Calls on other streams whose workspace overlaps [ws, ws + bytes): their queued layers go out and `st` waits for what
-// they have in flight, before a call on `st` carves that memory up for itself (g_overlap_mu held).
-cudaError_t drain_states_sharing(const OverlapState* mine, const void* ws, size_t bytes, cudaStream_t st, int* launches) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  DeviceStates& d = g_overlap[dev];
+// they have in flight, before a call on `st` carves that memory up for itself (g_lists_mu held).
+cudaError_t drain_states_sharing(DeviceStates* d, const ListState* mine, const void* ws, size_t bytes, cudaStream_t st,
+                                 int* launches) {
   const char* lo = static_cast<const char*>(ws);
   for (int i = 0; i < kStatesPerDevice; ++i) {
-    OverlapState& s = d.st[i];
-    if (!d.used[i] || &s == mine || !s.sig.ws || state_idle(s)) continue;
-    const char* olo = static_cast<const char*>(s.sig.ws);
-    if (olo + s.sig.ws_bytes <= lo || lo + bytes <= olo) continue;
-    e = flush_pending(&s, launches);
-    for (int h = 0; h < kSlots && e == cudaSuccess; ++h)
-      if (s.in_flight[h]) e = cudaStreamWaitEvent(st, s.done[h], 0);
+    ListState& s = d->st[i];
+    if (!d->used[i] || &s == mine || !s.ws || (s.n == 0 && !s.in_flight)) continue;
+    const char* olo = static_cast<const char*>(s.ws);
+    if (olo + s.ws_bytes <= lo || lo + bytes <= olo) continue;
+    cudaError_t e = flush_list(&s, d->owner[i], launches);
+    if (e == cudaSuccess) e = order_behind(&s, d->owner[i], st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-// Makes `st` wait for every overlapped call still in flight on this device, whatever stream it was made on (no host
-// wait).  Only the calls made on `st` itself are then forgotten: the others stay in flight for a join on their own
-// stream, which still has to be ordered behind them.
-cudaError_t join_overlapped(cudaStream_t st, int* launches) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaSuccess;
-  std::lock_guard<std::mutex> lock(g_overlap_mu);
-  DeviceStates& d = g_overlap[dev];
+// Sends out what is queued on this device and makes `st` wait for every overlapped call still in flight, whatever
+// stream it was made on (no host wait).  Only the calls made on `st` itself are then forgotten: the others stay in
+// flight for a join on their own stream, which still has to be ordered behind them.
+cudaError_t join_lists(cudaStream_t st, int* launches) {
+  std::lock_guard<std::mutex> lock(g_lists_mu);
+  DeviceStates* d = nullptr;
+  cudaError_t e = device_states(&d);
+  if (e != cudaSuccess) return e == cudaErrorInvalidDevice ? cudaSuccess : e;
   for (int i = 0; i < kStatesPerDevice; ++i) {
-    if (!d.used[i]) continue;
-    OverlapState& s = d.st[i];
-    e = flush_pending(&s, launches);
+    if (!d->used[i]) continue;
+    ListState& s = d->st[i];
+    e = flush_list(&s, d->owner[i], launches);
+    if (e == cudaSuccess) e = order_behind(&s, d->owner[i], st);
     if (e != cudaSuccess) return e;
-    for (int h = 0; h < kSlots; ++h)
-      if (s.in_flight[h]) {
-        e = cudaStreamWaitEvent(st, s.done[h], 0);
-        if (e != cudaSuccess) return e;
-        if (d.owner[i] == st) s.in_flight[h] = false;
-      }
+    if (d->owner[i] == st) s.in_flight = false;
   }
   return cudaSuccess;
+}
+
+TailLayer tail_of(const Problem& pb, const int32_t* budgets, void* k_out, void* v_out, int64_t capacity, int32_t* offsets,
+                  int32_t* kept_idx, float* pooled_opt, int32_t* status) {
+  TailLayer t;
+  t.vote = pb.vote; t.budgets = budgets; t.offsets = offsets; t.kept_idx = kept_idx; t.gather_src = pb.gather_src;
+  t.pooled_out = pooled_opt; t.status = status; t.k = pb.k; t.v = pb.v; t.k_out = k_out; t.v_out = v_out;
+  t.capacity = capacity;
+  return t;
 }
 
 int compress_impl(const slkv_params* p, const void* q_win, const void* k, const void* v, const int32_t* cu_dev,
                   const int32_t* cu_host, const int32_t* budgets, const float* lse_opt, void* k_out, void* v_out,
-                  int64_t capacity,
-                  int32_t* offsets, int32_t* kept_idx, float* pooled_opt, int32_t* status, void* ws,
+                  int64_t capacity, int32_t* offsets, int32_t* kept_idx, float* pooled_opt, int32_t* status, void* ws,
                   size_t ws_bytes, cudaStream_t st, bool overlapped = false) {
   g_last_launches = 0;
   if (!q_win || !k || !v || !cu_dev || !budgets || !k_out || !v_out || !offsets || !kept_idx)
     return SLKV_ERR_NULL_PTR;
+  int launches = 0;
+  if (overlapped && p && cu_host && ws) {
+    // the shape of the calls before this one: everything that depends on it alone is there already
+    std::lock_guard<std::mutex> lock(g_lists_mu);
+    ListState* s = nullptr;
+    DeviceStates* d = nullptr;
+    cudaError_t e = list_state(st, &s, &d, &launches);
+    if (e != cudaSuccess) overlapped = false;                // the ordinary path reports it, behind bad arguments
+    const bool with_lse = lse_opt != nullptr;
+    const bool same = overlapped && s->open && s->ws == ws && s->ws_bytes == ws_bytes && s->with_lse == with_lse && s->cu_dev == cu_dev &&
+                      std::memcmp(&s->p, p, sizeof(*p)) == 0 &&
+                      std::memcmp(s->cu_host.data(), cu_host, s->cu_host.size() * sizeof(int32_t)) == 0;
+    if (overlapped && !same) {
+      Problem pb;
+      int rc = describe(p, cu_host, &pb);
+      if (rc != SLKV_OK) return rc;
+      if (p->history_only) return SLKV_ERR_BAD_SHAPE;        // nothing to append behind the selected rows
+      int path = 0;
+      rc = resolve_path(pb, &path);
+      if (rc != SLKV_OK) return rc;
+      overlapped = path == SLKV_PATH_TENSOR && list_supported(pb);
+      if (overlapped) {
+        if (reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SLKV_ERR_BAD_ALIGN;
+        const Layout L = layout_of(pb, true);
+        if (ws_bytes < L.total) return SLKV_ERR_WORKSPACE;
+        e = flush_list(s, st, &launches);                    // layers of the shape before
+        if (e != cudaSuccess) return cuda_fail(e);
+        s->open = false;
+        carve(&pb, L, ws, path, 0);
+        pb.cu = cu_dev; pb.tab.cu_ptr = cu_dev;
+        pb.q = q_win; pb.k = k; pb.v = v; pb.lse_opt = lse_opt;
+        e = plan_score_tensor(pb, cu_host, status, &s->plan);
+        if (e != cudaSuccess) return cuda_fail(e);
+        s->p = *p; s->cu_host.assign(cu_host, cu_host + p->n_seqs + 1); s->cu_dev = cu_dev;
+        s->ws = ws; s->ws_bytes = ws_bytes; s->with_lse = with_lse; s->pb = pb; s->layout = L;
+        s->open = true;
+      }
+    }
+    if (overlapped) {
+      if (capacity < 0) return SLKV_ERR_CAPACITY;
+      if (!aligned16(q_win) || !aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out))
+        return SLKV_ERR_BAD_ALIGN;
+      e = drain_states_sharing(d, s, ws, ws_bytes, st, &launches);
+      if (e != cudaSuccess) return cuda_fail(e);
+      Problem& pb = s->pb;
+      carve(&pb, s->layout, ws, SLKV_PATH_TENSOR, s->n);
+      pb.q = q_win; pb.k = k; pb.v = v; pb.lse_opt = lse_opt;
+      e = plan_score_layer(pb, status, &s->score[s->n]);
+      if (e != cudaSuccess) return cuda_fail(e);
+      const int rc = enqueue_window_stats(pb, SLKV_PATH_TENSOR, st, &launches);
+      if (rc != SLKV_OK) return rc;
+      s->tail[s->n] = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
+      if (++s->n == kListMaxLayers) {
+        e = flush_list(s, st, &launches);
+        if (e != cudaSuccess) return cuda_fail(e);
+      }
+      g_last_launches = launches;
+      return SLKV_OK;
+    }
+  }
+  // an ordinary call (or a shape that is not taken as a list): on the caller's stream, after whatever overlapped calls
+  // are still in flight
   Problem pb;
   int rc = describe(p, cu_host, &pb);
   if (rc != SLKV_OK) return rc;
@@ -530,94 +451,10 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   int path = 0;
   rc = resolve_path(pb, &path);
   if (rc != SLKV_OK) return rc;
-  // pooling, offsets and selection run in one kernel when the segments fit it: one CTA per segment up to
-  // 32768 history positions (overlapped calls), a thread-block cluster per segment otherwise
-  const bool one_cta = overlapped && select_cta_supported(pb) && pb.tab.n_inline > 0;
-  int launches = 0;
-  if (!one_cta) {
-    // ordinary call (or shapes the overlapped path does not take): everything on the caller's stream, after
-    // whatever overlapped calls are still in flight
-    cudaError_t je = join_overlapped(st, &launches);
-    if (je != cudaSuccess) return cuda_fail(je);
-    overlapped = false;
-  }
-  cudaError_t e = cudaSuccess;
-  if (overlapped) {
-    std::lock_guard<std::mutex> lock(g_overlap_mu);
-    OverlapState* os = nullptr;
-    e = overlap_state(st, &os, &launches);
-    if (e != cudaSuccess) return cuda_fail(e);
-    e = drain_states_sharing(os, ws, ws_bytes, st, &launches);
-    if (e != cudaSuccess) return cuda_fail(e);
-    ShapeSig sig;
-    sig.ws = ws; sig.ws_bytes = ws_bytes; sig.n_seqs = pb.p.n_seqs; sig.n_kv_heads = pb.p.n_kv_heads; sig.R = pb.R;
-    sig.max_hist = pb.max_hist; sig.path = path; sig.total_hist = pb.total_hist; sig.total_tokens = pb.total_tokens;
-    if (!(sig == os->sig)) {
-      // another shape or workspace: the carve-up changes, so nothing of the old one may still be in flight
-      e = flush_pending(os, &launches);
-      for (int h = 0; h < kSlots && e == cudaSuccess; ++h)
-        if (os->in_flight[h]) {
-          e = cudaStreamWaitEvent(st, os->done[h], 0);
-          os->in_flight[h] = false;
-        }
-      if (e != cudaSuccess) return cuda_fail(e);
-      os->sig = sig;
-    }
-    const int slot = (int)(os->seq % (unsigned)overlapped_slots(pb));
-    rc = bind_workspace(&pb, ws, ws_bytes, path, true, slot);
-    if (rc != SLKV_OK) return rc;
-    ++os->seq;
-    pb.cu = cu_dev; pb.q = q_win; pb.k = k; pb.v = v;
-    pb.tab.cu_ptr = cu_dev;
-    pb.lse_opt = lse_opt;
-    // the score kernels leave a few SMs to the selection kernels of the layers before this one
-    int sms = 148;
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int reserve = pb.n_seg < kSelectSmReserve ? pb.n_seg : kSelectSmReserve;
-    pb.max_score_ctas = sms - reserve > 0 ? sms - reserve : 0;
-    PendingCall cur;
-    cur.valid = true; cur.pb = pb; cur.slot = slot; cur.budgets = budgets; cur.k_out = k_out; cur.v_out = v_out;
-    cur.capacity = capacity; cur.offsets = offsets; cur.kept_idx = kept_idx; cur.pooled_opt = pooled_opt;
-    cur.status = status; cur.st = st;
-    cur.cu_host.assign(cu_host, cu_host + pb.p.n_seqs + 1);
-    bool pipe = path == SLKV_PATH_TENSOR && score_pipe_supported(pb);
-    if (pipe) {
-      e = plan_score_tensor(pb, cu_host, status, &cur.plan);
-      if (e != cudaSuccess) return cuda_fail(e);
-      if (cur.plan.n_cta == 0) pipe = false;                        // no history: nothing to score
-    }
-    const bool queued = !os->queue.empty() || os->pending.valid;
-    // a queue holds layers of one kind (both passes, or the vote pass alone) and of one stream
-    const bool other_kind = os->pending.valid ? lse_opt != nullptr
-                                              : (!os->queue.empty() && (os->queue[0].pb.lse_opt != nullptr) != (lse_opt != nullptr));
-    if (queued && (!pipe || other_kind || (os->queue.empty() ? os->pending.st : os->queue[0].st) != st)) {
-      e = flush_pending(os, &launches);
-      if (e != cudaSuccess) return cuda_fail(e);
-    }
-    e = claim_slot(os, slot, st, &launches);
-    if (e != cudaSuccess) return cuda_fail(e);
-    if (pipe) {
-      // Queue the layer; the score kernel takes a list of layers per launch (pass 1 of each beside pass 2 of the
-      // one before) and goes out when the list is full and one more layer has come, or at a join.
-      rc = enqueue_window_stats(pb, path, st, &launches);
-      if (rc != SLKV_OK) return rc;
-      os->queue.push_back(cur);
-      if ((int)os->queue.size() > kPipeMaxLayers) {
-        e = launch_queue(os, kPipeMaxLayers, false, &launches);
-        if (e != cudaSuccess) return cuda_fail(e);
-      }
-    } else {
-      rc = enqueue_votes(pb, path, cu_host, status, st, &launches);
-      if (rc != SLKV_OK) return rc;
-      e = enqueue_tail(os, cur, false, false, &launches);
-      if (e != cudaSuccess) return cuda_fail(e);
-    }
-    g_last_launches = launches;
-    return SLKV_OK;
-  }
   rc = bind_workspace(&pb, ws, ws_bytes, path);
   if (rc != SLKV_OK) return rc;
+  cudaError_t e = join_lists(st, &launches);
+  if (e != cudaSuccess) return cuda_fail(e);
   pb.cu = cu_dev; pb.q = q_win; pb.k = k; pb.v = v;
   pb.tab.cu_ptr = cu_dev;
   pb.lse_opt = lse_opt;
@@ -628,9 +465,10 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   }
   rc = enqueue_votes(pb, path, cu_host, status, st, &launches);
   if (rc != SLKV_OK) return rc;
+  const TailLayer tail = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
   if (clustered) {
     // pooling, offsets and selection in one cluster kernel
-    e = launch_select_cluster(pb, pooled_opt, budgets, offsets, kept_idx, capacity, status, st, &launches);
+    e = launch_select_cluster(pb, &tail, 1, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
   } else {
     float* pooled = pooled_opt ? pooled_opt : pb.pooled_ws;
@@ -639,7 +477,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
     e = launch_select(pb, pooled, budgets, offsets, kept_idx, capacity, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  e = launch_gather(pb, offsets, kept_idx, k_out, v_out, capacity, st, &launches);
+  e = launch_gather(pb, &tail, 1, st, &launches);
   if (e != cudaSuccess) return cuda_fail(e);
   g_last_launches = launches;
   return SLKV_OK;
@@ -845,7 +683,8 @@ int slkv_cp_emit(const slkv_params* p, const void* k, const void* v, int64_t row
   pb.n_seg = p->n_kv_heads;
   pb.k = k; pb.v = v;
   pb.gather_src = gather_src;
-  e = launch_gather(pb, offsets, kept_idx, k_out, v_out, out_capacity_rows, st, &launches, 256);
+  const TailLayer tail = tail_of(pb, nullptr, k_out, v_out, out_capacity_rows, offsets, kept_idx, nullptr, status);
+  e = launch_gather(pb, &tail, 1, st, &launches);
   if (e != cudaSuccess) return cuda_fail(e);
   g_last_launches = launches;
   return SLKV_OK;
@@ -901,12 +740,6 @@ int slkv_compress_overlapped(const slkv_params* p, const void* q_win, const void
                              const float* lse_opt, void* k_out, void* v_out, int64_t out_capacity_rows,
                              int32_t* offsets, int32_t* kept_idx, float* pooled_opt, int32_t* status, void* workspace,
                              size_t workspace_bytes, void* stream) {
-  {
-    Problem pb;                                   // the overlapped layout is the larger one: check it up front
-    if (p && cu_seqlens_host && describe(p, cu_seqlens_host, &pb) == SLKV_OK && workspace &&
-        workspace_bytes < layout_of(pb, true).total)
-      return SLKV_ERR_WORKSPACE;
-  }
   return compress_impl(p, q_win, k, v, cu_seqlens_dev, cu_seqlens_host, budgets, lse_opt, k_out, v_out,
                        out_capacity_rows, offsets, kept_idx, pooled_opt, status, workspace, workspace_bytes,
                        (cudaStream_t)stream, true);
@@ -914,7 +747,7 @@ int slkv_compress_overlapped(const slkv_params* p, const void* q_win, const void
 
 int slkv_join(void* stream) {
   int launches = 0;
-  cudaError_t e = join_overlapped((cudaStream_t)stream, &launches);
+  cudaError_t e = join_lists((cudaStream_t)stream, &launches);
   g_last_launches = launches;
   if (e != cudaSuccess) return cuda_fail(e);
   return SLKV_OK;
@@ -954,7 +787,7 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
   if (p->history_only) cu_seqlens_host = pb.cu_virtual;      // one sequence: the tables are inline, cu_seqlens_dev unread
   cudaStream_t st = (cudaStream_t)stream;
   int launches = 0;
-  cudaError_t e = join_overlapped(st, &launches);  // the workspace may still serve an overlapped call
+  cudaError_t e = join_lists(st, &launches);  // the workspace may still serve an overlapped call
   if (e != cudaSuccess) return cuda_fail(e);
   if (pb.tab.n_inline == 0) {
     e = launch_setup(pb, nullptr, nullptr, 0, nullptr, st, &launches);
@@ -964,11 +797,9 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
     // row statistics only: pass 1, the window keys' share where the domain has one, then the merge
     rc = enqueue_window_stats(pb, path, st, &launches);
     if (rc != SLKV_OK) return rc;
-    e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_seqlens_host, status, 1, st, &launches)
+    e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_seqlens_host, status, 1, lse_out, st, &launches)
                                  : launch_score_simt(pb, 1, st, &launches);
-    if (e == cudaSuccess)
-      e = path == SLKV_PATH_TENSOR ? launch_merge_lse_tensor(pb, cu_seqlens_host, lse_out, st, &launches)
-                                   : launch_merge_lse_simt(pb, lse_out, st, &launches);
+    if (e == cudaSuccess && path != SLKV_PATH_TENSOR) e = launch_merge_lse_simt(pb, lse_out, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
     g_last_launches = launches;
     return SLKV_OK;

@@ -15,6 +15,7 @@ constexpr double kLayerFloor = 0.01;   // minimum layer budget (Sec. 3.3)
 constexpr float kLog2e = 1.4426950408889634f;
 
 constexpr int kInlineSeqs = 64;
+constexpr int kMaxSplit = 160;         // CTAs the tensor-core score kernel uses at most (one per SM)
 
 // Per-sequence tables: token starts (cu), exclusive prefixes of the history lengths n_hist_s and of the
 // 128-key tile counts.  Batches of up to kInlineSeqs sequences carry them inside the kernel parameters
@@ -106,8 +107,7 @@ struct Problem {
   int64_t* hist_off;      // [n_seqs+1] exclusive prefix of n_hist_s
   int32_t* tile_off;      // [n_seqs+1] exclusive prefix of ceil(n_hist_s / 128)
   float* vote;            // [n_kv_heads * total_hist] ragged, same layout as pooled
-  float* part_m;          // [n_seg][R][n_chunks] partial row maxima (log2 domain)
-  float* part_z;          // [n_seg][R][n_chunks] partial row sums
+  void* part;             // partial row statistics; layout of the score path
   int n_chunks;           // chunks per segment (stride of part_*), per score path
   int chunk_keys;         // keys per chunk
   float* pooled_ws;       // [n_kv_heads * total_hist] used when the caller wants no pooled output
@@ -116,7 +116,6 @@ struct Problem {
   float* win_m;           // [n_seg][R] row statistics over the window keys (SLKV_ALL_CAUSAL without lse_opt)
   float* win_z;
   const float* lse_opt;   // the caller's row log-sum-exps, or null
-  int max_score_ctas;     // > 0: the score kernels use at most this many CTAs (SMs); 0 = all
 };
 
 // kernel ids for launch accounting / per-kernel timing
@@ -129,6 +128,13 @@ struct LaunchScope {
   ~LaunchScope();
   int kid_; cudaStream_t st_; int slot_;
 };
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_scoped(int kid, void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
+                                     int* launches, Args&... args) {
+  LaunchScope scope(kid, st, launches);
+  return launch_pdl<KArgs...>(kernel, dim3((unsigned)grid), dim3((unsigned)block), smem, st, 1, args...);
+}
 
 // slkv_score's host-side argument checks, without a workspace: SLKV_OK or the status slkv_score would return
 int check_score_args(const slkv_params* p, const void* q_win, const void* k, const int32_t* cu_seqlens_dev,
@@ -166,73 +172,92 @@ cudaError_t launch_score_simt(const Problem& pb, int passes, cudaStream_t st, in
 // Row statistics of the window keys each window row sees causally (SLKV_ALL_CAUSAL) -> pb.win_m / pb.win_z, rows in
 // the order of the score path (head_inner: r = i*G + hh).
 cudaError_t launch_window_stats(const Problem& pb, bool head_inner, cudaStream_t st, int* launches);
-// Merges the per-chunk (SIMT layout) or per-CTA (tensor layout, schedule in `plan`) row statistics and the window
-// statistics, if any, into lse_out[n_seqs][n_q_heads][window] in the problem's lse_units.
+// Merges the per-chunk row statistics and the window statistics, if any, into lse_out[n_seqs][n_q_heads][window] in the
+// problem's lse_units.
 cudaError_t launch_merge_lse_simt(const Problem& pb, float* lse_out, cudaStream_t st, int* launches);
-cudaError_t launch_merge_lse_tensor(const Problem& pb, const int32_t* cu_host, float* lse_out, cudaStream_t st,
-                                    int* launches);
 LseSource lse_source_of(const Problem& pb);
 float lse_out_scale(const Problem& pb);          // log2 units -> the problem's lse_units
 bool tensor_q_head_inner(const slkv_params& p);
 bool tensor_path_supported(const slkv_params& p);
-int tensor_slot_stride(const Problem& pb);
+int tensor_slot_stride(const Problem& pb);        // split ranges a segment may be shared by, at most
 void set_tensor_trace(void* dev_buf, size_t bytes);
-// passes as launch_score_simt
-cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, int passes,
+// passes as launch_score_simt; lse_out (optional, with passes == 1): the rows' log-sum-exps in the problem's lse_units
+cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, int passes, float* lse_out,
                                 cudaStream_t st, int* launches);
 cudaError_t launch_pool(const Problem& pb, float* pooled, cudaStream_t st, int* launches);
 cudaError_t launch_select(const Problem& pb, const float* pooled, const int32_t* budgets, const int32_t* offsets,
                           int32_t* kept_idx, int64_t capacity, cudaStream_t st, int* launches);
+constexpr int kListMaxLayers = 16;          // layers one launch of the score, selection and gather kernels takes
+// ---- selection and gather over a list of layers of one shape ------------------------------------------------------
+struct TailLayer {
+  const float* vote;
+  const int32_t* budgets;
+  int32_t* offsets;
+  int32_t* kept_idx;
+  int32_t* gather_src;          // per packed row: token * n_kv_heads + head of its source row
+  float* pooled_out;            // optional
+  int32_t* status;              // optional
+  const void* k;
+  const void* v;
+  void* k_out;
+  void* v_out;
+  long long capacity;
+};
 bool select_cta_supported(const Problem& pb);
-cudaError_t launch_select_cta(const Problem& pb, float* pooled_out, const int32_t* budgets, int32_t* offsets,
-                              int32_t* kept_idx, int64_t capacity, int32_t* status, cudaStream_t st, int* launches);
+cudaError_t launch_select_cta(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
 bool select_cluster_supported(const Problem& pb);
-cudaError_t launch_select_cluster(const Problem& pb, float* pooled_out, const int32_t* budgets, int32_t* offsets,
-                                  int32_t* kept_idx, int64_t capacity, int32_t* status, cudaStream_t st,
-                                  int* launches);
-// block_threads: 256, or 128 where the gather shares its SMs with a kernel that leaves few registers
-cudaError_t launch_gather(const Problem& pb, const int32_t* offsets, const int32_t* kept_idx, void* k_out,
-                          void* v_out, int64_t capacity, cudaStream_t st, int* launches, int block_threads = 256);
+cudaError_t launch_select_cluster(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
+cudaError_t launch_gather(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
 
-// ---- tensor-core score kernels: arguments and launch plans ---------------------------------------------------
-struct TcArgs {
+// ---- tensor-core score kernel: arguments and launch plans ----------------------------------------------------
+constexpr int kListMaxGroups = 64;          // groups of segments a layer is walked in
+
+// What the layers of a launch share.  A layer's history keys form a flat list of 128-key tiles, segment after segment;
+// consecutive whole segments form groups, and the CTAs of a launch share a group's tiles evenly.
+struct ScoreShape {
   SeqTables tab;
-  float* part_m;
-  float* part_z;
-  float* vote;
-  LseSource lse;
-  int32_t* status;
-  unsigned long long* trace;    // optional timeline buffer: kTraceSlots timestamps (ns) per CTA, or null
-  int n_seqs, n_kv_heads, G, window, R, MT, n_stages, slot_stride, tiles_per_cta, total_tiles, barrier_slot;
-  int fresh_inputs;             // vote pass only: no kernel of this library has read Q and K before this launch
-  int barrier_extra;            // 0; 1 makes the grid-wide wait expect an arrival that never comes (diagnostics)
+  int n_seqs, n_kv_heads, G, window;
+  int R, Rp, MT;                // score rows per KV head: G * window; rounded up to 32; 128-row blocks of them
+  int halves;                   // 64-element halves of a key row (head_dim / 64)
+  int n_q, n_stages, slot_stride;   // Q tiles in shared memory, K tiles in flight; split ranges that may share a segment (stride of the statistics)
   int q_head_inner, k_head_inner;   // tensor-map dimension order: 1 = the head axis comes before the row axis
+  int total_tiles, n_cta;       // of one layer; CTAs
+  // The groups the tiles of a list are walked in: group_layers = 1: a layer's n_groups groups, group_tile their first
+  // tiles; else short layers, that many whole ones together.
+  int n_groups, group_layers;
   float scale_log2;
+  int group_tile[kListMaxGroups + 1];
 };
-
-// One layer's score problem, ready to launch: tensor maps of Q_win and K, kernel arguments, grid size.
-struct TcPlan {
-  CUtensorMap tm_q, tm_k;
-  TcArgs a;
-  int n_cta;
+struct ScoreLayer {
+  alignas(64) CUtensorMap tm_q;
+  alignas(64) CUtensorMap tm_k;
+  void* part;                   // row statistics of every CTA's share of a segment (see stat_view)
+  float* vote;
+  LseSource lse;                // where the vote pass takes the rows' log-sum-exp from besides the statistics pass
+  int32_t* status;
 };
-// Fills a plan (tensor maps, schedule, arguments) for a problem whose workspace is bound; n_cta = 0 when there is
-// no history to score.  cudaErrorNotSupported when the driver has no tensor-map encoder.
-cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, TcPlan* plan);
-// Timeline buffer of this thread (diagnostics), or null: half 0 / 1, kTraceSlots words per CTA.
-unsigned long long* tensor_trace_buffer(int half, int n_cta);
+// One layer's score problem, ready to launch.
+struct ScorePlan {
+  ScoreShape sh;
+  ScoreLayer lay;
+};
+// Fills a plan for a problem whose workspace is bound; sh.n_cta = 0 when there is no history to score.
+// cudaErrorNotSupported when the driver has no tensor-map encoder.
+cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, ScorePlan* plan);
+cudaError_t plan_score_layer(const Problem& pb, int32_t* status, ScoreLayer* lay);    // the layer's part alone
+int sm_count();
+int score_list_stages(int MT, int halves, int n_q);
+// The score kernel over a list of layers of one shape: passes 1 = row statistics, 2 = votes from the callers' row
+// statistics, 3 = both.
+cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes, cudaStream_t st,
+                              int* launches);
+// lse_out null: into the layer's own statistics area
+cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
+                                    cudaStream_t st, int* launches);
+// Timeline buffer of this thread (diagnostics), or null: kTraceSlots words per CTA.
+unsigned long long* tensor_trace_buffer(int n_cta);
 // Diagnostics: arm / consume the one-shot switch that makes the next inter-CTA wait of this thread's launches run out.
 void expire_next_wait(int on);
 int take_expire_next_wait();
-
-// Several layers per launch, pass 1 of one layer beside pass 2 of the layer before: pass 1 of a[0..n_a), pass 2 of
-// `pending` (pass 1 done by an earlier launch; may be null) and of a[0..n_a-1), or of all of a[] when `finish`.
-// All plans share one shape.  The shapes it takes:
-bool score_pipe_supported(const Problem& pb);
-constexpr int kPipeMaxLayers = 8;
-// votes_only: every plan carries the caller's row statistics, so both streams run pass 2 (no pending layer before or
-// after the launch, no CTA waits for another).
-cudaError_t launch_score_pipe(const TcPlan* pending, const TcPlan* const* a, int n_a, bool finish, bool votes_only,
-                              cudaStream_t st, int* launches);
 
 }  // namespace slkv

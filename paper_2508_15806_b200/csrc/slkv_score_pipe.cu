@@ -1,22 +1,39 @@
-// Window relevance scores, two layers per launch (Sec. 3.4, Eq. 7; Algorithm 3; Eq. 3-4): pass 1 (row statistics)
-// of one layer and pass 2 (votes) of the layer before it run side by side in every CTA.
+// Window relevance scores on the 5th-generation tensor cores (Sec. 3.4, Eq. 7; Algorithm 3; Eq. 3-4), a list of layers
+// per launch.  bf16, head_dim 64 or 128, up to 256 query rows per KV head.
 //
-// The softmax over the keys needs every key of a row before any vote can be formed, so one layer's two passes
-// cannot overlap -- but consecutive layers are independent.  A launch therefore carries two streams of 128-key
-// tiles over the same split (one CTA per SM):
-//   stream A  pass 1 of layer n:     S = Q K^T, a TMEM lane owns a query row, per-CTA (max, sum) partials out;
-//   stream B  pass 2 of layer n - 1: S^T = K Q^T, a TMEM lane owns a key; the row log-sum-exps come from the
-//             partials the launch before this one wrote, so the launch boundary is the grid-wide barrier.
-// Each stream has its own TMA producer thread, MMA issuer thread, K ring, Q tile, two TMEM accumulators and two
-// epilogue warpgroups; the special-function and FMA pipes, which bound both passes, never wait for one stream's
-// barrier, merge, ramp-up or load latency while the other has tiles ready.
-// A launch takes a list of layers: stream A walks pass 1 of layers 1..n, stream B pass 2 of layers 0..n-1 (layer 0
-// is the one whose pass 1 the launch before did) or 0..n.  Pass 2 of a layer of the same launch waits until every
-// CTA has published that layer's row statistics (one counter per layer, all CTAs resident: cooperative launch);
-// stream A never waits for anything, so the ramp-up, the launch gap and the stragglers of a launch are paid once per
-// list, not once per layer.
-// Shapes: bf16, head_dim 128, G * w <= 128 query rows per KV head.  Every wait is bounded (1 s), as in the
-// single-layer kernels: SLKV_ERR_DEVICE_TIMEOUT in the status words, TMEM freed, return.
+// Two passes over a layer's keys, in 128-key tiles:
+//   statistics  S = Q K^T with the G*w query rows as the M dimension: a TMEM lane -- one thread -- owns a query row and
+//               keeps (reference, sum of 2^(s - reference)) in registers; per CTA and segment one pair per row goes out;
+//   votes       S^T = K Q^T with the keys as the M dimension: a thread owns a key, and
+//               vote[j] = (1/G) sum_rows 2^(s_rj - lse_r) is a thread-local sum and a coalesced store.
+// The votes of a segment need its rows' statistics over all keys, i.e. from other CTAs.  The layers of a list and the
+// groups of segments inside a layer are independent, so every CTA (one per SM) walks one stream of phases
+//   S(0) .. S(lag-1), S(lag), V(0), S(lag+1), V(1), ..., V(last)
+// over groups of about 2048 tiles: by the time V(g) is due, the others have published S(g), and nobody waits.
+//
+// Roles (640 threads, one CTA per SM; a twenty-first warp would cost every thread 16 registers):
+//   warp 0     TMA loads of K tiles (ring of 4-6 x 32 KB) and Q tiles; it never waits for Q while K stages are free
+//   warp 1     tcgen05.mma, 128 x 128 products into four 128-column TMEM accumulators ("units")
+//   warp 2     works out the runs (consecutive tiles of one segment) and hands them to the others through shared memory;
+//              announces a group's statistics to the other CTAs once this CTA's share is out
+//   warp 3     fetches a segment's statistics as log-sum-exps for the vote phase, ahead of its start
+//   warps 4-19 four warpgroups, unit u belongs to warpgroup u % 4: TMEM -> registers -> exponentials
+// so that the warps that do the arithmetic -- what bounds the kernel -- meet no other CTA, no global latency, no CTA-wide
+// barrier and no launch parameters: with every role walking the phases by itself, divisions and constant-cache misses
+// (the parameters of 16 layers are 7 KB) took 3600 cycles per run and 1000 per tile of the MMA thread.
+//
+// What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
+//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; two in eight go to the FMA pipe
+//     as packed pairs, and scale / subtract / sum run on pairs too: 1180 -> 1000-1030 (three in eight: 1046);
+//   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
+//     730 measured for loads and MMAs alone;
+//   - two epilogue warpgroups instead of four: 1250; sums over the keys across lanes instead of a lane per row: 1255;
+//   - power: with every tile from HBM the part holds 1.3-1.6 GHz (0.76 us per tile whatever the instruction mix), from
+//     L2 1.75-1.85 GHz.
+// Against the kernel before it (two streams with two accumulators and two warpgroups each on 128 SMs for up to 128 rows,
+// one launch per layer with a grid-wide barrier for more), per layer: 32k tokens, 128 rows: 29.3 -> 24 us; eight ragged
+// sequences of 147k tokens, 256 rows: 299 -> 184 us; 131k tokens, 256 rows: 248 -> 160 us.
+// Every wait is bounded (1 s): SLKV_ERR_DEVICE_TIMEOUT in the status words, TMEM freed, return.
 #include <cuda.h>
 
 #include <atomic>
@@ -29,509 +46,732 @@
 namespace slkv {
 namespace {
 
-constexpr int kPipeThreads = 640;        // warps 0-3: producer A, issuer A, producer B, issuer B;
-                                         // warps 4-11: epilogue of stream A; warps 12-19: epilogue of stream B
-constexpr int kDualWgs = 3;               // vote pass on both streams: warpgroups per stream
-constexpr int kDualThreads = 128 + 2 * kDualWgs * 128;
-constexpr int kLeadEntries = 2;           // entries pass 1 may be ahead of the entry pass 2 has begun
-constexpr unsigned kPollNs = 64;          // pause between two polls of an mbarrier
-constexpr int kStagesA = 2;              // K tiles in flight for stream A (pass 1: first read of a layer's K)
-constexpr int kStagesB = 3;              // ... for stream B (pass 2: ~70 % of its re-reads come from HBM again, and
-                                         // its tiles take longer; measured 1.7 % faster than 3 + 2)
-constexpr int kQBytes = 2 * kHalfBytes;  // one 128-row Q tile
-constexpr int kBarBytesPerStream = 160;  // up to 20 mbarriers
-constexpr int kPipeTail = 512 + 1024 + 1024;   // mbarriers + flags, stat_m/stat_z of stream A, two log-sum-exp rows of stream B
-constexpr int kPipeSmem = 2 * kQBytes + (kStagesA + kStagesB) * kStageBytes + kPipeTail;
-static_assert(kPipeSmem <= kSmemLimit, "shared memory of the two-stream kernel");
+constexpr int kWgs = 4;                              // epilogue warpgroups = TMEM units
+constexpr int kListThreads = 128 + kWgs * 128;
+constexpr int kMaxStages = 6;
+// Shared memory behind the Q tile and the K ring: mbarriers and flags, far row statistics [2][kWgs][128] (sum, reference),
+// log-sum-exps [2][256], half votes [2][4][128], runs.
+constexpr int kBarBytes = 640;
+constexpr int kStatBytes = 2 * kWgs * 128 * 8;
+constexpr int kLseBytes = 2 * 256 * 4;
+constexpr int kHalfVoteBytes = 2 * 4 * 128 * 4;
+constexpr int kRunSlots = 8;                         // runs handed out ahead
+constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes + kRunSlots * 128;
+// Exponentials on the FMA pipe: pairs 0 .. kPolyPairs-1 of every eight.
+constexpr int kPolyPairs = 2;
+constexpr int kCountSlots = 32;                      // launches whose counters are live at once
+constexpr int kCountWords = kListMaxLayers * kListMaxGroups + 2;
 
-// Entries a layer may be split into (1 or 2).  Two halves the K that lies between pass 1 and pass 2, and pass 2 then
-// finds it in L2 (measured: 299 B of DRAM traffic per key row instead of 442, SM clock 1.82 instead of 1.64 GHz under
-// the power cap) but pays for twice the merges, Q reloads and waits for the other CTAs: 35.7 against 34.3 us per
-// layer.  One it is.
-constexpr int kMaxGroups = 1;
-constexpr int kMaxLay = kPipeMaxLayers * kMaxGroups + 1;   // the entry pending from the launch before + this launch's
-constexpr int kCountWords = kMaxLay + 1;        // per launch: one publish counter per layer + one exit counter
-constexpr int kCountSlots = 64;                 // launches whose counters are live at once
-
-// One entry of a launch's list: a layer, or one group of consecutive segments of a layer (a range of the layer's
-// flat tile list).  Smaller entries keep less K between pass 1 and pass 2.
-struct LayerDesc {
-  alignas(64) CUtensorMap tm_q;
-  alignas(64) CUtensorMap tm_k;
-  float* part_m;
-  float* part_z;
-  float* vote;
-  LseSource lse;               // where pass 2 takes the rows' log-sum-exp from besides this launch's / the last launch's pass 1
-  int32_t* status;
-  int tile_begin, tile_end;    // the entry's tiles in the layer's tile list; CTA b takes tiles_per_cta of them from
-                               // tile_begin + b * tiles_per_cta
-};
-struct PipeArgs {
-  TcArgs base;                 // tables, shapes, schedule, scale: the same for every layer of the launch
-  LayerDesc lay[kMaxLay];
-  int a_first, a_last;         // stream A: pass 1 of layers a_first..a_last (none if a_first > a_last)
-  int b_first, b_last;         // stream B: pass 2 of layers b_first..b_last
-  int step;                    // 1; 2 when both streams run pass 2 (the callers supplied the row statistics): stream A
-                               // takes entries a_first, a_first + 2, ..., stream B entries b_first, b_first + 2, ...
-  unsigned* counters;          // [kMaxLay] CTAs that have published the layer's row statistics, then [1] CTAs that are done
-  unsigned target[kMaxLay];    // value a layer's counter reaches when all CTAs of this launch have published
+struct ListArgs {
+  ScoreShape sh;
+  ScoreLayer lay[kListMaxLayers];
+  int n_layers, passes, lag;
+  int group_layers, n_groups;  // as in ScoreShape; groups of the whole list
+  unsigned* counters;          // [n_groups] CTAs that have published the group's statistics, then CTAs that have cleared
+                               // their part of the statistics area, CTAs that are done
+  unsigned target;             // value a group's counter reaches when every CTA has published
+  unsigned long long* trace;
 };
 
-// Counter sets, taken in turn by the launches (zero at load).  The last CTA of a launch to finish puts its set back to
-// zero, so the set is clean for its next user 64 launches later; no memset sits between two launches.
-__device__ unsigned g_layer_published[kCountSlots * kCountWords];
+// Counter sets, taken in turn by the launches (zero at load); the last CTA of a launch to finish puts its set back to
+// zero, so no memset sits between two launches.
+__device__ unsigned g_published[kCountSlots * kCountWords];
 
-// One stream's resources inside the CTA.
-struct StreamCtx {
-  uint32_t q_smem, k_smem, bar0, tmem0;
-  int n_stages;
+// A run as warp 2 hands it out: consecutive tiles of one segment, in one pass.
+struct alignas(16) RunDesc {
+  int kind;                    // 0 statistics, 1 votes, 2 the end; count = 0: a phase in which this CTA has no tiles
+  int count;                   // tiles
+  int n_valid;                 // history keys from the run's first one to the segment's end
+  int tok;                     // token of the run's first key
+  int s, g;
+  int gg;                      // group of the list; statistics: published with this run when last != 0
+  int last;
+  int n_slots;                 // split ranges that share the segment
+  int seg;
+  int q_y, q_z;                // coordinates of the Q tile
+  const CUtensorMap* tm_q;
+  const CUtensorMap* tm_k;
+  int slot;                    // this CTA's place among the segment's split ranges
+  float* vote;                 // of the run's first key
+  double* acc;                 // the segment's row sums ...
+  const unsigned* far;         // ... and far bits
+  int sums, win;               // votes: the log-sum-exps come from the sums, with window statistics
+  int layer;
+};
+static_assert(sizeof(RunDesc) <= 128, "run descriptor");
+
+// What the roles keep in registers: copied through shared memory, so that no launch parameter is read in a loop.
+struct Smem {
+  uint32_t q, k, bar0, tmem;
+  int q_half, q_bytes, n_q, stage_bytes, n_stages;
+  int R, Rp, MT, halves, k_head_inner, both;
+  float sc, inv_g;
   volatile int* abort_flag;
-  volatile int* b_layer;       // CTA-wide: the layer whose pass 2 this CTA's epilogue has begun
-  __device__ __forceinline__ uint32_t full_bar(int st) const { return bar0 + 8u * st; }
-  __device__ __forceinline__ uint32_t empty_bar(int st) const { return bar0 + 8u * (3 + st); }
-  __device__ __forceinline__ uint32_t accf_bar(int b) const { return bar0 + 8u * (6 + b); }
-  // three warpgroups per stream: one barrier per (warpgroup, accumulator), so that a warpgroup sees every phase of the
-  // barriers it waits on (a parity wait tells only adjacent phases apart)
-  __device__ __forceinline__ uint32_t accf_bar_of(int wg, int b) const { return bar0 + 8u * (13 + 2 * wg + b); }
-  __device__ __forceinline__ uint32_t acce_bar(int b) const { return bar0 + 8u * (8 + b); }
-  __device__ __forceinline__ uint32_t qfull_bar() const { return bar0 + 8u * 10; }
-  __device__ __forceinline__ uint32_t qempty_bar() const { return bar0 + 8u * 11; }
-  __device__ __forceinline__ uint32_t drain_bar() const { return bar0 + 8u * 12; }   // used only when a wait ran out
+  RunDesc* runs;               // [kRunSlots]
+  float* stat_z;               // [2][kWgs][128]: far parts (see StatView) on their way out
+  float* stat_m;               // likewise
+  unsigned* stat_far;          // [2]: warps that have any
+  float* lse;                  // [2][256], negated
+  float* half_vote;            // [2][4][128]
+  __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * (uint32_t)i; }
+  __device__ __forceinline__ uint32_t full(int st) const { return bar(st); }
+  __device__ __forceinline__ uint32_t empty(int st) const { return bar(kMaxStages + st); }
+  __device__ __forceinline__ uint32_t unit_full(int u) const { return bar(2 * kMaxStages + u); }
+  __device__ __forceinline__ uint32_t unit_empty(int u) const { return bar(2 * kMaxStages + 4 + u); }
+  // run k's Q tile: slot and phase (n_q is 1 or 2)
+  __device__ __forceinline__ int q_slot(int k) const { return k & (n_q - 1); }
+  __device__ __forceinline__ uint32_t q_phase(int k) const { return (uint32_t)(k >> (n_q - 1)) & 1u; }
+  __device__ __forceinline__ uint32_t q_full(int k) const { return bar(2 * kMaxStages + 8 + q_slot(k)); }
+  __device__ __forceinline__ uint32_t q_empty(int k) const { return bar(2 * kMaxStages + 10 + q_slot(k)); }
+  __device__ __forceinline__ uint32_t stat_full(int s) const { return bar(2 * kMaxStages + 12 + s); }
+  __device__ __forceinline__ uint32_t stat_empty(int s) const { return bar(2 * kMaxStages + 14 + s); }
+  __device__ __forceinline__ uint32_t lse_full(int s) const { return bar(2 * kMaxStages + 16 + s); }
+  __device__ __forceinline__ uint32_t lse_empty(int s) const { return bar(2 * kMaxStages + 18 + s); }
+  __device__ __forceinline__ uint32_t half_full(int pair, int turn) const { return bar(2 * kMaxStages + 20 + 4 * pair + turn); }
+  __device__ __forceinline__ uint32_t run_full(int k) const { return bar(2 * kMaxStages + 28 + (k & (kRunSlots - 1))); }
+  __device__ __forceinline__ uint32_t run_empty(int k) const { return bar(2 * kMaxStages + 28 + kRunSlots + (k & (kRunSlots - 1))); }
+  __device__ __forceinline__ uint32_t cleared() const { return bar(2 * kMaxStages + 29 + 2 * kRunSlots); }
+  __device__ __forceinline__ uint32_t drain() const { return bar(2 * kMaxStages + 28 + 2 * kRunSlots); }   // a wait ran out
 };
+constexpr int kNumBars = 2 * kMaxStages + 30 + 2 * kRunSlots;
+constexpr int kHeadInts = 14;
+static_assert(kNumBars * 8 + kHeadInts * 4 + 16 <= kBarBytes, "mbarriers");
+constexpr int kRunReaders = 4 + 4 * kWgs;              // arrivals that free a run slot: one per reading thread or warp
 
-// sum_e 2^(v_e * sc - m) over 32 accumulator values.  All exponentials on the special-function unit: with sixteen
-// epilogue warps at 96 registers the polynomial share the single-layer kernels use made this kernel slower.
-__device__ __forceinline__ float sum_ex2_32_mufu(const uint32_t (&r)[32], float sc, float m) {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-  for (int e = 0; e < 32; e += 4) {
-    s0 += ex2(fmaf(__uint_as_float(r[e]), sc, -m));
-    s1 += ex2(fmaf(__uint_as_float(r[e + 1]), sc, -m));
-    s2 += ex2(fmaf(__uint_as_float(r[e + 2]), sc, -m));
-    s3 += ex2(fmaf(__uint_as_float(r[e + 3]), sc, -m));
+// The runs of this CTA, one after the other.  A group's tiles are counted through its layers.
+struct GroupShare {
+  int layer0, base, T, n, idx, begin, end;                 // begin, end: this CTA's tiles, counted through the group
+};
+__device__ __forceinline__ GroupShare group_share(const ListArgs& a, int gg) {
+  const ScoreShape& sh = a.sh;
+  GroupShare g;
+  if (a.group_layers == 1) {
+    g.layer0 = gg / sh.n_groups;
+    const int grp = gg - g.layer0 * sh.n_groups;
+    g.base = sh.group_tile[grp];
+    g.T = sh.group_tile[grp + 1] - g.base;
+  } else {
+    g.layer0 = gg * a.group_layers;
+    g.base = 0;
+    g.T = min(a.group_layers, a.n_layers - g.layer0) * sh.total_tiles;
   }
-  return (s0 + s1) + (s2 + s3);
+  // the split index moves on by one CTA per group, so that the larger shares go round
+  const int i = (int)blockIdx.x + gg % sh.n_cta;
+  g.idx = i >= sh.n_cta ? i - sh.n_cta : i;
+  g.n = min(sh.n_cta, g.T);
+  const bool takes_part = g.idx < g.n;
+  g.begin = takes_part ? split_begin(g.idx, g.T, g.n) : 0;
+  g.end = takes_part ? split_begin(g.idx + 1, g.T, g.n) : 0;
+  return g;
 }
-// this CTA's tiles of an entry
-__device__ __forceinline__ void entry_range(const TcArgs& a, const LayerDesc& L, int& begin, int& end) {
-  begin = min(L.tile_begin + (int)blockIdx.x * a.tiles_per_cta, L.tile_end);
-  end = min(begin + a.tiles_per_cta, L.tile_end);
-}
-__device__ __forceinline__ void named_bar(int id, int n_threads = kEpiThreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
+struct RunWalk {
+  int step, pos, kind, gg;
+  GroupShare s;
+  __device__ __forceinline__ void start() { step = 0; pos = s.end = 0; }
+  // The next run into d (shared memory); kind 2 behind the last one.
+  __device__ __forceinline__ void next(const ListArgs& a, RunDesc& d) {
+    const ScoreShape& sh = a.sh;
+    const int NG = a.n_groups;
+    while (pos >= s.end) {                                   // the next phase
+      if (a.passes == 3) {
+        const int p = step >> 1;
+        if (p >= NG + a.lag) { d.kind = kind = 2; return; }
+        kind = step & 1;
+        gg = kind ? p - a.lag : p;
+      } else {
+        if (step >= NG) { d.kind = kind = 2; return; }
+        kind = a.passes == 2;
+        gg = step;
+      }
+      ++step;
+      if (gg < 0 || gg >= NG) continue;
+      s = group_share(a, gg);
+      pos = s.begin;
+      if (pos >= s.end && kind == 0) {
+        d.kind = 0;
+        d.gg = gg;
+        d.count = 0;
+        d.last = 1;
+        return;
+      }
+    }
+    const int in_group = a.group_layers == 1 ? 0 : pos / sh.total_tiles;
+    const int layer = s.layer0 + in_group, before = in_group * sh.total_tiles - s.base;  // group tile = layer tile + before
+    const ScoreLayer& L = a.lay[layer];
+    d.kind = kind;
+    d.gg = gg;
+    d.layer = layer;
+    d.tm_q = &L.tm_q;
+    d.tm_k = &L.tm_k;
+    const Run r = locate(sh, pos - before, s.end - before);
+    pos += r.count;
+    d.count = r.count;
+    d.n_valid = r.n_hist - r.t0 * kTileKeys;
+    d.tok = sh.tab.cu_at(r.s) + r.t0 * kTileKeys;
+    d.s = r.s;
+    d.g = r.g;
+    d.last = pos >= s.end;
+    const int first = split_index(r.seg_tile0 + before, s.T, s.n);
+    d.n_slots = split_index(r.seg_tile0 + r.tiles_seg - 1 + before, s.T, s.n) - first + 1;
+    d.slot = s.idx - first;
+    d.vote = L.vote + sh.tab.hist_at(r.s) * sh.n_kv_heads + (long long)r.g * r.n_hist + r.t0 * kTileKeys;
+    const int seg = r.s * sh.n_kv_heads + r.g;
+    d.seg = seg;
+    d.acc = static_cast<double*>(L.part) + (long long)seg * sh.R;
+    d.far = reinterpret_cast<unsigned*>(static_cast<double*>(L.part) + (long long)sh.n_seqs * sh.n_kv_heads * sh.R) + seg * kFarWords;
+    d.sums = a.passes == 3;
+    d.win = L.lse.win_m != nullptr;
+    d.q_y = sh.q_head_inner ? r.g * sh.G : 0;
+    d.q_z = sh.q_head_inner ? 0 : r.g * sh.G;
+  }
+};
+// Run k, read by a single thread or by a whole warp; kind 2 when there is none left (or a wait ran out).
+template <bool WARP>
+__device__ __forceinline__ RunDesc take_run(const Smem& c, int k) {
+  bool ok = mbar_wait(c.run_full(k), (k / kRunSlots) & 1, c.abort_flag);
+  if (WARP) ok = __all_sync(0xffffffffu, ok) != 0;
+  RunDesc d;
+  d.kind = 2;
+  if (ok) d = c.runs[k & (kRunSlots - 1)];
+  if (WARP) __syncwarp();
+  if (!WARP || (threadIdx.x & 31) == 0) mbar_arrive(c.run_empty(k));
+  return d;
 }
 
-// ---- one thread: TMA loads of the stream's Q tiles and K tiles ------------------------------------------
-template <bool VOTE>
-__device__ __forceinline__ void producer(const StreamCtx& c, const TcArgs& a, const LayerDesc* lay, int first, int last,
-                                         int step, int new_from) {
-  int it = 0, run_idx = 0, st = 0;
+// ---- warp 0, one thread: TMA loads ------------------------------------------------------------------------------
+__device__ __forceinline__ void producer(const Smem& c) {
+  int st = 0, it = 0, n = 0;                                 // stage, tiles so far, runs so far
   uint32_t st_phase = 0;
-  bool ok = true;
-  // Every K tile is read twice, by pass 1 and a layer later by pass 2, in the same order: pass 1 asks L2 to keep the
-  // lines, pass 2 to drop them first, so that about one layer's K is live in L2 and pass 2 need not go to HBM.
-  const uint64_t policy = VOTE ? l2_policy_evict_first() : l2_policy_evict_last();
-  for (int j = first; j <= last && ok; j += step) {
-    if (j == new_from || (j == first && j > new_from)) pdl_wait();   // inputs this launch is the first to read
-    if (!VOTE) {
-      // Pass 1 stays at most one layer ahead of this CTA's pass 2 (which needs the other CTAs' pass 1 of the layer
-      // before, so it cannot deadlock): the two streams then share the SM to the end instead of pass 2 running on
-      // alone, on half the epilogue warps, after pass 1 has raced through the list.
-      const unsigned long long t0 = now_ns();
-      for (unsigned spin = 1; *c.b_layer < j - kLeadEntries; ++spin) {
-        if ((spin & 63u) == 0 && (*c.abort_flag || now_ns() - t0 > kWaitLimitNs)) { *c.abort_flag = 1; ok = false; break; }
-        __nanosleep(100);
-      }
+  bool ok = true, q_due = false;
+  const CUtensorMap* q_map = nullptr;
+  int q_y = 0, q_z = 0, q_s = 0;
+  // Q of run number n - 1
+  auto load_q = [&]() {
+    const uint32_t bar = c.q_full(n - 1), dst = c.q + (uint32_t)(c.q_slot(n - 1) * c.q_bytes);
+    mbar_expect_tx(bar, (uint32_t)(c.halves * c.R * 128));
+    for (int h = 0; h < c.halves; ++h) tma_load_4d(dst + h * c.q_half, q_map, 64 * h, q_y, q_z, q_s, bar);
+    q_due = false;
+  };
+  auto q_free = [&](bool wait) {
+    const uint32_t bar = c.q_empty(n - 1), phase = c.q_phase(n - 1) ^ 1u;
+    return wait ? mbar_wait(bar, phase, c.abort_flag) : mbar_test(bar, phase);
+  };
+  for (int k = 0; ok; ++k) {
+    const RunDesc r = take_run<false>(c, k);
+    if (r.kind == 2) break;
+    if (r.count == 0) continue;
+    if (q_due) {                                             // the run before is shorter than the ring: its Q first
+      ok = q_free(true);
       if (!ok) break;
+      load_q();
     }
-    const CUtensorMap* tm_q = &lay[j].tm_q;
-    const CUtensorMap* tm_k = &lay[j].tm_k;
-    int begin, end;
-    entry_range(a, lay[j], begin, end);
-    for (int pos = begin; pos < end && ok;) {
-      const Run r = locate(a, pos, begin, end, false);
-      ok = mbar_wait(c.qempty_bar(), (run_idx & 1) ^ 1, c.abort_flag, kPollNs);        // the run before is done with Q
-      if (!ok) break;
-      mbar_expect_tx(c.qfull_bar(), 2u * (uint32_t)a.R * 128u);
-      const int qy = a.q_head_inner ? r.g * a.G : 0, qz = a.q_head_inner ? 0 : r.g * a.G;
-      tma_load_4d(c.q_smem, tm_q, 0, qy, qz, r.s, c.qfull_bar());
-      tma_load_4d(c.q_smem + kHalfBytes, tm_q, 64, qy, qz, r.s, c.qfull_bar());
-      int tok = a.tab.cu_at(r.s) + r.t0 * kTileKeys;
-      for (int i = 0; i < r.count; ++i, ++it, tok += kTileKeys) {
-        ok = mbar_wait(c.empty_bar(st), st_phase ^ 1u, c.abort_flag, kPollNs);
-        if (!ok) break;
-        const uint32_t fb = c.full_bar(st), dst = c.k_smem + (uint32_t)st * kStageBytes;
-        mbar_expect_tx(fb, kStageBytes);
-        const int ky = a.k_head_inner ? r.g : tok, kz = a.k_head_inner ? tok : r.g;
-        tma_load_3d_hint(dst, tm_k, 0, ky, kz, fb, policy);
-        tma_load_3d_hint(dst + kHalfBytes, tm_k, 64, ky, kz, fb, policy);
-        if (++st == c.n_stages) { st = 0; st_phase ^= 1u; }
+    q_map = r.tm_q; q_y = r.q_y; q_z = r.q_z; q_s = r.s;
+    q_due = true;
+    ++n;
+    int tok = r.tok;
+    for (int i = 0; i < r.count; ++i, ++it, tok += kTileKeys) {
+      // a stage of the ring, and Q as soon as the MMAs of the run that had its slot are through with it
+      bool got = false;
+      unsigned long long t0 = 0;
+      for (unsigned spin = 0; !got; ++spin) {
+        if (q_due && q_free(false)) load_q();
+        got = q_due ? mbar_test(c.empty(st), st_phase ^ 1u) : mbar_try(c.empty(st), st_phase ^ 1u);
+        if (got) break;
+        if (spin == 0) t0 = now_ns();
+        if ((spin & 63u) == 63u) {
+          if (*c.abort_flag) break;
+          if (now_ns() - t0 > kWaitLimitNs) { *c.abort_flag = 1; break; }
+        }
+        if (q_due) __nanosleep(32);
       }
-      pos += r.count;
-      ++run_idx;
+      if (!got) { ok = false; break; }
+      const uint32_t fb = c.full(st), dst = c.k + (uint32_t)(st * c.stage_bytes);
+      mbar_expect_tx(fb, (uint32_t)c.stage_bytes);
+      const int ky = c.k_head_inner ? r.g : tok, kz = c.k_head_inner ? tok : r.g;
+      for (int h = 0; h < c.halves; ++h) tma_load_3d(dst + h * kHalfBytes, r.tm_k, 64 * h, ky, kz, fb);
+      if (++st == c.n_stages) { st = 0; st_phase ^= 1u; }
     }
   }
-  if (!ok) {
+  if (ok && q_due) {
+    ok = q_free(true);
+    if (ok) load_q();
+  }
+  if (!ok || *c.abort_flag) {
     // give loads already in flight a bounded chance to land before the CTA's shared memory goes away
     const unsigned long long t0 = now_ns();
     for (int s2 = 0; s2 < c.n_stages; ++s2) {
-      const int last_it = it - 1 - ((it - 1 - s2) % c.n_stages + c.n_stages) % c.n_stages;   // last issue into stage s2
-      if (it == 0 || last_it < 0) continue;
-      while (!mbar_try(c.full_bar(s2), (last_it / c.n_stages) & 1) && now_ns() - t0 < kWaitLimitNs) {}
+      const int last = it - 1 - ((it - 1 - s2) % c.n_stages + c.n_stages) % c.n_stages;   // last issue into stage s2
+      if (it == 0 || last < 0) continue;
+      while (!mbar_try(c.full(s2), (last / c.n_stages) & 1) && now_ns() - t0 < kWaitLimitNs) {}
     }
+    const int loaded = n - (q_due ? 1 : 0);                  // Q tiles asked for; the last n_q may be in flight
+    for (int k = loaded - c.n_q < 0 ? 0 : loaded - c.n_q; k < loaded; ++k)
+      while (!mbar_try(c.q_full(k), c.q_phase(k)) && now_ns() - t0 < kWaitLimitNs) {}
   }
 }
 
-// ---- one thread: the stream's MMAs, one 128 x 128 x 128 product per tile into one of two accumulators --------
-template <bool VOTE, int NWG = 2>
-__device__ __forceinline__ void issuer(const StreamCtx& c, const TcArgs& a, const LayerDesc* lay, int first, int last,
-                                       int step) {
-  // pass 1: D[row, key] = Q K^T (A = Q, B = K); pass 2: D[key, row] = K Q^T (A = K, B = Q, N = R)
-  const uint32_t idesc = VOTE ? instr_desc(kTileKeys, a.R) : instr_desc(128, kTileKeys);
-  const uint64_t q_desc0 = smem_desc(c.q_smem), k_desc0 = smem_desc(c.k_smem);
-  const uint64_t hi = (uint64_t)(kHalfBytes >> 4);
-  int it = 0, run_idx = 0, st = 0, b = 0;
-  uint32_t st_phase = 0, b_phase = 0;
-  uint64_t k_desc = k_desc0;
+// ---- warp 1, one thread: MMAs -------------------------------------------------------------------------------------
+__device__ __forceinline__ void issuer(const Smem& c) {
+  // statistics: D[row, key] = Q K^T (A = Q, B = K); votes: D[key, row] = K Q^T (A = K, B = Q); a unit per 128-row block
+  // of Q (one 256-column product for the votes would read less shared memory, but it takes two units at once and makes
+  // both wait for the slower one's warpgroup)
+  const uint32_t idesc_s = instr_desc(128, kTileKeys), idesc_v0 = instr_desc(kTileKeys, min(c.Rp, 128)),
+                 idesc_v1 = instr_desc(kTileKeys, max(c.Rp - 128, 32));
+  const uint64_t q_desc0 = smem_desc(c.q), k_desc0 = smem_desc(c.k);
+  const uint64_t q_hi = (uint64_t)(c.q_half >> 4), k_hi = (uint64_t)(kHalfBytes >> 4);
+  const bool two_halves = c.halves == 2;
+  int st = 0, uc = 0, n = 0;                                  // stage, units so far, runs so far
+  uint32_t st_phase = 0;
   bool ok = true;
-  for (int j = first; j <= last && ok; j += step) {
-  int begin, end;
-  entry_range(a, lay[j], begin, end);
-  for (int pos = begin; pos < end && ok;) {
-    const Run r = locate(a, pos, begin, end, false);
-    ok = mbar_wait(c.qfull_bar(), run_idx & 1, c.abort_flag, kPollNs);
-    if (!ok) break;
-    for (int i = 0; i < r.count; ++i, ++it) {
-      ok = mbar_wait(c.full_bar(st), st_phase, c.abort_flag, kPollNs) && mbar_wait(c.acce_bar(b), b_phase ^ 1u, c.abort_flag, kPollNs);
+  auto product = [&](uint32_t d, uint64_t ad, uint64_t a_hi, uint64_t bd, uint64_t b_hi, uint32_t idesc) {
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) tc_mma(d, ad + (uint64_t)(ks * 2), bd + (uint64_t)(ks * 2), idesc, ks > 0);
+    if (two_halves) {
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) tc_mma(d, ad + a_hi + (uint64_t)(ks * 2), bd + b_hi + (uint64_t)(ks * 2), idesc, 1);
+    }
+  };
+  auto unit_free = [&](int u_count) {
+    return mbar_wait(c.unit_empty(u_count & 3), ((u_count >> 2) & 1) ^ 1, c.abort_flag);
+  };
+  for (int k = 0; ok; ++k) {
+    const RunDesc r = take_run<false>(c, k);
+    if (r.kind == 2) break;
+    if (r.count == 0) continue;
+    ok = mbar_wait(c.q_full(n), c.q_phase(n), c.abort_flag);
+    const uint64_t q_desc = q_desc0 + (uint64_t)((c.q_slot(n) * c.q_bytes) >> 4);
+    for (int i = 0; i < r.count && ok; ++i) {
+      ok = mbar_wait(c.full(st), st_phase, c.abort_flag);
       if (!ok) break;
-      tc_fence_after();
-      const uint32_t d0 = c.tmem0 + (uint32_t)(b * 128);
-#pragma unroll
-      for (int ks = 0; ks < 8; ++ks) {
-        const uint64_t off = (uint64_t)((ks & 3) * 2) + (ks >> 2) * hi;
-        if (VOTE) tc_mma(d0, k_desc + off, q_desc0 + off, idesc, ks > 0);
-        else tc_mma(d0, q_desc0 + off, k_desc + off, idesc, ks > 0);
+      const uint64_t kd = k_desc0 + (uint64_t)((st * c.stage_bytes) >> 4);
+      for (int mt = 0; mt < c.MT && ok; ++mt, ++uc) {
+        ok = unit_free(uc);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = c.tmem + (uint32_t)((uc & 3) * 128);
+        const uint64_t qd = q_desc + (uint64_t)(mt * ((128 * 128) >> 4));
+        if (r.kind == 0) product(d, qd, q_hi, kd, k_hi, idesc_s);
+        else product(d, kd, k_hi, qd, q_hi, mt == 0 ? idesc_v0 : idesc_v1);
+        if (mt == c.MT - 1) tc_commit(c.empty(st));            // K stage free once these MMAs have read it
+        tc_commit(c.unit_full(uc & 3));
       }
-      tc_commit(c.empty_bar(st));       // K stage free once these MMAs have read it
-      tc_commit(NWG == 2 ? c.accf_bar(b) : c.accf_bar_of(it % NWG, b));   // accumulator ready for the epilogue
-      k_desc += (uint64_t)(kStageBytes >> 4);
-      if (++st == c.n_stages) { st = 0; st_phase ^= 1u; k_desc = k_desc0; }
-      if (++b == 2) { b = 0; b_phase ^= 1u; }
+      if (++st == c.n_stages) { st = 0; st_phase ^= 1u; }
     }
-    tc_commit(c.qempty_bar());          // Q tile free once the run's MMAs are done
-    pos += r.count;
-    ++run_idx;
+    tc_commit(c.q_empty(n));              // Q tile free once the run's MMAs are done
+    ++n;
   }
-  }
-  if (!ok) {
+  if (!ok || *c.abort_flag) {
     // gave up: the MMAs this thread has issued must be through before the accumulators are released
-    tc_commit(c.drain_bar());
+    tc_commit(c.drain());
     const unsigned long long t0 = now_ns();
-    while (!mbar_try(c.drain_bar(), 0) && now_ns() - t0 < kWaitLimitNs) {}
+    while (!mbar_try(c.drain(), 0) && now_ns() - t0 < kWaitLimitNs) {}
   }
 }
 
-// ---- 256 threads: pass 1, row statistics (stream A) ----------------------------------------------------------
-__device__ __forceinline__ void epilogue_rows(const StreamCtx& c, const TcArgs& a, const PipeArgs& pa, int et, int warp,
-                                              float* stat_m, float* stat_z) {
-  const int wg = et >> 7, row = et & 127, lane = et & 31;
-  const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
-  const float sc = a.scale_log2;
-  const int R = a.R;
-  int it = 0;
-  bool ok = true;
-  for (int j = pa.a_first; j <= pa.a_last; ++j) {
-  const LayerDesc& L = pa.lay[j];
-  int begin, end;
-  entry_range(a, L, begin, end);
-  for (int pos = begin; pos < end;) {
-    const Run r = locate(a, pos, begin, end, false);
-    const int seg = r.s * a.n_kv_heads + r.g;
-    const int first_cta = (r.seg_tile0 - L.tile_begin) / a.tiles_per_cta;
-    float m = 0.f, z = 0.f;                                   // fixed reference 0 on the fast path
-    for (int i = 0; i < r.count; ++i, ++it) {
-      if ((it & 1) != wg) continue;
-      const int b = it & 1;
-      if (ok) ok = mbar_wait(c.accf_bar(b), (it >> 1) & 1, c.abort_flag, kPollNs);
-      ok = __all_sync(0xffffffffu, ok) != 0;                  // the TMEM loads below need the whole warp
-      if (!ok) continue;
-      tc_fence_after();
-      if (et == 0 && it == 0) trace_mark(a.trace, 2);
-      const int key0 = (r.t0 + i) * kTileKeys;
-      const int n_valid = min(r.n_hist - key0, kTileKeys);
-      const uint32_t tcol = c.tmem0 + lane_sel + (uint32_t)(b * 128);
-      // A fixed reference m per row (0 until a fallback moves it) instead of a running maximum: any reference gives
-      // the same log-sum-exp as long as nothing overflows and not everything underflows.  A chunk whose sum is not
-      // finite and positive is redone exactly from the registers, which moves the reference.  Keys past the
-      // segment's end (its ragged last tile) are left out chunk by chunk.
-      uint32_t ra[32], rb[32];
-      auto add_chunk = [&](const uint32_t (&rr)[32], int nv) {
-        if (nv <= 0) return;                                   // wholly past the segment's end
-        if (nv >= 32) {
-          const float zc = sum_ex2_32_mufu(rr, sc, m);
-          const float zn = z + zc;
-          if (zn < INFINITY && zn > kTinySum) { z = zn; return; }
+// ---- warp 2: hands out the runs; announces statistics -----------------------------------------------------------------
+// Whatever is possible next is done: a run slot that has come free is filled, statistics that are out are announced.
+__device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArgs& a) {
+  const int lane = threadIdx.x & 31;
+  int k_out = 0, k_in = 0;                 // runs handed out, runs done with as publisher
+  int n = 0;                               // statistics runs so far
+  bool all_out = false;
+  const int n_seg = a.sh.n_seqs * a.sh.n_kv_heads, stride = a.sh.slot_stride;
+  RunWalk w;
+  w.start();
+  unsigned long long t0 = 0;
+  unsigned idle = 0;
+  while (true) {
+    bool moved = false;
+    if (!all_out && __any_sync(0xffffffffu, mbar_test(c.run_empty(k_out), ((k_out / kRunSlots) & 1) ^ 1))) {
+      int kind = 0;
+      if (lane == 0) {
+        w.next(a, c.runs[k_out & (kRunSlots - 1)]);
+        kind = w.kind;
+        mbar_arrive(c.run_full(k_out));
+      }
+      all_out = __shfl_sync(0xffffffffu, kind, 0) == 2;    // also orders the lanes behind lane 0's stores
+      ++k_out;
+      moved = true;
+    }
+    if (k_in < k_out) {
+      const RunDesc& r = c.runs[k_in & (kRunSlots - 1)];
+      if (r.kind == 2) break;
+      const int slot = n & 1;
+      const bool stats = r.kind == 0 && r.count > 0;
+      if (!stats || __any_sync(0xffffffffu, mbar_test(c.stat_full(slot), (n >> 1) & 1))) {
+        if (stats) {
+          const unsigned far = c.stat_far[slot];
+          if (far) {                                           // rare: scores beyond fp64's range
+            const StatView st = stat_view(a.lay[r.layer].part, n_seg, c.R, stride);
+            const size_t at0 = ((size_t)r.seg * stride + r.slot) * c.R;
+            for (int row = lane; row < c.R; row += 32) {
+              float Z = 0.f, M = 0.f;
+              for (int wg = c.MT == 1 ? 0 : row >> 7; wg < kWgs; wg += c.MT)
+                if (far >> (wg * 4 + ((row & 127) >> 5)) & 1u) {
+                  const int at = (slot * kWgs + wg) * 128 + (row & 127);
+                  stat_add(Z, M, c.stat_z[at], c.stat_m[at]);
+                }
+              __stcg(st.far_z + at0 + row, Z);
+              __stcg(st.far_m + at0 + row, M);
+            }
+            if (lane == 0) {
+              atomicOr(st.far + (size_t)r.seg * kFarWords + (r.slot >> 5), 1u << (r.slot & 31));
+              c.stat_far[slot] = 0;
+            }
+          }
+          ++n;
         }
-        // rare: a copy goes through the stack so that the chunk registers themselves never have to
-        uint32_t tmp[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) tmp[e] = rr[e];
-        chunk_stats_exact(tmp, sc, nv < 32 ? nv : 32, m, z);
-      };
-      tc_ld32_issue(tcol, ra);
-#pragma unroll 1
-      for (int c0 = 0; c0 < kTileKeys; c0 += 64) {
-        const bool last = c0 + 64 >= kTileKeys;
-        tc_ld_wait(ra);
-        tc_ld32_issue(tcol + c0 + 32, rb);
-        if (last) {
-          // the whole accumulator is in registers (or on its way): hand the TMEM buffer back before the arithmetic
-          tc_ld_wait(rb);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(c.acce_bar(b));
+        const bool publish = r.kind == 0 && r.last && c.both;
+        const int gg = r.gg;
+        __syncwarp();
+        if (lane == 0) {
+          if (stats) mbar_arrive(c.stat_empty(slot));
+          if (publish) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + gg) : "memory");
+          mbar_arrive(c.run_empty(k_in));
         }
-        add_chunk(ra, n_valid - c0);
-        if (!last) {
-          tc_ld_wait(rb);
-          tc_ld32_issue(tcol + c0 + 64, ra);
-        }
-        add_chunk(rb, n_valid - c0 - 32);
+        ++k_in;
+        moved = true;
       }
     }
-    // combine the two warpgroups' statistics and publish this CTA's partial for the segment
-    const int slot = blockIdx.x - first_cta;
-    if (wg == 1) { stat_m[row] = m; stat_z[row] = z; }
-    named_bar(1);
-    if (wg == 0 && row < R) {
-      const float m1 = stat_m[row], z1 = stat_z[row];
-      const bool h0 = z > 0.f, h1 = z1 > 0.f;                  // a warpgroup without a tile in this run has z = 0
-      const float M = h0 && h1 ? fmaxf(m, m1) : (h0 ? m : m1);
-      float Z = 0.f;
-      if (h0) Z += z * ex2(m - M);
-      if (h1) Z += z1 * ex2(m1 - M);
-      L.part_m[((long long)seg * a.slot_stride + slot) * R + row] = M;
-      L.part_z[((long long)seg * a.slot_stride + slot) * R + row] = Z;
+    if (moved) { idle = 0; continue; }
+    if (idle == 0) t0 = now_ns();
+    if ((++idle & 63u) == 0 && (*c.abort_flag || now_ns() - t0 > kWaitLimitNs)) { *c.abort_flag = 1; break; }
+    __nanosleep(50);
+  }
+}
+
+// ---- warp 3: the rows' log-sum-exps (log2 units, negated) of the segments the vote phases take, ahead of them ------
+// From a CTA's last tile of a group to the log-sum-exps in every other CTA's shared memory there is one hop: add to the
+// rows' sums, release, acquire, load.  (Per-CTA partial sums that the consumers merge took 14 us at 37 shares, merged by
+// their owners in equal parts and fetched 11 us -- twice what the phases in between cover: beside warps that saturate the
+// issue slots every dependent step costs several times its latency.)
+__device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
+  const int lane = threadIdx.x & 31;
+  const int G = a.sh.G, window = a.sh.window, q_head_inner = a.sh.q_head_inner;
+  const int n_seg = a.sh.n_seqs * a.sh.n_kv_heads, stride = a.sh.slot_stride;
+  auto wait_count = [&](const unsigned* p, unsigned target) {
+    if (lane == 0) {
+      unsigned long long t0 = 0;
+      for (unsigned spin = 0;; ++spin) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        if (v >= target) break;
+        if (spin == 0) t0 = now_ns();
+        if ((spin & 15u) == 15u && (*c.abort_flag || now_ns() - t0 > kWaitLimitNs)) { *c.abort_flag = 1; break; }
+        __nanosleep(20);
+      }
     }
-    named_bar(1);
-    pos += r.count;
+    __syncwarp();
+    return __all_sync(0xffffffffu, *c.abort_flag == 0) != 0;
+  };
+  if (c.both) {
+    // this CTA's part of the layers' statistics areas is cleared; nobody adds to them before all parts are
+    const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);
+    const int w0 = split_begin(blockIdx.x, words, gridDim.x), w1 = split_begin(blockIdx.x + 1, words, gridDim.x);
+    for (int l = 0; l < a.n_layers; ++l)
+      for (int i = w0 + lane; i < w1; i += 32) __stcg(static_cast<unsigned*>(a.lay[l].part) + i, 0u);
+    __syncwarp();
+    if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + a.n_groups) : "memory");
+    if (!wait_count(a.counters + a.n_groups, gridDim.x)) return;
   }
-  // This CTA's row statistics of layer j are written (the barrier above orders the other threads' stores before
-  // this thread's release): one more CTA has published.
-  if (et == 0 && ok) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(pa.counters + j) : "memory");
-  if (et == 0 && j < 24) trace_mark(a.trace, 8 + 2 * j);
-  }
-}
-
-// sum_e 2^(v_e * sc - lse_e) over 32 accumulator values (32 query rows of one key)
-__device__ __forceinline__ float vote_chunk(const uint32_t (&r)[32], float sc, const float* lse) {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+  if (lane == 0) mbar_arrive(c.cleared());
+  int n = 0, seen = -1;                    // vote runs so far; the last group known to be published
+  for (int k = 0;; ++k) {
+    const RunDesc r = take_run<true>(c, k);
+    if (r.kind == 2) break;
+    if (r.kind == 0) continue;
+    // every CTA has published its share of the group (all CTAs are resident, and a statistics phase waits for nothing
+    // but vote phases that are due before it, so the count gets there; bounded all the same)
+    if (c.both && r.gg != seen) {
+      if (!wait_count(a.counters + r.gg, a.target)) break;
+      seen = r.gg;
+    }
+    // The common case, straight through: the sums are on their way while the slot comes free, and no launch parameter is
+    // touched.
+    double Z[8];
+    unsigned far = 0;
+    if (r.sums) {
 #pragma unroll
-  for (int e = 0; e < 32; e += 4) {
-    const float4 l4 = *reinterpret_cast<const float4*>(lse + e);
-    s0 += ex2(fmaf(__uint_as_float(r[e]), sc, -l4.x));
-    s1 += ex2(fmaf(__uint_as_float(r[e + 1]), sc, -l4.y));
-    s2 += ex2(fmaf(__uint_as_float(r[e + 2]), sc, -l4.z));
-    s3 += ex2(fmaf(__uint_as_float(r[e + 3]), sc, -l4.w));
+      for (int u = 0; u < 8; ++u)
+        if (u * 32 < c.R) Z[u] = u * 32 + lane < c.R ? __ldcg(r.acc + u * 32 + lane) : 1.0;
+      if (lane < kFarWords) far = __ldcg(r.far + lane);
+    }
+    const bool plain = r.sums && !r.win && !__any_sync(0xffffffffu, far != 0);
+    const bool ok = mbar_wait(c.lse_empty(n & 1), ((n >> 1) & 1) ^ 1, c.abort_flag);
+    if (!__all_sync(0xffffffffu, ok)) break;
+    float* lse = c.lse + (n & 1) * 256;
+    if (plain) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (u * 32 < c.R) lse[u * 32 + lane] = u * 32 + lane < c.R ? -log2_of(Z[u]) : -INFINITY;
+    } else {
+      const LseSource& src = a.lay[r.layer].lse;
+      const StatView st = stat_view(a.lay[r.layer].part, n_seg, c.R, stride);
+#pragma unroll 1
+      for (int row = lane; row < c.Rp; row += 32) {
+        float l2 = INFINITY;                                    // rows of padding: 2^(0 - inf) = 0
+        if (row < c.R) {
+          const size_t at = (size_t)r.seg * c.R + row;
+          if (src.lse_opt) l2 = src.caller_lse(r.s, r.g, row, G, window, q_head_inner != 0);
+          else if (!r.sums) l2 = __ldcg(st.lse + at);
+          else l2 = row_lse(st, __ldcg(st.acc + at), true, r.seg, row, c.R, stride, r.n_slots, r.win != 0,
+                            r.win ? src.win_m[at] : 0.f, r.win ? src.win_z[at] : 0.f);
+        }
+        lse[row] = -l2;
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(c.lse_full(n & 1));
+    if (n == 0 && lane == 0) trace_mark(a.trace, 3);
+    ++n;
   }
-  return (s0 + s1) + (s2 + s3);
 }
 
-// sum_e 2^(v_e * sc - lse_e) over 16 accumulator values
-__device__ __forceinline__ float vote_chunk16(const uint32_t (&r)[16], float sc, const float* lse) {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+// ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
+// sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators
+template <bool STATS>
+__device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 off, uint32_t off_sh, f32x2& s0,
+                                          f32x2& s1) {
 #pragma unroll
   for (int e = 0; e < 16; e += 4) {
-    const float4 l4 = *reinterpret_cast<const float4*>(lse + e);
-    s0 += ex2(fmaf(__uint_as_float(r[e]), sc, -l4.x));
-    s1 += ex2(fmaf(__uint_as_float(r[e + 1]), sc, -l4.y));
-    s2 += ex2(fmaf(__uint_as_float(r[e + 2]), sc, -l4.z));
-    s3 += ex2(fmaf(__uint_as_float(r[e + 3]), sc, -l4.w));
+    f32x2 o0 = off, o1 = off;
+    if (!STATS) {
+      // an explicit shared-memory load: a generic one takes another path
+      asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(o0), "=l"(o1) : "r"(off_sh + 4u * e));
+    }
+    const f32x2 x0 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, o0);
+    const f32x2 x1 = fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sc2, o1);
+    s0 = add2(s0, ((e >> 1) & 7) < kPolyPairs ? ex2_pair_poly<STATS>(x0) : ex2_pair(x0));
+    s1 = add2(s1, ((e >> 1) & 7) + 1 < kPolyPairs ? ex2_pair_poly<STATS>(x1) : ex2_pair(x1));
   }
-  return (s0 + s1) + (s2 + s3);
 }
 
-// ---- 256 threads: pass 2, votes (stream B) ---------------------------------------------------------------------
-// `first`, `last`, pa.step: the entries this stream takes; `bar_id`: the named barrier of its 256 threads; `is_b`: the
-// stream pass 1 of the same CTA keeps its distance to.
-template <int NWG>
-__device__ __forceinline__ void epilogue_votes(const StreamCtx& c, const TcArgs& a, const PipeArgs& pa, int et, int warp,
-                                               float* lse2, int first, int last, int bar_id, bool is_b) {
-  const int wg = et >> 7, row = et & 127, lane = et & 31;
-  const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
-  const float sc = a.scale_log2;
-  const float inv_g = 1.0f / (float)a.G;
-  const int R = a.R;
-  int it = 0, run_idx = 0;
-  int own0 = 0, own1 = 0;               // this warpgroup's tiles so far on either accumulator (three warpgroups)
-  bool ok = true;
-  for (int j = first; j <= last; j += pa.step) {
-  const LayerDesc& L = pa.lay[j];
-  if (pa.step == 1 && j >= pa.a_first && j <= pa.a_last && !L.lse.lse_opt) {
-    // the layer's pass 1 is part of this launch: wait until every CTA has published its row statistics (all CTAs
-    // are resident, and stream A waits for nothing, so the count gets there; bounded all the same)
-    if (et == 0 && ok) {
-      const unsigned long long t0 = now_ns();
-      for (unsigned spin = 1;; ++spin) {
-        unsigned v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(pa.counters + j) : "memory");
-        if ((int)(v - pa.target[j]) >= 0) break;
-        if ((spin & 63u) == 0 && (*c.abort_flag || now_ns() - t0 > kWaitLimitNs)) { *c.abort_flag = 1; break; }
-        __nanosleep(64);
+// An epilogue thread's unit.
+struct Unit {
+  uint32_t tcol;               // its TMEM lane and its warpgroup's unit
+  uint32_t full, empty;        // the unit's mbarriers
+  volatile int* abort_flag;
+};
+__device__ __forceinline__ bool unit_wait(const Unit& u, int nth) {
+  const bool ok = mbar_wait(u.full, nth & 1, u.abort_flag);
+  if (!__all_sync(0xffffffffu, ok)) return false;                        // the TMEM loads need the whole warp
+  tc_fence_after();
+  return true;
+}
+__device__ __forceinline__ void unit_release(const Unit& u) {
+  tc_fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(u.empty);
+}
+
+// The keys past the segment's end count nothing.
+__device__ __forceinline__ void drop_keys(uint32_t (&r)[16], int n_valid) {
+#pragma unroll
+  for (int e = 0; e < 16; ++e)
+    if (e >= n_valid) r[e] = __float_as_uint(-INFINITY);
+}
+
+// Statistics of one run for this thread's query row: tiles i0, i0 + every, ... < count.  z: the sum of 2^score, without a
+// reference; (far_z, far_m): what of it fp64 cannot hold (see StatView).  A tile is summed in fp32, without a reference
+// either as long as nothing overflows and not everything underflows; one whose sum is not finite and above kTinySum is
+// redone exactly.  false: a wait ran out.
+__device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i0, int every, int count, int n_valid0,
+                                          bool rows_here, double& z, float& far_z, float& far_m) {
+  z = 0.0;
+  far_z = far_m = 0.f;
+  const f32x2 sc2 = pack2(sc, sc);
+#pragma unroll 1
+  for (int i = i0; i < count; i += every, ++nth) {
+    if (!unit_wait(u, nth)) return false;
+    if (rows_here) {
+      const int n_valid = n_valid0 - i * kTileKeys;
+      uint32_t ra[16], rb[16];
+      f32x2 s0 = 0, s1 = 0;
+      tc_ld16_issue(u.tcol, ra);
+#pragma unroll 1
+      for (int c0 = 0; c0 < kTileKeys; c0 += 32) {
+        tc_ld_wait(ra);
+        tc_ld16_issue(u.tcol + c0 + 16, rb);
+        if (n_valid < kTileKeys) drop_keys(ra, n_valid - c0);
+        exp_chunk<true>(ra, sc2, 0, 0u, s0, s1);
+        tc_ld_wait(rb);
+        if (c0 + 32 < kTileKeys) tc_ld16_issue(u.tcol + c0 + 32, ra);
+        if (n_valid < kTileKeys) drop_keys(rb, n_valid - c0 - 16);
+        exp_chunk<true>(rb, sc2, 0, 0u, s0, s1);
+      }
+      const float tile = sum2(s0, s1);
+      const bool exact = !(tile < INFINITY && tile > kTinySum);
+      if (!__any_sync(0xffffffffu, exact)) {
+        z += (double)tile;
+      } else {                                                 // the exact path's TMEM loads need the whole warp
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, n_valid, tm, tz);
+        if (!exact) z += (double)tile;                         // the same value whatever the other rows hold
+        else if (fabsf(tm) <= kFarScore) z += scalbn((double)tz, (int)tm);
+        else stat_add(far_z, far_m, tz, tm);
       }
     }
-    named_bar(bar_id, NWG * 128);
-    ok = ok && *c.abort_flag == 0;
+    unit_release(u);
   }
-  if (et == 0 && is_b) *c.b_layer = j;
-  if (et == 0 && is_b && j < 24) trace_mark(a.trace, 9 + 2 * j);
-  int begin, end;
-  entry_range(a, L, begin, end);
-  for (int pos = begin; pos < end;) {
-    const Run r = locate(a, pos, begin, end, false);
-    const int seg = r.s * a.n_kv_heads + r.g;
-    const int first_cta = (r.seg_tile0 - L.tile_begin) / a.tiles_per_cta;
-    float* lse = lse2 + 128 * (run_idx & 1);
-    {
-      // the rows' log-sum-exp (log2 units): the caller's, or the per-CTA partials of this segment merged (two
-      // neighbouring lanes share a row)
-      const int n_slots = (r.seg_tile0 - L.tile_begin + r.tiles_seg - 1) / a.tiles_per_cta - first_cta + 1;
-      const int rr = (et >> 1) < R ? (et >> 1) : -1;
-      const int half = et & 1;
-      float l2;
-      if (L.lse.lse_opt) {
-        l2 = rr >= 0 ? L.lse.caller_lse(r.s, r.g, rr, a.G, a.window, a.q_head_inner != 0) : 0.f;
-      } else {
-        const bool has_win = L.lse.win_m != nullptr && rr >= 0;
-        l2 = merged_row_lse(L.part_m + (long long)seg * a.slot_stride * R, L.part_z + (long long)seg * a.slot_stride * R,
-                            n_slots, R, rr, half, 2, has_win, has_win ? L.lse.win_m[(long long)seg * R + rr] : 0.f,
-                            has_win ? L.lse.win_z[(long long)seg * R + rr] : 0.f);
-      }
-      if (half == 0 && rr >= 0) lse[rr] = l2;
+  return true;
+}
+
+// Votes of one run for this thread's key of every tile: the sum over this warpgroup's rows (cols of them, from its
+// log-sum-exps lse on).  MT = 2: the other 128 rows are the neighbouring warpgroup's; the first one, whose unit is filled
+// first, leaves its share in shared memory for the second (four slots in turn: a tile's second product waits until the
+// second warpgroup has given its unit back, so the first one cannot be more than three of its tiles ahead).
+// false: a wait ran out.
+__device__ __forceinline__ bool votes_run(const Unit u, int nth, float sc, int i0, int every, int count, int n_keys,
+                                       uint32_t lse, int cols, int half, float* half_vote, uint32_t half_bar, int n_half,
+                                       float inv_g, float* vote) {
+  const f32x2 sc2 = pack2(sc, sc);
+  const int row = threadIdx.x & 127;
+#pragma unroll 1
+  for (int i = i0; i < count; i += every, ++nth) {
+    if (!unit_wait(u, nth)) return false;
+    uint32_t ra[16], rb[16];
+    f32x2 s0 = 0, s1 = 0;
+    tc_ld16_issue(u.tcol, ra);
+#pragma unroll 1
+    for (int c0 = 0; c0 < cols; c0 += 32) {
+      tc_ld_wait(ra);
+      tc_ld16_issue(u.tcol + c0 + 16, rb);
+      exp_chunk<false>(ra, sc2, 0, lse + 4u * c0, s0, s1);
+      tc_ld_wait(rb);
+      if (c0 + 32 < cols) tc_ld16_issue(u.tcol + c0 + 32, ra); else unit_release(u);
+      exp_chunk<false>(rb, sc2, 0, lse + 4u * c0 + 64u, s0, s1);
     }
-    named_bar(bar_id, NWG * 128);
-    if (et == 0 && is_b && run_idx == 0) trace_mark(a.trace, 3);
-    for (int i = 0; i < r.count; ++i, ++it) {
-      const int b = it & 1;
-      if (NWG == 2) {
-        if ((it & 1) != wg) continue;
-        if (ok) ok = mbar_wait(c.accf_bar(b), (it >> 1) & 1, c.abort_flag, kPollNs);
-      } else {
-        if (it % NWG != wg) continue;
-        const int mine = b ? own1++ : own0++;
-        if (ok) ok = mbar_wait(c.accf_bar_of(wg, b), mine & 1, c.abort_flag, kPollNs);
-      }
-      ok = __all_sync(0xffffffffu, ok) != 0;
-      if (!ok) continue;
-      tc_fence_after();
-      const int key0 = (r.t0 + i) * kTileKeys;
-      const uint32_t tb = c.tmem0 + lane_sel + (uint32_t)(b * 128);
-      float acc = 0.f;
-      auto release = [&]() {
-        // the accumulator is in registers: hand its TMEM buffer back before the arithmetic and the vote's store
-        tc_fence_before();
+    float acc = sum2(s0, s1);
+    if (half >= 0) {
+      const int turn = n_half & 3;
+      const uint32_t parity = (n_half >> 2) & 1;
+      ++n_half;
+      if (half == 0) {
+        half_vote[turn * 128 + row] = acc;
         __syncwarp();
-        if (lane == 0) mbar_arrive(c.acce_bar(b));
-      };
-      if (NWG == 2) {
-        uint32_t ra[32], rb[32];
-        tc_ld32_issue(tb, ra);
-#pragma unroll 1
-        for (int c0 = 0; c0 < R; c0 += 64) {
-          tc_ld_wait(ra);
-          if (c0 + 32 < R) tc_ld32_issue(tb + c0 + 32, rb);
-          if (c0 + 32 >= R) release();
-          else if (c0 + 64 >= R) { tc_ld_wait(rb); release(); }
-          acc += vote_chunk(ra, sc, lse + c0);
-          if (c0 + 32 < R) {
-            if (c0 + 64 < R) { tc_ld_wait(rb); tc_ld32_issue(tb + c0 + 64, ra); }
-            acc += vote_chunk(rb, sc, lse + c0 + 32);
-          }
-        }
-      } else {
-        // three warpgroups per stream share the register file: rounds of 16 columns (R is a multiple of 32)
-        uint32_t ra[16], rb[16];
-        tc_ld16_issue(tb, ra);
-#pragma unroll 1
-        for (int c0 = 0; c0 < R; c0 += 32) {
-          tc_ld_wait16(ra);
-          tc_ld16_issue(tb + c0 + 16, rb);
-          acc += vote_chunk16(ra, sc, lse + c0);
-          tc_ld_wait16(rb);
-          if (c0 + 32 < R) tc_ld16_issue(tb + c0 + 32, ra); else release();
-          acc += vote_chunk16(rb, sc, lse + c0 + 16);
-        }
+        if ((threadIdx.x & 31) == 0) mbar_arrive(half_bar + 8u * turn);
+        continue;
       }
-      const int jk = key0 + row;
-      if (jk < r.n_hist) L.vote[a.tab.hist_at(r.s) * a.n_kv_heads + (long long)r.g * r.n_hist + jk] = acc * inv_g;
+      const bool ok = mbar_wait(half_bar + 8u * turn, parity, u.abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      acc += half_vote[turn * 128 + row];
     }
-    pos += r.count;
-    ++run_idx;
+    const int key = i * kTileKeys + row;
+    if (key < n_keys) vote[key] = acc * inv_g;
   }
+  return true;
+}
+
+__device__ __forceinline__ void epilogue(const Smem& c) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wg = (threadIdx.x - 128) >> 7, row = threadIdx.x & 127;
+  Unit u;
+  u.tcol = c.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(wg * 128);
+  u.full = c.unit_full(wg);
+  u.empty = c.unit_empty(wg);
+  u.abort_flag = c.abort_flag;
+  // MT = 1: unit u = tile u, this warpgroup's tiles are wg, wg + 4, ...; MT = 2: tile t has the units 2t (rows 0-127,
+  // or the votes' first 128 rows) and 2t + 1
+  const int every = c.MT == 1 ? kWgs : kWgs / 2, log_every = c.MT == 1 ? 2 : 1, mine = c.MT == 1 ? wg : wg >> 1, mt = c.MT == 1 ? 0 : wg & 1;
+  const bool rows_here = mt * 128 + (warp & 3) * 32 < c.R;                // some row of this warp's lanes exists
+  int it = 0, units = 0, n_stat = 0, n_vote = 0, n_half = 0;
+  for (int k = 0;; ++k) {
+    const RunDesc r = take_run<true>(c, k);
+    if (r.kind == 2) break;
+    if (r.count == 0) continue;
+    const int i0 = (mine - it) & (every - 1);                             // this warpgroup's first tile of the run
+    it += r.count;
+    const int n_mine = i0 < r.count ? ((r.count - 1 - i0) >> log_every) + 1 : 0;
+    bool ok;
+    if (r.kind == 0) {
+      double z;
+      float far_z, far_m;
+      ok = stats_run(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, z, far_z, far_m);
+      const int slot = n_stat & 1;
+      ok = ok && mbar_wait(c.stat_empty(slot), ((n_stat >> 1) & 1) ^ 1, c.abort_flag) && mbar_wait(c.cleared(), 0, c.abort_flag);
+      ++n_stat;
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (z > 0.0 && mt * 128 + row < c.R)
+        asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(r.acc + mt * 128 + row), "d"(z) : "memory");
+      if (__any_sync(0xffffffffu, far_z > 0.f)) {
+        c.stat_z[(slot * kWgs + wg) * 128 + row] = far_z;
+        c.stat_m[(slot * kWgs + wg) * 128 + row] = far_m;
+        if (lane == 0) atomicOr(c.stat_far + slot, 1u << (wg * 4 + (warp & 3)));
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.stat_full(slot));
+    } else {
+      const int slot = n_vote & 1;
+      ok = mbar_wait(c.lse_full(slot), (n_vote >> 1) & 1, c.abort_flag);
+      ++n_vote;
+      if (!__all_sync(0xffffffffu, ok)) break;
+      ok = votes_run(u, units, c.sc, i0, every, r.count, r.n_valid, smem_u32(c.lse + slot * 256 + mt * 128), min(c.Rp - mt * 128, 128),
+                     c.MT == 2 ? mt : -1, c.half_vote + mine * 512, c.half_full(mine, 0), n_half, c.inv_g, r.vote);
+      n_half += n_mine;
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (lane == 0) mbar_arrive(c.lse_empty(slot));
+    }
+    units += n_mine;
   }
 }
 
-// DUAL: both streams run pass 2 (every layer of the list came with its row statistics), each on every other entry.
-template <bool DUAL>
-__global__ void __launch_bounds__(DUAL ? kDualThreads : kPipeThreads, 1)
-k_score_pipe(const __grid_constant__ PipeArgs pa) {
+__global__ void __launch_bounds__(kListThreads, 1)
+k_score_list(const __grid_constant__ ListArgs a) {
   // Shared memory, all dynamic and 1024-byte aligned (the swizzled tiles need it):
-  //   [Q of A 32 KB][Q of B 32 KB][K ring of A 2 x 32 KB][K ring of B 3 x 32 KB][mbarriers, flags 512 B]
-  //   [stat_m, stat_z of A 1 KB][log-sum-exp rows of B 2 x 512 B]
+  //   [n_q Q tiles: halves x MT x 16 KB][K ring: n_stages x halves x 16 KB][mbarriers, flags][statistics][log-sum-exps][half votes]
   extern __shared__ __align__(1024) unsigned char smem[];
+  const ScoreShape& sh = a.sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  unsigned char* tail = smem + 2 * kQBytes + (kStagesA + kStagesB) * kStageBytes;
-  uint32_t& tmem_base_sh = *reinterpret_cast<uint32_t*>(tail + 2 * kBarBytesPerStream);
-  int& abort_sh = *reinterpret_cast<int*>(tail + 2 * kBarBytesPerStream + 4);
-  int& b_layer_sh = *reinterpret_cast<int*>(tail + 2 * kBarBytesPerStream + 8);   // the layer stream B's epilogue has begun
-  float* stat_m = reinterpret_cast<float*>(tail + 512);
-  float* stat_z = stat_m + 128;
-  float* lse2 = stat_m + 256;
-  const TcArgs& a = pa.base;
-  const bool has_a = pa.a_first <= pa.a_last, has_b = pa.b_first <= pa.b_last;
-  const int lay_lo = has_b ? min(pa.b_first, has_a ? pa.a_first : pa.b_first) : pa.a_first;
-  const int lay_hi = has_a ? max(pa.a_last, has_b ? pa.b_last : pa.a_last) : pa.b_last;
   if ((smem_u32(smem) & 1023u) != 0) {                      // never run on a skewed layout (uniform over the CTA)
     if (tid == 0)
-      for (int j = lay_lo; j <= lay_hi; ++j)
-        if (pa.lay[j].status) atomicExch(pa.lay[j].status, (int)SLKV_ERR_BAD_ALIGN);
+      for (int j = 0; j < a.n_layers; ++j)
+        if (a.lay[j].status) atomicExch(a.lay[j].status, (int)SLKV_ERR_BAD_ALIGN);
     return;
   }
-  StreamCtx ca, cb;
-  ca.q_smem = smem_u32(smem);
-  cb.q_smem = ca.q_smem + kQBytes;
-  ca.k_smem = ca.q_smem + 2 * kQBytes;
-  cb.k_smem = ca.k_smem + kStagesA * kStageBytes;
-  ca.bar0 = smem_u32(tail);
-  cb.bar0 = ca.bar0 + kBarBytesPerStream;
-  ca.n_stages = kStagesA;
-  cb.n_stages = kStagesB;
-  ca.abort_flag = cb.abort_flag = &abort_sh;
-  ca.b_layer = cb.b_layer = &b_layer_sh;
+  // the tail's place follows from launch parameters; everything the roles use in their loops goes through shared memory
+  unsigned char* tail = smem + sh.halves * (sh.n_q * sh.MT * 128 * 128 + sh.n_stages * kHalfBytes);
+  uint32_t& tmem_base_sh = *reinterpret_cast<uint32_t*>(tail + kBarBytes - 16);
+  int& abort_sh = *reinterpret_cast<int*>(tail + kBarBytes - 12);
+  volatile int* head = reinterpret_cast<volatile int*>(tail + kBarBytes - 16 - kHeadInts * 4);
+  Smem c;
+  c.bar0 = smem_u32(tail);
+  c.abort_flag = &abort_sh;
+  c.stat_z = reinterpret_cast<float*>(tail + kBarBytes);
+  c.stat_m = c.stat_z + 2 * kWgs * 128;
+  c.stat_far = reinterpret_cast<unsigned*>(tail + kBarBytes - 8);
+  c.lse = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes);
+  c.half_vote = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes + kLseBytes);
+  c.runs = reinterpret_cast<RunDesc*>(tail + kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes);
 
-  if (tid == 0) trace_mark(a.trace, 0);
-  if (tid == 0 && a.trace) a.trace[(size_t)blockIdx.x * kTraceSlots + 60] = (unsigned long long)clock64();
   if (tid == 0) {
-    if (has_a) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&pa.lay[pa.a_first].tm_k)) : "memory");
-    if (has_b) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&pa.lay[pa.b_first].tm_k)) : "memory");
-    if (has_a) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&pa.lay[pa.a_first].tm_q)) : "memory");
-    if (has_b) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&pa.lay[pa.b_first].tm_q)) : "memory");
+    trace_mark(a.trace, 0);
+    if (a.trace) a.trace[(size_t)blockIdx.x * kTraceSlots + 60] = (unsigned long long)clock64();
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&a.lay[0].tm_k)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&a.lay[0].tm_q)) : "memory");
     abort_sh = 0;
-    b_layer_sh = has_b ? pa.b_first - 1 : 1 << 30;
+    c.stat_far[0] = c.stat_far[1] = 0;
+    mbar_init(c.cleared(), 1);
+    for (int st = 0; st < kMaxStages; ++st) { mbar_init(c.full(st), 1); mbar_init(c.empty(st), 1); }
+    for (int u = 0; u < 4; ++u) { mbar_init(c.unit_full(u), 1); mbar_init(c.unit_empty(u), 4); }
     for (int s = 0; s < 2; ++s) {
-      const StreamCtx& c = s ? cb : ca;
-      for (int st = 0; st < 3; ++st) { mbar_init(c.full_bar(st), 1); mbar_init(c.empty_bar(st), 1); }
-      for (int b = 0; b < 2; ++b) { mbar_init(c.accf_bar(b), 1); mbar_init(c.acce_bar(b), 4); }
-      for (int g = 0; g < 6; ++g) mbar_init(c.accf_bar_of(g >> 1, g & 1), 1);
-      mbar_init(c.qfull_bar(), 1);
-      mbar_init(c.qempty_bar(), 1);
-      mbar_init(c.drain_bar(), 1);
+      mbar_init(c.stat_full(s), 4 * kWgs);
+      mbar_init(c.stat_empty(s), 1);
+      mbar_init(c.lse_full(s), 1);
+      mbar_init(c.lse_empty(s), 4 * kWgs);
+      for (int t = 0; t < 4; ++t) mbar_init(c.half_full(s, t), 4);
     }
+    c.n_q = 2;                                                // both slots' barriers, used or not
+    for (int k = 0; k < 2; ++k) { mbar_init(c.q_full(k), 1); mbar_init(c.q_empty(k), 1); }
+    for (int k = 0; k < kRunSlots; ++k) { mbar_init(c.run_full(k), 1); mbar_init(c.run_empty(k), kRunReaders); }
+    head[0] = sh.R; head[1] = sh.Rp; head[2] = sh.MT; head[3] = sh.halves;
+    head[4] = sh.n_q; head[5] = sh.n_stages; head[6] = sh.k_head_inner;
+    head[7] = a.passes == 3; head[8] = __float_as_int(sh.scale_log2); head[9] = __float_as_int(1.0f / (float)sh.G);
+    mbar_init(c.drain(), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // rows of a Q tile beyond R are never written by TMA: keep them zero
-  if (a.R != 128) {
-    for (int i = tid; i < 2 * kQBytes / 16; i += (int)blockDim.x) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+  // rows of the Q tile beyond R are never written by TMA: keep them zero
+  if (sh.R != sh.MT * 128) {
+    for (int i = tid; i < sh.n_q * sh.halves * sh.MT * 128 * 128 / 16; i += kListThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
@@ -541,240 +781,191 @@ k_score_pipe(const __grid_constant__ PipeArgs pa) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = tmem_base_sh;
-  ca.tmem0 = tmem_base;
-  cb.tmem0 = tmem_base + 256;
-  // With both streams on the vote pass the launch behind this one is another of its kind, and none of its CTAs fits
-  // on an SM this launch holds: released now they would only sit on the SMs left to the selection kernels until this
-  // launch ends.  They are released when this CTA is done instead.
-  if (!DUAL) pdl_launch_dependents();
+  c.tmem = tmem_base_sh;
+  c.R = head[0]; c.Rp = head[1]; c.MT = head[2]; c.halves = head[3];
+  c.n_q = head[4]; c.n_stages = head[5]; c.k_head_inner = head[6];
+  c.both = head[7]; c.sc = __int_as_float(head[8]); c.inv_g = __int_as_float(head[9]);
+  c.q_half = c.MT * 128 * 128;
+  c.q_bytes = c.halves * c.q_half;
+  c.stage_bytes = c.halves * kHalfBytes;
+  c.q = smem_u32(smem);
+  c.k = c.q + (uint32_t)(c.n_q * c.q_bytes);
+  // Everything above touched only this CTA's own resources.
+  pdl_launch_dependents();
+  pdl_wait();
+  if (tid == 0) trace_mark(a.trace, 1);
 
-  // Stream A reads its layers' Q and K for the first time and overwrites row statistics an earlier launch may still
-  // be merging: all its roles wait for the work before this launch.  Stream B's loads and MMAs need only Q and K,
-  // which are inputs, and for the pending layer have been read by the launch before: they start at once; its
-  // epilogue needs that launch's row statistics and waits.
   if (warp == 0) {
-    if (lane == 0 && has_a) {
-      if (DUAL) producer<true>(ca, a, pa.lay, pa.a_first, pa.a_last, pa.step, pa.a_first);
-      else producer<false>(ca, a, pa.lay, pa.a_first, pa.a_last, 1, pa.a_first);
-    }
+    if (lane == 0) producer(c);
   } else if (warp == 1) {
-    if (lane == 0 && has_a) {
-      if (DUAL) issuer<true, kDualWgs>(ca, a, pa.lay, pa.a_first, pa.a_last, pa.step);
-      else issuer<false>(ca, a, pa.lay, pa.a_first, pa.a_last, 1);
-    }
+    if (lane == 0) issuer(c);
   } else if (warp == 2) {
-    // normally entry 0 was read by the launch before; with both streams on pass 2 every entry is new to this launch
-    if (lane == 0 && has_b) producer<true>(cb, a, pa.lay, pa.b_first, pa.b_last, pa.step, DUAL ? pa.b_first : 1);
+    scheduler_publisher(c, a);
   } else if (warp == 3) {
-    if (lane == 0 && has_b) { if (DUAL) issuer<true, kDualWgs>(cb, a, pa.lay, pa.b_first, pa.b_last, pa.step); else issuer<true>(cb, a, pa.lay, pa.b_first, pa.b_last, pa.step); }
-  } else if (warp < (DUAL ? 4 + 4 * kDualWgs : 12)) {
-    if (has_a) {
-      pdl_wait();
-      if (tid == 128) trace_mark(a.trace, 1);
-      if (DUAL) epilogue_votes<kDualWgs>(ca, a, pa, tid - 128, warp, stat_m, pa.a_first, pa.a_last, 1, false);
-      else epilogue_rows(ca, a, pa, tid - 128, warp, stat_m, stat_z);
-      if (tid == 128) trace_mark(a.trace, 5);
-    }
+    fetch_lse(c, a);
   } else {
-    if (has_b) {
-      pdl_wait();
-      constexpr int kFirstB = DUAL ? 128 + 128 * kDualWgs : 384;
-      if (tid == kFirstB) trace_mark(a.trace, 7);
-      if (DUAL) epilogue_votes<kDualWgs>(cb, a, pa, tid - kFirstB, warp, lse2, pa.b_first, pa.b_last, 2, true);
-      else epilogue_votes<2>(cb, a, pa, tid - kFirstB, warp, lse2, pa.b_first, pa.b_last, 2, true);
-      if (tid == kFirstB) trace_mark(a.trace, 6);
-    }
+    epilogue(c);
   }
 
   tc_fence_before();
   __syncthreads();
-  if (DUAL) pdl_launch_dependents();
   if (abort_sh && tid == 0)
-    for (int j = lay_lo; j <= lay_hi; ++j)
-      if (pa.lay[j].status) atomicExch(pa.lay[j].status, (int)SLKV_ERR_DEVICE_TIMEOUT);
-  if (tid == 0) trace_mark(a.trace, 4);
-  if (tid == 0 && a.trace) a.trace[(size_t)blockIdx.x * kTraceSlots + 61] = (unsigned long long)clock64();
+    for (int j = 0; j < a.n_layers; ++j)
+      if (a.lay[j].status) atomicExch(a.lay[j].status, (int)SLKV_ERR_DEVICE_TIMEOUT);
   if (tid == 0) {
-    // every thread of this CTA is past its last use of the counters (the barrier above)
-    unsigned prev;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(pa.counters + kMaxLay) : "memory");
+    trace_mark(a.trace, 4);
+    if (a.trace) a.trace[(size_t)blockIdx.x * kTraceSlots + 61] = (unsigned long long)clock64();
+  }
+  if (warp == 0 && a.passes == 3) {
+    // every thread of this CTA is past its last use of the counters (the barrier above): the last CTA out cleans the set
+    const int n_words = a.n_groups + 1;
+    unsigned prev = 0;
+    if (lane == 0)
+      asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(a.counters + n_words) : "memory");
+    prev = __shfl_sync(0xffffffffu, prev, 0);
     if (prev == gridDim.x - 1) {
-      for (int j = 0; j <= kMaxLay; ++j) pa.counters[j] = 0;
+      for (int j = lane; j <= n_words; j += 32) a.counters[j] = 0;
       __threadfence();
     }
   }
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512u) : "memory");
   }
+}
+
+// One-shot diagnostic: the next launch of this thread whose CTAs wait for one another expects one arrival too many.
+thread_local int g_expire_next_wait = 0;
+
+// Timeline tracing (diagnostics): a caller-owned device buffer.
+thread_local unsigned long long* g_trace = nullptr;
+thread_local size_t g_trace_bytes = 0;
+
+// A phase should last about this many tiles-times-row-blocks per CTA before the phase that needs its results is due:
+// publishing, the other CTAs' counters and the merge take about 5 us, a unit about 0.6 us.
+constexpr int kLagUnits = 10;
+
+// A launch of the statistics pass alone finds the row sums cleared.
+cudaError_t clear_stats(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < n_layers && e == cudaSuccess; ++i)
+    e = cudaMemsetAsync(lay[i].part, 0, stat_clear_bytes(sh.n_seqs * sh.n_kv_heads, sh.R), st);
+  return e;
 }
 
 }  // namespace
 
-bool score_pipe_supported(const Problem& pb) {
-  return tensor_path_supported(pb.p) && pb.R <= 128;
+void expire_next_wait(int on) { g_expire_next_wait = on; }
+int take_expire_next_wait() { const int v = g_expire_next_wait; g_expire_next_wait = 0; return v; }
+
+void set_tensor_trace(void* dev_buf, size_t bytes) {
+  g_trace = static_cast<unsigned long long*>(dev_buf);
+  g_trace_bytes = bytes;
+}
+unsigned long long* tensor_trace_buffer(int n_cta) {
+  return g_trace && g_trace_bytes >= (size_t)n_cta * kTraceSlots * sizeof(unsigned long long) ? g_trace : nullptr;
 }
 
-// One launch: pass 1 of plans a[0..n_a) beside pass 2 of `pending` (the layer whose pass 1 an earlier launch did;
-// may be null) and of a[0..n_a-1), or of all of a[] when `finish` is set.  The plans share one shape and schedule.
-cudaError_t launch_score_pipe(const TcPlan* pending, const TcPlan* const* a, int n_a, bool finish, bool votes_only,
-                              cudaStream_t st, int* launches) {
-  if (n_a > kPipeMaxLayers) return cudaErrorInvalidValue;
-  if (votes_only && pending) return cudaErrorInvalidValue;     // nothing stays pending between vote-only launches
-  // Without cooperative launches (refused once on this device) no launch may hold both passes of a layer: one layer's
-  // pass 1 per launch, beside pass 2 of the layer before.
-  static thread_local bool no_coop[64] = {};
-  static const bool env_no_coop = [] {                // SLKV_NO_COOPERATIVE=1: behave as if they were refused (tests)
-    const char* v = std::getenv("SLKV_NO_COOPERATIVE");
-    return v && v[0] == '1';
-  }();
-  {
-    int d = 0;
-    if (env_no_coop && cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < 64) no_coop[d] = true;
-    if (!votes_only && cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < 64 && no_coop[d] &&
-        (n_a > 1 || (n_a == 1 && finish))) {
-      const TcPlan* prev = pending;
-      for (int i = 0; i < n_a; ++i) {
-        cudaError_t e1 = launch_score_pipe(prev, a + i, 1, false, false, st, launches);
-        if (e1 != cudaSuccess) return e1;
-        prev = a[i];
-      }
-      return finish ? launch_score_pipe(prev, nullptr, 0, true, false, st, launches) : cudaSuccess;
-    }
-  }
-  const TcPlan* any = pending && pending->n_cta > 0 ? pending : nullptr;
-  for (int i = 0; i < n_a && !any; ++i)
-    if (a[i]->n_cta > 0) any = a[i];
-  if (!any) return cudaSuccess;                       // no history anywhere: nothing to score
+// K tiles of the ring beside the Q tiles.
+int score_list_stages(int MT, int halves, int n_q) {
+  const int n = (kSmemLimit - kTail - n_q * halves * MT * 128 * 128) / (halves * kHalfBytes);
+  return n < kMaxStages ? n : kMaxStages;
+}
+
+cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes, cudaStream_t st,
+                              int* launches) {
+  if (n_layers < 1 || sh.n_cta == 0) return cudaSuccess;             // no history: nothing to score
+  if (n_layers > kListMaxLayers) return cudaErrorInvalidValue;
   static thread_local int configured_dev = -1;
   static thread_local unsigned* counters_base = nullptr;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(k_score_pipe<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPipeSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_score_pipe<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPipeSmem);
+    e = cudaFuncSetAttribute(k_score_list, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     void* sym = nullptr;
-    e = cudaGetSymbolAddress(&sym, g_layer_published);
+    e = cudaGetSymbolAddress(&sym, g_published);
     if (e != cudaSuccess) return e;
     counters_base = static_cast<unsigned*>(sym);
     configured_dev = dev;
   }
-  PipeArgs pa;
-  std::memset(&pa, 0, sizeof(pa));
-  pa.base = any->a;
-  pa.base.part_m = pa.base.part_z = pa.base.vote = nullptr;
-  pa.base.status = nullptr;
-  // A layer goes in as one entry, or as two (its first and second half of the segments) when the halves are whole
-  // segments and equal: pass 2 of an entry then follows its pass 1 after half a layer's time and half a layer's K.
-  const TcArgs& sh = any->a;
-  const int total = sh.total_tiles;
-  int groups = 1;
-  if (kMaxGroups >= 2 && total % 2 == 0 && sh.tab.n_inline > 0) {
-    const int mid = total / 2;
-    for (int q = 0; q < sh.tab.n_inline && groups == 1; ++q) {
-      const int t_seq = sh.tab.tile_off[q + 1] - sh.tab.tile_off[q];
-      for (int g = 0; g < sh.n_kv_heads; ++g)
-        if (sh.n_kv_heads * sh.tab.tile_off[q] + g * t_seq == mid) { groups = 2; break; }
-    }
-  }
-  int n_cta = any->n_cta;
-  if (groups == 2) {
-    const int per_group = total / 2;
-    int tpc = (per_group + n_cta - 1) / n_cta;
-    pa.base.tiles_per_cta = tpc;
-    n_cta = (per_group + tpc - 1) / tpc;
-  }
-  auto fill = [&](int j, const TcPlan* p, int group) {
-    pa.lay[j].tm_q = p->tm_q; pa.lay[j].tm_k = p->tm_k;
-    pa.lay[j].part_m = p->a.part_m; pa.lay[j].part_z = p->a.part_z; pa.lay[j].vote = p->a.vote;
-    pa.lay[j].status = p->a.status;
-    pa.lay[j].lse = p->a.lse;
-    pa.lay[j].tile_begin = groups == 2 ? group * (total / 2) : 0;
-    pa.lay[j].tile_end = groups == 2 ? (group + 1) * (total / 2) : total;
-  };
-  const bool has_pending = pending && pending->n_cta > 0;
-  if (has_pending) fill(0, pending, groups - 1);      // what is pending of a layer is its last group
-  int n_live = 0;
-  for (int i = 0; i < n_a; ++i)
-    if (a[i]->n_cta > 0)
-      for (int g = 0; g < groups; ++g) fill(++n_live, a[i], g);     // layers without history take no part
-  pa.a_first = 1; pa.a_last = n_live;
-  pa.b_first = has_pending ? 0 : 1;
-  pa.b_last = finish ? n_live : n_live - 1;
-  pa.step = 1;
-  if (votes_only) {                                   // both streams on pass 2, every other entry each
-    pa.step = 2;
-    pa.b_first = 2;
-    pa.b_last = n_live;
-  }
-  if (pa.a_first > pa.a_last && pa.b_first > pa.b_last) return cudaSuccess;
-  pa.base.trace = tensor_trace_buffer(0, n_cta);
-  // counters of this launch: a slot of the table, zeroed on the stream before the kernel
+  ListArgs a;
+  a.sh = sh;
+  std::memcpy(a.lay, lay, sizeof(ScoreLayer) * (size_t)n_layers);
+  a.n_layers = n_layers;
+  a.passes = passes;
+  a.group_layers = n_layers > 1 && sh.group_layers > 1 ? sh.group_layers : 1;
+  a.n_groups = a.group_layers == 1 ? n_layers * sh.n_groups : (n_layers + a.group_layers - 1) / a.group_layers;
+  // units per CTA and phase, about
+  const int per_phase = (int)((long long)sh.total_tiles * n_layers * sh.MT / ((long long)a.n_groups * sh.n_cta));
+  a.lag = kLagUnits / (per_phase > 0 ? per_phase : 1);
+  if (a.lag > a.n_groups - 1) a.lag = a.n_groups - 1;
+  if (a.lag < 1) a.lag = 1;
   static std::atomic<unsigned> launch_seq{0};
-  pa.counters = counters_base + (size_t)(launch_seq.fetch_add(1) % kCountSlots) * kCountWords;
-  const bool waits_inside = !votes_only && pa.b_last >= pa.a_first && pa.a_last >= pa.a_first;   // a layer's two passes in one launch
-  const unsigned extra = waits_inside && take_expire_next_wait() ? 1u : 0u;       // diagnostics: a wait that runs out
-  for (int j = 0; j < kMaxLay; ++j) pa.target[j] = (unsigned)n_cta + extra;
-  // CTAs that wait for one another must all be resident: cooperative launch.  Dependent launch on top where the
-  // device takes both (the kernel waits for the launch before it exactly where it needs that launch's results).
-  static thread_local int pdl_with_coop[64] = {};     // per device: 0 untried, 1 works, -1 refused
-  int& pc = pdl_with_coop[dev < 64 ? dev : 0];
+  a.counters = counters_base + (size_t)(launch_seq.fetch_add(1) % kCountSlots) * kCountWords;
+  const bool waits_inside = passes == 3;
+  a.target = (unsigned)sh.n_cta + (waits_inside && take_expire_next_wait() ? 1u : 0u);
+  a.trace = tensor_trace_buffer(sh.n_cta);
+  const size_t smem = (size_t)(sh.n_q * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + kTail);
+
+  // CTAs that wait for one another must all be resident: cooperative launch, with dependent launch on top where the
+  // device takes both.  Where it takes no cooperative launch, or the environment says so (tests), the two passes go out
+  // as two launches.
+  static const bool env_no_coop = [] {
+    const char* v = std::getenv("SLKV_NO_COOPERATIVE");
+    return v && v[0] == '1';
+  }();
+  static thread_local int coop_state[64] = {};        // per device: 0 untried, 1 with dependent launch, 2 without, -1 refused
+  int& cs = coop_state[dev < 64 ? dev : 0];
+  if (waits_inside && (env_no_coop || cs == -1 || sh.n_cta > sm_count())) {
+    a.passes = 1;
+    a.group_layers = 1;
+    a.n_groups = n_layers * sh.n_groups;
+    e = clear_stats(sh, lay, n_layers, st);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl_scoped(KID_SCORE_LSE, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
+    if (e != cudaSuccess) return e;
+    for (int i = 0; i < n_layers && e == cudaSuccess; ++i) e = launch_merge_lse_tensor(sh, lay[i], nullptr, 1.f, st, launches);
+    if (e != cudaSuccess) return e;
+    a.passes = 2;
+    return launch_pdl_scoped(KID_SCORE_VOTE, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
+  }
+  if (passes == 1) {
+    e = clear_stats(sh, lay, n_layers, st);
+    if (e != cudaSuccess) return e;
+  }
+  const int kid = passes == 1 ? KID_SCORE_LSE : (n_layers > 1 ? KID_SCORE_PIPE : (passes == 2 ? KID_SCORE_VOTE : KID_SCORE_FUSED));
+  if (!waits_inside) return launch_pdl_scoped(kid, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
   for (int attempt = 0; attempt < 2; ++attempt) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_cta);
-    cfg.blockDim = dim3(votes_only ? kDualThreads : kPipeThreads);
-    cfg.dynamicSmemBytes = kPipeSmem;
+    cfg.gridDim = dim3(sh.n_cta);
+    cfg.blockDim = dim3(kListThreads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[3];
-    int n = 0;
-    {
-      // ahead of the selections and gathers that become ready at the same moment on the side streams: when SMs
-      // come free, this kernel's CTAs are placed first
-      int least = 0, greatest = 0;
-      if (cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess && greatest != least) {
-        attr[n].id = cudaLaunchAttributePriority;
-        attr[n].val.priority = greatest;
-        ++n;
-      }
-    }
-    if (waits_inside) {
-      attr[n].id = cudaLaunchAttributeCooperative;
-      attr[n].val.cooperative = 1;
-      ++n;
-    }
-    const bool with_pdl = !waits_inside || pc >= 0;
-    if (with_pdl) {
-      attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[n].val.programmaticStreamSerializationAllowed = 1;
-      ++n;
-    }
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = n;
+    cfg.numAttrs = cs == 2 ? 1 : 2;
     cudaError_t le;
     {
-      LaunchScope scope(KID_SCORE_PIPE, st, launches);
-      le = votes_only ? cudaLaunchKernelEx(&cfg, k_score_pipe<true>, pa) : cudaLaunchKernelEx(&cfg, k_score_pipe<false>, pa);
+      LaunchScope scope(kid, st, launches);
+      le = cudaLaunchKernelEx(&cfg, k_score_list, a);
     }
     if (le == cudaSuccess) {
-      if (waits_inside && with_pdl) pc = 1;
+      if (cs == 0) cs = 1;
       return cudaSuccess;
     }
-    if (!waits_inside) return le;
     (void)cudaGetLastError();                         // not a sticky error: the launch was refused
     --*launches;
-    if (with_pdl && pc != 1) { pc = -1; continue; }   // once more without dependent launch
-    // cooperative launches do not work here: the list goes out one layer per launch from now on
-    no_coop[dev < 64 ? dev : 0] = true;
-    return launch_score_pipe(pending, a, n_a, finish, votes_only, st, launches);
+    if (cs == 2 || cs == 1) { cs = -1; break; }
+    cs = 2;                                           // once more without dependent launch
   }
-  return cudaErrorLaunchFailure;
+  cs = -1;
+  return launch_score_list(sh, lay, n_layers, passes, st, launches);
 }
-
-// The most layers one launch takes (pass 1); callers that queue layers launch when they have this many.
-int score_pipe_max_layers() { return kPipeMaxLayers; }
 
 }  // namespace slkv

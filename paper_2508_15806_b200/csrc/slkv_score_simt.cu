@@ -244,6 +244,9 @@ k_merge_lse_simt(const float* __restrict__ part_m, const float* __restrict__ par
   }
 }
 
+float* part_m_of(const Problem& pb) { return reinterpret_cast<float*>(pb.part); }
+float* part_z_of(const Problem& pb) { return part_m_of(pb) + (size_t)pb.n_seg * pb.R * pb.n_chunks; }
+
 template <typename T, int D>
 cudaError_t launch_passes(const Problem& pb, int passes, cudaStream_t st, int* launches) {
   const size_t smem = simt_smem_bytes(pb);
@@ -266,7 +269,7 @@ cudaError_t launch_passes(const Problem& pb, int passes, cudaStream_t st, int* l
   if (passes & 1) {
     LaunchScope scope(KID_SCORE_LSE, st, launches);
     e = launch_pdl(k_score_simt<T, D, 1>, grid, dim3(kThreads), smem, st, 1, (const T*)pb.q, (const T*)pb.k, pb.tab,
-                   pb.part_m, pb.part_z, pb.vote, lse, p.n_kv_heads, pb.G, p.window, pb.n_chunks,
+                   part_m_of(pb), part_z_of(pb), pb.vote, lse, p.n_kv_heads, pb.G, p.window, pb.n_chunks,
                    (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
                    (long long)p.q_stride_row, (long long)p.q_stride_head, scale_log2);
     if (e != cudaSuccess) return e;
@@ -274,7 +277,7 @@ cudaError_t launch_passes(const Problem& pb, int passes, cudaStream_t st, int* l
   if (!(passes & 2)) return cudaSuccess;
   LaunchScope scope(KID_SCORE_VOTE, st, launches);
   return launch_pdl(k_score_simt<T, D, 2>, grid, dim3(kThreads), smem, st, 1, (const T*)pb.q, (const T*)pb.k, pb.tab,
-                    pb.part_m, pb.part_z, pb.vote, lse, p.n_kv_heads, pb.G, p.window, pb.n_chunks,
+                    part_m_of(pb), part_z_of(pb), pb.vote, lse, p.n_kv_heads, pb.G, p.window, pb.n_chunks,
                     (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
                     (long long)p.q_stride_row, (long long)p.q_stride_head, scale_log2);
 }
@@ -330,8 +333,8 @@ float lse_out_scale(const Problem& pb) { return pb.p.lse_units == SLKV_LSE_LOG2 
 cudaError_t launch_merge_lse_simt(const Problem& pb, float* lse_out, cudaStream_t st, int* launches) {
   if (pb.max_hist <= 0) return cudaSuccess;
   LaunchScope scope(KID_MERGE_LSE, st, launches);
-  return launch_pdl(k_merge_lse_simt, dim3(pb.n_seg), dim3(kThreads), 0, st, 1, (const float*)pb.part_m,
-                    (const float*)pb.part_z, lse_source_of(pb), pb.tab, lse_out, pb.p.n_kv_heads, pb.G, pb.p.window,
+  return launch_pdl(k_merge_lse_simt, dim3(pb.n_seg), dim3(kThreads), 0, st, 1, (const float*)part_m_of(pb),
+                    (const float*)part_z_of(pb), lse_source_of(pb), pb.tab, lse_out, pb.p.n_kv_heads, pb.G, pb.p.window,
                     pb.n_chunks, pb.chunk_keys, lse_out_scale(pb));
 }
 

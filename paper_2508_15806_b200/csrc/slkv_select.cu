@@ -196,26 +196,32 @@ k_select(const float* __restrict__ pooled, const __grid_constant__ SeqTables tab
 // Copies the kept rows of K and V into the packed cache: 16 bytes per lane, a row per lane group.  The
 // selection kernel left the source row (token * n_kv_heads + head) of every packed row in gather_src, so a
 // row costs two dependent memory round trips (source index, then the row itself).
+struct GatherArgs {
+  int n_seg, n_kv_heads, row_bytes;
+  long long k_tok_bytes, k_head_bytes, v_tok_bytes, v_head_bytes, all_rows;
+  TailLayer lay[kListMaxLayers];
+};
 __global__ void __launch_bounds__(256)
-k_gather(const unsigned char* __restrict__ k, const unsigned char* __restrict__ v, unsigned char* __restrict__ k_out,
-         unsigned char* __restrict__ v_out, const int32_t* __restrict__ offsets,
-         const int32_t* __restrict__ gather_src, int n_seg, int n_kv_heads, int row_bytes, long long k_tok_bytes,
-         long long k_head_bytes, long long v_tok_bytes, long long v_head_bytes, long long max_rows) {
+k_gather(const __grid_constant__ GatherArgs g) {
   pdl_launch_dependents();
-  const int lanes = row_bytes >> 4;                       // 16-byte lanes per row (power of two <= 32)
+  const TailLayer& a = g.lay[blockIdx.y];
+  const int lanes = g.row_bytes >> 4;                       // 16-byte lanes per row (power of two <= 32)
   const int rows_per_cta = blockDim.x / lanes;
   const int lane = threadIdx.x % lanes, sub = threadIdx.x / lanes;
+  const long long max_rows = min(a.capacity, g.all_rows);
+  const unsigned char* k = static_cast<const unsigned char*>(a.k);
+  const unsigned char* v = static_cast<const unsigned char*>(a.v);
   pdl_wait();
-  const long long n_rows = min((long long)offsets[n_seg], max_rows);
+  const long long n_rows = min((long long)a.offsets[g.n_seg], max_rows);
   for (long long r = (long long)blockIdx.x * rows_per_cta + sub; r < max_rows;
        r += (long long)gridDim.x * rows_per_cta) {
-    const int src = gather_src[r];                        // in bounds for r < max_rows; valid for r < n_rows
+    const int src = a.gather_src[r];                        // in bounds for r < max_rows; valid for r < n_rows
     if (r >= n_rows) break;
-    const int tok = src / n_kv_heads, h = src - tok * n_kv_heads;
-    const uint4 kv = *reinterpret_cast<const uint4*>(k + tok * k_tok_bytes + h * k_head_bytes + lane * 16);
-    const uint4 vv = *reinterpret_cast<const uint4*>(v + tok * v_tok_bytes + h * v_head_bytes + lane * 16);
-    *reinterpret_cast<uint4*>(k_out + r * row_bytes + lane * 16) = kv;
-    *reinterpret_cast<uint4*>(v_out + r * row_bytes + lane * 16) = vv;
+    const int tok = src / g.n_kv_heads, h = src - tok * g.n_kv_heads;
+    const uint4 kv = *reinterpret_cast<const uint4*>(k + tok * g.k_tok_bytes + h * g.k_head_bytes + lane * 16);
+    const uint4 vv = *reinterpret_cast<const uint4*>(v + tok * g.v_tok_bytes + h * g.v_head_bytes + lane * 16);
+    *reinterpret_cast<uint4*>(static_cast<unsigned char*>(a.k_out) + r * g.row_bytes + lane * 16) = kv;
+    *reinterpret_cast<uint4*>(static_cast<unsigned char*>(a.v_out) + r * g.row_bytes + lane * 16) = vv;
   }
 }
 
@@ -243,24 +249,26 @@ cudaError_t launch_select(const Problem& pb, const float* pooled, const int32_t*
                     kept_idx, pb.gather_src, pb.p.n_kv_heads, pb.p.window, (long long)capacity);
 }
 
-cudaError_t launch_gather(const Problem& pb, const int32_t* offsets, const int32_t* kept_idx, void* k_out,
-                          void* v_out, int64_t capacity, cudaStream_t st, int* launches, int block_threads) {
-  (void)kept_idx;
-  const int row_bytes = pb.p.head_dim * pb.elem;
-  if (block_threads != 128) block_threads = 256;
-  const int rows_per_cta = block_threads / (row_bytes >> 4);
-  long long max_rows = (long long)pb.p.n_kv_heads * pb.total_tokens;
-  if (capacity < max_rows) max_rows = capacity;
+cudaError_t launch_gather(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
+  GatherArgs g;
+  g.n_seg = pb.n_seg; g.n_kv_heads = pb.p.n_kv_heads;
+  g.row_bytes = pb.p.head_dim * pb.elem;
+  g.k_tok_bytes = pb.p.k_stride_tok * pb.elem; g.k_head_bytes = pb.p.k_stride_head * pb.elem;
+  g.v_tok_bytes = pb.p.v_stride_tok * pb.elem; g.v_head_bytes = pb.p.v_stride_head * pb.elem;
+  g.all_rows = (long long)pb.p.n_kv_heads * pb.total_tokens;
+  long long max_rows = 0;
+  for (int i = 0; i < n_layers; ++i) {
+    g.lay[i] = lay[i];
+    const long long m = lay[i].capacity < g.all_rows ? lay[i].capacity : g.all_rows;
+    if (m > max_rows) max_rows = m;
+  }
   if (max_rows <= 0) return cudaSuccess;
-  long long want = (max_rows + rows_per_cta - 1) / rows_per_cta;
-  const int max_grid = 148 * 8 * (256 / block_threads);
-  int grid = (int)(want < max_grid ? want : max_grid);
+  const int rows_per_cta = 256 / (g.row_bytes >> 4);
+  const long long want = (max_rows + rows_per_cta - 1) / rows_per_cta;
+  const long long most = (148 * 8 * 2 + n_layers - 1) / n_layers;
+  const int grid = (int)(want < most ? want : most);
   LaunchScope scope(KID_GATHER, st, launches);
-  return launch_pdl(k_gather, dim3(grid), dim3(block_threads), 0, st, 1, (const unsigned char*)pb.k,
-                    (const unsigned char*)pb.v, (unsigned char*)k_out, (unsigned char*)v_out, offsets,
-                    (const int32_t*)pb.gather_src, pb.n_seg, pb.p.n_kv_heads, row_bytes,
-                    (long long)(pb.p.k_stride_tok * pb.elem), (long long)(pb.p.k_stride_head * pb.elem),
-                    (long long)(pb.p.v_stride_tok * pb.elem), (long long)(pb.p.v_stride_head * pb.elem), max_rows);
+  return launch_pdl(k_gather, dim3((unsigned)grid, (unsigned)n_layers), dim3(256), 0, st, 1, g);
 }
 
 }  // namespace slkv

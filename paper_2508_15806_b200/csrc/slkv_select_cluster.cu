@@ -23,17 +23,10 @@ constexpr int kMaxCluster = 8;
 constexpr int kBins = 2048;
 
 struct SelArgs {
-  const float* vote;
-  float* pooled_out;          // optional
   SeqTables tab;
-  const int32_t* budgets;
-  int32_t* offsets;
-  int32_t* kept_idx;
-  int32_t* gather_src;        // per packed row: token * n_kv_heads + head of the source row
-  int32_t* status;
   int n_seqs, n_kv_heads, window, pool_kernel, pool_mode;
   int keys_off;               // float index in shared memory where the pooled keys start
-  long long capacity;
+  TailLayer lay[kListMaxLayers];
 };
 
 __device__ __forceinline__ int kept_rows(int len, int budget, int window) { return min(len, max(budget, window)); }
@@ -62,7 +55,7 @@ __device__ __forceinline__ int block_incl_scan(int v, int* wtot, int* total) {
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_select_cluster(const __grid_constant__ SelArgs a) {
+k_select_cluster(const __grid_constant__ SelArgs args) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) int hist[kBins];
   __shared__ __align__(16) unsigned short hist16[2][kBins];   // a slice holds <= 16384 scores: counts fit 16 bits
@@ -78,22 +71,23 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
   const int tid = threadIdx.x, lane = tid & 31;
   pdl_launch_dependents();
   const int seg = blockIdx.x / CS;
-  const int s = seg / a.n_kv_heads, h = seg - s * a.n_kv_heads;
-  const int t0 = a.tab.cu_at(s);
-  const int len = a.tab.cu_at(s + 1) - t0;
-  const int n_hist = max(len - a.window, 0);
-  const int n_win = min(len, a.window);
-  const int n_seg = a.n_seqs * a.n_kv_heads;
+  const TailLayer& a = args.lay[blockIdx.y];
+  const int s = seg / args.n_kv_heads, h = seg - s * args.n_kv_heads;
+  const int t0 = args.tab.cu_at(s);
+  const int len = args.tab.cu_at(s + 1) - t0;
+  const int n_hist = max(len - args.window, 0);
+  const int n_win = min(len, args.window);
+  const int n_seg = args.n_seqs * args.n_kv_heads;
   // this CTA's slice [lo, hi) of the history
   const int per = ((n_hist + CS - 1) / CS + 3) & ~3;
   const int lo = min(rank * per, n_hist), hi = min(lo + per, n_hist);
   const int n_own = hi - lo;
-  const long long seg_base = a.tab.hist_at(s) * a.n_kv_heads + (long long)h * n_hist;
+  const long long seg_base = args.tab.hist_at(s) * args.n_kv_heads + (long long)h * n_hist;
   const float* vote = a.vote + seg_base;
-  const int r = a.pool_kernel >> 1;
+  const int r = args.pool_kernel >> 1;
   float* sv = reinterpret_cast<float*>(smem_raw);                    // votes of [lo - r, hi + r)
-  unsigned* keys = reinterpret_cast<unsigned*>(smem_raw) + a.keys_off;          // pooled bit patterns of [lo, hi)
-  const float pad = a.pool_mode == SLKV_POOL_MAX ? -INFINITY : 0.f;
+  unsigned* keys = reinterpret_cast<unsigned*>(smem_raw) + args.keys_off;          // pooled bit patterns of [lo, hi)
+  const float pad = args.pool_mode == SLKV_POOL_MAX ? -INFINITY : 0.f;
   pdl_wait();                                // budgets and votes may come from the kernels before this one
   // The first 8192 votes of the slice start their way from L2 now, under the offset arithmetic below.
   float x0[8];
@@ -102,15 +96,15 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
     const int i = u * kThreads + tid, j = lo - r + i;
     x0[u] = (i < n_own + 2 * r && j >= 0 && j < n_hist) ? __ldg(vote + j) : pad;
   }
-  const int k_keep = kept_rows(len, a.budgets[h], a.window) - n_win;    // C_H = C - window, clamped
+  const int k_keep = kept_rows(len, a.budgets[h], args.window) - n_win;    // C_H = C - window, clamped
 
   // packed row where this segment starts = kept rows of all earlier segments (Algorithm 3 l.1-4 per head)
   long long out0;
   {
     int part = 0;                            // < 2^31: the host checks n_kv_heads * total_tokens
     for (int g = tid; g < seg; g += kThreads) {
-      const int s2 = g / a.n_kv_heads, h2 = g - s2 * a.n_kv_heads;
-      part += kept_rows(a.tab.cu_at(s2 + 1) - a.tab.cu_at(s2), a.budgets[h2], a.window);
+      const int s2 = g / args.n_kv_heads, h2 = g - s2 * args.n_kv_heads;
+      part += kept_rows(args.tab.cu_at(s2 + 1) - args.tab.cu_at(s2), a.budgets[h2], args.window);
     }
     int tot;
     block_incl_scan(part, wtot, &tot);
@@ -124,7 +118,7 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
       }
     }
   }
-  const int src_base = t0 * a.n_kv_heads + h;            // source row of position j: src_base + j * n_kv_heads
+  const int src_base = t0 * args.n_kv_heads + h;            // source row of position j: src_base + j * n_kv_heads
 
   // window rows: always kept, after the history rows
   if (rank == 0)
@@ -132,7 +126,7 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
       const long long o = out0 + k_keep + t;
       if (o < a.capacity) {
         a.kept_idx[o] = len - n_win + t;
-        a.gather_src[o] = src_base + (len - n_win + t) * a.n_kv_heads;
+        a.gather_src[o] = src_base + (len - n_win + t) * args.n_kv_heads;
       }
     }
 
@@ -159,13 +153,13 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
     __syncthreads();
     for (int i = tid; i < n_own; i += kThreads) {
       float acc;
-      if (a.pool_mode == SLKV_POOL_MAX) {
+      if (args.pool_mode == SLKV_POOL_MAX) {
         acc = sv[i];
         for (int t = 1; t <= 2 * r; ++t) acc = fmaxf(acc, sv[i + t]);
       } else {
         acc = 0.f;
         for (int t = 0; t <= 2 * r; ++t) acc += sv[i + t];
-        acc = acc / (float)a.pool_kernel;
+        acc = acc / (float)args.pool_kernel;
       }
       keys[i] = __float_as_uint(acc);
       if (a.pooled_out) a.pooled_out[seg_base + lo + i] = acc;
@@ -178,7 +172,7 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
     for (int i = tid; i < n_own; i += kThreads)
       if (out0 + lo + i < a.capacity) {
         a.kept_idx[out0 + lo + i] = lo + i;
-        a.gather_src[out0 + lo + i] = src_base + (lo + i) * a.n_kv_heads;
+        a.gather_src[out0 + lo + i] = src_base + (lo + i) * args.n_kv_heads;
       }
     return;
   }
@@ -288,7 +282,7 @@ k_select_cluster(const __grid_constant__ SelArgs a) {
         const long long o = out0 + gt_before + min(eq_before, need);
         if (o < a.capacity) {
           a.kept_idx[o] = lo + i;
-          a.gather_src[o] = src_base + (lo + i) * a.n_kv_heads;
+          a.gather_src[o] = src_base + (lo + i) * args.n_kv_heads;
         }
       }
       gt_before += gt;
@@ -312,9 +306,7 @@ bool select_cluster_supported(const Problem& pb) {
   return (pb.max_hist + cs - 1) / cs + 4 <= kMaxSlice && pb.p.pool_kernel <= 129;
 }
 
-cudaError_t launch_select_cluster(const Problem& pb, float* pooled_out, const int32_t* budgets, int32_t* offsets,
-                                  int32_t* kept_idx, int64_t capacity, int32_t* status, cudaStream_t st,
-                                  int* launches) {
+cudaError_t launch_select_cluster(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
   const int cs = select_cluster_size(pb);
   const int per = (((pb.max_hist + cs - 1) / cs + 3) & ~3);
   const int keys_off = (per + 2 * (pb.p.pool_kernel >> 1) + 3) & ~3;
@@ -329,14 +321,13 @@ cudaError_t launch_select_cluster(const Problem& pb, float* pooled_out, const in
     configured_dev = dev;
   }
   SelArgs a;
-  a.vote = pb.vote; a.pooled_out = pooled_out; a.tab = pb.tab; a.budgets = budgets;
-  a.offsets = offsets; a.kept_idx = kept_idx; a.gather_src = pb.gather_src; a.status = status;
+  a.tab = pb.tab;
   a.n_seqs = pb.p.n_seqs; a.n_kv_heads = pb.p.n_kv_heads; a.window = pb.p.window;
-  a.pool_kernel = pb.p.pool_kernel; a.pool_mode = pb.p.pool_mode; a.capacity = capacity;
+  a.pool_kernel = pb.p.pool_kernel; a.pool_mode = pb.p.pool_mode;
   a.keys_off = keys_off;
-
+  for (int i = 0; i < n_layers; ++i) a.lay[i] = lay[i];
   LaunchScope scope(KID_SELECT, st, launches);
-  return launch_pdl(k_select_cluster, dim3((unsigned)(pb.n_seg * cs)), dim3(kThreads), smem, st, cs, a);
+  return launch_pdl(k_select_cluster, dim3((unsigned)(pb.n_seg * cs), (unsigned)n_layers), dim3(kThreads), smem, st, cs, a);
 }
 
 }  // namespace slkv

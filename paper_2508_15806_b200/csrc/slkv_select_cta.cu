@@ -24,16 +24,9 @@ __device__ __forceinline__ int padded(int i) { return i + 32 + ((i + 32) >> 5); 
 constexpr int kPaddedFloats = (kMaxHist + 64) + ((kMaxHist + 64) >> 5) + 1;
 
 struct SelCtaArgs {
-  const float* vote;
-  float* pooled_out;          // optional
-  const int32_t* budgets;
-  int32_t* offsets;
-  int32_t* kept_idx;
-  int32_t* gather_src;        // per packed row: token * n_kv_heads + head of the source row
-  int32_t* status;
-  int n_seqs, n_kv_heads, window, pool_mode;
-  long long capacity;
   SeqTables tab;
+  int n_seqs, n_kv_heads, window, pool_mode;
+  TailLayer lay[kListMaxLayers];
 };
 
 __device__ __forceinline__ int kept_rows(int len, int budget, int window) { return min(len, max(budget, window)); }
@@ -63,7 +56,7 @@ __device__ __forceinline__ unsigned block_incl_scan(unsigned v, unsigned* wtot, 
 
 template <int RAD>
 __global__ void __launch_bounds__(kThreads, 1)
-k_select_cta(const __grid_constant__ SelCtaArgs a) {
+k_select_cta(const __grid_constant__ SelCtaArgs args) {
   extern __shared__ __align__(16) float sv[];                // padded votes, kPaddedFloats
   __shared__ __align__(8) int hist[kBins];
   __shared__ unsigned wtot[kWarps];
@@ -73,15 +66,16 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
   const int tid = threadIdx.x;
   pdl_launch_dependents();
   const int seg = blockIdx.x;
-  const int s = seg / a.n_kv_heads, h = seg - s * a.n_kv_heads;
-  const int t0 = a.tab.cu_at(s);
-  const int len = a.tab.cu_at(s + 1) - t0;
-  const int n_hist = max(len - a.window, 0);
-  const int n_win = min(len, a.window);
-  const int n_seg = a.n_seqs * a.n_kv_heads;
-  const long long seg_base = a.tab.hist_at(s) * a.n_kv_heads + (long long)h * n_hist;
+  const TailLayer& a = args.lay[blockIdx.y];
+  const int s = seg / args.n_kv_heads, h = seg - s * args.n_kv_heads;
+  const int t0 = args.tab.cu_at(s);
+  const int len = args.tab.cu_at(s + 1) - t0;
+  const int n_hist = max(len - args.window, 0);
+  const int n_win = min(len, args.window);
+  const int n_seg = args.n_seqs * args.n_kv_heads;
+  const long long seg_base = args.tab.hist_at(s) * args.n_kv_heads + (long long)h * n_hist;
   const float* vote = a.vote + seg_base;
-  const float pad = a.pool_mode == SLKV_POOL_MAX ? -INFINITY : 0.f;
+  const float pad = args.pool_mode == SLKV_POOL_MAX ? -INFINITY : 0.f;
   pdl_wait();                                // budgets and votes may come from the kernels before this one
 
   // all of the segment's votes, coalesced, in flight together
@@ -91,15 +85,15 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
     const int i = k * kThreads + tid;
     x[k] = i < n_hist ? __ldg(vote + i) : pad;
   }
-  const int k_keep = kept_rows(len, a.budgets[h], a.window) - n_win;    // C_H = C - window, clamped
+  const int k_keep = kept_rows(len, a.budgets[h], args.window) - n_win;    // C_H = C - window, clamped
 
   // packed row where this segment starts = kept rows of all earlier segments (Algorithm 3 l.1-4 per head)
   long long out0;
   {
     unsigned part = 0;                       // < 2^31: the host checks n_kv_heads * total_tokens
     for (int g = tid; g < seg; g += kThreads) {
-      const int s2 = g / a.n_kv_heads, h2 = g - s2 * a.n_kv_heads;
-      part += (unsigned)kept_rows(a.tab.cu_at(s2 + 1) - a.tab.cu_at(s2), a.budgets[h2], a.window);
+      const int s2 = g / args.n_kv_heads, h2 = g - s2 * args.n_kv_heads;
+      part += (unsigned)kept_rows(args.tab.cu_at(s2 + 1) - args.tab.cu_at(s2), a.budgets[h2], args.window);
     }
     unsigned tot;
     block_incl_scan(part, wtot, &tot);
@@ -113,14 +107,14 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
       }
     }
   }
-  const int src_base = t0 * a.n_kv_heads + h;            // source row of position j: src_base + j * n_kv_heads
+  const int src_base = t0 * args.n_kv_heads + h;            // source row of position j: src_base + j * n_kv_heads
 
   // window rows: always kept, after the history rows
   for (int t = tid; t < n_win; t += kThreads) {
     const long long o = out0 + k_keep + t;
     if (o < a.capacity) {
       a.kept_idx[o] = len - n_win + t;
-      a.gather_src[o] = src_base + (len - n_win + t) * a.n_kv_heads;
+      a.gather_src[o] = src_base + (len - n_win + t) * args.n_kv_heads;
     }
   }
 
@@ -130,7 +124,7 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
       for (int i = tid; i < n_hist; i += kThreads)
         if (out0 + i < a.capacity) {
           a.kept_idx[out0 + i] = i;
-          a.gather_src[out0 + i] = src_base + i * a.n_kv_heads;
+          a.gather_src[out0 + i] = src_base + i * args.n_kv_heads;
         }
     }
     return;
@@ -149,7 +143,7 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
     float v[kItems + 2 * RAD];
 #pragma unroll
     for (int j = 0; j < kItems + 2 * RAD; ++j) v[j] = sv[padded(first - RAD + j)];
-    if (a.pool_mode == SLKV_POOL_MAX) {
+    if (args.pool_mode == SLKV_POOL_MAX) {
       // max over [j, j + 2 RAD] by doubling: windows of 2, 4, ... then two overlapping ones
       constexpr int W = 2 * RAD + 1;
       int have = 1;                                                    // v[j] = max of v[j .. j + have - 1]
@@ -192,7 +186,7 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
     for (int i = tid; i < n_hist; i += kThreads)
       if (out0 + i < a.capacity) {
         a.kept_idx[out0 + i] = i;
-        a.gather_src[out0 + i] = src_base + i * a.n_kv_heads;
+        a.gather_src[out0 + i] = src_base + i * args.n_kv_heads;
       }
     return;
   }
@@ -285,7 +279,7 @@ k_select_cta(const __grid_constant__ SelCtaArgs a) {
     const int j = __ffs(m) - 1;
     if (o < a.capacity) {
       a.kept_idx[o] = first + j;
-      a.gather_src[o] = src_base + (first + j) * a.n_kv_heads;
+      a.gather_src[o] = src_base + (first + j) * args.n_kv_heads;
     }
   }
 }
@@ -296,8 +290,7 @@ bool select_cta_supported(const Problem& pb) {
   return pb.max_hist <= kMaxHist && (pb.p.pool_kernel >> 1) <= kMaxRadius;
 }
 
-cudaError_t launch_select_cta(const Problem& pb, float* pooled_out, const int32_t* budgets, int32_t* offsets,
-                              int32_t* kept_idx, int64_t capacity, int32_t* status, cudaStream_t st, int* launches) {
+cudaError_t launch_select_cta(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
   typedef void (*Kern)(const SelCtaArgs);
   static const Kern kerns[kMaxRadius + 1] = {k_select_cta<0>, k_select_cta<1>, k_select_cta<2>, k_select_cta<3>,
                                              k_select_cta<4>};
@@ -314,12 +307,11 @@ cudaError_t launch_select_cta(const Problem& pb, float* pooled_out, const int32_
     configured_dev = dev;
   }
   SelCtaArgs a;
-  a.vote = pb.vote; a.pooled_out = pooled_out; a.budgets = budgets; a.offsets = offsets; a.kept_idx = kept_idx;
-  a.gather_src = pb.gather_src; a.status = status;
+  a.tab = pb.tab;
   a.n_seqs = pb.p.n_seqs; a.n_kv_heads = pb.p.n_kv_heads; a.window = pb.p.window; a.pool_mode = pb.p.pool_mode;
-  a.capacity = capacity; a.tab = pb.tab;
+  for (int i = 0; i < n_layers; ++i) a.lay[i] = lay[i];
   LaunchScope scope(KID_SELECT, st, launches);
-  return launch_pdl(kerns[pb.p.pool_kernel >> 1], dim3((unsigned)pb.n_seg), dim3(kThreads), smem, st, 1, a);
+  return launch_pdl(kerns[pb.p.pool_kernel >> 1], dim3((unsigned)pb.n_seg, (unsigned)n_layers), dim3(kThreads), smem, st, 1, a);
 }
 
 }  // namespace slkv

@@ -10,20 +10,10 @@ namespace slkv {
 
 namespace {
 
-constexpr int kTileKeys = 128;                 // keys per tile (MMA N in pass 1, M in pass 2)
-constexpr int kMaxStages = 6;                  // K tiles in flight in shared memory (as many as fit beside Q)
+constexpr int kTileKeys = 128;                 // keys per tile (MMA N in the statistics pass, M in the vote pass)
 constexpr int kHalfBytes = kTileKeys * 128;    // one 64-element (128-byte) half of a 128-row tile
-constexpr int kStageBytes = 2 * kHalfBytes;    // 32 KB
-constexpr int kTailBytes = 512 + 2048;         // mbarriers + flags, then 512 floats of row statistics
 constexpr int kSmemLimit = 227 * 1024;         // dynamic shared memory a CTA can have
-constexpr int kThreads = 384;                  // warps 0-3: TMA, MMA, 2 idle; warps 4-11: epilogue
-constexpr int kEpiThreads = 256;
-constexpr int kTraceSlots = 64;               // per CTA: 0 start, 1 set-up done, 2 Q landed, 3 first K landed,
-                                               // 4 end; 5 / 6 grid barrier reached / passed, 7 first log-sum-exp merged; 8+2i / 9+2i = epilogue of the
-                                               // CTA's i-th tile begins / ends.  Two-layer kernel: 0 start, 1 / 7 stream A / B
-                                               // past its wait for the launch before, 2 first accumulator of A ready,
-                                               // 3 first log-sum-exps of B merged, 5 / 6 epilogue of A / B done, 4 end,
-                                               // 8+2j / 9+2j layer j published by A / begun by B, 60 / 61 SM cycle counter at start / end
+constexpr int kTraceSlots = 64;                // timeline words per CTA (see slkv_trace_set_buffer)
 // A row sum under the fixed reference that is not above this has underflowed (terms below fp32's range are flushed
 // to zero, or clamped to 2^-125 on the polynomial path): the exact path then moves the reference.
 constexpr float kTinySum = 1e-30f;
@@ -50,6 +40,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(100u) : "memory");    // may sleep up to 0.1 us: a waiting thread must
                                                                    // not eat the issue slots of the epilogue warps
+  return ok != 0;
+}
+// The same without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -80,24 +80,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm,
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
       ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
-// The same load with an L2 eviction policy (from createpolicy) for the lines it touches.
-__device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar,
-                                                 uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3, %4}], [%5], %6;"
-      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy) : "memory");
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, int w,
                                             uint32_t bar) {
   asm volatile(
@@ -122,36 +104,70 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// 2^x on the FMA and integer pipes instead of the special-function unit, which is the busiest pipe of both
-// passes (one exponential per query row and key): x = n + f with n = round(x), 2^f by a degree-4 minimax
-// polynomial on [-0.5, 0.5] (relative error 2.7e-6 in fp32 Horner form), n added into the exponent field.
-// x is clamped to [-125, 128.5]: below, the result is 2^-125 at most (negligible in any sum that holds a term
-// near 1); above, the exponent field overflows to Inf/NaN, which the caller's overflow check catches.
-// One exponential in four goes this way; the split balances the pipes' issue slots.
-__device__ __forceinline__ float ex2_fma(float x, bool clamp_hi) {
-  x = fmaxf(x, -125.f);
-  if (clamp_hi) x = fminf(x, 128.5f);
-  const float t = x + 12582912.f;                    // 1.5 * 2^23: round(x) lands in the low mantissa bits
-  const float f = x - (t - 12582912.f);
-  float p = fmaf(0.009570101276040077f, f, 0.05591785907745361f);
-  p = fmaf(p, f, 0.240247443318367f);
-  p = fmaf(p, f, 0.6931217908859253f);
-  p = fmaf(p, f, 0.9999992847442627f);
-  return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
+// Pairs of fp32 values in one 64-bit register: fma / add on both with one instruction.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
 }
-// Issues a TMEM load of 32 consecutive columns of this thread's lane; the registers are valid only after
-// tc_ld_wait on the same array.
-__device__ __forceinline__ void tc_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
-// The same for 16 columns (half the registers of a round; used where more warps share the register file).
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float sum2(f32x2 a, f32x2 b) {
+  float x, y, z, w;
+  unpack2(a, x, y);
+  unpack2(b, z, w);
+  return (x + y) + (z + w);
+}
+// 2^x of both halves on the special-function unit.
+__device__ __forceinline__ f32x2 ex2_pair(f32x2 x) {
+  float a, b;
+  unpack2(x, a, b);
+  return pack2(ex2(a), ex2(b));
+}
+// 2^x of both halves on the FMA and integer pipes instead of the special-function unit, which is the busiest pipe of
+// both passes (one exponential per query row and key): x = n + f with n = round(x), 2^f by a degree-5 polynomial that
+// is minimax in relative error on [-0.5, 0.5] (Remez exchange; 2.1e-7 evaluated in fp32, ex2.approx has 2^-22 =
+// 2.4e-7), n added into the exponent field.  x is clamped at -125 (the result is then 2^-125: negligible in any sum
+// that holds a term near 1) and, where CLAMP_HI, at 128.5, from where the exponent field overflows to Inf / NaN, which
+// the statistics pass's overflow check catches.
+template <bool CLAMP_HI>
+__device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {
+  float a, b;
+  unpack2(x, a, b);
+  a = fmaxf(a, -125.f);
+  b = fmaxf(b, -125.f);
+  if (CLAMP_HI) {
+    a = fminf(a, 128.5f);
+    b = fminf(b, 128.5f);
+  }
+  x = pack2(a, b);
+  const f32x2 t = add2(x, pack2(12582912.f, 12582912.f));     // 1.5 * 2^23: round(x) lands in the low mantissa bits
+  const f32x2 f = fma2(add2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x);
+  f32x2 p = fma2(pack2(0.0013276472454890609f, 0.0013276472454890609f), f, pack2(0.009675540961325169f, 0.009675540961325169f));
+  p = fma2(p, f, pack2(0.05550713092088699f, 0.05550713092088699f));
+  p = fma2(p, f, pack2(0.24022120237350464f, 0.24022120237350464f));
+  p = fma2(p, f, pack2(0.6931469440460205f, 0.6931469440460205f));
+  p = fma2(p, f, pack2(1.0000001192092896f, 1.0000001192092896f));
+  float pa, pb, ta, tb;
+  unpack2(p, pa, pb);
+  unpack2(t, ta, tb);
+  return pack2(__int_as_float(__float_as_int(pa) + (__float_as_int(ta) << 23)),
+               __int_as_float(__float_as_int(pb) + (__float_as_int(tb) << 23)));
+}
+// Issues a TMEM load of 16 consecutive columns of this thread's lane; the registers are valid only after tc_ld_wait on
+// the same array.
 __device__ __forceinline__ void tc_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -159,22 +175,12 @@ __device__ __forceinline__ void tc_ld16_issue(uint32_t taddr, uint32_t (&r)[16])
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void tc_ld_wait16(uint32_t (&r)[16]) {
+// Waits for this thread's outstanding TMEM loads; naming the registers keeps their uses behind the wait.
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
       : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
         "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]) :: "memory");
 }
-// Waits for this thread's outstanding TMEM loads; naming the registers keeps their uses behind the wait.
-__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.wait::ld.sync.aligned;"
-      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
-        "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
-        "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
-        "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-      :: "memory");
-}
-__device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // K-major, 128-byte-swizzled operand: rows 128 bytes apart, 8-row groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
@@ -185,57 +191,74 @@ __device__ __forceinline__ uint32_t instr_desc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// Merges the per-CTA partial statistics [slot][row] of one row of a segment (pm / pz point at the segment's first
-// slot) into the row's log-sum-exp in log2 units, the window keys' statistics (wm, wz) folded in when has_win.  With
-// halves == 2 two neighbouring lanes share a row (even / odd slots) and combine through a shuffle, so all 32 lanes
-// of a warp must call it; lanes without a row pass rr < 0.  Every thread has all its loads in flight before it uses
-// one.  One definition for every kernel that merges, so that they agree bit for bit.
-__device__ __forceinline__ float merged_row_lse(const float* pm, const float* pz, int n_slots, int R, int rr, int half,
-                                                int halves, bool has_win, float wm, float wz) {
-  float M = -INFINITY, Z = 0.f;
-  if (rr >= 0) {
-    pm += rr;                                                              // [segment][slot][row]
-    pz += rr;
-    for (int c0 = half; c0 < n_slots; c0 += 12 * halves) {
-      float m12[12], z12[12];
-#pragma unroll
-      for (int u = 0; u < 12; ++u) {
-        const int c = c0 + u * halves;
-        const bool in = c < n_slots;
-        m12[u] = in ? __ldcg(pm + (long long)c * R) : -INFINITY;
-        z12[u] = in ? __ldcg(pz + (long long)c * R) : 0.f;
+// The part that share i of n takes of T items, and its inverse (the index whose
+// range holds tile x of the group): shares differ by one tile at most.
+__device__ __forceinline__ int split_begin(int i, int T, int n) { return (int)(((unsigned)i * (unsigned)T) / (unsigned)n); }
+__device__ __forceinline__ int split_index(int x, int T, int n) {
+  return (int)((((unsigned)x + 1u) * (unsigned)n - 1u) / (unsigned)T);
+}
+// Row statistics in global memory, per segment and row: acc = the sum of 2^score over all keys, in fp64 and without a
+// reference.  The terms are fp32 sums over one tile each, a few million times 2^-24 apart at most, so their fp64 sum is
+// exact in any order: shares are added atomically and the result depends neither on timing nor on how the keys were split.
+// Scores beyond fp64's range (above 900 or below -900 in log2 units) go elsewhere: share `slot` then holds such a part of
+// the row's sum as z * 2^m, and its bit in far[] is set.
+constexpr float kFarScore = 900.f;
+constexpr int kFarWords = kMaxSplit / 32;
+struct StatView {
+  double* acc;                 // [n_seg][R]
+  unsigned* far;               // [n_seg][kFarWords]; acc and far are cleared before use
+  float* far_z;                // [n_seg][stride][R]
+  float* far_m;                // likewise
+  float* lse;                  // [n_seg][R], where a kernel of its own merges (log2 units)
+};
+__host__ __device__ __forceinline__ size_t stat_clear_bytes(int n_seg, int R) {
+  return (size_t)n_seg * R * sizeof(double) + (size_t)n_seg * kFarWords * sizeof(unsigned);
+}
+__device__ __forceinline__ StatView stat_view(void* part, int n_seg, int R, int stride) {
+  StatView v;
+  v.acc = static_cast<double*>(part);
+  v.far = reinterpret_cast<unsigned*>(v.acc + (size_t)n_seg * R);
+  v.far_z = reinterpret_cast<float*>(v.far + (size_t)n_seg * kFarWords);
+  v.far_m = v.far_z + (size_t)n_seg * stride * R;
+  v.lse = v.far_m + (size_t)n_seg * stride * R;
+  return v;
+}
+// Folds (zo, mo) into (z, m): sums of 2^(x - m) with different references.
+__device__ __forceinline__ void stat_add(float& z, float& m, float zo, float mo) {
+  if (!(zo > 0.f)) return;
+  const float mn = z > 0.f ? fmaxf(m, mo) : mo;
+  z = (z > 0.f ? z * ex2(m - mn) : 0.f) + zo * ex2(mo - mn);
+  m = mn;
+}
+// log2 of a positive fp64 number, in fp32 arithmetic on its fraction and exponent.
+__device__ __forceinline__ float log2_of(double Z) {
+  const int hi = __double2hiint(Z);
+  return __fadd_rn((float)((hi >> 20) - 1023), log2f((float)__hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(Z))));
+}
+// The log-sum-exp (log2 units) of a row from its sum Z, the far parts of its segment's n_slots shares if there are any, and
+// the window keys' statistics (wm, wz), if any.  One definition for every kernel that merges.
+__device__ __forceinline__ float row_lse(const StatView& st, double Z, bool any_far, int seg, int row, int R, int stride,
+                                         int n_slots, bool has_win, float wm, float wz) {
+  if (!any_far && !has_win) return log2_of(Z);
+  float z = 0.f, m = 0.f;
+  if (Z > 0.0) {
+    m = (float)((__double2hiint(Z) >> 20) - 1023);
+    z = (float)__hiloint2double((__double2hiint(Z) & 0xfffff) | 0x3ff00000, __double2loint(Z));
+  }
+  if (any_far)
+    for (int c = 0; c < n_slots; ++c)
+      if (__ldcg(st.far + (size_t)seg * kFarWords + (c >> 5)) >> (c & 31) & 1u) {
+        const size_t at = ((size_t)seg * stride + c) * R + row;
+        stat_add(z, m, __ldcg(st.far_z + at), __ldcg(st.far_m + at));
       }
-#pragma unroll
-      for (int u = 0; u < 12; ++u)
-        if (z12[u] > 0.f) {                                                // empty partials carry z = 0
-          const float Mn = fmaxf(M, m12[u]);
-          Z = fmaf(Z, ex2(M - Mn), __fmul_rn(z12[u], ex2(m12[u] - Mn)));   // ex2(-inf) = 0 covers the first term;
-                                                                           // explicit rounding: the same in every kernel
-          M = Mn;
-        }
-    }
-  }
-  if (halves == 2) {                                                       // uniform over the warp
-    const float M1 = __shfl_xor_sync(0xffffffffu, M, 1), Z1 = __shfl_xor_sync(0xffffffffu, Z, 1);
-    const float Mn = fmaxf(M, M1);
-    float Zt = 0.f;
-    if (M > -INFINITY) Zt = __fmul_rn(Z, ex2(M - Mn));
-    if (M1 > -INFINITY) Zt = __fadd_rn(Zt, __fmul_rn(Z1, ex2(M1 - Mn)));
-    M = Mn; Z = Zt;
-  }
-  if (has_win && wz > 0.f) {
-    const float Mn = fmaxf(M, wm);
-    Z = __fadd_rn(M > -INFINITY ? __fmul_rn(Z, ex2(M - Mn)) : 0.f, __fmul_rn(wz, ex2(wm - Mn)));
-    M = Mn;
-  }
-  return __fadd_rn(M, log2f(Z));
+  if (has_win) stat_add(z, m, wz, wm);
+  return __fadd_rn(m, log2f(z));
 }
 
+// A run = consecutive tiles of one segment inside the CTA's range [begin, end) of a layer's flat tile list.
 struct Run { int s, g, t0, count, n_hist, seg_tile0, tiles_seg; };
 
-// A run = consecutive tiles of one segment inside the CTA's range [begin, end).  Forward walks (pass 1)
-// name a run by its first tile, backward walks (pass 2) by its last one.
-__device__ __forceinline__ Run locate(const TcArgs& a, int pos, int begin, int end, bool REV) {
+__device__ __forceinline__ Run locate(const ScoreShape& a, int pos, int end) {
   int lo = 0, hi = a.n_seqs;                       // last s with Hkv*tile_off[s] <= pos
   while (hi - lo > 1) {
     int mid = (lo + hi) >> 1;
@@ -246,84 +269,39 @@ __device__ __forceinline__ Run locate(const TcArgs& a, int pos, int begin, int e
   r.tiles_seg = a.tab.tile_at(lo + 1) - a.tab.tile_at(lo);
   const int rel = pos - a.n_kv_heads * a.tab.tile_at(lo);
   r.g = rel / r.tiles_seg;
-  const int t = rel - r.g * r.tiles_seg;
-  r.seg_tile0 = pos - t;
-  if (REV) {
-    r.t0 = max(r.seg_tile0, begin) - r.seg_tile0;
-    r.count = t - r.t0 + 1;
-  } else {
-    r.t0 = t;
-    r.count = min(end - pos, r.tiles_seg - t);
-  }
+  r.t0 = rel - r.g * r.tiles_seg;
+  r.seg_tile0 = pos - r.t0;
+  r.count = min(end - pos, r.tiles_seg - r.t0);
   r.n_hist = max(a.tab.cu_at(lo + 1) - a.tab.cu_at(lo) - a.window, 0);
   return r;
 }
 
-// sum_e 2^(v_e * sc - m) over 32 accumulator values, four independent chains
-__device__ __forceinline__ float sum_ex2_32(const uint32_t (&r)[32], float sc, float m) {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-  for (int e = 0; e < 32; e += 4) {
-    s0 += ex2(fmaf(__uint_as_float(r[e]), sc, -m));
-    s1 += ex2(fmaf(__uint_as_float(r[e + 1]), sc, -m));
-    s2 += ex2(fmaf(__uint_as_float(r[e + 2]), sc, -m));
-    s3 += ex2_fma(fmaf(__uint_as_float(r[e + 3]), sc, -m), true);
-  }
-  return (s0 + s1) + (s2 + s3);
-}
-// Adds one chunk of 32 accumulator values (the first nv of them) to a row's (reference m, sum z) pair exactly:
-// the reference moves to the running maximum and the sum is rescaled.  Taken when the fixed-reference sum of the
-// chunk over- or underflowed; works on the registers, so the accumulator may already be back with the tensor pipe.
-__device__ __noinline__ void chunk_stats_exact(const uint32_t (&r)[32], float sc, int nv, float& m_io, float& z_io) {
-  float mx = -INFINITY;
-#pragma unroll
-  for (int e = 0; e < 32; ++e)
-    if (e < nv) mx = fmaxf(mx, __uint_as_float(r[e]) * sc);
-  if (!(mx > -INFINITY)) return;                       // nothing valid (or only -inf scores)
-  const float m_new = z_io > 0.f ? fmaxf(m_io, mx) : mx;
-  float z = z_io > 0.f ? z_io * ex2(m_io - m_new) : 0.f;
-#pragma unroll
-  for (int e = 0; e < 32; ++e)
-    if (e < nv) z += ex2(fmaf(__uint_as_float(r[e]), sc, -m_new));
-  m_io = m_new; z_io = z;
-}
-__device__ __forceinline__ float max_32(const uint32_t (&r)[32], int n_valid_here) {
-  float t[32];
-#pragma unroll
-  for (int e = 0; e < 32; ++e) t[e] = e < n_valid_here ? __uint_as_float(r[e]) : -INFINITY;
-#pragma unroll
-  for (int w = 16; w >= 1; w >>= 1)
-#pragma unroll
-    for (int e = 0; e < w; ++e) t[e] = fmaxf(t[e], t[e + w]);
-  return t[0];
-}
-
-// Pass 1, exact path for one 128-row accumulator: running maximum and rescaled sum over the tile's first n_valid
-// keys.  Used for a segment's ragged last tile and when the fast path over- or underflows.  A function of its
-// own (not inlined) so that a CTA which will need it can run it once before the K stream starts: fetching
-// these instructions for the first time while the stream saturates the memory system stalled the tile for
-// microseconds.
-__device__ __noinline__ void tile_row_stats_exact(uint32_t tcol, float sc, int n_valid, float& m_io, float& z_io) {
-  uint32_t ra[32];
-  float m = m_io, z = z_io;
+// Statistics pass, exact path for this thread's row of one accumulator: z * 2^m = the sum over the tile's first n_valid
+// keys, m a whole number.  Used when the sum of the fast path over- or underflows.  Eight columns at a time: inlined beside
+// the fast path, it must not need registers of its own.
+__device__ __forceinline__ void tile_stats_exact(uint32_t tcol, float sc, int n_valid, float& m, float& z) {
+  m = 0.f;
+  z = 0.f;
 #pragma unroll 1
-  for (int c0 = 0; c0 < kTileKeys; c0 += 32) {
-    if (c0 >= n_valid) break;
-    tc_ld32_issue(tcol + c0, ra);
-    tc_ld_wait(ra);
-    // the reference a row starts with (0) is a guess, not a score: while nothing has been summed it gives way to
-    // the first maximum seen, however low
-    const float mx = max_32(ra, n_valid - c0) * sc;
-    const float mn = z > 0.f ? fmaxf(m, mx) : mx;
+  for (int c0 = 0; c0 < kTileKeys && c0 < n_valid; c0 += 8) {
+    uint32_t r[8];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(tcol + c0) : "memory");
+    float mx = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (c0 + e < n_valid) mx = fmaxf(mx, __uint_as_float(r[e]) * sc);
+    const bool any = mx > -INFINITY && mx < INFINITY;    // not only -inf scores
+    const float mn = !any ? m : (z > 0.f ? fmaxf(m, ceilf(mx)) : ceilf(mx));
     z = z > 0.f ? z * ex2(m - mn) : 0.f;
     m = mn;
-    float zc = 0.f;
 #pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (e < n_valid - c0) zc += ex2(fmaf(__uint_as_float(ra[e]), sc, -m));
-    z += zc;
+    for (int e = 0; e < 8; ++e)
+      if (any && c0 + e < n_valid) z += ex2(fmaf(__uint_as_float(r[e]), sc, -m));
   }
-  m_io = m; z_io = z;
 }
 
 }  // namespace

@@ -1,0 +1,78 @@
+"""GPU: the list score kernel at the sizes where its walk can go wrong -- rows that fill no 32-column block, one and two
+row blocks, both head dimensions, fewer tiles than CTAs, ragged last tiles, short layers sharing a group, lists that end
+in mid-group -- against the oracle, and against the same layers one call at a time."""
+import numpy as np
+import pytest
+import torch
+
+import parity as P
+from oracle import slkv_oracle as O
+from paper_2508_15806_b200 import binding as B
+from paper_2508_15806_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+def layer(seed, lens, hq, hkv, d, w):
+    g = torch.Generator().manual_seed(seed)
+    T = sum(lens)
+    q = torch.randn(len(lens), w, hq, d, generator=g)
+    k = torch.randn(T, hkv, d, generator=g) * torch.exp(0.5 * torch.randn(T, hkv, 1, generator=g))
+    return q.bfloat16(), k.bfloat16(), torch.randn(T, hkv, d, generator=g).bfloat16()
+
+
+@pytest.mark.parametrize("hq,hkv,d,w", [(4, 4, 64, 5), (8, 8, 128, 16), (6, 2, 64, 16), (8, 2, 128, 33), (8, 1, 64, 31),
+                                        (8, 2, 128, 64), (2, 2, 128, 129)])
+@pytest.mark.parametrize("lens", [[w0 for w0 in (700,)], [130, 1, 515, 257]])
+def test_rows_and_head_dims(hq, hkv, d, w, lens):
+    q, k, v = layer(hq * 100 + d + w + len(lens), lens, hq, hkv, d, w)
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    P.check_compress(q, k, v, cu, [w + 40] * hkv, w, 5, score_path=B.SLKV_PATH_TENSOR)
+
+
+@pytest.mark.parametrize("lens,n_layers,w,lse", [([300], 3, 32, False), ([4001], 19, 32, False), ([900, 33, 2000], 35, 16, True),
+                                                 ([9000, 20000], 5, 64, False), ([40000], 3, 32, False)])
+def test_lists_match_single_calls(lens, n_layers, w, lse):
+    hq, hkv, d = 16, 4, 128
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    xs = [tuple(t.to(DEV) for t in layer(50 + l, lens, hq, hkv, d, w)) for l in range(n_layers)]
+    p = B.make_params(*xs[0], w, 7)
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
+    bud = torch.tensor([w + 30 * (h + 1) for h in range(hkv)], dtype=torch.int32, device=DEV)
+    cap = sum(min(n, int(b)) for n in lens for b in bud.tolist())
+    ws = torch.empty(B.slkv_workspace_bytes_overlapped(p, cu), dtype=torch.uint8, device=DEV)
+    got = {}
+    for fn in (B.slkv_compress, B.slkv_compress_overlapped):
+        outs = []
+        for q, k, v in xs:
+            stats = None
+            if lse:
+                stats = torch.zeros(len(lens), hq, w, dtype=torch.float32, device=DEV)
+                B.slkv_row_lse(p, q, k, cu_dev, cu, stats, torch.empty_like(ws))
+            o = [torch.zeros(cap, d, dtype=torch.bfloat16, device=DEV), torch.zeros(cap, d, dtype=torch.bfloat16, device=DEV),
+                 torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.zeros(cap, dtype=torch.int32, device=DEV),
+                 torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV), stats]
+            fn(p, q, k, v, cu_dev, cu, bud, *o[:4], ws, o[4], o[5], lse=stats)
+            outs.append(o)
+        B.slkv_join()
+        torch.cuda.synchronize()
+        got[fn.__name__] = outs
+    for a, b in zip(*got.values()):
+        assert int(a[5]) == 0 and int(b[5]) == 0
+        for x, y in zip(a[:5], b[:5]):
+            assert torch.equal(x, y)
+
+
+def test_scores_beyond_the_range_of_sums_without_a_reference():
+    # logits of several thousand, some rows only far below zero: the rows' sums leave fp64's range
+    q, k, v = layer(9, [1500], 8, 2, 128, 32)
+    q, k = q * 40, k * 40
+    k[:, :, 0] += 300.0
+    q[:, :16, :, 0] = 80.0
+    q[:, 16:, :, 0] = -80.0
+    lse = P.gpu_row_lse(q, k, [0, 1500], 32)
+    ref = O.row_lse(P.to_np64(q), P.to_np64(k), [0, 1500], 32, "history")
+    got, ref = lse.cpu().double().numpy(), np.asarray(ref)
+    assert np.all(np.isfinite(got)) and np.abs(ref).max() > 2000
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-5
