@@ -33,7 +33,6 @@ constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 constexpr int kMaxWindow = 256;
-constexpr size_t kSimtSmemLimit = 192 * 1024;
 
 int cuda_fail(cudaError_t e) {
   g_last_cuda_error = (int)e;
@@ -81,13 +80,14 @@ int describe(const slkv_params* p, const int32_t* cu_host, Problem* pb) {
   if (p->history_only && (cu_host[1] < 0 || (int64_t)cu_host[1] + p->window >= (1ll << 31))) return SLKV_ERR_BAD_SHAPE;
   const int32_t cu_virtual[2] = {0, p->history_only ? cu_host[1] + p->window : 0};
   if (p->history_only) cu_host = cu_virtual;
-  int64_t total_hist = 0;
+  int64_t total_hist = 0, tiles = 0;
   int max_hist = 0;
   for (int s = 0; s < p->n_seqs; ++s) {
     int64_t len = (int64_t)cu_host[s + 1] - cu_host[s];
     if (len < 0) return SLKV_ERR_BAD_SHAPE;
     int64_t nh = len > p->window ? len - p->window : 0;
     total_hist += nh;
+    tiles += (nh + 127) / 128;
     if (nh > max_hist) max_hist = (int)nh;
   }
   const int64_t T = cu_host[p->n_seqs];
@@ -104,6 +104,7 @@ int describe(const slkv_params* p, const int32_t* cu_host, Problem* pb) {
     pb->cu_virtual[0] = cu_virtual[0]; pb->cu_virtual[1] = cu_virtual[1];
   }
   pb->total_hist = total_hist;
+  pb->n_tiles128 = tiles * p->n_kv_heads;
   pb->n_seg = p->n_seqs * p->n_kv_heads;
   if (p->n_seqs <= kInlineSeqs) {
     pb->tab.n_inline = p->n_seqs;
@@ -144,11 +145,10 @@ Layout layout_of(const Problem& pb, bool overlapped = false) {
   L.layer0 = o;
   size_t q = 0;
   L.vote = q; q = align_up(q + votes);
-  // row statistics per split range (tensor-core path: see stat_view) or chunk that shares a segment
+  // row statistics: see stat_view (tensor cores), SimtStats
   const size_t shares = (size_t)tensor_slot_stride(pb);
-  const size_t chunks = (size_t)(pb.max_hist + simt_chunk_keys() - 1) / simt_chunk_keys();
   const size_t by_tensor = (size_t)pb.n_seg * ((shares * 8 + 12) * (size_t)pb.R + kMaxSplit / 8);
-  const size_t by_simt = (size_t)pb.n_seg * pb.R * chunks * 8;
+  const size_t by_simt = simt_part_bytes(pb);
   L.part = q; q = align_up(q + (by_tensor > by_simt ? by_tensor : by_simt));
   L.gather_src = q; q = align_up(q + (size_t)pb.p.n_kv_heads * (size_t)pb.total_tokens * sizeof(int32_t));
   // row statistics over the window keys (all-causal softmax domain): [n_seg][R] maxima and sums
@@ -166,13 +166,12 @@ int resolve_path(const Problem& pb, int* path) {
   const bool tensor_ok = tensor_path_supported(pb.p);
   if (want == SLKV_PATH_AUTO) want = tensor_ok ? SLKV_PATH_TENSOR : SLKV_PATH_SIMT;
   if (want == SLKV_PATH_TENSOR && !tensor_ok) return SLKV_ERR_BAD_DTYPE;
-  if (want == SLKV_PATH_SIMT && simt_smem_bytes(pb) > kSimtSmemLimit) return SLKV_ERR_BAD_SHAPE;
   *path = want;
   return SLKV_OK;
 }
 
 // slot: the layer's place in the list (overlapped calls)
-void carve(Problem* pb, const Layout& L, void* ws, int path, int slot) {
+void carve(Problem* pb, const Layout& L, void* ws, int slot) {
   unsigned char* b = static_cast<unsigned char*>(ws);
   pb->hist_off = reinterpret_cast<int64_t*>(b + L.hist_off);
   pb->tile_off = reinterpret_cast<int32_t*>(b + L.tile_off);
@@ -186,17 +185,13 @@ void carve(Problem* pb, const Layout& L, void* ws, int path, int slot) {
   pb->gather_src = reinterpret_cast<int32_t*>(l + L.gather_src);
   pb->win_m = reinterpret_cast<float*>(l + L.win_m);
   pb->win_z = reinterpret_cast<float*>(l + L.win_z);
-  pb->chunk_keys = path == SLKV_PATH_TENSOR ? 128 : simt_chunk_keys();
-  pb->n_chunks = path == SLKV_PATH_TENSOR ? tensor_slot_stride(*pb)
-                                          : (pb->max_hist + pb->chunk_keys - 1) / pb->chunk_keys;
-  if (pb->n_chunks < 1) pb->n_chunks = 1;
 }
-int bind_workspace(Problem* pb, void* ws, size_t ws_bytes, int path) {
+int bind_workspace(Problem* pb, void* ws, size_t ws_bytes) {
   if (!ws) return SLKV_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SLKV_ERR_BAD_ALIGN;
   const Layout L = layout_of(*pb);
   if (ws_bytes < L.total) return SLKV_ERR_WORKSPACE;
-  carve(pb, L, ws, path, 0);
+  carve(pb, L, ws, 0);
   return SLKV_OK;
 }
 
@@ -218,7 +213,7 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
   if (rc != SLKV_OK) return rc;
   const int passes = pb.lse_opt ? 2 : 3;
   cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes, nullptr, st, launches)
-                                           : launch_score_simt(pb, passes, st, launches);
+                                           : launch_score_simt(pb, status, passes, st, launches);
   if (e != cudaSuccess) return cuda_fail(e);
   return SLKV_OK;
 }
@@ -407,7 +402,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
         e = flush_list(s, st, &launches);                    // layers of the shape before
         if (e != cudaSuccess) return cuda_fail(e);
         s->open = false;
-        carve(&pb, L, ws, path, 0);
+        carve(&pb, L, ws, 0);
         pb.cu = cu_dev; pb.tab.cu_ptr = cu_dev;
         pb.q = q_win; pb.k = k; pb.v = v; pb.lse_opt = lse_opt;
         e = plan_score_tensor(pb, cu_host, status, &s->plan);
@@ -424,7 +419,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
       e = drain_states_sharing(d, s, ws, ws_bytes, st, &launches);
       if (e != cudaSuccess) return cuda_fail(e);
       Problem& pb = s->pb;
-      carve(&pb, s->layout, ws, SLKV_PATH_TENSOR, s->n);
+      carve(&pb, s->layout, ws, s->n);
       pb.q = q_win; pb.k = k; pb.v = v; pb.lse_opt = lse_opt;
       e = plan_score_layer(pb, status, &s->score[s->n]);
       if (e != cudaSuccess) return cuda_fail(e);
@@ -451,7 +446,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   int path = 0;
   rc = resolve_path(pb, &path);
   if (rc != SLKV_OK) return rc;
-  rc = bind_workspace(&pb, ws, ws_bytes, path);
+  rc = bind_workspace(&pb, ws, ws_bytes);
   if (rc != SLKV_OK) return rc;
   cudaError_t e = join_lists(st, &launches);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -779,7 +774,7 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
   int path = 0;
   rc = resolve_path(pb, &path);
   if (rc != SLKV_OK) return rc;
-  rc = bind_workspace(&pb, workspace, workspace_bytes, path);
+  rc = bind_workspace(&pb, workspace, workspace_bytes);
   if (rc != SLKV_OK) return rc;
   pb.cu = cu_seqlens_dev; pb.q = q_win; pb.k = k; pb.v = nullptr;
   pb.tab.cu_ptr = cu_seqlens_dev;
@@ -798,7 +793,7 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
     rc = enqueue_window_stats(pb, path, st, &launches);
     if (rc != SLKV_OK) return rc;
     e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_seqlens_host, status, 1, lse_out, st, &launches)
-                                 : launch_score_simt(pb, 1, st, &launches);
+                                 : launch_score_simt(pb, status, 1, st, &launches);
     if (e == cudaSuccess && path != SLKV_PATH_TENSOR) e = launch_merge_lse_simt(pb, lse_out, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
     g_last_launches = launches;

@@ -108,8 +108,7 @@ struct Problem {
   int32_t* tile_off;      // [n_seqs+1] exclusive prefix of ceil(n_hist_s / 128)
   float* vote;            // [n_kv_heads * total_hist] ragged, same layout as pooled
   void* part;             // partial row statistics; layout of the score path
-  int n_chunks;           // chunks per segment (stride of part_*), per score path
-  int chunk_keys;         // keys per chunk
+  int64_t n_tiles128;     // 128-key tiles of all segments
   float* pooled_ws;       // [n_kv_heads * total_hist] used when the caller wants no pooled output
   int32_t* gather_src;    // [n_kv_heads * total_tokens] per packed row: token * n_kv_heads + head of its source
   int32_t* dev_flags;     // [8] scratch words (timeouts etc.)
@@ -165,10 +164,9 @@ cudaError_t launch_cp_emit(const float* pooled, long long row_stride, int own_be
 int cp_slices(int own_count);            // CTAs per head of the counting and packing kernels
 cudaError_t launch_setup(const Problem& pb, const int32_t* budgets, int32_t* offsets, int64_t capacity,
                          int32_t* status, cudaStream_t st, int* launches);
-int simt_chunk_keys();
-size_t simt_smem_bytes(const Problem& pb);
+size_t simt_part_bytes(const Problem& pb);
 // passes: 1 = row statistics only, 2 = votes only (the log-sum-exps come from lse_source_of), 3 = both
-cudaError_t launch_score_simt(const Problem& pb, int passes, cudaStream_t st, int* launches);
+cudaError_t launch_score_simt(const Problem& pb, int32_t* status, int passes, cudaStream_t st, int* launches);
 // Row statistics of the window keys each window row sees causally (SLKV_ALL_CAUSAL) -> pb.win_m / pb.win_z, rows in
 // the order of the score path (head_inner: r = i*G + hh).
 cudaError_t launch_window_stats(const Problem& pb, bool head_inner, cudaStream_t st, int* launches);

@@ -1,24 +1,45 @@
 // Window relevance scores with fp32 FMA arithmetic (Sec. 3.4, Eq. 7; Algorithm 3 l.6; Eq. 3-4).
 //
-// Serves the fp32 configuration and every shape the tensor-core kernels do not take.  One thread owns
-// one history key (its row of K lives in registers), the G*w query rows of the KV head's group sit in
-// shared memory, and a CTA walks a chunk of key tiles:
-//   pass 1  per query row: running max and sum of 2^(s - max) over the chunk's keys -> part_m / part_z
-//   pass 2  merges the chunks' partials into the row's log-sum-exp, then per key
-//           vote[j] = (1/G) sum_rows 2^(s_rj - lse_r)      (s in log2 units: s = q.k * log2(e)/sqrt(d))
-// The w x n_hist probability matrix never exists in memory.
+// Serves the fp32 configuration and every shape the tensor-core kernel does not take.  A register-tiled product: a CTA of
+// 256 threads forms 64 keys x 64 rows of scores at a time, 4 x 4 per thread in packed pairs (fma.rn.f32x2) over the head
+// dimension, K and Q as fp32 rows in shared memory, padded so that the 16-byte loads of a warp -- eight key groups, four row
+// groups -- are one wavefront each; eight of those feed 64 multiply-adds.  Persistent CTAs walk the segments' key tiles:
+//   statistics  row sums of 2^score per 32 keys, added up in fp64 with atomics (the order shows at 2^-53, not in the
+//               fp32 results); nothing is subtracted unless a sum over- or underflows, in which case every CTA learns so at
+//               the barrier and two more rounds find the rows' maxima and sum relative to them;
+//   votes       vote[j] = (1/G) sum_rows 2^(s_rj - lse_r), rows in a fixed order.
+// Both passes are one cooperative launch with a grid-wide barrier between them; score tiles that fit in shared memory are
+// kept over the barrier instead of being formed again.
+// What bounds it: latency at the small sizes (1024 tokens, 8 heads, 16 rows: two dot-product loops of one thread per key and
+// two launches took 80 us, this takes 10), the FMA pipe at the large ones.
+#include <atomic>
+#include <cstring>
+
 #include "slkv_internal.cuh"
 
 namespace slkv {
 namespace {
 
-constexpr int kThreads = 128;          // keys per tile
-constexpr int kTilesPerChunk = 8;      // key tiles a CTA walks
-constexpr int kRowBatch = 8;           // query rows reduced together in pass 1
+constexpr int kThreads = 256;
+constexpr int kKeys = 64;              // keys per tile
+constexpr int kRows = 64;              // rows per step
+constexpr int kSmemMost = 200 * 1024;
+constexpr unsigned long long kWaitLimitNs = 1000ull * 1000ull * 1000ull;
 
-template <typename T> struct Vec;      // 16-byte vector of T
-template <> struct Vec<float> { static constexpr int N = 4; };
-template <> struct Vec<__nv_bfloat16> { static constexpr int N = 8; };
+// stages of a launch
+enum { kStats = 1, kMaxima = 2, kFarSums = 4, kVotes = 8 };
+
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float sum_of(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a + b;
+}
 
 __device__ __forceinline__ void unpack(const uint4& u, float (&f)[4], float) {
   f[0] = __uint_as_float(u.x); f[1] = __uint_as_float(u.y); f[2] = __uint_as_float(u.z); f[3] = __uint_as_float(u.w);
@@ -31,281 +52,561 @@ __device__ __forceinline__ void unpack(const uint4& u, float (&f)[8], __nv_bfloa
   f[6] = __uint_as_float(u.w << 16); f[7] = __uint_as_float(u.w & 0xffff0000u);
 }
 
-template <typename T, int D>
-__device__ __forceinline__ float dot_row(const T* __restrict__ qrow /*smem*/, const float (&kreg)[D]) {
-  constexpr int VN = Vec<T>::N;
-  float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll
-  for (int c = 0; c < D / VN; ++c) {
-    uint4 u = *reinterpret_cast<const uint4*>(qrow + c * VN);
-    float f[VN];
-    unpack(u, f, T());
-#pragma unroll
-    for (int e = 0; e < VN; e += 2) {
-      acc0 = fmaf(f[e], kreg[c * VN + e], acc0);
-      acc1 = fmaf(f[e + 1], kreg[c * VN + e + 1], acc1);
-    }
+// The statistics area (pb.part): per segment and row the fp64 sum, then the same over relative to the row's maximum, then
+// the maxima (order-preserving integers), then one word: some sum over- or underflowed.  Cleared before use.
+struct SimtStats {
+  double* acc;
+  double* acc_far;
+  unsigned* row_max;
+  unsigned* far;
+};
+size_t simt_stat_bytes(int n_seg, int R) { return (size_t)n_seg * R * 20 + 8; }
+__host__ __device__ __forceinline__ SimtStats simt_stats(void* part, int n_seg, int R) {
+  SimtStats s;
+  s.acc = static_cast<double*>(part);
+  s.acc_far = s.acc + (size_t)n_seg * R;
+  s.row_max = reinterpret_cast<unsigned*>(s.acc_far + (size_t)n_seg * R);
+  s.far = s.row_max + (size_t)n_seg * R;
+  return s;
+}
+// order-preserving map of floats to unsigned integers; 0 is below every float
+__device__ __forceinline__ unsigned ordered(float x) {
+  const unsigned u = __float_as_uint(x);
+  return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float unordered(unsigned u) { return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u); }
+
+// Row log-sum-exp (log2 units), the window keys' statistics folded in when there are any (softmax over all causally
+// visible keys).  The same operations in every kernel that forms it.
+__device__ __forceinline__ float simt_row_lse(const SimtStats& st, size_t at, bool far, bool has_win, float wm, float wz) {
+  float M = far ? unordered(__ldcg(st.row_max + at)) : 0.f;
+  double Z = __ldcg((far ? st.acc_far : st.acc) + at);
+  if (has_win) {
+    const float Mn = fmaxf(M, wm);
+    Z = __dadd_rn(__dmul_rn(Z, (double)exp2f(M - Mn)), __dmul_rn((double)wz, (double)exp2f(wm - Mn)));
+    M = Mn;
   }
-  return acc0 + acc1;
+  return __fadd_rn(M, (float)log2(Z));
 }
 
-// Row log-sum-exp (log2 units) from the per-chunk statistics of the SIMT layout [row][chunk], the window keys'
-// statistics folded in when there are any (softmax over all causally visible keys).
-__device__ __forceinline__ float simt_row_lse(const float* pm, const float* pz, int nc, bool has_win, float wm,
-                                              float wz) {
-  float M = -INFINITY;
-  for (int c = 0; c < nc; ++c) M = fmaxf(M, pm[c]);
-  if (has_win) M = fmaxf(M, wm);
-  float Z = 0.f;
-  for (int c = 0; c < nc; ++c) Z = fmaf(pz[c], exp2f(pm[c] - M), Z);      // explicit rounding: the same in every kernel
-  if (has_win) Z = fmaf(wz, exp2f(wm - M), Z);
-  return __fadd_rn(M, log2f(Z));
-}
+struct SimtArgs {
+  SeqTables tab;
+  const void* q;
+  const void* k;
+  void* part;
+  float* vote;
+  LseSource lse;
+  int32_t* status;
+  int n_seqs, n_kv_heads, G, window, R, n_tiles, keep, q_rows, stages, coop, barrier_extra;
+  long long k_stride_tok, k_stride_head, q_stride_seq, q_stride_row, q_stride_head;
+  float scale_log2;
+  unsigned* counters;          // [8], zero: arrivals at the launch's barriers, CTAs that are done
+};
+constexpr int kCountSlots = 64;
+__device__ unsigned g_simt_counters[kCountSlots * 8];
 
-template <typename T, int D, int PASS>
-__global__ void __launch_bounds__(kThreads)
-k_score_simt(const T* __restrict__ q, const T* __restrict__ k, const __grid_constant__ SeqTables tab,
-             float* __restrict__ part_m, float* __restrict__ part_z,
-             float* __restrict__ vote, const LseSource lse, int n_kv_heads, int G, int window, int n_chunks, long long k_stride_tok,
-             long long k_stride_head, long long q_stride_seq, long long q_stride_row, long long q_stride_head,
-             float scale_log2) {
-  constexpr int VN = Vec<T>::N;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int R = G * window;
-  T* qs = reinterpret_cast<T*>(smem_raw);                               // [R][D]
-  float* fbuf = reinterpret_cast<float*>(smem_raw + (size_t)R * D * sizeof(T));
-  float* run_m = fbuf;                                                  // [R]  (pass 2: lse per row)
-  float* run_z = fbuf + R;                                              // [R]
-  float* wred = fbuf + 2 * R;                                           // [2][kRowBatch][4]
-
-  const int chunk = blockIdx.x, g = blockIdx.y, s = blockIdx.z;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  pdl_launch_dependents();
-  pdl_wait();
-  const int t0 = tab.cu_at(s);
-  const int n_hist = max(tab.cu_at(s + 1) - t0 - window, 0);
-  const int key0 = chunk * (kThreads * kTilesPerChunk);
-  if (key0 >= n_hist) return;
-  const int seg = s * n_kv_heads + g;
-
-  // the group's query rows: row r = hh*window + i  <->  query head g*G + hh, window row i
-  for (int idx = tid; idx < R * (D / VN); idx += kThreads) {
-    int r = idx / (D / VN), c = idx - r * (D / VN);
-    int hh = r / window, i = r - hh * window;
-    const T* src = q + s * q_stride_seq + i * q_stride_row + (long long)(g * G + hh) * q_stride_head + c * VN;
-    *reinterpret_cast<uint4*>(qs + r * D + c * VN) = *reinterpret_cast<const uint4*>(src);
-  }
-  if (PASS == 1) {
-    for (int r = tid; r < R; r += kThreads) { run_m[r] = -INFINITY; run_z[r] = 0.f; }
-  } else {
-    const int nc = (n_hist + kThreads * kTilesPerChunk - 1) / (kThreads * kTilesPerChunk);
-    for (int r = tid; r < R; r += kThreads) {
-      if (lse.lse_opt) {                                                  // the caller's row statistics
-        run_m[r] = lse.caller_lse(s, g, r, G, window, false);
-        continue;
-      }
-      const float* pm = part_m + ((long long)seg * R + r) * n_chunks;
-      const float* pz = part_z + ((long long)seg * R + r) * n_chunks;
-      const bool has_win = lse.win_m != nullptr;
-      run_m[r] = simt_row_lse(pm, pz, nc, has_win, has_win ? lse.win_m[(long long)seg * R + r] : 0.f,
-                              has_win ? lse.win_z[(long long)seg * R + r] : 0.f);
+// Waits, in one thread, until counter b has reached `target`.
+__device__ __forceinline__ int count_wait(const SimtArgs& a, int b, unsigned target) {
+  unsigned long long t0 = 0, t;
+  for (unsigned spin = 0;; ++spin) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.counters + b) : "memory");
+    if (v >= target) return 1;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    if (spin == 0) t0 = t;
+    if (t - t0 > kWaitLimitNs) {
+      if (a.status) atomicExch(a.status, (int)SLKV_ERR_DEVICE_TIMEOUT);
+      return 0;
     }
+    __nanosleep(20);
+  }
+}
+// Arrives at barrier number b of the launch and waits for all CTAs (bounded: false when the wait ran out).
+__device__ __forceinline__ bool grid_wait(const SimtArgs& a, int b, unsigned extra) {
+  __shared__ int ok_sh;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + b) : "memory");
+    ok_sh = count_wait(a, b, gridDim.x + extra);
   }
   __syncthreads();
+  return ok_sh != 0;
+}
 
-  for (int tile = 0; tile < kTilesPerChunk; ++tile) {
-    const int j = key0 + tile * kThreads + tid;
-    if (key0 + tile * kThreads >= n_hist) break;
-    const bool valid = j < n_hist;
-    float kreg[D];
-    {
-      const T* krow = k + (long long)(t0 + (valid ? j : 0)) * k_stride_tok + (long long)g * k_stride_head;
-#pragma unroll
-      for (int c = 0; c < D / VN; ++c) {
-        uint4 u = *reinterpret_cast<const uint4*>(krow + c * VN);
-        float f[VN];
-        unpack(u, f, T());
-#pragma unroll
-        for (int e = 0; e < VN; ++e) kreg[c * VN + e] = f[e];
-      }
-    }
-    if (PASS == 1) {
-      for (int r0 = 0; r0 < R; r0 += kRowBatch) {
-        float sv[kRowBatch], bm[kRowBatch];
-#pragma unroll
-        for (int b = 0; b < kRowBatch; ++b) {
-          int r = min(r0 + b, R - 1);
-          float d = dot_row<T, D>(qs + r * D, kreg) * scale_log2;
-          sv[b] = valid ? d : -INFINITY;
-          float m = sv[b];
-          for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-          if (lane == 0) wred[b * 4 + wid] = m;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int b = 0; b < kRowBatch; ++b) {
-          bm[b] = fmaxf(fmaxf(wred[b * 4], wred[b * 4 + 1]), fmaxf(wred[b * 4 + 2], wred[b * 4 + 3]));
-          float e = exp2f(sv[b] - bm[b]);
-          for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-          if (lane == 0) wred[kRowBatch * 4 + b * 4 + wid] = e;
-        }
-        __syncthreads();
-        if (tid < kRowBatch && r0 + tid < R) {
-          const int r = r0 + tid;
-          const float* ws = wred + kRowBatch * 4 + tid * 4;
-          float bs = (ws[0] + ws[1]) + (ws[2] + ws[3]);
-          const float* wm = wred + tid * 4;                 // the batch's warp maxima are still in place
-          float tm = fmaxf(fmaxf(wm[0], wm[1]), fmaxf(wm[2], wm[3]));
-          float om = run_m[r], nm = fmaxf(om, tm);
-          run_z[r] = run_z[r] * exp2f(om - nm) + bs * exp2f(tm - nm);
-          run_m[r] = nm;
-        }
-        __syncthreads();
-      }
-    } else {
-      float acc = 0.f;
-      for (int r = 0; r < R; ++r) acc += exp2f(dot_row<T, D>(qs + r * D, kreg) * scale_log2 - run_m[r]);
-      if (valid) vote[tab.hist_at(s) * n_kv_heads + (long long)g * n_hist + j] = acc / (float)G;
-    }
+template <typename T, int D>
+struct Tiles {
+  static constexpr int kVec = 16 / sizeof(T);                  // elements of a 16-byte load
+  static constexpr int kPitch = D + 4;                         // floats per row in shared memory
+  static constexpr int kPerRow = D / kVec;                     // 16-byte loads per row
+  static constexpr int kLoads = kKeys * kPerRow / kThreads;    // ... per thread for a key tile
+};
+
+// Where a tile of the flat list lies.
+struct Place { int seg, s, g, tile, n_hist, key0, t0; };
+__device__ __forceinline__ Place place_of(const SimtArgs& a, int t) {
+  // tile_off of the tables counts 128-key tiles; here a sequence has two of these per such tile
+  int lo = 0, hi = a.n_seqs;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (2 * a.n_kv_heads * a.tab.tile_at(mid) <= t) lo = mid; else hi = mid;
   }
-  if (PASS == 1) {
+  Place p;
+  p.s = lo;
+  const int per_head = 2 * (a.tab.tile_at(lo + 1) - a.tab.tile_at(lo));
+  const int rel = t - 2 * a.n_kv_heads * a.tab.tile_at(lo);
+  p.g = rel / per_head;
+  p.tile = rel - p.g * per_head;
+  p.seg = p.s * a.n_kv_heads + p.g;
+  p.t0 = a.tab.cu_at(lo);
+  p.n_hist = max(a.tab.cu_at(lo + 1) - p.t0 - a.window, 0);
+  p.key0 = p.tile * kKeys;                                     // may lie past the end: nothing valid then
+  return p;
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kThreads)
+k_score_simt(const __grid_constant__ SimtArgs a) {
+  using TT = Tiles<T, D>;
+  extern __shared__ __align__(16) float smem[];
+  float* ks = smem;                                            // [kKeys][kPitch]
+  float* qs = ks + kKeys * TT::kPitch;                         // [q_rows][kPitch]
+  float* lse_sh = qs + a.q_rows * TT::kPitch;                  // [chunks * kRows]
+  const int chunks = (a.R + kRows - 1) / kRows;
+  float* part_sh = lse_sh + chunks * kRows;                    // [4][kKeys]
+  float* kept = part_sh + 4 * kKeys;                           // [keep][chunks][16][kThreads]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int kw = (warp & 1) * 32 + (lane & 7), rw = (warp >> 1) * 16 + (lane >> 3);   // keys kw + 8 i, rows rw + 4 j
+  const T* q = static_cast<const T*>(a.q);
+  const T* k = static_cast<const T*>(a.k);
+  const int n_seg = a.n_seqs * a.n_kv_heads;
+  const SimtStats st = simt_stats(a.part, n_seg, a.R);
+  const int begin = (int)((long long)blockIdx.x * a.n_tiles / gridDim.x), end = (int)((long long)(blockIdx.x + 1) * a.n_tiles / gridDim.x);
+  pdl_launch_dependents();
+  pdl_wait();
+
+  if (a.coop) {
+    // clear the statistics area; nobody adds to it before all CTAs have done their part
+    const int words = (int)((size_t)n_seg * a.R * 5 + 2);
+    const int w0 = (int)((long long)blockIdx.x * words / gridDim.x), w1 = (int)((long long)(blockIdx.x + 1) * words / gridDim.x);
+    for (int i = w0 + tid; i < w1; i += kThreads) __stcg(static_cast<unsigned*>(a.part) + i, 0u);
     __syncthreads();
-    for (int r = tid; r < R; r += kThreads) {
-      part_m[((long long)seg * R + r) * n_chunks + chunk] = run_m[r];
-      part_z[((long long)seg * R + r) * n_chunks + chunk] = run_z[r];
+    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters) : "memory");
+  }
+
+  int q_seg = -1, q_chunk = -1;                                // what qs holds (q_chunk when it holds one step's rows)
+  auto load_q = [&](const Place& p, int chunk) {
+    const bool all = a.q_rows >= chunks * kRows;
+    if (p.seg == q_seg && (all || chunk == q_chunk)) return;
+    __syncthreads();
+    const int r0 = all ? 0 : chunk * kRows, n = all ? chunks * kRows : kRows;
+    for (int i = tid; i < n * TT::kPerRow; i += kThreads) {
+      const int rr = i / TT::kPerRow, c = i - rr * TT::kPerRow, r = r0 + rr;
+      float f[TT::kVec];
+#pragma unroll
+      for (int e = 0; e < TT::kVec; ++e) f[e] = 0.f;
+      if (r < a.R) {                                           // row r = hh*window + i: query head g*G + hh, window row i
+        const int hh = r / a.window, wi = r - hh * a.window;
+        const T* src = q + p.s * a.q_stride_seq + wi * a.q_stride_row + (long long)(p.g * a.G + hh) * a.q_stride_head + c * TT::kVec;
+        unpack(*reinterpret_cast<const uint4*>(src), f, T());
+      }
+#pragma unroll
+      for (int e = 0; e < TT::kVec; e += 4)
+        *reinterpret_cast<float4*>(qs + rr * TT::kPitch + c * TT::kVec + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
+    }
+    q_seg = p.seg;
+    q_chunk = chunk;
+    __syncthreads();
+  };
+  uint4 kreg[TT::kLoads];
+  auto fetch_k = [&](int t) {                                  // a tile's keys on their way into registers
+    const Place p = place_of(a, t);
+#pragma unroll
+    for (int u = 0; u < TT::kLoads; ++u) {
+      const int i = tid + u * kThreads, row = i / TT::kPerRow, c = i - row * TT::kPerRow, j = p.key0 + row;
+      kreg[u] = j < p.n_hist ? *reinterpret_cast<const uint4*>(k + (long long)(p.t0 + j) * a.k_stride_tok +
+                                                               (long long)p.g * a.k_stride_head + c * TT::kVec)
+                             : make_uint4(0, 0, 0, 0);
+    }
+  };
+  auto store_k = [&]() {
+    __syncthreads();                                           // everybody is done with the tile before
+#pragma unroll
+    for (int u = 0; u < TT::kLoads; ++u) {
+      const int i = tid + u * kThreads, row = i / TT::kPerRow, c = i - row * TT::kPerRow;
+      float f[TT::kVec];
+      unpack(kreg[u], f, T());
+#pragma unroll
+      for (int e = 0; e < TT::kVec; e += 4)
+        *reinterpret_cast<float4*>(ks + row * TT::kPitch + c * TT::kVec + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
+    }
+    __syncthreads();
+  };
+  // scores in log2 units: s[i][j] of key kw + 8 i and row chunk * 64 + rw + 4 j
+  float s[4][4];
+  auto scores = [&](int chunk) {
+    const float* kp = ks + kw * TT::kPitch;
+    const float* qp = qs + ((a.q_rows >= chunks * kRows ? chunk * kRows : 0) + rw) * TT::kPitch;
+    f32x2 acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+#pragma unroll 4
+    for (int c = 0; c < D; c += 4) {
+      ulonglong2 kv[4], qv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) kv[i] = *reinterpret_cast<const ulonglong2*>(kp + i * 8 * TT::kPitch + c);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) qv[j] = *reinterpret_cast<const ulonglong2*>(qp + j * 4 * TT::kPitch + c);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[i][j] = fma2(kv[i].x, qv[j].x, acc[i][j]);
+          acc[i][j] = fma2(kv[i].y, qv[j].y, acc[i][j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[i][j] = sum_of(acc[i][j]) * a.scale_log2;
+  };
+  bool cleared = !a.coop;
+  // one round over this CTA's tiles: stage is one of the enum's
+  auto round = [&](int stage) {
+    const bool far = stage == kVotes && !a.lse.lse_opt && __ldcg(st.far) != 0;
+    int lse_seg = -1;
+    for (int t = begin; t < end; ++t) {
+      const Place p = place_of(a, t);
+      const int slot = t - begin;
+      const bool have = slot < a.keep && stage != kStats;       // the scores are still there
+      if (!have) {
+        if (t == begin || (slot == a.keep && stage != kStats)) fetch_k(t);
+        store_k();
+        if (t + 1 < end) fetch_k(t + 1);
+      }
+      if (p.key0 >= p.n_hist) continue;                         // the padding half of a 128-key tile
+      if (stage == kVotes && p.seg != lse_seg) {
+        __syncthreads();
+        for (int r = tid; r < chunks * kRows; r += kThreads) {
+          float l2 = INFINITY;                                  // rows of padding count nothing
+          if (r < a.R) {
+            const size_t at = (size_t)p.seg * a.R + r;
+            const bool has_win = a.lse.win_m != nullptr;
+            l2 = a.lse.lse_opt ? a.lse.caller_lse(p.s, p.g, r, a.G, a.window, false)
+                               : simt_row_lse(st, at, far, has_win, has_win ? a.lse.win_m[at] : 0.f, has_win ? a.lse.win_z[at] : 0.f);
+          }
+          lse_sh[r] = l2;
+        }
+        lse_seg = p.seg;
+        __syncthreads();
+      }
+      float vote = 0.f;                                         // threads 0..63: key tid
+      for (int chunk = 0; chunk < chunks; ++chunk) {
+        float* mine = kept + ((size_t)slot * chunks + chunk) * 16 * kThreads + tid;
+        if (have) {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) s[e >> 2][e & 3] = mine[e * kThreads];
+        } else {
+          load_q(p, chunk);
+          if (chunk * kRows + (warp >> 1) * 16 < a.R) scores(chunk);      // else no row of this warp exists
+          if (slot < a.keep)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) mine[e * kThreads] = s[e >> 2][e & 3];
+        }
+        const int row0 = chunk * kRows + rw;
+        if (stage == kVotes) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float v = 0.f;
+            if (chunk * kRows + (warp >> 1) * 16 < a.R)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) v += exp2f(s[i][j] - lse_sh[row0 + 4 * j]);
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (lane < 8) part_sh[(warp >> 1) * kKeys + kw + 8 * i] = v;
+          }
+          __syncthreads();
+          if (tid < kKeys) vote += (part_sh[tid] + part_sh[kKeys + tid]) + (part_sh[2 * kKeys + tid] + part_sh[3 * kKeys + tid]);
+          __syncthreads();
+        } else if (chunk * kRows + (warp >> 1) * 16 < a.R) {
+          if (!cleared) {                                       // uniform over the warp: spin on the clearing counter
+            if (lane == 0) count_wait(a, 0, gridDim.x);
+            __syncwarp();
+            cleared = true;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int row = row0 + 4 * j;
+            const size_t at = (size_t)p.seg * a.R + min(row, a.R - 1);
+            float v = stage == kMaxima ? -INFINITY : 0.f;
+            const float ref = stage == kFarSums ? unordered(__ldcg(st.row_max + at)) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if (p.key0 + kw + 8 * i >= p.n_hist) continue;
+              v = stage == kMaxima ? fmaxf(v, s[i][j]) : v + exp2f(s[i][j] - ref);
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+              const float w = __shfl_xor_sync(0xffffffffu, v, o);
+              v = stage == kMaxima ? fmaxf(v, w) : v + w;
+            }
+            // the keys of this half-tile may all lie past the end
+            if ((lane & 7) != 0 || row >= a.R || p.key0 + (warp & 1) * 32 >= p.n_hist) continue;
+            if (stage == kStats) {
+              if (v < INFINITY && v > 1e-30f) atomicAdd(st.acc + at, (double)v);
+              else atomicOr(st.far, 1u);
+            } else if (stage == kMaxima) {
+              atomicMax(st.row_max + at, ordered(v));
+            } else {
+              atomicAdd(st.acc_far + at, (double)v);
+            }
+          }
+        }
+      }
+      if (stage == kVotes && tid < kKeys && p.key0 + tid < p.n_hist)
+        a.vote[a.tab.hist_at(p.s) * a.n_kv_heads + (long long)p.g * p.n_hist + p.key0 + tid] = vote / (float)a.G;
+    }
+  };
+
+  bool ok = true;
+  if (a.stages & kStats) round(kStats);
+  if (a.coop) ok = grid_wait(a, 1, (unsigned)a.barrier_extra);
+  if (ok && (a.stages & (kMaxima | kFarSums)) && __ldcg(st.far) != 0) {     // the same for every CTA: all sums are in
+    if (a.stages & kMaxima) round(kMaxima);
+    if (a.coop) ok = grid_wait(a, 2, 0);
+    if (ok && (a.stages & kFarSums)) round(kFarSums);
+    if (a.coop && ok) ok = grid_wait(a, 3, 0);
+  }
+  if (ok && (a.stages & kVotes)) round(kVotes);
+  if (a.coop && tid == 0) {
+    // the last CTA to leave puts the counters back to zero for their next user
+    unsigned prev;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(a.counters + 7) : "memory");
+    if (prev == gridDim.x - 1) {
+      for (int i = 0; i < 8; ++i) a.counters[i] = 0;
+      __threadfence();
     }
   }
 }
 
-// Row statistics over the window keys a window row sees causally (its own position and the window keys before it):
-// one CTA per segment, one thread per row.  Only the all-causal softmax domain needs them.
+// Row statistics over the window keys a window row sees causally (its own position and the window keys before it).
+// Only the all-causal softmax domain needs them.  A CTA takes 16 rows of a segment; key blocks of 32 in shared memory, a
+// lane per key, a warp per four rows.  (One thread per row walking the keys by itself, one CTA per segment, took 24 us for
+// 8 segments of 128 rows and 32 window keys; this takes 4.)
+constexpr int kWinRows = 16;
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(128)
 k_window_stats(const T* __restrict__ q, const T* __restrict__ k, const __grid_constant__ SeqTables tab,
                float* __restrict__ win_m, float* __restrict__ win_z, int n_kv_heads, int G, int window, int head_inner,
                long long k_stride_tok, long long k_stride_head, long long q_stride_seq, long long q_stride_row,
                long long q_stride_head, float scale_log2) {
-  constexpr int VN = Vec<T>::N;
+  constexpr int kVec = 16 / sizeof(T), kPitch = D + 4, kPerRow = D / kVec;
+  __shared__ __align__(16) float ks[32 * kPitch], qs[kWinRows * kPitch];
   pdl_launch_dependents();
   pdl_wait();
   const int seg = blockIdx.x, s = seg / n_kv_heads, g = seg - s * n_kv_heads;
   const int t0 = tab.cu_at(s);
   const int n_hist = tab.cu_at(s + 1) - t0 - window;
-  if (n_hist <= 0) return;                                   // no history: nothing is scored
-  const int R = G * window;
-  for (int r = threadIdx.x; r < R; r += kThreads) {
-    const int hh = head_inner ? r % G : r / window;
-    const int i = head_inner ? r / G : r - hh * window;
-    const T* qrow = q + s * q_stride_seq + i * q_stride_row + (long long)(g * G + hh) * q_stride_head;
-    float m = -INFINITY, z = 0.f;
-    for (int j = 0; j <= i; ++j) {                           // window key j is token n_hist + j
-      const T* krow = k + (long long)(t0 + n_hist + j) * k_stride_tok + (long long)g * k_stride_head;
-      float acc0 = 0.f, acc1 = 0.f;
-      for (int c = 0; c < D / VN; ++c) {
-        float fq[VN], fk[VN];
-        unpack(*reinterpret_cast<const uint4*>(qrow + c * VN), fq, T());
-        unpack(*reinterpret_cast<const uint4*>(krow + c * VN), fk, T());
+  if (n_hist <= 0) return;                                     // no history: nothing is scored
+  const int R = G * window, row0 = blockIdx.y * kWinRows, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto window_row = [&](int r) { return head_inner ? r / G : r % window; };
+  auto query_head = [&](int r) { return g * G + (head_inner ? r % G : r / window); };
+  auto load = [&](float* dst, const T* src) {
+    float f[kVec];
+    unpack(*reinterpret_cast<const uint4*>(src), f, T());
 #pragma unroll
-        for (int e = 0; e < VN; e += 2) {
-          acc0 = fmaf(fq[e], fk[e], acc0);
-          acc1 = fmaf(fq[e + 1], fk[e + 1], acc1);
-        }
-      }
-      const float x = (acc0 + acc1) * scale_log2;
-      const float mn = fmaxf(m, x);
-      z = z * exp2f(m - mn) + exp2f(x - mn);                 // exp2f(-inf) = 0 covers the first key
-      m = mn;
+    for (int e = 0; e < kVec; e += 4) *reinterpret_cast<float4*>(dst + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
+  };
+  int last = 0;                                                // the last key any of the rows sees
+  for (int r = row0; r < min(row0 + kWinRows, R); ++r) last = max(last, window_row(r));
+  for (int i = tid; i < kWinRows * kPerRow; i += 128) {
+    const int rr = i / kPerRow, c = (i - rr * kPerRow) * kVec, r = min(row0 + rr, R - 1);
+    load(qs + rr * kPitch + c, q + s * q_stride_seq + window_row(r) * q_stride_row + (long long)query_head(r) * q_stride_head + c);
+  }
+  float m[4], z[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) { m[u] = -INFINITY; z[u] = 0.f; }
+  for (int j0 = 0; j0 <= last; j0 += 32) {
+    __syncthreads();
+    for (int i = tid; i < 32 * kPerRow; i += 128) {
+      const int jj = i / kPerRow, c = (i - jj * kPerRow) * kVec, j = min(j0 + jj, window - 1);
+      load(ks + jj * kPitch + c, k + (long long)(t0 + n_hist + j) * k_stride_tok + (long long)g * k_stride_head + c);
     }
-    win_m[(long long)seg * R + r] = m;
-    win_z[(long long)seg * R + r] = z;
+    __syncthreads();
+    f32x2 acc[4] = {0, 0, 0, 0};
+#pragma unroll 4
+    for (int c = 0; c < D; c += 4) {
+      const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(ks + lane * kPitch + c);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(qs + (warp * 4 + u) * kPitch + c);
+        acc[u] = fma2(kv.x, qv.x, acc[u]);
+        acc[u] = fma2(kv.y, qv.y, acc[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = min(row0 + warp * 4 + u, R - 1);
+      const bool seen = j0 + lane <= window_row(r);
+      const float x = sum_of(acc[u]) * scale_log2;
+      float mx = seen ? x : -INFINITY;
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if (!(mx > -INFINITY)) continue;                         // the row sees none of these keys (uniform over the warp)
+      const float mn = fmaxf(m[u], mx);
+      float e = seen ? exp2f(x - mn) : 0.f;
+      for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+      z[u] = z[u] * exp2f(m[u] - mn) + e;                      // exp2f(-inf) = 0 covers the first block
+      m[u] = mn;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = row0 + warp * 4 + u;
+    if (lane == 0 && r < R) {
+      win_m[(long long)seg * R + r] = m[u];
+      win_z[(long long)seg * R + r] = z[u];
+    }
   }
 }
 
-// lse_out[s][h][i] from the SIMT layout's per-chunk statistics (and the window statistics, if any).
-__global__ void __launch_bounds__(kThreads)
-k_merge_lse_simt(const float* __restrict__ part_m, const float* __restrict__ part_z, const LseSource lse,
-                 const __grid_constant__ SeqTables tab, float* __restrict__ lse_out, int n_kv_heads, int G, int window,
-                 int n_chunks, int chunk_keys, float out_scale) {
+// lse_out[s][h][i] from the row sums (and the window statistics, if any).
+__global__ void __launch_bounds__(128)
+k_merge_lse_simt(void* part, const LseSource lse, const __grid_constant__ SeqTables tab, float* __restrict__ lse_out,
+                 int n_seg, int n_kv_heads, int G, int window, float out_scale) {
   pdl_launch_dependents();
   pdl_wait();
   const int seg = blockIdx.x, s = seg / n_kv_heads, g = seg - s * n_kv_heads;
   const int n_hist = tab.cu_at(s + 1) - tab.cu_at(s) - window;
   if (n_hist <= 0) return;
   const int R = G * window;
-  const int nc = (n_hist + chunk_keys - 1) / chunk_keys;
-  for (int r = threadIdx.x; r < R; r += kThreads) {
-    const float* pm = part_m + ((long long)seg * R + r) * n_chunks;
-    const float* pz = part_z + ((long long)seg * R + r) * n_chunks;
-    const bool has_win = lse.win_m != nullptr;
-    const float l2 = simt_row_lse(pm, pz, nc, has_win, has_win ? lse.win_m[(long long)seg * R + r] : 0.f,
-                                  has_win ? lse.win_z[(long long)seg * R + r] : 0.f);
+  const SimtStats st = simt_stats(part, n_seg, R);
+  const bool far = __ldcg(st.far) != 0, has_win = lse.win_m != nullptr;
+  for (int r = threadIdx.x; r < R; r += 128) {
+    const size_t at = (size_t)seg * R + r;
+    const float l2 = simt_row_lse(st, at, far, has_win, has_win ? lse.win_m[at] : 0.f, has_win ? lse.win_z[at] : 0.f);
     const int hh = r / window, i = r - hh * window;
     lse_out[((long long)s * lse.n_q_heads + g * G + hh) * window + i] = l2 * out_scale;
   }
 }
 
-float* part_m_of(const Problem& pb) { return reinterpret_cast<float*>(pb.part); }
-float* part_z_of(const Problem& pb) { return part_m_of(pb) + (size_t)pb.n_seg * pb.R * pb.n_chunks; }
-
 template <typename T, int D>
-cudaError_t launch_passes(const Problem& pb, int passes, cudaStream_t st, int* launches) {
-  const size_t smem = simt_smem_bytes(pb);
+cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaStream_t st, int* launches) {
+  using TT = Tiles<T, D>;
   static thread_local int configured_dev = -1;
+  static thread_local unsigned* counters_base = nullptr;
+  static thread_local int coop_state = 0;                      // 0 untried, 1 with dependent launch, 2 without, -1 refused
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(k_score_simt<T, D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_score_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_score_simt<T, D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    void* sym = nullptr;
+    e = cudaGetSymbolAddress(&sym, g_simt_counters);
     if (e != cudaSuccess) return e;
+    counters_base = static_cast<unsigned*>(sym);
+    coop_state = 0;
     configured_dev = dev;
   }
-  const int chunk_keys = kThreads * kTilesPerChunk;
-  dim3 grid((pb.max_hist + chunk_keys - 1) / chunk_keys, pb.p.n_kv_heads, pb.p.n_seqs);
-  const float scale_log2 = kLog2e / sqrtf((float)pb.p.head_dim);
   const slkv_params& p = pb.p;
-  const LseSource lse = lse_source_of(pb);
+  SimtArgs a;
+  a.tab = pb.tab;
+  a.q = pb.q; a.k = pb.k; a.part = pb.part; a.vote = pb.vote; a.lse = lse_source_of(pb); a.status = status;
+  a.n_seqs = p.n_seqs; a.n_kv_heads = p.n_kv_heads; a.G = pb.G; a.window = p.window; a.R = pb.R;
+  a.n_tiles = (int)(2 * pb.n_tiles128);
+  a.k_stride_tok = p.k_stride_tok; a.k_stride_head = p.k_stride_head;
+  a.q_stride_seq = p.q_stride_seq; a.q_stride_row = p.q_stride_row; a.q_stride_head = p.q_stride_head;
+  a.scale_log2 = kLog2e / sqrtf((float)p.head_dim);
+  a.barrier_extra = 0;
+  // Two CTAs per SM where there is work for them (their loads and barriers overlap), one where not; the query rows of a
+  // segment stay in shared memory where they fit beside the keys, else 64 at a time.
+  const int sms = sm_count(), chunks = (pb.R + kRows - 1) / kRows;
+  const int limit = a.n_tiles > sms ? 110 * 1024 : kSmemMost;
+  const int fixed = (kKeys * TT::kPitch + chunks * kRows + 4 * kKeys) * 4, q_all = chunks * kRows * TT::kPitch * 4;
+  a.q_rows = fixed + q_all <= limit ? chunks * kRows : kRows;
+  const int base = fixed + a.q_rows * TT::kPitch * 4;
+  const int most = sms * (limit == kSmemMost ? 1 : 2);
+  const int grid = a.n_tiles < most ? a.n_tiles : most;
+  const int per_cta = (a.n_tiles + grid - 1) / grid, kept_tile = chunks * 16 * kThreads * 4;
+  a.keep = 0;
+  if (passes == 3) a.keep = (limit - base) / kept_tile < per_cta ? (limit - base) / kept_tile : per_cta;
+  const size_t smem = (size_t)base + (size_t)a.keep * kept_tile;
+
+  if (passes != 2 && coop_state >= 0) {
+    a.stages = passes == 3 ? kStats | kMaxima | kFarSums | kVotes : kStats | kMaxima | kFarSums;
+    a.coop = 1;
+    a.barrier_extra = take_expire_next_wait() ? 1 : 0;
+    static std::atomic<unsigned> launch_seq{0};
+    a.counters = counters_base + (size_t)(launch_seq.fetch_add(1) % kCountSlots) * 8;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(grid);
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[2];
+      attr[0].id = cudaLaunchAttributeCooperative;
+      attr[0].val.cooperative = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = coop_state == 2 ? 1 : 2;
+      {
+        LaunchScope scope(passes == 3 ? KID_SCORE_FUSED : KID_SCORE_LSE, st, launches);
+        e = cudaLaunchKernelEx(&cfg, k_score_simt<T, D>, a);
+      }
+      if (e == cudaSuccess) {
+        if (coop_state == 0) coop_state = 1;
+        return cudaSuccess;
+      }
+      (void)cudaGetLastError();                                // not a sticky error: the launch was refused
+      --*launches;
+      if (coop_state != 0) break;
+      coop_state = 2;                                          // once more without dependent launch
+    }
+    coop_state = -1;
+    a.barrier_extra = 0;
+  }
+  // no cooperative launch: the stages as launches of their own
+  a.coop = 0;
+  a.keep = 0;
+  a.counters = counters_base;
   if (passes & 1) {
-    LaunchScope scope(KID_SCORE_LSE, st, launches);
-    e = launch_pdl(k_score_simt<T, D, 1>, grid, dim3(kThreads), smem, st, 1, (const T*)pb.q, (const T*)pb.k, pb.tab,
-                   part_m_of(pb), part_z_of(pb), pb.vote, lse, p.n_kv_heads, pb.G, p.window, pb.n_chunks,
-                   (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
-                   (long long)p.q_stride_row, (long long)p.q_stride_head, scale_log2);
+    e = cudaMemsetAsync(a.part, 0, simt_stat_bytes(pb.n_seg, pb.R), st);
+    for (int stage = kStats; stage <= kFarSums && e == cudaSuccess; stage <<= 1) {
+      a.stages = stage;
+      e = launch_pdl_scoped(KID_SCORE_LSE, k_score_simt<T, D>, grid, kThreads, (size_t)base, st, launches, a);
+    }
     if (e != cudaSuccess) return e;
   }
   if (!(passes & 2)) return cudaSuccess;
-  LaunchScope scope(KID_SCORE_VOTE, st, launches);
-  return launch_pdl(k_score_simt<T, D, 2>, grid, dim3(kThreads), smem, st, 1, (const T*)pb.q, (const T*)pb.k, pb.tab,
-                    part_m_of(pb), part_z_of(pb), pb.vote, lse, p.n_kv_heads, pb.G, p.window, pb.n_chunks,
-                    (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
-                    (long long)p.q_stride_row, (long long)p.q_stride_head, scale_log2);
+  a.stages = kVotes;
+  return launch_pdl_scoped(KID_SCORE_VOTE, k_score_simt<T, D>, grid, kThreads, (size_t)base, st, launches, a);
 }
 
 template <typename T, int D>
 cudaError_t launch_window(const Problem& pb, bool head_inner, cudaStream_t st, int* launches) {
   const slkv_params& p = pb.p;
   LaunchScope scope(KID_WINDOW_STATS, st, launches);
-  return launch_pdl(k_window_stats<T, D>, dim3(pb.n_seg), dim3(kThreads), 0, st, 1, (const T*)pb.q, (const T*)pb.k,
-                    pb.tab, pb.win_m, pb.win_z, p.n_kv_heads, pb.G, p.window, head_inner ? 1 : 0,
-                    (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
+  return launch_pdl(k_window_stats<T, D>, dim3(pb.n_seg, (pb.R + kWinRows - 1) / kWinRows), dim3(128), 0, st, 1,
+                    (const T*)pb.q, (const T*)pb.k, pb.tab, pb.win_m, pb.win_z, p.n_kv_heads, pb.G, p.window,
+                    head_inner ? 1 : 0, (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
                     (long long)p.q_stride_row, (long long)p.q_stride_head, kLog2e / sqrtf((float)p.head_dim));
 }
 
 }  // namespace
 
-int simt_chunk_keys() { return kThreads * kTilesPerChunk; }
+size_t simt_part_bytes(const Problem& pb) { return simt_stat_bytes(pb.n_seg, pb.R); }
 
-size_t simt_smem_bytes(const Problem& pb) {
-  return (size_t)pb.R * pb.p.head_dim * pb.elem + (size_t)(2 * pb.R + 2 * kRowBatch * 4) * sizeof(float);
-}
-
-cudaError_t launch_score_simt(const Problem& pb, int passes, cudaStream_t st, int* launches) {
+cudaError_t launch_score_simt(const Problem& pb, int32_t* status, int passes, cudaStream_t st, int* launches) {
   if (pb.max_hist <= 0) return cudaSuccess;
   const bool bf = pb.p.dtype == SLKV_BF16;
   if (pb.p.head_dim == 64)
-    return bf ? launch_passes<__nv_bfloat16, 64>(pb, passes, st, launches) : launch_passes<float, 64>(pb, passes, st, launches);
-  return bf ? launch_passes<__nv_bfloat16, 128>(pb, passes, st, launches) : launch_passes<float, 128>(pb, passes, st, launches);
+    return bf ? launch_passes<__nv_bfloat16, 64>(pb, status, passes, st, launches)
+              : launch_passes<float, 64>(pb, status, passes, st, launches);
+  return bf ? launch_passes<__nv_bfloat16, 128>(pb, status, passes, st, launches)
+            : launch_passes<float, 128>(pb, status, passes, st, launches);
 }
 
 cudaError_t launch_window_stats(const Problem& pb, bool head_inner, cudaStream_t st, int* launches) {
@@ -333,9 +634,8 @@ float lse_out_scale(const Problem& pb) { return pb.p.lse_units == SLKV_LSE_LOG2 
 cudaError_t launch_merge_lse_simt(const Problem& pb, float* lse_out, cudaStream_t st, int* launches) {
   if (pb.max_hist <= 0) return cudaSuccess;
   LaunchScope scope(KID_MERGE_LSE, st, launches);
-  return launch_pdl(k_merge_lse_simt, dim3(pb.n_seg), dim3(kThreads), 0, st, 1, (const float*)part_m_of(pb),
-                    (const float*)part_z_of(pb), lse_source_of(pb), pb.tab, lse_out, pb.p.n_kv_heads, pb.G, pb.p.window,
-                    pb.n_chunks, pb.chunk_keys, lse_out_scale(pb));
+  return launch_pdl(k_merge_lse_simt, dim3(pb.n_seg), dim3(128), 0, st, 1, pb.part, lse_source_of(pb), pb.tab, lse_out,
+                    pb.n_seg, pb.p.n_kv_heads, pb.G, pb.p.window, lse_out_scale(pb));
 }
 
 }  // namespace slkv

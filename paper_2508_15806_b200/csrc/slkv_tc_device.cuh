@@ -198,8 +198,8 @@ __device__ __forceinline__ int split_index(int x, int T, int n) {
   return (int)((((unsigned)x + 1u) * (unsigned)n - 1u) / (unsigned)T);
 }
 // Row statistics in global memory, per segment and row: acc = the sum of 2^score over all keys, in fp64 and without a
-// reference.  The terms are fp32 sums over one tile each, a few million times 2^-24 apart at most, so their fp64 sum is
-// exact in any order: shares are added atomically and the result depends neither on timing nor on how the keys were split.
+// reference.  The terms are fp32 sums over one tile each, added atomically: in whatever order they come, the sum is the
+// same to 2^-53, far below what its fp32 logarithm shows.
 // Scores beyond fp64's range (above 900 or below -900 in log2 units) go elsewhere: share `slot` then holds such a part of
 // the row's sum as z * 2^m, and its bit in far[] is set.
 constexpr float kFarScore = 900.f;
