@@ -220,8 +220,8 @@ struct ScoreShape {
   int n_q, n_stages, slot_stride;   // Q tiles in shared memory, K tiles in flight; split ranges that may share a segment (stride of the statistics)
   int q_head_inner, k_head_inner;   // tensor-map dimension order: 1 = the head axis comes before the row axis
   int total_tiles, n_cta;       // of one layer; CTAs
-  // The groups the tiles of a list are walked in: group_layers = 1: a layer's n_groups groups, group_tile their first
-  // tiles; else short layers, that many whole ones together.
+  // The groups the tiles of a list are walked in: group_layers = 0: a layer's n_groups groups, group_tile their first
+  // tiles; else that many whole layers together.
   int n_groups, group_layers;
   float scale_log2;
   int group_tile[kListMaxGroups + 1];

@@ -9,7 +9,8 @@
 // The votes of a segment need its rows' statistics over all keys, i.e. from other CTAs.  The layers of a list and the
 // groups of segments inside a layer are independent, so every CTA (one per SM) walks one stream of phases
 //   S(0) .. S(lag-1), S(lag), V(0), S(lag+1), V(1), ..., V(last)
-// over groups of about 2048 tiles: by the time V(g) is due, the others have published S(g), and nobody waits.
+// over groups of about 1024 tiles: by the time V(g) is due, the others have published S(g), nobody waits, and its keys are
+// still in L2.
 //
 // Roles (640 threads, one CTA per SM; a twenty-first warp would cost every thread 16 registers):
 //   warp 0     TMA loads of K tiles (ring of 4-6 x 32 KB) and Q tiles; it never waits for Q while K stages are free
@@ -28,8 +29,8 @@
 //   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
 //     730 measured for loads and MMAs alone;
 //   - two epilogue warpgroups instead of four: 1250; sums over the keys across lanes instead of a lane per row: 1255;
-//   - power: with every tile from HBM the part holds 1.3-1.6 GHz (0.76 us per tile whatever the instruction mix), from
-//     L2 1.75-1.85 GHz.
+//   - power: held for more than some milliseconds the part runs at its 1 kW limit, with every tile from HBM at 1.05 GHz
+//     (0.98 us per tile, MMAs alone 0.78), with tiles from L2 at 1.5 GHz (0.68 us).  Hence the groups.
 // Against the kernel before it (two streams with two accumulators and two warpgroups each on 128 SMs for up to 128 rows,
 // one launch per layer with a grid-wide barrier for more), per layer: 32k tokens, 128 rows: 29.3 -> 24 us; eight ragged
 // sequences of 147k tokens, 256 rows: 299 -> 184 us; 131k tokens, 256 rows: 248 -> 160 us.
@@ -145,7 +146,7 @@ struct GroupShare {
 __device__ __forceinline__ GroupShare group_share(const ListArgs& a, int gg) {
   const ScoreShape& sh = a.sh;
   GroupShare g;
-  if (a.group_layers == 1) {
+  if (a.group_layers == 0) {
     g.layer0 = gg / sh.n_groups;
     const int grp = gg - g.layer0 * sh.n_groups;
     g.base = sh.group_tile[grp];
@@ -195,7 +196,7 @@ struct RunWalk {
         return;
       }
     }
-    const int in_group = a.group_layers == 1 ? 0 : pos / sh.total_tiles;
+    const int in_group = a.group_layers == 0 ? 0 : pos / sh.total_tiles;
     const int layer = s.layer0 + in_group, before = in_group * sh.total_tiles - s.base;  // group tile = layer tile + before
     const ScoreLayer& L = a.lay[layer];
     d.kind = kind;
@@ -244,6 +245,8 @@ __device__ __forceinline__ void producer(const Smem& c) {
   uint32_t st_phase = 0;
   bool ok = true, q_due = false;
   const CUtensorMap* q_map = nullptr;
+  // the statistics pass asks L2 to keep its keys for the vote pass, which lets them go
+  const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
   int q_y = 0, q_z = 0, q_s = 0;
   // Q of run number n - 1
   auto load_q = [&]() {
@@ -268,6 +271,7 @@ __device__ __forceinline__ void producer(const Smem& c) {
     q_map = r.tm_q; q_y = r.q_y; q_z = r.q_z; q_s = r.s;
     q_due = true;
     ++n;
+    const uint64_t policy = r.kind == 0 && c.both ? keep : drop;
     int tok = r.tok;
     for (int i = 0; i < r.count; ++i, ++it, tok += kTileKeys) {
       // a stage of the ring, and Q as soon as the MMAs of the run that had its slot are through with it
@@ -288,7 +292,7 @@ __device__ __forceinline__ void producer(const Smem& c) {
       const uint32_t fb = c.full(st), dst = c.k + (uint32_t)(st * c.stage_bytes);
       mbar_expect_tx(fb, (uint32_t)c.stage_bytes);
       const int ky = c.k_head_inner ? r.g : tok, kz = c.k_head_inner ? tok : r.g;
-      for (int h = 0; h < c.halves; ++h) tma_load_3d(dst + h * kHalfBytes, r.tm_k, 64 * h, ky, kz, fb);
+      for (int h = 0; h < c.halves; ++h) tma_load_3d_hint(dst + h * kHalfBytes, r.tm_k, 64 * h, ky, kz, fb, policy);
       if (++st == c.n_stages) { st = 0; st_phase ^= 1u; }
     }
   }
@@ -895,8 +899,10 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   std::memcpy(a.lay, lay, sizeof(ScoreLayer) * (size_t)n_layers);
   a.n_layers = n_layers;
   a.passes = passes;
-  a.group_layers = n_layers > 1 && sh.group_layers > 1 ? sh.group_layers : 1;
-  a.n_groups = a.group_layers == 1 ? n_layers * sh.n_groups : (n_layers + a.group_layers - 1) / a.group_layers;
+  // A single pass needs no groups: the whole list is one (its tiles are counted in 32 bits times the CTAs).
+  const bool one_group = passes != 3 && (long long)sh.total_tiles * n_layers < (1 << 24);
+  a.group_layers = one_group ? n_layers : (n_layers > 1 ? sh.group_layers : 0);
+  a.n_groups = a.group_layers == 0 ? n_layers * sh.n_groups : (n_layers + a.group_layers - 1) / a.group_layers;
   // units per CTA and phase, about
   const int per_phase = (int)((long long)sh.total_tiles * n_layers * sh.MT / ((long long)a.n_groups * sh.n_cta));
   a.lag = kLagUnits / (per_phase > 0 ? per_phase : 1);
@@ -920,8 +926,6 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   int& cs = coop_state[dev < 64 ? dev : 0];
   if (waits_inside && (env_no_coop || cs == -1 || sh.n_cta > sm_count())) {
     a.passes = 1;
-    a.group_layers = 1;
-    a.n_groups = n_layers * sh.n_groups;
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
     e = launch_pdl_scoped(KID_SCORE_LSE, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);

@@ -10,11 +10,12 @@ namespace slkv {
 namespace {
 
 constexpr int kMergeThreads = 256;
-// Tiles per group.  A phase costs a CTA about 1.2 us beside its tiles (query tile, log-sum-exps of another segment, the
-// hop to the other CTAs where it is not covered), so phases are long: 2048 tiles, 14 per CTA.  At 512 tiles the vote pass
-// finds all of its keys in L2 (67 instead of 134 MB from HBM per layer of 32k tokens) and at 1024 half of them, but a
-// model of 32 such layers takes 1149 and 1008 us instead of 999.
-constexpr int kGroupTiles = 2048;
+// Tiles per group of a two-pass launch.  At 1024 tiles (34 MB of keys) the vote pass finds its keys in L2, given that it
+// lets them go itself: 68 MB from HBM per layer of 32k tokens and 8 heads instead of 134, and HBM reads are what the part's
+// power goes into (a 32 KB tile costs 4.9 uJ from HBM, 1.3 from L2; its MMAs 3.3, its exponentials 1.9).  A phase costs a
+// CTA about 1.2 us beside its tiles, so smaller groups lose more than they save.  32 such layers: 768 tiles 1083 us, 1024
+// 946, 2048 991.
+constexpr int kGroupTiles = 1024;
 
 // The rows' log-sum-exps from the statistics of a launch over one layer: lse_out[s][h][i], in the units out_scale converts
 // to, or (null) the layer's own array, which a vote pass reads.
@@ -184,9 +185,8 @@ cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t
   }
   a.group_tile[++ng] = (int)total;
   a.n_groups = ng;
-  a.group_layers = 1;
-  if (total < kGroupTiles * 3 / 4) {
-    // a short layer: several of a list together (the lists of one layer that n_groups stands for are unaffected)
+  a.group_layers = 0;
+  if (total < kGroupTiles * 3 / 4) {                     // short layers: several of a list together
     a.group_layers = (int)((kGroupTiles + total / 2) / total);
     if (a.group_layers > kListMaxLayers) a.group_layers = kListMaxLayers;
   }
