@@ -130,7 +130,7 @@ int describe(const slkv_params* p, const int32_t* cu_host, Problem* pb) {
 // Overlapped calls are launched as lists where the tensor-core score kernel and a list selection take the shape.
 bool list_supported(const Problem& pb) {
   return tensor_path_supported(pb.p) && pb.p.score_path != SLKV_PATH_SIMT && pb.tab.n_inline > 0 && pb.max_hist > 0 &&
-         (select_cta_supported(pb) || select_cluster_supported(pb));
+         (select_list_supported(pb) || select_cluster_supported(pb));
 }
 
 Layout layout_of(const Problem& pb, bool overlapped = false) {
@@ -262,8 +262,8 @@ cudaError_t flush_list(ListState* s, cudaStream_t owner, int* launches) {
   s->in_flight = true;
   cudaError_t e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, owner, launches);
   if (e == cudaSuccess)
-    e = select_cta_supported(s->pb) ? launch_select_cta(s->pb, s->tail, n, owner, launches)
-                                    : launch_select_cluster(s->pb, s->tail, n, owner, launches);
+    e = select_list_supported(s->pb) ? launch_select_list(s->pb, s->tail, n, owner, launches)
+                                     : launch_select_cluster(s->pb, s->tail, n, owner, launches);
   if (e == cudaSuccess) e = launch_gather(s->pb, s->tail, n, owner, launches);
   return e;
 }
@@ -453,17 +453,18 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   pb.cu = cu_dev; pb.q = q_win; pb.k = k; pb.v = v;
   pb.tab.cu_ptr = cu_dev;
   pb.lse_opt = lse_opt;
-  const bool clustered = select_cluster_supported(pb);
-  if (!clustered || pb.tab.n_inline == 0) {       // tables in global memory and / or the packed offsets
-    e = launch_setup(pb, clustered ? nullptr : budgets, offsets, capacity, status, st, &launches);
+  const bool one_kernel = select_list_supported(pb) || select_cluster_supported(pb);
+  if (!one_kernel || pb.tab.n_inline == 0) {       // tables in global memory and / or the packed offsets
+    e = launch_setup(pb, one_kernel ? nullptr : budgets, offsets, capacity, status, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   rc = enqueue_votes(pb, path, cu_host, status, st, &launches);
   if (rc != SLKV_OK) return rc;
   const TailLayer tail = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
-  if (clustered) {
-    // pooling, offsets and selection in one cluster kernel
-    e = launch_select_cluster(pb, &tail, 1, st, &launches);
+  if (one_kernel) {
+    // pooling, offsets and selection in one kernel
+    e = select_list_supported(pb) ? launch_select_list(pb, &tail, 1, st, &launches)
+                                  : launch_select_cluster(pb, &tail, 1, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
   } else {
     float* pooled = pooled_opt ? pooled_opt : pb.pooled_ws;

@@ -201,8 +201,8 @@ struct TailLayer {
   void* v_out;
   long long capacity;
 };
-bool select_cta_supported(const Problem& pb);
-cudaError_t launch_select_cta(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
+bool select_list_supported(const Problem& pb);
+cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
 bool select_cluster_supported(const Problem& pb);
 cudaError_t launch_select_cluster(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
 cudaError_t launch_gather(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);

@@ -1,29 +1,47 @@
-// Pooling + per-head variable-k selection, one CTA per (sequence, KV head) segment of up to 32768 history
-// positions (Sec. 3.4, Eq. 8; Algorithm 3 lines 1-4, 7-8).
+// Pooling + per-head variable-k selection for a list of layers (Sec. 3.4, Eq. 8; Algorithm 3 lines 1-4, 7-8): one CTA per
+// (sequence, KV head) segment of up to 32768 history positions, a cluster of up to eight for longer ones.
 //
-// A segment this size fits one CTA's registers: thread t owns the 32 consecutive positions [32t, 32t+32).
-// The votes arrive with coalesced loads, pass once through (bank-conflict-free, padded) shared memory to reach
-// their owners together with the pooling halo, and from then on the pooled scores live in registers.  The
-// k-th largest is found by a radix descent over the float bit patterns (11 + 11 + 10 bits; scores are >= 0,
-// so unsigned order = float order) with one shared-memory histogram per level; a thread feeds it one atomic
-// per run of equal digits among its positions (max pooling makes neighbours equal).  No step leaves the CTA,
-// so there is nothing to exchange between CTAs; integer counters only, so the result does not depend on timing.
+// The votes come into shared memory with asynchronous 16-byte copies (from an aligned start, whatever the segment's), a
+// thread pools 8, 16 or 32 consecutive positions of them and works with the scores' bit patterns (scores are >= 0, so
+// unsigned order = float order).  The k-th largest:
+//   1. 128 scores sampled evenly over the segment, ranked by counting: two of them bracket the k-th largest with four
+//      standard deviations to spare on either side;
+//   2. while pooling, every thread notes in bit masks which scores lie above and inside the bracket; their numbers tell
+//      whether the k-th lies inside (else the bracket becomes everything);
+//   3. a radix descent over the scores inside alone -- 2048 bins over the bracket's range -- until a bin's scores fit a list
+//      of 512 (mostly after one level), which is ranked by counting.
+// Then an ordered compaction from the masks.  Integer counters only: the result does not depend on timing, and not on the
+// sample either.
+// What bounds it: instructions.  A CTA's 32 warps on one SM pay eight cycles for each instruction per thread (about 1900 at
+// 32 positions per thread, half of the time), the rest is a dozen CTA-wide steps.  Against a descent from the top over all
+// scores: 16 layers of 8 segments of 131008 positions 290 -> 91 us, one segment per CTA of 1008 positions 13 -> 9 us.
+#include <cooperative_groups.h>
+
 #include "slkv_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace slkv {
 namespace {
 
 constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
-constexpr int kItems = 32;                            // positions per thread
-constexpr int kMaxHist = kThreads * kItems;           // 32768
+constexpr int kMaxItems = 32;                         // consecutive positions per thread: 8, 16 or 32
+constexpr int kMaxSlice = kThreads * kMaxItems;       // 32768 positions per CTA
+constexpr int kMaxCluster = 8;
+constexpr int kMaxRadius = 4;                         // pool_kernel <= 9: four values on either side are enough
 constexpr int kBins = 2048;
-constexpr int kMaxRadius = 4;                         // pool_kernel <= 9
-// position i (shifted by one 32-block so that the left halo exists) -> padded shared-memory index
-__device__ __forceinline__ int padded(int i) { return i + 32 + ((i + 32) >> 5); }
-constexpr int kPaddedFloats = (kMaxHist + 64) + ((kMaxHist + 64) >> 5) + 1;
+constexpr int kSamples = 128;
+constexpr int kList = 512;
+constexpr unsigned kAll = 0xffffffffu;
+// Shared memory of the votes: a thread's positions are `items` floats, then four unused ones -- the pitch makes the 16-byte
+// accesses of neighbouring threads conflict-free -- behind eight floats that hold the four before the first.
+constexpr int kLead = 8;
+__host__ __device__ __forceinline__ int vote_floats(int log_items) {
+  return kLead + (kThreads + 1) * ((1 << log_items) + 4);
+}
 
-struct SelCtaArgs {
+struct SelArgs {
   SeqTables tab;
   int n_seqs, n_kv_heads, window, pool_mode;
   TailLayer lay[kListMaxLayers];
@@ -31,287 +49,390 @@ struct SelCtaArgs {
 
 __device__ __forceinline__ int kept_rows(int len, int budget, int window) { return min(len, max(budget, window)); }
 
-// Inclusive scan of one value per thread over the CTA in thread order; *total = CTA sum.  `wtot` is 32 words.
-__device__ __forceinline__ unsigned block_incl_scan(unsigned v, unsigned* wtot, unsigned* total) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned inc = v;
+// Pooled values at x[4 .. 11] of 16 consecutive votes.
+template <int RAD>
+__device__ __forceinline__ void pool8(const float (&x)[16], bool max_mode, float (&y)[8]) {
+  constexpr int W = 2 * RAD + 1, F = 4 - RAD;          // window of y[e]: x[F + e .. F + e + W - 1]
+  if (max_mode) {
+    float m[16];
+    int have = 1;                                      // m[i] = max of x[i .. i + have - 1]
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  __syncthreads();                       // wtot may still be read from an earlier call
-  if (lane == 31) wtot[wid] = inc;
-  __syncthreads();
-  unsigned w = wtot[lane];               // every warp scans the 32 warp totals itself
+    for (int i = 0; i < 16; ++i) m[i] = x[i];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned n = __shfl_up_sync(0xffffffffu, w, o);
-    if (lane >= o) w += n;
+    for (int step = 1; 2 * step <= W; step *= 2) {
+#pragma unroll
+      for (int i = F; i + step < 16; ++i) m[i] = fmaxf(m[i], m[i + step]);
+      have = 2 * step;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) y[e] = have < W ? fmaxf(m[F + e], m[F + e + W - have]) : m[F + e];
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      float acc = x[F + e];
+#pragma unroll
+      for (int t = 1; t < W; ++t) acc += x[F + e + t];
+      y[e] = acc / (float)W;
+    }
   }
-  *total = __shfl_sync(0xffffffffu, w, 31);
-  const unsigned before = __shfl_sync(0xffffffffu, w, max(wid - 1, 0));
-  return inc + (wid > 0 ? before : 0u);
 }
 
 template <int RAD>
 __global__ void __launch_bounds__(kThreads, 1)
-k_select_cta(const __grid_constant__ SelCtaArgs args) {
-  extern __shared__ __align__(16) float sv[];                // padded votes, kPaddedFloats
-  __shared__ __align__(8) int hist[kBins];
-  __shared__ unsigned wtot[kWarps];
-  __shared__ unsigned sh_prefix;
-  __shared__ int sh_need;
+k_select_list(const __grid_constant__ SelArgs args) {
+  extern __shared__ __align__(16) float votes_sh[];
+  __shared__ __align__(16) int hist[kBins];
+  __shared__ __align__(16) unsigned samp[kSamples];
+  __shared__ __align__(16) unsigned list[kList];
+  __shared__ unsigned wsum[3][kWarps];
+  __shared__ int2 cta_tot;                              // read by the cluster's other CTAs
+  __shared__ unsigned sh_lo, sh_hi, sh_tau, sh_bin, sh_n;
+  __shared__ int sh_above, sh_m, sh_need;
 
-  const int tid = threadIdx.x;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  auto sync_all = [&]() { if (CS > 1) cluster.sync(); else __syncthreads(); };
   pdl_launch_dependents();
-  const int seg = blockIdx.x;
   const TailLayer& a = args.lay[blockIdx.y];
-  const int s = seg / args.n_kv_heads, h = seg - s * args.n_kv_heads;
-  const int t0 = args.tab.cu_at(s);
-  const int len = args.tab.cu_at(s + 1) - t0;
-  const int n_hist = max(len - args.window, 0);
-  const int n_win = min(len, args.window);
+  const int seg = blockIdx.x / CS, s = seg / args.n_kv_heads, h = seg - s * args.n_kv_heads;
+  const int t0 = args.tab.cu_at(s), len = args.tab.cu_at(s + 1) - t0;
+  const int n = max(len - args.window, 0), n_win = min(len, args.window);
   const int n_seg = args.n_seqs * args.n_kv_heads;
-  const long long seg_base = args.tab.hist_at(s) * args.n_kv_heads + (long long)h * n_hist;
+  const long long seg_base = args.tab.hist_at(s) * args.n_kv_heads + (long long)h * n;
   const float* vote = a.vote + seg_base;
-  const float pad = args.pool_mode == SLKV_POOL_MAX ? -INFINITY : 0.f;
-  pdl_wait();                                // budgets and votes may come from the kernels before this one
+  const bool max_mode = args.pool_mode == SLKV_POOL_MAX;
+  const float pad = max_mode ? -INFINITY : 0.f;
+  // this CTA's slice: places 0 .. own - 1, place i is position base + i (the first slice's first places may lie in the
+  // segment before: base <= 0)
+  const int shift = (int)(seg_base & 3);
+  const int slice = ((n + shift + CS - 1) / CS + 3) & ~3;
+  const int own = min(max(n + shift - rank * slice, 0), slice), base = rank * slice - shift;
+  const int my_end = min(base + own, n);
+  const int log_items = own <= 8 * kThreads ? 3 : (own <= 16 * kThreads ? 4 : 5);
+  const int items = 1 << log_items, pitch = items + 4;
+  float* votes = votes_sh + kLead;
+  auto at = [&](int i) { return (i >> log_items) * pitch + (i & (items - 1)); };      // a place's index (i >= -4)
+  const long long capacity = a.capacity;
+  if (tid == 0) { sh_lo = 0; sh_hi = 0x7f800000u; sh_n = 0; }
+  reinterpret_cast<int2*>(hist)[tid] = make_int2(0, 0);
+  pdl_wait();                                           // budgets and votes may come from the kernels before this one
 
-  // all of the segment's votes, coalesced, in flight together
-  float x[kItems];
+  // ---- the votes on their way, four places at a time, with one group on either side
+  for (int q = tid - 1; 4 * q <= own + 3; q += kThreads) {
+    const int p = base + 4 * q;
+    float* dst = votes + at(4 * q);
+    if (p >= 0 && p + 3 < n) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(vote + p) : "memory");
+    } else {
 #pragma unroll
-  for (int k = 0; k < kItems; ++k) {
-    const int i = k * kThreads + tid;
-    x[k] = i < n_hist ? __ldg(vote + i) : pad;
+      for (int e = 0; e < 4; ++e) dst[e] = p + e >= 0 && p + e < n ? __ldg(vote + p + e) : pad;
+    }
   }
-  const int k_keep = kept_rows(len, a.budgets[h], args.window) - n_win;    // C_H = C - window, clamped
-
-  // packed row where this segment starts = kept rows of all earlier segments (Algorithm 3 l.1-4 per head)
-  long long out0;
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  const int k_keep = kept_rows(len, a.budgets[h], args.window) - n_win;       // C_H = C - window, clamped
+  const bool choose = k_keep > 0 && k_keep < n;
+  if (choose && tid < kSamples) {
+    const int p = (int)(((long long)(2 * tid + 1) * n) / (2 * kSamples));
+    float w[2 * RAD + 1];
+#pragma unroll
+    for (int t = 0; t <= 2 * RAD; ++t) {
+      const int q = p - RAD + t;
+      w[t] = q >= 0 && q < n ? __ldg(vote + q) : pad;
+    }
+    float v = w[0];
+#pragma unroll
+    for (int t = 1; t <= 2 * RAD; ++t) v = max_mode ? fmaxf(v, w[t]) : v + w[t];
+    if (!max_mode) v /= (float)(2 * RAD + 1);
+    samp[tid] = (__float_as_uint(v) & ~(kSamples - 1u)) | (unsigned)tid;       // all different; the bracket is widened by it
+  }
   {
-    unsigned part = 0;                       // < 2^31: the host checks n_kv_heads * total_tokens
+    unsigned part = 0;                                  // < 2^31: the host checks n_kv_heads * total_tokens
     for (int g = tid; g < seg; g += kThreads) {
       const int s2 = g / args.n_kv_heads, h2 = g - s2 * args.n_kv_heads;
       part += (unsigned)kept_rows(args.tab.cu_at(s2 + 1) - args.tab.cu_at(s2), a.budgets[h2], args.window);
     }
-    unsigned tot;
-    block_incl_scan(part, wtot, &tot);
-    out0 = tot;
+    part = __reduce_add_sync(kAll, part);
+    if (lane == 0) wsum[0][wid] = part;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // packed row where this segment starts = kept rows of all earlier segments (Algorithm 3 l.1-4 per head)
+  const long long out0 = __reduce_add_sync(kAll, wsum[0][lane]);
+  const int src_base = t0 * args.n_kv_heads + h;         // source row of position j: src_base + j * n_kv_heads
+  auto put = [&](long long o, int position) {
+    if (o < capacity) {
+      a.kept_idx[o] = position;
+      a.gather_src[o] = src_base + position * args.n_kv_heads;
+    }
+  };
+  if (rank == 0) {
     if (tid == 0) {
-      a.offsets[seg] = (int32_t)tot;
+      a.offsets[seg] = (int32_t)out0;
       if (seg == n_seg - 1) {
         const long long all = out0 + k_keep + n_win;
         a.offsets[n_seg] = (int32_t)all;
-        if (all > a.capacity && a.status) *a.status = SLKV_ERR_CAPACITY;
+        if (all > capacity && a.status) *a.status = SLKV_ERR_CAPACITY;
       }
     }
+    for (int t = tid; t < n_win; t += kThreads) put(out0 + k_keep + t, len - n_win + t);    // window rows: always kept
   }
-  const int src_base = t0 * args.n_kv_heads + h;            // source row of position j: src_base + j * n_kv_heads
+  if (!choose) {                                         // uniform over the cluster: keep all of the history, or none
+    if (k_keep > 0)
+      for (int j = base + tid; j < my_end; j += kThreads)
+        if (j >= 0) put(out0 + j, j);
+    if (a.pooled_out == nullptr) return;
+  }
 
-  // window rows: always kept, after the history rows
-  for (int t = tid; t < n_win; t += kThreads) {
-    const long long o = out0 + k_keep + t;
-    if (o < a.capacity) {
-      a.kept_idx[o] = len - n_win + t;
-      a.gather_src[o] = src_base + (len - n_win + t) * args.n_kv_heads;
+  // ---- the bracket: ranks of the samples by counting, eight lanes per sample
+  if (choose) {
+    const float q = (float)kSamples * (float)k_keep / (float)n;
+    const float dev = 4.f * sqrtf(q * (1.f - (float)k_keep / (float)n)) + 1.f;
+    const int r_hi = (int)floorf(q - dev) - 1, r_lo = (int)ceilf(q + dev);     // outside 0 .. kSamples - 1: no bound there
+    const int i = tid >> 3, part = tid & 7;
+    const unsigned x = samp[i];
+    int above = 0;
+#pragma unroll
+    for (int j = 0; j < kSamples / 8; j += 4) {
+      const uint4 y = *reinterpret_cast<const uint4*>(samp + part * (kSamples / 8) + j);
+      above += (y.x > x) + (y.y > x) + (y.z > x) + (y.w > x);
     }
+    above += __shfl_xor_sync(kAll, above, 1);
+    above += __shfl_xor_sync(kAll, above, 2);
+    above += __shfl_xor_sync(kAll, above, 4);
+    if (part == 0 && above == r_hi) sh_hi = x | (kSamples - 1u);
+    if (part == 0 && above == r_lo) sh_lo = x & ~(kSamples - 1u);
   }
+  __syncthreads();
+  unsigned lo = sh_lo, hi = sh_hi;                       // every CTA of the cluster finds the same
 
-  const bool need_scores = (k_keep > 0 && k_keep < n_hist) || a.pooled_out != nullptr;
-  if (!need_scores) {
-    if (k_keep >= n_hist && k_keep > 0) {                              // nothing to drop (Alg. 3 l.1-3)
-      for (int i = tid; i < n_hist; i += kThreads)
-        if (out0 + i < a.capacity) {
-          a.kept_idx[out0 + i] = i;
-          a.gather_src[out0 + i] = src_base + i * args.n_kv_heads;
+  // ---- pooling; bit j of the masks is the thread's place j
+  const int i0 = tid << log_items;
+  const bool mine = i0 < own;
+  unsigned gt = 0, cand = 0, valid = 0;
+  float4 keep[kMaxItems / 4];
+  if (mine) {
+    const int p0 = base + i0, v_lo = max(-p0, 0), v_hi = min(my_end - p0, items);         // valid places of the thread
+    valid = (v_hi >= 32 ? kAll : (1u << max(v_hi, 0)) - 1u) & (v_lo >= 32 ? 0u : kAll << v_lo);
+    const float* src = votes + tid * pitch;
+    float x[16];
+    auto load4 = [&](const float* f, int k) {
+      const float4 v = *reinterpret_cast<const float4*>(f);
+      x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
+    };
+    load4(votes + at(i0 - 4), 8);
+    load4(src, 12);
+#pragma unroll
+    for (int g = 0; g < kMaxItems / 8; ++g) {
+      if (8 * g < items) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = x[k + 8];
+        load4(src + 8 * g + 4, 8);
+        load4(8 * g + 8 < items ? src + 8 * g + 8 : src + pitch, 12);      // the next thread's first four
+        float y[8];
+        pool8<RAD>(x, max_mode, y);
+        unsigned b_gt = 0, b_ge = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const unsigned v = __float_as_uint(y[e]);
+          b_gt |= v > hi ? 1u << e : 0u;
+          b_ge |= v >= lo ? 1u << e : 0u;
         }
+        gt |= b_gt << (8 * g);
+        cand |= b_ge << (8 * g);
+        keep[2 * g] = make_float4(y[0], y[1], y[2], y[3]);
+        keep[2 * g + 1] = make_float4(y[4], y[5], y[6], y[7]);
+      }
     }
-    return;
+    gt &= valid;
+    cand &= valid & ~gt;
   }
-
-  // ---- votes to their owners: thread t gets positions [32t - RAD, 32t + 32 + RAD)
-#pragma unroll
-  for (int k = 0; k < kItems; ++k) sv[padded(k * kThreads + tid)] = x[k];
-  if (tid < 32) sv[padded(tid - 32)] = pad;                            // left halo block
-  if (tid < 32) sv[padded(kMaxHist + tid)] = pad;                      // right halo block
-  __syncthreads();
-  const int first = kItems * tid;                                      // first position this thread owns
-  const int nv = min(max(n_hist - first, 0), kItems);                  // valid positions among its 32
-  unsigned key[kItems];                                                // pooled scores as bit patterns
   {
-    float v[kItems + 2 * RAD];
-#pragma unroll
-    for (int j = 0; j < kItems + 2 * RAD; ++j) v[j] = sv[padded(first - RAD + j)];
-    if (args.pool_mode == SLKV_POOL_MAX) {
-      // max over [j, j + 2 RAD] by doubling: windows of 2, 4, ... then two overlapping ones
-      constexpr int W = 2 * RAD + 1;
-      int have = 1;                                                    // v[j] = max of v[j .. j + have - 1]
-#pragma unroll
-      for (int step = 1; 2 * step <= W; step *= 2) {
-#pragma unroll
-        for (int j = 0; j + step < kItems + 2 * RAD; ++j) v[j] = fmaxf(v[j], v[j + step]);
-        have = 2 * step;
-      }
-      if (have < W) {
-#pragma unroll
-        for (int j = 0; j < kItems; ++j) v[j] = fmaxf(v[j], v[j + W - have]);
-      }
-#pragma unroll
-      for (int j = 0; j < kItems; ++j) key[j] = __float_as_uint(v[j]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < kItems; ++j) {
-        float acc = v[j];
-#pragma unroll
-        for (int t = 1; t <= 2 * RAD; ++t) acc += v[j + t];
-        key[j] = __float_as_uint(acc / (float)(2 * RAD + 1));
-      }
-    }
+    const unsigned both = __reduce_add_sync(kAll, (unsigned)__popc(gt) | ((unsigned)__popc(cand) << 16));
+    if (lane == 0) wsum[1][wid] = both;
   }
-  // the pooled keys also go back to shared memory: later steps visit single positions by index
-  __syncthreads();
+  __syncthreads();                                       // everybody has read the votes: the scores take their places
+  unsigned* keys = reinterpret_cast<unsigned*>(votes) + tid * pitch;
+  if (mine) {
 #pragma unroll
-  for (int j = 0; j < kItems; ++j) sv[padded(first + j)] = __uint_as_float(key[j]);
-  if (a.pooled_out) {                                                  // coalesced stores from shared memory
+    for (int g = 0; g < kMaxItems / 4; ++g)
+      if (4 * g < items) *reinterpret_cast<float4*>(keys + 4 * g) = keep[g];
+  }
+  if (a.pooled_out) {
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      const int i = k * kThreads + tid;
-      if (i < n_hist) a.pooled_out[seg_base + i] = sv[padded(i)];
-    }
+    for (int i = tid; i < own; i += kThreads)
+      if (base + i >= 0 && base + i < my_end) a.pooled_out[seg_base + base + i] = votes[at(i)];
   }
-  if (k_keep <= 0) return;
-  if (k_keep >= n_hist) {                                              // nothing to drop (Alg. 3 l.1-3)
-    for (int i = tid; i < n_hist; i += kThreads)
-      if (out0 + i < a.capacity) {
-        a.kept_idx[out0 + i] = i;
-        a.gather_src[out0 + i] = src_base + i * args.n_kv_heads;
-      }
-    return;
+  if (!choose) return;
+  int need = k_keep;
+  {
+    const unsigned tot = __reduce_add_sync(kAll, wsum[1][lane]);
+    int n_gt = (int)(tot & 0xffffu), n_cand = (int)(tot >> 16);
+    if (CS > 1) {
+      if (tid == 0) cta_tot = make_int2(n_gt, n_cand);
+      cluster.sync();
+      int2 o = make_int2(0, 0);
+      if (lane < CS) o = *cluster.map_shared_rank(&cta_tot, lane);
+      n_gt = (int)__reduce_add_sync(kAll, (unsigned)o.x);
+      n_cand = (int)__reduce_add_sync(kAll, (unsigned)o.y);
+      // cta_tot is written again only behind the cluster-wide barriers of the descent
+    }
+    if (n_gt < k_keep && k_keep <= n_gt + n_cand) {
+      need = k_keep - n_gt;
+    } else {
+      lo = 0; hi = kAll;
+      gt = 0; cand = valid;
+    }
   }
 
-  // ---- k-th largest pooled score: radix descent, one histogram per level
-  unsigned prefix = 0;
-  int need = k_keep;
-  unsigned live = nv >= kItems ? 0xffffffffu : ((1u << nv) - 1u);      // bit j: position first + j still a candidate
-#pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
-    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    const unsigned dmask = pass == 2 ? 1023u : 2047u;
+  // ---- radix descent inside [lo, hi]: `need` of the scores there, the largest, are kept
+  unsigned tau;
+  while (true) {
+    const unsigned span = hi - lo;
+    const int sh = span < (unsigned)kBins ? 0 : 21 - __clz(span);
+    for (unsigned m = cand; m != 0; m &= m - 1) atomicAdd(&hist[(keys[__ffs(m) - 1] - lo) >> sh], 1);
+    sync_all();
+    int2 c2 = reinterpret_cast<const int2*>(hist)[tid];
+    if (CS > 1)
+      for (int o = 1; o < CS; ++o) {
+        const int2 x = reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, (rank + o) % CS))[tid];
+        c2.x += x.x;
+        c2.y += x.y;
+      }
+    const unsigned sum = __reduce_add_sync(kAll, (unsigned)(c2.x + c2.y));
+    if (lane == 0) wsum[0][wid] = sum;
+    __syncthreads();
+    const int above_w = (int)__reduce_add_sync(kAll, lane > wid ? wsum[0][lane] : 0u);
+    if (above_w < need && need <= above_w + (int)sum) {   // the bin is one of this warp's 64
+      int inc = c2.x + c2.y;                              // suffix sum over the lanes
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_down_sync(kAll, inc, o);
+        if (lane + o < 32) inc += v;
+      }
+      const int above = above_w + inc - (c2.x + c2.y);
+      if (above < need && need <= above + c2.y) { sh_bin = 2 * tid + 1; sh_above = above; sh_m = c2.y; }
+      else if (above + c2.y < need && need <= above + c2.y + c2.x) { sh_bin = 2 * tid; sh_above = above + c2.y; sh_m = c2.x; }
+    }
+    sync_all();                                           // in a cluster also: nobody reads the others' bins any more
+    const int m_bin = sh_m;
+    need -= sh_above;
+    lo += sh_bin << sh;
+    hi = min(hi, lo + ((1u << sh) - 1u));
+    if (sh == 0) { tau = lo; break; }
+    // the bin's scores go on; where they fit, in a list of the cluster's first CTA (their order does not matter)
+    const bool listed = m_bin <= kList;
+    unsigned* list0 = CS > 1 ? cluster.map_shared_rank(list, 0) : list;
+    unsigned* n0 = CS > 1 ? cluster.map_shared_rank(&sh_n, 0) : &sh_n;
+    unsigned in_bin = 0;
+    for (unsigned m = cand; m != 0; m &= m - 1) {
+      const unsigned v = keys[__ffs(m) - 1], bit = m & (0u - m);
+      if (v > hi) gt |= bit;
+      else if (v >= lo) {
+        in_bin |= bit;
+        if (listed) list0[atomicAdd(n0, 1u)] = v;
+      }
+    }
+    cand = in_bin;
+    if (listed) {                                         // ranked by counting
+      sync_all();
+      if (CS > 1 && rank > 0) {
+        for (int i = tid; i < m_bin; i += kThreads) list[i] = list0[i];
+        __syncthreads();
+      }
+      int log_p = 5;                                      // 2^log_p lanes per score
+      while ((m_bin << log_p) > kThreads) --log_p;
+      const int i = tid >> log_p, P = 1 << log_p, part = tid & (P - 1);
+      if (wid << 5 >> log_p < m_bin) {                    // some score for this warp
+        const unsigned x = list[min(i, m_bin - 1)];
+        int above = 0, at_least = 0;
+        for (int j = part; j < m_bin; j += P) { const unsigned y = list[j]; above += y > x; at_least += y >= x; }
+        for (int o = 1; o < P; o <<= 1) {
+          above += __shfl_xor_sync(kAll, above, o);
+          at_least += __shfl_xor_sync(kAll, at_least, o);
+        }
+        if (i < m_bin && part == 0 && above < need && need <= at_least) { sh_tau = x; sh_need = need - above; }
+      }
+      __syncthreads();
+      tau = sh_tau;
+      need = sh_need;
+      break;
+    }
     reinterpret_cast<int2*>(hist)[tid] = make_int2(0, 0);
     __syncthreads();
-    if (pass == 0) {
-      // all positions, from registers: one atomic per run of equal digits (max pooling makes neighbours equal)
-      unsigned run_digit = key[0] >> 21;
-      int run_len = 0;
-#pragma unroll
-      for (int j = 0; j < kItems; ++j) {
-        const unsigned digit = key[j] >> 21;
-        if (j < nv) {
-          if (digit != run_digit) { atomicAdd(&hist[run_digit], run_len); run_len = 0; run_digit = digit; }
-          ++run_len;
-        }
-      }
-      if (run_len > 0) atomicAdd(&hist[run_digit], run_len);
-    } else {
-      for (unsigned m = live; m != 0; m &= m - 1) {
-        const int j = __ffs(m) - 1;
-        atomicAdd(&hist[(__float_as_uint(sv[padded(first + j)]) >> shift) & dmask], 1);
-      }
-    }
-    __syncthreads();
-    const int2 c = reinterpret_cast<const int2*>(hist)[tid];          // bins 2*tid (c.x) and 2*tid+1 (c.y)
-    unsigned tot;
-    const unsigned inc = block_incl_scan((unsigned)(c.x + c.y), wtot, &tot);
-    const int above_hi = (int)(tot - inc);                             // elements in bins above 2*tid+1
-    const int above_lo = above_hi + c.y;                               // above bin 2*tid
-    if (above_hi < need && need <= above_hi + c.y) {                   // exactly one bin satisfies this
-      sh_prefix = prefix | ((unsigned)(2 * tid + 1) << shift);
-      sh_need = need - above_hi;
-    } else if (above_lo < need && need <= above_lo + c.x) {
-      sh_prefix = prefix | ((unsigned)(2 * tid) << shift);
-      sh_need = need - above_lo;
-    }
-    __syncthreads();
-    prefix = sh_prefix;
-    need = sh_need;
-    if (pass == 0) {
-      const unsigned b0 = prefix >> 21;
-      unsigned keep = 0;
-#pragma unroll
-      for (int j = 0; j < kItems; ++j) keep |= ((key[j] >> 21) == b0 ? 1u : 0u) << j;
-      live &= keep;
-    } else if (pass == 1) {
-      const unsigned want = (prefix >> 10) & 2047u;
-      unsigned keep = 0;
-      for (unsigned m = live; m != 0; m &= m - 1) {
-        const int j = __ffs(m) - 1;
-        if (((__float_as_uint(sv[padded(first + j)]) >> 10) & 2047u) == want) keep |= 1u << j;
-      }
-      live = keep;
-    }
   }
-  const unsigned tau = prefix;            // the k-th largest score; `need` of the positions equal to it are kept
 
-  // ---- ordered compaction: threads own consecutive positions, so thread order is position order
-  unsigned gt_mask = 0, eq_mask = 0;
+  // ---- ordered compaction: the scores above tau, and the first `need` equal to it; threads own consecutive positions
+  unsigned eq = 0;
+  for (unsigned m = cand; m != 0; m &= m - 1) {
+    const unsigned v = keys[__ffs(m) - 1], bit = m & (0u - m);
+    if (v > tau) gt |= bit;
+    else if (v == tau) eq |= bit;
+  }
+  const unsigned cnt = (unsigned)__popc(gt) | ((unsigned)__popc(eq) << 16);
+  unsigned inc = cnt;                                     // both totals are <= 32768
 #pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    gt_mask |= (key[j] > tau ? 1u : 0u) << j;
-    eq_mask |= (key[j] == tau ? 1u : 0u) << j;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned x = __shfl_up_sync(kAll, inc, o);
+    if (lane >= o) inc += x;
   }
-  const unsigned valid = nv >= kItems ? 0xffffffffu : ((1u << nv) - 1u);
-  gt_mask &= valid; eq_mask &= valid;
-  const unsigned my_gt = __popc(gt_mask), my_eq = __popc(eq_mask);
-  // both totals are <= 32768: pack them into one scan (equal count in the high half)
-  unsigned tot_pack;
-  const unsigned inc_pack = block_incl_scan((my_eq << 16) | my_gt, wtot, &tot_pack);
-  const int gt_before = (int)((inc_pack & 0xffffu) - my_gt), eq_before = (int)((inc_pack >> 16) - my_eq);
-  // of the positions equal to tau, the first `need` (in position order) are kept
-  const int eq_take = min(max(need - eq_before, 0), (int)my_eq);
-  unsigned eq_kept = 0;
-  { unsigned m = eq_mask; for (int t = 0; t < eq_take; ++t) { eq_kept |= m & (0u - m); m &= m - 1; } }
-  const unsigned kept_mask = gt_mask | eq_kept;
-  // a kept position's output row: kept ones before it = (greater before) + min(equal before, need)
+  if (lane == 31) wsum[2][wid] = inc;
+  __syncthreads();
+  const unsigned before = __reduce_add_sync(kAll, lane < wid ? wsum[2][lane] : 0u) + inc - cnt;
+  int gt_before = (int)(before & 0xffffu), eq_before = (int)(before >> 16);
+  if (CS > 1) {
+    if (tid == kThreads - 1) cta_tot = make_int2(gt_before + __popc(gt), eq_before + __popc(eq));
+    cluster.sync();
+    int2 o = make_int2(0, 0);
+    if (lane < rank) o = *cluster.map_shared_rank(&cta_tot, lane);
+    gt_before += (int)__reduce_add_sync(kAll, (unsigned)o.x);
+    eq_before += (int)__reduce_add_sync(kAll, (unsigned)o.y);
+  }
+  // of the thread's scores equal to tau, the first `take`
+  const int take = min(max(need - eq_before, 0), __popc(eq));
+  unsigned kept = gt;
+  for (int t = 0; t < take; ++t) { kept |= eq & (0u - eq); eq &= eq - 1; }
   long long o = out0 + gt_before + min(eq_before, need);
-  for (unsigned m = kept_mask; m != 0; m &= m - 1, ++o) {
-    const int j = __ffs(m) - 1;
-    if (o < a.capacity) {
-      a.kept_idx[o] = first + j;
-      a.gather_src[o] = src_base + (first + j) * args.n_kv_heads;
-    }
-  }
+  for (unsigned m = kept; m != 0; m &= m - 1, ++o) put(o, base + i0 + __ffs(m) - 1);
+  if (CS > 1) cluster.sync();                             // nobody leaves while its shared memory may still be read
+}
+
+int cluster_size(const Problem& pb) {
+  int cs = 1;
+  while (cs < kMaxCluster && (pb.max_hist + 3 + cs - 1) / cs + 3 > kMaxSlice) cs *= 2;
+  return cs;
 }
 
 }  // namespace
 
-bool select_cta_supported(const Problem& pb) {
-  return pb.max_hist <= kMaxHist && (pb.p.pool_kernel >> 1) <= kMaxRadius;
+bool select_list_supported(const Problem& pb) {
+  return (pb.p.pool_kernel >> 1) <= kMaxRadius && (pb.max_hist + 3) / kMaxCluster + 4 <= kMaxSlice;
 }
 
-cudaError_t launch_select_cta(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
-  typedef void (*Kern)(const SelCtaArgs);
-  static const Kern kerns[kMaxRadius + 1] = {k_select_cta<0>, k_select_cta<1>, k_select_cta<2>, k_select_cta<3>,
-                                             k_select_cta<4>};
-  const size_t smem = (size_t)kPaddedFloats * sizeof(float);
+cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
+  typedef void (*Kern)(const SelArgs);
+  static const Kern kerns[kMaxRadius + 1] = {k_select_list<0>, k_select_list<1>, k_select_list<2>, k_select_list<3>,
+                                             k_select_list<4>};
+  const int cs = cluster_size(pb);
+  const int slice = ((pb.max_hist + 3 + cs - 1) / cs + 3) & ~3;
+  const size_t smem = (size_t)vote_floats(slice <= 8 * kThreads ? 3 : (slice <= 16 * kThreads ? 4 : 5)) * sizeof(float);
   static thread_local int configured_dev = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
     for (int r = 0; r <= kMaxRadius; ++r) {
-      e = cudaFuncSetAttribute(kerns[r], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(kerns[r], cudaFuncAttributeMaxDynamicSharedMemorySize, vote_floats(5) * (int)sizeof(float));
       if (e != cudaSuccess) return e;
     }
     configured_dev = dev;
   }
-  SelCtaArgs a;
+  SelArgs a;
   a.tab = pb.tab;
   a.n_seqs = pb.p.n_seqs; a.n_kv_heads = pb.p.n_kv_heads; a.window = pb.p.window; a.pool_mode = pb.p.pool_mode;
   for (int i = 0; i < n_layers; ++i) a.lay[i] = lay[i];
   LaunchScope scope(KID_SELECT, st, launches);
-  return launch_pdl(kerns[pb.p.pool_kernel >> 1], dim3((unsigned)pb.n_seg, (unsigned)n_layers), dim3(kThreads), smem, st, 1, a);
+  return launch_pdl(kerns[pb.p.pool_kernel >> 1], dim3((unsigned)(pb.n_seg * cs), (unsigned)n_layers), dim3(kThreads), smem, st, cs, a);
 }
 
 }  // namespace slkv

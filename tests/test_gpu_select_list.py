@@ -1,0 +1,66 @@
+"""GPU: the list selection at the edges of its rounds, slices and clusters, on scores with ties, plateaus, zeros and hostile
+orderings, against an exact sort of the scores it reports."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import slkv_oracle as O
+from paper_2508_15806_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+def run(lens, hkv, w, budgets, pool, mode, k_scale=1.0, k_fn=None):
+    d, T = 64, sum(lens)
+    g = torch.Generator(device=DEV).manual_seed(sum(lens) + pool)
+    q = torch.randn(len(lens), w, hkv, d, generator=g, device=DEV).bfloat16()
+    k = (torch.randn(T, hkv, d, generator=g, device=DEV) * k_scale)
+    k = (k if k_fn is None else k_fn(k)).bfloat16()
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    p = B.make_params(q, k, k, w, pool, mode)
+    bud = torch.tensor(budgets, dtype=torch.int32, device=DEV)
+    cap = sum(min(n, max(b, w)) for n in lens for b in budgets)
+    out = torch.zeros(cap, d, dtype=torch.bfloat16, device=DEV)
+    off = torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV)
+    kept = torch.full((cap,), -1, dtype=torch.int32, device=DEV)
+    pooled = torch.zeros(max(B.slkv_pooled_elems(p, cu), 1), device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    for want in (pooled, None):                         # the same with and without the scores written out
+        kept.fill_(-1)
+        B.slkv_compress(p, q, k, k, torch.tensor(cu, dtype=torch.int32, device=DEV), cu, bud, out, torch.zeros_like(out), off,
+                        kept, ws, want, status)
+        torch.cuda.synchronize()
+        assert int(status) == 0
+        sc, idx, o, at = pooled.cpu().numpy(), kept.cpu().numpy(), off.cpu().tolist(), 0
+        for s, n in enumerate(lens):
+            nh = max(n - w, 0)
+            for h in range(hkv):
+                seg = s * hkv + h
+                kh, nw = O.kept_counts(n, budgets[h], w)
+                ref = O.select_topk(sc[at:at + nh].astype(np.float64), kh) if kh else np.zeros(0, np.int64)
+                got = idx[o[seg]:o[seg + 1]]
+                assert got[:kh].tolist() == ref.tolist(), (s, h)
+                assert got[kh:].tolist() == list(range(n - nw, n))
+                at += nh
+
+
+@pytest.mark.parametrize("n", [1, 3, 5, 127, 128, 4095, 4096, 4097, 8190, 32764, 32765, 32768, 40001, 131071])
+@pytest.mark.parametrize("pool,mode", [(1, B.SLKV_POOL_MAX), (7, B.SLKV_POOL_MAX), (9, B.SLKV_POOL_AVG)])
+def test_lengths(n, pool, mode):
+    run([n + 8], 3, 8, [8 + max(1, n // 50), 8 + n // 2, 8 + n - 1], pool, mode)
+
+
+def test_ragged_segments_start_anywhere():
+    run([4100, 9, 8, 0, 700, 33001, 2], 3, 8, [40, 500, 9], 5, B.SLKV_POOL_MAX)
+
+
+@pytest.mark.parametrize("n", [6000, 70000])
+def test_ties_zeros_and_orderings(n):
+    same = lambda k: k[:1].expand_as(k).contiguous()                                             # noqa: E731
+    far = lambda k: torch.where(torch.arange(len(k), device=DEV).view(-1, 1, 1) % 97 == 0, k * 0.0 + 30.0, k * 0.0 - 30.0)   # noqa: E731
+    sort = lambda k: torch.sort(k, dim=0).values                                                 # noqa: E731
+    period = lambda k: k[torch.arange(len(k), device=DEV) % 128]                                 # noqa: E731
+    for fn in (same, far, sort, period):
+        run([n], 3, 4, [300, n // 3, n - 7], 3, B.SLKV_POOL_MAX, k_fn=fn)
