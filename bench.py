@@ -406,7 +406,8 @@ def run_cuda(args):
         ev_ms = timed(e2e_steps, e2e_step)
         wall_ms = (time.perf_counter() - t0) * 1e3
         e2e_ms = max(ev_ms, 0.0)
-        h2d = sum((Hh["q"].numel() + Hh["k"].numel() + Hh["v"].numel()) * e + (len(cu) + hkv) * 4
+        # of V only the kept rows cross the link (the buffers are page-locked)
+        h2d = sum((Hh["q"].numel() + Hh["k"].numel() + Hh["rows"] * d) * e + hkv * 4
                   for Hh in (host[l % n_host] for l in range(nl)))
         d2h = sum(host[l % n_host]["rows"] * (2 * d * e + 4) + (len(wl.seq_lens) * hkv + 1) * 4 for l in range(nl))
         e2e = {"value": whole_job_value(world, T, nl, e2e_ms / e2e_steps), "unit": UNIT, "h2d_bytes_per_step": h2d,

@@ -333,8 +333,8 @@ size_t slkv_compress_host_arena_bytes(const slkv_params* p, const int32_t* cu_se
  * offsets, kept_idx are HOST outputs.  `arena` is caller-owned DEVICE memory of at least
  * slkv_compress_host_arena_bytes, 256-byte aligned.  The call copies the inputs to the arena, runs the
  * kernels, copies offsets, kept_idx and the packed rows back and waits for `stream` before returning, so
- * the outputs are valid on return.  Pinned host buffers make the copies asynchronous and fast; pageable
- * ones work.  Returns SLKV_ERR_CAPACITY if out_capacity_rows is too small (nothing is copied back then
+ * the outputs are valid on return.  Page-locked host buffers make it fast (of V only the kept rows then cross
+ * the link, and the outputs are written without a copy); pageable ones work.  Returns SLKV_ERR_CAPACITY if out_capacity_rows is too small (nothing is copied back then
  * except offsets).  *rows_out (optional) receives offsets[last].
  */
 int slkv_compress_host(const slkv_params* p, const void* q_win, const void* k, const void* v,

@@ -199,6 +199,8 @@ struct TailLayer {
   const void* v;
   void* k_out;
   void* v_out;
+  int32_t* kept_copy;           // optional: kept_idx and offsets once more, written by the gather
+  int32_t* offsets_copy;
   long long capacity;
 };
 bool select_list_supported(const Problem& pb);

@@ -213,10 +213,13 @@ k_gather(const __grid_constant__ GatherArgs g) {
   const unsigned char* v = static_cast<const unsigned char*>(a.v);
   pdl_wait();
   const long long n_rows = min((long long)a.offsets[g.n_seg], max_rows);
+  if (a.offsets_copy && blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= g.n_seg; i += blockDim.x) a.offsets_copy[i] = a.offsets[i];
   for (long long r = (long long)blockIdx.x * rows_per_cta + sub; r < max_rows;
        r += (long long)gridDim.x * rows_per_cta) {
     const int src = a.gather_src[r];                        // in bounds for r < max_rows; valid for r < n_rows
     if (r >= n_rows) break;
+    if (a.kept_copy && lane == 0) a.kept_copy[r] = a.kept_idx[r];
     const int tok = src / g.n_kv_heads, h = src - tok * g.n_kv_heads;
     const uint4 kv = *reinterpret_cast<const uint4*>(k + tok * g.k_tok_bytes + h * g.k_head_bytes + lane * 16);
     const uint4 vv = *reinterpret_cast<const uint4*>(v + tok * g.v_tok_bytes + h * g.v_head_bytes + lane * 16);
