@@ -794,18 +794,24 @@ k_score_list(const __grid_constant__ ListArgs a) {
   c.stage_bytes = c.halves * kHalfBytes;
   c.q = smem_u32(smem);
   c.k = c.q + (uint32_t)(c.n_q * c.q_bytes);
-  // Everything above touched only this CTA's own resources.
+  // Everything above touched only this CTA's own resources, and so does all that follows up to the first load of a tile and
+  // the clearing of the statistics area: those two roles wait for the kernels before this one, the others get their work
+  // from them.  The first runs are worked out meanwhile.
   pdl_launch_dependents();
-  pdl_wait();
-  if (tid == 0) trace_mark(a.trace, 1);
 
   if (warp == 0) {
-    if (lane == 0) producer(c);
+    if (lane == 0) {
+      pdl_wait();
+      trace_mark(a.trace, 1);
+      producer(c);
+    }
   } else if (warp == 1) {
     if (lane == 0) issuer(c);
   } else if (warp == 2) {
+    if (sh.tab.n_inline == 0) pdl_wait();              // a kernel before this one writes the tables
     scheduler_publisher(c, a);
   } else if (warp == 3) {
+    pdl_wait();
     fetch_lse(c, a);
   } else {
     epilogue(c);

@@ -77,7 +77,8 @@ __device__ __forceinline__ void pool8(const float (&x)[16], bool max_mode, float
   }
 }
 
-template <int RAD>
+// CLUSTER: a segment is shared by the CTAs of a cluster (else every pointer below is known to be this CTA's own memory).
+template <int RAD, bool CLUSTER>
 __global__ void __launch_bounds__(kThreads, 1)
 k_select_list(const __grid_constant__ SelArgs args) {
   extern __shared__ __align__(16) float votes_sh[];
@@ -86,13 +87,13 @@ k_select_list(const __grid_constant__ SelArgs args) {
   __shared__ __align__(16) unsigned list[kList];
   __shared__ unsigned wsum[3][kWarps];
   __shared__ int2 cta_tot;                              // read by the cluster's other CTAs
-  __shared__ unsigned sh_lo, sh_hi, sh_tau, sh_bin, sh_n;
-  __shared__ int sh_above, sh_m, sh_need;
+  __shared__ unsigned sh_lo, sh_hi, sh_top, sh_tau, sh_bin, sh_n;
+  __shared__ int sh_above, sh_m, sh_need, sh_r[2];
 
   cg::cluster_group cluster = cg::this_cluster();
-  const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int CS = CLUSTER ? (int)cluster.num_blocks() : 1, rank = CLUSTER ? (int)cluster.block_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  auto sync_all = [&]() { if (CS > 1) cluster.sync(); else __syncthreads(); };
+  auto sync_all = [&]() { if (CLUSTER) cluster.sync(); else __syncthreads(); };
   pdl_launch_dependents();
   const TailLayer& a = args.lay[blockIdx.y];
   const int seg = blockIdx.x / CS, s = seg / args.n_kv_heads, h = seg - s * args.n_kv_heads;
@@ -130,9 +131,8 @@ k_select_list(const __grid_constant__ SelArgs args) {
     }
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
-  const int k_keep = kept_rows(len, a.budgets[h], args.window) - n_win;       // C_H = C - window, clamped
-  const bool choose = k_keep > 0 && k_keep < n;
-  if (choose && tid < kSamples) {
+  const int budget = __ldg(a.budgets + h);
+  if (n > 0 && tid < kSamples) {
     const int p = (int)(((long long)(2 * tid + 1) * n) / (2 * kSamples));
     float w[2 * RAD + 1];
 #pragma unroll
@@ -154,6 +154,14 @@ k_select_list(const __grid_constant__ SelArgs args) {
     }
     part = __reduce_add_sync(kAll, part);
     if (lane == 0) wsum[0][wid] = part;
+  }
+  const int k_keep = kept_rows(len, budget, args.window) - n_win;             // C_H = C - window, clamped
+  const bool choose = k_keep > 0 && k_keep < n;
+  if (wid == kWarps - 1 && choose) {
+    // sample ranks that bracket the k-th score; outside 0 .. kSamples - 1: no bound there
+    const float f = __fdividef((float)k_keep, (float)n), q = (float)kSamples * f;
+    const float dev = 4.f * sqrtf(q * (1.f - f)) + 1.f;
+    if (lane == 0) { sh_r[0] = (int)floorf(q - dev) - 1; sh_r[1] = (int)ceilf(q + dev); }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
@@ -186,9 +194,7 @@ k_select_list(const __grid_constant__ SelArgs args) {
 
   // ---- the bracket: ranks of the samples by counting, eight lanes per sample
   if (choose) {
-    const float q = (float)kSamples * (float)k_keep / (float)n;
-    const float dev = 4.f * sqrtf(q * (1.f - (float)k_keep / (float)n)) + 1.f;
-    const int r_hi = (int)floorf(q - dev) - 1, r_lo = (int)ceilf(q + dev);     // outside 0 .. kSamples - 1: no bound there
+    const int r_hi = sh_r[0], r_lo = sh_r[1];
     const int i = tid >> 3, part = tid & 7;
     const unsigned x = samp[i];
     int above = 0;
@@ -200,6 +206,7 @@ k_select_list(const __grid_constant__ SelArgs args) {
     above += __shfl_xor_sync(kAll, above, 1);
     above += __shfl_xor_sync(kAll, above, 2);
     above += __shfl_xor_sync(kAll, above, 4);
+    if (part == 0 && above == 0) sh_top = x | (kSamples - 1u);
     if (part == 0 && above == r_hi) sh_hi = x | (kSamples - 1u);
     if (part == 0 && above == r_lo) sh_lo = x & ~(kSamples - 1u);
   }
@@ -268,7 +275,7 @@ k_select_list(const __grid_constant__ SelArgs args) {
   {
     const unsigned tot = __reduce_add_sync(kAll, wsum[1][lane]);
     int n_gt = (int)(tot & 0xffffu), n_cand = (int)(tot >> 16);
-    if (CS > 1) {
+    if (CLUSTER) {
       if (tid == 0) cta_tot = make_int2(n_gt, n_cand);
       cluster.sync();
       int2 o = make_int2(0, 0);
@@ -286,14 +293,15 @@ k_select_list(const __grid_constant__ SelArgs args) {
   }
 
   // ---- radix descent inside [lo, hi]: `need` of the scores there, the largest, are kept
-  unsigned tau;
+  // the bins divide lo .. top, the last one takes what lies above; at first top is four times the largest sample
+  unsigned tau, top = max(min(sh_top + (2u << 23), hi), lo);
   while (true) {
-    const unsigned span = hi - lo;
+    const unsigned span = top - lo;
     const int sh = span < (unsigned)kBins ? 0 : 21 - __clz(span);
-    for (unsigned m = cand; m != 0; m &= m - 1) atomicAdd(&hist[(keys[__ffs(m) - 1] - lo) >> sh], 1);
+    for (unsigned m = cand; m != 0; m &= m - 1) atomicAdd(&hist[min((keys[__ffs(m) - 1] - lo) >> sh, kBins - 1u)], 1);
     sync_all();
     int2 c2 = reinterpret_cast<const int2*>(hist)[tid];
-    if (CS > 1)
+    if (CLUSTER)
       for (int o = 1; o < CS; ++o) {
         const int2 x = reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, (rank + o) % CS))[tid];
         c2.x += x.x;
@@ -318,25 +326,29 @@ k_select_list(const __grid_constant__ SelArgs args) {
     const int m_bin = sh_m;
     need -= sh_above;
     lo += sh_bin << sh;
-    hi = min(hi, lo + ((1u << sh) - 1u));
-    if (sh == 0) { tau = lo; break; }
+    if (sh_bin < kBins - 1u) hi = min(hi, lo + ((1u << sh) - 1u));
+    top = hi;
+    if (lo == hi) { tau = lo; break; }
     // the bin's scores go on; where they fit, in a list of the cluster's first CTA (their order does not matter)
     const bool listed = m_bin <= kList;
-    unsigned* list0 = CS > 1 ? cluster.map_shared_rank(list, 0) : list;
-    unsigned* n0 = CS > 1 ? cluster.map_shared_rank(&sh_n, 0) : &sh_n;
+    unsigned* list0 = CLUSTER ? cluster.map_shared_rank(list, 0) : nullptr;
+    unsigned* n0 = CLUSTER ? cluster.map_shared_rank(&sh_n, 0) : nullptr;
     unsigned in_bin = 0;
     for (unsigned m = cand; m != 0; m &= m - 1) {
       const unsigned v = keys[__ffs(m) - 1], bit = m & (0u - m);
       if (v > hi) gt |= bit;
       else if (v >= lo) {
         in_bin |= bit;
-        if (listed) list0[atomicAdd(n0, 1u)] = v;
+        if (listed) {
+          if (CLUSTER) list0[atomicAdd(n0, 1u)] = v;
+          else list[atomicAdd(&sh_n, 1u)] = v;
+        }
       }
     }
     cand = in_bin;
     if (listed) {                                         // ranked by counting
       sync_all();
-      if (CS > 1 && rank > 0) {
+      if (CLUSTER && rank > 0) {
         for (int i = tid; i < m_bin; i += kThreads) list[i] = list0[i];
         __syncthreads();
       }
@@ -380,7 +392,7 @@ k_select_list(const __grid_constant__ SelArgs args) {
   __syncthreads();
   const unsigned before = __reduce_add_sync(kAll, lane < wid ? wsum[2][lane] : 0u) + inc - cnt;
   int gt_before = (int)(before & 0xffffu), eq_before = (int)(before >> 16);
-  if (CS > 1) {
+  if (CLUSTER) {
     if (tid == kThreads - 1) cta_tot = make_int2(gt_before + __popc(gt), eq_before + __popc(eq));
     cluster.sync();
     int2 o = make_int2(0, 0);
@@ -394,7 +406,7 @@ k_select_list(const __grid_constant__ SelArgs args) {
   for (int t = 0; t < take; ++t) { kept |= eq & (0u - eq); eq &= eq - 1; }
   long long o = out0 + gt_before + min(eq_before, need);
   for (unsigned m = kept; m != 0; m &= m - 1, ++o) put(o, base + i0 + __ffs(m) - 1);
-  if (CS > 1) cluster.sync();                             // nobody leaves while its shared memory may still be read
+  if (CLUSTER) cluster.sync();                             // nobody leaves while its shared memory may still be read
 }
 
 int cluster_size(const Problem& pb) {
@@ -411,8 +423,9 @@ bool select_list_supported(const Problem& pb) {
 
 cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
   typedef void (*Kern)(const SelArgs);
-  static const Kern kerns[kMaxRadius + 1] = {k_select_list<0>, k_select_list<1>, k_select_list<2>, k_select_list<3>,
-                                             k_select_list<4>};
+  static const Kern kerns[2][kMaxRadius + 1] = {
+      {k_select_list<0, false>, k_select_list<1, false>, k_select_list<2, false>, k_select_list<3, false>, k_select_list<4, false>},
+      {k_select_list<0, true>, k_select_list<1, true>, k_select_list<2, true>, k_select_list<3, true>, k_select_list<4, true>}};
   const int cs = cluster_size(pb);
   const int slice = ((pb.max_hist + 3 + cs - 1) / cs + 3) & ~3;
   const size_t smem = (size_t)vote_floats(slice <= 8 * kThreads ? 3 : (slice <= 16 * kThreads ? 4 : 5)) * sizeof(float);
@@ -421,8 +434,8 @@ cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_la
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
-    for (int r = 0; r <= kMaxRadius; ++r) {
-      e = cudaFuncSetAttribute(kerns[r], cudaFuncAttributeMaxDynamicSharedMemorySize, vote_floats(5) * (int)sizeof(float));
+    for (int r = 0; r < 2 * (kMaxRadius + 1); ++r) {
+      e = cudaFuncSetAttribute(kerns[r & 1][r >> 1], cudaFuncAttributeMaxDynamicSharedMemorySize, vote_floats(5) * (int)sizeof(float));
       if (e != cudaSuccess) return e;
     }
     configured_dev = dev;
@@ -432,7 +445,7 @@ cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_la
   a.n_seqs = pb.p.n_seqs; a.n_kv_heads = pb.p.n_kv_heads; a.window = pb.p.window; a.pool_mode = pb.p.pool_mode;
   for (int i = 0; i < n_layers; ++i) a.lay[i] = lay[i];
   LaunchScope scope(KID_SELECT, st, launches);
-  return launch_pdl(kerns[pb.p.pool_kernel >> 1], dim3((unsigned)(pb.n_seg * cs), (unsigned)n_layers), dim3(kThreads), smem, st, cs, a);
+  return launch_pdl(kerns[cs > 1][pb.p.pool_kernel >> 1], dim3((unsigned)(pb.n_seg * cs), (unsigned)n_layers), dim3(kThreads), smem, st, cs, a);
 }
 
 }  // namespace slkv
