@@ -221,7 +221,7 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
 // ---- overlapped calls ---------------------------------------------------------------------------------------
 // A call queues its layer; a list of layers goes out as three launches on the caller's stream -- scores, selections,
 // gathers, each over all layers of the list -- when it is full or at a join.  What a list gives over single calls: the
-// statistics of one layer overlap the votes of another, 16 layers' selections fill the SMs side by side, and the host
+// statistics of one layer overlap the votes of another, all layers' selections fill the SMs side by side, and the host
 // makes three launches instead of 48.
 struct ListState {
   bool open = false;             // the shape below is valid

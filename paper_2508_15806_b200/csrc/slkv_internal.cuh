@@ -185,7 +185,7 @@ cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32
 cudaError_t launch_pool(const Problem& pb, float* pooled, cudaStream_t st, int* launches);
 cudaError_t launch_select(const Problem& pb, const float* pooled, const int32_t* budgets, const int32_t* offsets,
                           int32_t* kept_idx, int64_t capacity, cudaStream_t st, int* launches);
-constexpr int kListMaxLayers = 16;          // layers one launch of the score, selection and gather kernels takes
+constexpr int kListMaxLayers = 32;          // layers one launch of the score, selection and gather kernels takes
 // ---- selection and gather over a list of layers of one shape ------------------------------------------------------
 struct TailLayer {
   const float* vote;

@@ -21,7 +21,7 @@
 //   warps 4-19 four warpgroups, unit u belongs to warpgroup u % 4: TMEM -> registers -> exponentials
 // so that the warps that do the arithmetic -- what bounds the kernel -- meet no other CTA, no global latency, no CTA-wide
 // barrier and no launch parameters: with every role walking the phases by itself, divisions and constant-cache misses
-// (the parameters of 16 layers are 7 KB) took 3600 cycles per run and 1000 per tile of the MMA thread.
+// (the parameters of a list are kilobytes) took 3600 cycles per run and 1000 per tile of the MMA thread.
 //
 // What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
 //   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; two in eight go to the FMA pipe
