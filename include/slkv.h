@@ -305,7 +305,31 @@ int slkv_join(void* stream);
  *   ties_all   [n_parts][n_kv_heads]: every rank's slkv_cp_local_ties; part = this rank's index
  *   offsets    out, int32[n_kv_heads + 1]; kept_idx out, positions in the whole sequence; k_out, v_out as slkv_compress
  *   status     optional: SLKV_ERR_CAPACITY if offsets[n_kv_heads] > out_capacity_rows
+ *
+ * slkv_cp_step is steps 4 and 5 up to the packing with one launch between two collectives:
+ *   level 0            what slkv_cp_select_init does, then the level-0 histogram
+ *   level 1, 2         slkv_cp_descend of the level before on hist_sum, then this level's histogram
+ *   level 3            slkv_cp_descend of level 2, then the owned positions above the threshold and those equal to it:
+ *                      totals[0 .. n_kv_heads) above, totals[n_kv_heads .. 2 n_kv_heads) equal (= the ties to all-gather),
+ *                      and counts by slice into the workspace for slkv_cp_emit_counted (workspace: level 3 only)
+ *   state      int32 [4][2][n_kv_heads]: prefix and need after each level; state[3] goes to slkv_cp_emit_counted
+ *   hist, totals  ADDED to: zeroed by the caller before the call; hist_sum: the histograms of the level before, summed
+ *              over ranks
+ *   clear      optional: clear_bytes (a multiple of 16, from a 16-byte boundary) are set to zero by the same launch --
+ *              a share of k_out / v_out, where rows that nothing is packed into should be zero
+ * slkv_cp_emit_counted is slkv_cp_emit on those totals and counts (same workspace contents); it also sets kept_idx to -1
+ * behind the last packed row.  totals == NULL: exactly slkv_cp_emit.
  */
+int slkv_cp_step(const int32_t* budgets, int32_t n_kv_heads, int32_t window, int64_t seq_len, int32_t level,
+                 int32_t* state, const int32_t* hist_sum, const float* pooled, int64_t row_stride, int32_t own_begin,
+                 int32_t own_count, int32_t* hist, int32_t* totals, void* clear, size_t clear_bytes, void* workspace,
+                 size_t workspace_bytes, void* stream);
+int slkv_cp_emit_counted(const slkv_params* p, const void* k, const void* v, int64_t rows, const float* pooled,
+                         int64_t row_stride, int32_t own_begin, int32_t own_count, int64_t pos0,
+                         const uint32_t* threshold, const int32_t* need, const int32_t* ties_all, int32_t n_parts,
+                         int32_t part, int32_t window_rows, int64_t window_pos0, const int32_t* totals, void* k_out,
+                         void* v_out, int64_t out_capacity_rows, int32_t* offsets, int32_t* kept_idx, int32_t* status,
+                         void* workspace, size_t workspace_bytes, void* stream);
 int slkv_cp_merge_lse(const slkv_params* p, const float* lse_parts, int32_t n_parts, float* lse_out, void* stream);
 int slkv_cp_select_init(const int32_t* budgets, int32_t n_kv_heads, int32_t window, int64_t seq_len, uint32_t* prefix,
                         int32_t* need, void* stream);

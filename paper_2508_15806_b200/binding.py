@@ -401,6 +401,28 @@ def slkv_cp_local_ties(hist_local: torch.Tensor, prefix: torch.Tensor, ties: tor
     return ties
 
 
+def slkv_cp_step(budgets: Optional[torch.Tensor], n_kv_heads: int, window: int, seq_len: int, level: int, state,
+                 hist_sum: Optional[torch.Tensor], pooled: torch.Tensor, row_stride: int, own_begin: int, own_count: int,
+                 hist: Optional[torch.Tensor], totals: Optional[torch.Tensor] = None, clear=None, clear_bytes: int = 0,
+                 workspace=None, workspace_bytes: int = 0, stream=None) -> None:
+    """One launch between two collectives (see include/slkv.h).  state, clear and workspace: tensors or addresses."""
+    _check(_fn["slkv_cp_step"](stream, budgets, n_kv_heads, window, seq_len, level, state, hist_sum, pooled, row_stride,
+                               own_begin, own_count, hist, totals, clear, clear_bytes, workspace, workspace_bytes),
+           "slkv_cp_step")
+
+
+def slkv_cp_emit_counted(params: SlkvParams, k: torch.Tensor, v: torch.Tensor, rows: int, pooled: torch.Tensor,
+                         row_stride: int, own_begin: int, own_count: int, pos0: int, threshold, need,
+                         ties_all: torch.Tensor, part: int, window_rows: int, window_pos0: int, totals: torch.Tensor,
+                         k_out: torch.Tensor, v_out: torch.Tensor, offsets: torch.Tensor, kept_idx: torch.Tensor,
+                         workspace, workspace_bytes: int, status: Optional[torch.Tensor] = None, stream=None) -> None:
+    """slkv_cp_emit behind slkv_cp_step's level 3.  threshold, need and workspace: tensors or addresses."""
+    _check(_fn["slkv_cp_emit_counted"](stream, params, k, v, rows, pooled, row_stride, own_begin, own_count, pos0,
+                                       threshold, need, ties_all, ties_all.size(0), part, window_rows, window_pos0,
+                                       totals, k_out, v_out, k_out.size(0), offsets, kept_idx, status, workspace,
+                                       workspace_bytes), "slkv_cp_emit_counted")
+
+
 def slkv_cp_workspace_bytes(n_kv_heads: int, own_count: int, capacity_rows: int) -> int:
     return int(lib().slkv_cp_workspace_bytes(int(n_kv_heads), int(own_count), int(capacity_rows)))
 

@@ -97,63 +97,64 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
     in the whole sequence), status, pooled (the rank's scores, margins included) and lse (the merged row statistics)."""
     sh = shard
     assert sh.seq_len >= sh.window and comm.world == sh.world and comm.rank == sh.rank
-    dev = sh.k.device
-    w, hkv, hq, d = sh.window, sh.k.shape[1], sh.q_win.shape[2], sh.k.shape[2]
-    f32, i32 = dict(dtype=torch.float32, device=dev), dict(dtype=torch.int32, device=dev)
+    dev, dt = sh.k.device, sh.k.dtype
+    w, own, (rows, hkv, d), hq = sh.window, sh.own, sh.k.shape, sh.q_win.shape[2]
     n_win = w if sh.last else 0
-    status = torch.zeros(1, **i32)
-    cu_dev1 = torch.zeros(2, **i32)              # one sequence: the library's tables are inline, this is never read
+    n_ext = sh.margin_left + own + sh.margin_right
+    row_stride, cap = max(n_ext, 1), hkv * (own + n_win)
+    p = B.make_params(sh.q_win, sh.k, sh.v, w, pool_kernel, pool_mode, score_path, softmax_domain, B.SLKV_LSE_LOG2)
+    p.history_only = 0 if sh.last else 1
 
-    def params_for(k_rows: torch.Tensor, history_only: bool) -> B.SlkvParams:
-        p = B.make_params(sh.q_win, k_rows, None, w, pool_kernel, pool_mode, score_path, softmax_domain, B.SLKV_LSE_LOG2)
-        p.history_only = 1 if history_only else 0
-        return p
+    # one buffer for what has to start at zero, one for all scratch: the calls below come one after the other
+    zeroed = torch.zeros(3 * 2048 * hkv + 3 * hkv + 2, dtype=torch.int32, device=dev)
+    hists, totals, offsets, status = zeroed.split((3 * 2048 * hkv, 2 * hkv, hkv + 1, 1))
+    n_own = own + n_win
+    has_keys = own > 0 or (sh.last and softmax_domain == B.SLKV_ALL_CAUSAL)
+    ws_score = B.slkv_workspace_bytes(p, [0, rows]) if n_ext > 0 else 0
+    ws_lse = 0 if not has_keys else (ws_score if n_own == rows and n_ext > 0 else B.slkv_workspace_bytes(p, [0, n_own]))
+    ws_emit = B.slkv_cp_workspace_bytes(hkv, own, max(cap, 1))
+    state_bytes = -(-32 * hkv // 256) * 256                    # [4][2][hkv]: every head's prefix and need after each level
+    ws = torch.empty(state_bytes + max(ws_score, ws_lse, ws_emit), dtype=torch.uint8, device=dev)
+    state = ws.data_ptr()
+    scratch = ws[state_bytes:]
 
     # 1. the rows' log-sum-exp over the keys this rank owns (the last rank's range is an ordinary sequence tail)
-    k_own = sh.k[sh.margin_left:sh.margin_left + sh.own + n_win]
-    lse_local = torch.full((1, hq, w), float("-inf"), **f32)
-    if sh.own > 0 or (sh.last and softmax_domain == B.SLKV_ALL_CAUSAL):
-        p_own = params_for(k_own, not sh.last)
-        cu = [0, k_own.shape[0]]
-        ws = torch.empty(max(B.slkv_workspace_bytes(p_own, cu), 256), dtype=torch.uint8, device=dev)
-        B.slkv_row_lse(p_own, sh.q_win, k_own, cu_dev1, cu, lse_local, ws, status, stream)
+    if has_keys:
+        lse_local = torch.empty(hq, w, dtype=torch.float32, device=dev)
+        k_own = sh.k if n_own == rows else sh.k[sh.margin_left:sh.margin_left + n_own]
+        B.slkv_row_lse(p, sh.q_win, k_own, status, (0, n_own), lse_local, scratch, status, stream)
+    else:
+        lse_local = torch.full((hq, w), float("-inf"), dtype=torch.float32, device=dev)
     # 2. merged over the ranks
-    lse = torch.empty(1, hq, w, **f32)
-    p_any = params_for(sh.k, not sh.last)
-    B.slkv_cp_merge_lse(p_any, comm.all_gather(lse_local.reshape(hq, w)), lse, stream)
+    lse = torch.empty(1, hq, w, dtype=torch.float32, device=dev)
+    B.slkv_cp_merge_lse(p, comm.all_gather(lse_local), lse, stream)
     # 3. pooled scores of the owned rows and the neighbours' margins
-    n_ext = sh.margin_left + sh.own + sh.margin_right
-    pooled = torch.zeros(hkv * max(n_ext, 1), **f32)
     if n_ext > 0:
-        cu = [0, sh.k.shape[0]]
-        ws = torch.empty(max(B.slkv_workspace_bytes(p_any, cu), 256), dtype=torch.uint8, device=dev)
-        B.slkv_score(p_any, sh.q_win, sh.k, cu_dev1, cu, pooled, ws, status, stream, lse=lse)
-    # 4. every head's threshold: radix descent on histograms summed over the ranks
-    prefix, need = torch.zeros(hkv, **i32), torch.zeros(hkv, **i32)
-    B.slkv_cp_select_init(budgets_row, w, sh.seq_len, prefix, need, stream)
-    hist = torch.empty(hkv, 2048, **i32)
-    hist_own = hist
-    for level in range(3):
-        B.slkv_cp_histogram(pooled, hkv, max(n_ext, 1), sh.margin_left, sh.own, level, prefix, hist, stream)
-        if level == 2:
-            hist_own = hist.clone()
-        comm.all_reduce_sum(hist)
-        B.slkv_cp_descend(hist, level, prefix, need, stream)
+        pooled = torch.empty(hkv * n_ext, dtype=torch.float32, device=dev)
+        B.slkv_score(p, sh.q_win, sh.k, status, (0, rows), pooled, scratch, status, stream, lse=lse)
+    else:
+        pooled = torch.zeros(hkv, dtype=torch.float32, device=dev)
+    # 4. every head's threshold: radix descent on histograms summed over the ranks; the output rows are cleared meanwhile,
+    #    a quarter beside each level (every row is whole 16-byte units)
+    out_k, out_v = torch.empty(2, max(cap, 1), d, dtype=dt, device=dev).unbind(0)
+    clear, all16 = out_k.data_ptr(), 2 * out_k.numel() * out_k.element_size() // 16
+    hist_sum = None
+    for level, hist in enumerate((*hists.view(3, hkv, 2048).unbind(0), None)):
+        b, e = all16 * level // 4, all16 * (level + 1) // 4
+        B.slkv_cp_step(budgets_row, hkv, w, sh.seq_len, level, state, hist_sum, pooled, row_stride, sh.margin_left, own,
+                       hist, totals, clear + 16 * b, 16 * (e - b), scratch, ws_emit, stream)
+        if hist is not None:
+            comm.all_reduce_sum(hist)
+        hist_sum = hist
     # 5. ties in rank order, then this rank's packed rows
-    ties = torch.empty(hkv, **i32)
-    B.slkv_cp_local_ties(hist_own, prefix, ties, stream)
-    ties_all = comm.all_gather(ties)
-    cap = hkv * (sh.own + n_win)
-    out = dict(k_out=torch.zeros(max(cap, 1), d, dtype=sh.k.dtype, device=dev),
-               v_out=torch.zeros(max(cap, 1), d, dtype=sh.k.dtype, device=dev),
-               offsets=torch.zeros(hkv + 1, **i32), kept_idx=torch.full((max(cap, 1),), -1, **i32), status=status,
-               pooled=pooled, lse=lse, capacity=cap)
-    ws = torch.empty(max(B.slkv_cp_workspace_bytes(hkv, sh.own, max(cap, 1)), 256), dtype=torch.uint8, device=dev)
-    B.slkv_cp_emit(p_any, sh.k, sh.v, sh.k.shape[0], pooled, max(n_ext, 1), sh.margin_left, sh.own, sh.begin, prefix,
-                   need, ties_all, sh.rank, n_win, sh.seq_len - n_win, out["k_out"], out["v_out"], out["offsets"],
-                   out["kept_idx"], ws, status, stream)
-    out["keep_alive"] = (ws, hist, hist_own, ties_all, prefix, need, lse_local)
-    return out
+    ties_all = comm.all_gather(totals[hkv:])
+    kept_idx = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
+    threshold = state + 24 * hkv
+    B.slkv_cp_emit_counted(p, sh.k, sh.v, rows, pooled, row_stride, sh.margin_left, own, sh.begin, threshold,
+                           threshold + 4 * hkv, ties_all, sh.rank, n_win, sh.seq_len - n_win, totals, out_k, out_v,
+                           offsets, kept_idx, scratch, ws_emit, status, stream)
+    return dict(k_out=out_k, v_out=out_v, offsets=offsets, kept_idx=kept_idx, status=status, pooled=pooled, lse=lse,
+                capacity=cap, keep_alive=(ws, zeroed, ties_all, lse_local))
 
 
 def stitch_heads(per_rank: Sequence[dict], n_kv_heads: int) -> List[dict]:

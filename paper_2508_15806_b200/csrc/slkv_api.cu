@@ -358,6 +358,23 @@ cudaError_t join_lists(cudaStream_t st, int* launches) {
   return cudaSuccess;
 }
 
+// Workspace of the context-parallel packing: totals per head and counts per slice and head (above, equal), source rows
+// of the packed rows.
+struct CpWorkspace {
+  int32_t *totals, *cnt_gt, *cnt_eq, *gather_src;
+  size_t bytes;
+  CpWorkspace(void* ws, int32_t n_kv_heads, int32_t own_count, int64_t capacity) {
+    const size_t heads = 2 * align_up((size_t)n_kv_heads * sizeof(int32_t));
+    const size_t slices = align_up((size_t)cp_slices(own_count) * (size_t)n_kv_heads * sizeof(int32_t));
+    char* w = static_cast<char*>(ws);
+    totals = reinterpret_cast<int32_t*>(w);
+    cnt_gt = reinterpret_cast<int32_t*>(w + heads);
+    cnt_eq = reinterpret_cast<int32_t*>(w + heads + slices);
+    gather_src = reinterpret_cast<int32_t*>(w + heads + 2 * slices);
+    bytes = heads + 2 * slices + align_up((size_t)capacity * sizeof(int32_t));
+  }
+};
+
 TailLayer tail_of(const Problem& pb, const int32_t* budgets, void* k_out, void* v_out, int64_t capacity, int32_t* offsets,
                   int32_t* kept_idx, float* pooled_opt, int32_t* status) {
   TailLayer t;
@@ -602,8 +619,11 @@ int slkv_cp_select_init(const int32_t* budgets, int32_t n_kv_heads, int32_t wind
   if (!budgets || !prefix || !need) return SLKV_ERR_NULL_PTR;
   if (n_kv_heads < 1 || n_kv_heads > 65535 || window < 1 || window > kMaxWindow || seq_len < 0 || seq_len >= (1ll << 31))
     return SLKV_ERR_BAD_SHAPE;
+  CpStep a = {};
+  a.budgets = budgets; a.n_kv_heads = n_kv_heads; a.window = window; a.seq_len = seq_len;
+  a.prefix_out = prefix; a.need_out = need;
   int launches = 0;
-  cudaError_t e = launch_cp_need_init(budgets, n_kv_heads, window, seq_len, prefix, need, (cudaStream_t)stream, &launches);
+  cudaError_t e = launch_cp_step(a, (cudaStream_t)stream, &launches);
   return e == cudaSuccess ? SLKV_OK : cuda_fail(e);
 }
 
@@ -613,9 +633,13 @@ int slkv_cp_histogram(const float* pooled, int32_t n_kv_heads, int64_t row_strid
   if (n_kv_heads < 1 || n_kv_heads > 65535 || row_stride < 0 || own_begin < 0 || own_count < 0 ||
       (int64_t)own_begin + own_count > row_stride || level < 0 || level > 2)
     return SLKV_ERR_BAD_SHAPE;
+  cudaError_t e = cudaMemsetAsync(hist, 0, (size_t)n_kv_heads * kCpBins * sizeof(int32_t), (cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_fail(e);
+  CpStep a = {};
+  a.prefix_in = prefix; a.n_kv_heads = n_kv_heads; a.pooled = pooled; a.row_stride = row_stride;
+  a.own_begin = own_begin; a.own_count = own_count; a.level_out = level; a.hist = hist;
   int launches = 0;
-  cudaError_t e = launch_cp_histogram(pooled, n_kv_heads, row_stride, own_begin, own_count, level, prefix, hist,
-                                      (cudaStream_t)stream, &launches);
+  e = launch_cp_step(a, (cudaStream_t)stream, &launches);
   return e == cudaSuccess ? SLKV_OK : cuda_fail(e);
 }
 
@@ -623,8 +647,11 @@ int slkv_cp_descend(const int32_t* hist, int32_t n_kv_heads, int32_t level, uint
                     void* stream) {
   if (!hist || !prefix || !need) return SLKV_ERR_NULL_PTR;
   if (n_kv_heads < 1 || n_kv_heads > 65535 || level < 0 || level > 2) return SLKV_ERR_BAD_SHAPE;
+  CpStep a = {};
+  a.prefix_in = prefix; a.need_in = need; a.prefix_out = prefix; a.need_out = need;
+  a.n_kv_heads = n_kv_heads; a.hist_sum = hist; a.level_in = level;
   int launches = 0;
-  cudaError_t e = launch_cp_descend(hist, n_kv_heads, level, prefix, need, (cudaStream_t)stream, &launches);
+  cudaError_t e = launch_cp_step(a, (cudaStream_t)stream, &launches);
   return e == cudaSuccess ? SLKV_OK : cuda_fail(e);
 }
 
@@ -639,17 +666,55 @@ int slkv_cp_local_ties(const int32_t* hist_local, const uint32_t* prefix, int32_
 
 size_t slkv_cp_workspace_bytes(int32_t n_kv_heads, int32_t own_count, int64_t out_capacity_rows) {
   if (n_kv_heads < 1 || own_count < 0 || out_capacity_rows < 0) return 0;
-  // source rows of the packed rows; rows and tie shares per head; two counts per slice of the owned range and head
-  const size_t slices = (size_t)cp_slices(own_count) * (size_t)n_kv_heads;
-  return align_up((size_t)out_capacity_rows * sizeof(int32_t)) + 2 * align_up((size_t)n_kv_heads * sizeof(int32_t)) +
-         2 * align_up(slices * sizeof(int32_t));
+  return CpWorkspace(nullptr, n_kv_heads, own_count, out_capacity_rows).bytes;
 }
 
-int slkv_cp_emit(const slkv_params* p, const void* k, const void* v, int64_t rows, const float* pooled,
-                 int64_t row_stride, int32_t own_begin, int32_t own_count, int64_t pos0, const uint32_t* threshold,
-                 const int32_t* need, const int32_t* ties_all, int32_t n_parts, int32_t part, int32_t window_rows,
-                 int64_t window_pos0, void* k_out, void* v_out, int64_t out_capacity_rows, int32_t* offsets,
-                 int32_t* kept_idx, int32_t* status, void* workspace, size_t workspace_bytes, void* stream) {
+int slkv_cp_step(const int32_t* budgets, int32_t n_kv_heads, int32_t window, int64_t seq_len, int32_t level,
+                 int32_t* state, const int32_t* hist_sum, const float* pooled, int64_t row_stride, int32_t own_begin,
+                 int32_t own_count, int32_t* hist, int32_t* totals, void* clear, size_t clear_bytes, void* workspace,
+                 size_t workspace_bytes, void* stream) {
+  if (!state || !pooled || (level == 0 ? !budgets : !hist_sum) || (level < 3 ? !hist : !totals) || (clear_bytes && !clear))
+    return SLKV_ERR_NULL_PTR;
+  if (n_kv_heads < 1 || n_kv_heads > 65535 || window < 1 || window > kMaxWindow || seq_len < 0 ||
+      seq_len >= (1ll << 31) || row_stride < 0 || own_begin < 0 || own_count < 0 ||
+      (int64_t)own_begin + own_count > row_stride || level < 0 || level > 3 || clear_bytes % 16 != 0)
+    return SLKV_ERR_BAD_SHAPE;
+  if (!aligned16(clear)) return SLKV_ERR_BAD_ALIGN;
+  CpStep a = {};
+  a.n_kv_heads = n_kv_heads; a.window = window; a.seq_len = seq_len;
+  a.pooled = pooled; a.row_stride = row_stride; a.own_begin = own_begin; a.own_count = own_count;
+  a.clear = clear; a.clear_bytes = (long long)clear_bytes;
+  int32_t* mine = state + (size_t)level * 2 * n_kv_heads;          // state[level]: prefix, need
+  a.prefix_out = reinterpret_cast<unsigned*>(mine);
+  a.need_out = mine + n_kv_heads;
+  if (level == 0) {
+    a.budgets = budgets;
+  } else {
+    a.prefix_in = a.prefix_out - 2 * n_kv_heads;
+    a.need_in = a.need_out - 2 * n_kv_heads;
+    a.hist_sum = hist_sum;
+    a.level_in = level - 1;
+  }
+  if (level < 3) {
+    a.hist = hist;
+    a.level_out = level;
+  } else {
+    const CpWorkspace w(workspace, n_kv_heads, own_count, 0);
+    if (!workspace || workspace_bytes < w.bytes || reinterpret_cast<uintptr_t>(workspace) % kAlign != 0)
+      return SLKV_ERR_WORKSPACE;
+    a.cnt_gt = w.cnt_gt; a.cnt_eq = w.cnt_eq; a.tot_gt = totals; a.tot_eq = totals + n_kv_heads;
+  }
+  int launches = 0;
+  cudaError_t e = launch_cp_step(a, (cudaStream_t)stream, &launches);
+  return e == cudaSuccess ? SLKV_OK : cuda_fail(e);
+}
+
+int slkv_cp_emit_counted(const slkv_params* p, const void* k, const void* v, int64_t rows, const float* pooled,
+                         int64_t row_stride, int32_t own_begin, int32_t own_count, int64_t pos0,
+                         const uint32_t* threshold, const int32_t* need, const int32_t* ties_all, int32_t n_parts,
+                         int32_t part, int32_t window_rows, int64_t window_pos0, const int32_t* totals, void* k_out,
+                         void* v_out, int64_t out_capacity_rows, int32_t* offsets, int32_t* kept_idx, int32_t* status,
+                         void* workspace, size_t workspace_bytes, void* stream) {
   g_last_launches = 0;
   if (!p || !k || !v || !pooled || !threshold || !need || !ties_all || !k_out || !v_out || !offsets || !kept_idx)
     return SLKV_ERR_NULL_PTR;
@@ -664,30 +729,52 @@ int slkv_cp_emit(const slkv_params* p, const void* k, const void* v, int64_t row
     return SLKV_ERR_BAD_SHAPE;
   if (out_capacity_rows < 0) return SLKV_ERR_CAPACITY;
   if (!aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out)) return SLKV_ERR_BAD_ALIGN;
-  const size_t need_ws = slkv_cp_workspace_bytes(p->n_kv_heads, own_count, out_capacity_rows);
-  if (!workspace || workspace_bytes < need_ws || reinterpret_cast<uintptr_t>(workspace) % kAlign != 0)
+  const CpWorkspace w(workspace, p->n_kv_heads, own_count, out_capacity_rows);
+  if (!workspace || workspace_bytes < w.bytes || reinterpret_cast<uintptr_t>(workspace) % kAlign != 0)
     return SLKV_ERR_WORKSPACE;
-  char* w = static_cast<char*>(workspace);
-  int32_t* gather_src = reinterpret_cast<int32_t*>(w);
-  int32_t* rows_h = reinterpret_cast<int32_t*>(w + align_up((size_t)out_capacity_rows * sizeof(int32_t)));
-  int32_t* take_h = rows_h + align_up((size_t)p->n_kv_heads * sizeof(int32_t)) / sizeof(int32_t);
-  int32_t* cnt_gt = take_h + align_up((size_t)p->n_kv_heads * sizeof(int32_t)) / sizeof(int32_t);
-  int32_t* cnt_eq = cnt_gt + align_up((size_t)cp_slices(own_count) * p->n_kv_heads * sizeof(int32_t)) / sizeof(int32_t);
   cudaStream_t st = (cudaStream_t)stream;
   int launches = 0;
-  cudaError_t e = launch_cp_emit(pooled, row_stride, own_begin, own_count, pos0, threshold, need, ties_all,
-                                 p->n_kv_heads, part, window_rows, rows - window_rows, window_pos0, out_capacity_rows,
-                                 offsets, kept_idx, gather_src, rows_h, take_h, cnt_gt, cnt_eq, status, st, &launches);
+  cudaError_t e = cudaSuccess;
+  const bool counted = totals != nullptr;
+  if (!counted) {                                    // the counts of slkv_cp_step's last level
+    CpStep a = {};
+    a.prefix_in = threshold; a.n_kv_heads = p->n_kv_heads; a.pooled = pooled; a.row_stride = row_stride;
+    a.own_begin = own_begin; a.own_count = own_count;
+    a.cnt_gt = w.cnt_gt; a.cnt_eq = w.cnt_eq; a.tot_gt = w.totals; a.tot_eq = w.totals + p->n_kv_heads;
+    e = cudaMemsetAsync(w.totals, 0, 2 * (size_t)p->n_kv_heads * sizeof(int32_t), st);
+    if (e == cudaSuccess) e = launch_cp_step(a, st, &launches);
+    if (e != cudaSuccess) return cuda_fail(e);
+    totals = w.totals;
+  }
+  CpEmit m = {};
+  m.pooled = pooled; m.threshold = threshold; m.need = need; m.ties_all = ties_all;
+  m.cnt_gt = w.cnt_gt; m.cnt_eq = w.cnt_eq; m.tot_gt = totals; m.tot_eq = totals + p->n_kv_heads;
+  m.offsets = offsets; m.kept_idx = kept_idx; m.gather_src = w.gather_src; m.status = status;
+  m.row_stride = row_stride; m.pos0 = pos0; m.window_row0 = rows - window_rows; m.window_pos0 = window_pos0;
+  m.capacity = out_capacity_rows;
+  m.n_kv_heads = p->n_kv_heads; m.part = part; m.window_rows = window_rows; m.own_begin = own_begin;
+  m.own_count = own_count; m.fill_tail = counted;
+  e = launch_cp_emit(m, st, &launches);
   if (e != cudaSuccess) return cuda_fail(e);
   pb.total_tokens = rows;
   pb.n_seg = p->n_kv_heads;
   pb.k = k; pb.v = v;
-  pb.gather_src = gather_src;
+  pb.gather_src = w.gather_src;
   const TailLayer tail = tail_of(pb, nullptr, k_out, v_out, out_capacity_rows, offsets, kept_idx, nullptr, status);
   e = launch_gather(pb, &tail, 1, st, &launches);
   if (e != cudaSuccess) return cuda_fail(e);
   g_last_launches = launches;
   return SLKV_OK;
+}
+
+int slkv_cp_emit(const slkv_params* p, const void* k, const void* v, int64_t rows, const float* pooled,
+                 int64_t row_stride, int32_t own_begin, int32_t own_count, int64_t pos0, const uint32_t* threshold,
+                 const int32_t* need, const int32_t* ties_all, int32_t n_parts, int32_t part, int32_t window_rows,
+                 int64_t window_pos0, void* k_out, void* v_out, int64_t out_capacity_rows, int32_t* offsets,
+                 int32_t* kept_idx, int32_t* status, void* workspace, size_t workspace_bytes, void* stream) {
+  return slkv_cp_emit_counted(p, k, v, rows, pooled, row_stride, own_begin, own_count, pos0, threshold, need, ties_all,
+                              n_parts, part, window_rows, window_pos0, nullptr, k_out, v_out, out_capacity_rows, offsets,
+                              kept_idx, status, workspace, workspace_bytes, stream);
 }
 
 int slkv_alloc_budgets_ex(const float* inf_sc, int32_t n_layers, int32_t n_heads, int32_t fixed, int64_t total,

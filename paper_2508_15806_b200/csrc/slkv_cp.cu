@@ -11,9 +11,11 @@
 namespace slkv {
 namespace {
 
-constexpr int kCpBins = 2048;
 constexpr int kCpThreads = 1024;
-constexpr int kCpItems = 4;                 // consecutive positions per thread and round of k_cp_emit
+constexpr int kCpItems = 4;                 // consecutive positions per thread of k_cp_emit
+constexpr int kCpSlice = kCpThreads * kCpItems;       // positions counted, and packed, together
+constexpr int kCpStepThreads = 256;
+static_assert(kCpSlice == kCpStepThreads * 16 && kCpBins == kCpStepThreads * 8, "k_cp_step's shares of a thread");
 
 __device__ __forceinline__ unsigned cp_digit(unsigned bits, int level) {
   return level == 0 ? bits >> 21 : (level == 1 ? (bits >> 10) & 2047u : bits & 1023u);
@@ -37,110 +39,147 @@ __global__ void k_cp_merge_lse(const float* __restrict__ parts, int n_parts, lon
   out[i] = (m + log2f(z)) / to_log2;
 }
 
-// need[h] = history rows head h keeps of the whole sequence (Algorithm 3 l.1-3, l.7), prefix[h] = 0.
-__global__ void k_cp_need_init(const int32_t* __restrict__ budgets, int n_kv_heads, int window, long long seq_len,
-                               unsigned* __restrict__ prefix, int32_t* __restrict__ need) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= n_kv_heads) return;
-  const long long c = max((long long)budgets[h], (long long)window);
-  const long long kept = min(seq_len, c);
-  need[h] = (int32_t)(kept - min(seq_len, (long long)window));
-  prefix[h] = 0u;
-}
-
-// hist[h][d] += own positions of head h whose bits agree with prefix[h] above this level's digit and have digit d.
+// One step of the descent, with everything between two exchanges in one launch: per head
+//   start   from the budgets (level 0: need = the history rows the head keeps of the whole sequence, Algorithm 3 l.1-3,
+//           l.7; no prefix yet), or from a state, or from a state taken one level down on the histogram summed over all
+//           ranks: the digit d with count(digits > d) < need <= count(digits >= d) joins the prefix, need drops by the
+//           count above it (d = 0 if the counts above it never reach need; need == 0: the prefix becomes all ones --
+//           nothing lies above it -- and stays);
+//   count   the own positions by their digit of the next level, hist[h][d] += those whose bits agree with the prefix
+//           above it; or, with the threshold complete, by slice those above it and those equal to it, and their totals;
+//   clear   a share of the output buffers, by CTAs behind those that count.
+// Every CTA of a head repeats the start: 8 KB of bins from L2, less than a launch of its own (2.6 us).  The clearing is
+// what the memory is free for meanwhile: scores of 32k positions and 8 heads are 1 MB, the rows to clear 134 MB.
 // A thread takes 16 consecutive positions and adds a run of equal digits at once: pooled scores come in runs (a
 // maximum holds for pool_kernel positions), and neighbouring threads adding to the same bin one by one serialise.
-__global__ void __launch_bounds__(256)
-k_cp_histogram(const float* __restrict__ pooled, long long row_stride, int own_begin, int own_count, int level,
-               const unsigned* __restrict__ prefix, int32_t* __restrict__ hist) {
+__global__ void __launch_bounds__(kCpStepThreads) k_cp_step(const __grid_constant__ CpStep a) {
   __shared__ int sh[kCpBins];
-  pdl_launch_dependents();
-  const int h = blockIdx.y;
-  for (int b = threadIdx.x; b < kCpBins; b += blockDim.x) sh[b] = 0;
-  pdl_wait();
-  __syncthreads();
-  const unsigned pf = prefix[h];
-  const unsigned* row = reinterpret_cast<const unsigned*>(pooled + (long long)h * row_stride + own_begin);
-  for (long long j0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 16; j0 < own_count;
-       j0 += (long long)gridDim.x * blockDim.x * 16) {
-    int run_digit = -1, run = 0;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      int dg = -1;
-      if (j0 + q < own_count) {
-        const unsigned bits = row[j0 + q];
-        if (cp_match(bits, pf, level)) dg = (int)cp_digit(bits, level);
-      }
-      if (dg != run_digit) {
-        if (run_digit >= 0) atomicAdd(&sh[run_digit], run);
-        run_digit = dg; run = 0;
-      }
-      ++run;
-    }
-    if (run_digit >= 0) atomicAdd(&sh[run_digit], run);
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < kCpBins; b += blockDim.x)
-    if (sh[b]) atomicAdd(&hist[h * kCpBins + b], sh[b]);
-}
-
-// One level of the descent on the histogram summed over all ranks: the digit d with
-// count(digits > d) < need <= count(digits >= d) joins the prefix, need drops by the count above it (d = 0 if the counts
-// above it never reach need).  need == 0: the prefix becomes all ones (nothing lies above it) and stays.
-// One CTA of 256 threads per head; thread t holds the 8 digits 8t .. 8t+7 counted from the top.
-__global__ void __launch_bounds__(256)
-k_cp_descend(const int32_t* __restrict__ hist, int level, unsigned* __restrict__ prefix, int32_t* __restrict__ need) {
   __shared__ long long wtot[8];
-  __shared__ int sh_found;
+  __shared__ unsigned sh_prefix;
+  __shared__ int sh_need;
   pdl_launch_dependents();
-  pdl_wait();
-  const int h = blockIdx.x, t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  const int nd = need[h];
-  if (nd <= 0) {
-    if (t == 0) { prefix[h] = 0xffffffffu; need[h] = 0; }
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int n_work = a.n_kv_heads * a.ctas_per_head;
+  if ((int)blockIdx.x >= n_work) {
+    pdl_wait();
+    const long long n16 = a.clear_bytes >> 4, step = (long long)(gridDim.x - n_work) * kCpStepThreads;
+    uint4* dst = static_cast<uint4*>(a.clear);
+#pragma unroll 4
+    for (long long i = (long long)(blockIdx.x - n_work) * kCpStepThreads + t; i < n16; i += step)
+      dst[i] = make_uint4(0u, 0u, 0u, 0u);
     return;
   }
-  const int bins = level == 2 ? 1024 : kCpBins;
-  const int shift = level == 0 ? 21 : (level == 1 ? 10 : 0);
-  if (t == 0) sh_found = 0;
-  int c[8];
-  long long s = 0;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int d = bins - 1 - (8 * t + q);
-    c[q] = d >= 1 ? hist[h * kCpBins + d] : 0;           // digit 0 is where the search ends anyway
-    s += c[q];
+  const int h = blockIdx.x / a.ctas_per_head, part = blockIdx.x - h * a.ctas_per_head;
+  if (a.hist)
+    for (int b = t; b < kCpBins; b += kCpStepThreads) sh[b] = 0;
+  pdl_wait();
+
+  unsigned prefix;
+  int need;
+  if (a.budgets) {
+    const long long kept = min(a.seq_len, max((long long)a.budgets[h], (long long)a.window));
+    prefix = 0u;
+    need = (int)(kept - min(a.seq_len, (long long)a.window));
+  } else {
+    prefix = a.prefix_in[h];
+    need = a.need_in ? a.need_in[h] : 0;
   }
-  long long inc = s;
-  for (int o = 1; o < 32; o <<= 1) {
-    const long long n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  if (lane == 31) wtot[wid] = inc;
-  __syncthreads();
-  long long above = inc - s;
-  for (int w2 = 0; w2 < wid; ++w2) above += wtot[w2];
-  if (above < nd && above + s >= nd) {                   // the digit lies among this thread's eight
+  if (a.hist_sum && need <= 0) {
+    prefix = 0xffffffffu;
+    need = 0;
+  } else if (a.hist_sum) {
+    const int from = a.level_in, bins = from == 2 ? 1024 : kCpBins;
+    const int shift = from == 0 ? 21 : (from == 1 ? 10 : 0);
+    // thread t holds the 8 digits from bins - 1 - 8 t downwards; digit 0 is where the search ends anyway
+    int c[8];
+    long long s = 0;
+    const int top = bins - 1 - 8 * t;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      if (above + c[q] >= nd) {
-        prefix[h] |= (unsigned)(bins - 1 - (8 * t + q)) << shift;
-        need[h] = (int32_t)(nd - above);
-        sh_found = 1;
-        break;
+      c[q] = top - q >= 1 ? a.hist_sum[h * kCpBins + top - q] : 0;
+      s += c[q];
+    }
+    long long inc = s;
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long n = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += n;
+    }
+    if (lane == 31) wtot[wid] = inc;
+    __syncthreads();
+    long long above = inc - s, total = 0;
+    for (int w2 = 0; w2 < 8; ++w2) {
+      if (w2 < wid) above += wtot[w2];
+      total += wtot[w2];
+    }
+    if (t == 0 && total < need) {                        // the counts above digit 0 do not reach need: digit 0
+      sh_prefix = prefix;
+      sh_need = (int)(need - total);
+    }
+    if (above < need && above + s >= need) {             // the digit lies among this thread's eight
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (above + c[q] >= need) {
+          sh_prefix = prefix | (unsigned)(top - q) << shift;
+          sh_need = (int)(need - above);
+          break;
+        }
+        above += c[q];
       }
-      above += c[q];
+    }
+    __syncthreads();
+    prefix = sh_prefix;
+    need = sh_need;
+  }
+  if (part == 0 && t == 0 && a.prefix_out) {             // in place only with one CTA per head
+    a.prefix_out[h] = prefix;
+    a.need_out[h] = need;
+  }
+  if (!a.hist && !a.cnt_gt) return;
+
+  __syncthreads();                                       // sh cleared
+  const unsigned* row = reinterpret_cast<const unsigned*>(a.pooled + (long long)h * a.row_stride + a.own_begin);
+  const int level = a.level_out;
+  for (int blk = part; blk < a.n_blk; blk += a.ctas_per_head) {
+    const long long j0 = (long long)blk * kCpSlice + t * 16;
+    unsigned bits[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) bits[q] = j0 + q < a.own_count ? row[j0 + q] : 0u;
+    if (a.hist) {
+      int run_digit = -1, run = 0;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int dg = j0 + q < a.own_count && cp_match(bits[q], prefix, level) ? (int)cp_digit(bits[q], level) : -1;
+        if (dg != run_digit) {
+          if (run_digit >= 0) atomicAdd(&sh[run_digit], run);
+          run_digit = dg; run = 0;
+        }
+        ++run;
+      }
+      if (run_digit >= 0) atomicAdd(&sh[run_digit], run);
+    } else {
+      unsigned n = 0;                                    // equal ones in the high half, those above in the low half
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        if (j0 + q < a.own_count) n += (bits[q] > prefix ? 1u : 0u) + (bits[q] == prefix ? 65536u : 0u);
+      n = __reduce_add_sync(0xffffffffu, n);
+      __syncthreads();
+      if (lane == 0) sh[wid] = (int)n;
+      __syncthreads();
+      if (t == 0) {
+        unsigned all = 0;
+        for (int w2 = 0; w2 < 8; ++w2) all += (unsigned)sh[w2];
+        const int gt = (int)(all & 65535u), eq = (int)(all >> 16);
+        a.cnt_gt[h * a.n_blk + blk] = gt;
+        a.cnt_eq[h * a.n_blk + blk] = eq;
+        if (gt) atomicAdd(&a.tot_gt[h], gt);
+        if (eq) atomicAdd(&a.tot_eq[h], eq);
+      }
     }
   }
+  if (!a.hist) return;
   __syncthreads();
-  if (t == 0 && !sh_found) {                             // the counts above digit 0 do not reach need: digit 0
-    long long total = 0;
-    for (int w2 = 0; w2 < 8; ++w2) total += wtot[w2];
-    need[h] = (int32_t)(nd - total);
-  }
+  for (int b = t; b < kCpBins; b += kCpStepThreads)
+    if (sh[b]) atomicAdd(&a.hist[h * kCpBins + b], sh[b]);
 }
 
 // ties[h] = this rank's positions whose score equals the threshold = its last-level histogram at the threshold's digit.
@@ -153,106 +192,57 @@ __global__ void k_cp_local_ties(const int32_t* __restrict__ hist_local, const un
   ties[h] = prefix[h] == 0xffffffffu ? 0 : hist_local[h * kCpBins + (prefix[h] & 1023u)];
 }
 
-__device__ __forceinline__ int cp_block_sum(int v, int* red) {
-  __syncthreads();
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  int t = 0;
-  for (int w = 0; w < kCpThreads / 32; ++w) t += red[w];
-  return t;
-}
-
-constexpr int kCpSlice = kCpThreads * kCpItems;       // positions per CTA of k_cp_count / k_cp_emit
-
-// cnt_gt / cnt_eq[h][blk] = positions of slice blk of head h's owned range above / at the threshold.
-__global__ void __launch_bounds__(kCpThreads)
-k_cp_count(const float* __restrict__ pooled, long long row_stride, int own_begin, int own_count,
-           const unsigned* __restrict__ threshold, int n_blk, int32_t* __restrict__ cnt_gt, int32_t* __restrict__ cnt_eq) {
-  __shared__ int red[kCpThreads / 32];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int h = blockIdx.y, blk = blockIdx.x;
-  const unsigned tau = threshold[h];
-  const unsigned* row = reinterpret_cast<const unsigned*>(pooled + (long long)h * row_stride + own_begin);
-  const long long first = (long long)blk * kCpSlice + threadIdx.x * kCpItems;
-  int gt = 0, eq = 0;
-#pragma unroll
-  for (int q = 0; q < kCpItems; ++q)
-    if (first + q < own_count) {
-      const unsigned bits = row[first + q];
-      gt += bits > tau;
-      eq += bits == tau;
-    }
-  gt = cp_block_sum(gt, red);
-  eq = cp_block_sum(eq, red);
-  if (threadIdx.x == 0) { cnt_gt[h * n_blk + blk] = gt; cnt_eq[h * n_blk + blk] = eq; }
-}
-
-// Per head (one thread each): take[h] = its share of the ties = need[h] less the ties of the ranks before this one,
-// within [0, own ties]; rows[h] = scores above the threshold + take + window rows; the counts become exclusive prefixes
-// over the slices.  Then offsets = exclusive prefix of rows[] (thread 0).
-__global__ void k_cp_plan(const int32_t* __restrict__ need, const int32_t* __restrict__ ties_all, int n_kv_heads, int part,
-                          int window_rows, int n_blk, int32_t* __restrict__ cnt_gt, int32_t* __restrict__ cnt_eq,
-                          int32_t* __restrict__ rows, int32_t* __restrict__ take, long long capacity,
-                          int32_t* __restrict__ offsets, int32_t* __restrict__ status) {
-  pdl_launch_dependents();
-  pdl_wait();
-  for (int h = threadIdx.x; h < n_kv_heads; h += blockDim.x) {
-    int gt = 0, eq = 0;
-    for (int b = 0; b < n_blk; ++b) {
-      const int g = cnt_gt[h * n_blk + b], e = cnt_eq[h * n_blk + b];
-      cnt_gt[h * n_blk + b] = gt; cnt_eq[h * n_blk + b] = eq;
-      gt += g; eq += e;
-    }
-    long long before = 0;
-    for (int r = 0; r < part; ++r) before += ties_all[r * n_kv_heads + h];
-    long long t = (long long)need[h] - before;
-    t = t < 0 ? 0 : (t > eq ? eq : t);
-    take[h] = (int32_t)t;
-    rows[h] = gt + (int32_t)t + window_rows;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long o = 0;
-    for (int h = 0; h < n_kv_heads; ++h) { offsets[h] = (int32_t)o; o += rows[h]; }
-    offsets[n_kv_heads] = (int32_t)o;
-    if (o > capacity && status) atomicCAS(status, 0, (int)SLKV_ERR_CAPACITY);
-  }
-}
-
 // Packs slice blk of head h's kept positions in ascending order: kept_idx = position in the whole sequence,
 // gather_src = row of this rank's K / V (token * n_kv_heads + head); slice 0 also writes the window rows on the rank
-// that holds them.  A kept position's packed row = offsets[h] + (scores above the threshold before it) +
-// min(ties before it, take).
-__global__ void __launch_bounds__(kCpThreads)
-k_cp_emit(const float* __restrict__ pooled, long long row_stride, int own_begin, int own_count, long long pos0,
-          const unsigned* __restrict__ threshold, const int32_t* __restrict__ rows, const int32_t* __restrict__ take,
-          const int32_t* __restrict__ cnt_gt, const int32_t* __restrict__ cnt_eq, int n_blk, int n_kv_heads,
-          int window_rows, long long window_row0, long long window_pos0, long long capacity,
-          const int32_t* __restrict__ offsets, int32_t* __restrict__ kept_idx, int32_t* __restrict__ gather_src) {
+// that holds them, and the head's offset.  A head takes of its ties what the ranks before this one have left of need,
+// within [0, own ties]; its rows = scores above the threshold + ties taken + window rows.  A kept position's packed row
+// = the rows of the heads before + (scores above the threshold before it) + min(ties before it, ties taken).
+// Every CTA adds up the heads' rows and its own head's slices by itself: a few hundred counters from L2 instead of a
+// launch between the counting and the packing (5 us in a single CTA).
+__global__ void __launch_bounds__(kCpThreads) k_cp_emit(const __grid_constant__ CpEmit a) {
   __shared__ unsigned wtot[kCpThreads / 32];
+  __shared__ int red[kCpThreads / 32][4];
   pdl_launch_dependents();
   pdl_wait();
   const int h = blockIdx.y, blk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const long long out0 = offsets[h];
-  const unsigned tau = threshold[h];
-  const int tk = take[h];
-  const unsigned* row = reinterpret_cast<const unsigned*>(pooled + (long long)h * row_stride + own_begin);
+  auto take_of = [&](int g) {
+    long long t = a.need[g];
+    for (int r = 0; r < a.part; ++r) t -= a.ties_all[(long long)r * a.n_kv_heads + g];
+    const int own = a.tot_eq[g];
+    return t < 0 ? 0 : (t > own ? own : (int)t);
+  };
+  const unsigned tau = a.threshold[h];
+  const int tk = take_of(h), rows_h = a.tot_gt[h] + tk + a.window_rows;
+  const unsigned* row = reinterpret_cast<const unsigned*>(a.pooled + (long long)h * a.row_stride + a.own_begin);
   const long long first = (long long)blk * kCpSlice + tid * kCpItems;
   unsigned bits[kCpItems];
   unsigned packed = 0;                           // ties in the high half, scores above the threshold in the low half
 #pragma unroll
   for (int q = 0; q < kCpItems; ++q) {
-    bits[q] = first + q < own_count ? row[first + q] : 0u;
-    if (first + q < own_count) packed += (bits[q] > tau ? 1u : 0u) + (bits[q] == tau ? 65536u : 0u);
+    bits[q] = first + q < a.own_count ? row[first + q] : 0u;
+    if (first + q < a.own_count) packed += (bits[q] > tau ? 1u : 0u) + (bits[q] == tau ? 65536u : 0u);
   }
+  int before = 0, all = 0, gt0 = 0, eq0 = 0;     // rows of the heads before h, of all; the head's counts before the slice
+  for (int g = tid; g < a.n_kv_heads; g += kCpThreads) {
+    const int r = a.tot_gt[g] + take_of(g) + a.window_rows;
+    all += r;
+    if (g < h) before += r;
+  }
+  for (int b = tid; b < blk; b += kCpThreads) {
+    gt0 += a.cnt_gt[h * a.n_blk + b];
+    eq0 += a.cnt_eq[h * a.n_blk + b];
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  all = __reduce_add_sync(0xffffffffu, all);
+  gt0 = __reduce_add_sync(0xffffffffu, gt0);
+  eq0 = __reduce_add_sync(0xffffffffu, eq0);
   unsigned inc = packed;
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned n = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += n;
   }
   if (lane == 31) wtot[wid] = inc;
+  if (lane == 0) { red[wid][0] = before; red[wid][1] = all; red[wid][2] = gt0; red[wid][3] = eq0; }
   __syncthreads();
   if (wid == 0) {
     unsigned w = wtot[lane], winc = w;
@@ -261,19 +251,23 @@ k_cp_emit(const float* __restrict__ pooled, long long row_stride, int own_begin,
       if (lane >= o) winc += n;
     }
     wtot[lane] = winc - w;                       // exclusive over the warps
+  } else if (wid <= 4) {
+    const int v = __reduce_add_sync(0xffffffffu, red[lane][wid - 1]);
+    if (lane == 0) red[0][wid - 1] = v;          // the only warp that reads or writes this column
   }
   __syncthreads();
+  const long long out0 = red[0][0], total = red[0][1];
   const unsigned excl = wtot[wid] + inc - packed;
-  unsigned gb = (unsigned)cnt_gt[h * n_blk + blk] + (excl & 65535u), eb = (unsigned)cnt_eq[h * n_blk + blk] + (excl >> 16);
+  unsigned gb = (unsigned)red[0][2] + (excl & 65535u), eb = (unsigned)red[0][3] + (excl >> 16);
 #pragma unroll
   for (int q = 0; q < kCpItems; ++q) {
-    if (first + q >= own_count) break;
+    if (first + q >= a.own_count) break;
     const bool gt = bits[q] > tau, eq = bits[q] == tau;
     if (gt || (eq && (int)eb < tk)) {
       const long long o = out0 + gb + min(eb, (unsigned)tk);
-      if (o < capacity) {
-        kept_idx[o] = (int32_t)(pos0 + first + q);
-        gather_src[o] = (int32_t)((own_begin + first + q) * n_kv_heads + h);
+      if (o < a.capacity) {
+        a.kept_idx[o] = (int32_t)(a.pos0 + first + q);
+        a.gather_src[o] = (int32_t)((a.own_begin + first + q) * a.n_kv_heads + h);
       }
     }
     gb += gt;
@@ -281,13 +275,24 @@ k_cp_emit(const float* __restrict__ pooled, long long row_stride, int own_begin,
   }
   // window rows (Algorithm 3 l.4, l.10): always kept, behind the history rows, on the rank that holds them
   if (blk == 0) {
-    const long long w0 = out0 + rows[h] - window_rows;
-    for (int i = tid; i < window_rows; i += kCpThreads)
-      if (w0 + i < capacity) {
-        kept_idx[w0 + i] = (int32_t)(window_pos0 + i);
-        gather_src[w0 + i] = (int32_t)((window_row0 + i) * n_kv_heads + h);
+    const long long w0 = out0 + rows_h - a.window_rows;
+    for (int i = tid; i < a.window_rows; i += kCpThreads)
+      if (w0 + i < a.capacity) {
+        a.kept_idx[w0 + i] = (int32_t)(a.window_pos0 + i);
+        a.gather_src[w0 + i] = (int32_t)((a.window_row0 + i) * a.n_kv_heads + h);
       }
+    if (tid == 0) {
+      a.offsets[h] = (int32_t)out0;
+      if (h == 0) {
+        a.offsets[a.n_kv_heads] = (int32_t)total;
+        if (total > a.capacity && a.status) atomicCAS(a.status, 0, (int)SLKV_ERR_CAPACITY);
+      }
+    }
   }
+  if (a.fill_tail)                               // positions of the rows nobody fills: -1
+    for (long long o = total + ((long long)h * gridDim.x + blk) * kCpThreads + tid; o < a.capacity;
+         o += (long long)gridDim.x * gridDim.y * kCpThreads)
+      a.kept_idx[o] = -1;
 }
 
 }  // namespace
@@ -298,28 +303,16 @@ cudaError_t launch_cp_merge_lse(const float* parts, int n_parts, long long n, fl
   return launch_pdl(k_cp_merge_lse, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, parts, n_parts, n, to_log2, out);
 }
 
-cudaError_t launch_cp_need_init(const int32_t* budgets, int n_kv_heads, int window, long long seq_len, unsigned* prefix,
-                                int32_t* need, cudaStream_t st, int* launches) {
+cudaError_t launch_cp_step(CpStep a, cudaStream_t st, int* launches) {
+  a.n_blk = cp_slices(a.own_count);
+  // up to 64 CTAs per head to count: they repeat the start, and each adds its bins to the head's
+  a.ctas_per_head = a.hist || a.cnt_gt ? (a.hist && a.n_blk > 64 ? 64 : a.n_blk) : 1;
+  if (a.clear_bytes <= 0) a.clear_bytes = 0;
+  const long long want = (a.clear_bytes + kCpStepThreads * 64 - 1) / (kCpStepThreads * 64);     // 4 stores per thread
+  const int most = sm_count() * 4;                       // with the counting CTAs resident at once
+  const unsigned n_clear = (unsigned)(want < most ? want : most);
   LaunchScope scope(KID_CP, st, launches);
-  return launch_pdl(k_cp_need_init, dim3((n_kv_heads + 127) / 128), dim3(128), 0, st, 1, budgets, n_kv_heads, window,
-                    seq_len, prefix, need);
-}
-
-cudaError_t launch_cp_histogram(const float* pooled, int n_kv_heads, long long row_stride, int own_begin, int own_count,
-                                int level, const unsigned* prefix, int32_t* hist, cudaStream_t st, int* launches) {
-  cudaError_t e = cudaMemsetAsync(hist, 0, (size_t)n_kv_heads * kCpBins * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  int bx = (own_count + 256 * 16 - 1) / (256 * 16);
-  bx = bx < 1 ? 1 : (bx > 64 ? 64 : bx);
-  LaunchScope scope(KID_CP, st, launches);
-  return launch_pdl(k_cp_histogram, dim3(bx, n_kv_heads), dim3(256), 0, st, 1, pooled, row_stride, own_begin, own_count,
-                    level, prefix, hist);
-}
-
-cudaError_t launch_cp_descend(const int32_t* hist, int n_kv_heads, int level, unsigned* prefix, int32_t* need,
-                              cudaStream_t st, int* launches) {
-  LaunchScope scope(KID_CP, st, launches);
-  return launch_pdl(k_cp_descend, dim3(n_kv_heads), dim3(256), 0, st, 1, hist, level, prefix, need);
+  return launch_pdl(k_cp_step, dim3((unsigned)a.n_kv_heads * a.ctas_per_head + n_clear), dim3(kCpStepThreads), 0, st, 1, a);
 }
 
 cudaError_t launch_cp_local_ties(const int32_t* hist_local, const unsigned* prefix, int n_kv_heads, int32_t* ties,
@@ -331,29 +324,10 @@ cudaError_t launch_cp_local_ties(const int32_t* hist_local, const unsigned* pref
 
 int cp_slices(int own_count) { return own_count > 0 ? (own_count + kCpSlice - 1) / kCpSlice : 1; }
 
-cudaError_t launch_cp_emit(const float* pooled, long long row_stride, int own_begin, int own_count, long long pos0,
-                           const unsigned* threshold, const int32_t* need, const int32_t* ties_all, int n_kv_heads,
-                           int part, int window_rows, long long window_row0, long long window_pos0, long long capacity,
-                           int32_t* offsets, int32_t* kept_idx, int32_t* gather_src, int32_t* rows, int32_t* take,
-                           int32_t* cnt_gt, int32_t* cnt_eq, int32_t* status, cudaStream_t st, int* launches) {
-  const int n_blk = cp_slices(own_count);
-  {
-    LaunchScope scope(KID_CP, st, launches);
-    cudaError_t e = launch_pdl(k_cp_count, dim3(n_blk, n_kv_heads), dim3(kCpThreads), 0, st, 1, pooled, row_stride,
-                               own_begin, own_count, threshold, n_blk, cnt_gt, cnt_eq);
-    if (e != cudaSuccess) return e;
-  }
-  {
-    LaunchScope scope(KID_CP, st, launches);
-    cudaError_t e = launch_pdl(k_cp_plan, dim3(1), dim3(256), 0, st, 1, need, ties_all, n_kv_heads, part, window_rows,
-                               n_blk, cnt_gt, cnt_eq, rows, take, capacity, offsets, status);
-    if (e != cudaSuccess) return e;
-  }
+cudaError_t launch_cp_emit(CpEmit a, cudaStream_t st, int* launches) {
+  a.n_blk = cp_slices(a.own_count);
   LaunchScope scope(KID_CP, st, launches);
-  return launch_pdl(k_cp_emit, dim3(n_blk, n_kv_heads), dim3(kCpThreads), 0, st, 1, pooled, row_stride, own_begin,
-                    own_count, pos0, threshold, (const int32_t*)rows, (const int32_t*)take, (const int32_t*)cnt_gt,
-                    (const int32_t*)cnt_eq, n_blk, n_kv_heads, window_rows, window_row0, window_pos0, capacity,
-                    (const int32_t*)offsets, kept_idx, gather_src);
+  return launch_pdl(k_cp_emit, dim3(a.n_blk, a.n_kv_heads), dim3(kCpThreads), 0, st, 1, a);
 }
 
 }  // namespace slkv

@@ -148,20 +148,37 @@ cudaError_t launch_behavior(const float* attn, long long row_stride, int row_len
 // context-parallel selection (slkv_cp.cu)
 cudaError_t launch_cp_merge_lse(const float* parts, int n_parts, long long n, float to_log2, float* out,
                                 cudaStream_t st, int* launches);
-cudaError_t launch_cp_need_init(const int32_t* budgets, int n_kv_heads, int window, long long seq_len, unsigned* prefix,
-                                int32_t* need, cudaStream_t st, int* launches);
-cudaError_t launch_cp_histogram(const float* pooled, int n_kv_heads, long long row_stride, int own_begin, int own_count,
-                                int level, const unsigned* prefix, int32_t* hist, cudaStream_t st, int* launches);
-cudaError_t launch_cp_descend(const int32_t* hist, int n_kv_heads, int level, unsigned* prefix, int32_t* need,
-                              cudaStream_t st, int* launches);
+constexpr int kCpBins = 2048;           // of a head's histogram
+struct CpStep {                          // one launch of k_cp_step; see there
+  const int32_t* budgets;                // not null: start from them
+  const unsigned* prefix_in;             // else from this state,
+  const int32_t* need_in;
+  const int32_t* hist_sum;               // not null: taken down level level_in
+  unsigned* prefix_out;                  // may be null
+  int32_t* need_out;
+  const float* pooled;
+  int32_t* hist;                         // not null: histogram of level level_out added here
+  int32_t *cnt_gt, *cnt_eq, *tot_gt, *tot_eq;   // not null: slices counted against the complete prefix
+  void* clear;                           // 16-byte aligned; clear_bytes a multiple of 16
+  long long seq_len, row_stride, clear_bytes;
+  int n_kv_heads, window, level_in, level_out, own_begin, own_count;
+  int n_blk, ctas_per_head;              // set by launch_cp_step
+};
+cudaError_t launch_cp_step(CpStep a, cudaStream_t st, int* launches);
 cudaError_t launch_cp_local_ties(const int32_t* hist_local, const unsigned* prefix, int n_kv_heads, int32_t* ties,
                                  cudaStream_t st, int* launches);
-cudaError_t launch_cp_emit(const float* pooled, long long row_stride, int own_begin, int own_count, long long pos0,
-                           const unsigned* threshold, const int32_t* need, const int32_t* ties_all, int n_kv_heads,
-                           int part, int window_rows, long long window_row0, long long window_pos0, long long capacity,
-                           int32_t* offsets, int32_t* kept_idx, int32_t* gather_src, int32_t* rows, int32_t* take,
-                           int32_t* cnt_gt, int32_t* cnt_eq, int32_t* status, cudaStream_t st, int* launches);
-int cp_slices(int own_count);            // CTAs per head of the counting and packing kernels
+struct CpEmit {                          // one launch of k_cp_emit; see there
+  const float* pooled;
+  const unsigned* threshold;
+  const int32_t *need, *ties_all, *cnt_gt, *cnt_eq, *tot_gt, *tot_eq;
+  int32_t *offsets, *kept_idx, *gather_src, *status;
+  long long row_stride, pos0, window_row0, window_pos0, capacity;
+  int n_kv_heads, part, window_rows, own_begin, own_count;
+  int fill_tail;                         // 1: kept_idx of the rows behind the last one is set to -1
+  int n_blk;                             // set by launch_cp_emit
+};
+cudaError_t launch_cp_emit(CpEmit a, cudaStream_t st, int* launches);
+int cp_slices(int own_count);            // slices of the owned range that are counted and packed together
 cudaError_t launch_setup(const Problem& pb, const int32_t* budgets, int32_t* offsets, int64_t capacity,
                          int32_t* status, cudaStream_t st, int* launches);
 size_t simt_part_bytes(const Problem& pb);

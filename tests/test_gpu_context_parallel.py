@@ -208,6 +208,26 @@ def test_selection_is_exact_on_given_scores_with_many_ties(seed):
         assert np.array_equal(np.concatenate(kept[h]), want), (h, world, n_hist)
 
 
+@pytest.mark.parametrize("n_hist,world", [(0, 1), (1, 1), (4095, 1), (4096, 1), (4097, 1), (2 * 4096 + 3, 2),
+                                          (65 * 4096 + 17, 1)])
+def test_edges_of_the_counted_slices_and_rows_nothing_is_packed_into(n_hist, world):
+    # slices of 4096 positions, above 64 of them several per CTA of the histograms; the output rows behind the packed ones
+    Hq, Hkv, w, p, d = 4, 2, 16, 5, 64
+    L = n_hist + w
+    q, k, v = rand_seq(Hq, Hkv, w, L, seed=n_hist, d=d)
+    bud = [w + n_hist // 3, w + 1]
+    ref = P.oracle_pooled(q, k, [0, L], w, p)
+    outs = run_ranks(world, q, k, v, bud, w, p)
+    for o in outs:
+        n = int(o["offsets"][-1])
+        assert int(o["status"].item()) == 0 and o["kept_idx"].numel() == max(o["capacity"], 1)
+        assert bool((o["kept_idx"][n:] == -1).all()) and bool((o["kept_idx"][:n] >= 0).all())
+        assert not bool(o["k_out"][n:].any()) and not bool(o["v_out"][n:].any())
+    gpu = as_one_layer(outs, world, L, w, p, Hkv)
+    P.assert_pooled_close(gpu["pooled"], ref, [0, L], Hkv, w)
+    P.assert_selection_valid(gpu, ref, [0, L], bud, w, k, v)
+
+
 @pytest.mark.parametrize("path,dtype,d,w,Hq,Hkv", [(B.SLKV_PATH_TENSOR, torch.bfloat16, 128, 32, 8, 2),
                                                    (B.SLKV_PATH_SIMT, torch.float32, 64, 16, 8, 8)])
 def test_history_only_rows_score_as_the_history_of_a_longer_sequence(path, dtype, d, w, Hq, Hkv):
