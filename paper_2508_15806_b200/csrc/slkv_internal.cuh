@@ -236,7 +236,7 @@ struct ScoreShape {
   int n_seqs, n_kv_heads, G, window;
   int R, Rp, MT;                // score rows per KV head: G * window; rounded up to 32; 128-row blocks of them
   int halves;                   // 64-element halves of a key row (head_dim / 64)
-  int n_q, n_stages, slot_stride;   // Q tiles in shared memory, K tiles in flight; split ranges that may share a segment (stride of the statistics)
+  int n_stages, slot_stride;        // K tiles in flight; split ranges that may share a segment (stride of the statistics)
   int q_head_inner, k_head_inner;   // tensor-map dimension order: 1 = the head axis comes before the row axis
   int total_tiles, n_cta;       // of one layer; CTAs
   // The groups the tiles of a list are walked in: group_layers = 0: a layer's n_groups groups, group_tile their first
@@ -263,7 +263,7 @@ struct ScorePlan {
 cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, ScorePlan* plan);
 cudaError_t plan_score_layer(const Problem& pb, int32_t* status, ScoreLayer* lay);    // the layer's part alone
 int sm_count();
-int score_list_stages(int MT, int halves, int n_q);
+int score_list_stages(int MT, int halves);
 // The score kernel over a list of layers of one shape: passes 1 = row statistics, 2 = votes from the callers' row
 // statistics, 3 = both.
 cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes, cudaStream_t st,

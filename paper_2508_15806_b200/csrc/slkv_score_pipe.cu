@@ -13,7 +13,7 @@
 // still in L2.
 //
 // Roles (640 threads, one CTA per SM; a twenty-first warp would cost every thread 16 registers):
-//   warp 0     TMA loads of K tiles (ring of 4-6 x 32 KB) and Q tiles; it never waits for Q while K stages are free
+//   warp 0     TMA loads of K tiles (ring of 2-4 x 32 KB, or more of 16 KB) and Q tiles; it never waits for Q while K stages are free
 //   warp 1     tcgen05.mma, 128 x 128 products into four 128-column TMEM accumulators ("units")
 //   warp 2     works out the runs (consecutive tiles of one segment) and hands them to the others through shared memory;
 //              announces a group's statistics to the other CTAs once this CTA's share is out
@@ -56,6 +56,10 @@ constexpr int kBarBytes = 640;
 constexpr int kStatBytes = 2 * kWgs * 128 * 8;
 constexpr int kLseBytes = 2 * 256 * 4;
 constexpr int kHalfVoteBytes = 2 * 4 * 128 * 4;
+// Two Q tiles, also where that leaves the ring no more than two K tiles (R > 128, d = 128): the next run's queries are
+// there when its keys are.  One Q tile and four K tiles cost a pause of 1.6 us in every run of about 25: 128k positions
+// 5935 -> 5810 us, eight sequences of 4k - 32k 6830 -> 6690 us (32 layers each).
+constexpr int kQTiles = 2;
 constexpr int kRunSlots = 8;                         // runs handed out ahead
 constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes + kRunSlots * 128;
 // Exponentials on the FMA pipe: pairs 0 .. kPolyPairs-1 of every eight.
@@ -104,7 +108,7 @@ static_assert(sizeof(RunDesc) <= 128, "run descriptor");
 // What the roles keep in registers: copied through shared memory, so that no launch parameter is read in a loop.
 struct Smem {
   uint32_t q, k, bar0, tmem;
-  int q_half, q_bytes, n_q, stage_bytes, n_stages;
+  int q_half, q_bytes, stage_bytes, n_stages;
   int R, Rp, MT, halves, k_head_inner, both;
   float sc, inv_g;
   volatile int* abort_flag;
@@ -119,9 +123,9 @@ struct Smem {
   __device__ __forceinline__ uint32_t empty(int st) const { return bar(kMaxStages + st); }
   __device__ __forceinline__ uint32_t unit_full(int u) const { return bar(2 * kMaxStages + u); }
   __device__ __forceinline__ uint32_t unit_empty(int u) const { return bar(2 * kMaxStages + 4 + u); }
-  // run k's Q tile: slot and phase (n_q is 1 or 2)
-  __device__ __forceinline__ int q_slot(int k) const { return k & (n_q - 1); }
-  __device__ __forceinline__ uint32_t q_phase(int k) const { return (uint32_t)(k >> (n_q - 1)) & 1u; }
+  // run k's Q tile: slot and phase
+  __device__ __forceinline__ int q_slot(int k) const { return k & (kQTiles - 1); }
+  __device__ __forceinline__ uint32_t q_phase(int k) const { return (uint32_t)(k / kQTiles) & 1u; }
   __device__ __forceinline__ uint32_t q_full(int k) const { return bar(2 * kMaxStages + 8 + q_slot(k)); }
   __device__ __forceinline__ uint32_t q_empty(int k) const { return bar(2 * kMaxStages + 10 + q_slot(k)); }
   __device__ __forceinline__ uint32_t stat_full(int s) const { return bar(2 * kMaxStages + 12 + s); }
@@ -308,8 +312,8 @@ __device__ __forceinline__ void producer(const Smem& c) {
       if (it == 0 || last < 0) continue;
       while (!mbar_try(c.full(s2), (last / c.n_stages) & 1) && now_ns() - t0 < kWaitLimitNs) {}
     }
-    const int loaded = n - (q_due ? 1 : 0);                  // Q tiles asked for; the last n_q may be in flight
-    for (int k = loaded - c.n_q < 0 ? 0 : loaded - c.n_q; k < loaded; ++k)
+    const int loaded = n - (q_due ? 1 : 0);                  // Q tiles asked for; the last kQTiles may be in flight
+    for (int k = loaded - kQTiles < 0 ? 0 : loaded - kQTiles; k < loaded; ++k)
       while (!mbar_try(c.q_full(k), c.q_phase(k)) && now_ns() - t0 < kWaitLimitNs) {}
   }
 }
@@ -722,7 +726,7 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
 __global__ void __launch_bounds__(kListThreads, 1)
 k_score_list(const __grid_constant__ ListArgs a) {
   // Shared memory, all dynamic and 1024-byte aligned (the swizzled tiles need it):
-  //   [n_q Q tiles: halves x MT x 16 KB][K ring: n_stages x halves x 16 KB][mbarriers, flags][statistics][log-sum-exps][half votes]
+  //   [kQTiles Q tiles: halves x MT x 16 KB][K ring: n_stages x halves x 16 KB][mbarriers, flags][statistics][log-sum-exps][half votes]
   extern __shared__ __align__(1024) unsigned char smem[];
   const ScoreShape& sh = a.sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -733,7 +737,7 @@ k_score_list(const __grid_constant__ ListArgs a) {
     return;
   }
   // the tail's place follows from launch parameters; everything the roles use in their loops goes through shared memory
-  unsigned char* tail = smem + sh.halves * (sh.n_q * sh.MT * 128 * 128 + sh.n_stages * kHalfBytes);
+  unsigned char* tail = smem + sh.halves * (kQTiles * sh.MT * 128 * 128 + sh.n_stages * kHalfBytes);
   uint32_t& tmem_base_sh = *reinterpret_cast<uint32_t*>(tail + kBarBytes - 16);
   int& abort_sh = *reinterpret_cast<int*>(tail + kBarBytes - 12);
   volatile int* head = reinterpret_cast<volatile int*>(tail + kBarBytes - 16 - kHeadInts * 4);
@@ -764,18 +768,17 @@ k_score_list(const __grid_constant__ ListArgs a) {
       mbar_init(c.lse_empty(s), 4 * kWgs);
       for (int t = 0; t < 4; ++t) mbar_init(c.half_full(s, t), 4);
     }
-    c.n_q = 2;                                                // both slots' barriers, used or not
-    for (int k = 0; k < 2; ++k) { mbar_init(c.q_full(k), 1); mbar_init(c.q_empty(k), 1); }
+    for (int k = 0; k < kQTiles; ++k) { mbar_init(c.q_full(k), 1); mbar_init(c.q_empty(k), 1); }
     for (int k = 0; k < kRunSlots; ++k) { mbar_init(c.run_full(k), 1); mbar_init(c.run_empty(k), kRunReaders); }
     head[0] = sh.R; head[1] = sh.Rp; head[2] = sh.MT; head[3] = sh.halves;
-    head[4] = sh.n_q; head[5] = sh.n_stages; head[6] = sh.k_head_inner;
+    head[5] = sh.n_stages; head[6] = sh.k_head_inner;
     head[7] = a.passes == 3; head[8] = __float_as_int(sh.scale_log2); head[9] = __float_as_int(1.0f / (float)sh.G);
     mbar_init(c.drain(), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // rows of the Q tile beyond R are never written by TMA: keep them zero
   if (sh.R != sh.MT * 128) {
-    for (int i = tid; i < sh.n_q * sh.halves * sh.MT * 128 * 128 / 16; i += kListThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < kQTiles * sh.halves * sh.MT * 128 * 128 / 16; i += kListThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
@@ -787,13 +790,13 @@ k_score_list(const __grid_constant__ ListArgs a) {
   tc_fence_after();
   c.tmem = tmem_base_sh;
   c.R = head[0]; c.Rp = head[1]; c.MT = head[2]; c.halves = head[3];
-  c.n_q = head[4]; c.n_stages = head[5]; c.k_head_inner = head[6];
+  c.n_stages = head[5]; c.k_head_inner = head[6];
   c.both = head[7]; c.sc = __int_as_float(head[8]); c.inv_g = __int_as_float(head[9]);
   c.q_half = c.MT * 128 * 128;
   c.q_bytes = c.halves * c.q_half;
   c.stage_bytes = c.halves * kHalfBytes;
   c.q = smem_u32(smem);
-  c.k = c.q + (uint32_t)(c.n_q * c.q_bytes);
+  c.k = c.q + (uint32_t)(kQTiles * c.q_bytes);
   // Everything above touched only this CTA's own resources, and so does all that follows up to the first load of a tile and
   // the clearing of the statistics area: those two roles wait for the kernels before this one, the others get their work
   // from them.  The first runs are worked out meanwhile.
@@ -877,8 +880,8 @@ unsigned long long* tensor_trace_buffer(int n_cta) {
 }
 
 // K tiles of the ring beside the Q tiles.
-int score_list_stages(int MT, int halves, int n_q) {
-  const int n = (kSmemLimit - kTail - n_q * halves * MT * 128 * 128) / (halves * kHalfBytes);
+int score_list_stages(int MT, int halves) {
+  const int n = (kSmemLimit - kTail - kQTiles * halves * MT * 128 * 128) / (halves * kHalfBytes);
   return n < kMaxStages ? n : kMaxStages;
 }
 
@@ -919,7 +922,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   const bool waits_inside = passes == 3;
   a.target = (unsigned)sh.n_cta + (waits_inside && take_expire_next_wait() ? 1u : 0u);
   a.trace = tensor_trace_buffer(sh.n_cta);
-  const size_t smem = (size_t)(sh.n_q * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + kTail);
+  const size_t smem = (size_t)(kQTiles * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + kTail);
 
   // CTAs that wait for one another must all be resident: cooperative launch, with dependent launch on top where the
   // device takes both.  Where it takes no cooperative launch, or the environment says so (tests), the two passes go out

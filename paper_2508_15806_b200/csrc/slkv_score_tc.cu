@@ -150,9 +150,7 @@ cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t
   a.Rp = (pb.R + 31) / 32 * 32;
   a.MT = (pb.R + 127) / 128;
   a.halves = p.head_dim / 64;
-  // a second Q tile where it leaves the ring four stages: the next run's queries are then there when its keys are
-  a.n_q = a.MT * a.halves <= 2 ? 2 : 1;
-  a.n_stages = score_list_stages(a.MT, a.halves, a.n_q);
+  a.n_stages = score_list_stages(a.MT, a.halves);
   a.slot_stride = tensor_slot_stride(pb);
   a.q_head_inner = tensor_q_head_inner(p) ? 1 : 0;
   a.k_head_inner = p.k_stride_head <= p.k_stride_tok;
