@@ -210,13 +210,15 @@ def slkv_alloc_budgets(inf_sc: torch.Tensor, fixed: int, total: int, budgets: Op
 def slkv_behavior_scores(attn: torch.Tensor, needle_idx: torch.Tensor, topk_idx: torch.Tensor, stream=None):
     """Algorithm 1 for a batch: attn CUDA float32 [n_rows, row_len]; needle_idx / topk_idx CUDA int32 [n_rows, n] or
     [n] (one list for all rows), entries < 0 are padding.  Returns (SF_sc, LG_sc, INF_sc), CUDA float32 [n_rows]."""
-    assert attn.is_cuda and attn.dtype == torch.float32 and attn.dim() == 2 and attn.stride(1) == 1
     n_rows, row_len = attn.shape
-    sf, lg, inf = torch.empty((3, n_rows), dtype=torch.float32, device=attn.device).unbind(0)
+    row_stride, one = attn.stride()
+    assert attn.is_cuda and attn.dtype == torch.float32 and one == 1
     for t in (needle_idx, topk_idx):
         assert t.is_cuda and t.dtype == torch.int32 and t.is_contiguous() and t.dim() in (1, 2)
-    nn, tn = needle_idx.shape[-1], topk_idx.shape[-1]
-    rc = _fn["slkv_behavior_scores"](stream, attn, n_rows, row_len, attn.stride(0), needle_idx, nn,
+    sf = torch.empty(n_rows, dtype=torch.float32, device=attn.device)      # three tensors: cheaper than views of one
+    lg, inf = torch.empty_like(sf), torch.empty_like(sf)
+    nn, tn = needle_idx.size(-1), topk_idx.size(-1)
+    rc = _fn["slkv_behavior_scores"](stream, attn, n_rows, row_len, row_stride, needle_idx, nn,
                                      nn if needle_idx.dim() == 2 else 0, topk_idx, tn, tn if topk_idx.dim() == 2 else 0,
                                      sf, lg, inf)
     if rc != SLKV_OK:

@@ -81,3 +81,15 @@ def test_printed_table_values():
     got = gpu_rows(torch.tensor(W, dtype=torch.float32), torch.tensor([0, 1], dtype=torch.int32), torch.tensor([0, 2], dtype=torch.int32))
     for r, h in enumerate(heads):
         assert abs(got[r, 0] - sf[h]) < 1e-6 and abs(got[r, 2] - inf[h]) < 1e-6
+
+
+@pytest.mark.parametrize("n_needle,top_k", [(1, 3), (32, 31), (33, 32), (5, 64), (65, 64), (128, 100), (30, 129)])
+def test_list_lengths_at_the_edges_of_a_warp_and_its_registers(n_needle, top_k):
+    rng = np.random.default_rng(n_needle * 1000 + top_k)
+    n_rows, row_len = 37, 300
+    attn = torch.from_numpy(rng.random((n_rows, row_len)).astype(np.float32))
+    # few distinct positions, some outside the row: repeats in both lists and across lanes' entries
+    draw = lambda n: torch.from_numpy(rng.integers(-3, row_len // 4 if n < 100 else row_len + 3, (n_rows, n)).astype(np.int32))
+    needle, topk = draw(n_needle), draw(top_k)
+    got, ref = gpu_rows(attn, needle, topk), oracle_rows(attn.numpy(), needle.numpy(), topk.numpy())
+    assert np.all(np.abs(got - ref) <= TOL * (1.0 + np.abs(ref)))
