@@ -476,8 +476,16 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     // this CTA's part of the layers' statistics areas is cleared; nobody adds to them before all parts are
     const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);
     const int w0 = split_begin(blockIdx.x, words, gridDim.x), w1 = split_begin(blockIdx.x + 1, words, gridDim.x);
-    for (int l = 0; l < a.n_layers; ++l)
-      for (int i = w0 + lane; i < w1; i += 32) __stcg(static_cast<unsigned*>(a.lay[l].part) + i, 0u);
+    // The areas' addresses in one load, a lane each, through the generic address of the parameters: read one by one from
+    // the constant bank, where each is a miss, they took 15 us for 32 layers, and every CTA's first sums waited for that.
+    static_assert(kListMaxLayers <= 32, "a lane per layer");
+    const ListArgs* args;
+    asm volatile("mov.u64 %0, %1;" : "=l"(args) : "l"(&a));
+    const unsigned long long part = lane < a.n_layers ? reinterpret_cast<unsigned long long>(args->lay[lane].part) : 0ull;
+    for (int l = 0; l < a.n_layers; ++l) {
+      unsigned* p = reinterpret_cast<unsigned*>(__shfl_sync(0xffffffffu, part, l));
+      for (int i = w0 + lane; i < w1; i += 32) __stcg(p + i, 0u);
+    }
     __syncwarp();
     if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + a.n_groups) : "memory");
     if (!wait_count(a.counters + a.n_groups, gridDim.x)) return;
