@@ -24,16 +24,16 @@
 // (the parameters of a list are kilobytes) took 3600 cycles per run and 1000 per tile of the MMA thread.
 //
 // What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
-//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; two in eight go to the FMA pipe
-//     as packed pairs, and scale / subtract / sum run on pairs too: 1180 -> 1000-1030 (three in eight: 1046);
+//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in sixteen goes to the FMA
+//     pipe, and scale / subtract / sum run on packed pairs;
 //   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
 //     730 measured for loads and MMAs alone;
 //   - two epilogue warpgroups instead of four: 1250; sums over the keys across lanes instead of a lane per row: 1255;
 //   - power: held for more than some milliseconds the part runs at its 1 kW limit, with every tile from HBM at 1.05 GHz
 //     (0.98 us per tile, MMAs alone 0.78), with tiles from L2 at 1.5 GHz (0.68 us).  Hence the groups.
-// Against the kernel before it (two streams with two accumulators and two warpgroups each on 128 SMs for up to 128 rows,
-// one launch per layer with a grid-wide barrier for more), per layer: 32k tokens, 128 rows: 29.3 -> 24 us; eight ragged
-// sequences of 147k tokens, 256 rows: 299 -> 184 us; 131k tokens, 256 rows: 248 -> 160 us.
+// Against the kernels before it (two streams with two accumulators and two warpgroups each on 128 SMs for up to 128 rows,
+// one launch per layer with a grid-wide barrier for more), a step of 32 layers, held: 32k tokens, 128 rows: 1120 -> 862 us;
+// eight ragged sequences of 147k tokens, 256 rows: 9890 -> 6690 us; 131k tokens, 256 rows: 9210 -> 5810 us.
 // Every wait is bounded (1 s): SLKV_ERR_DEVICE_TIMEOUT in the status words, TMEM freed, return.
 #include <cuda.h>
 
@@ -62,8 +62,6 @@ constexpr int kHalfVoteBytes = 2 * 4 * 128 * 4;
 constexpr int kQTiles = 2;
 constexpr int kRunSlots = 8;                         // runs handed out ahead
 constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes + kRunSlots * 128;
-// Exponentials on the FMA pipe: pairs 0 .. kPolyPairs-1 of every eight.
-constexpr int kPolyPairs = 2;
 constexpr int kCountSlots = 32;                      // launches whose counters are live at once
 constexpr int kCountWords = kListMaxLayers * kListMaxGroups + 2;
 
@@ -544,8 +542,12 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
 }
 
 // ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
-// sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators
-template <bool STATS>
+// sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials go
+// to the FMA pipe; every other chunk does that, one exponential in sixteen.  The special-function unit alone would take one
+// in eight or four (32 layers, none / one in sixteen / eight / four: 4k positions 140.2 / 140.3 / 141.6 / 143.4 us, 32k
+// 862 / 862 / 877 / 890, 128k 5866 / 5810 / 5806 / 5905), but an exponential there is fourteen instructions to two, which
+// at the power limit costs more clock than it saves cycles.
+template <bool STATS, bool POLY>
 __device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 off, uint32_t off_sh, f32x2& s0,
                                           f32x2& s1) {
 #pragma unroll
@@ -557,8 +559,8 @@ __device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, f3
     }
     const f32x2 x0 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, o0);
     const f32x2 x1 = fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sc2, o1);
-    s0 = add2(s0, ((e >> 1) & 7) < kPolyPairs ? ex2_pair_poly<STATS>(x0) : ex2_pair(x0));
-    s1 = add2(s1, ((e >> 1) & 7) + 1 < kPolyPairs ? ex2_pair_poly<STATS>(x1) : ex2_pair(x1));
+    s0 = add2(s0, POLY && e == 0 ? ex2_pair_poly<STATS>(x0) : ex2_pair(x0));
+    s1 = add2(s1, ex2_pair(x1));
   }
 }
 
@@ -609,11 +611,11 @@ __device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i
         tc_ld_wait(ra);
         tc_ld16_issue(u.tcol + c0 + 16, rb);
         if (n_valid < kTileKeys) drop_keys(ra, n_valid - c0);
-        exp_chunk<true>(ra, sc2, 0, 0u, s0, s1);
+        exp_chunk<true, true>(ra, sc2, 0, 0u, s0, s1);
         tc_ld_wait(rb);
         if (c0 + 32 < kTileKeys) tc_ld16_issue(u.tcol + c0 + 32, ra);
         if (n_valid < kTileKeys) drop_keys(rb, n_valid - c0 - 16);
-        exp_chunk<true>(rb, sc2, 0, 0u, s0, s1);
+        exp_chunk<true, false>(rb, sc2, 0, 0u, s0, s1);
       }
       const float tile = sum2(s0, s1);
       const bool exact = !(tile < INFINITY && tile > kTinySum);
@@ -652,10 +654,10 @@ __device__ __forceinline__ bool votes_run(const Unit u, int nth, float sc, int i
     for (int c0 = 0; c0 < cols; c0 += 32) {
       tc_ld_wait(ra);
       tc_ld16_issue(u.tcol + c0 + 16, rb);
-      exp_chunk<false>(ra, sc2, 0, lse + 4u * c0, s0, s1);
+      exp_chunk<false, true>(ra, sc2, 0, lse + 4u * c0, s0, s1);
       tc_ld_wait(rb);
       if (c0 + 32 < cols) tc_ld16_issue(u.tcol + c0 + 32, ra); else unit_release(u);
-      exp_chunk<false>(rb, sc2, 0, lse + 4u * c0 + 64u, s0, s1);
+      exp_chunk<false, false>(rb, sc2, 0, lse + 4u * c0 + 64u, s0, s1);
     }
     float acc = sum2(s0, s1);
     if (half >= 0) {
