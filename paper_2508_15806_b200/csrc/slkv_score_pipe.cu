@@ -24,7 +24,7 @@
 // (the parameters of a list are kilobytes) took 3600 cycles per run and 1000 per tile of the MMA thread.
 //
 // What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
-//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in sixteen goes to the FMA
+//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in eight goes to the FMA
 //     pipe, and scale / subtract / sum run on packed pairs;
 //   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
 //     730 measured for loads and MMAs alone;
@@ -32,8 +32,8 @@
 //   - power: held for more than some milliseconds the part runs at its 1 kW limit, with every tile from HBM at 1.05 GHz
 //     (0.98 us per tile, MMAs alone 0.78), with tiles from L2 at 1.5 GHz (0.68 us).  Hence the groups.
 // Against the kernels before it (two streams with two accumulators and two warpgroups each on 128 SMs for up to 128 rows,
-// one launch per layer with a grid-wide barrier for more), a step of 32 layers, held: 32k tokens, 128 rows: 1120 -> 862 us;
-// eight ragged sequences of 147k tokens, 256 rows: 9890 -> 6690 us; 131k tokens, 256 rows: 9210 -> 5810 us.
+// one launch per layer with a grid-wide barrier for more), a step of 32 layers, held: 32k tokens, 128 rows: 1120 -> 850 us;
+// eight ragged sequences of 147k tokens, 256 rows: 9890 -> 6600 us; 131k tokens, 256 rows: 9210 -> 5720 us.
 // Every wait is bounded (1 s): SLKV_ERR_DEVICE_TIMEOUT in the status words, TMEM freed, return.
 #include <cuda.h>
 
@@ -543,10 +543,14 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
 
 // ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
 // sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials go
-// to the FMA pipe; every other chunk does that, one exponential in sixteen.  The special-function unit alone would take one
-// in eight or four (32 layers, none / one in sixteen / eight / four: 4k positions 140.2 / 140.3 / 141.6 / 143.4 us, 32k
-// 862 / 862 / 877 / 890, 128k 5866 / 5810 / 5806 / 5905), but an exponential there is fourteen instructions to two, which
-// at the power limit costs more clock than it saves cycles.
+// to the FMA pipe.  The special-function unit alone would take two pairs of every eight, but an exponential there is fourteen
+// instructions to two, which at the power limit costs more clock than it saves cycles (32 layers of 32k / 128k positions,
+// every chunk none of eight pairs 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: one in eight in the statistics, one
+// in sixteen in the votes.
+// The loops around this are kept small, the statistics' one chunk at a time with the last keys of a segment outside: four
+// warps on a scheduler hide a TMEM load's latency, and the epilogue warps are spread over both passes' loops, which have to
+// stay in the instruction cache (4k positions: statistics loop unrolled four times 154 us, twice 144, two chunks with the
+// last keys masked inside 140.9, as it is 140.1; 128k: 6147, 5865, 5868, 5820).
 template <bool STATS, bool POLY>
 __device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 off, uint32_t off_sh, f32x2& s0,
                                           f32x2& s1) {
@@ -582,13 +586,6 @@ __device__ __forceinline__ void unit_release(const Unit& u) {
   if ((threadIdx.x & 31) == 0) mbar_arrive(u.empty);
 }
 
-// The keys past the segment's end count nothing.
-__device__ __forceinline__ void drop_keys(uint32_t (&r)[16], int n_valid) {
-#pragma unroll
-  for (int e = 0; e < 16; ++e)
-    if (e >= n_valid) r[e] = __float_as_uint(-INFINITY);
-}
-
 // Statistics of one run for this thread's query row: tiles i0, i0 + every, ... < count.  z: the sum of 2^score, without a
 // reference; (far_z, far_m): what of it fp64 cannot hold (see StatView).  A tile is summed in fp32, without a reference
 // either as long as nothing overflows and not everything underflows; one whose sum is not finite and above kTinySum is
@@ -603,27 +600,27 @@ __device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i
     if (!unit_wait(u, nth)) return false;
     if (rows_here) {
       const int n_valid = n_valid0 - i * kTileKeys;
-      uint32_t ra[16], rb[16];
+      const int whole = n_valid < kTileKeys ? n_valid & ~15 : kTileKeys;
       f32x2 s0 = 0, s1 = 0;
-      tc_ld16_issue(u.tcol, ra);
 #pragma unroll 1
-      for (int c0 = 0; c0 < kTileKeys; c0 += 32) {
-        tc_ld_wait(ra);
-        tc_ld16_issue(u.tcol + c0 + 16, rb);
-        if (n_valid < kTileKeys) drop_keys(ra, n_valid - c0);
-        exp_chunk<true, true>(ra, sc2, 0, 0u, s0, s1);
-        tc_ld_wait(rb);
-        if (c0 + 32 < kTileKeys) tc_ld16_issue(u.tcol + c0 + 32, ra);
-        if (n_valid < kTileKeys) drop_keys(rb, n_valid - c0 - 16);
-        exp_chunk<true, false>(rb, sc2, 0, 0u, s0, s1);
+      for (int c0 = 0; c0 < whole; c0 += 16) {
+        uint32_t v[16];
+        tc_ld16_issue(u.tcol + c0, v);
+        tc_ld_wait(v);
+        exp_chunk<true, true>(v, sc2, 0, 0u, s0, s1);
       }
-      const float tile = sum2(s0, s1);
+      float tile = sum2(s0, s1);
+      if (n_valid < kTileKeys) {                               // the segment's last keys; those past its end count nothing
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
+        tile += tz * ex2(tm);
+      }
       const bool exact = !(tile < INFINITY && tile > kTinySum);
       if (!__any_sync(0xffffffffu, exact)) {
         z += (double)tile;
       } else {                                                 // the exact path's TMEM loads need the whole warp
         float tm, tz;
-        tile_stats_exact(u.tcol, sc, n_valid, tm, tz);
+        tile_stats_exact(u.tcol, sc, 0, n_valid, tm, tz);
         if (!exact) z += (double)tile;                         // the same value whatever the other rows hold
         else if (fabsf(tm) <= kFarScore) z += scalbn((double)tz, (int)tm);
         else stat_add(far_z, far_m, tz, tm);

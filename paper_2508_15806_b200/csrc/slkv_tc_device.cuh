@@ -294,14 +294,14 @@ __device__ __forceinline__ Run locate(const ScoreShape& a, int pos, int end) {
   return r;
 }
 
-// Statistics pass, exact path for this thread's row of one accumulator: z * 2^m = the sum over the tile's first n_valid
-// keys, m a whole number.  Used when the sum of the fast path over- or underflows.  Eight columns at a time: inlined beside
-// the fast path, it must not need registers of its own.
-__device__ __forceinline__ void tile_stats_exact(uint32_t tcol, float sc, int n_valid, float& m, float& z) {
+// Statistics pass, exact path for this thread's row of one accumulator: z * 2^m = the sum over the tile's keys
+// first .. n_valid - 1 (first a multiple of 8), m a whole number.  For tiles whose sum over- or underflows on the fast path,
+// and a segment's last keys.  Eight columns at a time: inlined beside the fast path, it must not need registers of its own.
+__device__ __forceinline__ void tile_stats_exact(uint32_t tcol, float sc, int first, int n_valid, float& m, float& z) {
   m = 0.f;
   z = 0.f;
 #pragma unroll 1
-  for (int c0 = 0; c0 < kTileKeys && c0 < n_valid; c0 += 8) {
+  for (int c0 = first; c0 < kTileKeys && c0 < n_valid; c0 += 8) {
     uint32_t r[8];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
