@@ -261,7 +261,7 @@ def run_cuda(args):
     use_graph = overlap and not args.no_graph
 
     def captured(fn):
-        """fn's calls captured once in a CUDA graph (they are stream-ordered and allocate nothing; the side streams
+        """fn's calls captured once in a CUDA graph (they are stream-ordered and allocate nothing; other streams
         of the overlapped calls fork from and rejoin the captured stream); returns the replaying step."""
         nonlocal stream
         cap = torch.cuda.Stream()
@@ -317,7 +317,7 @@ def run_cuda(args):
         n_eager = max(10, min(steps, 300))
         eager_us_per_layer = timed(n_eager, eager_step) / n_eager * 1e3 / nl
     # ---- attribution, (1): the score kernels alone bracketed by event pairs, everything else where it normally runs
-    # (selections and gathers on their side streams): the dominant kernel's time in the regime of the timed step,
+    # (the other kernels without any): the dominant kernel's time in the regime of the timed step,
     # taken right behind it
     prof_steps = min(max(steps, 10), 50)
     B.slkv_profile_enable(2)

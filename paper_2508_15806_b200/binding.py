@@ -346,7 +346,7 @@ def slkv_compress_host(params: SlkvParams, q_win, k, v, cu_seqlens: Sequence[int
 
 
 def slkv_profile_enable(on) -> None:
-    """False / 0: off; True / 1: every kernel (one stream); 2: the score kernels only, side streams kept."""
+    """False / 0: off; True / 1: every kernel (one stream); 2: the score kernels only."""
     lib().slkv_profile_enable(int(on))
 
 

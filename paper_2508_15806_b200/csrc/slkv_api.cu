@@ -14,7 +14,7 @@ thread_local int g_last_launches = 0;
 
 // ---- per-kernel timing (off by default) -----------------------------------------------------------
 struct TimedLaunch { int kid; cudaEvent_t a, b; };
-thread_local int g_prof_on = 0;          // 0 off, 1 every kernel (one stream), 2 the score kernels only (side streams kept)
+thread_local int g_prof_on = 0;          // 0 off, 1 every kernel (one stream), 2 the score kernels only
 thread_local std::vector<TimedLaunch>* g_prof = nullptr;      // records of the current thread
 thread_local std::vector<cudaEvent_t>* g_prof_free = nullptr;
 
