@@ -261,8 +261,7 @@ def run_cuda(args):
     use_graph = overlap and not args.no_graph
 
     def captured(fn):
-        """fn's calls captured once in a CUDA graph (they are stream-ordered and allocate nothing; other streams
-        of the overlapped calls fork from and rejoin the captured stream); returns the replaying step."""
+        """fn's calls captured once in a CUDA graph (they are stream-ordered and allocate nothing); returns the replaying step."""
         nonlocal stream
         cap = torch.cuda.Stream()
         stream = cap
