@@ -1,5 +1,6 @@
 // extern "C" entry points of libslkv: argument validation, workspace carve-up, launch sequencing.
 // No step of the method runs here; every step is a kernel in the other translation units.
+#include <atomic>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -41,7 +42,7 @@ int cuda_fail(cudaError_t e) {
 
 constexpr int kLaySlots = kListMaxLayers;      // overlapped calls: layers a launch takes
 struct Layout {
-  size_t hist_off, tile_off, pooled, flags, total;
+  size_t hist_off, tile_off, pooled, sync, total;
   size_t layer0, layer_bytes;                  // per-layer part: layer i's begins at layer0 + i * layer_bytes
   size_t vote, part, gather_src, win_m, win_z; // ... with these in it
 };
@@ -140,7 +141,7 @@ Layout layout_of(const Problem& pb, bool overlapped = false) {
   L.tile_off = o; o = align_up(o + (size_t)(pb.p.n_seqs + 1) * sizeof(int32_t));
   const size_t votes = (size_t)pb.p.n_kv_heads * (size_t)pb.total_hist * sizeof(float);
   L.pooled = o; o = align_up(o + votes);
-  L.flags = o; o = align_up(o + 8 * sizeof(int32_t));
+  L.sync = o; o = align_up(o + kSyncBytes);
   // Every layer of a list has its own votes, row statistics and source-row list; ordinary calls use the first.
   L.layer0 = o;
   size_t q = 0;
@@ -178,7 +179,7 @@ void carve(Problem* pb, const Layout& L, void* ws, int slot) {
   pb->tab.tile_ptr = pb->tile_off;
   pb->tab.hist_ptr = reinterpret_cast<const long long*>(pb->hist_off);
   pb->pooled_ws = reinterpret_cast<float*>(b + L.pooled);
-  pb->dev_flags = reinterpret_cast<int32_t*>(b + L.flags);
+  pb->sync = reinterpret_cast<unsigned long long*>(b + L.sync);
   unsigned char* l = b + L.layer0 + (size_t)slot * L.layer_bytes;
   pb->vote = reinterpret_cast<float*>(l + L.vote);
   pb->part = l + L.part;
@@ -501,6 +502,16 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
 }
 
 }  // namespace
+
+// Launch number times an odd constant: none comes twice in 2^48 - 1 launches, none is zero, and none looks like a small
+// number or an address, which workspaces are full of.
+unsigned long long next_launch_tag() {
+  static std::atomic<unsigned long long> launches{0};
+  const unsigned long long mask = (1ull << 48) - 1;
+  unsigned long long n;
+  do n = (launches.fetch_add(1, std::memory_order_relaxed) + 1) & mask; while (n == 0);
+  return n * 0x9E3779B97F4Bull & mask;
+}
 
 LaunchScope::LaunchScope(int kid, cudaStream_t st, int* launches) : kid_(kid), st_(st), slot_(-1) {
   ++*launches;

@@ -12,9 +12,6 @@
 // kept over the barrier instead of being formed again.
 // What bounds it: latency at the small sizes (1024 tokens, 8 heads, 16 rows: two dot-product loops of one thread per key and
 // two launches took 80 us, this takes 10), the FMA pipe at the large ones.
-#include <atomic>
-#include <cstring>
-
 #include "slkv_internal.cuh"
 
 namespace slkv {
@@ -100,17 +97,17 @@ struct SimtArgs {
   int n_seqs, n_kv_heads, G, window, R, n_tiles, keep, q_rows, stages, coop, barrier_extra;
   long long k_stride_tok, k_stride_head, q_stride_seq, q_stride_row, q_stride_head;
   float scale_log2;
-  unsigned* counters;          // [8], zero: arrivals at the launch's barriers, CTAs that are done
+  LaunchSync sync;             // counts 0 .. 2: arrivals at the barriers 1 .. 3
 };
-constexpr int kCountSlots = 64;
-__device__ unsigned g_simt_counters[kCountSlots * 8];
+constexpr int kBarriers = 3;
 
-// Waits, in one thread, until counter b has reached `target`.
+// Waits, in one thread, until all CTAs have cleared their part (b = 0), or `target` have arrived at barrier b.
 __device__ __forceinline__ int count_wait(const SimtArgs& a, int b, unsigned target) {
   unsigned long long t0 = 0, t;
   for (unsigned spin = 0;; ++spin) {
     unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.counters + b) : "memory");
+    if (b == 0) v = a.sync.arrived(0);
+    else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.sync.counts() + b - 1) : "memory");
     if (v >= target) return 1;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     if (spin == 0) t0 = t;
@@ -121,13 +118,17 @@ __device__ __forceinline__ int count_wait(const SimtArgs& a, int b, unsigned tar
     __nanosleep(20);
   }
 }
-// Arrives at barrier number b of the launch and waits for all CTAs (bounded: false when the wait ran out).
-__device__ __forceinline__ bool grid_wait(const SimtArgs& a, int b, unsigned extra) {
+// Arrives at barrier number b (1 .. 3) of the launch and waits for all CTAs (bounded: false when the wait ran out).
+// cleared: this thread knows that all CTAs have done their part of the clearing, the barriers' counts included.
+__device__ __forceinline__ bool grid_wait(const SimtArgs& a, int b, unsigned extra, bool cleared) {
   __shared__ int ok_sh;
   __syncthreads();
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + b) : "memory");
-    ok_sh = count_wait(a, b, gridDim.x + extra);
+    ok_sh = cleared || count_wait(a, 0, gridDim.x);
+    if (ok_sh) {
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.sync.counts() + b - 1) : "memory");
+      ok_sh = count_wait(a, b, gridDim.x + extra);
+    }
   }
   __syncthreads();
   return ok_sh != 0;
@@ -185,12 +186,14 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
   pdl_wait();
 
   if (a.coop) {
-    // clear the statistics area; nobody adds to it before all CTAs have done their part
+    // clear the statistics area and the barriers' counts; nobody adds to them before all CTAs have done their part
     const int words = (int)((size_t)n_seg * a.R * 5 + 2);
     const int w0 = (int)((long long)blockIdx.x * words / gridDim.x), w1 = (int)((long long)(blockIdx.x + 1) * words / gridDim.x);
     for (int i = w0 + tid; i < w1; i += kThreads) __stcg(static_cast<unsigned*>(a.part) + i, 0u);
+    if (blockIdx.x == 0 && tid < kBarriers) __stcg(a.sync.counts() + tid, 0u);
+    if (blockIdx.x == 0 && tid == 32) a.sync.put_tag(1, 0);
     __syncthreads();
-    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters) : "memory");
+    if (tid == 0) a.sync.arrive(0, false);
   }
 
   int q_seg = -1, q_chunk = -1;                                // what qs holds (q_chunk when it holds one step's rows)
@@ -371,22 +374,17 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
 
   bool ok = true;
   if (a.stages & kStats) round(kStats);
-  if (a.coop) ok = grid_wait(a, 1, (unsigned)a.barrier_extra);
+  if (a.coop) ok = grid_wait(a, 1, (unsigned)a.barrier_extra, cleared);
   if (ok && (a.stages & (kMaxima | kFarSums)) && __ldcg(st.far) != 0) {     // the same for every CTA: all sums are in
     if (a.stages & kMaxima) round(kMaxima);
-    if (a.coop) ok = grid_wait(a, 2, 0);
+    if (a.coop) ok = grid_wait(a, 2, 0, true);
     if (ok && (a.stages & kFarSums)) round(kFarSums);
-    if (a.coop && ok) ok = grid_wait(a, 3, 0);
+    if (a.coop && ok) ok = grid_wait(a, 3, 0, true);
   }
   if (ok && (a.stages & kVotes)) round(kVotes);
   if (a.coop && tid == 0) {
-    // the last CTA to leave puts the counters back to zero for their next user
-    unsigned prev;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(a.counters + 7) : "memory");
-    if (prev == gridDim.x - 1) {
-      for (int i = 0; i < 8; ++i) a.counters[i] = 0;
-      __threadfence();
-    }
+    // past a barrier the second word's tag is there; the last CTA to leave takes the tags away
+    if (a.sync.arrive(1, ok) == gridDim.x - 1) a.sync.words[0] = a.sync.words[1] = 0;
   }
 }
 
@@ -494,7 +492,6 @@ template <typename T, int D>
 cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaStream_t st, int* launches) {
   using TT = Tiles<T, D>;
   static thread_local int configured_dev = -1;
-  static thread_local unsigned* counters_base = nullptr;
   static thread_local int coop_state = 0;                      // 0 untried, 1 with dependent launch, 2 without, -1 refused
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -502,10 +499,6 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
   if (configured_dev != dev) {
     e = cudaFuncSetAttribute(k_score_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
     if (e != cudaSuccess) return e;
-    void* sym = nullptr;
-    e = cudaGetSymbolAddress(&sym, g_simt_counters);
-    if (e != cudaSuccess) return e;
-    counters_base = static_cast<unsigned*>(sym);
     coop_state = 0;
     configured_dev = dev;
   }
@@ -537,8 +530,8 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
     a.stages = passes == 3 ? kStats | kMaxima | kFarSums | kVotes : kStats | kMaxima | kFarSums;
     a.coop = 1;
     a.barrier_extra = take_expire_next_wait() ? 1 : 0;
-    static std::atomic<unsigned> launch_seq{0};
-    a.counters = counters_base + (size_t)(launch_seq.fetch_add(1) % kCountSlots) * 8;
+    a.sync.words = pb.sync;
+    a.sync.tag = next_launch_tag();
     for (int attempt = 0; attempt < 2; ++attempt) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(grid);
@@ -571,7 +564,8 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
   // no cooperative launch: the stages as launches of their own
   a.coop = 0;
   a.keep = 0;
-  a.counters = counters_base;
+  a.sync.words = nullptr;
+  a.sync.tag = 0;
   if (passes & 1) {
     e = cudaMemsetAsync(a.part, 0, simt_stat_bytes(pb.n_seg, pb.R), st);
     for (int stage = kStats; stage <= kFarSums && e == cudaSuccess; stage <<= 1) {

@@ -176,3 +176,86 @@ def test_more_streams_than_the_library_keeps_states_for():
     torch.cuda.synchronize()
     for outs in alive:
         job.assert_equal(outs, ref)
+
+
+class ScoreJob:
+    """slkv_score on one stream: its own inputs, output and workspace."""
+
+    def __init__(self, dt, d, path, seed):
+        g = torch.Generator(device=DEV).manual_seed(seed)
+        lens, w, hq, hkv = [500, 300], 16, 8, 4          # some 50 CTAs: two such launches are resident together
+        self.q = torch.randn(2, w, hq, d, generator=g, device=DEV).to(dt)
+        self.k = torch.randn(sum(lens), hkv, d, generator=g, device=DEV).to(dt)
+        self.cu = [0, lens[0], sum(lens)]
+        self.cu_dev = torch.tensor(self.cu, dtype=torch.int32, device=DEV)
+        self.params = B.make_params(self.q, self.k, None, w, 5, score_path=path)
+        self.ws = torch.randint(-2 ** 31, 2 ** 31 - 1, (B.slkv_workspace_bytes(self.params, self.cu) // 4,), generator=g,
+                                dtype=torch.int32, device=DEV).view(torch.uint8)      # whatever an allocator left there
+        self.status = torch.zeros(1, dtype=torch.int32, device=DEV)
+        self.n = B.slkv_pooled_elems(self.params, self.cu)
+        self.ref = self.call(self.out(), None).clone()
+        torch.cuda.synchronize()
+
+    def out(self):
+        return torch.zeros(self.n, dtype=torch.float32, device=DEV)
+
+    def call(self, out, stream):
+        return B.slkv_score(self.params, self.q, self.k, self.cu_dev, self.cu, out, self.ws, self.status, stream)
+
+    def check(self, outs):
+        assert int(self.status.item()) == 0
+        for o in outs:
+            # row sums are added in fp64 in an order that varies (2^-53 of the sum): the fp32 log-sum-exp behind them
+            # moves by one unit in the last place at most, 2^-20 here (|lse| < 16 in log2 units), the votes by as much
+            assert torch.allclose(o, self.ref, rtol=2.0 ** -20, atol=0.0)
+
+
+def test_fma_path_launches_of_different_types_side_by_side():
+    # launches of the FMA kernel's four instantiations wait inside for their own CTAs only, whatever runs beside them:
+    # called from two threads, and replayed from captured graphs
+    kinds = [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64), (torch.bfloat16, 128)]
+    jobs = [ScoreJob(dt, d, B.SLKV_PATH_SIMT, 7 + i) for i, (dt, d) in enumerate(kinds)]
+    streams = [torch.cuda.Stream() for _ in jobs]
+    run_side_by_side(jobs, streams)
+
+
+def run_side_by_side(jobs, streams, n=150):
+    outs = [[j.out() for _ in range(n)] for j in jobs]
+    errors = []
+    torch.cuda.synchronize()
+
+    def worker(t):
+        try:
+            torch.cuda.set_device(0)
+            for o in outs[t]:
+                jobs[t].call(o, streams[t])
+        except Exception as e:                          # noqa: BLE001 - reported below, in the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=worker, args=(t,)) for t in range(len(jobs))]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join(timeout=300)
+    assert not errors and all(not th.is_alive() for th in threads), errors
+    torch.cuda.synchronize()
+    for j, o in zip(jobs, outs):
+        j.check(o)
+    # graphs that are replayed beside one another, and over and over with the counters they were captured with
+    for st in [torch.cuda.Stream() for _ in range(32)] + [None]:      # torch's whole pool: nothing uncaptured is left
+        B.slkv_join(st)                                               # in flight for a captured call to be ordered behind
+    torch.cuda.synchronize()
+    graphs, last = [], []
+    for j, st in zip(jobs, streams):
+        g, o = torch.cuda.CUDAGraph(), j.out()
+        with torch.cuda.graph(g, stream=st):
+            j.call(o, st)
+        graphs.append(g)
+        last.append(o)
+    for _ in range(n):
+        for g, st in zip(graphs, streams):
+            with torch.cuda.stream(st):
+                g.replay()
+    torch.cuda.synchronize()
+    for j, o in zip(jobs, last):
+        j.check([o])
