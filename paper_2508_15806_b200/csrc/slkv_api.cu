@@ -261,7 +261,7 @@ cudaError_t flush_list(ListState* s, cudaStream_t owner, int* launches) {
   const int n = s->n;
   s->n = 0;
   s->in_flight = true;
-  cudaError_t e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, owner, launches);
+  cudaError_t e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, s->pb.sync, owner, launches);
   if (e == cudaSuccess)
     e = select_list_supported(s->pb) ? launch_select_list(s->pb, s->tail, n, owner, launches)
                                      : launch_select_cluster(s->pb, s->tail, n, owner, launches);

@@ -307,9 +307,9 @@ cudaError_t plan_score_layer(const Problem& pb, int32_t* status, ScoreLayer* lay
 int sm_count();
 int score_list_stages(int MT, int halves);
 // The score kernel over a list of layers of one shape: passes 1 = row statistics, 2 = votes from the callers' row
-// statistics, 3 = both.
-cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes, cudaStream_t st,
-                              int* launches);
+// statistics, 3 = both; sync: Problem's.
+cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
+                              unsigned long long* sync, cudaStream_t st, int* launches);
 // lse_out null: into the layer's own statistics area
 cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
                                     cudaStream_t st, int* launches);

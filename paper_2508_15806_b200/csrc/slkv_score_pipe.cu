@@ -37,7 +37,6 @@
 // Every wait is bounded (1 s): SLKV_ERR_DEVICE_TIMEOUT in the status words, TMEM freed, return.
 #include <cuda.h>
 
-#include <atomic>
 #include <cstdlib>
 #include <cstring>
 
@@ -62,23 +61,16 @@ constexpr int kHalfVoteBytes = 2 * 4 * 128 * 4;
 constexpr int kQTiles = 2;
 constexpr int kRunSlots = 8;                         // runs handed out ahead
 constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes + kRunSlots * 128;
-constexpr int kCountSlots = 32;                      // launches whose counters are live at once
-constexpr int kCountWords = kListMaxLayers * kListMaxGroups + 2;
 
 struct ListArgs {
   ScoreShape sh;
   ScoreLayer lay[kListMaxLayers];
   int n_layers, passes, lag;
   int group_layers, n_groups;  // as in ScoreShape; groups of the whole list
-  unsigned* counters;          // [n_groups] CTAs that have published the group's statistics, then CTAs that have cleared
-                               // their part of the statistics area, CTAs that are done
-  unsigned target;             // value a group's counter reaches when every CTA has published
+  LaunchSync sync;             // counts [n_groups]: CTAs that have published the group's statistics
+  unsigned target;             // value a group's count reaches when every CTA has published
   unsigned long long* trace;
 };
-
-// Counter sets, taken in turn by the launches (zero at load); the last CTA of a launch to finish puts its set back to
-// zero, so no memset sits between two launches.
-__device__ unsigned g_published[kCountSlots * kCountWords];
 
 // A run as warp 2 hands it out: consecutive tiles of one segment, in one pass.
 struct alignas(16) RunDesc {
@@ -403,8 +395,10 @@ __device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArg
       const RunDesc& r = c.runs[k_in & (kRunSlots - 1)];
       if (r.kind == 2) break;
       const int slot = n & 1;
-      const bool stats = r.kind == 0 && r.count > 0;
-      if (!stats || __any_sync(0xffffffffu, mbar_test(c.stat_full(slot), (n >> 1) & 1))) {
+      const bool stats = r.kind == 0 && r.count > 0, publish = r.kind == 0 && r.last && c.both;
+      // the epilogue warps have waited for the clearing before their statistics are out; an empty share waits here
+      const bool ready = stats ? mbar_test(c.stat_full(slot), (n >> 1) & 1) : !publish || mbar_test(c.cleared(), 0);
+      if (__any_sync(0xffffffffu, ready)) {
         if (stats) {
           const unsigned far = c.stat_far[slot];
           if (far) {                                           // rare: scores beyond fp64's range
@@ -427,12 +421,11 @@ __device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArg
           }
           ++n;
         }
-        const bool publish = r.kind == 0 && r.last && c.both;
         const int gg = r.gg;
         __syncwarp();
         if (lane == 0) {
           if (stats) mbar_arrive(c.stat_empty(slot));
-          if (publish) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + gg) : "memory");
+          if (publish) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.sync.counts() + gg) : "memory");
           mbar_arrive(c.run_empty(k_in));
         }
         ++k_in;
@@ -455,12 +448,14 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
   const int lane = threadIdx.x & 31;
   const int G = a.sh.G, window = a.sh.window, q_head_inner = a.sh.q_head_inner;
   const int n_seg = a.sh.n_seqs * a.sh.n_kv_heads, stride = a.sh.slot_stride;
-  auto wait_count = [&](const unsigned* p, unsigned target) {
+  // until all CTAs have cleared their part (group = -1), or have published the group
+  auto wait_count = [&](int group, unsigned target) {
     if (lane == 0) {
       unsigned long long t0 = 0;
       for (unsigned spin = 0;; ++spin) {
         unsigned v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        if (group < 0) v = a.sync.arrived(0);
+        else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.sync.counts() + group) : "memory");
         if (v >= target) break;
         if (spin == 0) t0 = now_ns();
         if ((spin & 15u) == 15u && (*c.abort_flag || now_ns() - t0 > kWaitLimitNs)) { *c.abort_flag = 1; break; }
@@ -471,7 +466,9 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     return __all_sync(0xffffffffu, *c.abort_flag == 0) != 0;
   };
   if (c.both) {
-    // this CTA's part of the layers' statistics areas is cleared; nobody adds to them before all parts are
+    // this CTA's part of the groups' counts and the layers' statistics areas is cleared; nobody adds to them before all are
+    if (blockIdx.x == 0 && lane == 0) a.sync.put_tag(1, 0);
+    for (int i = blockIdx.x + lane * gridDim.x; i < a.n_groups; i += 32 * gridDim.x) __stcg(a.sync.counts() + i, 0u);
     const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);
     const int w0 = split_begin(blockIdx.x, words, gridDim.x), w1 = split_begin(blockIdx.x + 1, words, gridDim.x);
     // The areas' addresses in one load, a lane each, through the generic address of the parameters: read one by one from
@@ -485,8 +482,8 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
       for (int i = w0 + lane; i < w1; i += 32) __stcg(p + i, 0u);
     }
     __syncwarp();
-    if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + a.n_groups) : "memory");
-    if (!wait_count(a.counters + a.n_groups, gridDim.x)) return;
+    if (lane == 0) a.sync.arrive(0, false);
+    if (!wait_count(-1, gridDim.x)) return;
   }
   if (lane == 0) mbar_arrive(c.cleared());
   int n = 0, seen = -1;                    // vote runs so far; the last group known to be published
@@ -497,7 +494,7 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     // every CTA has published its share of the group (all CTAs are resident, and a statistics phase waits for nothing
     // but vote phases that are due before it, so the count gets there; bounded all the same)
     if (c.both && r.gg != seen) {
-      if (!wait_count(a.counters + r.gg, a.target)) break;
+      if (!wait_count(r.gg, a.target)) break;
       seen = r.gg;
     }
     // The common case, straight through: the sums are on their way while the slot comes free, and no launch parameter is
@@ -836,18 +833,9 @@ k_score_list(const __grid_constant__ ListArgs a) {
     trace_mark(a.trace, 4);
     if (a.trace) a.trace[(size_t)blockIdx.x * kTraceSlots + 61] = (unsigned long long)clock64();
   }
-  if (warp == 0 && a.passes == 3) {
-    // every thread of this CTA is past its last use of the counters (the barrier above): the last CTA out cleans the set
-    const int n_words = a.n_groups + 1;
-    unsigned prev = 0;
-    if (lane == 0)
-      asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(a.counters + n_words) : "memory");
-    prev = __shfl_sync(0xffffffffu, prev, 0);
-    if (prev == gridDim.x - 1) {
-      for (int j = lane; j <= n_words; j += 32) a.counters[j] = 0;
-      __threadfence();
-    }
-  }
+  // Every thread of this CTA is past its last use of the counts (the barrier above).  Where no wait ran out the second
+  // word's tag is there; the last CTA out takes the tags away.
+  if (tid == 0 && a.passes == 3 && a.sync.arrive(1, abort_sh == 0) == gridDim.x - 1) a.sync.words[0] = a.sync.words[1] = 0;
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512u) : "memory");
@@ -892,22 +880,17 @@ int score_list_stages(int MT, int halves) {
   return n < kMaxStages ? n : kMaxStages;
 }
 
-cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes, cudaStream_t st,
-                              int* launches) {
+cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
+                              unsigned long long* sync, cudaStream_t st, int* launches) {
   if (n_layers < 1 || sh.n_cta == 0) return cudaSuccess;             // no history: nothing to score
   if (n_layers > kListMaxLayers) return cudaErrorInvalidValue;
   static thread_local int configured_dev = -1;
-  static thread_local unsigned* counters_base = nullptr;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
     e = cudaFuncSetAttribute(k_score_list, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
-    void* sym = nullptr;
-    e = cudaGetSymbolAddress(&sym, g_published);
-    if (e != cudaSuccess) return e;
-    counters_base = static_cast<unsigned*>(sym);
     configured_dev = dev;
   }
   ListArgs a;
@@ -924,8 +907,8 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   a.lag = kLagUnits / (per_phase > 0 ? per_phase : 1);
   if (a.lag > a.n_groups - 1) a.lag = a.n_groups - 1;
   if (a.lag < 1) a.lag = 1;
-  static std::atomic<unsigned> launch_seq{0};
-  a.counters = counters_base + (size_t)(launch_seq.fetch_add(1) % kCountSlots) * kCountWords;
+  a.sync.words = sync;
+  a.sync.tag = next_launch_tag();
   const bool waits_inside = passes == 3;
   a.target = (unsigned)sh.n_cta + (waits_inside && take_expire_next_wait() ? 1u : 0u);
   a.trace = tensor_trace_buffer(sh.n_cta);
@@ -985,7 +968,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     cs = 2;                                           // once more without dependent launch
   }
   cs = -1;
-  return launch_score_list(sh, lay, n_layers, passes, st, launches);
+  return launch_score_list(sh, lay, n_layers, passes, sync, st, launches);
 }
 
 }  // namespace slkv

@@ -219,6 +219,13 @@ def test_fma_path_launches_of_different_types_side_by_side():
     run_side_by_side(jobs, streams)
 
 
+def test_tensor_path_launches_side_by_side():
+    # as above for the tensor-core kernel, scores and statistics with different numbers of tiles per CTA
+    kinds = [(torch.bfloat16, 64, 21), (torch.bfloat16, 128, 22), (torch.bfloat16, 64, 23)]
+    jobs = [ScoreJob(dt, d, B.SLKV_PATH_TENSOR, seed) for dt, d, seed in kinds]
+    run_side_by_side(jobs, [torch.cuda.Stream() for _ in jobs])
+
+
 def run_side_by_side(jobs, streams, n=150):
     outs = [[j.out() for _ in range(n)] for j in jobs]
     errors = []
