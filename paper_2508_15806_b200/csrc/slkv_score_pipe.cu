@@ -469,8 +469,8 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     // this CTA's part of the groups' counts and the layers' statistics areas is cleared; nobody adds to them before all are
     if (blockIdx.x == 0 && lane == 0) a.sync.put_tag(1, 0);
     for (int i = blockIdx.x + lane * gridDim.x; i < a.n_groups; i += 32 * gridDim.x) __stcg(a.sync.counts() + i, 0u);
-    const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);
-    const int w0 = split_begin(blockIdx.x, words, gridDim.x), w1 = split_begin(blockIdx.x + 1, words, gridDim.x);
+    const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);       // < 2^30; times the CTAs it takes more than 32 bits
+    const int w0 = (int)((long long)blockIdx.x * words / gridDim.x), w1 = (int)((long long)(blockIdx.x + 1) * words / gridDim.x);
     // The areas' addresses in one load, a lane each, through the generic address of the parameters: read one by one from
     // the constant bank, where each is a miss, they took 15 us for 32 layers, and every CTA's first sums waited for that.
     static_assert(kListMaxLayers <= 32, "a lane per layer");

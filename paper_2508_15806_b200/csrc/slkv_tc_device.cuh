@@ -210,7 +210,8 @@ __device__ __forceinline__ uint32_t instr_desc(int M, int N) {
 }
 
 // The part that share i of n takes of T items, and its inverse (the index whose
-// range holds tile x of the group): shares differ by one tile at most.
+// range holds tile x of the group): shares differ by one tile at most.  The products fit 32 bits for tiles: describe() lets
+// through fewer than 2^31 / 128 + 2^20 of a layer, a list of one group has fewer than 2^24, and n is 160 at most.
 __device__ __forceinline__ int split_begin(int i, int T, int n) { return (int)(((unsigned)i * (unsigned)T) / (unsigned)n); }
 __device__ __forceinline__ int split_index(int x, int T, int n) {
   return (int)((((unsigned)x + 1u) * (unsigned)n - 1u) / (unsigned)T);

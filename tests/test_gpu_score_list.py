@@ -76,3 +76,25 @@ def test_scores_beyond_the_range_of_sums_without_a_reference():
     got, ref = lse.cpu().double().numpy(), np.asarray(ref)
     assert np.all(np.isfinite(got)) and np.abs(ref).max() > 2000
     assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-5
+
+
+def test_many_sequences_statistics_cleared_to_the_end():
+    # 7100 sequences x 8 heads x 256 rows: the statistics area times the CTAs that clear it is more than 2^32 words.  The
+    # queries overlap in memory (sequence s starts at row s), the keys are two of history and one of window per sequence.
+    n, hkv, R, d = 7100, 8, 256, 64
+    g = torch.Generator(device=DEV).manual_seed(5)
+    rows = torch.randn(n + hkv * R, d, generator=g, device=DEV).bfloat16()
+    q = rows.as_strided((n, 1, hkv * R, d), (d, hkv * R * d, d, 1))
+    k = torch.randn(3 * n, hkv, d, generator=g, device=DEV).bfloat16()
+    cu = list(range(0, 3 * n + 1, 3))
+    p = B.make_params(q, k, None, 1, 1, score_path=B.SLKV_PATH_TENSOR)
+    ws = torch.full((B.slkv_workspace_bytes(p, cu),), 0x42, dtype=torch.uint8, device=DEV)
+    pooled, status = torch.zeros(n, hkv, 2, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.slkv_score(p, q, k, torch.tensor(cu, dtype=torch.int32, device=DEV), cu, pooled, ws, status)
+    assert int(status) == 0
+    hist = k.view(n, 3, hkv, d)[:, :2].double()
+    for a in range(0, n, 500):
+        b = min(a + 500, n)
+        s = torch.einsum("nhrd,njhd->nhrj", q[a:b, 0].reshape(b - a, hkv, R, d).double(), hist[a:b]) / d ** 0.5
+        ref = torch.softmax(s, dim=3).mean(dim=2)
+        assert torch.allclose(pooled[a:b].double(), ref, rtol=P.REL_TOL, atol=0.0), a
