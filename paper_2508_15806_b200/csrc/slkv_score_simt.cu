@@ -187,9 +187,9 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
 
   if (a.coop) {
     // clear the statistics area and the barriers' counts; nobody adds to them before all CTAs have done their part
-    const int words = (int)((size_t)n_seg * a.R * 5 + 2);
-    const int w0 = (int)((long long)blockIdx.x * words / gridDim.x), w1 = (int)((long long)(blockIdx.x + 1) * words / gridDim.x);
-    for (int i = w0 + tid; i < w1; i += kThreads) __stcg(static_cast<unsigned*>(a.part) + i, 0u);
+    const long long words = (long long)n_seg * a.R * 5 + 2;            // may be more than 2^31
+    const long long w0 = blockIdx.x * words / gridDim.x, w1 = (blockIdx.x + 1) * words / gridDim.x;
+    for (long long i = w0 + tid; i < w1; i += kThreads) __stcg(static_cast<unsigned*>(a.part) + i, 0u);
     if (blockIdx.x == 0 && tid < kBarriers) __stcg(a.sync.counts() + tid, 0u);
     if (blockIdx.x == 0 && tid == 32) a.sync.put_tag(1, 0);
     __syncthreads();

@@ -37,3 +37,20 @@ def test_sums_beyond_fp32(d):
     lse = P.gpu_row_lse(q, k, [0, 900], 8, score_path=B.SLKV_PATH_SIMT).cpu().double().numpy()
     ref = np.asarray(O.row_lse(P.to_np64(q), P.to_np64(k), [0, 900], 8, "history"))
     assert np.abs(ref).max() > 200 and np.max(np.abs(lse - ref) / np.abs(ref)) < 1e-5
+
+
+def test_many_sequences_statistics_cleared_to_the_end():
+    # 52430 sequences x 8 heads x 1024 rows: the statistics area is more than 2^31 words.  One history key per sequence
+    # takes every row's whole weight.  The queries overlap in memory (sequence s starts at row s).
+    n, hkv, R, d = 52430, 8, 1024, 64
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev).manual_seed(6)
+    q = torch.randn(n + hkv * R, d, generator=g, device=dev).as_strided((n, 1, hkv * R, d), (d, hkv * R * d, d, 1))
+    k = torch.randn(2 * n, hkv, d, generator=g, device=dev)
+    cu = list(range(0, 2 * n + 1, 2))
+    p = B.make_params(q, k, None, 1, 1, score_path=B.SLKV_PATH_SIMT)
+    ws = torch.full((B.slkv_workspace_bytes(p, cu),), 0x42, dtype=torch.uint8, device=dev)
+    pooled, status = torch.zeros(n * hkv, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    B.slkv_score(p, q, k, torch.tensor(cu, dtype=torch.int32, device=dev), cu, pooled, ws, status)
+    assert int(status) == 0
+    assert torch.allclose(pooled, torch.ones_like(pooled), rtol=P.REL_TOL, atol=0.0)
