@@ -433,8 +433,8 @@ int slkv_trace_set_buffer(void* dev_buf, size_t bytes);
  * Test hook for the bounded waits (no counterpart in the paper).  Where the CTAs of a launch wait for one another
  * (the counters between the two passes of the score kernel), every wait gives up after one second, sets SLKV_ERR_DEVICE_TIMEOUT in the
  * call's status word, releases what the CTA holds and returns.  With the hook armed (on != 0) the next such launch made
- * by the calling thread waits for one arrival more than there are CTAs, so that exactly this path runs: the call's
- * results are then incomplete and its status word says so; the calls after it are unaffected.  One-shot: the launch
+ * by the calling thread waits for one arrival more than there are CTAs -- on = 2: where its CTAs wait for the clearing of
+ * the statistics, else where they wait for the statistics -- so that exactly this path runs: the call's results are then incomplete and its status word says so; the calls after it are unaffected.  One-shot: the launch
  * that takes it disarms it.
  */
 int slkv_debug_expire_next_wait(int on);

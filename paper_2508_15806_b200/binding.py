@@ -275,8 +275,9 @@ def slkv_row_lse(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_de
     return lse_out
 
 
-def slkv_debug_expire_next_wait(on: bool = True) -> None:
-    lib().slkv_debug_expire_next_wait(1 if on else 0)
+def slkv_debug_expire_next_wait(on=True) -> None:
+    """False / 0: off; True / 1: the wait for the statistics; 2: the wait for their clearing."""
+    lib().slkv_debug_expire_next_wait(int(on))
 
 
 def slkv_score_noalloc(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_dev: torch.Tensor,

@@ -595,7 +595,7 @@ int slkv_last_launch_count(void) { return g_last_launches; }
 int slkv_version(void) { return 300; }
 
 int slkv_debug_expire_next_wait(int on) {
-  expire_next_wait(on != 0);
+  expire_next_wait(on == 2 ? 2 : on != 0);
   return SLKV_OK;
 }
 

@@ -69,6 +69,7 @@ struct ListArgs {
   int group_layers, n_groups;  // as in ScoreShape; groups of the whole list
   LaunchSync sync;             // counts [n_groups]: CTAs that have published the group's statistics
   unsigned target;             // value a group's count reaches when every CTA has published
+  unsigned clear_target;       // ... the first word's when every CTA has done its part of the clearing
   unsigned long long* trace;
 };
 
@@ -483,7 +484,7 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     }
     __syncwarp();
     if (lane == 0) a.sync.arrive(0, false);
-    if (!wait_count(-1, gridDim.x)) return;
+    if (!wait_count(-1, a.clear_target)) return;
   }
   if (lane == 0) mbar_arrive(c.cleared());
   int n = 0, seen = -1;                    // vote runs so far; the last group known to be published
@@ -910,7 +911,9 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   a.sync.words = sync;
   a.sync.tag = next_launch_tag();
   const bool waits_inside = passes == 3;
-  a.target = (unsigned)sh.n_cta + (waits_inside && take_expire_next_wait() ? 1u : 0u);
+  const int expire = waits_inside ? take_expire_next_wait() : 0;
+  a.target = (unsigned)sh.n_cta + (expire == 1);
+  a.clear_target = (unsigned)sh.n_cta + (expire == 2);
   a.trace = tensor_trace_buffer(sh.n_cta);
   const size_t smem = (size_t)(kQTiles * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + kTail);
 

@@ -94,7 +94,8 @@ struct SimtArgs {
   float* vote;
   LseSource lse;
   int32_t* status;
-  int n_seqs, n_kv_heads, G, window, R, n_tiles, keep, q_rows, stages, coop, barrier_extra;
+  int n_seqs, n_kv_heads, G, window, R, n_tiles, keep, q_rows, stages, coop;
+  unsigned clear_target, barrier_target;      // arrivals that end the waits for the clearing and at barrier 1: the CTAs
   long long k_stride_tok, k_stride_head, q_stride_seq, q_stride_row, q_stride_head;
   float scale_log2;
   LaunchSync sync;             // counts 0 .. 2: arrivals at the barriers 1 .. 3
@@ -119,15 +120,16 @@ __device__ __forceinline__ int count_wait(const SimtArgs& a, int b, unsigned tar
   }
 }
 // Arrives at barrier number b (1 .. 3) of the launch and waits for all CTAs (bounded: false when the wait ran out).
-// cleared: this thread knows that all CTAs have done their part of the clearing, the barriers' counts included.
-__device__ __forceinline__ bool grid_wait(const SimtArgs& a, int b, unsigned extra, bool cleared) {
+// cleared: this thread knows that all CTAs have done their part of the clearing, the barriers' counts included; stuck: its
+// wait for that ran out, so that something is missing from the sums.
+__device__ __forceinline__ bool grid_wait(const SimtArgs& a, int b, unsigned target, bool cleared, bool stuck) {
   __shared__ int ok_sh;
-  __syncthreads();
+  if (__syncthreads_or(stuck)) return false;
   if (threadIdx.x == 0) {
-    ok_sh = cleared || count_wait(a, 0, gridDim.x);
+    ok_sh = cleared || count_wait(a, 0, a.clear_target);
     if (ok_sh) {
       asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.sync.counts() + b - 1) : "memory");
-      ok_sh = count_wait(a, b, gridDim.x + extra);
+      ok_sh = count_wait(a, b, target);
     }
   }
   __syncthreads();
@@ -274,7 +276,7 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) s[i][j] = sum_of(acc[i][j]) * a.scale_log2;
   };
-  bool cleared = !a.coop;
+  bool cleared = !a.coop, stuck = false;
   // one round over this CTA's tiles: stage is one of the enum's
   auto round = [&](int stage) {
     const bool far = stage == kVotes && !a.lse.lse_opt && __ldcg(st.far) != 0;
@@ -334,12 +336,11 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
           __syncthreads();
         } else if (chunk * kRows + (warp >> 1) * 16 < a.R) {
           if (!cleared) {                                       // uniform over the warp: spin on the clearing counter
-            if (lane == 0) count_wait(a, 0, gridDim.x);
-            __syncwarp();
-            cleared = true;
+            if (!stuck) cleared = __shfl_sync(0xffffffffu, lane == 0 ? count_wait(a, 0, a.clear_target) : 0, 0) != 0;
+            stuck = !cleared;
           }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < 4 && cleared; ++j) {
             const int row = row0 + 4 * j;
             const size_t at = (size_t)p.seg * a.R + min(row, a.R - 1);
             float v = stage == kMaxima ? -INFINITY : 0.f;
@@ -374,12 +375,12 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
 
   bool ok = true;
   if (a.stages & kStats) round(kStats);
-  if (a.coop) ok = grid_wait(a, 1, (unsigned)a.barrier_extra, cleared);
+  if (a.coop) ok = grid_wait(a, 1, a.barrier_target, cleared, stuck);
   if (ok && (a.stages & (kMaxima | kFarSums)) && __ldcg(st.far) != 0) {     // the same for every CTA: all sums are in
     if (a.stages & kMaxima) round(kMaxima);
-    if (a.coop) ok = grid_wait(a, 2, 0, true);
+    if (a.coop) ok = grid_wait(a, 2, gridDim.x, true, false);
     if (ok && (a.stages & kFarSums)) round(kFarSums);
-    if (a.coop && ok) ok = grid_wait(a, 3, 0, true);
+    if (a.coop && ok) ok = grid_wait(a, 3, gridDim.x, true, false);
   }
   if (ok && (a.stages & kVotes)) round(kVotes);
   if (a.coop && tid == 0) {
@@ -511,7 +512,6 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
   a.k_stride_tok = p.k_stride_tok; a.k_stride_head = p.k_stride_head;
   a.q_stride_seq = p.q_stride_seq; a.q_stride_row = p.q_stride_row; a.q_stride_head = p.q_stride_head;
   a.scale_log2 = kLog2e / sqrtf((float)p.head_dim);
-  a.barrier_extra = 0;
   // Two CTAs per SM where there is work for them (their loads and barriers overlap), one where not; the query rows of a
   // segment stay in shared memory where they fit beside the keys, else 64 at a time.
   const int sms = sm_count(), chunks = (pb.R + kRows - 1) / kRows;
@@ -521,6 +521,7 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
   const int base = fixed + a.q_rows * TT::kPitch * 4;
   const int most = sms * (limit == kSmemMost ? 1 : 2);
   const int grid = a.n_tiles < most ? a.n_tiles : most;
+  a.clear_target = a.barrier_target = (unsigned)grid;
   const int per_cta = (a.n_tiles + grid - 1) / grid, kept_tile = chunks * 16 * kThreads * 4;
   a.keep = 0;
   if (passes == 3) a.keep = (limit - base) / kept_tile < per_cta ? (limit - base) / kept_tile : per_cta;
@@ -529,7 +530,9 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
   if (passes != 2 && coop_state >= 0) {
     a.stages = passes == 3 ? kStats | kMaxima | kFarSums | kVotes : kStats | kMaxima | kFarSums;
     a.coop = 1;
-    a.barrier_extra = take_expire_next_wait() ? 1 : 0;
+    const int expire = take_expire_next_wait();
+    a.barrier_target += expire == 1;
+    a.clear_target += expire == 2;
     a.sync.words = pb.sync;
     a.sync.tag = next_launch_tag();
     for (int attempt = 0; attempt < 2; ++attempt) {
@@ -559,7 +562,6 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
       coop_state = 2;                                          // once more without dependent launch
     }
     coop_state = -1;
-    a.barrier_extra = 0;
   }
   // no cooperative launch: the stages as launches of their own
   a.coop = 0;

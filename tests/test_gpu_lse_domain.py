@@ -212,3 +212,27 @@ def test_a_wait_that_runs_out_in_the_list_kernel():
         ref = P.oracle_pooled(xs[i][0], xs[i][1], cu, w, p)
         P.assert_pooled_close(gpu["pooled"], ref, cu, 2, w)
         P.assert_selection_valid(gpu, ref, cu, buds[i], w, xs[i][1], xs[i][2])
+
+
+@pytest.mark.parametrize("path,dt", [(B.SLKV_PATH_SIMT, torch.float32), (B.SLKV_PATH_TENSOR, torch.bfloat16)])
+def test_nothing_is_added_to_statistics_that_may_not_be_clear(path, dt):
+    # the wait for the clearing runs out (every CTA has cleared its part all the same): the sums stay as the clearing left
+    # them -- zero, in a workspace that was nowhere zero before -- the status says so, and the next call is right
+    dev = torch.device("cuda:0")
+    q, k, v, cu = rand_case(8, 2, 32, [1500, 300], seed=41, dtype=dt)
+    qd, kd = q.to(dev), k.to(dev)
+    p = B.make_params(qd, kd, None, 32, 7, score_path=path)
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=dev)
+    pooled, status = torch.zeros(B.slkv_pooled_elems(p, cu), device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    ws = torch.full((B.slkv_workspace_bytes(p, cu),), 0x42, dtype=torch.uint8, device=dev)
+    B.slkv_debug_expire_next_wait(2)
+    B.slkv_score(p, qd, kd, cu_dev, cu, pooled, ws, status)
+    torch.cuda.synchronize()
+    assert int(status) == B.ERR["DEVICE_TIMEOUT"]
+    n_seg, R = 4, 128                                   # words: sums and far sums in fp64, maxima; sums and far bits
+    words = n_seg * R * 5 + 2 if path == B.SLKV_PATH_SIMT else n_seg * (R * 2 + 5)
+    assert int((ws.view(torch.int32) == 0).sum()) >= words
+    status.zero_()
+    B.slkv_score(p, qd, kd, cu_dev, cu, pooled, ws, status)
+    assert int(status) == 0
+    P.assert_pooled_close(pooled.cpu().numpy(), P.oracle_pooled(q, k, cu, 32, 7), cu, 2, 32)
