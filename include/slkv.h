@@ -241,7 +241,9 @@ int slkv_compress(const slkv_params* p, const void* q_win, const void* k, const 
  * statistics first (the softmax of Eq. 7 runs over all keys).  This entry point therefore works on several layers
  * at once: a call queues its layer, and a list of layers goes out as three launches on `stream` -- the score kernel, in
  * which the row-statistics pass of later layers runs between the vote passes of earlier ones, then the selections and the
- * gathers of all layers of the list -- when thirty-two layers are queued, or at slkv_join.  Consequences:
+ * gathers of all layers of the list -- when the queued layers come to some 0.4 ms of work, which is eight to thirty-two
+ * layers (thirty-two of up to 16k tokens, sixteen of 32k, eight of 64k and more, at 8 KV heads and 128 score rows), or at
+ * slkv_join.  Consequences:
  *   - Nothing of a call needs to have been enqueued when it returns: slkv_join(stream) enqueues whatever is still
  *     queued and makes `stream` wait for every overlapped call made so far on the current device (no host wait);
  *     consume outputs, or free / overwrite any input, output or workspace buffer -- q_win, k, v, cu_seqlens_dev
@@ -256,7 +258,7 @@ int slkv_compress(const slkv_params* p, const void* q_win, const void* k, const 
  *     streams per device keep a sequence each, a ninth takes over the one used longest ago once that one's
  *     stream has been made to wait for what it had in flight.
  *   - workspace must hold slkv_workspace_bytes_overlapped: votes, source-row lists and row statistics for the
- *     thirty-two layers of a list (one layer's worth for shapes that are not taken as lists).  Successive calls share one
+ *     layers of a list (one layer's worth for shapes that are not taken as lists).  Successive calls share one
  *     workspace; a call with another shape or workspace first sends out what is queued.  q_win, k, v, budgets and the
  *     outputs of calls that may be in flight together must not alias each other's outputs.
  *   - The call sequence is stream-ordered and allocates nothing on the device, so a step's calls plus the join can be

@@ -40,7 +40,6 @@ int cuda_fail(cudaError_t e) {
   return SLKV_ERR_CUDA;
 }
 
-constexpr int kLaySlots = kListMaxLayers;      // overlapped calls: layers a launch takes
 struct Layout {
   size_t hist_off, tile_off, pooled, sync, total;
   size_t layer0, layer_bytes;                  // per-layer part: layer i's begins at layer0 + i * layer_bytes
@@ -134,6 +133,21 @@ bool list_supported(const Problem& pb) {
          (select_list_supported(pb) || select_cluster_supported(pb));
 }
 
+// Layers of a list.  A list costs some 23 us beside its layers (pipeline fill and tail, selections and gathers that nothing
+// runs beside), and its layers wait for the last of them to be called: it goes out when it holds about 0.4 ms of work, 32768
+// products of 128 keys x 128 rows, or eight layers.  Steps of 32 layers, us in a row / by themselves from an idle GPU, with 32, 16, 8 and 4
+// layers to a list:
+//   4001 tokens, 128 rows    132 / 197    154 / 191    202 / 228    329 / 348
+//   32768 tokens, 128 rows   734 / 879    756 / 889    804 / 887    946 / 1017
+//   131072 tokens, 256 rows  5175 / 5717  5147 / 5690  5130 / 5697  5101 / 5746
+constexpr int64_t kListProducts = 32768;
+constexpr int kListMinLayers = 8;      // four: eight ragged sequences of 147k tokens, held, 6504 -> 6696 us
+int list_layers(const Problem& pb) {
+  const int64_t per_layer = pb.n_tiles128 * ((pb.R + 127) / 128);
+  const int64_t n = per_layer > 0 ? (kListProducts + per_layer - 1) / per_layer : kListMaxLayers;
+  return n < kListMinLayers ? kListMinLayers : (n > kListMaxLayers ? kListMaxLayers : (int)n);
+}
+
 Layout layout_of(const Problem& pb, bool overlapped = false) {
   Layout L;
   size_t o = 0;
@@ -157,7 +171,7 @@ Layout layout_of(const Problem& pb, bool overlapped = false) {
   L.win_m = q; q = align_up(q + wins);
   L.win_z = q; q = align_up(q + wins);
   L.layer_bytes = q;
-  L.total = o + q * (size_t)(overlapped && list_supported(pb) ? kLaySlots : 1);
+  L.total = o + q * (size_t)(overlapped && list_supported(pb) ? list_layers(pb) : 1);
   return L;
 }
 
@@ -221,7 +235,7 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
 
 // ---- overlapped calls ---------------------------------------------------------------------------------------
 // A call queues its layer; a list of layers goes out as three launches on the caller's stream -- scores, selections,
-// gathers, each over all layers of the list -- when it is full or at a join.  What a list gives over single calls: the
+// gathers, each over all layers of the list -- when it is full (list_layers) or at a join.  What a list gives over single calls: the
 // statistics of one layer overlap the votes of another, all layers' selections fill the SMs side by side, and the host
 // makes three launches instead of 48.
 struct ListState {
@@ -235,7 +249,7 @@ struct ListState {
   Problem pb;                    // of the shape; the per-layer pointers are set call by call
   Layout layout;
   ScorePlan plan;
-  int n = 0;                     // layers queued
+  int n = 0, n_max = 0;          // layers queued; those a list goes out at
   ScoreLayer score[kListMaxLayers];
   TailLayer tail[kListMaxLayers];
   bool in_flight = false;        // lists have gone out since this stream's last join
@@ -429,6 +443,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
         if (e != cudaSuccess) return cuda_fail(e);
         s->p = *p; s->cu_host.assign(cu_host, cu_host + p->n_seqs + 1); s->cu_dev = cu_dev;
         s->ws = ws; s->ws_bytes = ws_bytes; s->with_lse = with_lse; s->pb = pb; s->layout = L;
+        s->n_max = list_layers(pb);
         s->open = true;
       }
     }
@@ -446,7 +461,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
       const int rc = enqueue_window_stats(pb, SLKV_PATH_TENSOR, st, &launches);
       if (rc != SLKV_OK) return rc;
       s->tail[s->n] = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
-      if (++s->n == kListMaxLayers) {
+      if (++s->n == s->n_max) {
         e = flush_list(s, st, &launches);
         if (e != cudaSuccess) return cuda_fail(e);
       }

@@ -98,3 +98,27 @@ def test_many_sequences_statistics_cleared_to_the_end():
         s = torch.einsum("nhrd,njhd->nhrj", q[a:b, 0].reshape(b - a, hkv, R, d).double(), hist[a:b]) / d ** 0.5
         ref = torch.softmax(s, dim=3).mean(dim=2)
         assert torch.allclose(pooled[a:b].double(), ref, rtol=P.REL_TOL, atol=0.0), a
+
+
+@pytest.mark.parametrize("hist,w,layers", [(1000, 32, 32), (32768, 32, 16), (40000, 32, 14), (65536, 64, 8)])
+def test_a_list_goes_out_before_the_join(hist, w, layers):
+    # layers are queued until they come to 32768 products of 128 keys x 128 rows, eight at least and thirty-two at most
+    hq, hkv, d, n = 32, 8, 128, hist + w
+    g = torch.Generator(device=DEV).manual_seed(hist)
+    q, k = (torch.randn(*s, generator=g, device=DEV, dtype=torch.bfloat16) for s in ((1, w, hq, d), (n, hkv, d)))
+    p, cu = B.make_params(q, k, k, w, 7), [0, n]
+    cap = hkv * (w + 10)
+    bud = torch.full((hkv,), w + 10, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes_overlapped(p, cu), dtype=torch.uint8, device=DEV)
+    assert ws.numel() <= layers * B.slkv_workspace_bytes(p, cu)
+    outs = torch.zeros(2 * layers, 2, cap, d, dtype=torch.bfloat16, device=DEV)
+    off, kept = (torch.zeros(2 * layers, m, dtype=torch.int32, device=DEV) for m in (hkv + 1, cap))
+    cu_dev, launches = torch.tensor(cu, dtype=torch.int32, device=DEV), []
+    B.slkv_join()
+    for l in range(2 * layers):
+        B.slkv_compress_overlapped(p, q, k, k, cu_dev, cu, bud, outs[l, 0], outs[l, 1], off[l], kept[l], ws)
+        launches.append(B.slkv_last_launch_count())
+    B.slkv_join()
+    torch.cuda.synchronize()
+    assert launches == 2 * ([0] * (layers - 1) + [3]) and B.slkv_last_launch_count() == 0
+    assert (off[:, -1] == cap).all() and torch.equal(kept, kept[:1].expand_as(kept))
