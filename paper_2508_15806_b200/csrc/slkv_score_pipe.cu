@@ -9,8 +9,8 @@
 // The votes of a segment need its rows' statistics over all keys, i.e. from other CTAs.  The layers of a list and the
 // groups of segments inside a layer are independent, so every CTA (one per SM) walks one stream of phases
 //   S(0) .. S(lag-1), S(lag), V(0), S(lag+1), V(1), ..., V(last)
-// over groups of about 1024 tiles: by the time V(g) is due, the others have published S(g), nobody waits, and its keys are
-// still in L2.
+// over groups of about 32 MB of keys (1024 tiles at head_dim 128): by the time V(g) is due, the others have published S(g),
+// nobody waits, and its keys are still in L2.
 //
 // Roles (640 threads, one CTA per SM; a twenty-first warp would cost every thread 16 registers):
 //   warp 0     TMA loads of K tiles (ring of 2-4 x 32 KB, or more of 16 KB) and Q tiles; it never waits for Q while K stages are free

@@ -10,12 +10,22 @@ namespace slkv {
 namespace {
 
 constexpr int kMergeThreads = 256;
-// Tiles per group of a two-pass launch.  At 1024 tiles (34 MB of keys) the vote pass finds its keys in L2, given that it
-// lets them go itself: 68 MB from HBM per layer of 32k tokens and 8 heads instead of 134, and HBM reads are what the part's
-// power goes into (a 32 KB tile costs 4.9 uJ from HBM, 1.3 from L2; its MMAs 3.3, its exponentials 1.9).  A phase costs a
-// CTA about 1.2 us beside its tiles, so smaller groups lose more than they save.  32 such layers: 768 tiles 1083 us, 1024
-// 946, 2048 991.
-constexpr int kGroupTiles = 1024;
+// Keys per group of a two-pass launch, in bytes: 1024 tiles at head_dim 128, 2048 at 64.  At 32 MB the vote pass finds its
+// keys in L2, given that it lets them go itself: 68 MB from HBM per layer of 32k tokens and 8 heads instead of 134, and HBM
+// reads are what the part's power goes into (a 32 KB tile costs 4.9 uJ from HBM, 1.3 from L2; its MMAs 3.3, its exponentials
+// 1.9).  A phase costs a CTA about 1.2 us beside its tiles, so smaller groups lose more than they save.  Steps of 32 layers
+// (16 for the last two), held, us:
+//   head_dim 128, 128 rows            16 MB   24 MB   32 MB   48 MB   64 MB
+//     4001 tokens                       154     144     136     138     137
+//     32768 tokens                     1059     960     866     952     931
+//     8 x 4k-32k tokens, 256 rows      3631    3437    3394    3480    3538
+//     131072 tokens, 256 rows          2940    2945    2950    3025    3088
+//   head_dim 64, 128 rows                      16 MB   24 MB   32 MB   40 MB
+//     8192 tokens                               195     187     184     183
+//     32768 tokens                              663     641     644     644
+//     8 x 4k-32k tokens, 256 rows              2605    2572    2561    2554
+//     131072 tokens, 256 rows                  2257    2226    2223    2282
+constexpr long long kGroupBytes = 32ll << 20;
 
 // The rows' log-sum-exps from the statistics of a launch over one layer: lse_out[s][h][i], in the units out_scale converts
 // to, or (null) the layer's own array, which a vote pass reads.
@@ -167,7 +177,8 @@ cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t
   if (n_cta > kMaxSplit) n_cta = kMaxSplit;
   a.n_cta = total < n_cta ? (int)total : n_cta;
   // groups of whole segments, of about equal size
-  long long want = (total + kGroupTiles / 2) / kGroupTiles;
+  const long long group_tiles = kGroupBytes / (a.halves * kHalfBytes);
+  long long want = (total + group_tiles / 2) / group_tiles;
   if (want > kListMaxGroups) want = kListMaxGroups;
   if (want < 1) want = 1;
   long long acc = 0;
@@ -184,8 +195,8 @@ cudaError_t plan_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t
   a.group_tile[++ng] = (int)total;
   a.n_groups = ng;
   a.group_layers = 0;
-  if (total < kGroupTiles * 3 / 4) {                     // short layers: several of a list together
-    a.group_layers = (int)((kGroupTiles + total / 2) / total);
+  if (total < group_tiles * 3 / 4) {                     // short layers: several of a list together
+    a.group_layers = (int)((group_tiles + total / 2) / total);
     if (a.group_layers > kListMaxLayers) a.group_layers = kListMaxLayers;
   }
   return cudaSuccess;

@@ -64,6 +64,29 @@ def test_lists_match_single_calls(lens, n_layers, w, lse):
             assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("lens", [[12000], [24700], [26000, 30000, 45]])
+def test_groups_of_narrow_keys(lens):
+    # head_dim 64: a group is 2048 tiles of 16 KB -- layers that share one, that fill one, that are walked in several
+    hq, hkv, d, w = 16, 8, 64, 16
+    q, k, v = layer(70 + len(lens), lens, hq, hkv, d, w)
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    ref = P.oracle_pooled(q, k, cu, w, 5)
+    p = B.make_params(q, k, v, w, 5)
+    qd, kd, vd = (t.to(DEV) for t in (q, k, v))
+    cu_dev, bud = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.full((hkv,), w + 50, dtype=torch.int32, device=DEV)
+    cap = sum(min(n, w + 50) for n in lens) * hkv
+    ws = torch.empty(B.slkv_workspace_bytes_overlapped(p, cu), dtype=torch.uint8, device=DEV)
+    outs = [[torch.zeros(*s, dtype=t, device=DEV) for s, t in (((cap, d), torch.bfloat16), ((cap, d), torch.bfloat16),
+             ((len(lens) * hkv + 1,), torch.int32), ((cap,), torch.int32), ((B.slkv_pooled_elems(p, cu),), torch.float32),
+             ((1,), torch.int32))] for _ in range(5)]
+    for o in outs:
+        B.slkv_compress_overlapped(p, qd, kd, vd, cu_dev, cu, bud, *o[:4], ws, o[4], o[5])
+    B.slkv_join()
+    for o in outs:
+        assert int(o[5]) == 0
+        P.assert_pooled_close(o[4].cpu().numpy(), ref, cu, hkv, w)
+
+
 def test_scores_beyond_the_range_of_sums_without_a_reference():
     # logits of several thousand, some rows only far below zero: the rows' sums leave fp64's range
     q, k, v = layer(9, [1500], 8, 2, 128, 32)
