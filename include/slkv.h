@@ -204,9 +204,16 @@ int slkv_score(const slkv_params* p, const void* q_win, const void* k, const int
  * The row statistics alone (Eq. 3-4 with Eq. 7's key set): lse_out[s][h][i] = log sum_j exp(q_i . k_j /
  * sqrt(head_dim)) over the softmax domain of p->softmax_domain, in p->lse_units, for the window rows of
  * every sequence longer than the window (rows of shorter sequences are left untouched).  It is what
- * slkv_score computes first when lse_opt is NULL; fed back as lse_opt it reproduces that call bit for bit
- * with SLKV_LSE_LOG2 (the kernels' own unit), and to rounding with SLKV_LSE_LN.  Callers that shard the
- * keys of one sequence over several devices merge these per shard and pass the result as lse_opt.
+ * slkv_score computes first when lse_opt is NULL; fed back as lse_opt it reproduces that call with SLKV_LSE_LOG2
+ * (the kernels' own unit), and to rounding with SLKV_LSE_LN.  Callers that shard the keys of one sequence over
+ * several devices merge these per shard and pass the result as lse_opt.
+ * "Reproduces", here and where the overlapped calls promise the results of single ones: a row's sum is added up from
+ * the fp32 sums of its tiles (128 keys; 32 on the FMA path) by fp64 additions whose order varies from launch to launch.
+ * Where the largest and the smallest of a row's n tile sums are no more than a factor 2^29 / n apart (2^19 at 131072
+ * keys) these additions are exact, and everything is the same bit for bit.  Beyond that, sums agree to 2^-53 times
+ * a few: the fp32 log-sum-exp of about one row in 10^8 differs in its last bit, its votes by 10^-6 of their value, and
+ * which of two positions is kept whose scores are that close.  With scores beyond fp64's range (900 in log2 units)
+ * the log-sum-exps agree to fp32 rounding.
  *   lse_out   dev, out, float[n_seqs][n_q_heads][window]
  * Other arguments and errors as slkv_score.
  */

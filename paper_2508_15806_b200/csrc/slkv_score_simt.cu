@@ -4,8 +4,8 @@
 // 256 threads forms 64 keys x 64 rows of scores at a time, 4 x 4 per thread in packed pairs (fma.rn.f32x2) over the head
 // dimension, K and Q as fp32 rows in shared memory, padded so that the 16-byte loads of a warp -- eight key groups, four row
 // groups -- are one wavefront each; eight of those feed 64 multiply-adds.  Persistent CTAs walk the segments' key tiles:
-//   statistics  row sums of 2^score per 32 keys, added up in fp64 with atomics (the order shows at 2^-53, not in the
-//               fp32 results); nothing is subtracted unless a sum over- or underflows, in which case every CTA learns so at
+//   statistics  row sums of 2^score per 32 keys, added up in fp64 with atomics (exact, whatever the order, where n such
+//               sums are within a factor 2^29 / n of one another; else the same to 2^-53 times a few); nothing is subtracted unless a sum over- or underflows, in which case every CTA learns so at
 //               the barrier and two more rounds find the rows' maxima and sum relative to them;
 //   votes       vote[j] = (1/G) sum_rows 2^(s_rj - lse_r), rows in a fixed order.
 // Both passes are one cooperative launch with a grid-wide barrier between them; score tiles that fit in shared memory are

@@ -217,8 +217,9 @@ __device__ __forceinline__ int split_index(int x, int T, int n) {
   return (int)((((unsigned)x + 1u) * (unsigned)n - 1u) / (unsigned)T);
 }
 // Row statistics in global memory, per segment and row: acc = the sum of 2^score over all keys, in fp64 and without a
-// reference.  The terms are fp32 sums over one tile each, added atomically: in whatever order they come, the sum is the
-// same to 2^-53, far below what its fp32 logarithm shows.
+// reference.  The terms are fp32 sums over one tile each, added atomically in whatever order they come.  n of them within a
+// factor 2^29 / n of one another fit one 53-bit window, the additions are exact and the order shows nowhere; else the sum is
+// the same to 2^-53 times a few, and about one fp32 logarithm in 10^8 differs in its last bit.
 // Scores beyond fp64's range (above 900 or below -900 in log2 units) go elsewhere: share `slot` then holds such a part of
 // the row's sum as z * 2^m, and its bit in far[] is set.
 constexpr float kFarScore = 900.f;
