@@ -3,7 +3,7 @@
 //
 // Two passes over a layer's keys, in 128-key tiles:
 //   statistics  S = Q K^T with the G*w query rows as the M dimension: a TMEM lane -- one thread -- owns a query row and
-//               keeps (reference, sum of 2^(s - reference)) in registers; per CTA and segment one pair per row goes out;
+//               sums 2^s over a tile's keys in fp32, over a run of tiles in fp64, and adds the run's sum to the row's;
 //   votes       S^T = K Q^T with the keys as the M dimension: a thread owns a key, and
 //               vote[j] = (1/G) sum_rows 2^(s_rj - lse_r) is a thread-local sum and a coalesced store.
 // The votes of a segment need its rows' statistics over all keys, i.e. from other CTAs.  The layers of a list and the
@@ -130,7 +130,7 @@ struct Smem {
   __device__ __forceinline__ uint32_t drain() const { return bar(2 * kMaxStages + 28 + 2 * kRunSlots); }   // a wait ran out
 };
 constexpr int kNumBars = 2 * kMaxStages + 30 + 2 * kRunSlots;
-constexpr int kHeadInts = 14;
+constexpr int kHeadInts = 9;
 static_assert(kNumBars * 8 + kHeadInts * 4 + 16 <= kBarBytes, "mbarriers");
 constexpr int kRunReaders = 4 + 4 * kWgs;              // arrivals that free a run slot: one per reading thread or warp
 
@@ -776,8 +776,8 @@ k_score_list(const __grid_constant__ ListArgs a) {
     for (int k = 0; k < kQTiles; ++k) { mbar_init(c.q_full(k), 1); mbar_init(c.q_empty(k), 1); }
     for (int k = 0; k < kRunSlots; ++k) { mbar_init(c.run_full(k), 1); mbar_init(c.run_empty(k), kRunReaders); }
     head[0] = sh.R; head[1] = sh.Rp; head[2] = sh.MT; head[3] = sh.halves;
-    head[5] = sh.n_stages; head[6] = sh.k_head_inner;
-    head[7] = a.passes == 3; head[8] = __float_as_int(sh.scale_log2); head[9] = __float_as_int(1.0f / (float)sh.G);
+    head[4] = sh.n_stages; head[5] = sh.k_head_inner;
+    head[6] = a.passes == 3; head[7] = __float_as_int(sh.scale_log2); head[8] = __float_as_int(1.0f / (float)sh.G);
     mbar_init(c.drain(), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -795,8 +795,8 @@ k_score_list(const __grid_constant__ ListArgs a) {
   tc_fence_after();
   c.tmem = tmem_base_sh;
   c.R = head[0]; c.Rp = head[1]; c.MT = head[2]; c.halves = head[3];
-  c.n_stages = head[5]; c.k_head_inner = head[6];
-  c.both = head[7]; c.sc = __int_as_float(head[8]); c.inv_g = __int_as_float(head[9]);
+  c.n_stages = head[4]; c.k_head_inner = head[5];
+  c.both = head[6]; c.sc = __int_as_float(head[7]); c.inv_g = __int_as_float(head[8]);
   c.q_half = c.MT * 128 * 128;
   c.q_bytes = c.halves * c.q_half;
   c.stage_bytes = c.halves * kHalfBytes;

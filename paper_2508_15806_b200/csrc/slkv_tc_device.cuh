@@ -14,8 +14,8 @@ constexpr int kTileKeys = 128;                 // keys per tile (MMA N in the st
 constexpr int kHalfBytes = kTileKeys * 128;    // one 64-element (128-byte) half of a 128-row tile
 constexpr int kSmemLimit = 227 * 1024;         // dynamic shared memory a CTA can have
 constexpr int kTraceSlots = 64;                // timeline words per CTA (see slkv_trace_set_buffer)
-// A row sum under the fixed reference that is not above this has underflowed (terms below fp32's range are flushed
-// to zero, or clamped to 2^-125 on the polynomial path): the exact path then moves the reference.
+// A tile's row sum that is not above this has underflowed (terms below fp32's range are flushed to zero, or clamped to
+// 2^-125 on the polynomial path): the exact path then sums relative to the tile's maximum.
 constexpr float kTinySum = 1e-30f;
 constexpr unsigned long long kWaitLimitNs = 1000ull * 1000ull * 1000ull;   // 1 s per wait
 
@@ -61,12 +61,10 @@ __device__ __forceinline__ void trace_mark(const unsigned long long* base, int s
   if (base) const_cast<unsigned long long*>(base)[(size_t)blockIdx.x * kTraceSlots + slot] = now_ns();
 }
 // Waits for the phase with the given parity.  false = gave up (limit reached or another thread did).
-// backoff_ns > 0: sleep that long between polls, so that a waiting warp leaves the issue slots to the working ones.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned backoff_ns = 0) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = now_ns();
   for (unsigned it = 1;; ++it) {
-    if (backoff_ns) __nanosleep(backoff_ns);
     if (mbar_try(bar, parity)) return true;
     if ((it & 63u) == 0) {
       if (*abort_flag) return false;
@@ -75,12 +73,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
-}
-// The same load with an L2 eviction policy (from createpolicy) for the lines it touches.
+// policy: L2 eviction policy (from createpolicy) for the lines the load touches
 __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar,
                                                  uint64_t policy) {
   asm volatile(
