@@ -33,7 +33,7 @@ UNIT = "tokens/s/layer"
 WORKLOAD_INDEX = 2          # the 32k-context, 32-layer configuration (third of the five workloads)
 TOTAL_INDEX = 1             # average budget 512 per KV head
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_per_key_row.txt")
-KERNEL_SOURCES = {"k_score_pipe": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"],
+KERNEL_SOURCES = {"k_score_list": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"],
                   "k_score_fused": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"]}
 
 
@@ -315,8 +315,7 @@ def run_cuda(args):
         # the same calls issued every step, right behind the timed run (same clocks and temperature)
         n_eager = max(10, min(steps, 300))
         eager_us_per_layer = timed(n_eager, eager_step) / n_eager * 1e3 / nl
-    # ---- attribution, (1): the score kernels alone bracketed by event pairs, everything else where it normally runs
-    # (the other kernels without any): the dominant kernel's time in the regime of the timed step,
+    # ---- attribution, (1): the score kernels alone bracketed by event pairs: the dominant kernel's time in the regime of the timed step,
     # taken right behind it
     prof_steps = min(max(steps, 10), 50)
     B.slkv_profile_enable(2)
@@ -361,8 +360,8 @@ def run_cuda(args):
             with_lse["sustained_us_per_layer"] = held * 1e3 / nl
             with_lse["sustained_clocks"] = lse_sampler.summary()
 
-    # ---- attribution, (2): every kernel bracketed, on one stream: the other kernels' own times (that step is slower
-    # than the timed one); the score kernels' figures stay those of (1)
+    # ---- attribution, (2): every kernel bracketed: the other kernels' own times (that step is slower than the timed one);
+    # the score kernels' figures stay those of (1)
     B.slkv_profile_enable(1)
     barrier()
     for _ in range(prof_steps):
@@ -421,7 +420,7 @@ def run_cuda(args):
     q_bytes = len(wl.seq_lens) * w * wl.n_q_heads * d * e
     k_scan = hkv * n_hist * d * e
     rows_avg = sum(L["rows"] for L in layers) / nl
-    alg = {"k_score_fused": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_pipe": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_lse": k_scan + q_bytes, "k_score_vote": k_scan + q_bytes + 4 * hkv * n_hist,
+    alg = {"k_score_fused": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_list": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_lse": k_scan + q_bytes, "k_score_vote": k_scan + q_bytes + 4 * hkv * n_hist,
            "k_pool": 8 * hkv * n_hist, "k_select": 4 * hkv * n_hist + 4 * rows_avg,
            "k_gather": 4 * rows_avg * d * e + 4 * rows_avg, "k_setup": 0}
     kern = {}
@@ -430,8 +429,8 @@ def run_cuda(args):
         kern[name] = {"launches_per_step": cnt / prof_steps, "avg_us": ms * 1e3 / cnt, "share": ms / prof_total}
     top = max(per_kernel, key=lambda n: per_kernel[n][0])
     top_us = kern[top]["avg_us"]
-    # the two-layer score kernel takes a list of layers per launch: a launch's units are those of all its layers
-    layers_per_launch = nl / kern[top]["launches_per_step"] if top == "k_score_pipe" else 1.0
+    # a launch of k_score_list takes a list of layers: its units are those of all its layers
+    layers_per_launch = nl / kern[top]["launches_per_step"] if top == "k_score_list" else 1.0
     alg_top = alg[top] * layers_per_launch
     achieved = alg_top / (top_us * 1e-6) / 1e9
     layer_bytes = k_scan + q_bytes + 4 * rows_avg * d * e
@@ -453,7 +452,7 @@ def run_cuda(args):
     # The score kernel's own ceiling is the special-function unit, not HBM: two exponentials per (query row, key)
     # at 16 ex2.approx per clock per SM need longer than streaming K once.  Reported beside the HBM figures.
     if top.startswith("k_score"):
-        n_exp = (exps_layer if top in ("k_score_fused", "k_score_pipe") else exps_layer / 2) * layers_per_launch
+        n_exp = (exps_layer if top in ("k_score_fused", "k_score_list") else exps_layer / 2) * layers_per_launch
         peak_gexp = 148 * 16 * 1965e6 / 1e9
         roofline["alu"] = {"bound": "alu", "unit": "Gexp/s", "achieved": n_exp / (top_us * 1e-6) / 1e9, "peak": peak_gexp,
                            "frac": n_exp / (top_us * 1e-6) / 1e9 / peak_gexp, "exps_per_launch": n_exp,

@@ -271,7 +271,7 @@ int slkv_compress(const slkv_params* p, const void* q_win, const void* k, const 
  *   - The call sequence is stream-ordered and allocates nothing on the device, so a step's calls plus the join can be
  *     captured in a CUDA graph.
  *   - Lists take bf16 and (n_q_heads / n_kv_heads) * window <= 256, at most 64 sequences, segments the one-launch
- *     selections take (up to 131072 history positions).  Other shapes run as slkv_compress does, on `stream`, after a join.
+ *     selections take (up to 262116 history positions with pool_kernel <= 9, up to 131040 with pool_kernel <= 129).  Other shapes run as slkv_compress does, on `stream`, after a join.
  * Arguments, results and error codes otherwise as slkv_compress.
  */
 int slkv_compress_overlapped(const slkv_params* p, const void* q_win, const void* k, const void* v,
@@ -416,9 +416,8 @@ int slkv_last_launch_count(void);
  * Per-kernel timing for benchmarks (no counterpart in the paper).  While enabled on the calling thread,
  * every kernel the library enqueues is bracketed by a CUDA event pair on its stream (events are created
  * on demand and reused; this adds host work per launch, so headline timings are taken with it off).
- * on = 1: every kernel, and the overlapped entry point keeps selections and gathers on the caller's stream so that
- * the pairs do not overlap (the step is then slower than untimed); on = 2: the score kernels only, everything else
- * where it normally runs -- the score kernels' times in the regime of an untimed step; on = 0: off.
+ * on = 1: every kernel (each then waits for the one before it to end, so that the step is slower than untimed); on = 2:
+ * the score kernels only -- their times in the regime of an untimed step; on = 0: off.
  * slkv_profile_collect waits for the recorded events, adds each kernel's elapsed milliseconds and launch
  * count into total_ms[id] / launches[id] (arrays of n_kernels entries, overwritten) and forgets the records.
  * Kernel ids run from 0 to slkv_kernel_count()-1; slkv_kernel_name gives their names.

@@ -15,7 +15,7 @@ thread_local int g_last_launches = 0;
 
 // ---- per-kernel timing (off by default) -----------------------------------------------------------
 struct TimedLaunch { int kid; cudaEvent_t a, b; };
-thread_local int g_prof_on = 0;          // 0 off, 1 every kernel (one stream), 2 the score kernels only
+thread_local int g_prof_on = 0;          // 0 off, 1 every kernel, 2 the score kernels only
 thread_local std::vector<TimedLaunch>* g_prof = nullptr;      // records of the current thread
 thread_local std::vector<cudaEvent_t>* g_prof_free = nullptr;
 
@@ -160,7 +160,7 @@ Layout layout_of(const Problem& pb, bool overlapped = false) {
   L.layer0 = o;
   size_t q = 0;
   L.vote = q; q = align_up(q + votes);
-  // row statistics: see stat_view (tensor cores), SimtStats
+  // row statistics: StatView (tensor cores), SimtStats
   const size_t shares = (size_t)tensor_slot_stride(pb);
   const size_t by_tensor = (size_t)pb.n_seg * ((shares * 8 + 12) * (size_t)pb.R + kMaxSplit / 8);
   const size_t by_simt = simt_part_bytes(pb);
@@ -531,7 +531,7 @@ unsigned long long next_launch_tag() {
 LaunchScope::LaunchScope(int kid, cudaStream_t st, int* launches) : kid_(kid), st_(st), slot_(-1) {
   ++*launches;
   if (!g_prof_on) return;
-  const bool score_kid = kid == KID_SCORE_LSE || kid == KID_SCORE_VOTE || kid == KID_SCORE_FUSED || kid == KID_SCORE_PIPE;
+  const bool score_kid = kid == KID_SCORE_LSE || kid == KID_SCORE_VOTE || kid == KID_SCORE_FUSED || kid == KID_SCORE_LIST;
   if (g_prof_on == 2 && !score_kid) return;
   if (!g_prof) g_prof = new std::vector<TimedLaunch>();
   TimedLaunch t{kid, prof_event(), prof_event()};
@@ -593,7 +593,7 @@ int slkv_profile_collect(float* total_ms, int32_t* launches, int32_t n_kernels) 
 
 const char* slkv_kernel_name(int kernel_id) {
   static const char* names[KID_COUNT] = {"k_setup", "k_score_lse", "k_score_vote", "k_pool", "k_select",
-                                         "k_gather", "k_alloc", "k_score_fused", "k_score_pipe", "k_window_stats",
+                                         "k_gather", "k_alloc", "k_score_fused", "k_score_list", "k_window_stats",
                                          "k_merge_lse", "k_behavior", "k_cp"};
   return (kernel_id >= 0 && kernel_id < KID_COUNT) ? names[kernel_id] : "";
 }
@@ -1070,7 +1070,9 @@ int slkv_compress_host(const slkv_params* p, const void* q_win, const void* k, c
   // What bounds this call is the host link.  Only the keys have to cross it: of V, page-locked memory is read by the gather
   // kernel where it lies, kept rows only, and page-locked outputs are written by that kernel directly (one launch instead of
   // four copies; 32k tokens, 8 heads, 512 rows kept per head: 2585 -> 1350 us, the keys alone 1210).  Pageable buffers are
-  // copied as a whole.
+  // copied as a whole.  However much is kept, reading page-locked V in place is faster than copying it (us, in place / copied,
+  // 32k tokens, d = 128: 1/16 kept 1529 / 2678, 1/4 2121 / 3170, 1/2 2878 / 3834, everything 4312 / 5129; d = 64, everything
+  // 2248 / 2605; 4k tokens, d = 128, everything 655 / 691).
   const size_t kv_bytes = (size_t)pb.total_tokens * p->n_kv_heads * d * e, out_bytes = (size_t)rows * d * e;
   const void* v_dev = pinned_address(v, kv_bytes);
   void* k_dst = pinned_address(k_out, out_bytes);

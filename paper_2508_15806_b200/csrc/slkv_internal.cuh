@@ -35,8 +35,7 @@ struct SeqTables {
 #endif
 };
 
-// Where a vote pass takes the window rows' log-sum-exp from when it does not merge the row statistics of the keys
-// it scored itself alone: the caller's array (lse_opt of the public entry points), and / or the statistics of the
+// Where a vote pass takes the window rows' log-sum-exp from, besides the row sums of the statistics pass: the caller's array (lse_opt of the public entry points), and / or the statistics of the
 // window keys (softmax over all causally visible keys).  Row r of a segment is query head g*G + hh, window row i with
 // r = i*G + hh (head_inner) or r = hh*window + i.
 struct LseSource {
@@ -152,7 +151,7 @@ struct Problem {
   int64_t* hist_off;      // [n_seqs+1] exclusive prefix of n_hist_s
   int32_t* tile_off;      // [n_seqs+1] exclusive prefix of ceil(n_hist_s / 128)
   float* vote;            // [n_kv_heads * total_hist] ragged, same layout as pooled
-  void* part;             // partial row statistics; layout of the score path
+  void* part;             // row statistics; layout of the score path (StatView, SimtStats)
   int64_t n_tiles128;     // 128-key tiles of all segments
   float* pooled_ws;       // [n_kv_heads * total_hist] used when the caller wants no pooled output
   int32_t* gather_src;    // [n_kv_heads * total_tokens] per packed row: token * n_kv_heads + head of its source
@@ -163,7 +162,7 @@ struct Problem {
 };
 
 // kernel ids for launch accounting / per-kernel timing
-enum KernelId { KID_SETUP = 0, KID_SCORE_LSE, KID_SCORE_VOTE, KID_POOL, KID_SELECT, KID_GATHER, KID_ALLOC, KID_SCORE_FUSED, KID_SCORE_PIPE, KID_WINDOW_STATS, KID_MERGE_LSE, KID_BEHAVIOR, KID_CP, KID_COUNT };
+enum KernelId { KID_SETUP = 0, KID_SCORE_LSE, KID_SCORE_VOTE, KID_POOL, KID_SELECT, KID_GATHER, KID_ALLOC, KID_SCORE_FUSED, KID_SCORE_LIST, KID_WINDOW_STATS, KID_MERGE_LSE, KID_BEHAVIOR, KID_CP, KID_COUNT };
 
 // Brackets one kernel launch: counts it and, when per-kernel timing is on for this thread, records a
 // CUDA event pair around it on the launch stream.
@@ -232,8 +231,7 @@ cudaError_t launch_score_simt(const Problem& pb, int32_t* status, int passes, cu
 // Row statistics of the window keys each window row sees causally (SLKV_ALL_CAUSAL) -> pb.win_m / pb.win_z, rows in
 // the order of the score path (head_inner: r = i*G + hh).
 cudaError_t launch_window_stats(const Problem& pb, bool head_inner, cudaStream_t st, int* launches);
-// Merges the per-chunk row statistics and the window statistics, if any, into lse_out[n_seqs][n_q_heads][window] in the
-// problem's lse_units.
+// lse_out[n_seqs][n_q_heads][window] in the problem's lse_units from the row sums and the window statistics, if any.
 cudaError_t launch_merge_lse_simt(const Problem& pb, float* lse_out, cudaStream_t st, int* launches);
 LseSource lse_source_of(const Problem& pb);
 float lse_out_scale(const Problem& pb);          // log2 units -> the problem's lse_units
@@ -290,7 +288,7 @@ struct ScoreShape {
 struct ScoreLayer {
   alignas(64) CUtensorMap tm_q;
   alignas(64) CUtensorMap tm_k;
-  void* part;                   // row statistics of every CTA's share of a segment (see stat_view)
+  void* part;                   // row statistics (see StatView)
   float* vote;
   LseSource lse;                // where the vote pass takes the rows' log-sum-exp from besides the statistics pass
   int32_t* status;

@@ -24,16 +24,16 @@
 // (the parameters of a list are kilobytes) took 3600 cycles per run and 1000 per tile of the MMA thread.
 //
 // What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
-//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in eight goes to the FMA
-//     pipe, and scale / subtract / sum run on packed pairs;
+//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in eight (statistics) or
+//     sixteen (votes) goes to the FMA pipe, and scale / subtract / sum run on packed pairs;
 //   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
 //     730 measured for loads and MMAs alone;
 //   - two epilogue warpgroups instead of four: 1250; sums over the keys across lanes instead of a lane per row: 1255;
 //   - power: held for more than some milliseconds the part runs at its 1 kW limit, with every tile from HBM at 1.05 GHz
 //     (0.98 us per tile, MMAs alone 0.78), with tiles from L2 at 1.5 GHz (0.68 us).  Hence the groups.
 // Against the kernels before it (two streams with two accumulators and two warpgroups each on 128 SMs for up to 128 rows,
-// one launch per layer with a grid-wide barrier for more), a step of 32 layers, held: 32k tokens, 128 rows: 1120 -> 850 us;
-// eight ragged sequences of 147k tokens, 256 rows: 9890 -> 6600 us; 131k tokens, 256 rows: 9210 -> 5720 us.
+// one launch per layer with a grid-wide barrier for more), a step of 32 layers, held: 32k tokens, 128 rows: 1120 -> 870 us;
+// eight ragged sequences of 147k tokens, 256 rows: 9890 -> 6640 us; 131k tokens, 256 rows: 9210 -> 5820 us.
 // Every wait is bounded (1 s): SLKV_ERR_DEVICE_TIMEOUT in the status words, TMEM freed, return.
 #include <cuda.h>
 
@@ -541,10 +541,10 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
 
 // ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
 // sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials go
-// to the FMA pipe.  The special-function unit alone would take two pairs of every eight, but an exponential there is fourteen
-// instructions to two, which at the power limit costs more clock than it saves cycles (32 layers of 32k / 128k positions,
-// every chunk none of eight pairs 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: one in eight in the statistics, one
-// in sixteen in the votes.
+// to the FMA pipe, where it takes fourteen instructions instead of two.  By cycles alone two pairs of eight would go there;
+// at the power limit the instructions cost more clock than they save cycles (32 layers of 32k / 128k positions, in both
+// passes no pair of a chunk's eight on the FMA pipe 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: one pair of eight
+// in the statistics, in the votes one in every other chunk.
 // The loops around this are kept small, the statistics' one chunk at a time with the last keys of a segment outside: four
 // warps on a scheduler hide a TMEM load's latency, and the epilogue warps are spread over both passes' loops, which have to
 // stay in the instruction cache (4k positions: statistics loop unrolled four times 154 us, twice 144, two chunks with the
@@ -941,7 +941,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
   }
-  const int kid = passes == 1 ? KID_SCORE_LSE : (n_layers > 1 ? KID_SCORE_PIPE : (passes == 2 ? KID_SCORE_VOTE : KID_SCORE_FUSED));
+  const int kid = passes == 1 ? KID_SCORE_LSE : (n_layers > 1 ? KID_SCORE_LIST : (passes == 2 ? KID_SCORE_VOTE : KID_SCORE_FUSED));
   if (!waits_inside) return launch_pdl_scoped(kid, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
   for (int attempt = 0; attempt < 2; ++attempt) {
     cudaLaunchConfig_t cfg = {};

@@ -301,6 +301,7 @@ int select_cluster_size(const Problem& pb) {
   return cs;
 }
 
+// up to 131040 history positions
 bool select_cluster_supported(const Problem& pb) {
   const int cs = select_cluster_size(pb);
   return (pb.max_hist + cs - 1) / cs + 4 <= kMaxSlice && pb.p.pool_kernel <= 129;

@@ -129,9 +129,8 @@ def overlapped_layers(xs, cu, buds, w, p, domain=B.SLKV_HISTORY, lses=None, want
 
 @pytest.mark.parametrize("n_layers", [1, 2, 5, 11, 43])
 def test_overlapped_calls_with_supplied_lse(n_layers):
-    # every layer comes with its row statistics: the list kernel runs the vote pass on both of its streams.  The
-    # selections of a full list are held back until the next list is out; 43 layers take every workspace slot more
-    # than twice while some are held back (inputs cycle through 6 cases, the budgets differ per layer).
+    # every layer comes with its row statistics: the list kernel runs the vote phases alone.  43 layers are a full list and
+    # a part of one, in the same workspace (inputs cycle through 6 cases, the budgets differ per layer).
     w, p, lens = 32, 7, [1500, 700]
     cases = []
     for c in range(min(n_layers, 6)):
@@ -177,16 +176,15 @@ def test_all_causal_on_a_full_cfg2_layer():
 
 # ---- bounded waits -----------------------------------------------------------------------------------------------
 def test_a_wait_that_runs_out_is_reported_and_leaves_the_next_call_intact():
-    # The grid-wide barrier of the fused score kernel is told to expect one arrival more than there are CTAs: every
-    # CTA gives up after its time limit, the status word says so, and the following call -- which may land on the same
-    # barrier slot 64 launches later -- is correct.
+    # The score kernel is told to expect one arrival more than there are CTAs where it waits for the others' statistics:
+    # every CTA gives up after its time limit, the status word says so, and the calls that follow are correct.
     q, k, v, cu = rand_case(8, 2, 32, [6000], seed=31)
     bud = [100, 400]
     B.slkv_debug_expire_next_wait(True)
     broken = P.gpu_compress(q, k, v, cu, bud, 32, 7, score_path=B.SLKV_PATH_TENSOR)
     assert broken["status"] == B.ERR["DEVICE_TIMEOUT"]
     ref = P.oracle_pooled(q, k, cu, 32, 7)
-    for _ in range(66):                                   # once around the table of barrier slots
+    for _ in range(66):
         good = P.gpu_compress(q, k, v, cu, bud, 32, 7, score_path=B.SLKV_PATH_TENSOR, want_pooled=False)
         assert good["status"] == 0
     good = P.gpu_compress(q, k, v, cu, bud, 32, 7, score_path=B.SLKV_PATH_TENSOR)

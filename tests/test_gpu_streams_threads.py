@@ -1,8 +1,8 @@
 """GPU: slkv_compress_overlapped from two host threads and on several streams (Algorithm 3, same results).
 
-Calls made on different streams keep separate queues, slots and events inside the library; a join orders its stream
-behind every call made so far and forgets only the calls of its own stream.  Every case is compared bit for bit with
-slkv_compress, one call at a time.
+Calls made on different streams keep separate queues inside the library; a join orders its stream behind every call made
+so far and forgets only the calls of its own stream.  Every such case is compared bit for bit with slkv_compress, one call
+at a time.  Launches whose CTAs wait for one another wait for their own only, whatever runs beside them.
 """
 import threading
 
@@ -70,8 +70,8 @@ class Job:
 
 
 def test_two_host_threads_each_on_its_own_stream():
-    # 21 and 13 layers of different shapes (more than a list, more than the slots of a workspace), three times each,
-    # the two threads free-running against each other; one of them hands its layers' log-sum-exps over
+    # 21 and 13 layers of different shapes, three times each, the two threads free-running against each other; one of them
+    # hands its layers' log-sum-exps over
     jobs = [Job([6000], 21, 300, 0), Job([2500, 1200], 13, 200, 5, with_lse=True)]
     refs = [j.reference() for j in jobs]
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
