@@ -518,14 +518,13 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
 
 }  // namespace
 
-// Launch number times an odd constant: none comes twice in 2^48 - 1 launches, none is zero, and none looks like a small
-// number or an address, which workspaces are full of.
+// Launch number times an odd constant: none looks like a small number or an address, which workspaces are full of, and in
+// 2^40 - 1 launches none comes twice and none is zero, in the low 40 bits either.
 unsigned long long next_launch_tag() {
   static std::atomic<unsigned long long> launches{0};
-  const unsigned long long mask = (1ull << 48) - 1;
   unsigned long long n;
-  do n = (launches.fetch_add(1, std::memory_order_relaxed) + 1) & mask; while (n == 0);
-  return n * 0x9E3779B97F4Bull & mask;
+  do n = launches.fetch_add(1, std::memory_order_relaxed) + 1; while ((n & ((1ull << 40) - 1)) == 0);
+  return n * 0x9E3779B97F4A7C15ull;
 }
 
 LaunchScope::LaunchScope(int kid, cudaStream_t st, int* launches) : kid_(kid), st_(st), slot_(-1) {

@@ -63,46 +63,15 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 constexpr int kListMaxLayers = 32;          // layers one launch of the score, selection and gather kernels takes
 constexpr int kListMaxGroups = 64;          // groups of segments a layer is walked in
 
-// Counters of a launch whose CTAs wait for one another.  They lie in the caller's workspace, which belongs to one call at a
-// time, so launches on other streams -- other threads' calls, replays of captured graphs -- never meet in them.  Nobody
-// zeroes a workspace: the first two words carry the launch's own 48-bit tag above a 16-bit count, and whoever finds another
-// value there puts the tag first.  Everything else that has to start at zero, the counts behind them included, is cleared by
-// the launch's CTAs and touched only once all of them have arrived at the first word.  The last CTA to leave puts both words
-// back to zero, so that a replay, which brings the same tag, starts as the first launch did.  (A memset in front of the
-// launch would do as well, for 2.6 us a call: it cuts the dependent launch.)
-struct LaunchSync {
-  unsigned long long* words;   // [0] CTAs that have done their share of the clearing, [1] CTAs that are done; then counts
-  unsigned long long tag;      // 1 .. 2^48 - 1, another one for every launch
-#ifdef __CUDACC__
-  __device__ __forceinline__ unsigned* counts() const { return reinterpret_cast<unsigned*>(words + 2); }
-  // The launch's tag with count `first` into word w unless the tag is there: true when this call put it.
-  __device__ __forceinline__ bool put_tag(int w, unsigned first) const {
-    unsigned long long seen = 0;                           // what a launch leaves behind
-    for (int i = 0; i < 3; ++i) {                          // the word changes once, from whatever it was to the tag
-      unsigned long long old;
-      asm volatile("atom.acq_rel.gpu.global.cas.b64 %0, [%1], %2, %3;"
-                   : "=l"(old) : "l"(words + w), "l"(seen), "l"(tag << 16 | first) : "memory");
-      if (old == seen) return true;
-      if (old >> 16 == tag) return false;
-      seen = old;
-    }
-    return false;
-  }
-  // Arrives at word w, whose tag is there for certain (tagged) or not; returns the arrivals before.
-  __device__ __forceinline__ unsigned arrive(int w, bool tagged) const {
-    if (!tagged && put_tag(w, 1)) return 0;
-    unsigned long long old;
-    asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], 1;" : "=l"(old) : "l"(words + w) : "memory");
-    return (unsigned)(old & 0xffffu);
-  }
-  __device__ __forceinline__ unsigned arrived(int w) const {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(words + w) : "memory");
-    return v >> 16 == tag ? (unsigned)(v & 0xffffu) : 0u;
-  }
-#endif
-};
-constexpr size_t kSyncBytes = 16 + sizeof(unsigned) * (size_t)(kListMaxLayers * kListMaxGroups);
+// What the CTAs of a launch tell one another lies in the caller's workspace, which belongs to one call at a time, so launches
+// on other streams -- other threads' calls, replays of captured graphs -- never meet there.  Nobody zeroes a workspace: the
+// CTAs clear what has to start at zero, their counts included, and touch none of it before all have said that they are done.
+// They say so in words that carry the launch's own tag (WordSync, FlagSync in the two score kernels), which whatever a
+// workspace held before does not, and leave the words without it, so that a replay, which brings the same tag, starts as the
+// first launch did.  (A memset in front of the launch would do as well, for 2.6 us a call: it cuts the dependent launch.)
+constexpr int kSyncFlags = 320;             // tagged words: two CTAs per SM
+constexpr int kSyncCounts = kListMaxLayers * kListMaxGroups;
+constexpr size_t kSyncBytes = sizeof(unsigned long long) * kSyncFlags + sizeof(unsigned) * kSyncCounts;
 unsigned long long next_launch_tag();
 
 // Launches `kernel` with the programmatic-serialisation attribute (and optionally a cluster shape).
@@ -155,7 +124,7 @@ struct Problem {
   int64_t n_tiles128;     // 128-key tiles of all segments
   float* pooled_ws;       // [n_kv_heads * total_hist] used when the caller wants no pooled output
   int32_t* gather_src;    // [n_kv_heads * total_tokens] per packed row: token * n_kv_heads + head of its source
-  unsigned long long* sync;   // kSyncBytes: counters of the launches whose CTAs wait for one another (LaunchSync)
+  unsigned long long* sync;   // kSyncBytes: what the CTAs of a launch tell one another (WordSync, FlagSync)
   float* win_m;           // [n_seg][R] row statistics over the window keys (SLKV_ALL_CAUSAL without lse_opt)
   float* win_z;
   const float* lse_opt;   // the caller's row log-sum-exps, or null

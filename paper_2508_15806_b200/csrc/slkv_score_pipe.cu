@@ -62,14 +62,48 @@ constexpr int kQTiles = 2;
 constexpr int kRunSlots = 8;                         // runs handed out ahead
 constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes + kRunSlots * 128;
 
+// The clearing of the statistics and the groups' counts: one word with the launch's tag (40 bits) above two counts of 12 bits,
+// CTAs that are done and CTAs that have cleared their share.  A CTA that finds another value puts the tag first; the last CTA
+// out puts the word back to zero.  (A flag per CTA, as the FMA kernel has it, saves that round trip, but here it is hidden
+// behind the first tiles, and 148 CTAs polling 148 flags are not: 32 layers of 4001 tokens 127.4 -> 130.4 us.)
+struct WordSync {
+  unsigned long long* word;    // the counts begin kSyncFlags words further on
+  unsigned long long tag;
+  unsigned expect;             // CTAs to wait for: all of them
+  __device__ __forceinline__ unsigned* counts() const { return reinterpret_cast<unsigned*>(word + kSyncFlags); }
+  // This CTA has cleared its share (one thread, behind a barrier with those that did).
+  __device__ __forceinline__ void arrive() const {
+    unsigned long long seen = 0;                             // what a launch leaves behind
+    for (int i = 0; i < 3; ++i) {                            // the word changes once, from whatever it was to the tag
+      unsigned long long old;
+      asm volatile("atom.acq_rel.gpu.global.cas.b64 %0, [%1], %2, %3;"
+                   : "=l"(old) : "l"(word), "l"(seen), "l"(tag << 24 | 1u) : "memory");
+      if (old == seen) return;
+      if (old >> 24 == tag) break;
+      seen = old;
+    }
+    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(word) : "memory");
+  }
+  __device__ __forceinline__ bool all_arrived() const {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
+    return v >> 24 == tag && (unsigned)(v & 0xfffu) >= expect;
+  }
+  // This CTA, which has arrived, will not touch the counts any more.
+  __device__ __forceinline__ void leave() const {
+    unsigned long long old;
+    asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], 4096;" : "=l"(old) : "l"(word) : "memory");
+    if ((unsigned)(old >> 12 & 0xfffu) == gridDim.x - 1) *word = 0;
+  }
+};
+
 struct ListArgs {
   ScoreShape sh;
   ScoreLayer lay[kListMaxLayers];
   int n_layers, passes, lag;
   int group_layers, n_groups;  // as in ScoreShape; groups of the whole list
-  LaunchSync sync;             // counts [n_groups]: CTAs that have published the group's statistics
+  WordSync sync;               // counts [n_groups]: CTAs that have published the group's statistics
   unsigned target;             // value a group's count reaches when every CTA has published
-  unsigned clear_target;       // ... the first word's when every CTA has done its part of the clearing
   unsigned long long* trace;
 };
 
@@ -450,14 +484,17 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
   const int G = a.sh.G, window = a.sh.window, q_head_inner = a.sh.q_head_inner;
   const int n_seg = a.sh.n_seqs * a.sh.n_kv_heads, stride = a.sh.slot_stride;
   // until all CTAs have cleared their part (group = -1), or have published the group
-  auto wait_count = [&](int group, unsigned target) {
+  auto wait_count = [&](int group) {
     if (lane == 0) {
       unsigned long long t0 = 0;
       for (unsigned spin = 0;; ++spin) {
-        unsigned v;
-        if (group < 0) v = a.sync.arrived(0);
-        else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.sync.counts() + group) : "memory");
-        if (v >= target) break;
+        if (group < 0) {
+          if (a.sync.all_arrived()) break;
+        } else {
+          unsigned v;
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.sync.counts() + group) : "memory");
+          if (v >= a.target) break;
+        }
         if (spin == 0) t0 = now_ns();
         if ((spin & 15u) == 15u && (*c.abort_flag || now_ns() - t0 > kWaitLimitNs)) { *c.abort_flag = 1; break; }
         __nanosleep(20);
@@ -468,7 +505,6 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
   };
   if (c.both) {
     // this CTA's part of the groups' counts and the layers' statistics areas is cleared; nobody adds to them before all are
-    if (blockIdx.x == 0 && lane == 0) a.sync.put_tag(1, 0);
     for (int i = blockIdx.x + lane * gridDim.x; i < a.n_groups; i += 32 * gridDim.x) __stcg(a.sync.counts() + i, 0u);
     const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);       // < 2^30; times the CTAs it takes more than 32 bits
     const int w0 = (int)((long long)blockIdx.x * words / gridDim.x), w1 = (int)((long long)(blockIdx.x + 1) * words / gridDim.x);
@@ -483,8 +519,8 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
       for (int i = w0 + lane; i < w1; i += 32) __stcg(p + i, 0u);
     }
     __syncwarp();
-    if (lane == 0) a.sync.arrive(0, false);
-    if (!wait_count(-1, a.clear_target)) return;
+    if (lane == 0) a.sync.arrive();
+    if (!wait_count(-1)) return;
   }
   if (lane == 0) mbar_arrive(c.cleared());
   int n = 0, seen = -1;                    // vote runs so far; the last group known to be published
@@ -495,7 +531,7 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     // every CTA has published its share of the group (all CTAs are resident, and a statistics phase waits for nothing
     // but vote phases that are due before it, so the count gets there; bounded all the same)
     if (c.both && r.gg != seen) {
-      if (!wait_count(r.gg, a.target)) break;
+      if (!wait_count(r.gg)) break;
       seen = r.gg;
     }
     // The common case, straight through: the sums are on their way while the slot comes free, and no launch parameter is
@@ -834,9 +870,7 @@ k_score_list(const __grid_constant__ ListArgs a) {
     trace_mark(a.trace, 4);
     if (a.trace) a.trace[(size_t)blockIdx.x * kTraceSlots + 61] = (unsigned long long)clock64();
   }
-  // Every thread of this CTA is past its last use of the counts (the barrier above).  Where no wait ran out the second
-  // word's tag is there; the last CTA out takes the tags away.
-  if (tid == 0 && a.passes == 3 && a.sync.arrive(1, abort_sh == 0) == gridDim.x - 1) a.sync.words[0] = a.sync.words[1] = 0;
+  if (tid == 0 && a.passes == 3) a.sync.leave();     // every thread is past its last use of the counts (the barrier above)
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512u) : "memory");
@@ -908,12 +942,12 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   a.lag = kLagUnits / (per_phase > 0 ? per_phase : 1);
   if (a.lag > a.n_groups - 1) a.lag = a.n_groups - 1;
   if (a.lag < 1) a.lag = 1;
-  a.sync.words = sync;
-  a.sync.tag = next_launch_tag();
+  a.sync.word = sync;
+  a.sync.tag = next_launch_tag() & ((1ull << 40) - 1);
   const bool waits_inside = passes == 3;
   const int expire = waits_inside ? take_expire_next_wait() : 0;
   a.target = (unsigned)sh.n_cta + (expire == 1);
-  a.clear_target = (unsigned)sh.n_cta + (expire == 2);
+  a.sync.expect = (unsigned)sh.n_cta + (expire == 2);
   a.trace = tensor_trace_buffer(sh.n_cta);
   const size_t smem = (size_t)(kQTiles * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + kTail);
 
