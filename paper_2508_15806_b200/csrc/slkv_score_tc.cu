@@ -3,6 +3,8 @@
 // slkv_row_lse.
 #include <cuda.h>
 
+#include <atomic>
+
 #include "slkv_internal.cuh"
 #include "slkv_tc_device.cuh"
 
@@ -58,17 +60,17 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
+  static std::atomic<EncodeTiledFn> known{nullptr};             // several threads may be the first
+  EncodeTiledFn fn = known.load(std::memory_order_relaxed);
   if (!fn) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
+      known.store(fn = reinterpret_cast<EncodeTiledFn>(p), std::memory_order_relaxed);
   }
   return fn;
 }
-
 
 }  // namespace
 
