@@ -385,9 +385,10 @@ int slkv_compress_host(const slkv_params* p, const void* q_win, const void* k, c
  * only by synchronising the whole device and shrinking somebody else's pool, and torch's allocator is not
  * the caller's to use.  Such a caller still owns its inputs and outputs; what it lacks is scratch.
  *
- * The scratch is a fixed array of SLKV_NOALLOC_SCRATCH_BYTES inside the library's device image: every GPU
- * that loads the library holds that much memory until the process exits, used or not.  The call computes
- * exactly what slkv_score computes, with the same kernels and the same results.
+ * The scratch is a fixed array of SLKV_NOALLOC_SCRATCH_BYTES (and 10 KB for what the CTAs of a launch tell one
+ * another) inside the library's device image: every GPU that loads the library holds that much memory until the
+ * process exits, used or not.  The call computes exactly what slkv_score computes, with the same kernels and the
+ * same results.
  *   - Shapes whose slkv_workspace_bytes exceed the array are rejected with SLKV_ERR_WORKSPACE before anything
  *     is enqueued (32k tokens x 8 KV heads x 128 score rows needs about 5.3 MB).
  *   - The first call on each device looks up the array's device address (a CUDA runtime query, made with that

@@ -10,7 +10,9 @@
 
 namespace {
 
-constexpr size_t kScratchBytes = SLKV_NOALLOC_SCRATCH_BYTES;
+// What the CTAs of a launch tell one another comes on top of the documented bytes (but for the 256 that every workspace has
+// had for such words): it takes nothing from the shapes that fit them.
+constexpr size_t kScratchBytes = SLKV_NOALLOC_SCRATCH_BYTES + (slkv::kSyncBytes + 255) / 256 * 256 - 256;
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -41,7 +43,7 @@ thread_local int g_noalloc_cuda_error = 0;
 
 extern "C" {
 
-size_t slkv_noalloc_scratch_bytes(void) { return kScratchBytes; }
+size_t slkv_noalloc_scratch_bytes(void) { return SLKV_NOALLOC_SCRATCH_BYTES; }
 
 int slkv_noalloc_last_cuda_error(void) { return g_noalloc_cuda_error; }
 

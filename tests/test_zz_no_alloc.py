@@ -63,6 +63,30 @@ def test_fp32_path_too():
     P.assert_pooled_close(got, P.oracle_pooled(q, k, cu, 16, 5), cu, k.shape[1], 16)
 
 
+@pytest.mark.gpu
+def test_the_words_of_a_launch_take_nothing_from_the_array():
+    # what the CTAs of a launch tell one another has room beside the documented bytes: the longest sequence taken is the one
+    # whose workspace comes to them without those words
+    words = 10496
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev).manual_seed(4)
+    q = torch.randn(1, 16, 8, 64, generator=g, device=dev).bfloat16()
+    k = torch.randn(100000, 8, 64, generator=g, device=dev).bfloat16()
+    p = B.make_params(q, k, None, 16, 7)
+    lo, hi = 60000, 100000
+    while hi - lo > 1:                                   # the last length that fits
+        mid = (lo + hi) // 2
+        lo, hi = (mid, hi) if B.slkv_workspace_bytes(p, [0, mid]) <= B.slkv_noalloc_scratch_bytes() + words else (lo, mid)
+    assert B.slkv_workspace_bytes(p, [0, lo]) > B.slkv_noalloc_scratch_bytes()
+    cu_dev = torch.tensor([0, lo], dtype=torch.int32, device=dev)
+    ref, got = (torch.zeros(B.slkv_pooled_elems(p, [0, lo]), device=dev) for _ in range(2))
+    B.slkv_score(p, q, k, cu_dev, [0, lo], ref, B.new_workspace(p, [0, lo], dev))
+    B.slkv_score_noalloc(p, q, k, cu_dev, [0, lo], got)
+    assert torch.equal(got, ref)
+    with pytest.raises(B.SlkvError):
+        B.slkv_score_noalloc(p, q, k, cu_dev, [0, hi], got)
+
+
 def test_oversized_shapes_are_rejected_on_the_host():
     # decided before any CUDA call, so this runs without a GPU
     builder.build()
