@@ -64,3 +64,19 @@ def test_ties_zeros_and_orderings(n):
     period = lambda k: k[torch.arange(len(k), device=DEV) % 128]                                 # noqa: E731
     for fn in (same, far, sort, period):
         run([n], 3, 4, [300, n // 3, n - 7], 3, B.SLKV_POOL_MAX, k_fn=fn)
+
+
+@pytest.mark.parametrize("n", [2045, 2048, 2049, 4093, 4097, 8189, 8193, 16381, 16385])
+@pytest.mark.parametrize("many", [False, True])
+def test_edges_of_the_variants(n, many):
+    # few CTAs (an SM each), and more of them than SMs; a short sequence in between moves the segments off 16-byte boundaries
+    run(([n + 8] + [8 + 9] * 60 + [n + 8]) if many else [n + 8], 3, 8, [8 + max(1, n // 50), 8 + n // 2, 8 + n - 1], 7, B.SLKV_POOL_MAX)
+
+
+@pytest.mark.parametrize("n", [8192, 16000, 32768, 70000])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_a_sample_that_misleads(n, sign):
+    # every 16th (32nd) position is the one that is sampled: those positions high, or low, and the rest the other way
+    for step in (16, 32):
+        odd = lambda k: torch.where(torch.arange(len(k), device=DEV).view(-1, 1, 1) % step == step // 2, k * 0.05 + sign, k * 0.05 - sign)   # noqa: E731,B023
+        run([n + 4], 3, 4, [300, n // 4, n - n // 10], 1, B.SLKV_POOL_MAX, k_fn=odd)
