@@ -233,6 +233,12 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
   return SLKV_OK;
 }
 
+// CTAs per segment where one launch does the whole layer, else 0.  A wait that is to run out (slkv_debug_expire_next_wait) is one
+// of the kernels whose CTAs wait for words in memory; these have none.
+int layer_cluster(const Problem& pb, int path) {
+  return path == SLKV_PATH_TENSOR && !next_wait_expires() ? layer_tc_cluster(pb) : 0;
+}
+
 // ---- overlapped calls ---------------------------------------------------------------------------------------
 // A call queues its layer; a list of layers goes out as three launches on the caller's stream -- scores, selections,
 // gathers, each over all layers of the list -- when it is full (list_layers) or at a join.  What a list gives over single calls: the
@@ -488,6 +494,15 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   pb.cu = cu_dev; pb.q = q_win; pb.k = k; pb.v = v;
   pb.tab.cu_ptr = cu_dev;
   pb.lse_opt = lse_opt;
+  TailLayer tail = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
+  // One launch for the whole layer where that is quicker.  With pooled_opt the call takes the general path, launch by launch:
+  // that is a caller who looks into the steps, and how the two are held against each other on the same inputs.
+  if (const int cs = !kept_copy && !offsets_copy && !pooled_opt ? layer_cluster(pb, path) : 0) {
+    e = launch_layer_tc(pb, cs, &tail, nullptr, status, st, &launches);
+    if (e != cudaSuccess) return cuda_fail(e);
+    g_last_launches = launches;
+    return SLKV_OK;
+  }
   const bool one_kernel = select_list_supported(pb) || select_cluster_supported(pb);
   if (!one_kernel || pb.tab.n_inline == 0) {       // tables in global memory and / or the packed offsets
     e = launch_setup(pb, one_kernel ? nullptr : budgets, offsets, capacity, status, st, &launches);
@@ -495,7 +510,6 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   }
   rc = enqueue_votes(pb, path, cu_host, status, st, &launches);
   if (rc != SLKV_OK) return rc;
-  TailLayer tail = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
   tail.kept_copy = kept_copy;
   tail.offsets_copy = offsets_copy;
   if (one_kernel) {
@@ -593,7 +607,7 @@ int slkv_profile_collect(float* total_ms, int32_t* launches, int32_t n_kernels) 
 const char* slkv_kernel_name(int kernel_id) {
   static const char* names[KID_COUNT] = {"k_setup", "k_score_lse", "k_score_vote", "k_pool", "k_select",
                                          "k_gather", "k_alloc", "k_score_fused", "k_score_list", "k_window_stats",
-                                         "k_merge_lse", "k_behavior", "k_cp"};
+                                         "k_merge_lse", "k_behavior", "k_cp", "k_layer"};
   return (kernel_id >= 0 && kernel_id < KID_COUNT) ? names[kernel_id] : "";
 }
 
@@ -912,6 +926,12 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
     e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_seqlens_host, status, 1, lse_out, st, &launches)
                                  : launch_score_simt(pb, status, 1, st, &launches);
     if (e == cudaSuccess && path != SLKV_PATH_TENSOR) e = launch_merge_lse_simt(pb, lse_out, st, &launches);
+    if (e != cudaSuccess) return cuda_fail(e);
+    g_last_launches = launches;
+    return SLKV_OK;
+  }
+  if (const int cs = layer_cluster(pb, path)) {
+    e = launch_layer_tc(pb, cs, nullptr, pooled, status, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
     g_last_launches = launches;
     return SLKV_OK;

@@ -131,7 +131,7 @@ struct Problem {
 };
 
 // kernel ids for launch accounting / per-kernel timing
-enum KernelId { KID_SETUP = 0, KID_SCORE_LSE, KID_SCORE_VOTE, KID_POOL, KID_SELECT, KID_GATHER, KID_ALLOC, KID_SCORE_FUSED, KID_SCORE_LIST, KID_WINDOW_STATS, KID_MERGE_LSE, KID_BEHAVIOR, KID_CP, KID_COUNT };
+enum KernelId { KID_SETUP = 0, KID_SCORE_LSE, KID_SCORE_VOTE, KID_POOL, KID_SELECT, KID_GATHER, KID_ALLOC, KID_SCORE_FUSED, KID_SCORE_LIST, KID_WINDOW_STATS, KID_MERGE_LSE, KID_BEHAVIOR, KID_CP, KID_LAYER, KID_COUNT };
 
 // Brackets one kernel launch: counts it and, when per-kernel timing is on for this thread, records a
 // CUDA event pair around it on the launch stream.
@@ -280,10 +280,16 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
 // lse_out null: into the layer's own statistics area
 cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
                                     cudaStream_t st, int* launches);
+// ---- a whole layer in one launch (slkv_layer_tc.cu) ----------------------------------------------------------------
+// CTAs per segment, or 0 where the shape is not taken; tail null: the pooled scores alone.  pooled may be null with a tail.
+int layer_tc_cluster(const Problem& pb);
+cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,
+                            int* launches);
 // Timeline buffer of this thread (diagnostics), or null: kTraceSlots words per CTA.
 unsigned long long* tensor_trace_buffer(int n_cta);
 // Diagnostics: arm / consume the one-shot switch that makes the next inter-CTA wait of this thread's launches run out.
 void expire_next_wait(int on);
 int take_expire_next_wait();
+bool next_wait_expires();                        // armed
 
 }  // namespace slkv

@@ -13,6 +13,7 @@
 // What bounds it: latency at the small sizes (1024 tokens, 8 heads, 16 rows: two dot-product loops of one thread per key and
 // two launches took 80 us, this takes 10), the FMA pipe at the large ones.
 #include "slkv_internal.cuh"
+#include "slkv_fma_device.cuh"
 
 namespace slkv {
 namespace {
@@ -25,29 +26,6 @@ constexpr unsigned long long kWaitLimitNs = 1000ull * 1000ull * 1000ull;
 
 // stages of a launch
 enum { kStats = 1, kMaxima = 2, kFarSums = 4, kVotes = 8 };
-
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ float sum_of(f32x2 v) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-  return a + b;
-}
-
-__device__ __forceinline__ void unpack(const uint4& u, float (&f)[4], float) {
-  f[0] = __uint_as_float(u.x); f[1] = __uint_as_float(u.y); f[2] = __uint_as_float(u.z); f[3] = __uint_as_float(u.w);
-}
-__device__ __forceinline__ void unpack(const uint4& u, float (&f)[8], __nv_bfloat16) {
-  // a bf16 is the high half of an fp32
-  f[0] = __uint_as_float(u.x << 16); f[1] = __uint_as_float(u.x & 0xffff0000u);
-  f[2] = __uint_as_float(u.y << 16); f[3] = __uint_as_float(u.y & 0xffff0000u);
-  f[4] = __uint_as_float(u.z << 16); f[5] = __uint_as_float(u.z & 0xffff0000u);
-  f[6] = __uint_as_float(u.w << 16); f[7] = __uint_as_float(u.w & 0xffff0000u);
-}
 
 // The statistics area (pb.part): per segment and row the fp64 sum, then the same over relative to the row's maximum, then
 // the maxima (order-preserving integers), then one word: some sum over- or underflowed.  Cleared before use.
@@ -436,83 +414,23 @@ k_score_simt(const __grid_constant__ SimtArgs a) {
 }
 
 // Row statistics over the window keys a window row sees causally (its own position and the window keys before it).
-// Only the all-causal softmax domain needs them.  A CTA takes 16 rows of a segment; key blocks of 32 in shared memory, a
-// lane per key, a warp per four rows.  (One thread per row walking the keys by itself, one CTA per segment, took 24 us for
-// 8 segments of 128 rows and 32 window keys; this takes 4.)
-constexpr int kWinRows = 16;
+// Only the all-causal softmax domain needs them.  A CTA takes 16 rows of a segment (window_rows).  (One thread per row walking
+// the keys by itself, one CTA per segment, took 24 us for 8 segments of 128 rows and 32 window keys; this takes 4.)
 template <typename T, int D>
 __global__ void __launch_bounds__(128)
-k_window_stats(const T* __restrict__ q, const T* __restrict__ k, const __grid_constant__ SeqTables tab,
-               float* __restrict__ win_m, float* __restrict__ win_z, int n_kv_heads, int G, int window, int head_inner,
-               long long k_stride_tok, long long k_stride_head, long long q_stride_seq, long long q_stride_row,
-               long long q_stride_head, float scale_log2) {
-  constexpr int kVec = 16 / sizeof(T), kPitch = D + 4, kPerRow = D / kVec;
-  __shared__ __align__(16) float ks[32 * kPitch], qs[kWinRows * kPitch];
+k_window_stats(const WindowArgs a, const __grid_constant__ SeqTables tab, float* __restrict__ win_m, float* __restrict__ win_z) {
+  __shared__ __align__(16) float sh[window_floats(D)];
   pdl_launch_dependents();
   pdl_wait();
-  const int seg = blockIdx.x, s = seg / n_kv_heads, g = seg - s * n_kv_heads;
+  const int seg = blockIdx.x, s = seg / a.n_kv_heads, g = seg - s * a.n_kv_heads;
   const int t0 = tab.cu_at(s);
-  const int n_hist = tab.cu_at(s + 1) - t0 - window;
+  const int n_hist = tab.cu_at(s + 1) - t0 - a.window;
   if (n_hist <= 0) return;                                     // no history: nothing is scored
-  const int R = G * window, row0 = blockIdx.y * kWinRows, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  auto window_row = [&](int r) { return head_inner ? r / G : r % window; };
-  auto query_head = [&](int r) { return g * G + (head_inner ? r % G : r / window); };
-  auto load = [&](float* dst, const T* src) {
-    float f[kVec];
-    unpack(*reinterpret_cast<const uint4*>(src), f, T());
-#pragma unroll
-    for (int e = 0; e < kVec; e += 4) *reinterpret_cast<float4*>(dst + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
-  };
-  int last = 0;                                                // the last key any of the rows sees
-  for (int r = row0; r < min(row0 + kWinRows, R); ++r) last = max(last, window_row(r));
-  for (int i = tid; i < kWinRows * kPerRow; i += 128) {
-    const int rr = i / kPerRow, c = (i - rr * kPerRow) * kVec, r = min(row0 + rr, R - 1);
-    load(qs + rr * kPitch + c, q + s * q_stride_seq + window_row(r) * q_stride_row + (long long)query_head(r) * q_stride_head + c);
-  }
-  float m[4], z[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) { m[u] = -INFINITY; z[u] = 0.f; }
-  for (int j0 = 0; j0 <= last; j0 += 32) {
-    __syncthreads();
-    for (int i = tid; i < 32 * kPerRow; i += 128) {
-      const int jj = i / kPerRow, c = (i - jj * kPerRow) * kVec, j = min(j0 + jj, window - 1);
-      load(ks + jj * kPitch + c, k + (long long)(t0 + n_hist + j) * k_stride_tok + (long long)g * k_stride_head + c);
-    }
-    __syncthreads();
-    f32x2 acc[4] = {0, 0, 0, 0};
-#pragma unroll 4
-    for (int c = 0; c < D; c += 4) {
-      const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(ks + lane * kPitch + c);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(qs + (warp * 4 + u) * kPitch + c);
-        acc[u] = fma2(kv.x, qv.x, acc[u]);
-        acc[u] = fma2(kv.y, qv.y, acc[u]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = min(row0 + warp * 4 + u, R - 1);
-      const bool seen = j0 + lane <= window_row(r);
-      const float x = sum_of(acc[u]) * scale_log2;
-      float mx = seen ? x : -INFINITY;
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (!(mx > -INFINITY)) continue;                         // the row sees none of these keys (uniform over the warp)
-      const float mn = fmaxf(m[u], mx);
-      float e = seen ? exp2f(x - mn) : 0.f;
-      for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-      z[u] = z[u] * exp2f(m[u] - mn) + e;                      // exp2f(-inf) = 0 covers the first block
-      m[u] = mn;
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = row0 + warp * 4 + u;
-    if (lane == 0 && r < R) {
-      win_m[(long long)seg * R + r] = m[u];
-      win_z[(long long)seg * R + r] = z[u];
-    }
-  }
+  const int R = a.G * a.window;
+  window_rows<T, D, 0>(a, sh, threadIdx.x, s, g, t0 + n_hist, blockIdx.y * kWinRows, [&](int r, float m, float z) {
+    win_m[(long long)seg * R + r] = m;
+    win_z[(long long)seg * R + r] = z;
+  });
 }
 
 // lse_out[s][h][i] from the row sums (and the window statistics, if any).
@@ -628,12 +546,9 @@ cudaError_t launch_passes(const Problem& pb, int32_t* status, int passes, cudaSt
 
 template <typename T, int D>
 cudaError_t launch_window(const Problem& pb, bool head_inner, cudaStream_t st, int* launches) {
-  const slkv_params& p = pb.p;
   LaunchScope scope(KID_WINDOW_STATS, st, launches);
   return launch_pdl(k_window_stats<T, D>, dim3(pb.n_seg, (pb.R + kWinRows - 1) / kWinRows), dim3(128), 0, st, 1,
-                    (const T*)pb.q, (const T*)pb.k, pb.tab, pb.win_m, pb.win_z, p.n_kv_heads, pb.G, p.window,
-                    head_inner ? 1 : 0, (long long)p.k_stride_tok, (long long)p.k_stride_head, (long long)p.q_stride_seq,
-                    (long long)p.q_stride_row, (long long)p.q_stride_head, kLog2e / sqrtf((float)p.head_dim));
+                    window_args(pb, head_inner), pb.tab, pb.win_m, pb.win_z);
 }
 
 }  // namespace

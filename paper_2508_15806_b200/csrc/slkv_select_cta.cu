@@ -14,11 +14,7 @@
 // the k-th largest by 128 ranked samples and a descent over the bracket took as many steps again, and its loops an atomic
 // with a result per score: whole layers of 8 segments 21.7 -> 16.9 us at 1024 positions, 26.4 -> 22.7 at 4096, 29.9 -> 26.4 at
 // 8192, 33.7 -> 30.7 at 12000, 32 layers of 4001 129.5 -> 118 (all in a graph).
-#include <cooperative_groups.h>
-
-#include "slkv_internal.cuh"
-
-namespace cg = cooperative_groups;
+#include "slkv_select_device.cuh"
 
 namespace slkv {
 namespace {
@@ -27,22 +23,6 @@ constexpr int kMaxThreads = 1024;
 constexpr int kMaxItems = 32;                         // consecutive positions per thread
 constexpr int kMaxSlice = kMaxThreads * kMaxItems;    // 32768 positions per CTA
 constexpr int kMaxCluster = 8;
-constexpr int kMaxRadius = 4;                         // pool_kernel <= 9: four values on either side are enough
-constexpr int kBins = 2048;
-constexpr unsigned kAll = 0xffffffffu;
-// First level's bins: 64 to an octave from 2^-24 up to 2^8 (a vote is at most the window, 256), the scores below in bin 0,
-// whatever lies above in the last.
-constexpr unsigned kFloorBits = (127u - 24u) << 23;
-constexpr int kFirstShift = 17;
-__device__ __forceinline__ unsigned first_bin(unsigned v) {
-  const unsigned base = kFloorBits - (1u << kFirstShift);
-  return min((max(v, base) - base) >> kFirstShift, kBins - 1u);
-}
-// Shared memory of the votes: a thread's positions are `items` floats, then four unused ones -- the pitch makes the 16-byte
-// accesses of neighbouring threads conflict-free -- behind eight floats that hold the four before the first.
-constexpr int kLead = 8;
-template <int IT> constexpr int kLogItems = IT == 8 ? 3 : (IT == 16 ? 4 : 5);
-constexpr int vote_floats(int threads, int items) { return kLead + (threads + 1) * (items + 4); }
 
 struct SelArgs {
   SeqTables tab;
@@ -50,57 +30,18 @@ struct SelArgs {
   TailLayer lay[kListMaxLayers];
 };
 
-__device__ __forceinline__ int kept_rows(int len, int budget, int window) { return min(len, max(budget, window)); }
-
-// Pooled values at x[4 .. 11] of 16 consecutive votes.
-template <int RAD>
-__device__ __forceinline__ void pool8(const float (&x)[16], bool max_mode, float (&y)[8]) {
-  constexpr int W = 2 * RAD + 1, F = 4 - RAD;          // window of y[e]: x[F + e .. F + e + W - 1]
-  if (max_mode) {
-    float m[16];
-    int have = 1;                                      // m[i] = max of x[i .. i + have - 1]
-#pragma unroll
-    for (int i = 0; i < 16; ++i) m[i] = x[i];
-#pragma unroll
-    for (int step = 1; 2 * step <= W; step *= 2) {
-#pragma unroll
-      for (int i = F; i + step < 16; ++i) m[i] = fmaxf(m[i], m[i + step]);
-      have = 2 * step;
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) y[e] = have < W ? fmaxf(m[F + e], m[F + e + W - have]) : m[F + e];
-  } else {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      float acc = x[F + e];
-#pragma unroll
-      for (int t = 1; t < W; ++t) acc += x[F + e + t];
-      y[e] = acc / (float)W;
-    }
-  }
-}
-
 // T threads with IT consecutive positions each.  CLUSTER: a segment is shared by the CTAs of a cluster (else every pointer
 // below is known to be this CTA's own memory).
 template <int T, int IT, int RAD, bool CLUSTER>
 __global__ void __launch_bounds__(T, T == 1024 ? 1 : 1024 / T)
 k_select_list(const __grid_constant__ SelArgs args) {
-  constexpr int kWarps = T / 32, kPitch = IT + 4, kPer = kBins / T;     // bins per thread
-  constexpr int kList = 512;
-  constexpr bool kSample = IT > 8;
+  constexpr int kWarps = T / 32, kPitch = IT + 4, kPer = kBins / T;
   extern __shared__ __align__(16) float votes_sh[];
-  __shared__ __align__(16) int hist[kBins + 1];        // the last one: places that do not count
-  __shared__ __align__(16) int sample[kSample ? kBins : 2];
-  __shared__ __align__(16) unsigned list[kList];
-  __shared__ unsigned wsum[3][32];
-  __shared__ int2 cta_tot;                              // read by the cluster's other CTAs
-  __shared__ unsigned sh_tau, sh_bin, sh_n;
-  __shared__ int sh_above, sh_m, sh_need;
+  __shared__ SelShared sh;
 
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = CLUSTER ? (int)cluster.num_blocks() : 1, rank = CLUSTER ? (int)cluster.block_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  auto sync_all = [&]() { if (CLUSTER) cluster.sync(); else __syncthreads(); };
   pdl_launch_dependents();
   const TailLayer& a = args.lay[blockIdx.y];
   const int seg = blockIdx.x / CS, s = seg / args.n_kv_heads, h = seg - s * args.n_kv_heads;
@@ -125,11 +66,11 @@ k_select_list(const __grid_constant__ SelArgs args) {
   int32_t* const gather_src = a.gather_src;
   float* const pooled_out = a.pooled_out;
   asm volatile("" ::"l"(capacity), "l"(kept_idx), "l"(gather_src), "l"(pooled_out), "l"(a.offsets));
-  if (tid == 0) sh_n = 0;
+  if (tid == 0) sh.n_list = 0;
 #pragma unroll
   for (int i = 0; i < kPer; i += 2) {
-    reinterpret_cast<int2*>(hist)[(tid * kPer + i) / 2] = make_int2(0, 0);
-    if (kSample) reinterpret_cast<int2*>(sample)[(tid * kPer + i) / 2] = make_int2(0, 0);
+    reinterpret_cast<int2*>(sh.hist)[(tid * kPer + i) / 2] = make_int2(0, 0);
+    reinterpret_cast<int2*>(sh.sample)[(tid * kPer + i) / 2] = make_int2(0, 0);
   }
   pdl_wait();                                           // budgets and votes may come from the kernels before this one
 
@@ -153,14 +94,14 @@ k_select_list(const __grid_constant__ SelArgs args) {
       part += (unsigned)kept_rows(args.tab.cu_at(s2 + 1) - args.tab.cu_at(s2), a.budgets[h2], args.window);
     }
     part = __reduce_add_sync(kAll, part);
-    if (lane == 0) wsum[0][wid] = part;
+    if (lane == 0) sh.wsum[0][wid] = part;
   }
   const int k_keep = kept_rows(len, budget, args.window) - n_win;             // C_H = C - window, clamped
   const bool choose = k_keep > 0 && k_keep < n;
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   // packed row where this segment starts = kept rows of all earlier segments (Algorithm 3 l.1-4 per head)
-  const long long out0 = __reduce_add_sync(kAll, lane < kWarps ? wsum[0][lane] : 0u);
+  const long long out0 = __reduce_add_sync(kAll, lane < kWarps ? sh.wsum[0][lane] : 0u);
   const int src_base = t0 * args.n_kv_heads + h;         // source row of position j: src_base + j * n_kv_heads
   auto put = [&](long long o, int position) {
     if (o < capacity) {
@@ -193,254 +134,24 @@ k_select_list(const __grid_constant__ SelArgs args) {
   if (mine) {
     const int p0 = base + i0, v_lo = max(-p0, 0), v_hi = min(my_end - p0, IT);            // valid places of the thread
     valid = (v_hi >= 32 ? kAll : (1u << max(v_hi, 0)) - 1u) & (v_lo >= 32 ? 0u : kAll << v_lo);
-    const float* src = votes + tid * kPitch;
-    float x[16];
-    auto load4 = [&](const float* f, int k) {
-      const float4 v = *reinterpret_cast<const float4*>(f);
-      x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
-    };
-    load4(votes + at(i0 - 4), 8);
-    load4(src, 12);
-#pragma unroll
-    for (int g = 0; g < IT / 8; ++g) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) x[k] = x[k + 8];
-      load4(src + 8 * g + 4, 8);
-      load4(8 * g + 8 < IT ? src + 8 * g + 8 : src + kPitch, 12);          // the next thread's first four
-      float y[8];
-      pool8<RAD>(x, max_mode, y);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) key[8 * g + e] = __float_as_uint(y[e]);
-    }
-    if (pooled_out) {
-      float* dst = pooled_out + seg_base + p0;           // 16-byte aligned where the array is
-      const bool wide = (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
-#pragma unroll
-      for (int g = 0; g < IT; g += 4) {
-        if (wide && (valid >> g & 15u) == 15u) {
-          *reinterpret_cast<uint4*>(dst + g) = make_uint4(key[g], key[g + 1], key[g + 2], key[g + 3]);
-        } else {
-#pragma unroll
-          for (int e = g; e < g + 4; ++e)
-            if (valid >> e & 1u) dst[e] = __uint_as_float(key[e]);
-        }
-      }
-    }
+    pool_places<RAD>(votes + tid * kPitch, votes + at(i0 - 4), max_mode, key);
+    if (pooled_out) store_scores(pooled_out + seg_base + p0, key, valid);
   }
   if (!choose) return;
 
-  // ---- the k-th largest by histograms.  bin_of: the bin that holds the `want` largest score of `bins` (more than that are
-  // counted there), how many lie above it and in it; with no such bin, sh_bin = kBins.
-  auto bin_of = [&](int* bins, int want) {
-    if (tid == 0) sh_bin = kBins;
-    int c[kPer], sum = 0;
-#pragma unroll
-    for (int i = 0; i < kPer; i += 2) {
-      int2 v = reinterpret_cast<const int2*>(bins)[(tid * kPer + i) / 2];
-      if (CLUSTER)
-        for (int o = 1; o < CS; ++o) {
-          const int2 w = reinterpret_cast<const int2*>(cluster.map_shared_rank(bins, (rank + o) % CS))[(tid * kPer + i) / 2];
-          v.x += w.x;
-          v.y += w.y;
-        }
-      c[i] = v.x;
-      c[i + 1] = v.y;
-      sum += v.x + v.y;
-    }
-    const int warp_sum = (int)__reduce_add_sync(kAll, (unsigned)sum);
-    if (lane == 0) wsum[1][wid] = (unsigned)warp_sum;
-    __syncthreads();
-    const int above_w = (int)__reduce_add_sync(kAll, lane > wid && lane < kWarps ? wsum[1][lane] : 0u);
-    if (above_w < want && want <= above_w + warp_sum) {   // the bin is one of this warp's
-      int inc = sum;                                      // suffix sum over the lanes
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_down_sync(kAll, inc, o);
-        if (lane + o < 32) inc += v;
-      }
-      int above = above_w + inc - sum;
-#pragma unroll
-      for (int i = kPer - 1; i >= 0; --i) {
-        if (above < want && want <= above + c[i]) { sh_bin = kPer * tid + i; sh_above = above; sh_m = c[i]; }
-        above += c[i];
-      }
-    }
-    sync_all();                                           // in a cluster also: nobody reads the others' bins any more
-  };
-  // Long slices: one place in IT is counted first.  Of these, the rank that the k-th largest has among them, plus four
-  // standard deviations, bounds it from below, and only the scores above that bound are counted (an atomic on shared memory
-  // takes seven cycles of the SM per warp, whether one lane adds or 32).
-  unsigned bound = 0;
-  uint4* const shelf = reinterpret_cast<uint4*>(votes + tid * kPitch);
-  if (kSample) {
-    if (mine && valid >> (IT / 2) & 1u) atomicAdd(&sample[first_bin(key[IT / 2])], 1);
-    sync_all();                                          // everybody has read the votes, too: the scores take their places
-    if (mine)
-#pragma unroll
-      for (int g = 0; g < IT; g += 4) shelf[g / 4] = make_uint4(key[g], key[g + 1], key[g + 2], key[g + 3]);
-    const float f = __fdividef((float)k_keep, (float)n), q = f * (float)(n / IT);
-    bin_of(sample, (int)(q + 4.f * sqrtf(q * (1.f - f))) + 2);
-    const unsigned bin = sh_bin;
-    if (bin > 0 && bin < (unsigned)kBins) bound = kFloorBits + ((bin - 1) << kFirstShift);
-  }
-  // f(e, score) for the thread's places
-  auto each = [&](auto f) {
-#pragma unroll
-    for (int g = 0; g < IT; g += 4) {
-      const uint4 v = kSample ? shelf[g / 4] : make_uint4(key[g], key[g + 1], key[g + 2], key[g + 3]);
-      f(g, v.x); f(g + 1, v.y); f(g + 2, v.z); f(g + 3, v.w);
-    }
-  };
-  int need = k_keep;
-  unsigned lo = 0, hi = kAll, gt = 0, cand = valid, tau;
-  int sh = kFirstShift;
-  bool first = true;
-  while (true) {
-    auto index = [&](unsigned v) { return (int)(first ? first_bin(v) : min((v - lo) >> sh, kBins - 1u)); };
-    // equal neighbours are added at once: a maximum holds for up to pool_kernel positions
-    if (kSample && mine) {
-      unsigned ends = 0, counted = 0, next = 0;           // places whose right neighbour's score is another; those that count
-      each([&](int e, unsigned v) {
-        if (e > 0) ends |= v != next ? 1u << (e - 1) : 0u;
-        counted |= v >= bound ? 1u << e : 0u;
-        next = v;
-      });
-      counted &= cand;
-      ends = (ends | ~(counted >> 1)) & counted;
-      const unsigned* keys = reinterpret_cast<const unsigned*>(shelf);
-      int from = -1;                                      // the last place before the run
-      for (unsigned m = ends, c = counted; m != 0; m &= m - 1) {
-        const int e = __ffs(m) - 1;
-        from = __ffs(c) - 2;
-        atomicAdd(&hist[index(keys[e])], e - from);
-        c &= e == 31 ? 0u : kAll << (e + 1);
-      }
-    } else if (mine) {
-      int bin = kBins, run = 0;
-      each([&](int e, unsigned v) {
-        const int b = cand >> e & 1u ? index(v) : kBins;
-        if (e > 0 && b != bin) { atomicAdd(&hist[bin], run); run = 0; }
-        bin = b;
-        ++run;
-      });
-      atomicAdd(&hist[bin], run);
-    }
-    sync_all();
-    bin_of(hist, need);
-    const unsigned bin = sh_bin;
-    if (kSample && bin == (unsigned)kBins) {              // the bound was too high: everything counts
-      bound = 0;
-#pragma unroll
-      for (int i = 0; i < kPer; i += 2) reinterpret_cast<int2*>(hist)[(tid * kPer + i) / 2] = make_int2(0, 0);
-      __syncthreads();
-      continue;
-    }
-    const int m_bin = sh_m;
-    need -= sh_above;
-    if (first) {
-      if (bin > 0) lo = kFloorBits + ((bin - 1) << kFirstShift);
-      if (bin < kBins - 1u) hi = kFloorBits + (bin << kFirstShift) - 1u;
-    } else {
-      lo += bin << sh;
-      if (bin < kBins - 1u) hi = min(hi, lo + ((1u << sh) - 1u));
-    }
-    first = false;
-    // the bin's scores go on; where they fit, in a list of the cluster's first CTA (their order does not matter)
-    const bool listed = m_bin <= kList && lo != hi;
-    if (mine) {
-      unsigned in_bin = 0;
-      each([&](int e, unsigned v) {
-        const unsigned bit = cand & 1u << e;
-        gt |= v > hi ? bit : 0u;
-        in_bin |= v >= lo && v <= hi ? bit : 0u;
-      });
-      cand = in_bin;
-      if (listed && in_bin) {
-        unsigned* dst = (CLUSTER ? cluster.map_shared_rank(list, 0) : list) +
-                        atomicAdd(CLUSTER ? cluster.map_shared_rank(&sh_n, 0) : &sh_n, (unsigned)__popc(in_bin));
-        if (kSample) {
-          const unsigned* keys = reinterpret_cast<const unsigned*>(shelf);
-          for (unsigned m = in_bin; m != 0; m &= m - 1) *dst++ = keys[__ffs(m) - 1];
-        } else {
-          each([&](int e, unsigned v) { if (in_bin >> e & 1u) *dst++ = v; });
-        }
-      }
-    }
-    if (lo == hi) { tau = lo; break; }
-    if (listed) {                                         // ranked by counting
-      sync_all();
-      if (CLUSTER && rank > 0) {
-        const unsigned* list0 = cluster.map_shared_rank(list, 0);
-        for (int i = tid; i < m_bin; i += T) list[i] = list0[i];
-        __syncthreads();
-      }
-      int log_p = 5;                                      // 2^log_p lanes per score
-      while ((m_bin << log_p) > T) --log_p;
-      const int i = tid >> log_p, P = 1 << log_p, part = tid & (P - 1);
-      if (wid << 5 >> log_p < m_bin) {                    // some score for this warp
-        const unsigned x = list[min(i, m_bin - 1)];
-        int above = 0, at_least = 0;
-        for (int j = part; j < m_bin; j += P) { const unsigned y = list[j]; above += y > x; at_least += y >= x; }
-        for (int o = 1; o < P; o <<= 1) {
-          above += __shfl_xor_sync(kAll, above, o);
-          at_least += __shfl_xor_sync(kAll, at_least, o);
-        }
-        if (i < m_bin && part == 0 && above < need && need <= at_least) { sh_tau = x; sh_need = need - above; }
-      }
-      __syncthreads();
-      tau = sh_tau;
-      need = sh_need;
-      break;
-    }
-    const unsigned span = hi - lo;
-    sh = span < (unsigned)kBins ? 0 : 21 - __clz(span);
-    bound = lo;
-#pragma unroll
-    for (int i = 0; i < kPer; i += 2) reinterpret_cast<int2*>(hist)[(tid * kPer + i) / 2] = make_int2(0, 0);
-    __syncthreads();
-  }
-
-  // ---- ordered compaction: the scores above tau, and the first `need` equal to it; threads own consecutive positions
-  unsigned eq = 0;
-  if (mine)
-    each([&](int e, unsigned v) {
-      const unsigned bit = cand & 1u << e;
-      gt |= v > tau ? bit : 0u;
-      eq |= v == tau ? bit : 0u;
-    });
-  const unsigned cnt = (unsigned)__popc(gt) | ((unsigned)__popc(eq) << 16);
-  unsigned inc = cnt;                                     // both totals are <= 32768
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned x = __shfl_up_sync(kAll, inc, o);
-    if (lane >= o) inc += x;
-  }
-  if (lane == 31) wsum[2][wid] = inc;
-  __syncthreads();
-  const unsigned before = __reduce_add_sync(kAll, lane < wid ? wsum[2][lane] : 0u) + inc - cnt;
-  int gt_before = (int)(before & 0xffffu), eq_before = (int)(before >> 16);
-  if (CLUSTER) {
-    if (tid == T - 1) cta_tot = make_int2(gt_before + __popc(gt), eq_before + __popc(eq));
-    cluster.sync();
-    int2 o = make_int2(0, 0);
-    if (lane < rank) o = *cluster.map_shared_rank(&cta_tot, lane);
-    gt_before += (int)__reduce_add_sync(kAll, (unsigned)o.x);
-    eq_before += (int)__reduce_add_sync(kAll, (unsigned)o.y);
-  }
-  // of the thread's scores equal to tau, the first `take`
-  const int take = min(max(need - eq_before, 0), __popc(eq));
-  unsigned kept = gt;
-  for (int t = 0; t < take; ++t) { kept |= eq & (0u - eq); eq &= eq - 1; }
+  // (0: a barrier of all T threads)
+  int o_mine;
+  const unsigned kept = select_places<T, IT, CLUSTER, 0>(sh, tid, key, valid, mine, reinterpret_cast<uint4*>(votes + tid * kPitch), n,
+                                                         k_keep, rank, CS, o_mine);
   // the kept positions, in shared memory first (where the votes were): whole lines then go out
   int* const stage = reinterpret_cast<int*>(votes_sh);
-  const int o_mine = gt_before + min(eq_before, need);
   int o0 = 0, o1 = k_keep;                                 // the CTA's rows among the segment's
   if (CLUSTER) {
-    if (tid == 0) sh_above = o_mine;
-    if (tid == T - 1) sh_m = o_mine + __popc(kept);
+    if (tid == 0) sh.above = o_mine;
+    if (tid == T - 1) sh.m = o_mine + __popc(kept);
     __syncthreads();
-    o0 = sh_above;
-    o1 = sh_m;
+    o0 = sh.above;
+    o1 = sh.m;
   }
   int* dst = stage + (o_mine - o0);
   for (unsigned m = kept; m != 0; m &= m - 1) *dst++ = base + i0 + __ffs(m) - 1;

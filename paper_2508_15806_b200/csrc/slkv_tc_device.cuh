@@ -5,6 +5,7 @@
 #include <cuda.h>
 
 #include "slkv_internal.cuh"
+#include "slkv_fma_device.cuh"
 
 namespace slkv {
 
@@ -73,6 +74,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
+}
 // policy: L2 eviction policy (from createpolicy) for the lines the load touches
 __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar,
                                                  uint64_t policy) {
@@ -116,7 +122,6 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 // Pairs of fp32 values in one 64-bit register: fma / add on both with one instruction.
-typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float a, float b) {
   f32x2 r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -124,11 +129,6 @@ __device__ __forceinline__ f32x2 pack2(float a, float b) {
 }
 __device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
 }
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   f32x2 r;
@@ -315,6 +315,143 @@ __device__ __forceinline__ void tile_stats_exact(uint32_t tcol, float sc, int fi
     for (int e = 0; e < 8; ++e)
       if (any && c0 + e < n_valid) z += ex2(fmaf(__uint_as_float(r[e]), sc, -m));
   }
+}
+
+// ---- the epilogue warps' arithmetic on accumulators --------------------------------------------------------------------
+// sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials go
+// to the FMA pipe, where it takes fourteen instructions instead of two.  By cycles alone two pairs of eight would go there;
+// at the power limit the instructions cost more clock than they save cycles (32 layers of 32k / 128k positions, in both
+// passes no pair of a chunk's eight on the FMA pipe 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: one pair of eight
+// in the statistics, in the votes one in every other chunk.
+// The loops around this are kept small, the statistics' one chunk at a time with the last keys of a segment outside: four
+// warps on a scheduler hide a TMEM load's latency, and the epilogue warps are spread over both passes' loops, which have to
+// stay in the instruction cache (4k positions: statistics loop unrolled four times 154 us, twice 144, two chunks with the
+// last keys masked inside 140.9, as it is 140.1; 128k: 6147, 5865, 5868, 5820).
+template <bool STATS, bool POLY>
+__device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 off, uint32_t off_sh, f32x2& s0,
+                                          f32x2& s1) {
+#pragma unroll
+  for (int e = 0; e < 16; e += 4) {
+    f32x2 o0 = off, o1 = off;
+    if (!STATS) {
+      // an explicit shared-memory load: a generic one takes another path
+      asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(o0), "=l"(o1) : "r"(off_sh + 4u * e));
+    }
+    const f32x2 x0 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, o0);
+    const f32x2 x1 = fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sc2, o1);
+    s0 = add2(s0, POLY && e == 0 ? ex2_pair_poly<STATS>(x0) : ex2_pair(x0));
+    s1 = add2(s1, ex2_pair(x1));
+  }
+}
+
+// An epilogue thread's unit.
+struct Unit {
+  uint32_t tcol;               // its TMEM lane and its warpgroup's unit
+  uint32_t full, empty;        // the unit's mbarriers
+  volatile int* abort_flag;
+};
+__device__ __forceinline__ bool unit_wait(const Unit& u, int nth) {
+  const bool ok = mbar_wait(u.full, nth & 1, u.abort_flag);
+  if (!__all_sync(0xffffffffu, ok)) return false;                        // the TMEM loads need the whole warp
+  tc_fence_after();
+  return true;
+}
+__device__ __forceinline__ void unit_release(const Unit& u) {
+  tc_fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(u.empty);
+}
+
+// Statistics of one run for this thread's query row: tiles i0, i0 + every, ... < count.  z: the sum of 2^score, without a
+// reference; (far_z, far_m): what of it fp64 cannot hold (see StatView).  A tile is summed in fp32, without a reference
+// either as long as nothing overflows and not everything underflows; one whose sum is not finite and above kTinySum is
+// redone exactly.  false: a wait ran out.
+__device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i0, int every, int count, int n_valid0,
+                                          bool rows_here, double& z, float& far_z, float& far_m) {
+  z = 0.0;
+  far_z = far_m = 0.f;
+  const f32x2 sc2 = pack2(sc, sc);
+#pragma unroll 1
+  for (int i = i0; i < count; i += every, ++nth) {
+    if (!unit_wait(u, nth)) return false;
+    if (rows_here) {
+      const int n_valid = n_valid0 - i * kTileKeys;
+      const int whole = n_valid < kTileKeys ? n_valid & ~15 : kTileKeys;
+      f32x2 s0 = 0, s1 = 0;
+#pragma unroll 1
+      for (int c0 = 0; c0 < whole; c0 += 16) {
+        uint32_t v[16];
+        tc_ld16_issue(u.tcol + c0, v);
+        tc_ld_wait(v);
+        exp_chunk<true, true>(v, sc2, 0, 0u, s0, s1);
+      }
+      float tile = sum2(s0, s1);
+      if (n_valid < kTileKeys) {                               // the segment's last keys; those past its end count nothing
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
+        tile += tz * ex2(tm);
+      }
+      const bool exact = !(tile < INFINITY && tile > kTinySum);
+      if (!__any_sync(0xffffffffu, exact)) {
+        z += (double)tile;
+      } else {                                                 // the exact path's TMEM loads need the whole warp
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, 0, n_valid, tm, tz);
+        if (!exact) z += (double)tile;                         // the same value whatever the other rows hold
+        else if (fabsf(tm) <= kFarScore) z += scalbn((double)tz, (int)tm);
+        else stat_add(far_z, far_m, tz, tm);
+      }
+    }
+    unit_release(u);
+  }
+  return true;
+}
+
+// Votes of one run for this thread's key of every tile, handed to out(key, vote): the sum over this warpgroup's rows (cols of them, from its
+// log-sum-exps lse on).  MT = 2: the other 128 rows are the neighbouring warpgroup's; the first one, whose unit is filled
+// first, leaves its share in shared memory for the second (four slots in turn: a tile's second product waits until the
+// second warpgroup has given its unit back, so the first one cannot be more than three of its tiles ahead).
+// false: a wait ran out.
+template <typename Out>
+__device__ __forceinline__ bool votes_run(const Unit u, int nth, float sc, int i0, int every, int count, int n_keys,
+                                       uint32_t lse, int cols, int half, float* half_vote, uint32_t half_bar, int n_half,
+                                       float inv_g, Out out) {
+  const f32x2 sc2 = pack2(sc, sc);
+  const int row = threadIdx.x & 127;
+#pragma unroll 1
+  for (int i = i0; i < count; i += every, ++nth) {
+    if (!unit_wait(u, nth)) return false;
+    uint32_t ra[16], rb[16];
+    f32x2 s0 = 0, s1 = 0;
+    tc_ld16_issue(u.tcol, ra);
+#pragma unroll 1
+    for (int c0 = 0; c0 < cols; c0 += 32) {
+      tc_ld_wait(ra);
+      tc_ld16_issue(u.tcol + c0 + 16, rb);
+      exp_chunk<false, true>(ra, sc2, 0, lse + 4u * c0, s0, s1);
+      tc_ld_wait(rb);
+      if (c0 + 32 < cols) tc_ld16_issue(u.tcol + c0 + 32, ra); else unit_release(u);
+      exp_chunk<false, false>(rb, sc2, 0, lse + 4u * c0 + 64u, s0, s1);
+    }
+    float acc = sum2(s0, s1);
+    if (half >= 0) {
+      const int turn = n_half & 3;
+      const uint32_t parity = (n_half >> 2) & 1;
+      ++n_half;
+      if (half == 0) {
+        half_vote[turn * 128 + row] = acc;
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(half_bar + 8u * turn);
+        continue;
+      }
+      const bool ok = mbar_wait(half_bar + 8u * turn, parity, u.abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      acc += half_vote[turn * 128 + row];
+    }
+    const int key = i * kTileKeys + row;
+    if (key < n_keys) out(key, acc * inv_g);
+  }
+  return true;
 }
 
 }  // namespace

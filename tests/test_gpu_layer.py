@@ -1,0 +1,123 @@
+"""GPU: single calls that do the whole layer in one launch (a cluster of CTAs per segment), against the general path launch by
+launch -- which a call that asks for the pooled scores takes -- and the scores alone against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import parity as P
+from paper_2508_15806_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+def inputs(seed, lens, hq, hkv, d, w, dt=torch.bfloat16, scale=1.0):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    T = sum(lens)
+    q, k, v = (torch.randn(*s, generator=g, device=DEV) for s in ((len(lens), w, hq, d), (T, hkv, d), (T, hkv, d)))
+    return (q * scale).to(dt), (k * scale).to(dt), v.to(dt), np.concatenate([[0], np.cumsum(lens)]).tolist()
+
+
+def both(q, k, v, cu, w, pool, budgets, mode=B.SLKV_POOL_MAX, domain=B.SLKV_HISTORY, lse=None, cap=None, one_launch=True, calls=1):
+    """(one launch, general path): offsets, kept positions, rows."""
+    p = B.make_params(q, k, v, w, pool, mode, softmax_domain=domain, lse_units=B.SLKV_LSE_LOG2)
+    hkv, d, n = k.shape[1], k.shape[2], len(cu) - 1
+    bud = torch.tensor(budgets, dtype=torch.int32, device=DEV)
+    cap = cap if cap is not None else max(sum(min(b - a, max(c, w)) for a, b in zip(cu, cu[1:]) for c in budgets), 1)
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    res = []
+    for pooled in (None, torch.zeros(max(B.slkv_pooled_elems(p, cu), 1), device=DEV)):
+        ko, vo = (torch.zeros(max(cap, 1), d, dtype=k.dtype, device=DEV) for _ in range(2))
+        off, kept = torch.full((n * hkv + 1,), -1, dtype=torch.int32, device=DEV), torch.full((max(cap, 1),), -1, dtype=torch.int32, device=DEV)
+        status = torch.zeros(1, dtype=torch.int32, device=DEV)
+        for _ in range(calls):
+            B.slkv_compress(p, q, k, v, cu_dev, cu, bud, ko[:cap], vo[:cap], off, kept, ws, pooled, status, lse=lse)
+        if pooled is None:
+            assert (B.slkv_last_launch_count() == 1) == one_launch
+        torch.cuda.synchronize()
+        res.append((off, kept, ko, vo, status))
+    return res
+
+
+def same(res, status=0):
+    a, b = res
+    assert int(a[4]) == status and int(b[4]) == status
+    for x, y in zip(a[:4], b[:4]):
+        assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("hq,hkv,d,w", [(8, 8, 128, 1), (8, 4, 64, 16), (32, 8, 128, 32), (5, 1, 64, 25), (24, 8, 128, 32)])
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 1023, 1025, 2000, 4096, 4097, 8191, 8192])
+def test_lengths(hq, hkv, d, w, n):
+    q, k, v, cu = inputs(n + hq, [n + w], hq, hkv, d, w)
+    same(both(q, k, v, cu, w, 7, [(0, w, w + 1, w + n // 3, w + n - 1, w + n, w + n + 9, w + 64)[h] for h in range(hkv)],
+              one_launch=hkv > 1 or n <= 4096))
+
+
+@pytest.mark.parametrize("lens", [[3000, 0, 31, 32, 33, 700], [160, 1100] * 4, [300] * 8])
+@pytest.mark.parametrize("mode,pool", [(B.SLKV_POOL_MAX, 1), (B.SLKV_POOL_AVG, 5), (B.SLKV_POOL_AVG, 9), (B.SLKV_POOL_MAX, 3)])
+def test_ragged_batches(lens, mode, pool):
+    q, k, v, cu = inputs(len(lens) + pool, lens, 16, 4 if len(lens) == 6 else 8, 64, 32)
+    same(both(q, k, v, cu, 32, pool, [40, 300, 33, 5000][:k.shape[1]] * (k.shape[1] // 4), mode))
+
+
+@pytest.mark.parametrize("d,w,hq,hkv,n", [(64, 32, 32, 8, 4061), (128, 17, 4, 4, 900), (128, 64, 2, 1, 2500), (64, 100, 2, 2, 4000)])
+def test_domains_and_supplied_statistics(d, w, hq, hkv, n):
+    q, k, v, cu = inputs(d + w, [n + w], hq, hkv, d, w)
+    bud = [w + 10 + 50 * h for h in range(hkv)]
+    same(both(q, k, v, cu, w, 5, bud, domain=B.SLKV_ALL_CAUSAL))
+    p = B.make_params(q, k, v, w, 5, softmax_domain=B.SLKV_ALL_CAUSAL, lse_units=B.SLKV_LSE_LOG2)
+    lse = torch.zeros(1, hq, w, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
+    B.slkv_row_lse(p, q, k, cu_dev, cu, lse, ws)
+    same(both(q, k, v, cu, w, 5, bud, lse=lse))
+    # the scores alone, with the library's statistics and with the same handed in
+    own, fed = (torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) for _ in range(2))
+    B.slkv_score(p, q, k, cu_dev, cu, own, ws)
+    assert B.slkv_last_launch_count() == 1
+    B.slkv_score(p, q, k, cu_dev, cu, fed, ws, lse=lse)
+    assert torch.equal(own, fed)
+    ref = P.oracle_pooled(q.cpu(), k.cpu(), cu, w, 5, domain=B.SLKV_ALL_CAUSAL)
+    P.assert_pooled_close(own.cpu().numpy(), ref, cu, hkv, w)
+
+
+def test_scores_beyond_fp32_and_fp64():
+    # log-sum-exps of up to some 6000 in log2 units are rounded to 2^-11, which a vote shows as 2^-11 ln 2 of its value, twice
+    for scale, shift in ((6.0, 40.0), (40.0, 300.0)):
+        q, k, v, cu = inputs(3, [1500], 8, 2, 128, 32, scale=scale)
+        k[:, :, 0] += shift
+        q[:, :16, :, 0], q[:, 16:, :, 0] = 80.0, -80.0
+        p = B.make_params(q, k, v, 32, 7)
+        one, general = (torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) for _ in range(2))
+        status = torch.zeros(1, dtype=torch.int32, device=DEV)
+        cu_dev, bud = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.tensor([100, 200], dtype=torch.int32, device=DEV)
+        ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+        B.slkv_score(p, q, k, cu_dev, cu, one, ws, status)
+        assert int(status) == 0 and B.slkv_last_launch_count() == 1
+        out = torch.zeros(300, 128, dtype=torch.bfloat16, device=DEV)
+        B.slkv_compress(p, q, k, v, cu_dev, cu, bud, out, torch.zeros_like(out), torch.zeros(3, dtype=torch.int32, device=DEV),
+                        torch.zeros(300, dtype=torch.int32, device=DEV), ws, general, status)
+        assert int(status) == 0 and torch.isfinite(one).all() and (one > 0).any()
+        assert torch.allclose(one, general, rtol=7e-4, atol=1e-30)
+
+
+def test_views_and_capacity():
+    # K and V slices of one fused buffer, heads outermost; then too little room
+    w, n, hkv, d = 32, 1900, 4, 128
+    q, _, _, cu = inputs(5, [n], 16, hkv, d, w)
+    kv = torch.randn(2 * hkv, n + 5, d, device=DEV).bfloat16()
+    k, v = kv[:hkv, 5:].transpose(0, 1), kv[hkv:, 5:].transpose(0, 1)
+    qt = q.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+    for qq in (q, qt):
+        same(both(qq, k, v, cu, w, 7, [100, 1500, 33, 64]))
+    same(both(q, k, v, cu, w, 7, [100, 1500, 33, 64], cap=777), status=B.ERR["CAPACITY"])
+    same(both(q, k, v, cu, w, 7, [100, 1500, 33, 64], cap=1), status=B.ERR["CAPACITY"])
+
+
+@pytest.mark.parametrize("n", [1500, 8192])
+def test_many_calls_in_a_row(n):
+    # 8192 positions: a CTA's tiles go round the ring of K tiles, and come back for the votes
+    q, k, v, cu = inputs(n, [n + 32], 32, 8, 128, 32)
+    same(both(q, k, v, cu, 32, 7, [64 + 100 * h for h in range(8)], calls=1000))
