@@ -8,7 +8,7 @@ namespace slkv {
 namespace {
 
 constexpr int kLayerThreads = 512;            // threads that select and copy
-constexpr int kLayerMaxCluster = 8;
+constexpr int kLayerMaxCluster = 10;          // above eight: where the device has room for such clusters
 
 // Pooling, selection and gather of a launch.
 struct LayerTail {
@@ -164,6 +164,21 @@ __device__ __forceinline__ void layer_gather(const LayerTail& a, const Segment& 
     default: layer_gather_rows<32>(a, x, r, stage, tid, rank, CS); break;
   }
 }
+
+// Between the CTAs of a cluster data goes in bulk copies: plain stores to another CTA's shared memory move some 7 bytes per
+// clock (32 KB of votes into one CTA: 1.5-2 us).
+__device__ __forceinline__ uint32_t in_cta(const void* p, int rank) {           // p's place in another CTA's shared memory
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+// 16-byte aligned, a multiple of 16 bytes; completes on bar in the CTA that receives.  The writers of src have made their
+// writes visible to such copies (publish_for_copy) in front of a barrier with this thread.
+__device__ __forceinline__ void copy_to_cta(const void* dst, const void* src, int bytes, const void* bar, int rank) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(in_cta(dst, rank)), "r"((uint32_t)__cvta_generic_to_shared(src)), "r"(bytes), "r"(in_cta(bar, rank)) : "memory");
+}
+__device__ __forceinline__ void publish_for_copy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // A cluster's barrier in two halves; whole warps.
 __device__ __forceinline__ void cluster_arrive() {

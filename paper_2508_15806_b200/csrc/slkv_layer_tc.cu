@@ -12,8 +12,9 @@
 //   warp 2     the segment's packed rows from the budgets
 //   warps 4-19 the arithmetic of the list kernel, tile by tile the same (results are the same bit for bit where the fp64 sums
 //              are exact); then, in the first CTA, pooling and selection; then the CTA's share of the rows
-// What bounds it: latency -- keys on their way 2 us, exponentials 0.55 us per tile and pass, two exchanges of 1 us, the
-// selection's chain of 3-4 us, rows in and out 1.5 us.
+// What bounds it: latency -- keys on their way 2 us, exponentials 0.6-0.8 us per tile and pass, exchanges of 1 us, the
+// selection's chain of 2-4 us, rows in and out 1.5 us (8 segments of 8192 positions, 7 tiles per CTA: statistics 6, exchange
+// 1.6, votes 5.8 with their way into the first CTA, selection 5, rows 1.6).
 #include <cuda.h>
 
 #include "slkv_layer_device.cuh"
@@ -40,14 +41,14 @@ struct LayerArgs {
 // Shared memory behind the Q tile and the K ring.
 template <int IT> struct Far {
   alignas(16) float votes_mem[(vote_floats(kLayerThreads, IT) > window_floats(128) ? vote_floats(kLayerThreads, IT) : window_floats(128)) + 3 & ~3];
-  double z_all[kLayerMaxCluster][128];         // row sums of the cluster's CTAs
+  struct alignas(16) Sums { double z[128]; int far, unused[3]; };
+  Sums all[kLayerMaxCluster];                  // row sums of the cluster's CTAs; far: some of them are in far[] there
   double z_wg[4][128];                         // ... of this CTA's warpgroups
   float2 far_wg[4][128];                       // what fp64 cannot hold of them (sum, reference)
   float2 far[128];                             // the same of the CTA; read by the others
-  float win_m[128], win_z[128];                // the window keys' share
+  alignas(16) float2 win[128];                 // the window keys' share (maximum, sum)
   float lse[128];                              // log-sum-exps, negated
-  unsigned long long bars[2 * kMaxStages + 10];
-  int far_any[kLayerMaxCluster];
+  unsigned long long bars[2 * kMaxStages + 10], sums_bar, votes_bar;
   int far_here, abort_flag;
   uint32_t tmem;
   SegmentRows rows;
@@ -81,6 +82,8 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
   const int first = tiles * rank / CS, n_t = tiles * (rank + 1) / CS - first;          // this CTA's tiles
   const bool stats = a.passes == 3;
   const Ring ring = {n_t, a.n_stages};
+  const int window_blocks = (a.R + kWinRows - 1) / kWinRows, my_blocks = rank < window_blocks ? (window_blocks - rank - 1) / CS + 1 : 0;
+  constexpr int vote_bytes = kTileKeys / IT * (IT + 4) * 4;                            // of a tile, as they lie in shared memory
 
   pdl_launch_dependents();
   if (tid == 0) {
@@ -92,6 +95,11 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
     for (int u = 0; u < 4; ++u) { mbar_init(unit_full(u), 1); mbar_init(unit_empty(u), 4); }
     mbar_init(q_full, 1);
     mbar_init(drain, 1);
+    mbar_init(smem_u32(&f.sums_bar), 1);
+    mbar_init(smem_u32(&f.votes_bar), 1);
+    if (stats) mbar_expect_tx(smem_u32(&f.sums_bar), (uint32_t)((CS - 1) * sizeof(typename Far<IT>::Sums) +
+                                                                 (a.all_causal && x.n > 0 ? (window_blocks - my_blocks) * kWinRows * 8 : 0)));
+    if (rank == 0) mbar_expect_tx(smem_u32(&f.votes_bar), (uint32_t)((tiles - n_t) * vote_bytes));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // rows of the Q tile beyond R are never written by TMA: keep them zero
@@ -107,8 +115,8 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = f.tmem;
-  // Barriers of the cluster, which every thread passes whatever happens: 0 everybody is there, 1 row sums, 2 votes, 3 kept
-  // positions, 4 nobody reads another CTA's memory any more.
+  // Barriers of the cluster, which every thread passes whatever happens: 0 everybody is there, 1 kept positions, 2 nobody reads
+  // another CTA's memory any more.  Row sums and votes are waited for where they arrive.
   cluster_arrive();                                                                        // 0
 
   if (warp == 0) {
@@ -133,8 +141,6 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
         if (ok) load(i);
       }
     }
-    cluster_wait();                                                                        // 0
-    cluster_arrive();                                                                      // 1
     if (lane == 0 && n_t > 0 && stats)
       for (int i = n_t - 1 - a.n_stages; i >= 0 && ok; --i) {
         const int st = i % a.n_stages, uses = ring.uses(st), q = i / a.n_stages;
@@ -179,8 +185,6 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
       if (stats)
         for (int i = 0; i < n_t && ok; ++i) product(i, i / a.n_stages, false);
     }
-    cluster_wait();                                                                        // 0
-    cluster_arrive();                                                                      // 1
     if (lane == 0 && n_t > 0) {
       for (int i = n_t - 1; i >= 0 && ok; --i) {
         const int uses = ring.uses(i % a.n_stages), q = i / a.n_stages;
@@ -200,8 +204,6 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
       const SegmentRows r = segment_rows(a.tail, x);
       if (lane == 0) f.rows = r;
     }
-    cluster_wait();                                                                        // 0
-    cluster_arrive();                                                                      // 1
   } else {
     const int t = tid - 128, wg = t >> 7, row = t & 127;
     float* votes = f.votes_mem + kLead;
@@ -215,22 +217,13 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
     if (stats) {
       // the window keys' statistics, 16 rows at a time, while the keys are on their way (in the votes' memory)
       const bool win = a.all_causal && x.n > 0;
-      float win_m = 0.f, win_z = 0.f;
-      int win_row = -1;
-      if (win && wg == 0) {
-        auto rows16 = [&](int row0) {
-          auto out = [&](int r, float m, float z) {           // everybody needs them; the others are known to be there at barrier 0
-            f.win_m[r] = m;
-            f.win_z[r] = z;
-          };
-          if (a.halves == 2) window_rows<__nv_bfloat16, 128, 2>(a.win, f.votes_mem, t, x.s, x.g, x.t0 + x.n, row0, out);
-          else window_rows<__nv_bfloat16, 64, 2>(a.win, f.votes_mem, t, x.s, x.g, x.t0 + x.n, row0, out);
+      if (win && wg == 0)
+        for (int b = rank; b < window_blocks; b += CS) {
+          auto out = [&](int r, float m, float z) { f.win[r] = make_float2(m, z); };
+          if (a.halves == 2) window_rows<__nv_bfloat16, 128, 2>(a.win, f.votes_mem, t, x.s, x.g, x.t0 + x.n, b * kWinRows, out);
+          else window_rows<__nv_bfloat16, 64, 2>(a.win, f.votes_mem, t, x.s, x.g, x.t0 + x.n, b * kWinRows, out);
           asm volatile("bar.sync 2, 128;" ::: "memory");
-        };
-        for (int b = rank; b * kWinRows < a.R; b += CS) rows16(b * kWinRows);
-        // this thread hands on row `row`, if the CTA has it
-        if (row < a.R && row / kWinRows % CS == rank) { win_row = row; win_m = f.win_m[row]; win_z = f.win_z[row]; }
-      }
+        }
       double z;
       float far_z, far_m;
       stats_run(u, 0, a.scale_log2, wg, 4, n_t, x.n - first * kTileKeys, (warp & 3) * 32 < a.R, z, far_z, far_m);
@@ -239,29 +232,33 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
       if (far_z > 0.f) f.far_here = 1;
       sync();
       const bool far = f.far_here != 0;
-      const double z_cta = (f.z_wg[0][row] + f.z_wg[1][row]) + (f.z_wg[2][row] + f.z_wg[3][row]);
-      if (far && wg == 0) {
-        float fz = 0.f, fm = 0.f;
-        for (int w = 0; w < 4; ++w) stat_add(fz, fm, f.far_wg[w][row].x, f.far_wg[w][row].y);
-        f.far[row] = make_float2(fz, fm);
+      if (wg == 0) {
+        f.all[rank].z[row] = (f.z_wg[0][row] + f.z_wg[1][row]) + (f.z_wg[2][row] + f.z_wg[3][row]);
+        if (row == 0) f.all[rank].far = far;
+        if (far) {
+          float fz = 0.f, fm = 0.f;
+          for (int w = 0; w < 4; ++w) stat_add(fz, fm, f.far_wg[w][row].x, f.far_wg[w][row].y);
+          f.far[row] = make_float2(fz, fm);
+          asm volatile("fence.acq_rel.cluster;" ::: "memory");                             // read by the others once they have `far`
+        }
+        publish_for_copy();
+        cluster_wait();                                                                    // 0
+        asm volatile("bar.sync 2, 128;" ::: "memory");
+        if (t < CS && t != rank) {
+          copy_to_cta(&f.all[rank], &f.all[rank], sizeof(f.all[0]), &f.sums_bar, t);
+          if (win)
+            for (int b = rank; b < window_blocks; b += CS) copy_to_cta(&f.win[b * kWinRows], &f.win[b * kWinRows], kWinRows * 8, &f.sums_bar, t);
+        }
+        mbar_wait(smem_u32(&f.sums_bar), 0, abort_flag);
+      } else {
+        cluster_wait();                                                                    // 0
       }
-      cluster_wait();                                                                      // 0
-      for (int c = wg; c < CS; c += 4) *cluster.map_shared_rank(&f.z_all[rank][row], c) = z_cta;
-      if (t < CS) *cluster.map_shared_rank(&f.far_any[rank], t) = far;
-      if (win_row >= 0)
-        for (int c = 0; c < CS; ++c)
-          if (c != rank) {
-            *cluster.map_shared_rank(&f.win_m[row], c) = win_m;
-            *cluster.map_shared_rank(&f.win_z[row], c) = win_z;
-          }
-      cluster_arrive();                                                                    // 1
-      cluster_wait();
       if (wg == 0) {
         float l2 = INFINITY;                                   // rows of padding: 2^(0 - inf) = 0
         if (row < a.R) {
           double Z = 0.0;
           bool any_far = false;
-          for (int c = 0; c < CS; ++c) { Z += f.z_all[c][row]; any_far |= f.far_any[c] != 0; }
+          for (int c = 0; c < CS; ++c) { Z += f.all[c].z[row]; any_far |= f.all[c].far != 0; }
           if (!any_far && !win) {
             l2 = log2_of(Z);
           } else {                                             // as row_lse
@@ -271,11 +268,11 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
               sz = (float)__hiloint2double((__double2hiint(Z) & 0xfffff) | 0x3ff00000, __double2loint(Z));
             }
             for (int c = 0; c < CS; ++c)
-              if (f.far_any[c]) {
+              if (f.all[c].far) {
                 const float2 o = *cluster.map_shared_rank(&f.far[row], c);
                 stat_add(sz, sm, o.x, o.y);
               }
-            if (win) stat_add(sz, sm, f.win_z[row], f.win_m[row]);
+            if (win) stat_add(sz, sm, f.win[row].y, f.win[row].x);
             l2 = __fadd_rn(sm, log2f(sz));
           }
         }
@@ -284,8 +281,6 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
     } else {
       if (wg == 0) f.lse[row] = row < a.R ? -a.lse.caller_lse(x.s, x.g, row, a.G, a.tail.window, a.q_head_inner != 0) : -INFINITY;
       cluster_wait();                                                                      // 0
-      cluster_arrive();                                                                    // 1
-      cluster_wait();
     }
     const float pad = a.tail.pool_mode == SLKV_POOL_MAX ? -INFINITY : 0.f;
     if (rank == 0 && wg == 1 && row < 8) {
@@ -294,29 +289,35 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
     }
     sync();
     {
-      float* dst = cluster.map_shared_rank(votes, 0);
       const int j0 = (wg - (stats ? n_t : 0)) & 3, nth = stats && wg < n_t ? ((n_t - 1 - wg) >> 2) + 1 : 0;
       const int n_here = x.n - first * kTileKeys;
       votes_run(u, nth, a.scale_log2, j0, 4, n_t, 0x7fffffff, smem_u32(f.lse), a.Rp, -1, nullptr, 0u, 0, 1.0f / (float)a.G,
                 [&](int j, float v) {
                   const int key = (n_t - 1 - (j >> 7)) * kTileKeys + (j & 127);
-                  if (key < n_here) dst[vote_at<IT>(first * kTileKeys + key)] = v;
+                  votes[vote_at<IT>(first * kTileKeys + key)] = key < n_here ? v : pad;
                 });
+      publish_for_copy();
     }
-    cluster_arrive();                                                                      // 2
-    cluster_wait();
+    sync();
+    if (rank == 0) {
+      mbar_wait(smem_u32(&f.votes_bar), 0, abort_flag);
+    } else if (t == 0 && n_t > 0) {
+      float* mine = votes + vote_at<IT>(first * kTileKeys);
+      copy_to_cta(mine, mine, n_t * vote_bytes, &f.votes_bar, 0);
+    }
     const SegmentRows r = f.rows;
     if (rank == 0) layer_select<IT, 1>(a.tail, x, r.k_keep, votes, *reinterpret_cast<SelShared*>(smem), t);
-    cluster_arrive();                                                                      // 3
+    cluster_arrive();                                                                      // 1
     cluster_wait();
     if (a.tail.select) layer_gather(a.tail, x, r, reinterpret_cast<const int*>(cluster.map_shared_rank(f.votes_mem, 0)), t, rank, CS);
   }
   if (warp < 4) {
-    cluster_wait();                                                                        // 1
-    for (int b = 2; b <= 3; ++b) { cluster_arrive(); cluster_wait(); }
+    cluster_wait();                                                                        // 0
+    cluster_arrive();                                                                      // 1
+    cluster_wait();
   }
   tc_fence_before();
-  cluster_arrive();                                                                        // 4
+  cluster_arrive();                                                                        // 2
   cluster_wait();
   tc_fence_after();
   if (f.abort_flag && tid == 0 && a.status) atomicExch(a.status, (int)SLKV_ERR_DEVICE_TIMEOUT);
@@ -330,32 +331,6 @@ template <int IT> int layer_stages(int halves) {
   return n < kMaxStages ? n : kMaxStages;
 }
 
-// Clusters of each size that run at the same time, per device (0: not asked yet).
-int clusters_at_once(int log_cs) {
-  static thread_local int dev_known = -1, known[4];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (dev != dev_known) {
-    for (int l = 0; l < 4; ++l) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(1u << l);
-      cfg.blockDim = dim3(kThreads);
-      cfg.dynamicSmemBytes = layer_smem<16>(2, layer_stages<16>(2));
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = 1u << l; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&known[l], k_layer_tc<16>, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        known[l] = 0;
-      }
-    }
-    dev_known = dev;
-  }
-  return known[log_cs];
-}
-
 cudaError_t configure() {
   static thread_local int configured_dev = -1;
   int dev = 0;
@@ -363,37 +338,61 @@ cudaError_t configure() {
   if (e != cudaSuccess || configured_dev == dev) return e;
   for (Kern k : {k_layer_tc<8>, k_layer_tc<16>}) {
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
   configured_dev = dev;
   return e;
 }
 
+// Clusters of cs CTAs that run at the same time on the current device.
+int clusters_at_once(int cs) {
+  static thread_local int dev_known = -1, known[kLayerMaxCluster + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev != dev_known) {
+    for (int c = 2; c <= kLayerMaxCluster; ++c) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)c);
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = layer_smem<16>(2, layer_stages<16>(2));
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = (unsigned)c; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&known[c], k_layer_tc<16>, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();                        // not a sticky error
+        known[c] = 0;
+      }
+    }
+    dev_known = dev;
+  }
+  return known[cs];
+}
+
 }  // namespace
 
-// CTAs per segment, 0: the shape is not taken.  The largest cluster of which there is one for every segment at the same time,
-// as long as a CTA has few tiles: these run on n_seg * CS SMs, while the general path spreads the tiles over all of them but
-// takes three launches and exchanges through memory.  One layer of head_dim 128 and 128 rows, us in a graph / from a stream,
-// here (CTAs per segment) and on the general path:
-//   segments   1000 tokens                  4000 tokens                  8000 tokens
-//   1          11.7/12.2 (8) 16.4/22.3      15.6/16.2 (8) 18.0/22.5      23.9/24.2 (8) 19.3/23.7
-//   8          12.5/12.9 (8) 18.1/24.9      16.4/16.9 (8) 22.5/25.0      24.9/25.1 (8) 25.8/28.9
-//   16         14.0/14.6 (4) 21.6/24.8      23.4/24.1 (4) 25.6/28.9      36.2/36.7 (4) 31.2/34.9
-//   32         14.6/14.8 (4) 24.5/27.4      24.4/24.7 (4) 31.0/34.8      37.7/37.8 (4) 38.1/41.4
-//   40         18.3/18.6 (2) 25.3/28.9      36.5/36.9 (2) 33.6/37.1      62.0/62.7 (2) 44.5/47.5
-//   64         18.6/19.0 (2) 28.2/31.1      38.1/38.5 (2) 39.1/43.3      63.3/63.9 (2) 64.7/68.1
-// Two rounds of clusters: 16 segments of 1000 tokens in clusters of 8 24.1, of 4 14.0.
+// CTAs per segment, 0: the shape is not taken.  The largest cluster of which there is one for every segment at the same time
+// (eight segments: of ten CTAs; sixteen: of six), two CTAs at least: the clusters run on n_seg * CS SMs, while the general path
+// spreads a layer's tiles over all of them but takes three launches and exchanges through memory.  One layer of head_dim 128 and
+// 128 rows, us in a graph / from a stream, here and on the general path:
+//   segments   1000 tokens            4000 tokens            8000 tokens
+//   1          10.9/11.6  16.3/20.6   15.1/15.5  18.0/22.7   21.5/21.8  19.3/24.3
+//   8          12.0/12.4  18.0/22.6   16.0/16.5  22.3/25.0   22.6/22.8  25.3/28.8
+//   16         13.4/13.7  21.3/24.7   19.7/20.1  25.2/28.8   28.5/29.0  30.9/34.5
+//   32         14.2/14.3  24.2/27.1   23.8/24.1  30.6/33.8   37.3/37.4  37.8/41.1
+//   40         15.9/16.3  25.1/28.7   27.9/28.3  33.5/37.0   45.1/45.5  44.0/46.9
+//   64         18.1/18.7  28.0/30.9   37.5/37.8  38.8/42.9   62.6/63.0  63.5/66.9
+// and with 32 rows 8 x 8000 19.7/20.0 24.5/27.6, 64 x 8000 58.4/58.8 58.4/61.7.  More segments than clusters: two rounds (16
+// segments of 1000 tokens in clusters of eight 24.1, of four 14.0).
 int layer_tc_cluster(const Problem& pb) {
   const slkv_params& p = pb.p;
   if (!tensor_path_supported(p) || pb.R > 128 || (p.pool_kernel >> 1) > kMaxRadius || p.history_only || pb.tab.n_inline == 0 ||
       pb.max_hist < 1 || pb.max_hist > 16 * kLayerThreads || configure() != cudaSuccess)
     return 0;
-  const int tiles = (pb.max_hist + kTileKeys - 1) / kTileKeys;
-  for (int l = 3; l >= 1; --l) {
-    if (pb.n_seg > clusters_at_once(l)) continue;
-    const int cs = 1 << l, ctas = pb.n_seg * cs, per_cta = (tiles + cs - 1) / cs;
-    return per_cta <= (ctas < 32 ? 4 : 8) || 4 * ctas >= 3 * sm_count() ? cs : 0;
-  }
+  for (int cs = kLayerMaxCluster; cs >= 2; --cs)
+    if (pb.n_seg <= clusters_at_once(cs)) return cs;
   return 0;
 }
 
