@@ -280,9 +280,13 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
 // lse_out null: into the layer's own statistics area
 cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
                                     cudaStream_t st, int* launches);
-// ---- a whole layer in one launch (slkv_layer_tc.cu) ----------------------------------------------------------------
+// ---- a whole layer in one launch (slkv_layer_tc.cu, slkv_layer_fma.cu) ---------------------------------------------
 // CTAs per segment, or 0 where the shape is not taken; tail null: the pooled scores alone.  pooled may be null with a tail.
+int layer_tc_clusters_for(int n_seg);
 int layer_tc_cluster(const Problem& pb);
+int layer_fma_cluster(const Problem& pb);
+cudaError_t launch_layer_fma(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,
+                             int* launches);
 cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,
                             int* launches);
 // Timeline buffer of this thread (diagnostics), or null: kTraceSlots words per CTA.

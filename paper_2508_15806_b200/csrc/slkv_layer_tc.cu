@@ -373,6 +373,14 @@ int clusters_at_once(int cs) {
 
 }  // namespace
 
+// The largest cluster, two CTAs at least, of which n_seg run at the same time, an SM for each CTA; 0: none.
+int layer_tc_clusters_for(int n_seg) {
+  if (configure() != cudaSuccess) return 0;
+  for (int cs = kLayerMaxCluster; cs >= 2; --cs)
+    if (n_seg <= clusters_at_once(cs)) return cs;
+  return 0;
+}
+
 // CTAs per segment, 0: the shape is not taken.  The largest cluster of which there is one for every segment at the same time
 // (eight segments: of ten CTAs; sixteen: of six), two CTAs at least: the clusters run on n_seg * CS SMs, while the general path
 // spreads a layer's tiles over all of them but takes three launches and exchanges through memory.  One layer of head_dim 128 and
@@ -389,11 +397,9 @@ int clusters_at_once(int cs) {
 int layer_tc_cluster(const Problem& pb) {
   const slkv_params& p = pb.p;
   if (!tensor_path_supported(p) || pb.R > 128 || (p.pool_kernel >> 1) > kMaxRadius || p.history_only || pb.tab.n_inline == 0 ||
-      pb.max_hist < 1 || pb.max_hist > 16 * kLayerThreads || configure() != cudaSuccess)
+      pb.max_hist < 1 || pb.max_hist > 16 * kLayerThreads)
     return 0;
-  for (int cs = kLayerMaxCluster; cs >= 2; --cs)
-    if (pb.n_seg <= clusters_at_once(cs)) return cs;
-  return 0;
+  return layer_tc_clusters_for(pb.n_seg);
 }
 
 cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,

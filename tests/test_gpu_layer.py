@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import parity as P
+from oracle import slkv_oracle as O
 from paper_2508_15806_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
@@ -120,3 +121,69 @@ def test_many_calls_in_a_row(n):
     # 8192 positions: a CTA's tiles go round the ring of K tiles, and come back for the votes
     q, k, v, cu = inputs(n, [n + 32], 32, 8, 128, 32)
     same(both(q, k, v, cu, 32, 7, [64 + 100 * h for h in range(8)], calls=1000))
+
+
+# ---- fp32 -------------------------------------------------------------------------------------------------------------
+def check_fp32(hq, hkv, d, w, lens, pool=5, mode=B.SLKV_POOL_MAX, domain=B.SLKV_HISTORY, q_fn=None, rtol=1e-5, one_launch=True):
+    """Scores and row statistics of the one launch (without and with supplied statistics) against the general path's, the kept
+    positions against an exact sort of the scores."""
+    q, k, v, cu = inputs(hq + d + w + sum(lens), lens, hq, hkv, d, w, torch.float32)
+    if q_fn:
+        q_fn(q, k)
+    p = B.make_params(q, k, v, w, pool, mode, softmax_domain=domain, lse_units=B.SLKV_LSE_LOG2)
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    lse = torch.zeros(len(lens), hq, w, device=DEV)
+    own, fed, general = (torch.full((max(B.slkv_pooled_elems(p, cu), 1),), 7.0, device=DEV) for _ in range(3))
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.slkv_row_lse(p, q, k, cu_dev, cu, lse, ws, status)
+    B.slkv_score(p, q, k, cu_dev, cu, own, ws, status)
+    assert not one_launch or B.slkv_last_launch_count() == 1
+    B.slkv_score(p, q, k, cu_dev, cu, fed, ws, status, lse=lse)
+    assert torch.equal(own, fed)
+    budgets = [w + 3 + 37 * h for h in range(hkv)]
+    res = both(q, k, v, cu, w, pool, budgets, mode, domain, one_launch=one_launch)
+    bud, cap = torch.tensor(budgets, dtype=torch.int32, device=DEV), res[0][2].shape[0]
+    B.slkv_compress(p, q, k, v, cu_dev, cu, bud, torch.zeros(cap, d, device=DEV), torch.zeros(cap, d, device=DEV),
+                    torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.zeros(cap, dtype=torch.int32, device=DEV), ws,
+                    general, status)
+    assert int(status) == 0 and torch.allclose(own, general, rtol=rtol, atol=1e-30)
+    off, kept, ko, vo, st = res[0]
+    assert int(st) == 0 and torch.equal(off, res[1][0])
+    sc, at = own.cpu().numpy(), 0
+    for s, n in enumerate(lens):
+        nh = max(n - w, 0)
+        for h in range(hkv):
+            kh, nw = O.kept_counts(n, budgets[h], w)
+            ref = O.select_topk(sc[at:at + nh].astype(np.float64), kh) if kh else np.zeros(0, np.int64)
+            a, b = int(off[s * hkv + h]), int(off[s * hkv + h + 1])
+            got = kept[a:b].cpu()
+            assert got.tolist() == ref.tolist() + list(range(n - nw, n)), (s, h)
+            assert torch.equal(ko[a:b], k[cu[s] + got.to(DEV).long(), h]) and torch.equal(vo[a:b], v[cu[s] + got.to(DEV).long(), h])
+            at += nh
+
+
+@pytest.mark.parametrize("hq,hkv,d,w", [(8, 8, 64, 16), (2, 2, 128, 1), (16, 8, 128, 16), (6, 2, 64, 21), (16, 4, 64, 32)])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 319, 321, 400, 1008])
+def test_fp32_lengths(hq, hkv, d, w, n):
+    check_fp32(hq, hkv, d, w, [n + w])
+
+
+@pytest.mark.parametrize("hq,hkv,d,w,n", [(8, 8, 64, 16, 5000), (8, 4, 128, 8, 8192), (4, 4, 128, 16, 4096), (4, 4, 64, 16, 4097), (32, 8, 128, 16, 2400)])
+@pytest.mark.parametrize("domain", [B.SLKV_HISTORY, B.SLKV_ALL_CAUSAL])
+def test_fp32_long(hq, hkv, d, w, n, domain):
+    check_fp32(hq, hkv, d, w, [n + w], 7, domain=domain, one_launch=hkv == 8)
+
+
+@pytest.mark.parametrize("mode,pool", [(B.SLKV_POOL_MAX, 1), (B.SLKV_POOL_AVG, 9)])
+def test_fp32_ragged_batch(mode, pool):
+    check_fp32(8, 4, 64, 32, [900, 0, 31, 32, 33, 1100], pool, mode, B.SLKV_ALL_CAUSAL)
+
+
+def test_fp32_beyond_its_range():
+    def far(q, k):
+        k[:, :, 0] += 60.0
+        q[:, :4, :, 0], q[:, 4:, :, 0] = 70.0, -70.0
+    # log-sum-exps of some 750 in log2 units, rounded to 2^-14: a vote shows that twice
+    for domain in (B.SLKV_HISTORY, B.SLKV_ALL_CAUSAL):
+        check_fp32(4, 2, 64, 8, [900], domain=domain, q_fn=far, rtol=1e-4)
