@@ -8,20 +8,23 @@
 // rounded IEEE operation (__dadd_rn / __dmul_rn / __ddiv_rn stop the compiler from fusing them), so the integers that
 // come out do not depend on the launch shape.
 //
-// What bounds it: latency.  The order of the sums is part of the result, so one chain of N dependent fp64 additions
-// stays; everything else runs on all threads -- the weights (two fp64 divisions each, formerly part of that chain) are
-// in shared memory before the chain starts, which then only loads and adds, and the largest remainders are found by a
-// comparison of all pairs split over the whole CTA (N <= 1024) or by a radix descent (beyond), not by one thread per
-// head walking all the others.  256 heads: 70.5 -> 7 us.
+// What bounds it: latency.  The order of the sums is part of the result, so one chain of N dependent fp64 additions stays
+// (5 ns each); everything else runs on all threads: the weights (two fp64 divisions each) are in shared memory before the chain
+// starts, and the largest remainders are found by counting them in 1024 parts of [0, 1) -- of a few hundred remainders one or
+// two share a part.  In a graph, us: 256 heads 70.5 with all of it in one thread, 8.3 with all pairs of remainders compared, 5.7
+// now; 1024 heads (all pairs) 61.1 -> 10.5; 1536 (a radix descent) 19.5 -> 13.8; 3072 29.4 -> 23.1.
 #include "slkv_internal.cuh"
 
 namespace slkv {
 namespace {
 
 constexpr int kAllocThreads = 1024;
-constexpr int kPairsMax = 1024;        // heads up to which all pairs of remainders are compared: at 1024 a thread compares
-                                       // its head with all others (~5 us); beyond that the radix descent's eight
-                                       // levels of about 1 us each cost less
+constexpr int kPairsMost = 96;         // heads up to which all pairs of remainders are compared: us with the pairs / counted in
+                                       // parts 32 heads 4.2 / 4.5, 64 4.5 / 4.8, 96 5.0 / 5.0, 128 5.25 / 4.9, 256 8.3 / 5.7
+constexpr int kParts = kAllocThreads;  // parts of [0, 1) the remainders are counted in
+constexpr int kSmemMost = (16384 + 1024) * 8 + 16384 * 5;      // 16384 heads in 1024 layers
+constexpr int kListMost = 256;         // remainders of one part up to which they are ranked by counting (2 us); where more are
+                                       // (nearly) equal, a radix descent over all of them takes eight levels of about 1 us
 
 struct AllocOpts {
   int within_layer;      // head share over the layer's sum (prose under Eq. 6) instead of the grand sum (Algorithm 2)
@@ -76,11 +79,12 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
   unsigned char* active = reinterpret_cast<unsigned char*>(fl + N);   // [N] head still below the cap
   __shared__ long long red[kAllocThreads / 32];
   __shared__ double sh_Ls, sh_W;
-  __shared__ int hist[256];
-  __shared__ int sh_digit, sh_above;
+  __shared__ int hist[256], parts[kParts], list[kListMost];
+  __shared__ int sh_digit, sh_above, sh_count, sh_same;
   const int tid = threadIdx.x;
   const long long D = total - (long long)N * fixed;
   const bool within = opt.within_layer != 0;
+  if (N > kPairsMost) parts[tid] = 0;
   pdl_launch_dependents();
   pdl_wait();
 
@@ -163,23 +167,59 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
       if (active[a]) fl[a] += (int)each;
     Rleft -= each * n_active;
   }
-  if (Rleft > 0) {
+  if (Rleft > 0 && N <= kPairsMost) {
     // largest remainder first, ties -> lower index: head a gets +1 iff fewer than Rleft heads precede it
-    if (N <= kPairsMax) {
-      int lanes = 1;                                                  // threads per head, neighbours in a warp
-      while (lanes < 32 && 2 * lanes * N <= kAllocThreads) lanes *= 2;
-      const int a = tid / lanes, sub = tid % lanes;
-      const unsigned long long ka = a < N ? key[a] : 0ull;
-      int rank = 0;
-      if (ka) {
-#pragma unroll 8
-        for (int b = sub; b < N; b += lanes) {
-          const unsigned long long kb = key[b];
-          rank += (kb > ka) || (kb == ka && b < a);
-        }
+    int lanes = 1;                                                    // threads per head, neighbours in a warp
+    while (lanes < 32 && 2 * lanes * N <= kAllocThreads) lanes *= 2;
+    const int a = tid / lanes, sub = tid % lanes;
+    const unsigned long long ka = a < N ? key[a] : 0ull;
+    int rank = 0;
+    if (ka)
+      for (int b = sub; b < N; b += lanes) {
+        const unsigned long long kb = key[b];
+        rank += (kb > ka) || (kb == ka && b < a);
       }
-      for (int o = 1; o < lanes; o *= 2) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-      if (ka && sub == 0 && rank < Rleft) fl[a] += 1;
+    for (int o = 1; o < lanes; o *= 2) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (ka && sub == 0 && rank < Rleft) fl[a] += 1;
+  } else if (Rleft > 0) {
+    // the Rleft-th largest remainder lies in one of 1024 equal parts of [0, 1); what lies in a part above it gets +1, what lies
+    // in the same part is ranked by counting
+    auto part_of = [&](unsigned long long k) { return min((int)(__longlong_as_double((long long)(k - 1ull)) * (double)kParts), kParts - 1); };
+    for (int a = tid; a < N; a += kAllocThreads)
+      if (key[a]) atomicAdd(&parts[part_of(key[a])], 1);
+    __syncthreads();
+    const int lane0 = tid & 31, warp0 = tid >> 5, mine = parts[kParts - 1 - tid];           // from the top
+    int upto = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane0 >= o) upto += n;
+    }
+    if (lane0 == 31) hist[warp0] = upto;
+    __syncthreads();
+    upto += (int)__reduce_add_sync(0xffffffffu, lane0 < warp0 ? (unsigned)hist[lane0] : 0u);
+    if (upto - mine < Rleft && Rleft <= upto) { sh_digit = kParts - 1 - tid; sh_above = upto - mine; sh_count = 0; sh_same = mine; }
+    __syncthreads();
+    const int same = sh_same, part = sh_digit;
+    if (same <= kListMost) {
+      const int need = (int)Rleft - sh_above;
+      for (int a = tid; a < N; a += kAllocThreads) {
+        if (!key[a]) continue;
+        const int p = part_of(key[a]);
+        if (p > part) fl[a] += 1;
+        else if (p == part) list[atomicAdd(&sh_count, 1)] = a;
+      }
+      __syncthreads();
+      if (tid < same) {
+        const int a = list[tid];
+        const unsigned long long ka = key[a];
+        int rank = 0;
+        for (int j = 0; j < same; ++j) {
+          const int b2 = list[j];
+          const unsigned long long kb = key[b2];
+          rank += (kb > ka) || (kb == ka && b2 < a);
+        }
+        if (rank < need) fl[a] += 1;
+      }
     } else {
       // the Rleft-th largest key by a radix descent, eight bits at a time
       unsigned long long prefix = 0, mask = 0;
@@ -272,7 +312,7 @@ cudaError_t launch_alloc(const float* inf, int n_layers, int n_heads, int fixed,
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(k_alloc, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+    e = cudaFuncSetAttribute(k_alloc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
     if (e != cudaSuccess) return e;
     configured_dev = dev;
   }

@@ -51,6 +51,17 @@ def test_edge_tables():
         assert st == 0 and np.array_equal(got, O.alloc_budgets(inf.numpy(), fixed, total))
 
 
+@pytest.mark.parametrize("n", [95, 96, 97, 256, 257, 300, 1024, 1025])
+def test_remainders_ranked_by_pairs_parts_and_digits(n):
+    # all remainders alike (one part holds them all: up to 256 are listed, more go by digits), two values, and any
+    rng = np.random.default_rng(n)
+    for inf in (np.ones(n), 1.0 + (np.arange(n) % 3 == 0) * 1e-7, rng.lognormal(0, 2.0, n)):
+        t = torch.from_numpy(inf.astype(np.float32)).view(1, n)
+        for extra in (1, n // 2, n - 1, 7 * n + 5):
+            got, st = gpu_budgets(t, 3, 3 * n + extra)
+            assert st == 0 and np.array_equal(got, O.alloc_budgets(t.numpy(), 3, 3 * n + extra))
+
+
 def test_bad_inf_sets_status_word():
     for bad in (-1.0, float("nan"), float("inf")):
         inf = torch.ones(2, 4)
