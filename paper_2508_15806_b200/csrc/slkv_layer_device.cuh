@@ -80,7 +80,7 @@ __device__ __forceinline__ void layer_select(const LayerTail& a, const Segment& 
   constexpr int kPer = kBins / kLayerThreads;
   const bool choose = a.select && k_keep > 0 && k_keep < x.n, max_mode = a.pool_mode == SLKV_POOL_MAX;
   if (choose) {
-    if (tid == 0) sh.n_list = 0;
+    if (tid == 0) { sh.n_list = 0; sh.sure = 0; }
 #pragma unroll
     for (int i = 0; i < kPer; i += 2) {
       reinterpret_cast<int2*>(sh.hist)[(tid * kPer + i) / 2] = make_int2(0, 0);

@@ -4,16 +4,17 @@
 // The votes come into shared memory with asynchronous 16-byte copies (from an aligned start, whatever the segment's), a
 // thread pools 8, 16 or 32 consecutive positions of them and works with the scores' bit patterns (scores are >= 0, so
 // unsigned order = float order).  The k-th largest:
-//   1. with 16 or 32 positions per thread, a histogram of every 16th or 32nd score: the rank that the k-th largest has among
-//      these, plus four standard deviations, bounds it from below (else the bound is zero);
-//   2. a histogram of the scores above the bound, 2048 bins, 64 to an octave; the bin with the k-th largest;
+//   1. with 16 or 32 positions per thread, a histogram of every 16th or 32nd score: the ranks that the k-th largest has among
+//      these, give or take four standard deviations, bound it from both sides (where there are none, nothing bounds it);
+//   2. a histogram of the scores between the bounds, 2048 bins, 64 to an octave; the bin with the k-th largest;
 //   3. where that bin's scores fit a list of 512 (mostly), they are ranked by counting, else a histogram of that bin, and so on.
 // Then an ordered compaction from bit masks.  Integer counters only: the result does not depend on timing, and not on the
 // sample either.
 // What bounds it: a chain of some ten CTA-wide steps of 0.2-0.6 us, and at 32 positions per thread instructions.  Bracketing
 // the k-th largest by 128 ranked samples and a descent over the bracket took as many steps again, and its loops an atomic
 // with a result per score: whole layers of 8 segments 21.7 -> 16.9 us at 1024 positions, 26.4 -> 22.7 at 4096, 29.9 -> 26.4 at
-// 8192, 33.7 -> 30.7 at 12000, 32 layers of 4001 129.5 -> 118 (all in a graph).
+// 8192, 33.5 -> 30.1 at 12000, 32 layers of 4001 129.5 -> 118 (all in a graph).  With a bound from below alone and every position
+// looked at in each step 30.6 at 12000, 44.9 at 32000 (now 42.6), 78.1 at 64000 (75.4).
 #include "slkv_select_device.cuh"
 
 namespace slkv {
@@ -66,7 +67,7 @@ k_select_list(const __grid_constant__ SelArgs args) {
   int32_t* const gather_src = a.gather_src;
   float* const pooled_out = a.pooled_out;
   asm volatile("" ::"l"(capacity), "l"(kept_idx), "l"(gather_src), "l"(pooled_out), "l"(a.offsets));
-  if (tid == 0) sh.n_list = 0;
+  if (tid == 0) { sh.n_list = 0; sh.sure = 0; }
 #pragma unroll
   for (int i = 0; i < kPer; i += 2) {
     reinterpret_cast<int2*>(sh.hist)[(tid * kPer + i) / 2] = make_int2(0, 0);

@@ -66,15 +66,15 @@ struct alignas(16) SelShared {
   unsigned list[kList];
   unsigned wsum[3][32];
   int2 cta_tot;                // read by the cluster's other CTAs
-  unsigned tau, bin, n_list;
-  int above, m, need;
+  unsigned tau, bin, bin2, n_list;
+  int above, m, need, sure;
 };
 
 // A thread's kept places of a segment: T threads (numbered tid) with IT consecutive places each, their scores' bit patterns
 // in key (scores are >= 0: unsigned order = float order), those that exist in valid.  k_keep of the n scores are kept, the
 // largest, ties to the lower place.  CLUSTER: the segment is shared by the CTAs of a cluster (rank, CS).  BAR: the named
 // barrier of the T threads.  shelf: the thread's row of the votes' shared memory, which the scores take over once all T
-// threads are past their pooling (IT > 8 only).  sh.hist, sh.sample and sh.n_list are zero, for all to see.
+// threads are past their pooling (IT > 8 only).  sh.hist, sh.sample, sh.n_list and sh.sure are zero, for all to see.
 // Returns the kept places as a mask and, in o_mine, how many of the segment's lie before the thread's.
 template <int T, int IT, bool CLUSTER, int BAR>
 __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsigned (&key)[IT], unsigned valid, bool mine,
@@ -90,9 +90,9 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
     for (int i = 0; i < kPer; i += 2) reinterpret_cast<int2*>(hist)[(tid * kPer + i) / 2] = make_int2(0, 0);
   };
   // ---- the k-th largest by histograms.  bin_of: the bin that holds the `want` largest score of `bins` (more than that are
-  // counted there), how many lie above it and in it; with no such bin, sh_.bin = kBins.
-  auto bin_of = [&](int* bins, int want) {
-    if (tid == 0) sh_.bin = kBins;
+  // counted there), how many lie above it and in it; with no such bin, sh_.bin = kBins.  want2: likewise, the bin alone.
+  auto bin_of = [&](int* bins, int want, int want2) {
+    if (tid == 0) sh_.bin = sh_.bin2 = kBins;
     int c[kPer], sum = 0;
 #pragma unroll
     for (int i = 0; i < kPer; i += 2) {
@@ -111,7 +111,7 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
     if (lane == 0) sh_.wsum[1][wid] = (unsigned)warp_sum;
     sync();
     const int above_w = (int)__reduce_add_sync(kAll, lane > wid && lane < kWarps ? sh_.wsum[1][lane] : 0u);
-    if (above_w < want && want <= above_w + warp_sum) {   // the bin is one of this warp's
+    if ((above_w < want && want <= above_w + warp_sum) || (above_w < want2 && want2 <= above_w + warp_sum)) {   // one of this warp's
       int inc = sum;                                      // suffix sum over the lanes
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -122,15 +122,17 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
 #pragma unroll
       for (int i = kPer - 1; i >= 0; --i) {
         if (above < want && want <= above + c[i]) { sh_.bin = kPer * tid + i; sh_.above = above; sh_.m = c[i]; }
+        if (above < want2 && want2 <= above + c[i]) sh_.bin2 = kPer * tid + i;
         above += c[i];
       }
     }
     sync_all();                                           // in a cluster also: nobody reads the others' bins any more
   };
-  // Long slices: one place in IT is counted first.  Of these, the rank that the k-th largest has among them, plus four
-  // standard deviations, bounds it from below, and only the scores above that bound are counted (an atomic on shared memory
-  // takes seven cycles of the SM per warp, whether one lane adds or 32).
-  unsigned bound = 0;
+  // Long slices: one place in IT is counted first.  Of these, the rank that the k-th largest has among them, give or take four
+  // standard deviations, bounds it from below and above: only the scores between the bounds, an eighth of them at most, go
+  // through the bins (an atomic on shared memory takes seven cycles of the SM per warp, whether one lane adds or 32, and a loop
+  // over the bits of a mask as many turns as the warp's fullest lane), those above are counted together.
+  unsigned bound = 0, sure_above = kAll;
   if (kSample) {
     if (mine && valid >> (IT / 2) & 1u) atomicAdd(&sh_.sample[first_bin(key[IT / 2])], 1);
     sync_all();                                          // everybody has read the votes, too: the scores take their places
@@ -138,9 +140,11 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
 #pragma unroll
       for (int g = 0; g < IT; g += 4) shelf[g / 4] = make_uint4(key[g], key[g + 1], key[g + 2], key[g + 3]);
     const float f = __fdividef((float)k_keep, (float)n), q = f * (float)(n / IT);
-    bin_of(sh_.sample, (int)(q + 4.f * sqrtf(q * (1.f - f))) + 2);
-    const unsigned bin = sh_.bin;
+    const float dev = 4.f * sqrtf(q * (1.f - f));
+    bin_of(sh_.sample, (int)(q + dev) + 2, (int)floorf(q - dev) - 1);
+    const unsigned bin = sh_.bin, bin2 = sh_.bin2;
     if (bin > 0 && bin < (unsigned)kBins) bound = kFloorBits + ((bin - 1) << kFirstShift);
+    if (bin2 < kBins - 1u) sure_above = kFloorBits + (bin2 << kFirstShift) - 1u;
   }
   // f(e, score) for the thread's places
   auto each = [&](auto f) {
@@ -150,30 +154,37 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
       f(g, v.x); f(g + 1, v.y); f(g + 2, v.z); f(g + 3, v.w);
     }
   };
+  const unsigned* keys = reinterpret_cast<const unsigned*>(shelf);
+  // of the thread's places, those between the bounds, and the last ones of each run of equal scores among them (a maximum holds
+  // for up to pool_kernel positions); runs: f(score, the run's places)
+  unsigned between = 0, ends = 0;
+  auto runs = [&](auto f) {
+    for (unsigned m = ends, left = between; m != 0; m &= m - 1) {
+      const unsigned last = m & (0u - m), run = left & (last | (last - 1));
+      left ^= run;
+      f(keys[__ffs(m) - 1], run);
+    }
+  };
   int need = k_keep;
   unsigned lo = 0, hi = kAll, gt = 0, cand = valid, tau;
   int sh = kFirstShift;
   bool first = true;
   while (true) {
     auto index = [&](unsigned v) { return (int)(first ? first_bin(v) : min((v - lo) >> sh, kBins - 1u)); };
-    // equal neighbours are added at once: a maximum holds for up to pool_kernel positions
+    // neighbours of one bin, or of one score, are added at once
     if (kSample && mine) {
-      unsigned ends = 0, counted = 0, next = 0;           // places whose right neighbour's score is another; those that count
+      unsigned sure = 0, next = 0;
+      between = ends = 0;
       each([&](int e, unsigned v) {
         if (e > 0) ends |= v != next ? 1u << (e - 1) : 0u;
-        counted |= v >= bound ? 1u << e : 0u;
+        between |= v >= bound ? 1u << e : 0u;
+        sure |= v > sure_above ? 1u << e : 0u;
         next = v;
       });
-      counted &= cand;
-      ends = (ends | ~(counted >> 1)) & counted;
-      const unsigned* keys = reinterpret_cast<const unsigned*>(shelf);
-      int from = -1;                                      // the last place before the run
-      for (unsigned m = ends, c = counted; m != 0; m &= m - 1) {
-        const int e = __ffs(m) - 1;
-        from = __ffs(c) - 2;
-        atomicAdd(&hist[index(keys[e])], e - from);
-        c &= e == 31 ? 0u : kAll << (e + 1);
-      }
+      between &= cand & ~sure;
+      gt |= sure & cand;
+      ends = (ends | ~(between >> 1)) & between;
+      runs([&](unsigned v, unsigned run) { atomicAdd(&hist[index(v)], __popc(run)); });
     } else if (mine) {
       int bin = kBins, run = 0;
       each([&](int e, unsigned v) {
@@ -184,16 +195,29 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
       });
       atomicAdd(&hist[bin], run);
     }
+    int n_sure = 0;
+    if (kSample && first) {
+      const unsigned w = __reduce_add_sync(kAll, (unsigned)__popc(gt));
+      if (lane == 0 && w) atomicAdd(&sh_.sure, (int)w);
+    }
     sync_all();
-    bin_of(hist, need);
+    if (kSample && first) {
+      n_sure = sh_.sure;
+      if (CLUSTER) n_sure = (int)__reduce_add_sync(kAll, lane < CS ? (unsigned)*cg::this_cluster().map_shared_rank(&sh_.sure, lane) : 0u);
+    }
+    bin_of(hist, need - n_sure, 0);
     const unsigned bin = sh_.bin;
-    if (kSample && bin == (unsigned)kBins) {              // the bound was too high: everything counts
+    if (kSample && bin == (unsigned)kBins) {              // the k-th largest lies outside: everything goes through the bins
       bound = 0;
+      sure_above = kAll;
+      gt = 0;
+      if (tid == 0) sh_.sure = 0;
       clear_hist();
       sync();
       continue;
     }
     const int m_bin = sh_.m;
+    need -= n_sure;
     need -= sh_.above;
     if (first) {
       if (bin > 0) lo = kFloorBits + ((bin - 1) << kFirstShift);
@@ -207,17 +231,22 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
     const bool listed = m_bin <= kList && lo != hi;
     if (mine) {
       unsigned in_bin = 0;
-      each([&](int e, unsigned v) {
-        const unsigned bit = cand & 1u << e;
-        gt |= v > hi ? bit : 0u;
-        in_bin |= v >= lo && v <= hi ? bit : 0u;
-      });
+      if (kSample) {
+        runs([&](unsigned v, unsigned run) {
+          if (v > hi) gt |= run; else if (v >= lo) in_bin |= run;
+        });
+      } else {
+        each([&](int e, unsigned v) {
+          const unsigned bit = cand & 1u << e;
+          gt |= v > hi ? bit : 0u;
+          in_bin |= v >= lo && v <= hi ? bit : 0u;
+        });
+      }
       cand = in_bin;
       if (listed && in_bin) {
         unsigned* dst = (CLUSTER ? cg::this_cluster().map_shared_rank(sh_.list, 0) : sh_.list) +
                         atomicAdd(CLUSTER ? cg::this_cluster().map_shared_rank(&sh_.n_list, 0) : &sh_.n_list, (unsigned)__popc(in_bin));
         if (kSample) {
-          const unsigned* keys = reinterpret_cast<const unsigned*>(shelf);
           for (unsigned m = in_bin; m != 0; m &= m - 1) *dst++ = keys[__ffs(m) - 1];
         } else {
           each([&](int e, unsigned v) { if (in_bin >> e & 1u) *dst++ = v; });
@@ -253,18 +282,25 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
     const unsigned span = hi - lo;
     sh = span < (unsigned)kBins ? 0 : 21 - __clz(span);
     bound = lo;
+    sure_above = kAll;
     clear_hist();
     sync();
   }
 
   // ---- ordered compaction: the scores above tau, and the first `need` equal to it; threads own consecutive positions
   unsigned eq = 0;
-  if (mine)
+  if (kSample) {
+    for (unsigned m = cand; m != 0; m &= m - 1) {
+      const unsigned v = keys[__ffs(m) - 1], bit = m & (0u - m);
+      if (v > tau) gt |= bit; else if (v == tau) eq |= bit;
+    }
+  } else if (mine) {
     each([&](int e, unsigned v) {
       const unsigned bit = cand & 1u << e;
       gt |= v > tau ? bit : 0u;
       eq |= v == tau ? bit : 0u;
     });
+  }
   const unsigned cnt = (unsigned)__popc(gt) | ((unsigned)__popc(eq) << 16);
   unsigned inc = cnt;                                     // both totals are <= 32768
 #pragma unroll
