@@ -340,6 +340,11 @@ int slkv_cp_emit_counted(const slkv_params* p, const void* k, const void* v, int
                          void* v_out, int64_t out_capacity_rows, int32_t* offsets, int32_t* kept_idx, int32_t* status,
                          void* workspace, size_t workspace_bytes, void* stream);
 int slkv_cp_merge_lse(const slkv_params* p, const float* lse_parts, int32_t n_parts, float* lse_out, void* stream);
+/* slkv_row_lse on a workspace that is zero throughout (step 1: a caller that clears several buffers at once spares the call its
+ * own clearing, which stands between the kernels before and the statistics). */
+int slkv_cp_row_lse(const slkv_params* p, const void* q_win, const void* k, const int32_t* cu_seqlens_dev,
+                    const int32_t* cu_seqlens_host, float* lse_out, int32_t* status, void* zeroed_workspace,
+                    size_t workspace_bytes, void* stream);
 int slkv_cp_select_init(const int32_t* budgets, int32_t n_kv_heads, int32_t window, int64_t seq_len, uint32_t* prefix,
                         int32_t* need, void* stream);
 int slkv_cp_histogram(const float* pooled, int32_t n_kv_heads, int64_t row_stride, int32_t own_begin, int32_t own_count,

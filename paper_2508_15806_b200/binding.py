@@ -25,6 +25,7 @@ SLKV_POOL_MAX, SLKV_POOL_AVG = 0, 1
 SLKV_HISTORY, SLKV_ALL_CAUSAL = 0, 1
 SLKV_LSE_LN, SLKV_LSE_LOG2 = 0, 1
 SLKV_PATH_AUTO, SLKV_PATH_SIMT, SLKV_PATH_TENSOR = 0, 1, 2
+_DTYPES = {torch.float32: SLKV_F32, torch.bfloat16: SLKV_BF16}
 
 
 class SlkvParams(C.Structure):
@@ -168,14 +169,12 @@ def make_params(q_win: torch.Tensor, k: torch.Tensor, v: Optional[torch.Tensor],
     assert q_win.dim() == 4 and k.dim() == 3 and q_win.stride(3) == 1 and k.stride(2) == 1
     if v is None:
         v = k
-    dt = {torch.float32: SLKV_F32, torch.bfloat16: SLKV_BF16}[k.dtype]
+    dt = _DTYPES[k.dtype]
     assert q_win.dtype == k.dtype == v.dtype
-    return SlkvParams(n_seqs=q_win.shape[0], n_q_heads=q_win.shape[2], n_kv_heads=k.shape[1], head_dim=k.shape[2],
-                      window=window, pool_kernel=pool_kernel, dtype=dt, pool_mode=pool_mode,
-                      softmax_domain=softmax_domain, score_path=score_path, lse_units=lse_units, history_only=0,
-                      k_stride_tok=k.stride(0), k_stride_head=k.stride(1),
-                      v_stride_tok=v.stride(0), v_stride_head=v.stride(1),
-                      q_stride_seq=q_win.stride(0), q_stride_row=q_win.stride(1), q_stride_head=q_win.stride(2))
+    (n_seqs, _, n_q_heads, _), (_, n_kv_heads, head_dim) = q_win.shape, k.shape
+    (k_tok, k_head, _), (v_tok, v_head, _), (q_seq, q_row, q_head, _) = k.stride(), v.stride(), q_win.stride()
+    return SlkvParams(n_seqs, n_q_heads, n_kv_heads, head_dim, window, pool_kernel, dt, pool_mode, softmax_domain, score_path,
+                      lse_units, 0, k_tok, k_head, v_tok, v_head, q_seq, q_row, q_head)
 
 
 def slkv_version() -> int:
@@ -380,6 +379,25 @@ def slkv_cp_merge_lse(params: SlkvParams, lse_parts: torch.Tensor, lse_out: torc
     """lse_parts: CUDA float32 [n_parts, n_q_heads, window] (contiguous); lse_out: [1, n_q_heads, window]."""
     _check(_fn["slkv_cp_merge_lse"](stream, params, lse_parts, lse_parts.size(0), lse_out), "slkv_cp_merge_lse")
     return lse_out
+
+
+def slkv_cp_row_lse(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_dev: torch.Tensor, cu_seqlens: Sequence[int],
+                    lse_out: torch.Tensor, zeroed_workspace, workspace_bytes: int, status: Optional[torch.Tensor] = None,
+                    stream=None) -> torch.Tensor:
+    """slkv_row_lse on a workspace (a tensor or an address) that is zero throughout."""
+    _lse(lse_out, params)
+    _check(_fn["slkv_cp_row_lse"](stream, params, q_win, k, cu_dev, _cu_list(cu_seqlens), lse_out, status, zeroed_workspace,
+                                  workspace_bytes), "slkv_cp_row_lse")
+    return lse_out
+
+
+def slkv_score_at(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_dev: torch.Tensor, cu_seqlens: Sequence[int],
+                  pooled: torch.Tensor, workspace: int, workspace_bytes: int, status: Optional[torch.Tensor] = None, stream=None,
+                  lse: Optional[torch.Tensor] = None) -> torch.Tensor:
+    """slkv_score with the workspace given as an address."""
+    _check(_fn["slkv_score"](stream, params, q_win, k, cu_dev, _cu_list(cu_seqlens), _lse(lse, params), pooled, status, workspace,
+                             workspace_bytes), "slkv_score")
+    return pooled
 
 
 def slkv_cp_select_init(budgets: torch.Tensor, window: int, seq_len: int, prefix: torch.Tensor, need: torch.Tensor,

@@ -105,35 +105,36 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
     p = B.make_params(sh.q_win, sh.k, sh.v, w, pool_kernel, pool_mode, score_path, softmax_domain, B.SLKV_LSE_LOG2)
     p.history_only = 0 if sh.last else 1
 
-    # one buffer for what has to start at zero, one for all scratch: the calls below come one after the other
-    zeroed = torch.zeros(3 * 2048 * hkv + 3 * hkv + 2, dtype=torch.int32, device=dev)
-    hists, totals, offsets, status = zeroed.split((3 * 2048 * hkv, 2 * hkv, hkv + 1, 1))
+    # One buffer, zero at the start, for all scratch and all outputs but the packed rows: what the steps add to (row sums,
+    # histograms, totals) is cleared by one launch in front of them all, and a view is a third of an allocation.
     n_own = own + n_win
     has_keys = own > 0 or (sh.last and softmax_domain == B.SLKV_ALL_CAUSAL)
-    ws_score = B.slkv_workspace_bytes(p, [0, rows]) if n_ext > 0 else 0
-    ws_lse = 0 if not has_keys else (ws_score if n_own == rows and n_ext > 0 else B.slkv_workspace_bytes(p, [0, n_own]))
+    ws_score = B.slkv_workspace_bytes(p, (0, rows)) if n_ext > 0 else 0
+    ws_lse = 0 if not has_keys else (ws_score if n_own == rows and n_ext > 0 else B.slkv_workspace_bytes(p, (0, n_own)))
     ws_emit = B.slkv_cp_workspace_bytes(hkv, own, max(cap, 1))
     state_bytes = -(-32 * hkv // 256) * 256                    # [4][2][hkv]: every head's prefix and need after each level
-    ws = torch.empty(state_bytes + max(ws_score, ws_lse, ws_emit), dtype=torch.uint8, device=dev)
+    sizes = ((state_bytes + max(ws_score, ws_lse, ws_emit)) // 4, 3 * 2048 * hkv, hkv, hkv, hkv + 1, 1, hq * w,
+             hkv * row_stride, max(cap, 1))
+    buf = torch.zeros(sum(sizes), dtype=torch.int32, device=dev)
+    ws, hists, totals, ties, offsets, status, lse_local, pooled, kept_idx = buf.split(sizes)
     state = ws.data_ptr()
-    scratch = ws[state_bytes:]
+    scratch = state + state_bytes
+    lse_local, pooled = lse_local.view(torch.float32).view(hq, w), pooled.view(torch.float32)
 
     # 1. the rows' log-sum-exp over the keys this rank owns (the last rank's range is an ordinary sequence tail)
     if has_keys:
-        lse_local = torch.empty(hq, w, dtype=torch.float32, device=dev)
         k_own = sh.k if n_own == rows else sh.k[sh.margin_left:sh.margin_left + n_own]
-        B.slkv_row_lse(p, sh.q_win, k_own, status, (0, n_own), lse_local, scratch, status, stream)
+        B.slkv_cp_row_lse(p, sh.q_win, k_own, status, (0, n_own), lse_local, scratch, ws_lse, status, stream)
     else:
-        lse_local = torch.full((hq, w), float("-inf"), dtype=torch.float32, device=dev)
-    # 2. merged over the ranks
-    lse = torch.empty(1, hq, w, dtype=torch.float32, device=dev)
-    B.slkv_cp_merge_lse(p, comm.all_gather(lse_local), lse, stream)
+        lse_local.fill_(float("-inf"))
+    # 2. merged over the ranks (one rank's are what they are)
+    lse = comm.all_gather(lse_local)
+    if sh.world > 1:
+        parts, lse = lse, torch.empty(1, hq, w, dtype=torch.float32, device=dev)
+        B.slkv_cp_merge_lse(p, parts, lse, stream)
     # 3. pooled scores of the owned rows and the neighbours' margins
     if n_ext > 0:
-        pooled = torch.empty(hkv * n_ext, dtype=torch.float32, device=dev)
-        B.slkv_score(p, sh.q_win, sh.k, status, (0, rows), pooled, scratch, status, stream, lse=lse)
-    else:
-        pooled = torch.zeros(hkv, dtype=torch.float32, device=dev)
+        B.slkv_score_at(p, sh.q_win, sh.k, status, (0, rows), pooled, scratch, ws_score, status, stream, lse)
     # 4. every head's threshold: radix descent on histograms summed over the ranks; the output rows are cleared meanwhile,
     #    a quarter beside each level (every row is whole 16-byte units)
     out_k, out_v = torch.empty(2, max(cap, 1), d, dtype=dt, device=dev).unbind(0)
@@ -147,14 +148,13 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
             comm.all_reduce_sum(hist)
         hist_sum = hist
     # 5. ties in rank order, then this rank's packed rows
-    ties_all = comm.all_gather(totals[hkv:])
-    kept_idx = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
+    ties_all = comm.all_gather(ties)
     threshold = state + 24 * hkv
     B.slkv_cp_emit_counted(p, sh.k, sh.v, rows, pooled, row_stride, sh.margin_left, own, sh.begin, threshold,
                            threshold + 4 * hkv, ties_all, sh.rank, n_win, sh.seq_len - n_win, totals, out_k, out_v,
                            offsets, kept_idx, scratch, ws_emit, status, stream)
     return dict(k_out=out_k, v_out=out_v, offsets=offsets, kept_idx=kept_idx, status=status, pooled=pooled, lse=lse,
-                capacity=cap, keep_alive=(ws, zeroed, ties_all, lse_local))
+                capacity=cap, keep_alive=(buf, ties_all))
 
 
 def stitch_heads(per_rank: Sequence[dict], n_kv_heads: int) -> List[dict]:

@@ -227,7 +227,7 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
   int rc = enqueue_window_stats(pb, path, st, launches);
   if (rc != SLKV_OK) return rc;
   const int passes = pb.lse_opt ? 2 : 3;
-  cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes, nullptr, st, launches)
+  cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes, nullptr, false, st, launches)
                                            : launch_score_simt(pb, status, passes, st, launches);
   if (e != cudaSuccess) return cuda_fail(e);
   return SLKV_OK;
@@ -901,7 +901,7 @@ namespace {
 // slkv_score and slkv_row_lse: the votes pooled into `pooled`, or the rows' log-sum-exp into `lse_out`.
 int score_impl(const slkv_params* p, const void* q_win, const void* k, const int32_t* cu_seqlens_dev,
                const int32_t* cu_seqlens_host, const float* lse_opt, float* pooled, float* lse_out, int32_t* status,
-               void* workspace, size_t workspace_bytes, void* stream) {
+               void* workspace, size_t workspace_bytes, void* stream, bool cleared = false) {
   g_last_launches = 0;
   if (!q_win || !k || !cu_seqlens_dev || (!pooled && !lse_out)) return SLKV_ERR_NULL_PTR;
   Problem pb;
@@ -929,7 +929,7 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
     // row statistics only: pass 1, the window keys' share where the domain has one, then the merge
     rc = enqueue_window_stats(pb, path, st, &launches);
     if (rc != SLKV_OK) return rc;
-    e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_seqlens_host, status, 1, lse_out, st, &launches)
+    e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_seqlens_host, status, 1, lse_out, cleared, st, &launches)
                                  : launch_score_simt(pb, status, 1, st, &launches);
     if (e == cudaSuccess && path != SLKV_PATH_TENSOR) e = launch_merge_lse_simt(pb, lse_out, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
@@ -965,6 +965,14 @@ int slkv_row_lse(const slkv_params* p, const void* q_win, const void* k, const i
   if (!lse_out) return SLKV_ERR_NULL_PTR;
   return score_impl(p, q_win, k, cu_seqlens_dev, cu_seqlens_host, nullptr, nullptr, lse_out, status, workspace,
                     workspace_bytes, stream);
+}
+
+int slkv_cp_row_lse(const slkv_params* p, const void* q_win, const void* k, const int32_t* cu_seqlens_dev,
+                    const int32_t* cu_seqlens_host, float* lse_out, int32_t* status, void* zeroed_workspace,
+                    size_t workspace_bytes, void* stream) {
+  if (!lse_out) return SLKV_ERR_NULL_PTR;
+  return score_impl(p, q_win, k, cu_seqlens_dev, cu_seqlens_host, nullptr, nullptr, lse_out, status, zeroed_workspace,
+                    workspace_bytes, stream, true);
 }
 
 }  // extern "C"

@@ -208,8 +208,9 @@ bool tensor_q_head_inner(const slkv_params& p);
 bool tensor_path_supported(const slkv_params& p);
 int tensor_slot_stride(const Problem& pb);        // split ranges a segment may be shared by, at most
 void set_tensor_trace(void* dev_buf, size_t bytes);
-// passes as launch_score_simt; lse_out (optional, with passes == 1): the rows' log-sum-exps in the problem's lse_units
-cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, int passes, float* lse_out,
+// passes as launch_score_simt; lse_out (optional, with passes == 1): the rows' log-sum-exps in the problem's lse_units;
+// cleared: the workspace is zero (the row sums of a launch of the statistics alone have to be)
+cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, int passes, float* lse_out, bool cleared,
                                 cudaStream_t st, int* launches);
 cudaError_t launch_pool(const Problem& pb, float* pooled, cudaStream_t st, int* launches);
 cudaError_t launch_select(const Problem& pb, const float* pooled, const int32_t* budgets, const int32_t* offsets,
@@ -276,7 +277,7 @@ int score_list_stages(int MT, int halves);
 // The score kernel over a list of layers of one shape: passes 1 = row statistics, 2 = votes from the callers' row
 // statistics, 3 = both; sync: Problem's.
 cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
-                              unsigned long long* sync, cudaStream_t st, int* launches);
+                              unsigned long long* sync, cudaStream_t st, int* launches, bool cleared = false);
 // lse_out null: into the layer's own statistics area
 cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
                                     cudaStream_t st, int* launches);

@@ -783,7 +783,7 @@ int score_list_stages(int MT, int halves) {
 }
 
 cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
-                              unsigned long long* sync, cudaStream_t st, int* launches) {
+                              unsigned long long* sync, cudaStream_t st, int* launches, bool cleared) {
   if (n_layers < 1 || sh.n_cta == 0) return cudaSuccess;             // no history: nothing to score
   if (n_layers > kListMaxLayers) return cudaErrorInvalidValue;
   static thread_local int configured_dev = -1;
@@ -838,7 +838,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     a.passes = 2;
     return launch_pdl_scoped(KID_SCORE_VOTE, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
   }
-  if (passes == 1) {
+  if (passes == 1 && !cleared) {
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
   }

@@ -212,12 +212,12 @@ cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay,
                     lay.lse, lse_out, out_scale);
 }
 
-cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, int passes, float* lse_out,
+cudaError_t launch_score_tensor(const Problem& pb, const int32_t* cu_host, int32_t* status, int passes, float* lse_out, bool cleared,
                                 cudaStream_t st, int* launches) {
   ScorePlan plan;
   cudaError_t e = plan_score_tensor(pb, cu_host, status, &plan);
   if (e != cudaSuccess || plan.sh.n_cta == 0) return e;
-  e = launch_score_list(plan.sh, &plan.lay, 1, passes, pb.sync, st, launches);
+  e = launch_score_list(plan.sh, &plan.lay, 1, passes, pb.sync, st, launches, cleared);
   if (e != cudaSuccess || !lse_out) return e;
   return launch_merge_lse_tensor(plan.sh, plan.lay, lse_out, lse_out_scale(pb), st, launches);
 }

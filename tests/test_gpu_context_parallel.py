@@ -260,3 +260,18 @@ def test_history_only_rows_score_as_the_history_of_a_longer_sequence(path, dtype
     B.slkv_score(prm, qd, kd, cu_dev, cu, pooled2, ws, status, lse=lse)
     torch.cuda.synchronize()
     P.assert_pooled_close(pooled2.cpu().numpy(), ref, cu_pad, Hkv, w)
+
+
+@pytest.mark.parametrize("dt,hq,w,n", [(torch.bfloat16, 8, 32, 5000), (torch.bfloat16, 32, 64, 1500), (torch.float32, 4, 16, 700)])
+def test_row_lse_on_a_zeroed_workspace(dt, hq, w, n):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k = (torch.randn(*s, generator=g, device="cuda").to(dt) for s in ((1, w, hq, 64), (n, 2, 64)))
+    p = B.make_params(q, k, None, w, 7, lse_units=B.SLKV_LSE_LOG2)
+    cu, size = torch.tensor([0, n], dtype=torch.int32, device="cuda"), B.slkv_workspace_bytes(p, [0, n])
+    got = []
+    for ws, fn in ((torch.full((size,), 0x42, dtype=torch.uint8, device="cuda"), B.slkv_row_lse),
+                   (torch.zeros(size, dtype=torch.uint8, device="cuda"), lambda *a: B.slkv_cp_row_lse(*a[:6], a[6], size))):
+        lse = torch.zeros(1, hq, w, device="cuda")
+        fn(p, q, k, cu, [0, n], lse, ws)
+        got.append(lse)
+    assert torch.equal(*got)
