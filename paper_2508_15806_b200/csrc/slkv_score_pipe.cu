@@ -102,6 +102,7 @@ struct ListArgs {
   ScoreLayer lay[kListMaxLayers];
   int n_layers, passes, lag;
   int group_layers, n_groups;  // as in ScoreShape; groups of the whole list
+  int first_layers;            // layers whose statistics are cleared before any CTA adds to some (see fetch_lse)
   WordSync sync;               // counts [n_groups]: CTAs that have published the group's statistics
   unsigned target;             // value a group's count reaches when every CTA has published
   unsigned long long* trace;
@@ -162,8 +163,9 @@ struct Smem {
   __device__ __forceinline__ uint32_t run_empty(int k) const { return bar(2 * kMaxStages + 28 + kRunSlots + (k & (kRunSlots - 1))); }
   __device__ __forceinline__ uint32_t cleared() const { return bar(2 * kMaxStages + 29 + 2 * kRunSlots); }
   __device__ __forceinline__ uint32_t drain() const { return bar(2 * kMaxStages + 28 + 2 * kRunSlots); }   // a wait ran out
+  __device__ __forceinline__ uint32_t rest_cleared() const { return bar(2 * kMaxStages + 30 + 2 * kRunSlots); }
 };
-constexpr int kNumBars = 2 * kMaxStages + 30 + 2 * kRunSlots;
+constexpr int kNumBars = 2 * kMaxStages + 31 + 2 * kRunSlots;
 constexpr int kHeadInts = 9;
 static_assert(kNumBars * 8 + kHeadInts * 4 + 16 <= kBarBytes, "mbarriers");
 constexpr int kRunReaders = 4 + 4 * kWgs;              // arrivals that free a run slot: one per reading thread or warp
@@ -432,7 +434,8 @@ __device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArg
       const int slot = n & 1;
       const bool stats = r.kind == 0 && r.count > 0, publish = r.kind == 0 && r.last && c.both;
       // the epilogue warps have waited for the clearing before their statistics are out; an empty share waits here
-      const bool ready = stats ? mbar_test(c.stat_full(slot), (n >> 1) & 1) : !publish || mbar_test(c.cleared(), 0);
+      bool ready = stats ? mbar_test(c.stat_full(slot), (n >> 1) & 1) : !publish || mbar_test(c.cleared(), 0);
+      if (publish && r.gg == 0) ready = ready && mbar_test(c.rest_cleared(), 0);
       if (__any_sync(0xffffffffu, ready)) {
         if (stats) {
           const unsigned far = c.stat_far[slot];
@@ -504,7 +507,10 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     return __all_sync(0xffffffffu, *c.abort_flag == 0) != 0;
   };
   if (c.both) {
-    // this CTA's part of the groups' counts and the layers' statistics areas is cleared; nobody adds to them before all are
+    // This CTA's part of the groups' counts and the layers' statistics areas is cleared; nobody adds to them before all are.
+    // The layers that come before the first vote phase first: that the others are cleared, too, a CTA says as it publishes
+    // group 0, which its vote phase waits for in every other.  (All layers first: the first sums of 32 layers waited
+    // until 12 us into the launch, a phase and a half.  32 layers of 4001 tokens 129 -> 127 us, of 8000 236 -> 232.)
     for (int i = blockIdx.x + lane * gridDim.x; i < a.n_groups; i += 32 * gridDim.x) __stcg(a.sync.counts() + i, 0u);
     const int words = (int)(stat_clear_bytes(n_seg, c.R) / 4);       // < 2^30; times the CTAs it takes more than 32 bits
     const int w0 = (int)((long long)blockIdx.x * words / gridDim.x), w1 = (int)((long long)(blockIdx.x + 1) * words / gridDim.x);
@@ -514,12 +520,17 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
     const ListArgs* args;
     asm volatile("mov.u64 %0, %1;" : "=l"(args) : "l"(&a));
     const unsigned long long part = lane < a.n_layers ? reinterpret_cast<unsigned long long>(args->lay[lane].part) : 0ull;
-    for (int l = 0; l < a.n_layers; ++l) {
-      unsigned* p = reinterpret_cast<unsigned*>(__shfl_sync(0xffffffffu, part, l));
-      for (int i = w0 + lane; i < w1; i += 32) __stcg(p + i, 0u);
-    }
-    __syncwarp();
+    auto clear = [&](int l0, int l1) {
+      for (int l = l0; l < l1; ++l) {
+        unsigned* p = reinterpret_cast<unsigned*>(__shfl_sync(0xffffffffu, part, l));
+        for (int i = w0 + lane; i < w1; i += 32) __stcg(p + i, 0u);
+      }
+      __syncwarp();
+    };
+    clear(0, a.first_layers);
     if (lane == 0) a.sync.arrive();
+    clear(a.first_layers, a.n_layers);
+    if (lane == 0) mbar_arrive(c.rest_cleared());
     if (!wait_count(-1)) return;
   }
   if (lane == 0) mbar_arrive(c.cleared());
@@ -666,6 +677,7 @@ k_score_list(const __grid_constant__ ListArgs a) {
     abort_sh = 0;
     c.stat_far[0] = c.stat_far[1] = 0;
     mbar_init(c.cleared(), 1);
+    mbar_init(c.rest_cleared(), 1);
     for (int st = 0; st < kMaxStages; ++st) { mbar_init(c.full(st), 1); mbar_init(c.empty(st), 1); }
     for (int u = 0; u < 4; ++u) { mbar_init(c.unit_full(u), 1); mbar_init(c.unit_empty(u), 4); }
     for (int s = 0; s < 2; ++s) {
@@ -809,6 +821,13 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   a.lag = kLagUnits / (per_phase > 0 ? per_phase : 1);
   if (a.lag > a.n_groups - 1) a.lag = a.n_groups - 1;
   if (a.lag < 1) a.lag = 1;
+  // Layers of the phases S(0) .. S(lag); all of them where a CTA may have no share of V(0) to wait for.
+  a.first_layers = n_layers;
+  const long long tiles0 = a.group_layers == 0 ? sh.group_tile[1] : (long long)a.group_layers * sh.total_tiles;
+  if (tiles0 >= sh.n_cta) {
+    const int before = a.group_layers == 0 ? a.lag / sh.n_groups + 1 : (a.lag + 1) * a.group_layers;
+    if (before < n_layers) a.first_layers = before;
+  }
   a.sync.word = sync;
   a.sync.tag = next_launch_tag() & ((1ull << 40) - 1);
   const bool waits_inside = passes == 3;

@@ -145,3 +145,27 @@ def test_a_list_goes_out_before_the_join(hist, w, layers):
     torch.cuda.synchronize()
     assert launches == 2 * ([0] * (layers - 1) + [3]) and B.slkv_last_launch_count() == 0
     assert (off[:, -1] == cap).all() and torch.equal(kept, kept[:1].expand_as(kept))
+
+
+@pytest.mark.parametrize("lens,n_layers,w", [([4001], 32, 32), ([2000, 33], 32, 64), ([9000, 20000], 7, 64), ([70000], 8, 32)])
+def test_statistics_cleared_layer_by_layer(lens, n_layers, w):
+    # layers whose statistics are cleared only after the first ones' are in use, in a workspace full of something else
+    hq, hkv, d = 16, 4, 128
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    xs = [tuple(t.to(DEV) for t in layer(20 + l, lens, hq, hkv, d, w)) for l in range(4)]
+    p = B.make_params(*xs[0], w, 7)
+    cu_dev, bud = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.full((hkv,), w + 30, dtype=torch.int32, device=DEV)
+    cap, n = sum(min(x, w + 30) for x in lens) * hkv, B.slkv_workspace_bytes_overlapped(p, cu)
+    ws = torch.empty(n, dtype=torch.uint8, device=DEV)
+    kv, off, kept = torch.zeros(2, cap, d, dtype=torch.bfloat16, device=DEV), torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.zeros(cap, dtype=torch.int32, device=DEV)
+    scores, status = torch.zeros(4 + 2 * n_layers, B.slkv_pooled_elems(p, cu), device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    for l, x in enumerate(xs):
+        B.slkv_compress(p, *x, cu_dev, cu, bud, *kv, off, kept, ws, scores[l], status)
+    for turn in range(2):
+        ws.fill_(0x42)
+        for l in range(n_layers):
+            B.slkv_compress_overlapped(p, *xs[l % 4], cu_dev, cu, bud, *kv, off, kept, ws, scores[4 + turn * n_layers + l], status)
+        B.slkv_join()
+    assert int(status) == 0
+    for l in range(2 * n_layers):
+        assert torch.equal(scores[4 + l], scores[l % n_layers % 4])
