@@ -135,7 +135,7 @@ static_assert(sizeof(RunDesc) <= 128, "run descriptor");
 struct Smem {
   uint32_t q, k, bar0, tmem;
   int q_half, q_bytes, stage_bytes, n_stages;
-  int R, Rp, MT, halves, k_head_inner, both;
+  int R, Rp, k_head_inner, both;
   float sc, inv_g;
   volatile int* abort_flag;
   RunDesc* runs;               // [kRunSlots]
@@ -166,7 +166,7 @@ struct Smem {
   __device__ __forceinline__ uint32_t rest_cleared() const { return bar(2 * kMaxStages + 30 + 2 * kRunSlots); }
 };
 constexpr int kNumBars = 2 * kMaxStages + 31 + 2 * kRunSlots;
-constexpr int kHeadInts = 9;
+constexpr int kHeadInts = 7;
 static_assert(kNumBars * 8 + kHeadInts * 4 + 16 <= kBarBytes, "mbarriers");
 constexpr int kRunReaders = 4 + 4 * kWgs;              // arrivals that free a run slot: one per reading thread or warp
 
@@ -271,6 +271,7 @@ __device__ __forceinline__ RunDesc take_run(const Smem& c, int k) {
 }
 
 // ---- warp 0, one thread: TMA loads ------------------------------------------------------------------------------
+template <int HALVES>
 __device__ __forceinline__ void producer(const Smem& c) {
   int st = 0, it = 0, n = 0;                                 // stage, tiles so far, runs so far
   uint32_t st_phase = 0;
@@ -282,8 +283,8 @@ __device__ __forceinline__ void producer(const Smem& c) {
   // Q of run number n - 1
   auto load_q = [&]() {
     const uint32_t bar = c.q_full(n - 1), dst = c.q + (uint32_t)(c.q_slot(n - 1) * c.q_bytes);
-    mbar_expect_tx(bar, (uint32_t)(c.halves * c.R * 128));
-    for (int h = 0; h < c.halves; ++h) tma_load_4d(dst + h * c.q_half, q_map, 64 * h, q_y, q_z, q_s, bar);
+    mbar_expect_tx(bar, (uint32_t)(HALVES * c.R * 128));
+    for (int h = 0; h < HALVES; ++h) tma_load_4d(dst + h * c.q_half, q_map, 64 * h, q_y, q_z, q_s, bar);
     q_due = false;
   };
   auto q_free = [&](bool wait) {
@@ -323,7 +324,7 @@ __device__ __forceinline__ void producer(const Smem& c) {
       const uint32_t fb = c.full(st), dst = c.k + (uint32_t)(st * c.stage_bytes);
       mbar_expect_tx(fb, (uint32_t)c.stage_bytes);
       const int ky = c.k_head_inner ? r.g : tok, kz = c.k_head_inner ? tok : r.g;
-      for (int h = 0; h < c.halves; ++h) tma_load_3d_hint(dst + h * kHalfBytes, r.tm_k, 64 * h, ky, kz, fb, policy);
+      for (int h = 0; h < HALVES; ++h) tma_load_3d_hint(dst + h * kHalfBytes, r.tm_k, 64 * h, ky, kz, fb, policy);
       if (++st == c.n_stages) { st = 0; st_phase ^= 1u; }
     }
   }
@@ -346,6 +347,7 @@ __device__ __forceinline__ void producer(const Smem& c) {
 }
 
 // ---- warp 1, one thread: MMAs -------------------------------------------------------------------------------------
+template <int MT, int HALVES>
 __device__ __forceinline__ void issuer(const Smem& c) {
   // statistics: D[row, key] = Q K^T (A = Q, B = K); votes: D[key, row] = K Q^T (A = K, B = Q); a unit per 128-row block
   // of Q (one 256-column product for the votes would read less shared memory, but it takes two units at once and makes
@@ -354,7 +356,7 @@ __device__ __forceinline__ void issuer(const Smem& c) {
                  idesc_v1 = instr_desc(kTileKeys, max(c.Rp - 128, 32));
   const uint64_t q_desc0 = smem_desc(c.q), k_desc0 = smem_desc(c.k);
   const uint64_t q_hi = (uint64_t)(c.q_half >> 4), k_hi = (uint64_t)(kHalfBytes >> 4);
-  const bool two_halves = c.halves == 2;
+  constexpr bool two_halves = HALVES == 2;
   int st = 0, uc = 0, n = 0;                                  // stage, units so far, runs so far
   uint32_t st_phase = 0;
   bool ok = true;
@@ -379,7 +381,7 @@ __device__ __forceinline__ void issuer(const Smem& c) {
       ok = mbar_wait(c.full(st), st_phase, c.abort_flag);
       if (!ok) break;
       const uint64_t kd = k_desc0 + (uint64_t)((st * c.stage_bytes) >> 4);
-      for (int mt = 0; mt < c.MT && ok; ++mt, ++uc) {
+      for (int mt = 0; mt < MT && ok; ++mt, ++uc) {
         ok = unit_free(uc);
         if (!ok) break;
         tc_fence_after();
@@ -387,7 +389,7 @@ __device__ __forceinline__ void issuer(const Smem& c) {
         const uint64_t qd = q_desc + (uint64_t)(mt * ((128 * 128) >> 4));
         if (r.kind == 0) product(d, qd, q_hi, kd, k_hi, idesc_s);
         else product(d, kd, k_hi, qd, q_hi, mt == 0 ? idesc_v0 : idesc_v1);
-        if (mt == c.MT - 1) tc_commit(c.empty(st));            // K stage free once these MMAs have read it
+        if (mt == MT - 1) tc_commit(c.empty(st));            // K stage free once these MMAs have read it
         tc_commit(c.unit_full(uc & 3));
       }
       if (++st == c.n_stages) { st = 0; st_phase ^= 1u; }
@@ -405,6 +407,7 @@ __device__ __forceinline__ void issuer(const Smem& c) {
 
 // ---- warp 2: hands out the runs; announces statistics -----------------------------------------------------------------
 // Whatever is possible next is done: a run slot that has come free is filled, statistics that are out are announced.
+template <int MT>
 __device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArgs& a) {
   const int lane = threadIdx.x & 31;
   int k_out = 0, k_in = 0;                 // runs handed out, runs done with as publisher
@@ -444,7 +447,7 @@ __device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArg
             const size_t at0 = ((size_t)r.seg * stride + r.slot) * c.R;
             for (int row = lane; row < c.R; row += 32) {
               float Z = 0.f, M = 0.f;
-              for (int wg = c.MT == 1 ? 0 : row >> 7; wg < kWgs; wg += c.MT)
+              for (int wg = MT == 1 ? 0 : row >> 7; wg < kWgs; wg += MT)
                 if (far >> (wg * 4 + ((row & 127) >> 5)) & 1u) {
                   const int at = (slot * kWgs + wg) * 128 + (row & 127);
                   stat_add(Z, M, c.stat_z[at], c.stat_m[at]);
@@ -587,6 +590,7 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
 }
 
 // ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
+template <int MT>
 __device__ __forceinline__ void epilogue(const Smem& c) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wg = (threadIdx.x - 128) >> 7, row = threadIdx.x & 127;
@@ -597,7 +601,8 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
   u.abort_flag = c.abort_flag;
   // MT = 1: unit u = tile u, this warpgroup's tiles are wg, wg + 4, ...; MT = 2: tile t has the units 2t (rows 0-127,
   // or the votes' first 128 rows) and 2t + 1
-  const int every = c.MT == 1 ? kWgs : kWgs / 2, log_every = c.MT == 1 ? 2 : 1, mine = c.MT == 1 ? wg : wg >> 1, mt = c.MT == 1 ? 0 : wg & 1;
+  constexpr int every = MT == 1 ? kWgs : kWgs / 2, log_every = MT == 1 ? 2 : 1;
+  const int mine = MT == 1 ? wg : wg >> 1, mt = MT == 1 ? 0 : wg & 1;
   const bool rows_here = mt * 128 + (warp & 3) * 32 < c.R;                // some row of this warp's lanes exists
   int it = 0, units = 0, n_stat = 0, n_vote = 0, n_half = 0;
   for (int k = 0;; ++k) {
@@ -631,7 +636,7 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
       ++n_vote;
       if (!__all_sync(0xffffffffu, ok)) break;
       ok = votes_run(u, units, c.sc, i0, every, r.count, r.n_valid, smem_u32(c.lse + slot * 256 + mt * 128), min(c.Rp - mt * 128, 128),
-                     c.MT == 2 ? mt : -1, c.half_vote + mine * 512, c.half_full(mine, 0), n_half, c.inv_g,
+                     MT == 2 ? mt : -1, c.half_vote + mine * 512, c.half_full(mine, 0), n_half, c.inv_g,
                      [&](int key, float v) { r.vote[key] = v; });
       n_half += n_mine;
       if (!__all_sync(0xffffffffu, ok)) break;
@@ -641,6 +646,11 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
   }
 }
 
+// MT: blocks of 128 query rows (1 or 2); HALVES: 64-element halves of head_dim (1 or 2).  A kernel for each: the code of the warps
+// that do the arithmetic is what the instruction caches have to hold, and a row block's constants are folded into it.  With one
+// kernel for all, 32 layers of 4001 / 8000 / 32k tokens, 128 rows: 123.7 / 225 / 838 us, now 121.1 / 220 / 812; 16000 tokens, 64 rows
+// 376 -> 353; four sequences of 5k - 10k 689 -> 658; 256 rows as before.
+template <int MT, int HALVES>
 __global__ void __launch_bounds__(kListThreads, 1)
 k_score_list(const __grid_constant__ ListArgs a) {
   // Shared memory, all dynamic and 1024-byte aligned (the swizzled tiles need it):
@@ -655,7 +665,7 @@ k_score_list(const __grid_constant__ ListArgs a) {
     return;
   }
   // the tail's place follows from launch parameters; everything the roles use in their loops goes through shared memory
-  unsigned char* tail = smem + sh.halves * (kQTiles * sh.MT * 128 * 128 + sh.n_stages * kHalfBytes);
+  unsigned char* tail = smem + HALVES * (kQTiles * MT * 128 * 128 + sh.n_stages * kHalfBytes);
   uint32_t& tmem_base_sh = *reinterpret_cast<uint32_t*>(tail + kBarBytes - 16);
   int& abort_sh = *reinterpret_cast<int*>(tail + kBarBytes - 12);
   volatile int* head = reinterpret_cast<volatile int*>(tail + kBarBytes - 16 - kHeadInts * 4);
@@ -689,15 +699,15 @@ k_score_list(const __grid_constant__ ListArgs a) {
     }
     for (int k = 0; k < kQTiles; ++k) { mbar_init(c.q_full(k), 1); mbar_init(c.q_empty(k), 1); }
     for (int k = 0; k < kRunSlots; ++k) { mbar_init(c.run_full(k), 1); mbar_init(c.run_empty(k), kRunReaders); }
-    head[0] = sh.R; head[1] = sh.Rp; head[2] = sh.MT; head[3] = sh.halves;
-    head[4] = sh.n_stages; head[5] = sh.k_head_inner;
-    head[6] = a.passes == 3; head[7] = __float_as_int(sh.scale_log2); head[8] = __float_as_int(1.0f / (float)sh.G);
+    head[0] = sh.R; head[1] = sh.Rp;
+    head[2] = sh.n_stages; head[3] = sh.k_head_inner;
+    head[4] = a.passes == 3; head[5] = __float_as_int(sh.scale_log2); head[6] = __float_as_int(1.0f / (float)sh.G);
     mbar_init(c.drain(), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // rows of the Q tile beyond R are never written by TMA: keep them zero
-  if (sh.R != sh.MT * 128) {
-    for (int i = tid; i < kQTiles * sh.halves * sh.MT * 128 * 128 / 16; i += kListThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+  if (sh.R != MT * 128) {
+    for (int i = tid; i < kQTiles * HALVES * MT * 128 * 128 / 16; i += kListThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
@@ -708,12 +718,12 @@ k_score_list(const __grid_constant__ ListArgs a) {
   __syncthreads();
   tc_fence_after();
   c.tmem = tmem_base_sh;
-  c.R = head[0]; c.Rp = head[1]; c.MT = head[2]; c.halves = head[3];
-  c.n_stages = head[4]; c.k_head_inner = head[5];
-  c.both = head[6]; c.sc = __int_as_float(head[7]); c.inv_g = __int_as_float(head[8]);
-  c.q_half = c.MT * 128 * 128;
-  c.q_bytes = c.halves * c.q_half;
-  c.stage_bytes = c.halves * kHalfBytes;
+  c.R = head[0]; c.Rp = head[1];
+  c.n_stages = head[2]; c.k_head_inner = head[3];
+  c.both = head[4]; c.sc = __int_as_float(head[5]); c.inv_g = __int_as_float(head[6]);
+  c.q_half = MT * 128 * 128;
+  c.q_bytes = HALVES * c.q_half;
+  c.stage_bytes = HALVES * kHalfBytes;
   c.q = smem_u32(smem);
   c.k = c.q + (uint32_t)(kQTiles * c.q_bytes);
   // Everything above touched only this CTA's own resources, and so does all that follows up to the first load of a tile and
@@ -725,18 +735,18 @@ k_score_list(const __grid_constant__ ListArgs a) {
     if (lane == 0) {
       pdl_wait();
       trace_mark(a.trace, 1);
-      producer(c);
+      producer<HALVES>(c);
     }
   } else if (warp == 1) {
-    if (lane == 0) issuer(c);
+    if (lane == 0) issuer<MT, HALVES>(c);
   } else if (warp == 2) {
     if (sh.tab.n_inline == 0) pdl_wait();              // a kernel before this one writes the tables
-    scheduler_publisher(c, a);
+    scheduler_publisher<MT>(c, a);
   } else if (warp == 3) {
     pdl_wait();
     fetch_lse(c, a);
   } else {
-    epilogue(c);
+    epilogue<MT>(c);
   }
 
   tc_fence_before();
@@ -765,6 +775,8 @@ thread_local size_t g_trace_bytes = 0;
 // A phase should last about this many tiles-times-row-blocks per CTA before the phase that needs its results is due:
 // publishing, the other CTAs' counters and the merge take about 5 us, a unit about 0.6 us.
 constexpr int kLagUnits = 10;
+
+typedef void (*Kern)(const ListArgs);
 
 // A launch of the statistics pass alone finds the row sums cleared.
 cudaError_t clear_stats(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, cudaStream_t st) {
@@ -798,12 +810,15 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
                               unsigned long long* sync, cudaStream_t st, int* launches, bool cleared) {
   if (n_layers < 1 || sh.n_cta == 0) return cudaSuccess;             // no history: nothing to score
   if (n_layers > kListMaxLayers) return cudaErrorInvalidValue;
-  static thread_local int configured_dev = -1;
+  const Kern kernel = sh.MT == 1 ? (sh.halves == 1 ? k_score_list<1, 1> : k_score_list<1, 2>)
+                                 : (sh.halves == 1 ? k_score_list<2, 1> : k_score_list<2, 2>);
+  static thread_local int configured_on[2][2] = {{-1, -1}, {-1, -1}};
+  int& configured_dev = configured_on[sh.MT - 1][sh.halves - 1];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(k_score_list, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     configured_dev = dev;
   }
@@ -850,19 +865,19 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     a.passes = 1;
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
-    e = launch_pdl_scoped(KID_SCORE_LSE, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
+    e = launch_pdl_scoped(KID_SCORE_LSE, kernel, sh.n_cta, kListThreads, smem, st, launches, a);
     if (e != cudaSuccess) return e;
     for (int i = 0; i < n_layers && e == cudaSuccess; ++i) e = launch_merge_lse_tensor(sh, lay[i], nullptr, 1.f, st, launches);
     if (e != cudaSuccess) return e;
     a.passes = 2;
-    return launch_pdl_scoped(KID_SCORE_VOTE, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
+    return launch_pdl_scoped(KID_SCORE_VOTE, kernel, sh.n_cta, kListThreads, smem, st, launches, a);
   }
   if (passes == 1 && !cleared) {
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
   }
   const int kid = passes == 1 ? KID_SCORE_LSE : (n_layers > 1 ? KID_SCORE_LIST : (passes == 2 ? KID_SCORE_VOTE : KID_SCORE_FUSED));
-  if (!waits_inside) return launch_pdl_scoped(kid, k_score_list, sh.n_cta, kListThreads, smem, st, launches, a);
+  if (!waits_inside) return launch_pdl_scoped(kid, kernel, sh.n_cta, kListThreads, smem, st, launches, a);
   for (int attempt = 0; attempt < 2; ++attempt) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sh.n_cta);
@@ -879,7 +894,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     cudaError_t le;
     {
       LaunchScope scope(kid, st, launches);
-      le = cudaLaunchKernelEx(&cfg, k_score_list, a);
+      le = cudaLaunchKernelEx(&cfg, kernel, a);
     }
     if (le == cudaSuccess) {
       if (cs == 0) cs = 1;
