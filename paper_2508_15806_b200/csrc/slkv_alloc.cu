@@ -10,19 +10,20 @@
 //
 // What bounds it: latency.  The order of the sums is part of the result, so one chain of N dependent fp64 additions stays
 // (5 ns each); everything else runs on all threads: the weights (two fp64 divisions each) are in shared memory before the chain
-// starts, and the largest remainders are found by counting them in 1024 parts of [0, 1) -- of a few hundred remainders one or
-// two share a part.  In a graph, us: 256 heads 70.5 with all of it in one thread, 8.3 with all pairs of remainders compared, 5.7
-// now; 1024 heads (all pairs) 61.1 -> 10.5; 1536 (a radix descent) 19.5 -> 13.8; 3072 29.4 -> 23.1.
+// starts, and the largest remainders are found by counting them in as many parts of [0, 1) as there are threads -- of a few
+// hundred remainders one or two share a part -- or, up to 96 heads, in pairs.  A thread per head up to 1024: a barrier of 1024
+// threads costs a quarter of a microsecond more than one of 256.  In a graph, us, with all of it in one thread 256 heads 70.5;
+// with 1024 threads and all pairs of remainders compared / 1024 threads and parts / as it is: 16 heads 4.1 / - / 3.1, 64: 4.3 / 4.8
+// / 3.3, 100: 5.0 / 5.0 / 4.2, 256: 8.2 / 5.6 / 4.9, 384: 12.9 / 6.4 / 5.7, 512: 19.2 / 7.1 / 6.5, 1024: 61.1 / 10.5.
 #include "slkv_internal.cuh"
 
 namespace slkv {
 namespace {
 
-constexpr int kAllocThreads = 1024;
+constexpr int kMost = 16384;           // heads
 constexpr int kPairsMost = 96;         // heads up to which all pairs of remainders are compared: us with the pairs / counted in
-                                       // parts 32 heads 4.2 / 4.5, 64 4.5 / 4.8, 96 5.0 / 5.0, 128 5.25 / 4.9, 256 8.3 / 5.7
-constexpr int kParts = kAllocThreads;  // parts of [0, 1) the remainders are counted in
-constexpr int kSmemMost = (16384 + 1024) * 8 + 16384 * 5;      // 16384 heads in 1024 layers
+                                       // parts, 1024 threads, 32 heads 4.2 / 4.5, 64 4.5 / 4.8, 96 5.0 / 5.0, 128 5.25 / 4.9
+constexpr int kSmemMost = (kMost + 1024) * 8 + kMost * 5;      // 16384 heads in 1024 layers
 constexpr int kListMost = 256;         // remainders of one part up to which they are ranked by counting (2 us); where more are
                                        // (nearly) equal, a radix descent over all of them takes eight levels of about 1 us
 
@@ -56,19 +57,24 @@ __device__ __forceinline__ double ordered_sum(const double* v, int n) {
   return acc;
 }
 
+// Over a CTA of T threads.
+template <int T>
 __device__ long long block_sum_ll(long long v, long long* red) {
   __syncthreads();
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  long long t = red[threadIdx.x & 31];
+  long long t = (threadIdx.x & 31) < T / 32 ? red[threadIdx.x & 31] : 0;
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   return t;
 }
 
-__global__ void __launch_bounds__(kAllocThreads, 1)
+// COUNT: remainders counted in parts, else by pairs.  Up to MOST heads.
+template <int T, bool COUNT, int MOST>
+__global__ void __launch_bounds__(T, 1)
 k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total, const AllocOpts opt,
         int32_t* __restrict__ budgets, int32_t* __restrict__ status) {
+  constexpr int kParts = T;              // parts of [0, 1) the remainders are counted in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = L * H;
   double* wt = reinterpret_cast<double*>(smem_raw);        // [N] INF_sc, then the weights (0 once a head is filled), then
@@ -77,19 +83,19 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
   double* La = wt + N;                                     // [L] layer sums
   int* fl = reinterpret_cast<int*>(La + L);                // [N] dynamic parts
   unsigned char* active = reinterpret_cast<unsigned char*>(fl + N);   // [N] head still below the cap
-  __shared__ long long red[kAllocThreads / 32];
+  __shared__ long long red[T / 32];
   __shared__ double sh_Ls, sh_W;
-  __shared__ int hist[256], parts[kParts], list[kListMost];
+  __shared__ int hist[COUNT ? 256 : 1], parts[COUNT ? kParts : 1], list[COUNT ? kListMost : 1];
   __shared__ int sh_digit, sh_above, sh_count, sh_same;
   const int tid = threadIdx.x;
   const long long D = total - (long long)N * fixed;
   const bool within = opt.within_layer != 0;
-  if (N > kPairsMost) parts[tid] = 0;
+  if (COUNT) parts[tid] = 0;
   pdl_launch_dependents();
   pdl_wait();
 
   int bad = 0;
-  for (int a = tid; a < N; a += kAllocThreads) {
+  for (int a = tid; a < N; a += T) {
     const float x = inf[a];
     bad |= !(x >= 0.0f) || !(x <= 3.402823466e38f);                  // negative, NaN or infinite
     wt[a] = (double)x;
@@ -99,7 +105,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     if (tid == 0 && status) *status = SLKV_ERR_NEG_INF_SC;
     return;
   }
-  for (int i = tid; i < L; i += kAllocThreads) La[i] = ordered_sum(wt + (size_t)i * H, H);
+  for (int i = tid; i < L; i += T) La[i] = ordered_sum(wt + (size_t)i * H, H);
   __syncthreads();
   if (tid == 0) sh_Ls = ordered_sum(La, L);
   __syncthreads();
@@ -108,7 +114,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
 
   if (opt.paper_rounding) {
     // Algorithm 2's own last line: C = floor(max(0, fixed + D * w) + 0.5), clipped at the cap; nothing is normalised
-    for (int a = tid; a < N; a += kAllocThreads) {
+    for (int a = tid; a < N; a += T) {
       const double w = uniform ? __ddiv_rn(1.0, (double)N) : head_weight(wt[a], La[a / H], Ls, H, within);
       const double b = __dadd_rn((double)fixed, __dmul_rn((double)D, w));
       long long c = (long long)floor(__dadd_rn(fmax(0.0, b), 0.5));
@@ -117,7 +123,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     }
     return;
   }
-  for (int a = tid; a < N; a += kAllocThreads) wt[a] = uniform ? 1.0 : head_weight(wt[a], La[a / H], Ls, H, within);
+  for (int a = tid; a < N; a += T) wt[a] = uniform ? 1.0 : head_weight(wt[a], La[a / H], Ls, H, within);
 
   // Heads that would rise above the cap are filled and taken out (their weight becomes 0, which leaves the ordered sum
   // of the others as it is), the rest share what is left, until none does (without a cap: one round, nobody is taken
@@ -136,12 +142,12 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     if (flat) W = (double)n_active;
     if (room < 0 || n_active == 0) break;
     long long filled = 0;
-    for (int a = tid; a < N; a += kAllocThreads) {
+    for (int a = tid; a < N; a += T) {
       if (!active[a]) continue;
       const double q = __ddiv_rn(__dmul_rn((double)d_rem, flat ? 1.0 : wt[a]), W);
       if (q >= (double)room) { active[a] = 0; wt[a] = 0.0; fl[a] = (int)room; ++filled; }
     }
-    filled = block_sum_ll(filled, red);
+    filled = block_sum_ll<T>(filled, red);
     if (filled == 0) break;
     d_rem -= filled * room;
     n_active -= (int)filled;
@@ -149,7 +155,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
 
   // quotas, floors, remainders of the heads still below the cap
   long long fsum = 0;
-  for (int a = tid; a < N; a += kAllocThreads) {
+  for (int a = tid; a < N; a += T) {
     unsigned long long kk = 0;
     if (active[a]) {
       const double q = __ddiv_rn(__dmul_rn((double)d_rem, flat ? 1.0 : wt[a]), W);
@@ -160,17 +166,17 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     }
     key[a] = kk;
   }
-  long long Rleft = d_rem - block_sum_ll(fsum, red);                  // its barriers also publish key[] and fl[]
+  long long Rleft = d_rem - block_sum_ll<T>(fsum, red);                  // its barriers also publish key[] and fl[]
   if (n_active > 0 && Rleft >= n_active) {                            // not reachable in exact arithmetic
     const long long each = Rleft / n_active;
-    for (int a = tid; a < N; a += kAllocThreads)
+    for (int a = tid; a < N; a += T)
       if (active[a]) fl[a] += (int)each;
     Rleft -= each * n_active;
   }
-  if (Rleft > 0 && N <= kPairsMost) {
+  if (!COUNT && Rleft > 0) {
     // largest remainder first, ties -> lower index: head a gets +1 iff fewer than Rleft heads precede it
     int lanes = 1;                                                    // threads per head, neighbours in a warp
-    while (lanes < 32 && 2 * lanes * N <= kAllocThreads) lanes *= 2;
+    while (lanes < 32 && 2 * lanes * N <= T) lanes *= 2;
     const int a = tid / lanes, sub = tid % lanes;
     const unsigned long long ka = a < N ? key[a] : 0ull;
     int rank = 0;
@@ -181,11 +187,11 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
       }
     for (int o = 1; o < lanes; o *= 2) rank += __shfl_xor_sync(0xffffffffu, rank, o);
     if (ka && sub == 0 && rank < Rleft) fl[a] += 1;
-  } else if (Rleft > 0) {
+  } else if (COUNT && Rleft > 0) {
     // the Rleft-th largest remainder lies in one of 1024 equal parts of [0, 1); what lies in a part above it gets +1, what lies
     // in the same part is ranked by counting
     auto part_of = [&](unsigned long long k) { return min((int)(__longlong_as_double((long long)(k - 1ull)) * (double)kParts), kParts - 1); };
-    for (int a = tid; a < N; a += kAllocThreads)
+    for (int a = tid; a < N; a += T)
       if (key[a]) atomicAdd(&parts[part_of(key[a])], 1);
     __syncthreads();
     const int lane0 = tid & 31, warp0 = tid >> 5, mine = parts[kParts - 1 - tid];           // from the top
@@ -202,7 +208,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     const int same = sh_same, part = sh_digit;
     if (same <= kListMost) {
       const int need = (int)Rleft - sh_above;
-      for (int a = tid; a < N; a += kAllocThreads) {
+      for (int a = tid; a < N; a += T) {
         if (!key[a]) continue;
         const int p = part_of(key[a]);
         if (p > part) fl[a] += 1;
@@ -227,7 +233,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
       for (int shift = 56; shift >= 0; shift -= 8) {
         if (tid < 256) hist[tid] = 0;
         __syncthreads();
-        for (int a = tid; a < N; a += kAllocThreads) {
+        for (int a = tid; a < N; a += T) {
           const unsigned long long k = key[a];
           if (k && (k & mask) == prefix) atomicAdd(&hist[(int)(k >> shift) & 255], 1);
         }
@@ -255,7 +261,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
         __syncthreads();
       }
       // keys above `prefix` and, in index order, the first `need` equal to it
-      const int per = (N + kAllocThreads - 1) / kAllocThreads;
+      const int per = (N + T - 1) / T;
       const int a0 = min(tid * per, N), a1 = min(a0 + per, N);
       int eq = 0;
       for (int a = a0; a < a1; ++a) eq += key[a] == prefix;
@@ -279,9 +285,9 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     // floors overshot the pool (rounding): take one back from the smallest remainders, ties -> higher index
     __syncthreads();
     long long taken = 0;
-    int dec[(16384 + kAllocThreads - 1) / kAllocThreads];
+    int dec[(MOST + T - 1) / T];
     int nd = 0;
-    for (int a = tid; a < N; a += kAllocThreads, ++nd) {
+    for (int a = tid; a < N; a += T, ++nd) {
       dec[nd] = 0;
       if (!active[a] || fl[a] <= 0) continue;
       int rank = 0;
@@ -293,12 +299,12 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     }
     __syncthreads();
     nd = 0;
-    for (int a = tid; a < N; a += kAllocThreads, ++nd)
+    for (int a = tid; a < N; a += T, ++nd)
       if (dec[nd]) fl[a] -= 1;
-    Rleft += block_sum_ll(taken, red);
+    Rleft += block_sum_ll<T>(taken, red);
   }
   __syncthreads();
-  for (int a = tid; a < N; a += kAllocThreads) budgets[a] = fl[a] + fixed;
+  for (int a = tid; a < N; a += T) budgets[a] = fl[a] + fixed;
 }
 
 }  // namespace
@@ -307,12 +313,17 @@ cudaError_t launch_alloc(const float* inf, int n_layers, int n_heads, int fixed,
                          int paper_rounding, long long cap, int32_t* budgets, int32_t* status, cudaStream_t st) {
   const size_t n = (size_t)n_layers * n_heads;
   const size_t smem = (n + n_layers) * sizeof(double) + n * (sizeof(int) + 1);
+  // A thread per head (below kPairsMost several); half the threads for 257-512 heads take 0.5 us longer.
+  const bool many = n > 512;
+  auto* const kernel = n <= kPairsMost ? k_alloc<256, false, kPairsMost>
+                       : n <= 256 ? k_alloc<256, true, 256> : n <= 512 ? k_alloc<512, true, 512> : k_alloc<1024, true, kMost>;
+  const int threads = n <= 256 ? 256 : n <= 512 ? 512 : 1024;
   static thread_local int configured_dev = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(k_alloc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
+  if (many && configured_dev != dev) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
     if (e != cudaSuccess) return e;
     configured_dev = dev;
   }
@@ -320,7 +331,7 @@ cudaError_t launch_alloc(const float* inf, int n_layers, int n_heads, int fixed,
   opt.within_layer = within_layer; opt.paper_rounding = paper_rounding; opt.cap = cap;
   int launches = 0;
   LaunchScope scope(KID_ALLOC, st, &launches);
-  return launch_pdl(k_alloc, dim3(1), dim3(kAllocThreads), smem, st, 1, inf, n_layers, n_heads, fixed, total, opt,
+  return launch_pdl(kernel, dim3(1), dim3(threads), smem, st, 1, inf, n_layers, n_heads, fixed, total, opt,
                     budgets, status);
 }
 

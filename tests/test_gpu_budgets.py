@@ -51,7 +51,7 @@ def test_edge_tables():
         assert st == 0 and np.array_equal(got, O.alloc_budgets(inf.numpy(), fixed, total))
 
 
-@pytest.mark.parametrize("n", [95, 96, 97, 256, 257, 300, 1024, 1025])
+@pytest.mark.parametrize("n", [95, 96, 97, 256, 257, 300, 512, 513, 1024, 1025])
 def test_remainders_ranked_by_pairs_parts_and_digits(n):
     # all remainders alike (one part holds them all: up to 256 are listed, more go by digits), two values, and any
     rng = np.random.default_rng(n)
