@@ -422,7 +422,8 @@ def run_cuda(args):
     rows_avg = sum(L["rows"] for L in layers) / nl
     alg = {"k_score_fused": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_list": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_lse": k_scan + q_bytes, "k_score_vote": k_scan + q_bytes + 4 * hkv * n_hist,
            "k_pool": 8 * hkv * n_hist, "k_select": 4 * hkv * n_hist + 4 * rows_avg,
-           "k_gather": 4 * rows_avg * d * e + 4 * rows_avg, "k_setup": 0}
+           "k_gather": 4 * rows_avg * d * e + 4 * rows_avg, "k_setup": 0,
+           "k_layer": k_scan + q_bytes + 4 * rows_avg * d * e}           # a short layer's steps in one launch
     kern = {}
     prof_total = sum(ms for ms, _ in per_kernel.values()) or 1.0
     for name, (ms, cnt) in per_kernel.items():
