@@ -7,7 +7,8 @@
 //   1. with 16 or 32 positions per thread, a histogram of every 16th or 32nd score: the ranks that the k-th largest has among
 //      these, give or take four standard deviations, bound it from both sides (where there are none, nothing bounds it);
 //   2. a histogram of the scores between the bounds, 2048 bins, 64 to an octave; the bin with the k-th largest;
-//   3. where that bin's scores fit a list of 512 (mostly), they are ranked by counting, else a histogram of that bin, and so on.
+//   3. where that bin's scores fit a list of 512, or of a score for each of 256 threads (mostly), they are ranked by counting,
+//      else a histogram of that bin, and so on.
 // Then an ordered compaction from bit masks.  Integer counters only: the result does not depend on timing, and not on the
 // sample either.
 // What bounds it: a chain of some ten CTA-wide steps of 0.2-0.6 us, and at 32 positions per thread instructions.  Bracketing

@@ -13,7 +13,7 @@ namespace cg = cooperative_groups;
 
 constexpr int kMaxRadius = 4;                         // pool_kernel <= 9: four values on either side are enough
 constexpr int kBins = 2048;
-constexpr int kList = 512;                            // scores that are ranked by counting
+constexpr int kList = 512;                            // scores that are ranked by counting, at most; a thread for each
 constexpr unsigned kAll = 0xffffffffu;
 // First level's bins: 64 to an octave from 2^-24 up to 2^8 (a vote is at most the window, 256), the scores below in bin 0,
 // whatever lies above in the last.
@@ -80,6 +80,8 @@ template <int T, int IT, bool CLUSTER, int BAR>
 __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsigned (&key)[IT], unsigned valid, bool mine,
                                                   uint4* shelf, int n, int k_keep, int rank, int CS, int& o_mine) {
   constexpr int kWarps = T / 32, kPer = kBins / T;      // bins per thread
+  constexpr int kRanked = kList < T ? kList : T;        // a bin of more scores goes through another level of bins
+  static_assert(kRanked <= T && kRanked <= kList && kPer % 2 == 0 && kWarps <= 32, "a thread per listed score, whole int2 of bins");
   constexpr bool kSample = IT > 8;
   const int lane = tid & 31, wid = tid >> 5;
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(T) : "memory"); };
@@ -228,7 +230,7 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
     }
     first = false;
     // the bin's scores go on; where they fit, in a list of the cluster's first CTA (their order does not matter)
-    const bool listed = m_bin <= kList && lo != hi;
+    const bool listed = m_bin <= kRanked && lo != hi;
     if (mine) {
       unsigned in_bin = 0;
       if (kSample) {
@@ -261,7 +263,7 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
         for (int i = tid; i < m_bin; i += T) sh_.list[i] = list0[i];
         sync();
       }
-      int log_p = 5;                                      // 2^log_p lanes per score
+      int log_p = 5;                                      // 2^log_p lanes per score; m_bin <= T: one at least
       while ((m_bin << log_p) > T) --log_p;
       const int i = tid >> log_p, P = 1 << log_p, part = tid & (P - 1);
       if (wid << 5 >> log_p < m_bin) {                    // some score for this warp

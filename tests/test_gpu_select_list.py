@@ -80,3 +80,52 @@ def test_a_sample_that_misleads(n, sign):
     for step in (16, 32):
         odd = lambda k: torch.where(torch.arange(len(k), device=DEV).view(-1, 1, 1) % step == step // 2, k * 0.05 + sign, k * 0.05 - sign)   # noqa: E731,B023
         run([n + 4], 3, 4, [300, n // 4, n - n // 10], 1, B.SLKV_POOL_MAX, k_fn=odd)
+
+
+def short_keys(kind):
+    """Keys of a segment whose scores share first-level bins: all equal, nearly uniform, in runs, in a trend, or all but a few so
+    small (below 2^-24) that the lowest bin holds them."""
+    at = lambda k: torch.arange(len(k), device=DEV)                                              # noqa: E731
+    return {"equal": lambda k: k[:1].expand_as(k).contiguous(), "flat": lambda k: k * 0.1, "flatter": lambda k: k * 0.01,
+            "periodic": lambda k: k[at(k) % 7], "pairs": lambda k: k[at(k) // 2] * 0.1,
+            "ordered": lambda k: torch.sort(k, dim=0).values * 0.2,
+            "tiny": lambda k: torch.where(at(k).view(-1, 1, 1) < 32, k * 40.0, k)}[kind]
+
+
+@pytest.mark.parametrize("n", [200, 255, 256, 257, 258, 300, 400, 511, 512, 513, 600, 768, 1000, 1020, 1021, 1022])
+@pytest.mark.parametrize("kind", ["equal", "flat", "flatter", "periodic", "pairs", "ordered", "tiny"])
+def test_short_segments_in_one_bin(n, kind):
+    for pool in (1, 7):
+        run([n + 4], 3, 4, [4 + n // 10, 4 + n // 2, n + 1], pool, B.SLKV_POOL_MAX, k_fn=short_keys(kind))
+    run([n + 4], 3, 4, [4 + n // 10, 4 + n // 2, n + 1], 5, B.SLKV_POOL_AVG, k_fn=short_keys(kind))
+
+
+@pytest.mark.parametrize("n", [256, 257, 400, 512, 513, 1000])
+@pytest.mark.parametrize("kind", ["equal", "flat", "tiny"])
+def test_short_segments_of_many_rows_and_in_lists(n, kind):
+    # 160 query rows per KV head, which only the list kernels take; one call, and a list of three layers
+    w, hq, hkv, d, pool = 40, 8, 2, 64, 5
+    g = torch.Generator(device=DEV).manual_seed(n)
+    q = torch.randn(1, w, hq, d, generator=g, device=DEV).bfloat16()
+    ks = [short_keys(kind)(torch.randn(n + w, hkv, d, generator=g, device=DEV)).bfloat16() for _ in range(3)]
+    p, cu, budgets = B.make_params(q, ks[0], ks[0], w, pool), [0, n + w], [w + n // 8, w + n - 3]
+    cap = sum(budgets)
+    cu_dev, bud = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.tensor(budgets, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes_overlapped(p, cu), dtype=torch.uint8, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    for call, layers in ((B.slkv_compress, ks[:1]), (B.slkv_compress_overlapped, ks)):
+        res = []
+        for k in layers:
+            out = torch.zeros(2, cap, d, dtype=torch.bfloat16, device=DEV)
+            off, kept = torch.zeros(hkv + 1, dtype=torch.int32, device=DEV), torch.full((cap,), -1, dtype=torch.int32, device=DEV)
+            pooled = torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV)
+            call(p, q, k, k, cu_dev, cu, bud, out[0], out[1], off, kept, ws, pooled, status)
+            res.append((pooled, kept, off, out))                   # a list writes them when it goes out
+        B.slkv_join()
+        torch.cuda.synchronize()
+        assert int(status) == 0
+        for pooled, kept, off, _ in res:
+            sc, o = pooled.cpu().numpy().astype(np.float64), off.tolist()
+            for h in range(hkv):
+                ref = O.select_topk(sc[h * n:(h + 1) * n], budgets[h] - w)
+                assert kept[o[h]:o[h + 1]].tolist() == ref.tolist() + list(range(n, n + w)), h
