@@ -203,6 +203,8 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
       pdl_wait();
       const SegmentRows r = segment_rows(a.tail, x);
       if (lane == 0) f.rows = r;
+      __syncwarp();
+      asm volatile("bar.sync 3, %0;" ::"n"(kLayerThreads + 32) : "memory");
     }
   } else {
     const int t = tid - 128, wg = t >> 7, row = t & 127;
@@ -298,7 +300,8 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
                 });
       publish_for_copy();
     }
-    sync();
+    // with warp 2: a CTA without tiles may be here before the budgets are
+    asm volatile("bar.sync 3, %0;" ::"n"(kLayerThreads + 32) : "memory");
     if (rank == 0) {
       mbar_wait(smem_u32(&f.votes_bar), 0, abort_flag);
     } else if (t == 0 && n_t > 0) {

@@ -123,6 +123,36 @@ def test_many_calls_in_a_row(n):
     same(both(q, k, v, cu, 32, 7, [64 + 100 * h for h in range(8)], calls=1000))
 
 
+@pytest.mark.parametrize("lens", [[100], [300], [700], [1000], [1180], [40, 1100, 33, 200], [600, 34, 8000]])
+def test_rows_of_ctas_without_tiles(lens):
+    # Segments of fewer tiles than their cluster has CTAs, log-sum-exps handed in: a CTA without tiles gets to its rows with
+    # nothing to wait for but the budgets, which another warp reads -- from HBM, while the log-sum-exps lie in L2.
+    w, hq, hkv, d = 32, 8, 4, 64
+    q, k, v, cu = inputs(sum(lens), lens, hq, hkv, d, w)
+    p = B.make_params(q, k, v, w, 7, lse_units=B.SLKV_LSE_LOG2)
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    lse = torch.zeros(len(lens), hq, w, device=DEV)
+    B.slkv_row_lse(p, q, k, cu_dev, cu, lse, ws)
+    sweep = torch.empty(1 << 28, dtype=torch.uint8, device=DEV)
+    rng = np.random.default_rng(sum(lens))
+    for _ in range(40):
+        budgets = rng.integers(1, max(lens) + 40, hkv).tolist()
+        bud = torch.tensor(budgets, dtype=torch.int32, device=DEV)
+        cap = sum(min(n, max(c, w)) for n in lens for c in budgets)
+        res = []
+        for pooled in (None, torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV)):
+            ko, vo = (torch.zeros(cap, d, dtype=k.dtype, device=DEV) for _ in range(2))
+            off, kept = torch.full((len(lens) * hkv + 1,), -1, dtype=torch.int32, device=DEV), torch.full((cap,), -1, dtype=torch.int32, device=DEV)
+            status = torch.zeros(1, dtype=torch.int32, device=DEV)
+            sweep.zero_()
+            lse.add_(0.0)
+            B.slkv_compress(p, q, k, v, cu_dev, cu, bud, ko, vo, off, kept, ws, pooled, status, lse=lse)
+            assert pooled is not None or B.slkv_last_launch_count() == 1
+            res.append((off, kept, ko, vo, status))
+        same(res)
+
+
 # ---- fp32 -------------------------------------------------------------------------------------------------------------
 def check_fp32(hq, hkv, d, w, lens, pool=5, mode=B.SLKV_POOL_MAX, domain=B.SLKV_HISTORY, q_fn=None, rtol=1e-5, one_launch=True):
     """Scores and row statistics of the one launch (without and with supplied statistics) against the general path's, the kept
