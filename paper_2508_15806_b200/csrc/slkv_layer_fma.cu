@@ -4,7 +4,8 @@
 //
 // As slkv_layer_tc.cu: row sums, votes and kept positions go from CTA to CTA in bulk copies, nothing is cleared, nothing
 // polled.  A CTA takes whole blocks of 32 keys, forms their scores 32 keys x 8 or 16 rows per warp out of shared memory (the
-// same operations in the same order as k_score_simt: a row's statistics are the same bit for bit) and keeps them for the votes.
+// same operations in the same order as k_score_simt: a row's statistics and a key's vote are the same bit for bit) and keeps them
+// for the votes.
 // What bounds it: latency at the small sizes (8 heads, 1024 positions, 16 rows, head_dim 64: 24.6 us from a stream as three
 // launches with two meetings of all CTAs, 11.7 here: keys 0.7, products 1.0, exchange 1, log-sum-exps 0.9, votes 1.4, selection
 // 2.4, rows 1.5), shared-memory reads of the operands beyond: a clock per register of a warp, twice what the FMAs take.
@@ -296,22 +297,50 @@ k_layer_fma(const __grid_constant__ LayerFmaArgs a) {
   }
   sync();
 
-  // ---- votes: a key per thread, its rows split over groups of threads where there are threads left
+  // ---- votes.  A key's rows are added up in one order whatever CTA it lies in, and that of k_score_simt: four rows 4 apart to a
+  // part, the parts in a binary tree.  A key per thread, or a subtree of it where there are threads left (1008 keys of 16 rows: as
+  // quick as rows dealt out to the threads in turn, whose sums depended on how many keys a CTA has).
   {
     const int span = n_b * kBlock;                             // keys and padding
-    int groups = 1;
-    while (2 * groups * span <= kLayerThreads && groups < 8) groups *= 2;
+    int parts = 4, groups = 1;                                 // parts: 16 rows have four
+    while (4 * parts < a.R) parts *= 2;
+    while (2 * groups * span <= kLayerThreads && groups < min(parts, 8)) groups *= 2;
+    const int per = parts / groups;
     for (int j0 = 0; j0 < span; j0 += kLayerThreads / groups) {
       const int grp = groups > 1 ? tid / span : 0, key = groups > 1 ? tid - grp * span : j0 + tid;
       const bool on = key < span && grp < groups;
       float v = 0.f;
-      if (on && key < n_here)
-        for (int r = grp; r < a.R; r += groups) v += exp2f(sc[r * a.s_pitch + key] - f.lse[r]);
+      if (on && key < n_here) {
+        float left[5];                                         // level l: the sum of 2^l parts that waits for its right half
+        for (int i = 0; i < per; ++i) {
+          const int part = grp * per + i, r0 = (part >> 2) * 16 + (part & 3);
+          float e[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int r = min(r0 + 4 * j, a.R - 1);
+            e[j] = exp2f(sc[r * a.s_pitch + key] - f.lse[r]);
+          }
+          v = r0 < a.R ? e[0] : 0.f;
+#pragma unroll
+          for (int j = 1; j < 4; ++j) v += r0 + 4 * j < a.R ? e[j] : 0.f;
+          if (per == 1) break;
+          bool carry = true;
+#pragma unroll
+          for (int l = 0; l < 5; ++l) {
+            if (carry && (i >> l & 1)) v = left[l] + v;
+            else if (carry) { left[l] = v; carry = false; }
+          }
+        }
+      }
       if (groups > 1) {
         if (on && grp > 0) f.part[(grp - 1) * span + key] = v;
         sync();
-        if (on && grp == 0)
-          for (int g = 1; g < groups; ++g) v += f.part[(g - 1) * span + key];
+        if (on && grp == 0) {
+          auto p = [&](int g) { return f.part[(g - 1) * span + key]; };
+          v += p(1);
+          if (groups > 2) v += p(2) + p(3);
+          if (groups > 4) v += (p(4) + p(5)) + (p(6) + p(7));
+        }
       }
       if (on && grp == 0) votes[vote_at<IT>(key0 + key)] = key < n_here ? v / (float)a.G : pad;
       if (groups > 1) break;

@@ -217,3 +217,33 @@ def test_fp32_beyond_its_range():
     # log-sum-exps of some 750 in log2 units, rounded to 2^-14: a vote shows that twice
     for domain in (B.SLKV_HISTORY, B.SLKV_ALL_CAUSAL):
         check_fp32(4, 2, 64, 8, [900], domain=domain, q_fn=far, rtol=1e-4)
+
+
+@pytest.mark.parametrize("hq,hkv,d,w", [(8, 8, 64, 16), (4, 2, 64, 5), (2, 1, 128, 17), (8, 4, 64, 33), (2, 1, 64, 64)])
+@pytest.mark.parametrize("n", [300, 700, 735, 1400, 1450, 2600, 2740])
+def test_fp32_equal_keys_have_equal_scores(hq, hkv, d, w, n):
+    # The CTAs of a segment hold blocks of keys that differ by one in number, which the threads of a CTA share out differently:
+    # a key's score is the same wherever it lies, bit for bit, and the same as the general path's.
+    for domain, every in ((B.SLKV_HISTORY, 1), (B.SLKV_ALL_CAUSAL, 37)):
+        q, k, v, cu = inputs(n + w, [n + w], hq, hkv, d, w, torch.float32)
+        k[:n] = k[torch.arange(n, device=DEV) % every]
+        p = B.make_params(q, k, v, w, 1, softmax_domain=domain)
+        cu_dev, status = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+        ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+        own, general = (torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) for _ in range(2))
+        B.slkv_score(p, q, k, cu_dev, cu, own, ws, status)
+        took_one = B.slkv_last_launch_count() == 1
+        assert took_one or n > 735                                 # with many rows the longer ones are the general path's
+        scores = own.view(hkv, n)
+        assert (scores == scores[:, torch.arange(n, device=DEV) % every]).all()
+        budgets = [w + 5 + 90 * h for h in range(hkv)]
+        off, kept, _, _, st = both(q, k, v, cu, w, 1, budgets, domain=domain, one_launch=took_one)[0]
+        for h in range(hkv):
+            ref = O.select_topk(scores[h].cpu().numpy().astype(np.float64), min(n, 5 + 90 * h)).tolist()
+            assert kept[int(off[h]):int(off[h + 1])].tolist() == ref + list(range(n, n + w))
+        assert every > 1 or ref == list(range(len(ref)))
+        cap = int(off[-1])
+        out = torch.zeros(2, cap, d, device=DEV)
+        B.slkv_compress(p, q, k, v, cu_dev, cu, torch.tensor(budgets, dtype=torch.int32, device=DEV), out[0], out[1],
+                        torch.zeros(hkv + 1, dtype=torch.int32, device=DEV), torch.zeros(cap, dtype=torch.int32, device=DEV), ws, general, status)
+        assert int(status) == 0 and int(st) == 0 and torch.equal(own, general)
