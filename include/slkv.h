@@ -445,11 +445,13 @@ int slkv_trace_set_buffer(void* dev_buf, size_t bytes);
 
 /*
  * Test hook for the bounded waits (no counterpart in the paper).  Where the CTAs of a launch wait for one another
- * (the counters between the two passes of the score kernel), every wait gives up after one second, sets SLKV_ERR_DEVICE_TIMEOUT in the
- * call's status word, releases what the CTA holds and returns.  With the hook armed (on != 0) the next such launch made
- * by the calling thread waits for one arrival more than there are CTAs -- on = 2: where its CTAs wait for the clearing of
- * the statistics, else where they wait for the statistics -- so that exactly this path runs: the call's results are then incomplete and its status word says so; the calls after it are unaffected.  One-shot: the launch
- * that takes it disarms it.
+ * (the counters between the two passes of the score kernel; row sums and votes between the CTAs of a segment where one launch does
+ * a short layer), every wait gives up after one second, sets SLKV_ERR_DEVICE_TIMEOUT in the call's status word, releases what the CTA
+ * holds and returns.  With the hook armed (on != 0) the next such launch made by the calling thread waits for one arrival more than
+ * there are -- on = 1: where the CTAs of a score launch wait for the statistics, 2: for their clearing, 3: where those of a
+ * one-launch layer wait for the row sums, 4: for the votes -- so that exactly this path runs: the call's results are then incomplete
+ * and its status word says so; the calls after it are unaffected.  While it is armed with 1 or 2, short layers go the way of the
+ * others.  One-shot: the launch that takes it disarms it.
  */
 int slkv_debug_expire_next_wait(int on);
 

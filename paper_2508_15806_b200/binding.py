@@ -275,7 +275,8 @@ def slkv_row_lse(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_de
 
 
 def slkv_debug_expire_next_wait(on=True) -> None:
-    """False / 0: off; True / 1: the wait for the statistics; 2: the wait for their clearing."""
+    """False / 0: off; True / 1: the wait for the statistics; 2: the wait for their clearing; of a layer in one launch, 3: the wait
+    for the row sums, 4: the wait for the votes."""
     lib().slkv_debug_expire_next_wait(int(on))
 
 

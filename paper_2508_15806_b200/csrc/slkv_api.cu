@@ -233,8 +233,8 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
   return SLKV_OK;
 }
 
-// CTAs per segment where one launch does the whole layer, else 0.  A wait that is to run out (slkv_debug_expire_next_wait) is one
-// of the kernels whose CTAs wait for words in memory; these have none.
+// CTAs per segment where one launch does the whole layer, else 0.  A wait for words in memory that is to run out
+// (slkv_debug_expire_next_wait) is one of the other kernels'.
 int layer_cluster(const Problem& pb, int path) {
   if (next_wait_expires()) return 0;
   return path == SLKV_PATH_TENSOR ? layer_tc_cluster(pb) : layer_fma_cluster(pb);
@@ -629,7 +629,7 @@ int slkv_last_launch_count(void) { return g_last_launches; }
 int slkv_version(void) { return 300; }
 
 int slkv_debug_expire_next_wait(int on) {
-  expire_next_wait(on == 2 ? 2 : on != 0);
+  expire_next_wait(on >= 2 && on <= 4 ? on : on != 0);
   return SLKV_OK;
 }
 

@@ -72,11 +72,13 @@ __device__ __forceinline__ SegmentRows segment_rows(const LayerTail& a, const Se
 
 // The first CTA, kLayerThreads threads (numbered tid, named barrier BAR): pools the segment's votes (place p at
 // votes[vote_at<IT>(p)], places -4 .. -1 and n .. n + 3 hold the padding), writes the scores where they are wanted and leaves
-// the kept history positions in ascending order at the start of votes' memory (votes - kLead).
+// the kept history positions in ascending order at the start of votes' memory (votes - kLead).  gave_up, in shared
+// memory: set where a wait of these threads has run out; nothing is selected then (sh may lie where loads still land).
 template <int IT>
 __device__ __forceinline__ int vote_at(int p) { return (p >> kLogItems<IT>) * (IT + 4) + (p & (IT - 1)); }
 template <int IT, int BAR>
-__device__ __forceinline__ void layer_select(const LayerTail& a, const Segment& x, int k_keep, float* votes, SelShared& sh, int tid) {
+__device__ __forceinline__ void layer_select(const LayerTail& a, const Segment& x, int k_keep, float* votes, SelShared& sh, int tid,
+                                             const volatile int* gave_up) {
   constexpr int kPer = kBins / kLayerThreads;
   const bool choose = a.select && k_keep > 0 && k_keep < x.n, max_mode = a.pool_mode == SLKV_POOL_MAX;
   if (choose) {
@@ -105,6 +107,7 @@ __device__ __forceinline__ void layer_select(const LayerTail& a, const Segment& 
   }
   if (!choose) return;
   asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(kLayerThreads) : "memory");
+  if (*gave_up) return;                         // written in front of the barrier, if at all
   int o;
   const unsigned kept = select_places<kLayerThreads, IT, false, BAR>(sh, tid, key, valid, mine, reinterpret_cast<uint4*>(votes + vote_at<IT>(i0)),
                                                                      x.n, k_keep, 0, 1, o);
@@ -112,7 +115,8 @@ __device__ __forceinline__ void layer_select(const LayerTail& a, const Segment& 
   for (unsigned m = kept; m != 0; m &= m - 1) *dst++ = i0 + __ffs(m) - 1;
 }
 
-// Every CTA, kLayerThreads threads: its share of the segment's rows.  stage: the first CTA's list of kept positions.
+// Every CTA, kLayerThreads threads: its share of the segment's rows.  stage: the first CTA's list of kept positions; where that CTA
+// has given up there is none, and whatever lies there is held inside the sequence.
 template <int LANES>
 __device__ __forceinline__ void layer_gather_rows(const LayerTail& a, const Segment& x, const SegmentRows r, const int* stage, int tid, int rank,
                                                   int CS) {
@@ -130,7 +134,7 @@ __device__ __forceinline__ void layer_gather_rows(const LayerTail& a, const Segm
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
       const int i = i0 + u * CS * kRows;
-      if (i < rows) pos[u] = i >= r.k_keep ? x.len - x.n_win + (i - r.k_keep) : (choose ? stage[i] : i);
+      if (i < rows) pos[u] = i >= r.k_keep ? x.len - x.n_win + (i - r.k_keep) : (choose ? (int)min((unsigned)stage[i], (unsigned)x.len - 1u) : i);
     }
 #pragma unroll
     for (int u = 0; u < kFly; ++u)

@@ -27,6 +27,7 @@ struct LayerFmaArgs {
   LseSource lse;
   WindowArgs win;              // Q, K and their strides, too
   int all_causal, stats;       // stats 0: the caller's log-sum-exps
+  int expire;                  // diagnostics: 1 the wait for the row sums runs out, 2 the one for the votes
   int G, R, q_rows, s_pitch;   // rows of Q's and pitch of the scores' shared memory
   int chunk;                   // keys that are loaded together, whole blocks; two chunks fit, or one that is all of a CTA's
   int32_t* status;
@@ -37,8 +38,8 @@ __device__ __forceinline__ unsigned long long now() {
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded (1 s): false when the wait ran out.
-__device__ __forceinline__ bool bar_wait(const void* bar, int32_t* status) {
+// Bounded (1 s): *gave_up is set, and the status, when the wait ran out.
+__device__ __forceinline__ void bar_wait(const void* bar, volatile int* gave_up, int32_t* status) {
   const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
@@ -47,11 +48,12 @@ __device__ __forceinline__ bool bar_wait(const void* bar, int32_t* status) {
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0, 100;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(b) : "memory");
-    if (ok) return true;
+    if (ok) return;
     if (it == 0) t0 = now();
     if ((it & 63u) == 63u && now() - t0 > 1000ull * 1000ull * 1000ull) {
+      *gave_up = 1;
       if (status) atomicExch(status, (int)SLKV_ERR_DEVICE_TIMEOUT);
-      return false;
+      return;
     }
   }
 }
@@ -65,12 +67,12 @@ template <int D, int IT> struct FmaShared {
   alignas(16) float2 win[kMaxRows];            // the window keys' share (maximum, sum)
   float lse[kMaxRows];
   float part[kMaxScores / kBlock];             // sums of a block's keys [block][row]; the votes' row groups
-  unsigned long long sums_bar, votes_bar;
+  unsigned long long sums_bar, votes_bar, max_bar, far_bar;
   SegmentRows rows;
-  int far_here;
+  int far_here, gave_up;
   // then Q [q_rows][kPitch], the scores [R][s_pitch] and the keys [chunk or 2 chunk][kPitch], whose memory is later used by
   union Later {
-    struct { double z[kLayerMaxCluster][kMaxRows]; float row_max[kLayerMaxCluster][kMaxRows]; } beyond;   // scores beyond fp32's range
+    struct alignas(16) { double z[kLayerMaxCluster][kMaxRows]; float row_max[kLayerMaxCluster][kMaxRows]; } beyond;   // scores beyond fp32's range
     SelShared select;                                                                                  // the first CTA
   };
 };
@@ -100,15 +102,20 @@ k_layer_fma(const __grid_constant__ LayerFmaArgs a) {
   const bool win = a.stats && a.all_causal && x.n > 0;
   constexpr int vote_bytes = kBlock / IT * (IT + 4) * 4;       // of a block, as they lie in shared memory
   float* votes = f.votes_mem + kLead;
+  auto expect = [&](const void* b, int bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)), "r"(bytes) : "memory");
+  };
   pdl_launch_dependents();
   if (tid == 0) {
-    f.far_here = 0;
-    for (const void* b : {(const void*)&f.sums_bar, (const void*)&f.votes_bar})
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    auto expect = [&](const void* b, int bytes) {
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)), "r"(bytes) : "memory");
+    f.far_here = f.gave_up = 0;
+    auto init = [&](const void* b, int count) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)), "r"(count) : "memory");
     };
+    init(&f.sums_bar, 1 + (a.expire == 1));
+    init(&f.votes_bar, 1 + (a.expire == 2));
+    init(&f.max_bar, 1);
+    init(&f.far_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     expect(&f.sums_bar, (CS - 1) * (int)sizeof(typename F::Sums) + (win ? (window_blocks - my_blocks) * kWinRows * 8 : 0));
     if (rank == 0) expect(&f.votes_bar, (blocks - n_b) * vote_bytes);
   }
@@ -235,20 +242,28 @@ k_layer_fma(const __grid_constant__ LayerFmaArgs a) {
     } else {
       cluster_wait();
     }
-    bar_wait(&f.sums_bar, a.status);
+    bar_wait(&f.sums_bar, &f.gave_up, a.status);
     sync();
+    // The same in every CTA, and without meetings of them all, which a CTA that gives up would have to come to as well.
     bool far = false;
-    for (int c = 0; c < CS; ++c) far |= f.all[c].far != 0;     // the same in every CTA
+    for (int c = 0; c < CS; ++c) far |= f.all[c].far != 0;
+    far = far && f.gave_up == 0;                               // else they need not all be there
+    auto to_all = [&](const void* row, int bytes, const void* bar) {
+      publish_for_copy();
+      sync();
+      if (tid == rank) expect(bar, (CS - 1) * bytes);
+      else if (tid < CS) copy_to_cta(row, row, bytes, bar, tid);
+      bar_wait(bar, &f.gave_up, a.status);
+    };
     if (far) {
       // some block's sum left fp32's range: the rows' maxima, then sums relative to them
       for (int r = warp; r < a.R; r += kWarps) {
         float m = -INFINITY;
         for (int j = lane; j < n_here; j += 32) m = fmaxf(m, sc[r * a.s_pitch + j]);
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-        if (lane < CS) *cluster.map_shared_rank(&later.beyond.row_max[rank][r], lane) = m;
+        if (lane == 0) later.beyond.row_max[rank][r] = m;
       }
-      cluster_arrive();
-      cluster_wait();
+      to_all(later.beyond.row_max[rank], sizeof(later.beyond.row_max[0]), &f.max_bar);
       for (int u = warp; u < n_b * ((a.R + 3) / 4); u += kWarps) {           // a block and four rows per warp
         const int b = u / ((a.R + 3) / 4), r = u % ((a.R + 3) / 4) * 4 + (lane >> 3);
         float m = -INFINITY, v = 0.f;
@@ -266,10 +281,9 @@ k_layer_fma(const __grid_constant__ LayerFmaArgs a) {
       if (row < a.R) {
         double z = 0.0;
         for (int b = 0; b < n_b; ++b) z += (double)f.part[b * a.R + row];
-        for (int c = 0; c < CS; ++c) *cluster.map_shared_rank(&later.beyond.z[rank][row], c) = z;
+        later.beyond.z[rank][row] = z;
       }
-      cluster_arrive();
-      cluster_wait();
+      to_all(later.beyond.z[rank], sizeof(later.beyond.z[0]), &f.far_bar);
     }
     if (row < a.R) {
       float M = 0.f;
@@ -349,13 +363,13 @@ k_layer_fma(const __grid_constant__ LayerFmaArgs a) {
   }
   sync();
   if (rank == 0) {
-    bar_wait(&f.votes_bar, a.status);
+    bar_wait(&f.votes_bar, &f.gave_up, a.status);
   } else if (tid == 0 && n_b > 0) {
     float* mine = votes + vote_at<IT>(key0);
     copy_to_cta(mine, mine, n_b * vote_bytes, &f.votes_bar, 0);
   }
   const SegmentRows r = f.rows;
-  if (rank == 0) layer_select<IT, 0>(a.tail, x, r.k_keep, votes, later.select, tid);
+  if (rank == 0) layer_select<IT, 0>(a.tail, x, r.k_keep, votes, later.select, tid, &f.gave_up);
   cluster_arrive();
   cluster_wait();
   if (a.tail.select) layer_gather(a.tail, x, r, reinterpret_cast<const int*>(cluster.map_shared_rank(f.votes_mem, 0)), tid, rank, CS);
@@ -447,6 +461,7 @@ cudaError_t launch_layer_fma(const Problem& pb, int cs, const TailLayer* tail, f
   a.s_pitch = score_pitch(pb, cs);
   a.chunk = chunk_for(pb, cs);
   a.status = status;
+  a.expire = take_expire_next_layer_wait(a.stats != 0);
   const bool small = few_positions(pb);
   if (pb.p.head_dim == 64) return small ? launch<64, 8>(pb, cs, a, st, launches) : launch<64, 16>(pb, cs, a, st, launches);
   return small ? launch<128, 8>(pb, cs, a, st, launches) : launch<128, 16>(pb, cs, a, st, launches);

@@ -33,6 +33,7 @@ struct LayerArgs {
   LseSource lse;
   WindowArgs win;
   int all_causal, passes;      // passes: 3, or 2: the caller's log-sum-exps
+  int expire;                  // diagnostics: 1 the wait for the row sums runs out, 2 the one for the votes
   int G, R, Rp, halves, n_stages, q_head_inner, k_head_inner;
   float scale_log2;
   int32_t* status;
@@ -95,8 +96,8 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
     for (int u = 0; u < 4; ++u) { mbar_init(unit_full(u), 1); mbar_init(unit_empty(u), 4); }
     mbar_init(q_full, 1);
     mbar_init(drain, 1);
-    mbar_init(smem_u32(&f.sums_bar), 1);
-    mbar_init(smem_u32(&f.votes_bar), 1);
+    mbar_init(smem_u32(&f.sums_bar), 1 + (a.expire == 1));
+    mbar_init(smem_u32(&f.votes_bar), 1 + (a.expire == 2));
     if (stats) mbar_expect_tx(smem_u32(&f.sums_bar), (uint32_t)((CS - 1) * sizeof(typename Far<IT>::Sums) +
                                                                  (a.all_causal && x.n > 0 ? (window_blocks - my_blocks) * kWinRows * 8 : 0)));
     if (rank == 0) mbar_expect_tx(smem_u32(&f.votes_bar), (uint32_t)((tiles - n_t) * vote_bytes));
@@ -309,7 +310,7 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
       copy_to_cta(mine, mine, n_t * vote_bytes, &f.votes_bar, 0);
     }
     const SegmentRows r = f.rows;
-    if (rank == 0) layer_select<IT, 1>(a.tail, x, r.k_keep, votes, *reinterpret_cast<SelShared*>(smem), t);
+    if (rank == 0) layer_select<IT, 1>(a.tail, x, r.k_keep, votes, *reinterpret_cast<SelShared*>(smem), t, abort_flag);
     cluster_arrive();                                                                      // 1
     cluster_wait();
     if (a.tail.select) layer_gather(a.tail, x, r, reinterpret_cast<const int*>(cluster.map_shared_rank(f.votes_mem, 0)), t, rank, CS);
@@ -426,6 +427,7 @@ cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, fl
   a.halves = p.head_dim / 64;
   a.scale_log2 = kLog2e / sqrtf((float)p.head_dim);
   a.status = status;
+  a.expire = take_expire_next_layer_wait(a.passes == 3);
   const bool small = pb.max_hist <= 8 * kLayerThreads;
   a.n_stages = small ? layer_stages<8>(a.halves) : layer_stages<16>(a.halves);
   const size_t smem = small ? layer_smem<8>(a.halves, a.n_stages) : layer_smem<16>(a.halves, a.n_stages);

@@ -247,3 +247,37 @@ def test_fp32_equal_keys_have_equal_scores(hq, hkv, d, w, n):
         B.slkv_compress(p, q, k, v, cu_dev, cu, torch.tensor(budgets, dtype=torch.int32, device=DEV), out[0], out[1],
                         torch.zeros(hkv + 1, dtype=torch.int32, device=DEV), torch.zeros(cap, dtype=torch.int32, device=DEV), ws, general, status)
         assert int(status) == 0 and int(st) == 0 and torch.equal(own, general)
+
+
+# ---- waits that run out -------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("dt,scale", [(torch.bfloat16, 1.0), (torch.bfloat16, 40.0), (torch.float32, 1.0), (torch.float32, 40.0)])
+@pytest.mark.parametrize("on,supplied", [(3, False), (4, False), (4, True)])
+def test_a_wait_that_runs_out_is_reported(dt, scale, on, supplied):
+    # One arrival too many is expected where a segment's CTAs wait for one another: they give up after a second, the status says
+    # so, whatever is written lies in the outputs, and the calls after it are right -- with scores beyond fp32's range, too, whose
+    # CTAs meet twice more.
+    w, hq, hkv, d, n = 16, 8, 4, 64, 1400
+    q, k, v, cu = inputs(17, [n, 30, 500], hq, hkv, d, w, dt, scale)
+    p = B.make_params(q, k, v, w, 7, lse_units=B.SLKV_LSE_LOG2)
+    cu_dev, status = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    lse = None
+    if supplied:
+        lse = torch.zeros(3, hq, w, device=DEV)
+        B.slkv_row_lse(p, q, k, cu_dev, cu, lse, ws, status)
+    budgets = [40, 700, 16, 333]
+    bud = torch.tensor(budgets, dtype=torch.int32, device=DEV)
+    rows = sum(min(a, max(c, w)) for a in (n, 30, 500) for c in budgets)
+    out = torch.full((2, rows + 64, d), 9.0, dtype=dt, device=DEV)
+    off, kept = torch.zeros(3 * hkv + 1, dtype=torch.int32, device=DEV), torch.full((rows + 64,), -7, dtype=torch.int32, device=DEV)
+    assert int(status) == 0
+    B.slkv_debug_expire_next_wait(on)
+    B.slkv_compress(p, q, k, v, cu_dev, cu, bud, out[0, :rows], out[1, :rows], off, kept[:rows], ws, None, status, lse=lse)
+    assert B.slkv_last_launch_count() == 1
+    torch.cuda.synchronize()
+    assert int(status) == B.ERR["DEVICE_TIMEOUT"]
+    assert (out[:, rows:] == 9.0).all() and (kept[rows:] == -7).all()
+    a = both(q, k, v, cu, w, 7, budgets, lse=lse)
+    if scale == 1.0:
+        same(a)
+    assert int(a[0][4]) == 0 and int(a[1][4]) == 0 and torch.equal(a[0][0], a[1][0])
