@@ -127,11 +127,9 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
         B.slkv_cp_row_lse(p, sh.q_win, k_own, status, (0, n_own), lse_local, scratch, ws_lse, status, stream)
     else:
         lse_local.fill_(float("-inf"))
-    # 2. merged over the ranks (one rank's are what they are)
-    lse = comm.all_gather(lse_local)
-    if sh.world > 1:
-        parts, lse = lse, torch.empty(1, hq, w, dtype=torch.float32, device=dev)
-        B.slkv_cp_merge_lse(p, parts, lse, stream)
+    # 2. merged over the ranks
+    lse = torch.empty(1, hq, w, dtype=torch.float32, device=dev)
+    B.slkv_cp_merge_lse(p, comm.all_gather(lse_local), lse, stream)
     # 3. pooled scores of the owned rows and the neighbours' margins
     if n_ext > 0:
         B.slkv_score_at(p, sh.q_win, sh.k, status, (0, rows), pooled, scratch, ws_score, status, stream, lse)

@@ -228,6 +228,22 @@ def test_edges_of_the_counted_slices_and_rows_nothing_is_packed_into(n_hist, wor
     P.assert_selection_valid(gpu, ref, [0, L], bud, w, k, v)
 
 
+def test_one_rank_goes_the_way_of_several():
+    # the row statistics a rank returns are merged ones of its own, not the communicator's buffer
+    class Keeping(ThreadComm):
+        def all_gather(self, t):
+            self.got = [*getattr(self, "got", []), super().all_gather(t)]
+            return self.got[-1]
+
+    q, k, v = (x.to(DEV) for x in rand_seq(8, 2, 32, 3000, seed=4, d=64))
+    comm = Keeping(ThreadComm.Shared(1), 0)
+    o = CP.compress_rank(CP.shard_of(q, k, v, 32, 7, 0, 1), torch.tensor([100, 700], dtype=torch.int32, device=DEV), 7, comm)
+    parts = comm.got[0]
+    assert int(o["status"]) == 0 and torch.equal(o["lse"], parts)
+    parts.zero_()
+    assert bool((o["lse"] != 0).all())
+
+
 @pytest.mark.parametrize("path,dtype,d,w,Hq,Hkv", [(B.SLKV_PATH_TENSOR, torch.bfloat16, 128, 32, 8, 2),
                                                    (B.SLKV_PATH_SIMT, torch.float32, 64, 16, 8, 8)])
 def test_history_only_rows_score_as_the_history_of_a_longer_sequence(path, dtype, d, w, Hq, Hkv):
