@@ -105,21 +105,23 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
     p = B.make_params(sh.q_win, sh.k, sh.v, w, pool_kernel, pool_mode, score_path, softmax_domain, B.SLKV_LSE_LOG2)
     p.history_only = 0 if sh.last else 1
 
-    # One buffer, zero at the start, for all scratch and all outputs but the packed rows: what the steps add to (row sums,
-    # histograms, totals) is cleared by one launch in front of them all, and a view is a third of an allocation.
+    # One buffer for all scratch, zero at the start: what the steps add to (row sums, histograms, totals) is cleared by one launch
+    # in front of them all.  Another for the small outputs, which a caller keeps without any scratch, and without the scores.
     n_own = own + n_win
     has_keys = own > 0 or (sh.last and softmax_domain == B.SLKV_ALL_CAUSAL)
     ws_score = B.slkv_workspace_bytes(p, (0, rows)) if n_ext > 0 else 0
     ws_lse = 0 if not has_keys else (ws_score if n_own == rows and n_ext > 0 else B.slkv_workspace_bytes(p, (0, n_own)))
     ws_emit = B.slkv_cp_workspace_bytes(hkv, own, max(cap, 1))
     state_bytes = -(-32 * hkv // 256) * 256                    # [4][2][hkv]: every head's prefix and need after each level
-    sizes = ((state_bytes + max(ws_score, ws_lse, ws_emit)) // 4, 3 * 2048 * hkv, hkv, hkv, hkv + 1, 1, hq * w,
-             hkv * row_stride, max(cap, 1))
+    sizes = ((state_bytes + max(ws_score, ws_lse, ws_emit)) // 4, 3 * 2048 * hkv, hkv, hkv, hq * w)
     buf = torch.zeros(sum(sizes), dtype=torch.int32, device=dev)
-    ws, hists, totals, ties, offsets, status, lse_local, pooled, kept_idx = buf.split(sizes)
+    ws, hists, totals, ties, lse_local = buf.split(sizes)
+    out_sizes = (max(cap, 1), hq * w, hkv + 1, 1)
+    kept_idx, lse, offsets, status = torch.zeros(sum(out_sizes), dtype=torch.int32, device=dev).split(out_sizes)
+    pooled = (torch.empty if n_ext > 0 else torch.zeros)(hkv * row_stride, dtype=torch.float32, device=dev)
     state = ws.data_ptr()
     scratch = state + state_bytes
-    lse_local, pooled = lse_local.view(torch.float32).view(hq, w), pooled.view(torch.float32)
+    lse_local, lse = lse_local.view(torch.float32).view(hq, w), lse.view(torch.float32).view(1, hq, w)
 
     # 1. the rows' log-sum-exp over the keys this rank owns (the last rank's range is an ordinary sequence tail)
     if has_keys:
@@ -128,7 +130,6 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
     else:
         lse_local.fill_(float("-inf"))
     # 2. merged over the ranks
-    lse = torch.empty(1, hq, w, dtype=torch.float32, device=dev)
     B.slkv_cp_merge_lse(p, comm.all_gather(lse_local), lse, stream)
     # 3. pooled scores of the owned rows and the neighbours' margins
     if n_ext > 0:

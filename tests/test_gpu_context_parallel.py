@@ -244,6 +244,18 @@ def test_one_rank_goes_the_way_of_several():
     assert bool((o["lse"] != 0).all())
 
 
+@pytest.mark.parametrize("world", [1, 3])
+def test_results_that_are_kept_hold_no_scratch(world):
+    # each result's memory is its own and that of others no larger than it, K's and V's rows together
+    q, k, v = rand_seq(8, 2, 32, 9000, seed=5, d=64)
+    for o in run_ranks(world, q, k, v, [100, 700], 32, 7):
+        size = {x: o[x].numel() * o[x].element_size() for x in ("offsets", "kept_idx", "status", "pooled", "lse", "k_out", "v_out")}
+        held = {x: o[x].untyped_storage().nbytes() for x in size}
+        assert held["pooled"] <= size["pooled"] and held["k_out"] <= 2 * size["k_out"] and held["v_out"] <= 2 * size["v_out"]
+        small = sum(size[x] for x in ("offsets", "kept_idx", "status", "lse"))
+        assert all(held[x] <= small for x in ("offsets", "kept_idx", "status", "lse"))
+
+
 @pytest.mark.parametrize("path,dtype,d,w,Hq,Hkv", [(B.SLKV_PATH_TENSOR, torch.bfloat16, 128, 32, 8, 2),
                                                    (B.SLKV_PATH_SIMT, torch.float32, 64, 16, 8, 8)])
 def test_history_only_rows_score_as_the_history_of_a_longer_sequence(path, dtype, d, w, Hq, Hkv):
