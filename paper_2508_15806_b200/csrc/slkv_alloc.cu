@@ -21,8 +21,9 @@ namespace slkv {
 namespace {
 
 constexpr int kMost = 16384;           // heads
-constexpr int kPairsMost = 96;         // heads up to which all pairs of remainders are compared: us with the pairs / counted in
-                                       // parts, 1024 threads, 32 heads 4.2 / 4.5, 64 4.5 / 4.8, 96 5.0 / 5.0, 128 5.25 / 4.9
+constexpr int kPairsMost = 96;         // heads up to which all pairs of remainders are compared: us in a graph with the pairs / counted
+                                       // in parts, 256 threads, 32 heads 3.2 / 3.6, 64 3.4 / 3.8, 80 4.0 / 4.1, 96 4.1 / 4.1, 112 4.5 /
+                                       // 4.3, 128 4.5 / 4.2, 160 6.1 / 4.5, 256 7.9 / 4.9
 constexpr int kSmemMost = (kMost + 1024) * 8 + kMost * 5;      // 16384 heads in 1024 layers
 constexpr int kListMost = 256;         // remainders of one part up to which they are ranked by counting (2 us); where more are
                                        // (nearly) equal, a radix descent over all of them takes eight levels of about 1 us
@@ -188,7 +189,7 @@ k_alloc(const float* __restrict__ inf, int L, int H, int fixed, long long total,
     for (int o = 1; o < lanes; o *= 2) rank += __shfl_xor_sync(0xffffffffu, rank, o);
     if (ka && sub == 0 && rank < Rleft) fl[a] += 1;
   } else if (COUNT && Rleft > 0) {
-    // the Rleft-th largest remainder lies in one of 1024 equal parts of [0, 1); what lies in a part above it gets +1, what lies
+    // the Rleft-th largest remainder lies in one of kParts equal parts of [0, 1); what lies in a part above it gets +1, what lies
     // in the same part is ranked by counting
     auto part_of = [&](unsigned long long k) { return min((int)(__longlong_as_double((long long)(k - 1ull)) * (double)kParts), kParts - 1); };
     for (int a = tid; a < N; a += T)

@@ -12,6 +12,7 @@ namespace {
 
 thread_local int g_last_cuda_error = 0;
 thread_local int g_last_launches = 0;
+thread_local int g_expire_next_layer_wait = 0;
 
 // ---- per-kernel timing (off by default) -----------------------------------------------------------
 struct TimedLaunch { int kid; cudaEvent_t a, b; };
@@ -135,11 +136,12 @@ bool list_supported(const Problem& pb) {
 
 // Layers of a list.  A list costs some 23 us beside its layers (pipeline fill and tail, selections and gathers that nothing
 // runs beside), and its layers wait for the last of them to be called: it goes out when it holds about 0.4 ms of work, 32768
-// products of 128 keys x 128 rows, or eight layers.  Steps of 32 layers, us in a row / by themselves from an idle GPU, with 32, 16, 8 and 4
+// products of 128 keys x 128 rows in both passes, or eight layers (with log-sum-exps handed in, one pass: half as long).  Steps of 32 layers, us in a row / by themselves from an idle GPU, with 32, 16, 8 and 4
 // layers to a list:
 //   4001 tokens, 128 rows    132 / 197    154 / 191    202 / 228    329 / 348
 //   32768 tokens, 128 rows   734 / 879    756 / 889    804 / 887    946 / 1017
 //   131072 tokens, 256 rows  5175 / 5717  5147 / 5690  5130 / 5697  5101 / 5746
+// At 32768 tokens 32 layers to a list would be 1-3 % quicker than the 16 of the rule, for twice the workspace.
 constexpr int64_t kListProducts = 32768;
 constexpr int kListMinLayers = 8;      // four: eight ragged sequences of 147k tokens, held, 6504 -> 6696 us
 int list_layers(const Problem& pb) {
@@ -547,6 +549,14 @@ unsigned long long next_launch_tag() {
   return n * 0x9E3779B97F4A7C15ull;
 }
 
+void expire_next_layer_wait(int on) { g_expire_next_layer_wait = on; }
+int take_expire_next_layer_wait(bool sums) {
+  const int v = g_expire_next_layer_wait;
+  if (v == 1 && !sums) return 0;
+  g_expire_next_layer_wait = 0;
+  return v;
+}
+
 LaunchScope::LaunchScope(int kid, cudaStream_t st, int* launches) : kid_(kid), st_(st), slot_(-1) {
   ++*launches;
   if (!g_prof_on) return;
@@ -629,7 +639,9 @@ int slkv_last_launch_count(void) { return g_last_launches; }
 int slkv_version(void) { return 300; }
 
 int slkv_debug_expire_next_wait(int on) {
-  expire_next_wait(on >= 2 && on <= 4 ? on : on != 0);
+  const int layer = on == 3 || on == 4 ? on - 2 : 0;
+  expire_next_layer_wait(layer);
+  expire_next_wait(layer ? 0 : on == 2 ? 2 : on != 0);
   return SLKV_OK;
 }
 

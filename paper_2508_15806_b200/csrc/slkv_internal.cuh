@@ -292,11 +292,13 @@ cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, fl
                             int* launches);
 // Timeline buffer of this thread (diagnostics), or null: kTraceSlots words per CTA.
 unsigned long long* tensor_trace_buffer(int n_cta);
-// Diagnostics: arm / consume the one-shot switch that makes an inter-CTA wait of this thread's next launch run out: 1, 2 a wait for
-// words in memory (slkv_score_pipe.cu, slkv_score_simt.cu), 3, 4 one of the kernels that do a whole layer.
+// Diagnostics: arm / consume the one-shot switches that make an inter-CTA wait of this thread's next launch run out: a wait for words
+// in memory (slkv_score_pipe.cu, slkv_score_simt.cu; 1, 2), one of the kernels that do a whole layer (1 for the row sums, where the
+// launch forms them, 2 for the votes).
 void expire_next_wait(int on);
 int take_expire_next_wait();
-bool next_wait_expires();                        // armed with 1 or 2
-int take_expire_next_layer_wait(bool sums);      // 1 the row sums (where the launch forms them), 2 the votes
+bool next_wait_expires();                        // armed
+void expire_next_layer_wait(int on);
+int take_expire_next_layer_wait(bool sums);
 
 }  // namespace slkv

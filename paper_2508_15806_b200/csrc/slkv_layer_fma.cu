@@ -7,7 +7,7 @@
 // same operations in the same order as k_score_simt: a row's statistics and a key's vote are the same bit for bit) and keeps them
 // for the votes.
 // What bounds it: latency at the small sizes (8 heads, 1024 positions, 16 rows, head_dim 64: 24.6 us from a stream as three
-// launches with two meetings of all CTAs, 11.7 here: keys 0.7, products 1.0, exchange 1, log-sum-exps 0.9, votes 1.4, selection
+// launches with two meetings of all CTAs, 12.0 here: keys 0.7, products 1.0, exchange 1, log-sum-exps 0.9, votes 1.4, selection
 // 2.4, rows 1.5), shared-memory reads of the operands beyond: a clock per register of a warp, twice what the FMAs take.
 #include <type_traits>
 

@@ -788,20 +788,9 @@ cudaError_t clear_stats(const ScoreShape& sh, const ScoreLayer* lay, int n_layer
 
 }  // namespace
 
-bool next_wait_expires() { return g_expire_next_wait == 1 || g_expire_next_wait == 2; }
+bool next_wait_expires() { return g_expire_next_wait != 0; }
 void expire_next_wait(int on) { g_expire_next_wait = on; }
-int take_expire_next_wait() {
-  if (!next_wait_expires()) return 0;
-  const int v = g_expire_next_wait;
-  g_expire_next_wait = 0;
-  return v;
-}
-int take_expire_next_layer_wait(bool sums) {
-  if (!(g_expire_next_wait == 3 && sums) && g_expire_next_wait != 4) return 0;
-  const int v = g_expire_next_wait - 2;
-  g_expire_next_wait = 0;
-  return v;
-}
+int take_expire_next_wait() { const int v = g_expire_next_wait; g_expire_next_wait = 0; return v; }
 
 void set_tensor_trace(void* dev_buf, size_t bytes) {
   g_trace = static_cast<unsigned long long*>(dev_buf);
