@@ -105,8 +105,8 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
     p = B.make_params(sh.q_win, sh.k, sh.v, w, pool_kernel, pool_mode, score_path, softmax_domain, B.SLKV_LSE_LOG2)
     p.history_only = 0 if sh.last else 1
 
-    # One buffer for all scratch, zero at the start: what the steps add to (row sums, histograms, totals) is cleared by one launch
-    # in front of them all.  Another for the small outputs, which a caller keeps without any scratch, and without the scores.
+    # One buffer for all scratch, zero at the start: what the steps add to (row sums, histograms, totals).  Another for the small
+    # outputs, which a caller keeps without any scratch, and without the scores.  One call clears both, in front of all steps.
     n_own = own + n_win
     has_keys = own > 0 or (sh.last and softmax_domain == B.SLKV_ALL_CAUSAL)
     ws_score = B.slkv_workspace_bytes(p, (0, rows)) if n_ext > 0 else 0
@@ -114,10 +114,11 @@ def compress_rank(shard: RankShard, budgets_row: torch.Tensor, pool_kernel: int,
     ws_emit = B.slkv_cp_workspace_bytes(hkv, own, max(cap, 1))
     state_bytes = -(-32 * hkv // 256) * 256                    # [4][2][hkv]: every head's prefix and need after each level
     sizes = ((state_bytes + max(ws_score, ws_lse, ws_emit)) // 4, 3 * 2048 * hkv, hkv, hkv, hq * w)
-    buf = torch.zeros(sum(sizes), dtype=torch.int32, device=dev)
-    ws, hists, totals, ties, lse_local = buf.split(sizes)
     out_sizes = (max(cap, 1), hq * w, hkv + 1, 1)
-    kept_idx, lse, offsets, status = torch.zeros(sum(out_sizes), dtype=torch.int32, device=dev).split(out_sizes)
+    buf, out = torch.empty(sum(sizes), dtype=torch.int32, device=dev), torch.empty(sum(out_sizes), dtype=torch.int32, device=dev)
+    torch._foreach_zero_((buf, out))
+    ws, hists, totals, ties, lse_local = buf.split(sizes)
+    kept_idx, lse, offsets, status = out.split(out_sizes)
     pooled = (torch.empty if n_ext > 0 else torch.zeros)(hkv * row_stride, dtype=torch.float32, device=dev)
     state = ws.data_ptr()
     scratch = state + state_bytes
