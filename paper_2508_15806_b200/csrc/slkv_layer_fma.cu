@@ -427,16 +427,21 @@ cudaError_t launch(const Problem& pb, int cs, LayerFmaArgs& a, cudaStream_t st, 
 }  // namespace
 
 // CTAs per segment, 0: the shape is not taken.  The clusters are those of slkv_layer_tc.cu; their CTAs are fewer than the SMs,
-// which tells where the products take most of the time: with few segments only what a CTA loads at once is taken.  us in a
-// graph / from a stream, here and on the general path:
-//                          1000 tokens            2000                   4000
-//   2 segs, d  64, 16 rows 11.3/11.7  16.8/18.6   12.4/12.9  17.1/19.3   15.7/16.2  18.5/20.6
-//   2 segs, d 128, 16 rows 13.2/13.6  18.5/21.7   15.4/16.0  19.3/22.6   24.3/24.8  21.7/22.8 (two chunks)
-//   2 segs, d 128, 64 rows 19.1/19.5  22.2/24.7   28.8/29.3  23.2/24.7 (two chunks)
-//   8 segs, d  64, 16 rows 11.9/12.2  18.5/20.6   13.0/13.3  19.4/22.4   16.3/16.5  24.3/26.8
-//   8 segs, d 128, 32 rows 15.6/16.1  22.2/22.7   20.1/20.5  24.3/26.5   34.1/34.6  31.7/34.9 (two chunks)
-//   8 segs, d 128, 64 rows 19.9/20.3  27.3/26.7   29.5/30.0  29.2/31.1 (two chunks)
-//   40 segs, d 64, 16 rows 15.8/16.3  31.4/34.6   22.4/23.0  45.1/47.8
+// which tells where the products take most of the time.  What a CTA loads at once is taken; in two chunks, with few segments
+// nothing is, with head_dim 64 everything else, with 128 where the products take no longer than the general path's: a block of 32
+// keys costs a CTA half a unit of 32 keys x 16 rows beside its units, the general path takes a step of all SMs for every 296 tiles
+// of 64 keys x 64 rows, the longer the more of the rows exist.  us in a graph / from a stream, here and on the general path (r: lengths from half to the
+// whole; two chunks from * on; - not taken):
+//                       1200 tokens            2300                    3000                    4000
+//   2 segs, d 128, 16   13.2/14.0  18.4/21.9   16.2/16.9  20.5/22.6   -
+//   8 segs, d  64, 16   11.9/12.4  18.8/20.7   13.7/14.2  19.2/22.5   14.9/15.4  23.4/26.8   16.7/17.2  24.1/26.8
+//   8 segs, d 128, 16   13.9/14.7  21.1/24.1   16.8/17.7  21.8/24.7   21.8/22.7  28.9/32.9 * 25.9/26.8  29.0/32.9
+//   8 segs, d 128, 32   16.1/16.9  22.1/24.8   21.0/21.8  22.8/25.5 * 29.7/30.5  30.1/33.0   35.3/36.2  31.5/35.0 -
+//   8 segs, d 128, 64   20.4/21.3  26.9/29.3 * 32.6/33.5  27.8/30.9 -
+//   16 r,   d 128, 32   21.1/22.0  24.5/26.8 * 32.2/33.1  31.5/34.9   40.9/41.8  31.0/34.0 -
+//   40 segs, d 64, 16   17.2/18.2  31.8/35.0 * 23.9/24.7  44.8/47.4   29.5/30.4  61.4/64.3   -
+// Of 402 shapes in two chunks that were measured both ways, 379 are taken, none of them slower from a stream; without the last
+// condition 18 were, by up to 8 us.
 int layer_fma_cluster(const Problem& pb) {
   const slkv_params& p = pb.p;
   if (p.dtype != SLKV_F32 || pb.R > kMaxRows || (p.pool_kernel >> 1) > kMaxRadius || p.history_only || pb.tab.n_inline == 0 ||
@@ -444,8 +449,13 @@ int layer_fma_cluster(const Problem& pb) {
     return 0;
   const int cs = layer_tc_clusters_for(pb.n_seg);
   if (cs < 2 || (long long)keys_per_cta(pb, cs) * pb.R > kMaxScores) return 0;
-  const int chunk = chunk_for(pb, cs);
-  return chunk > 0 && (chunk >= keys_per_cta(pb, cs) || 2 * pb.n_seg * cs >= sm_count()) ? cs : 0;
+  const int chunk = chunk_for(pb, cs), keys = keys_per_cta(pb, cs), sms = sm_count();
+  if (chunk >= keys) return cs;
+  if (chunk == 0 || 2 * pb.n_seg * cs < sms) return 0;
+  if (p.head_dim == 64) return cs;
+  const int units = (pb.R + 15) / 16;
+  const long long steps = (2 * pb.n_tiles128 + 2 * sms - 1) / (2 * sms) * ((pb.R + 63) / 64);
+  return keys / kBlock * (2 * units + 1) <= 5 * (units + 4) * steps ? cs : 0;
 }
 
 cudaError_t launch_layer_fma(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,

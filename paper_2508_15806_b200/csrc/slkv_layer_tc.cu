@@ -386,24 +386,29 @@ int layer_tc_clusters_for(int n_seg) {
 }
 
 // CTAs per segment, 0: the shape is not taken.  The largest cluster of which there is one for every segment at the same time
-// (eight segments: of ten CTAs; sixteen: of six), two CTAs at least: the clusters run on n_seg * CS SMs, while the general path
-// spreads a layer's tiles over all of them but takes three launches and exchanges through memory.  One layer of head_dim 128 and
-// 128 rows, us in a graph / from a stream, here and on the general path:
-//   segments   1000 tokens            4000 tokens            8000 tokens
-//   1          10.9/11.6  16.3/20.6   15.1/15.5  18.0/22.7   21.5/21.8  19.3/24.3
-//   8          12.0/12.4  18.0/22.6   16.0/16.5  22.3/25.0   22.6/22.8  25.3/28.8
-//   16         13.4/13.7  21.3/24.7   19.7/20.1  25.2/28.8   28.5/29.0  30.9/34.5
-//   32         14.2/14.3  24.2/27.1   23.8/24.1  30.6/33.8   37.3/37.4  37.8/41.1
-//   40         15.9/16.3  25.1/28.7   27.9/28.3  33.5/37.0   45.1/45.5  44.0/46.9
-//   64         18.1/18.7  28.0/30.9   37.5/37.8  38.8/42.9   62.6/63.0  63.5/66.9
-// and with 32 rows 8 x 8000 19.7/20.0 24.5/27.6, 64 x 8000 58.4/58.8 58.4/61.7.  More segments than clusters: two rounds (16
-// segments of 1000 tokens in clusters of eight 24.1, of four 14.0).
+// (eight segments: of ten CTAs; sixteen: of six), two CTAs at least: the clusters run on n_seg * CS SMs and as long as the longest
+// segment's, while the general path spreads a layer's tiles over all SMs but takes three launches and exchanges through memory,
+// some 8 us.  A tile costs a CTA 1.1 us here: no more than seven of them over an even share.  One layer of head_dim 128 and 128
+// rows, us in a graph / from a stream, here and on the general path (r: lengths from half to the whole):
+//   segments   2000 tokens            4000 tokens            6000 tokens            8100 tokens
+//   2          12.0/13.0  16.8/21.2   15.0/15.7  17.8/22.6   18.4/19.1  18.4/22.7   21.1/21.9  19.5/24.7
+//   8          13.3/13.7  19.0/23.3   16.0/16.4  21.3/24.7   19.6/20.2  23.6/26.8   22.5/23.1  25.4/28.8
+//   16         14.8/15.4  22.9/26.8   19.5/20.2  24.9/28.2   24.1/24.9  28.2/31.0   28.4/29.3  30.5/33.4
+//   32         20.6/21.5  25.8/29.0   27.4/28.3  30.6/33.2   34.8/35.5  35.3/39.0   41.2/41.6  38.7/41.9
+//   40         19.3/20.0  27.6/30.9   27.5/28.3  33.2/36.7   36.4/37.2  36.0/39.1   44.5/45.1  43.7/47.2
+//   40 r       18.8/19.7  26.1/28.9   27.0/27.7  30.3/33.0   35.9/36.7  35.0/38.8   43.2/44.2  37.6/41.2 (not taken)
+//   64         24.2/25.1  32.0/35.1   36.4/37.1  37.7/41.2   49.3/49.8  51.7/55.2   61.9/62.4  62.6/65.7
+//   64 r       23.5/24.4  30.1/33.0   35.3/36.1  36.9/40.7   47.5/48.4  41.5/45.2   60.4/61.6  52.4/55.5 (the last two not taken)
+// and with 16 rows 8 x 8100 19.5/20.1 23.7/26.9, 64 x 8100 57.7/58.2 55.4/58.3, 64 r x 8100 (not taken) 55.2/56.2 45.1/48.5.
+// More segments than clusters: two rounds (16 segments of 1000 tokens in clusters of eight 24.1, of four 14.0).
+constexpr int kTilesOverShare = 7;
 int layer_tc_cluster(const Problem& pb) {
   const slkv_params& p = pb.p;
   if (!tensor_path_supported(p) || pb.R > 128 || (p.pool_kernel >> 1) > kMaxRadius || p.history_only || pb.tab.n_inline == 0 ||
       pb.max_hist < 1 || pb.max_hist > 16 * kLayerThreads)
     return 0;
-  return layer_tc_clusters_for(pb.n_seg);
+  const int cs = layer_tc_clusters_for(pb.n_seg), tiles = (pb.max_hist + kTileKeys - 1) / kTileKeys;
+  return cs >= 2 && (tiles + cs - 1) / cs <= pb.n_tiles128 / sm_count() + kTilesOverShare ? cs : 0;
 }
 
 cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,

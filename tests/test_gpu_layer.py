@@ -123,7 +123,7 @@ def test_many_calls_in_a_row(n):
     same(both(q, k, v, cu, 32, 7, [64 + 100 * h for h in range(8)], calls=1000))
 
 
-@pytest.mark.parametrize("lens", [[100], [300], [700], [1000], [1180], [40, 1100, 33, 200], [600, 34, 8000]])
+@pytest.mark.parametrize("lens", [[100], [300], [700], [1000], [1180], [40, 1100, 33, 200], [600, 34, 6000]])
 def test_rows_of_ctas_without_tiles(lens):
     # Segments of fewer tiles than their cluster has CTAs, log-sum-exps handed in: a CTA without tiles gets to its rows with
     # nothing to wait for but the budgets, which another warp reads -- from HBM, while the log-sum-exps lie in L2.
@@ -247,6 +247,24 @@ def test_fp32_equal_keys_have_equal_scores(hq, hkv, d, w, n):
         B.slkv_compress(p, q, k, v, cu_dev, cu, torch.tensor(budgets, dtype=torch.int32, device=DEV), out[0], out[1],
                         torch.zeros(hkv + 1, dtype=torch.int32, device=DEV), torch.zeros(cap, dtype=torch.int32, device=DEV), ws, general, status)
         assert int(status) == 0 and int(st) == 0 and torch.equal(own, general)
+
+
+@pytest.mark.parametrize("dt,d,hq,hkv,w,lens,one", [
+    (torch.bfloat16, 128, 32, 8, 32, [8100], True), (torch.bfloat16, 128, 32, 8, 32, [8100] * 8, True),
+    (torch.bfloat16, 128, 32, 8, 32, [4050 + 4050 * i // 7 for i in range(8)], False),
+    (torch.bfloat16, 64, 16, 8, 32, [8100, 100, 100, 100, 100], False),
+    (torch.float32, 128, 8, 8, 32, [3000], True), (torch.float32, 128, 8, 8, 32, [4000], False),
+    (torch.float32, 128, 8, 8, 32, [1500, 3000], False), (torch.float32, 128, 8, 8, 16, [6000], True),
+    (torch.float32, 64, 8, 8, 24, [2000, 4000], True), (torch.float32, 128, 8, 8, 24, [2000, 4000], False)])
+def test_what_goes_which_way(dt, d, hq, hkv, w, lens, one):
+    # either side of the lines drawn for segments of unequal length and for keys that do not fit at once
+    q, k, v, cu = inputs(sum(lens), lens, hq, hkv, d, w, dt)
+    p = B.make_params(q, k, v, w, 5)
+    cu_dev, ws = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
+    pooled, status = torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.slkv_score(p, q, k, cu_dev, cu, pooled, ws, status)
+    assert (B.slkv_last_launch_count() == 1) == one and int(status) == 0
+    same(both(q, k, v, cu, w, 5, [w + 40 * h for h in range(hkv)], one_launch=one))
 
 
 # ---- waits that run out -------------------------------------------------------------------------------------------------
