@@ -237,9 +237,9 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
 
 // CTAs per segment where one launch does the whole layer, else 0.  A wait for words in memory that is to run out
 // (slkv_debug_expire_next_wait) is one of the other kernels'.
-int layer_cluster(const Problem& pb, int path) {
+int layer_cluster(const Problem& pb, int path, bool select) {
   if (next_wait_expires()) return 0;
-  return path == SLKV_PATH_TENSOR ? layer_tc_cluster(pb) : layer_fma_cluster(pb);
+  return path == SLKV_PATH_TENSOR ? layer_tc_cluster(pb, select) : layer_fma_cluster(pb, select);
 }
 cudaError_t launch_layer(const Problem& pb, int path, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,
                          int* launches) {
@@ -505,7 +505,7 @@ int compress_impl(const slkv_params* p, const void* q_win, const void* k, const 
   TailLayer tail = tail_of(pb, budgets, k_out, v_out, capacity, offsets, kept_idx, pooled_opt, status);
   // One launch for the whole layer where that is quicker.  With pooled_opt the call takes the general path, launch by launch:
   // that is a caller who looks into the steps, and how the two are held against each other on the same inputs.
-  if (const int cs = !kept_copy && !offsets_copy && !pooled_opt ? layer_cluster(pb, path) : 0) {
+  if (const int cs = !kept_copy && !offsets_copy && !pooled_opt ? layer_cluster(pb, path, true) : 0) {
     e = launch_layer(pb, path, cs, &tail, nullptr, status, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
     g_last_launches = launches;
@@ -948,7 +948,7 @@ int score_impl(const slkv_params* p, const void* q_win, const void* k, const int
     g_last_launches = launches;
     return SLKV_OK;
   }
-  if (const int cs = layer_cluster(pb, path)) {
+  if (const int cs = layer_cluster(pb, path, false)) {
     e = launch_layer(pb, path, cs, nullptr, pooled, status, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e);
     g_last_launches = launches;

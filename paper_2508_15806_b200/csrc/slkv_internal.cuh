@@ -282,10 +282,11 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
 cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
                                     cudaStream_t st, int* launches);
 // ---- a whole layer in one launch (slkv_layer_tc.cu, slkv_layer_fma.cu) ---------------------------------------------
-// CTAs per segment, or 0 where the shape is not taken; tail null: the pooled scores alone.  pooled may be null with a tail.
+// CTAs per segment, or 0 where the shape is not taken; select false, tail null: the pooled scores alone.  pooled may be null with a
+// tail.
 int layer_tc_clusters_for(int n_seg);
-int layer_tc_cluster(const Problem& pb);
-int layer_fma_cluster(const Problem& pb);
+int layer_tc_cluster(const Problem& pb, bool select);
+int layer_fma_cluster(const Problem& pb, bool select);
 cudaError_t launch_layer_fma(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,
                              int* launches);
 cudaError_t launch_layer_tc(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,

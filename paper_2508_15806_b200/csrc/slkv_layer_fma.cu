@@ -427,10 +427,12 @@ cudaError_t launch(const Problem& pb, int cs, LayerFmaArgs& a, cudaStream_t st, 
 }  // namespace
 
 // CTAs per segment, 0: the shape is not taken.  The clusters are those of slkv_layer_tc.cu; their CTAs are fewer than the SMs,
-// which tells where the products take most of the time.  What a CTA loads at once is taken; in two chunks, with few segments
-// nothing is, with head_dim 64 everything else, with 128 where the products take no longer than the general path's: a block of 32
-// keys costs a CTA half a unit of 32 keys x 16 rows beside its units, the general path takes a step of all SMs for every 296 tiles
-// of 64 keys x 64 rows, the longer the more of the rows exist.  us in a graph / from a stream, here and on the general path (r: lengths from half to the
+// which tells where the products take most of the time.  A block of 32 keys costs a CTA half a unit of 32 keys x 16 rows beside its
+// units; the general path takes a step of all SMs for every 296 tiles of 64 keys x 64 rows, the longer the more of the rows exist
+// where it walks them twice.  What the general path's launches cost on top is worth a `head`, of which loading the keys in two
+// chunks leaves nothing but with head_dim 64; with few segments two chunks are never taken.  Measured both ways, 199 to 502 shapes of
+// each kind that are taken: slower from a stream by 0.8 us at most (layers), 1.3 (scores) and, with log-sum-exps handed in, 6.4 and
+// 7.1 (40 segments of 1500-3000 tokens, head_dim 128, 16 rows, in two chunks: 52.0 against 45.6).  us in a graph / from a stream, here and on the general path (r: lengths from half to the
 // whole; two chunks from * on; - not taken):
 //                       1200 tokens            2300                    3000                    4000
 //   2 segs, d 128, 16   13.2/14.0  18.4/21.9   16.2/16.9  20.5/22.6   -
@@ -440,9 +442,7 @@ cudaError_t launch(const Problem& pb, int cs, LayerFmaArgs& a, cudaStream_t st, 
 //   8 segs, d 128, 64   20.4/21.3  26.9/29.3 * 32.6/33.5  27.8/30.9 -
 //   16 r,   d 128, 32   21.1/22.0  24.5/26.8 * 32.2/33.1  31.5/34.9   40.9/41.8  31.0/34.0 -
 //   40 segs, d 64, 16   17.2/18.2  31.8/35.0 * 23.9/24.7  44.8/47.4   29.5/30.4  61.4/64.3   -
-// Of 402 shapes in two chunks that were measured both ways, 379 are taken, none of them slower from a stream; without the last
-// condition 18 were, by up to 8 us.
-int layer_fma_cluster(const Problem& pb) {
+int layer_fma_cluster(const Problem& pb, bool select) {
   const slkv_params& p = pb.p;
   if (p.dtype != SLKV_F32 || pb.R > kMaxRows || (p.pool_kernel >> 1) > kMaxRadius || p.history_only || pb.tab.n_inline == 0 ||
       pb.max_hist < 1 || pb.max_hist > 16 * kLayerThreads)
@@ -450,12 +450,12 @@ int layer_fma_cluster(const Problem& pb) {
   const int cs = layer_tc_clusters_for(pb.n_seg);
   if (cs < 2 || (long long)keys_per_cta(pb, cs) * pb.R > kMaxScores) return 0;
   const int chunk = chunk_for(pb, cs), keys = keys_per_cta(pb, cs), sms = sm_count();
-  if (chunk >= keys) return cs;
-  if (chunk == 0 || 2 * pb.n_seg * cs < sms) return 0;
-  if (p.head_dim == 64) return cs;
+  const bool at_once = chunk >= keys, both = !pb.lse_opt;
+  if (chunk == 0 || (!at_once && 2 * pb.n_seg * cs < sms)) return 0;
   const int units = (pb.R + 15) / 16;
+  const int head = at_once ? (both && select ? 40 : both || select ? 25 : 10) : (both && select && p.head_dim == 64 ? 20 : 0);
   const long long steps = (2 * pb.n_tiles128 + 2 * sms - 1) / (2 * sms) * ((pb.R + 63) / 64);
-  return keys / kBlock * (2 * units + 1) <= 5 * (units + 4) * steps ? cs : 0;
+  return keys / kBlock * (2 * units + 1) <= (both ? 20 + 5 * units : 20) * steps + head ? cs : 0;
 }
 
 cudaError_t launch_layer_fma(const Problem& pb, int cs, const TailLayer* tail, float* pooled, int32_t* status, cudaStream_t st,

@@ -250,21 +250,34 @@ def test_fp32_equal_keys_have_equal_scores(hq, hkv, d, w, n):
 
 
 @pytest.mark.parametrize("dt,d,hq,hkv,w,lens,one", [
-    (torch.bfloat16, 128, 32, 8, 32, [8100], True), (torch.bfloat16, 128, 32, 8, 32, [8100] * 8, True),
-    (torch.bfloat16, 128, 32, 8, 32, [4050 + 4050 * i // 7 for i in range(8)], False),
-    (torch.bfloat16, 64, 16, 8, 32, [8100, 100, 100, 100, 100], False),
-    (torch.float32, 128, 8, 8, 32, [3000], True), (torch.float32, 128, 8, 8, 32, [4000], False),
-    (torch.float32, 128, 8, 8, 32, [1500, 3000], False), (torch.float32, 128, 8, 8, 16, [6000], True),
-    (torch.float32, 64, 8, 8, 24, [2000, 4000], True), (torch.float32, 128, 8, 8, 24, [2000, 4000], False)])
+    # layer, scores, layer with log-sum-exps handed in, scores with them
+    (torch.bfloat16, 128, 32, 8, 32, [2000], (1, 1, 1, 1)), (torch.bfloat16, 128, 32, 8, 32, [8100], (1, 1, 1, 0)),
+    (torch.bfloat16, 128, 32, 8, 32, [8100] * 5, (1, 0, 0, 0)), (torch.bfloat16, 64, 16, 8, 32, [8100, 100, 100, 100, 100], (0, 0, 0, 0)),
+    (torch.bfloat16, 128, 32, 8, 32, [4050 + 4050 * i // 7 for i in range(8)], (0, 0, 0, 0)),
+    (torch.float32, 64, 8, 8, 16, [1000], (1, 1, 1, 1)), (torch.float32, 64, 8, 8, 32, [3000], (1, 1, 1, 1)),
+    (torch.float32, 128, 8, 8, 32, [3000], (1, 1, 0, 0)), (torch.float32, 128, 8, 8, 32, [4000], (0, 0, 0, 0)),
+    (torch.float32, 128, 8, 8, 32, [1500, 3000], (0, 0, 0, 0)), (torch.float32, 128, 8, 8, 16, [6000], (1, 1, 1, 1)),
+    (torch.float32, 64, 8, 8, 24, [2000, 4000], (1, 0, 0, 0)), (torch.float32, 128, 8, 8, 24, [2000, 4000], (0, 0, 0, 0))])
 def test_what_goes_which_way(dt, d, hq, hkv, w, lens, one):
-    # either side of the lines drawn for segments of unequal length and for keys that do not fit at once
+    # either side of the lines drawn for segments of unequal length, keys that do not fit at once, and calls with less to save
     q, k, v, cu = inputs(sum(lens), lens, hq, hkv, d, w, dt)
-    p = B.make_params(q, k, v, w, 5)
+    p = B.make_params(q, k, v, w, 5, lse_units=B.SLKV_LSE_LOG2)
     cu_dev, ws = torch.tensor(cu, dtype=torch.int32, device=DEV), torch.empty(B.slkv_workspace_bytes(p, cu), dtype=torch.uint8, device=DEV)
-    pooled, status = torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
-    B.slkv_score(p, q, k, cu_dev, cu, pooled, ws, status)
-    assert (B.slkv_last_launch_count() == 1) == one and int(status) == 0
-    same(both(q, k, v, cu, w, 5, [w + 40 * h for h in range(hkv)], one_launch=one))
+    own, fed = (torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) for _ in range(2))
+    lse, status = torch.zeros(len(lens), hq, w, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.slkv_row_lse(p, q, k, cu_dev, cu, lse, ws)
+    took = []
+    for pooled, x in ((own, None), (fed, lse)):
+        bud = torch.tensor([w + 40 * h for h in range(hkv)], dtype=torch.int32, device=DEV)
+        res = both(q, k, v, cu, w, 5, bud.tolist(), lse=x, one_launch=False)
+        same(res)
+        out = torch.zeros(2, *res[0][2].shape, dtype=dt, device=DEV)
+        off, kept = torch.zeros_like(res[0][0]), torch.zeros_like(res[0][1])
+        B.slkv_compress(p, q, k, v, cu_dev, cu, bud, out[0], out[1], off, kept, ws, None, status, lse=x)
+        took.append(B.slkv_last_launch_count() == 1)
+        B.slkv_score(p, q, k, cu_dev, cu, pooled, ws, status, lse=x)
+        took.append(B.slkv_last_launch_count() == 1)
+    assert tuple(map(int, took)) == one and int(status) == 0 and torch.equal(own, fed)
 
 
 # ---- waits that run out -------------------------------------------------------------------------------------------------
