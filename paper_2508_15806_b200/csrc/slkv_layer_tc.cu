@@ -391,9 +391,9 @@ int layer_tc_clusters_for(int n_seg) {
 // some 8 us.  A tile costs a CTA 1.1 us here, one of an even share over all SMs 0.8 there, so as many of the first as make up for
 // the launches may stand over three quarters of the second; fewer where there is less to save -- the scores alone take two launches,
 // log-sum-exps handed in the exchange.  Measured both ways, 99 to 276 shapes of each kind that are taken: slower from a stream by 1.5
-// us at most (layers), 1.2 (scores), 3.7 and 1.0 (with log-sum-exps: 32 heads of 7000 tokens, 16 rows, 26.9 against 23.3).  One layer of head_dim 128 and 128
-// rows, us in a graph / from a stream, here and on the general path (r: lengths from half to the whole;
-// -: not taken):
+// us at most (layers), 1.2 (scores), 3.7 and 1.0 (with log-sum-exps: 32 heads of 7000 tokens, 16 rows, 26.9 against 23.3).  One
+// layer of head_dim 128 and 128 rows, us in a graph / from a stream, here and on the general path (r: lengths from half to the
+// whole; -: not taken):
 //   segments   2000 tokens            4000 tokens            6000 tokens            8100 tokens
 //   2          12.0/13.0  16.8/21.2   15.0/15.7  17.8/22.6   18.4/19.1  18.4/22.7   21.1/21.9  19.5/24.7
 //   8          13.3/13.7  19.0/23.3   16.0/16.4  21.3/24.7   19.6/20.2  23.6/26.8   22.5/23.1  25.4/28.8
@@ -401,9 +401,9 @@ int layer_tc_clusters_for(int n_seg) {
 //   32         20.6/21.5  25.8/29.0   27.4/28.3  30.6/33.2   34.8/35.5  35.3/39.0   41.2/41.6  38.7/41.9
 //   40         19.3/20.0  27.6/30.9   27.5/28.3  33.2/36.7   36.4/37.2  36.0/39.1   44.5/45.1  43.7/47.2
 //   40 r       18.8/19.7  26.1/28.9   27.0/27.7  30.3/33.0   35.9/36.7  35.0/38.8   43.2/44.2  37.6/41.2 -
-//   64         24.2/25.1  32.0/35.1   36.4/37.1  37.7/41.2   49.3/49.8  51.7/55.2   61.9/62.4  62.6/65.7
-//   64 r       23.5/24.4  30.1/33.0   35.3/36.1  36.9/40.7   47.5/48.4  41.5/45.2   60.4/61.6  52.4/55.5 -
-// and with 16 rows 8 x 8100 19.5/20.1 23.7/26.9, 64 x 8100 57.7/58.2 55.4/58.3, 64 r x 8100 55.2/56.2 45.1/48.5.
+//   64         24.2/25.1  32.0/35.1   36.4/37.1  37.7/41.2   49.3/49.8  51.7/55.2   61.9/62.4  62.6/65.7 -
+//   64 r       23.5/24.4  30.1/33.0   35.3/36.1  36.9/40.7   47.5/48.4  41.5/45.2 - 60.4/61.6  52.4/55.5 -
+// and with 16 rows 8 x 8100 19.5/20.1 23.7/26.9, 64 x 8100 57.7/58.2 55.4/58.3 -, 64 r x 8100 55.2/56.2 45.1/48.5 -.
 // More segments than clusters: two rounds (16 segments of 1000 tokens in clusters of eight 24.1, of four 14.0).
 int layer_tc_cluster(const Problem& pb, bool select) {
   const slkv_params& p = pb.p;
