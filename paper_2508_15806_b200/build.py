@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libslkv.so")
 CALL = os.path.join(HERE, "_slkv_call.so")
 SOURCES = ["slkv_api.cu", "slkv_alloc.cu", "slkv_score_simt.cu", "slkv_score_tc.cu", "slkv_score_pipe.cu", "slkv_select.cu", "slkv_select_cluster.cu", "slkv_select_cta.cu",
-           "slkv_layer_tc.cu", "slkv_layer_fma.cu", "slkv_noalloc.cu", "slkv_behavior.cu", "slkv_cp.cu"]
+           "slkv_layer_tc.cu", "slkv_layer_fma.cu", "slkv_bound.cu", "slkv_noalloc.cu", "slkv_behavior.cu", "slkv_cp.cu"]
 
 
 def _nvcc() -> str:

@@ -289,7 +289,15 @@ cudaError_t flush_list(ListState* s, cudaStream_t owner, int* launches) {
   const int n = s->n;
   s->n = 0;
   s->in_flight = true;
-  cudaError_t e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, s->pb.sync, owner, launches);
+  cudaError_t e;
+  bool bound = !s->with_lse && !next_wait_expires() && bound_list_supported(s->pb);
+  for (int i = 0; i < n; ++i) bound = bound && s->tail[i].pooled_out == nullptr;
+  if (bound) {
+    e = launch_bound_list(s->pb, s->plan.sh, s->score, s->tail, n, owner, launches);
+    if (e == cudaSuccess) e = launch_gather(s->pb, s->tail, n, owner, launches);
+    if (e != cudaErrorNotSupported) return e;
+  }
+  e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, s->pb.sync, owner, launches);
   if (e == cudaSuccess)
     e = select_list_supported(s->pb) ? launch_select_list(s->pb, s->tail, n, owner, launches)
                                      : launch_select_cluster(s->pb, s->tail, n, owner, launches);

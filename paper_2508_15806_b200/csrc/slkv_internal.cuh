@@ -233,6 +233,7 @@ struct TailLayer {
   long long capacity;
 };
 bool select_list_supported(const Problem& pb);
+int select_list_cluster(const Problem& pb);      // CTAs per segment
 cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
 bool select_cluster_supported(const Problem& pb);
 cudaError_t launch_select_cluster(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches);
@@ -262,6 +263,7 @@ struct ScoreLayer {
   float* vote;
   LseSource lse;                // where the vote pass takes the rows' log-sum-exp from besides the statistics pass
   int32_t* status;
+  const int32_t* budgets;       // launches for bounds alone
 };
 // One layer's score problem, ready to launch.
 struct ScorePlan {
@@ -275,9 +277,22 @@ cudaError_t plan_score_layer(const Problem& pb, int32_t* status, ScoreLayer* lay
 int sm_count();
 int score_list_stages(int MT, int halves);
 // The score kernel over a list of layers of one shape: passes 1 = row statistics, 2 = votes from the callers' row
-// statistics, 3 = both; sync: Problem's.
+// statistics, 3 = both, kScoreBound = row statistics and estimated votes (slkv_bound.cu); sync: Problem's.
+constexpr int kScoreBound = 4;
+// A list for bounds computes every vote of a segment that keeps so many positions and that share of them.
+constexpr int kEveryVoteCount = 512, kEveryVoteShare = 64;
+#ifdef __CUDACC__
+__device__ __forceinline__ bool every_vote(int len, int budget, int window) {
+  const int n = len - window, k = min(len, max(budget, window)) - window;
+  return k >= kEveryVoteCount && k < n && (long long)k * kEveryVoteShare >= n;
+}
+#endif
 cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
                               unsigned long long* sync, cudaStream_t st, int* launches, bool cleared = false);
+// Scores and selection of a list in one product with every key (slkv_bound.cu).  cudaErrorNotSupported: nothing is launched.
+bool bound_list_supported(const Problem& pb);
+cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const ScoreLayer* lay, const TailLayer* tail, int n_layers,
+                              cudaStream_t st, int* launches);
 // lse_out null: into the layer's own statistics area
 cudaError_t launch_merge_lse_tensor(const ScoreShape& sh, const ScoreLayer& lay, float* lse_out, float out_scale,
                                     cudaStream_t st, int* launches);

@@ -109,8 +109,9 @@ __device__ __forceinline__ void layer_select(const LayerTail& a, const Segment& 
   asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(kLayerThreads) : "memory");
   if (*gave_up) return;                         // written in front of the barrier, if at all
   int o;
+  unsigned tau;
   const unsigned kept = select_places<kLayerThreads, IT, false, BAR>(sh, tid, key, valid, mine, reinterpret_cast<uint4*>(votes + vote_at<IT>(i0)),
-                                                                     x.n, k_keep, 0, 1, o);
+                                                                     x.n, k_keep, 0, 1, o, tau);
   int* dst = reinterpret_cast<int*>(votes - kLead) + o;
   for (unsigned m = kept; m != 0; m &= m - 1) *dst++ = i0 + __ffs(m) - 1;
 }

@@ -1,7 +1,7 @@
 // Window relevance scores on the 5th-generation tensor cores (Sec. 3.4, Eq. 7; Algorithm 3; Eq. 3-4), a list of layers
 // per launch.  bf16, head_dim 64 or 128, up to 256 query rows per KV head.
 //
-// Two passes over a layer's keys, in 128-key tiles:
+// Two passes over a layer's keys, in 128-key tiles (one where all that is asked for is what is kept: slkv_bound.cu):
 //   statistics  S = Q K^T with the G*w query rows as the M dimension: a TMEM lane -- one thread -- owns a query row and
 //               sums 2^s over a tile's keys in fp32, over a run of tiles in fp64, and adds the run's sum to the row's;
 //   votes       S^T = K Q^T with the keys as the M dimension: a thread owns a key, and
@@ -24,8 +24,8 @@
 // (the parameters of a list are kilobytes) took 3600 cycles per run and 1000 per tile of the MMA thread.
 //
 // What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
-//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in eight (statistics) or
-//     sixteen (votes) goes to the FMA pipe, and scale / subtract / sum run on packed pairs;
+//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; of the votes' one in sixteen goes
+//     to the FMA pipe, and scale / subtract / sum run on packed pairs;
 //   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
 //     730 measured for loads and MMAs alone;
 //   - two epilogue warpgroups instead of four: 1250; sums over the keys across lanes instead of a lane per row: 1255;
@@ -54,13 +54,14 @@ constexpr int kMaxStages = 6;
 constexpr int kBarBytes = 640;
 constexpr int kStatBytes = 2 * kWgs * 128 * 8;
 constexpr int kLseBytes = 2 * 256 * 4;
-constexpr int kHalfVoteBytes = 2 * 4 * 128 * 4;
+constexpr int kPartBytes = kWgs * 2 * 4 * 128 * 4;      // per warpgroup two slots of its warps' shares, see bound_run; half votes take a quarter
 // Two Q tiles, also where that leaves the ring no more than two K tiles (R > 128, d = 128): the next run's queries are
 // there when its keys are.  One Q tile and four K tiles cost a pause of 1.6 us in every run of about 25: 128k positions
 // 5935 -> 5810 us, eight sequences of 4k - 32k 6830 -> 6690 us (32 layers each).
 constexpr int kQTiles = 2;
 constexpr int kRunSlots = 8;                         // runs handed out ahead
-constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes + kRunSlots * 128;
+constexpr int kFirstBytes = 2 * kWgs * 128 * 4;      // [2][kWgs][128]: sums over the first tiles of a run, see bound_run
+constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kPartBytes + kFirstBytes + kRunSlots * 128;
 
 // The clearing of the statistics and the groups' counts: one word with the launch's tag (40 bits) above two counts of 12 bits,
 // CTAs that are done and CTAs that have cleared their share.  A CTA that finds another value puts the tag first; the last CTA
@@ -124,6 +125,8 @@ struct alignas(16) RunDesc {
   const CUtensorMap* tm_k;
   int slot;                    // this CTA's place among the segment's split ranges
   float* vote;                 // of the run's first key
+  float* weight;               // bounds: where the run's row weights go, the second ones `second` floats further on
+  int second;
   double* acc;                 // the segment's row sums ...
   const unsigned* far;         // ... and far bits
   int sums, win;               // votes: the log-sum-exps come from the sums, with window statistics
@@ -143,7 +146,8 @@ struct Smem {
   float* stat_m;               // likewise
   unsigned* stat_far;          // [2]: warps that have any
   float* lse;                  // [2][256], negated
-  float* half_vote;            // [2][4][128]
+  float* half_vote;            // [2][4][128]; bounds: see bound_run
+  float* first;                // [2][kWgs][128]
   __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * (uint32_t)i; }
   __device__ __forceinline__ uint32_t full(int st) const { return bar(st); }
   __device__ __forceinline__ uint32_t empty(int st) const { return bar(kMaxStages + st); }
@@ -164,8 +168,11 @@ struct Smem {
   __device__ __forceinline__ uint32_t cleared() const { return bar(2 * kMaxStages + 29 + 2 * kRunSlots); }
   __device__ __forceinline__ uint32_t drain() const { return bar(2 * kMaxStages + 28 + 2 * kRunSlots); }   // a wait ran out
   __device__ __forceinline__ uint32_t rest_cleared() const { return bar(2 * kMaxStages + 30 + 2 * kRunSlots); }
+  __device__ __forceinline__ uint32_t part_full(int i) const { return bar(2 * kMaxStages + 33 + 2 * kRunSlots + i); }   // [sharers][2]
+  __device__ __forceinline__ uint32_t again_full() const { return bar(2 * kMaxStages + 41 + 2 * kRunSlots); }
+  __device__ __forceinline__ uint32_t first_full(int s) const { return bar(2 * kMaxStages + 31 + 2 * kRunSlots + s); }
 };
-constexpr int kNumBars = 2 * kMaxStages + 31 + 2 * kRunSlots;
+constexpr int kNumBars = 2 * kMaxStages + 42 + 2 * kRunSlots;
 constexpr int kHeadInts = 7;
 static_assert(kNumBars * 8 + kHeadInts * 4 + 16 <= kBarBytes, "mbarriers");
 constexpr int kRunReaders = 4 + 4 * kWgs;              // arrivals that free a run slot: one per reading thread or warp
@@ -196,6 +203,7 @@ __device__ __forceinline__ GroupShare group_share(const ListArgs& a, int gg) {
   g.end = takes_part ? split_begin(g.idx + 1, g.T, g.n) : 0;
   return g;
 }
+template <bool BOUND>
 struct RunWalk {
   int step, pos, kind, gg;
   GroupShare s;
@@ -205,14 +213,14 @@ struct RunWalk {
     const ScoreShape& sh = a.sh;
     const int NG = a.n_groups;
     while (pos >= s.end) {                                   // the next phase
-      if (a.passes == 3) {
+      if (!BOUND && a.passes == 3) {
         const int p = step >> 1;
         if (p >= NG + a.lag) { d.kind = kind = 2; return; }
         kind = step & 1;
         gg = kind ? p - a.lag : p;
       } else {
         if (step >= NG) { d.kind = kind = 2; return; }
-        kind = a.passes == 2;
+        kind = !BOUND && a.passes == 2;
         gg = step;
       }
       ++step;
@@ -251,10 +259,94 @@ struct RunWalk {
     d.seg = seg;
     d.acc = static_cast<double*>(L.part) + (long long)seg * sh.R;
     d.far = reinterpret_cast<unsigned*>(static_cast<double*>(L.part) + (long long)sh.n_seqs * sh.n_kv_heads * sh.R) + seg * kFarWords;
+    d.second = sh.n_seqs * sh.n_kv_heads * sh.slot_stride * sh.R;
+    // the places of this CTA's far part, which a segment with estimates does not use
+    d.weight = const_cast<float*>(reinterpret_cast<const float*>(d.far + (sh.n_seqs * sh.n_kv_heads - seg) * kFarWords)) + ((long long)seg * sh.slot_stride + d.slot) * sh.R;
     d.sums = a.passes == 3;
     d.win = L.lse.win_m != nullptr;
     d.q_y = sh.q_head_inner ? r.g * sh.G : 0;
     d.q_z = sh.q_head_inner ? 0 : r.g * sh.G;
+  }
+};
+// The segments of a list all of whose votes are computed: warp 2's way through their tiles, which the CTAs share evenly.
+struct FullWalk {
+  int pos, end;
+  // Segment i of the list: tiles that count.
+  static __device__ __forceinline__ int tiles(const ListArgs& a, int i) {
+    const ScoreShape& sh = a.sh;
+    const int n_seg = sh.n_seqs * sh.n_kv_heads, layer = i / n_seg, seg = i - layer * n_seg, s = seg / sh.n_kv_heads;
+    if (layer >= a.n_layers) return 0;
+    const int len = sh.tab.cu_at(s + 1) - sh.tab.cu_at(s);
+    return every_vote(len, __ldcg(a.lay[layer].budgets + (seg - s * sh.n_kv_heads)), sh.window) ? sh.tab.tile_at(s + 1) - sh.tab.tile_at(s) : 0;
+  }
+  // The segment that holds tile x, and the tiles before it; with no such tile, -1 and the number of tiles.
+  static __device__ __forceinline__ int find(const ListArgs& a, int x, int& before) {
+    const int lane = threadIdx.x & 31, n = a.n_layers * a.sh.n_seqs * a.sh.n_kv_heads;
+    before = 0;
+    for (int base = 0; base < n; base += 32) {
+      const int t = tiles(a, base + lane);
+      int inc = t;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      const unsigned hit = __ballot_sync(0xffffffffu, x >= before + inc - t && x < before + inc);
+      if (hit) {
+        const int l = __ffs(hit) - 1;
+        before += __shfl_sync(0xffffffffu, inc - t, l);
+        return base + l;
+      }
+      before += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    return -1;
+  }
+  __device__ __forceinline__ void start(const ListArgs& a) {
+    int all;
+    find(a, 0x7fffffff, all);
+    pos = split_begin((int)blockIdx.x, all, (int)gridDim.x);
+    end = split_begin((int)blockIdx.x + 1, all, (int)gridDim.x);
+  }
+  // The next run into d (lane 0); its kind.
+  __device__ __forceinline__ int next(const ListArgs& a, RunDesc& d) {
+    if (pos >= end) {
+      if ((threadIdx.x & 31) == 0) d.kind = 2;
+      return 2;
+    }
+    int before;
+    const int i = find(a, pos, before);
+    const ScoreShape& sh = a.sh;
+    const int n_seg = sh.n_seqs * sh.n_kv_heads, layer = i / n_seg, seg = i - layer * n_seg, s = seg / sh.n_kv_heads, g = seg - s * sh.n_kv_heads;
+    const int tiles_seg = sh.tab.tile_at(s + 1) - sh.tab.tile_at(s), t0 = pos - before, count = min(end - pos, tiles_seg - t0);
+    pos += count;
+    if ((threadIdx.x & 31) == 0) {
+      const ScoreLayer& L = a.lay[layer];
+      const int n_hist = sh.tab.cu_at(s + 1) - sh.tab.cu_at(s) - sh.window;
+      d.kind = 1;
+      d.gg = 0;
+      d.layer = layer;
+      d.tm_q = &L.tm_q;
+      d.tm_k = &L.tm_k;
+      d.count = count;
+      d.n_valid = n_hist - t0 * kTileKeys;
+      d.tok = sh.tab.cu_at(s) + t0 * kTileKeys;
+      d.s = s;
+      d.g = g;
+      d.last = 0;
+      d.n_slots = list_slots(sh, a.n_layers, layer, s, g).n;
+      d.slot = 0;
+      d.vote = L.vote + sh.tab.hist_at(s) * sh.n_kv_heads + (long long)g * n_hist + t0 * kTileKeys;
+      d.seg = seg;
+      d.acc = static_cast<double*>(L.part) + (long long)seg * sh.R;
+      d.far = reinterpret_cast<unsigned*>(static_cast<double*>(L.part) + (long long)n_seg * sh.R) + seg * kFarWords;
+      d.weight = nullptr;
+      d.second = 0;
+      d.sums = 1;
+      d.win = L.lse.win_m != nullptr;
+      d.q_y = sh.q_head_inner ? g * sh.G : 0;
+      d.q_z = sh.q_head_inner ? 0 : g * sh.G;
+    }
+    return 1;
   }
 };
 // Run k, read by a single thread or by a whole warp; kind 2 when there is none left (or a wait ran out).
@@ -271,7 +363,7 @@ __device__ __forceinline__ RunDesc take_run(const Smem& c, int k) {
 }
 
 // ---- warp 0, one thread: TMA loads ------------------------------------------------------------------------------
-template <int HALVES>
+template <int MT, int HALVES, bool BOUND>
 __device__ __forceinline__ void producer(const Smem& c) {
   int st = 0, it = 0, n = 0;                                 // stage, tiles so far, runs so far
   uint32_t st_phase = 0;
@@ -303,9 +395,10 @@ __device__ __forceinline__ void producer(const Smem& c) {
     q_map = r.tm_q; q_y = r.q_y; q_z = r.q_z; q_s = r.s;
     q_due = true;
     ++n;
-    const uint64_t policy = r.kind == 0 && c.both ? keep : drop;
-    int tok = r.tok;
-    for (int i = 0; i < r.count; ++i, ++it, tok += kTileKeys) {
+    const uint64_t policy = !BOUND && r.kind == 0 && c.both ? keep : drop;
+    const Spread<MT> order(BOUND && r.kind == 0 ? r.count : 0);
+    for (int i = 0; i < r.count; ++i, ++it) {
+      const int tok = r.tok + (BOUND && r.kind == 0 ? order.tile(i) : i) * kTileKeys;
       // a stage of the ring, and Q as soon as the MMAs of the run that had its slot are through with it
       bool got = false;
       unsigned long long t0 = 0;
@@ -407,26 +500,38 @@ __device__ __forceinline__ void issuer(const Smem& c) {
 
 // ---- warp 2: hands out the runs; announces statistics -----------------------------------------------------------------
 // Whatever is possible next is done: a run slot that has come free is filled, statistics that are out are announced.
-template <int MT>
+template <int MT, bool BOUND>
 __device__ __forceinline__ void scheduler_publisher(const Smem& c, const ListArgs& a) {
   const int lane = threadIdx.x & 31;
   int k_out = 0, k_in = 0;                 // runs handed out, runs done with as publisher
   int n = 0;                               // statistics runs so far
   bool all_out = false;
   const int n_seg = a.sh.n_seqs * a.sh.n_kv_heads, stride = a.sh.slot_stride;
-  RunWalk w;
+  RunWalk<BOUND> w;
   w.start();
+  FullWalk full;
+  bool votes = false;                      // bounds: behind the statistics' last run
   unsigned long long t0 = 0;
   unsigned idle = 0;
   while (true) {
     bool moved = false;
     if (!all_out && __any_sync(0xffffffffu, mbar_test(c.run_empty(k_out), ((k_out / kRunSlots) & 1) ^ 1))) {
       int kind = 0;
-      if (lane == 0) {
-        w.next(a, c.runs[k_out & (kRunSlots - 1)]);
+      RunDesc& d = c.runs[k_out & (kRunSlots - 1)];
+      if (lane == 0 && !(BOUND && votes)) {
+        w.next(a, d);
         kind = w.kind;
-        mbar_arrive(c.run_full(k_out));
       }
+      if constexpr (BOUND) {
+        kind = __shfl_sync(0xffffffffu, kind, 0);
+        if (kind == 2 && !votes) {
+          votes = true;
+          pdl_wait();                                        // budgets may come from a kernel before this one
+          full.start(a);
+        }
+        if (votes) kind = full.next(a, d);
+      }
+      if (lane == 0) mbar_arrive(c.run_full(k_out));
       all_out = __shfl_sync(0xffffffffu, kind, 0) == 2;    // also orders the lanes behind lane 0's stores
       ++k_out;
       moved = true;
@@ -590,7 +695,7 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
 }
 
 // ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
-template <int MT>
+template <int MT, bool BOUND>
 __device__ __forceinline__ void epilogue(const Smem& c) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wg = (threadIdx.x - 128) >> 7, row = threadIdx.x & 127;
@@ -604,7 +709,8 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
   constexpr int every = MT == 1 ? kWgs : kWgs / 2, log_every = MT == 1 ? 2 : 1;
   const int mine = MT == 1 ? wg : wg >> 1, mt = MT == 1 ? 0 : wg & 1;
   const bool rows_here = mt * 128 + (warp & 3) * 32 < c.R;                // some row of this warp's lanes exists
-  int it = 0, units = 0, n_stat = 0, n_vote = 0, n_half = 0;
+  const int own = BOUND ? (row & ~31) + quad_row() : row;                // the row whose statistics this thread ends up with
+  int it = 0, units = 0, n_stat = 0, n_vote = 0, n_half = 0, n_part = 0, n_again = 0;
   for (int k = 0;; ++k) {
     const RunDesc r = take_run<true>(c, k);
     if (r.kind == 2) break;
@@ -616,16 +722,37 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
     if (r.kind == 0) {
       double z;
       float far_z, far_m;
-      ok = stats_run(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, z, far_z, far_m);
+      if constexpr (BOUND) {
+        const int sharers = MT == 1 ? wg : mine;               // the warpgroups that share a tile share a buffer and its barriers
+        BoundRun b;
+        b.sums = c.first + (n_stat & 1) * (kWgs * 128);
+        b.sums_bar = c.first_full(n_stat & 1);
+        b.sums_parity = (uint32_t)(n_stat >> 1) & 1u;
+        b.part = c.half_vote + sharers * (MT * 1024);
+        b.part_bars = c.part_full(2 * sharers);
+        b.n_part = n_part;
+        b.again_bar = c.again_full();
+        b.again_parity = (uint32_t)n_again & 1u;
+        n_again += second_weights(r.count) < r.count;
+        b.weight = r.weight;
+        b.second = r.second;
+        b.est = r.vote;
+        b.rows = c.R;
+        b.n_warps = (c.R + 31) >> 5;
+        ok = bound_run<MT>(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, wg, b, z, far_z, far_m);
+        n_part += n_mine;
+      } else {
+        ok = stats_run(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, z, far_z, far_m);
+      }
       const int slot = n_stat & 1;
       ok = ok && mbar_wait(c.stat_empty(slot), ((n_stat >> 1) & 1) ^ 1, c.abort_flag) && mbar_wait(c.cleared(), 0, c.abort_flag);
       ++n_stat;
       if (!__all_sync(0xffffffffu, ok)) break;
-      if (z > 0.0 && mt * 128 + row < c.R)
-        asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(r.acc + mt * 128 + row), "d"(z) : "memory");
+      if (z > 0.0 && mt * 128 + own < c.R)
+        asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(r.acc + mt * 128 + own), "d"(z) : "memory");
       if (__any_sync(0xffffffffu, far_z > 0.f)) {
-        c.stat_z[(slot * kWgs + wg) * 128 + row] = far_z;
-        c.stat_m[(slot * kWgs + wg) * 128 + row] = far_m;
+        c.stat_z[(slot * kWgs + wg) * 128 + own] = far_z;
+        c.stat_m[(slot * kWgs + wg) * 128 + own] = far_m;
         if (lane == 0) atomicOr(c.stat_far + slot, 1u << (wg * 4 + (warp & 3)));
       }
       __syncwarp();
@@ -650,7 +777,9 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
 // that do the arithmetic is what the instruction caches have to hold, and a row block's constants are folded into it.  With one
 // kernel for all, 32 layers of 4001 / 8000 / 32k tokens, 128 rows: 123.7 / 225 / 838 us, now 121.1 / 220 / 812; 16000 tokens, 64 rows
 // 376 -> 353; four sequences of 5k - 10k 689 -> 658; 256 rows as before.
-template <int MT, int HALVES>
+// BOUND: statistics and estimated votes in one pass over the list, then the votes of the segments that need them all
+// (slkv_bound.cu); a kernel of its own, so that neither kind's loops grow.
+template <int MT, int HALVES, bool BOUND>
 __global__ void __launch_bounds__(kListThreads, 1)
 k_score_list(const __grid_constant__ ListArgs a) {
   // Shared memory, all dynamic and 1024-byte aligned (the swizzled tiles need it):
@@ -677,7 +806,8 @@ k_score_list(const __grid_constant__ ListArgs a) {
   c.stat_far = reinterpret_cast<unsigned*>(tail + kBarBytes - 8);
   c.lse = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes);
   c.half_vote = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes + kLseBytes);
-  c.runs = reinterpret_cast<RunDesc*>(tail + kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes);
+  c.first = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes + kLseBytes + kPartBytes);
+  c.runs = reinterpret_cast<RunDesc*>(tail + kBarBytes + kStatBytes + kLseBytes + kPartBytes + kFirstBytes);
 
   if (tid == 0) {
     trace_mark(a.trace, 0);
@@ -688,6 +818,7 @@ k_score_list(const __grid_constant__ ListArgs a) {
     c.stat_far[0] = c.stat_far[1] = 0;
     mbar_init(c.cleared(), 1);
     mbar_init(c.rest_cleared(), 1);
+    mbar_init(c.again_full(), 4 * kWgs);
     for (int st = 0; st < kMaxStages; ++st) { mbar_init(c.full(st), 1); mbar_init(c.empty(st), 1); }
     for (int u = 0; u < 4; ++u) { mbar_init(c.unit_full(u), 1); mbar_init(c.unit_empty(u), 4); }
     for (int s = 0; s < 2; ++s) {
@@ -695,7 +826,8 @@ k_score_list(const __grid_constant__ ListArgs a) {
       mbar_init(c.stat_empty(s), 1);
       mbar_init(c.lse_full(s), 1);
       mbar_init(c.lse_empty(s), 4 * kWgs);
-      for (int t = 0; t < 4; ++t) mbar_init(c.half_full(s, t), 4);
+      for (int t = 0; t < 4; ++t) { mbar_init(c.half_full(s, t), 4); mbar_init(c.part_full(4 * s + t), 4 * MT); }
+      mbar_init(c.first_full(s), 4 * kWgs);
     }
     for (int k = 0; k < kQTiles; ++k) { mbar_init(c.q_full(k), 1); mbar_init(c.q_empty(k), 1); }
     for (int k = 0; k < kRunSlots; ++k) { mbar_init(c.run_full(k), 1); mbar_init(c.run_empty(k), kRunReaders); }
@@ -735,18 +867,18 @@ k_score_list(const __grid_constant__ ListArgs a) {
     if (lane == 0) {
       pdl_wait();
       trace_mark(a.trace, 1);
-      producer<HALVES>(c);
+      producer<MT, HALVES, BOUND>(c);
     }
   } else if (warp == 1) {
     if (lane == 0) issuer<MT, HALVES>(c);
   } else if (warp == 2) {
     if (sh.tab.n_inline == 0) pdl_wait();              // a kernel before this one writes the tables
-    scheduler_publisher<MT>(c, a);
+    scheduler_publisher<MT, BOUND>(c, a);
   } else if (warp == 3) {
     pdl_wait();
     fetch_lse(c, a);
   } else {
-    epilogue<MT>(c);
+    epilogue<MT, BOUND>(c);
   }
 
   tc_fence_before();
@@ -810,10 +942,14 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
                               unsigned long long* sync, cudaStream_t st, int* launches, bool cleared) {
   if (n_layers < 1 || sh.n_cta == 0) return cudaSuccess;             // no history: nothing to score
   if (n_layers > kListMaxLayers) return cudaErrorInvalidValue;
-  const Kern kernel = sh.MT == 1 ? (sh.halves == 1 ? k_score_list<1, 1> : k_score_list<1, 2>)
-                                 : (sh.halves == 1 ? k_score_list<2, 1> : k_score_list<2, 2>);
-  static thread_local int configured_on[2][2] = {{-1, -1}, {-1, -1}};
-  int& configured_dev = configured_on[sh.MT - 1][sh.halves - 1];
+  const bool bound = passes == kScoreBound;
+  if (bound) passes = 3;
+  const Kern kernel = sh.MT == 1 ? (sh.halves == 1 ? (bound ? k_score_list<1, 1, true> : k_score_list<1, 1, false>)
+                                                   : (bound ? k_score_list<1, 2, true> : k_score_list<1, 2, false>))
+                                 : (sh.halves == 1 ? (bound ? k_score_list<2, 1, true> : k_score_list<2, 1, false>)
+                                                   : (bound ? k_score_list<2, 2, true> : k_score_list<2, 2, false>));
+  static thread_local int configured_on[2][2][2] = {{{-1, -1}, {-1, -1}}, {{-1, -1}, {-1, -1}}};
+  int& configured_dev = configured_on[sh.MT - 1][sh.halves - 1][bound];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -827,8 +963,9 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   std::memcpy(a.lay, lay, sizeof(ScoreLayer) * (size_t)n_layers);
   a.n_layers = n_layers;
   a.passes = passes;
-  // A single pass needs no groups: the whole list is one (its tiles are counted in 32 bits times the CTAs).
-  const bool one_group = passes != 3 && (long long)sh.total_tiles * n_layers < (1 << 24);
+  // A single product needs no groups: the whole list is one (its tiles are counted in 32 bits times the CTAs).
+  const bool one_group = (bound || passes != 3) && (long long)sh.total_tiles * n_layers < (1 << 24);
+  if (bound && !one_group) return cudaErrorNotSupported;
   a.group_layers = one_group ? n_layers : (n_layers > 1 ? sh.group_layers : 0);
   a.n_groups = a.group_layers == 0 ? n_layers * sh.n_groups : (n_layers + a.group_layers - 1) / a.group_layers;
   // units per CTA and phase, about
@@ -862,6 +999,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   static thread_local int coop_state[64] = {};        // per device: 0 untried, 1 with dependent launch, 2 without, -1 refused
   int& cs = coop_state[dev < 64 ? dev : 0];
   if (waits_inside && (env_no_coop || cs == -1 || sh.n_cta > sm_count())) {
+    if (bound) return cudaErrorNotSupported;
     a.passes = 1;
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
@@ -906,6 +1044,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     cs = 2;                                           // once more without dependent launch
   }
   cs = -1;
+  if (bound) return cudaErrorNotSupported;
   return launch_score_list(sh, lay, n_layers, passes, sync, st, launches);
 }
 

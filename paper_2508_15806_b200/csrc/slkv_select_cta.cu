@@ -143,8 +143,9 @@ k_select_list(const __grid_constant__ SelArgs args) {
 
   // (0: a barrier of all T threads)
   int o_mine;
+  unsigned tau;
   const unsigned kept = select_places<T, IT, CLUSTER, 0>(sh, tid, key, valid, mine, reinterpret_cast<uint4*>(votes + tid * kPitch), n,
-                                                         k_keep, rank, CS, o_mine);
+                                                         k_keep, rank, CS, o_mine, tau);
   // the kept positions, in shared memory first (where the votes were): whole lines then go out
   int* const stage = reinterpret_cast<int*>(votes_sh);
   int o0 = 0, o1 = k_keep;                                 // the CTA's rows among the segment's
@@ -166,13 +167,12 @@ k_select_list(const __grid_constant__ SelArgs args) {
 // cluster cost as much as the smaller slices save (one layer of 8 segments, the whole call in us with 1, 2, 4 and 8 CTAs of an
 // earlier selection per segment: 1024 tokens 26.6, 30.7, 30.8, 32.7; 8192 tokens 32.8, 35.4, 36.8, 38.6; 32768 tokens 48.6, 49.2,
 // 48.2, 49.3).
-int cluster_size(const Problem& pb) {
+}  // namespace
+int select_list_cluster(const Problem& pb) {
   int cs = 1;
   while (cs < kMaxCluster && (pb.max_hist + 3 + cs - 1) / cs + 3 > kMaxSlice) cs *= 2;
   return cs;
 }
-
-}  // namespace
 
 // up to 262116 history positions
 bool select_list_supported(const Problem& pb) {
@@ -206,7 +206,7 @@ const SelVariant& variant_for(int cs, int slice, long long ctas) {
 }  // namespace
 
 cudaError_t launch_select_list(const Problem& pb, const TailLayer* lay, int n_layers, cudaStream_t st, int* launches) {
-  const int cs = cluster_size(pb);
+  const int cs = select_list_cluster(pb);
   const int slice = ((pb.max_hist + 3 + cs - 1) / cs + 3) & ~3;
   const SelVariant& var = variant_for(cs, slice, (long long)pb.n_seg * n_layers);
   const size_t smem = (size_t)vote_floats(var.threads, var.items) * sizeof(float);

@@ -27,7 +27,7 @@ __device__ __forceinline__ unsigned first_bin(unsigned v) {
 // accesses of neighbouring threads conflict-free -- behind eight floats that hold the four before the first.
 constexpr int kLead = 8;
 template <int IT> constexpr int kLogItems = IT == 8 ? 3 : (IT == 16 ? 4 : 5);
-constexpr int vote_floats(int threads, int items) { return kLead + (threads + 1) * (items + 4); }
+__host__ __device__ constexpr int vote_floats(int threads, int items) { return kLead + (threads + 1) * (items + 4); }
 
 __device__ __forceinline__ int kept_rows(int len, int budget, int window) { return min(len, max(budget, window)); }
 
@@ -75,10 +75,10 @@ struct alignas(16) SelShared {
 // largest, ties to the lower place.  CLUSTER: the segment is shared by the CTAs of a cluster (rank, CS).  BAR: the named
 // barrier of the T threads.  shelf: the thread's row of the votes' shared memory, which the scores take over once all T
 // threads are past their pooling (IT > 8 only).  sh.hist, sh.sample, sh.n_list and sh.sure are zero, for all to see.
-// Returns the kept places as a mask and, in o_mine, how many of the segment's lie before the thread's.
+// Returns the kept places as a mask and, in o_mine, how many of the segment's lie before the thread's; tau: the k-th largest score.
 template <int T, int IT, bool CLUSTER, int BAR>
 __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsigned (&key)[IT], unsigned valid, bool mine,
-                                                  uint4* shelf, int n, int k_keep, int rank, int CS, int& o_mine) {
+                                                  uint4* shelf, int n, int k_keep, int rank, int CS, int& o_mine, unsigned& tau) {
   constexpr int kWarps = T / 32, kPer = kBins / T;      // bins per thread
   constexpr int kRanked = kList < T ? kList : T;        // a bin of more scores goes through another level of bins
   static_assert(kRanked <= T && kRanked <= kList && kPer % 2 == 0 && kWarps <= 32, "a thread per listed score, whole int2 of bins");
@@ -168,7 +168,7 @@ __device__ __forceinline__ unsigned select_places(SelShared& sh_, int tid, unsig
     }
   };
   int need = k_keep;
-  unsigned lo = 0, hi = kAll, gt = 0, cand = valid, tau;
+  unsigned lo = 0, hi = kAll, gt = 0, cand = valid;
   int sh = kFirstShift;
   bool first = true;
   while (true) {

@@ -151,18 +151,12 @@ __device__ __forceinline__ f32x2 ex2_pair(f32x2 x) {
 // both passes (one exponential per query row and key): x = n + f with n = round(x), 2^f by a degree-5 polynomial that
 // is minimax in relative error on [-0.5, 0.5] (Remez exchange; 2.1e-7 evaluated in fp32, ex2.approx has 2^-22 =
 // 2.4e-7), n added into the exponent field.  x is clamped at -125 (the result is then 2^-125: negligible in any sum
-// that holds a term near 1) and, where CLAMP_HI, at 128.5, from where the exponent field overflows to Inf / NaN, which
-// the statistics pass's overflow check catches.
-template <bool CLAMP_HI>
+// that holds a term near 1).
 __device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {
   float a, b;
   unpack2(x, a, b);
   a = fmaxf(a, -125.f);
   b = fmaxf(b, -125.f);
-  if (CLAMP_HI) {
-    a = fminf(a, 128.5f);
-    b = fminf(b, 128.5f);
-  }
   x = pack2(a, b);
   const f32x2 t = add2(x, pack2(12582912.f, 12582912.f));     // 1.5 * 2^23: round(x) lands in the low mantissa bits
   const f32x2 f = fma2(add2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x);
@@ -208,6 +202,26 @@ __device__ __forceinline__ uint32_t instr_desc(int M, int N) {
 __device__ __forceinline__ int split_begin(int i, int T, int n) { return (int)(((unsigned)i * (unsigned)T) / (unsigned)n); }
 __device__ __forceinline__ int split_index(int x, int T, int n) {
   return (int)((((unsigned)x + 1u) * (unsigned)n - 1u) / (unsigned)T);
+}
+// In how many parts the CTAs of a launch whose list is one group share a segment (n, from the `first` of the split on).
+struct SegmentSlots {
+  int before, tiles, shares, first, n;         // of the list's tiles: before the segment, all; shares they are split into
+  int tiles_seg;
+  __device__ __forceinline__ int slot(int tile) const { return split_index(before + tile, tiles, shares) - first; }
+  // Part c: its first tile, of the segment, and how many.
+  __device__ __forceinline__ int begin(int c) const { return max(split_begin(first + c, tiles, shares) - before, 0); }
+  __device__ __forceinline__ int count(int c) const { return min(split_begin(first + c + 1, tiles, shares) - before, tiles_seg) - begin(c); }
+};
+__device__ __forceinline__ SegmentSlots list_slots(const ScoreShape& sh, int n_layers, int layer, int s, int g) {
+  SegmentSlots x;
+  const int tiles_seg = sh.tab.tile_at(s + 1) - sh.tab.tile_at(s);
+  x.tiles = n_layers * sh.total_tiles;
+  x.tiles_seg = tiles_seg;
+  x.shares = min(sh.n_cta, x.tiles);
+  x.before = layer * sh.total_tiles + sh.n_kv_heads * sh.tab.tile_at(s) + g * tiles_seg;
+  x.first = split_index(x.before, x.tiles, x.shares);
+  x.n = split_index(x.before + tiles_seg - 1, x.tiles, x.shares) - x.first + 1;
+  return x;
 }
 // Row statistics in global memory, per segment and row: acc = the sum of 2^score over all keys, in fp64 and without a
 // reference.  The terms are fp32 sums over one tile each, added atomically in whatever order they come.  n of them within a
@@ -318,31 +332,40 @@ __device__ __forceinline__ void tile_stats_exact(uint32_t tcol, float sc, int fi
 }
 
 // ---- the epilogue warps' arithmetic on accumulators --------------------------------------------------------------------
-// sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials go
-// to the FMA pipe, where it takes fourteen instructions instead of two.  By cycles alone two pairs of eight would go there;
+// Votes: sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials
+// go to the FMA pipe, where it takes fourteen instructions instead of two.  By cycles alone two pairs of eight would go there;
 // at the power limit the instructions cost more clock than they save cycles (32 layers of 32k / 128k positions, in both
-// passes no pair of a chunk's eight on the FMA pipe 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: one pair of eight
-// in the statistics, in the votes one in every other chunk.
+// passes no pair of a chunk's eight on the FMA pipe 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: none in the
+// statistics, in the votes one in every other chunk.
 // The loops around this are kept small, the statistics' one chunk at a time with the last keys of a segment outside: four
 // warps on a scheduler hide a TMEM load's latency, and the epilogue warps are spread over both passes' loops, which have to
 // stay in the instruction cache (4k positions: statistics loop unrolled four times 154 us, twice 144, two chunks with the
 // last keys masked inside 140.9, as it is 140.1; 128k: 6147, 5865, 5868, 5820).
-template <bool STATS, bool POLY>
-__device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 off, uint32_t off_sh, f32x2& s0,
-                                          f32x2& s1) {
+template <bool POLY>
+__device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, uint32_t off_sh, f32x2& s0, f32x2& s1) {
 #pragma unroll
   for (int e = 0; e < 16; e += 4) {
-    f32x2 o0 = off, o1 = off;
-    if (!STATS) {
-      // an explicit shared-memory load: a generic one takes another path
-      asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(o0), "=l"(o1) : "r"(off_sh + 4u * e));
-    }
+    f32x2 o0, o1;
+    // an explicit shared-memory load: a generic one takes another path
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(o0), "=l"(o1) : "r"(off_sh + 4u * e));
     const f32x2 x0 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, o0);
     const f32x2 x1 = fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sc2, o1);
-    s0 = add2(s0, POLY && e == 0 ? ex2_pair_poly<STATS>(x0) : ex2_pair(x0));
+    s0 = add2(s0, POLY && e == 0 ? ex2_pair_poly(x0) : ex2_pair(x0));
     s1 = add2(s1, ex2_pair(x1));
   }
 }
+// Statistics: a row's sum of 2^(v * sc) over a tile goes through eight accumulators, one for each column modulo 8, here four
+// pairs; stats_sum adds those up.  (Eight, because that is how the columns lie in the lanes of bound_run.)
+__device__ __forceinline__ void stats_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 (&s)[4]) {
+#pragma unroll
+  for (int e = 0; e < 16; e += 2) s[(e >> 1) & 3] = add2(s[(e >> 1) & 3], ex2_pair(fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, 0)));
+}
+__device__ __forceinline__ float pair_sum(f32x2 v) {
+  float a, b;
+  unpack2(v, a, b);
+  return a + b;
+}
+__device__ __forceinline__ float stats_sum(const f32x2 (&s)[4]) { return (pair_sum(s[0]) + pair_sum(s[1])) + (pair_sum(s[2]) + pair_sum(s[3])); }
 
 // An epilogue thread's unit.
 struct Unit {
@@ -377,15 +400,15 @@ __device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i
     if (rows_here) {
       const int n_valid = n_valid0 - i * kTileKeys;
       const int whole = n_valid < kTileKeys ? n_valid & ~15 : kTileKeys;
-      f32x2 s0 = 0, s1 = 0;
+      f32x2 s[4] = {0, 0, 0, 0};
 #pragma unroll 1
       for (int c0 = 0; c0 < whole; c0 += 16) {
         uint32_t v[16];
         tc_ld16_issue(u.tcol + c0, v);
         tc_ld_wait(v);
-        exp_chunk<true, true>(v, sc2, 0, 0u, s0, s1);
+        stats_chunk(v, sc2, s);
       }
-      float tile = sum2(s0, s1);
+      float tile = stats_sum(s);
       if (n_valid < kTileKeys) {                               // the segment's last keys; those past its end count nothing
         float tm, tz;
         tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
@@ -403,6 +426,259 @@ __device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i
       }
     }
     unit_release(u);
+  }
+  return true;
+}
+
+// ---- statistics and estimated votes from one product ------------------------------------------------------------------------
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// Both halves rounded to bf16, the first in the low half.
+__device__ __forceinline__ uint32_t bf16_pair(f32x2 v) {
+  float a, b;
+  unpack2(v, a, b);
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
+__device__ __forceinline__ uint32_t add_bf16(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+// 16 TMEM columns of this warp's 32 lanes as a matrix operand lies in registers: thread 4 g + t has the columns 2 t and 2 t + 1 of
+// the eight at 8 b for the rows g + 8 q in v[8 (q >> 1) + 4 b + 2 (q & 1)] and the one behind it.
+__device__ __forceinline__ void tc_ld_quads(uint32_t taddr, uint32_t (&v)[16]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[8 * i]), "=r"(v[8 * i + 1]), "=r"(v[8 * i + 2]), "=r"(v[8 * i + 3]), "=r"(v[8 * i + 4]), "=r"(v[8 * i + 5]),
+                   "=r"(v[8 * i + 6]), "=r"(v[8 * i + 7])
+                 : "r"(taddr + ((uint32_t)i << 20)) : "memory");
+}
+// The row, of the warp's 32, whose sum a thread has in the end.
+__device__ __forceinline__ int quad_row() { return ((threadIdx.x & 31) >> 2) + 8 * (threadIdx.x & 3); }
+// stats_chunk for four rows of two columns in eight, whose sums these are bit for bit (s[q]: row g + 8 q), and the four rows'
+// weight * exponential of the two columns in h[b], rounded to bf16.
+__device__ __forceinline__ void bound_chunk(const uint32_t (&v)[16], f32x2 sc2, const f32x2 (&w2)[4], f32x2 (&s)[4], uint32_t* h) {
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    f32x2 est = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int at = 8 * (q >> 1) + 4 * b + 2 * (q & 1);
+      const f32x2 p = ex2_pair(fma2(pack2(__uint_as_float(v[at]), __uint_as_float(v[at + 1])), sc2, 0));
+      s[q] = add2(s[q], p);
+      est = q == 0 ? mul2(p, w2[0]) : fma2(p, w2[q], est);
+    }
+    h[b] = bf16_pair(est);
+  }
+}
+// stats_sum of the thread's row: of the four rows that lie in four lanes each, a lane keeps one.
+__device__ __forceinline__ float quad_sum(const f32x2 (&s)[4]) {
+  const bool odd = threadIdx.x & 1, high = threadIdx.x & 2;
+  float a[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) a[q] = pair_sum(s[q]);
+  const float lo = (odd ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, odd ? a[0] : a[1], 1);
+  const float hi = (odd ? a[3] : a[2]) + __shfl_xor_sync(0xffffffffu, odd ? a[2] : a[3], 1);
+  return (high ? hi : lo) + __shfl_xor_sync(0xffffffffu, high ? lo : hi, 2);
+}
+// The sums over the warp's rows of 64 columns (h[b]: of those at 8 b) or of 16, out[0 ..]: of two registers a lane keeps one and
+// sends the other.
+__device__ __forceinline__ void lane_sums(uint32_t (&h)[8], float* out) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = 4; n >= 1; n >>= 1)
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const uint32_t keep = lane & (4 * n) ? h[i + n] : h[i], send = lane & (4 * n) ? h[i] : h[i + n];
+      h[i] = add_bf16(keep, __shfl_xor_sync(0xffffffffu, send, 4 * n));
+    }
+  reinterpret_cast<float2*>(out)[lane] = make_float2(__uint_as_float(h[0] << 16), __uint_as_float(h[0] & 0xffff0000u));
+}
+__device__ __forceinline__ void lane_sums(uint32_t (&h)[2], float* out) {
+  const int lane = threadIdx.x & 31;
+  uint32_t x = add_bf16(lane & 16 ? h[1] : h[0], __shfl_xor_sync(0xffffffffu, lane & 16 ? h[0] : h[1], 16));
+  x = add_bf16(x, __shfl_xor_sync(0xffffffffu, x, 8));
+  x = add_bf16(x, __shfl_xor_sync(0xffffffffu, x, 4));
+  if ((lane & 12) == 0) reinterpret_cast<float2*>(out)[4 * (lane >> 4) + (lane & 3)] = make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
+}
+
+// The order in which a run's tiles are taken where the first kFirst are to be spread over it: tile j and tile
+// j (count - 1) / (kFirst - 1) change places.
+template <int MT>
+struct Spread {
+  static constexpr int kFirst = MT == 1 ? 4 : 2;
+  int to[kFirst];                                              // where tile j lies; tile 0 stays
+  __device__ __forceinline__ explicit Spread(int count) {
+#pragma unroll
+    for (int j = 0; j < kFirst; ++j) to[j] = count >= 16 ? j * (count - 1) / (kFirst - 1) : j;
+  }
+  __device__ __forceinline__ int tile(int i) const {
+    int t = i;
+#pragma unroll
+    for (int j = 1; j < kFirst; ++j) t = i == j ? to[j] : (i == to[j] ? j : t);
+    return t;
+  }
+};
+
+// In the order of Spread, the first tile with the second set of weights, the reciprocals of the rows' sums over the tiles before it:
+// a quarter of a long run, none of a short one.
+__device__ __forceinline__ int second_weights(int count) { return count >= 64 ? count >> 2 : 0x7fffffff; }
+
+// What the warpgroups of a CTA tell one another in a run for bounds.
+struct BoundRun {
+  float* sums;                 // [4][128]: the rows' sums over the warpgroup's first tile
+  uint32_t sums_bar;           // every epilogue warp
+  uint32_t sums_parity;
+  uint32_t again_bar;          // the same for the second weights
+  uint32_t again_parity;
+  float* part;                 // two slots of the sharing warpgroups' warps' shares [4 MT][128]
+  uint32_t part_bars;
+  int n_part;                  // tiles these warpgroups have been through
+  float* weight;               // where the rows' weights go; the second ones `second` floats further on
+  int second;
+  float* est;                  // estimated votes, of the run's first key
+  int rows, n_warps;           // rows per KV head, warps that hold some
+};
+
+// Statistics of one run, as stats_run (the sums are the same bit for bit, but of row quad_row() of the warp's), and with the same exponentials an estimate of every key's
+// vote, est[key] = sum_rows weight_r * 2^score.  The rows' sums are not known yet: weight_r is the reciprocal of the row's sum over
+// the run's first tiles in the order of Spread, one per warpgroup (two: per pair), whose accumulators are read twice for it, and from a
+// quarter of the run on over that quarter (the bounds are three to five times as tight in the keys that they let through).  The
+// warps' shares of a tile, 32 rows each, meet in shared memory, two slots in turn (a warp is back at a slot only once all have
+// passed the barrier of the one behind, and so have read it).
+template <int MT>
+__device__ __forceinline__ bool bound_run(const Unit u, int nth, float sc, int i0, int every, int count, int n_valid0, bool rows_here,
+                                          int wg, BoundRun b, double& z, float& far_z, float& far_m) {
+  constexpr int kShare = 4 * MT * 128;
+  z = 0.0;
+  far_z = far_m = 0.f;
+  const f32x2 sc2 = pack2(sc, sc);
+  const int row = threadIdx.x & 127, lane = threadIdx.x & 31, mt = MT == 1 ? 0 : wg & 1, warp = mt * 4 + (row >> 5);
+  const Spread<MT> order(count);
+  float first = 0.f;
+  if (i0 < count) {
+    if (!unit_wait(u, nth)) return false;
+    if (rows_here) {
+      const int n_valid = n_valid0 - order.tile(i0) * kTileKeys, whole = n_valid < kTileKeys ? n_valid & ~15 : kTileKeys;
+      f32x2 s[4] = {0, 0, 0, 0};
+#pragma unroll 1
+      for (int c0 = 0; c0 < whole; c0 += 16) {
+        uint32_t v[16];
+        tc_ld16_issue(u.tcol + c0, v);
+        tc_ld_wait(v);
+        stats_chunk(v, sc2, s);
+      }
+      first = stats_sum(s);
+      if (whole < n_valid && whole < kTileKeys) {
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
+        first += tz * ex2(tm);
+      }
+    }
+  }
+  b.sums[wg * 128 + row] = first;
+  __syncwarp();
+  if (lane == 0) mbar_arrive(b.sums_bar);
+  const bool there = mbar_wait(b.sums_bar, b.sums_parity, u.abort_flag);
+  if (!__all_sync(0xffffffffu, there)) return false;
+  // Sums between 2^-60 and 2^100: what fp32 flushes to zero is then 2^-66 of a row at most and nothing overflows.  A weight that is not
+  // finite makes every estimate so.
+  const int row0 = mt * 128 + (row & ~31), own = quad_row();
+  f32x2 w2[4];
+  auto weigh = [&](float* out) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = row0 + (lane >> 2) + 8 * q;
+      float total = b.sums[r];                                 // of warpgroup mt, rows of block mt
+#pragma unroll
+      for (int w = MT; w < 4; w += MT) total += b.sums[w * 128 + r];
+      float weight = total >= 0x1p-60f && total <= 0x1p100f ? __fdividef(1.f, total) : __int_as_float(0x7fffffff);
+      if (r >= b.rows) weight = 0.f;
+      else if (wg < MT && q == (lane & 3)) __stcg(out + r, weight);
+      w2[q] = pack2(weight, weight);
+    }
+  };
+  weigh(b.weight);
+  int refresh = second_weights(count);
+#pragma unroll 1
+  for (int i = i0; i < count; i += every, ++nth, ++b.n_part) {
+    if (i >= refresh) {
+      // all warpgroups get here: a run this long has tiles for each behind that; and none still reads the first sums, for which
+      // its first unit had to be given back
+      refresh = 0x7fffffff;
+      b.sums[wg * 128 + (row & ~31) + own] = (float)z;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b.again_bar);
+      const bool all = mbar_wait(b.again_bar, b.again_parity, u.abort_flag);
+      if (!__all_sync(0xffffffffu, all)) return false;
+      weigh(b.weight + b.second);
+    }
+    if (!unit_wait(u, nth)) return false;
+    const int tile = order.tile(i), n_valid = n_valid0 - tile * kTileKeys, slot = b.n_part & 1;
+    float* const mine = b.part + slot * kShare + warp * 128;
+    if (rows_here) {
+      f32x2 s[4] = {0, 0, 0, 0};
+      float sum;
+      if (n_valid >= kTileKeys) {
+#pragma unroll 1
+        for (int c0 = 0; c0 < kTileKeys; c0 += 64) {
+          uint32_t v[16], h[8];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            tc_ld_quads(u.tcol + c0 + 16 * c, v);
+            tc_ld_wait(v);
+            bound_chunk(v, sc2, w2, s, h + 2 * c);
+          }
+          lane_sums(h, mine + c0);
+        }
+        sum = quad_sum(s);
+      } else {                                                 // a segment's last keys: the sums as in stats_run
+        const int whole = n_valid & ~15;
+        f32x2 unused[4] = {0, 0, 0, 0};
+#pragma unroll 1
+        for (int c0 = 0; c0 < n_valid; c0 += 16) {
+          uint32_t v[16], h[2];
+          tc_ld_quads(u.tcol + c0, v);
+          tc_ld_wait(v);
+          if (c0 < whole) bound_chunk(v, sc2, w2, s, h);
+          else bound_chunk(v, sc2, w2, unused, h);
+          lane_sums(h, mine + c0);
+        }
+        sum = quad_sum(s);
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
+        sum += __shfl_sync(0xffffffffu, tz * ex2(tm), own);
+      }
+      const bool exact = !(sum < INFINITY && sum > kTinySum);
+      if (!__any_sync(0xffffffffu, exact)) {
+        z += (double)sum;
+      } else {
+        float tm, tz;
+        tile_stats_exact(u.tcol, sc, 0, n_valid, tm, tz);
+        tm = __shfl_sync(0xffffffffu, tm, own);
+        tz = __shfl_sync(0xffffffffu, tz, own);
+        if (!exact) z += (double)sum;
+        else if (fabsf(tm) <= kFarScore) z += scalbn((double)tz, (int)tm);
+        else stat_add(far_z, far_m, tz, tm);
+      }
+    }
+    unit_release(u);
+    const uint32_t bar = b.part_bars + 8u * (uint32_t)slot;
+    if (lane == 0) mbar_arrive(bar);                           // behind the whole warp's stores: unit_release's __syncwarp
+    const bool ok = mbar_wait(bar, (b.n_part >> 1) & 1, u.abort_flag);
+    if (!__all_sync(0xffffffffu, ok)) return false;
+    if (MT == 1 || (row >> 6) == mt) {
+      const float* shares = b.part + slot * kShare + row;
+      float sum = shares[0];
+      for (int w = 1; w < b.n_warps; ++w) sum += shares[w * 128];
+      if (row < n_valid) b.est[tile * kTileKeys + row] = sum;
+    }
   }
   return true;
 }
@@ -428,10 +704,10 @@ __device__ __forceinline__ bool votes_run(const Unit u, int nth, float sc, int i
     for (int c0 = 0; c0 < cols; c0 += 32) {
       tc_ld_wait(ra);
       tc_ld16_issue(u.tcol + c0 + 16, rb);
-      exp_chunk<false, true>(ra, sc2, 0, lse + 4u * c0, s0, s1);
+      exp_chunk<true>(ra, sc2, lse + 4u * c0, s0, s1);
       tc_ld_wait(rb);
       if (c0 + 32 < cols) tc_ld16_issue(u.tcol + c0 + 32, ra); else unit_release(u);
-      exp_chunk<false, false>(rb, sc2, 0, lse + 4u * c0 + 64u, s0, s1);
+      exp_chunk<false>(rb, sc2, lse + 4u * c0 + 64u, s0, s1);
     }
     float acc = sum2(s0, s1);
     if (half >= 0) {
@@ -452,6 +728,23 @@ __device__ __forceinline__ bool votes_run(const Unit u, int nth, float sc, int i
     if (key < n_keys) out(key, acc * inv_g);
   }
   return true;
+}
+
+// A thread's key against this accumulator's rows (cols of them): votes_run's sum, bit for bit.
+__device__ __forceinline__ float key_vote(uint32_t tcol, int cols, float sc, uint32_t lse) {
+  const f32x2 sc2 = pack2(sc, sc);
+  uint32_t v[16];
+  f32x2 s0 = 0, s1 = 0;
+#pragma unroll 1
+  for (int c0 = 0; c0 < cols; c0 += 32) {
+    tc_ld16_issue(tcol + c0, v);
+    tc_ld_wait(v);
+    exp_chunk<true>(v, sc2, lse + 4u * c0, s0, s1);
+    tc_ld16_issue(tcol + c0 + 16, v);
+    tc_ld_wait(v);
+    exp_chunk<false>(v, sc2, lse + 4u * c0 + 64u, s0, s1);
+  }
+  return sum2(s0, s1);
 }
 
 }  // namespace

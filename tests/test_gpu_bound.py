@@ -1,0 +1,126 @@
+"""GPU: lists whose pooled scores nobody asks for take one product with every key and exact votes for the keys that may be kept
+(slkv_bound.cu); the same list with pooled scores takes the votes of all keys.  What is kept is the same bit for bit, whatever the
+sizes, strides, budgets and values: estimates that bound nothing, ties, scores beyond fp32's range, values that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2508_15806_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+LONG = 66000            # a sequence that sends a list this way, whatever else is in it
+
+
+def inputs(kind, seed, lens, hq, hkv, d, w):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    T, n, G = sum(lens), len(lens), hq // hkv
+    q = torch.randn(n, w, hq, d, generator=g, device=DEV)
+    k = torch.randn(T, hkv, d, generator=g, device=DEV)
+    v = torch.randn(T, hkv, d, generator=g, device=DEV).bfloat16()
+    if kind == "stripes":                                # keys that all rows look at, and some rows' own
+        u = torch.randn(1, hkv, d, generator=g, device=DEV)
+        u = u / u.norm(dim=2, keepdim=True)
+        q = q + 4.0 * u.repeat_interleave(G, dim=1)
+        amp = 1.5 * torch.randn(T, hkv, 1, generator=g, device=DEV)
+        amp[torch.randint(0, T, (1 + T // 500,), generator=g, device=DEV)] += 8.0
+        k = k + amp * u * (d ** 0.5 / 4.0)
+    elif kind == "ties":                                 # a few different keys, and many of each
+        k = k[torch.randint(0, 5, (T,), generator=g, device=DEV)]
+    elif kind == "same":
+        k = k[:1].expand(T, hkv, d).clone()
+    elif kind == "late":                                 # the rows' mass lies in one key, behind all samples, a key for each row
+        k[T - w - 3] *= 6.0
+        k[T // 2] *= 8.0
+    elif kind == "large":                                # scores of +- 1000 and more
+        q, k = 30.0 * q, 10.0 * k
+    elif kind == "small":                                # every score near -200: sums below fp32's range
+        q = torch.ones_like(q) + 0.01 * q
+        k = -200.0 / d ** 0.5 + 0.3 * k
+    elif kind == "cancel":                               # small differences of large products
+        q[..., ::2] += 40.0
+        q[..., 1::2] -= 40.0
+        k[..., ::2] += 20.0
+        k[..., 1::2] += 20.0
+    elif kind == "not finite":
+        k[T // 3, 0, 0] = float("inf")
+        k[T // 5, hkv - 1, 1] = float("nan")
+        q[0, 0, 0, 0] = float("nan")
+    return q.bfloat16(), k.bfloat16(), v
+
+
+def both_ways(layers, lens, w, pool, budgets, **kw):
+    """The list without and with pooled scores."""
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    p = B.make_params(*layers[0], w, pool, **kw)
+    hkv, d = layers[0][1].shape[1:]
+    cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.slkv_workspace_bytes_overlapped(p, cu), dtype=torch.uint8, device=DEV)
+    got = []
+    for pooled in (False, True):
+        ws.fill_(0x5a)
+        outs = []
+        for (q, k, v), bud in zip(layers, budgets):
+            cap = sum(min(n, max(int(b), w)) for n in lens for b in bud)
+            b = torch.tensor(bud, dtype=torch.int32, device=DEV)
+            o = [torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV), torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV),
+                 torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.full((cap,), -1, dtype=torch.int32, device=DEV),
+                 torch.zeros(1, dtype=torch.int32, device=DEV)]
+            scores = torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) if pooled else None
+            B.slkv_compress_overlapped(p, q, k, v, cu_dev, cu, b, *o[:4], ws, scores, o[4])
+            outs.append(o + [b, scores])                 # the calls are queued: what they use stays
+        B.slkv_join()
+        torch.cuda.synchronize()
+        got.append(outs)
+    for one, all_votes in zip(*got):
+        assert int(one[4]) == 0 and int(all_votes[4]) == 0
+        assert torch.equal(one[2], all_votes[2])
+        assert torch.equal(one[3], all_votes[3])
+        for i in (0, 1):
+            assert torch.equal(one[i].view(torch.int16), all_votes[i].view(torch.int16))
+
+
+KINDS = ["gaussian", "stripes", "ties", "same", "late", "large", "small", "cancel", "not finite"]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("hq,hkv,d,w,lens", [(8, 2, 128, 32, [4000, LONG]), (8, 4, 64, 64, [700, 33, 2500, 2 * LONG]), (16, 2, 128, 20, [33001]),
+                                             (8, 1, 64, 31, [LONG, 300])])
+def test_what_is_kept_is_what_all_votes_keep(kind, hq, hkv, d, w, lens):
+    layers = [inputs(kind, 31 * l + w, lens, hq, hkv, d, w) for l in range(3)]
+    budgets = [[w + x for x in (0, 1, 9, 100)][:hkv] if hkv > 2 else [w + 3 ** (l + 2), w + 11 * (l + 1)][:hkv] for l in range(3)]
+    both_ways(layers, lens, w, 7, budgets)
+
+
+@pytest.mark.parametrize("hq,hkv,d,w", [(3, 1, 128, 22), (8, 1, 64, 9), (2, 1, 64, 64), (8, 2, 128, 33), (3, 1, 128, 85), (8, 2, 128, 64)])
+@pytest.mark.parametrize("n", [1, 15, 16, 127, 128, 129, 2047, 2049, 4097, 8195, 16390])
+def test_rows_and_tile_edges(hq, hkv, d, w, n):
+    layers = [inputs("stripes", n + l, [LONG, n + w], hq, hkv, d, w) for l in range(2)]
+    both_ways(layers, [LONG, n + w], w, 5, [[w + max(1, n // 40)] * hkv, [w + 1] * hkv])
+
+
+@pytest.mark.parametrize("pool", [1, 3, 5, 9])
+@pytest.mark.parametrize("share", [0.0, 0.001, 0.0158, 0.016, 0.1, 0.3, 0.97, 1.0])
+def test_budgets_around_the_line_to_all_votes(pool, share):
+    w, n, hkv = 32, 32100, 4
+    layers = [inputs("stripes", l, [n + w], 16, hkv, 128, w) for l in range(3)]
+    k = int(share * n)
+    both_ways(layers, [n + w], w, pool, [[w + k, w + 20, w + k + 1, w - 5], [w + 7] * 4, [w + k] * 4])
+
+
+def test_all_causal_domain_and_strides():
+    w, n, hq, hkv, d = 24, 33003, 8, 2, 128
+    layers = []
+    for l in range(3):
+        q, k, v = inputs("stripes", l, [n + w], hq, hkv, d, w)
+        fused = torch.cat([k, v], dim=1).contiguous()              # K and V slices of one buffer, heads outside tokens for q
+        layers.append((q.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3), fused[:, :hkv], fused[:, hkv:]))
+    both_ways(layers, [n + w], w, 7, [[w + 60, w + 5]] * 3, softmax_domain=B.SLKV_ALL_CAUSAL)
+
+
+@pytest.mark.parametrize("lens,w", [([131072], 64), ([40000, 100, 262000], 17)])
+def test_segments_of_several_ctas(lens, w):
+    layers = [inputs("stripes", l, lens, 8, 2, 128, w) for l in range(2)]
+    both_ways(layers, lens, w, 7, [[w + 300, w + 2], [w + 1500, w + 9000]])
