@@ -505,8 +505,7 @@ struct Variant {
 #define SLKV_SEL(T, IT, C) \
   {T, IT, {k_select_bound<T, IT, 0, C>, k_select_bound<T, IT, 1, C>, k_select_bound<T, IT, 2, C>, k_select_bound<T, IT, 3, C>, k_select_bound<T, IT, 4, C>}}
 const Variant kVariants[] = {SLKV_SEL(512, 8, false), SLKV_SEL(512, 16, false), SLKV_SEL(1024, 16, false), SLKV_SEL(1024, 32, false),
-                             SLKV_SEL(1024, 32, true),
-                             SLKV_SEL(512, 16, true)};
+                             SLKV_SEL(1024, 32, true)};
 #undef SLKV_SEL
 
 size_t select_bytes(const ScoreShape& sh, const Variant& v, int k_tiles) {
@@ -519,15 +518,16 @@ size_t select_bytes(const ScoreShape& sh, const Variant& v, int k_tiles) {
 }  // namespace
 
 // Where the second product is worth more than the longer selection.  32 layers (16 above 40000 tokens), us, two products / one:
-//   128 rows     one sequence of 24000 567 / 574, 32768 839 / 750, 60000 867 / 836, 120000 1594 / 1332; four of 12000-24000 851 / 1238
-//   256 rows     one sequence of 12000 497 / 583, 20000 795 / 867, 131072 5775 / 3859; four of 8000-16000 1009 / 890, eight of
-//                4096-32768 6613 / 5411
-//   64 rows      one sequence of 20000 428 / 519
+//   128 rows     one sequence of 8192 203 / 233, 12000 298 / 284, 16384 376 / 327, 24000 567 / 490, 32768 840 / 690, 60000 867 / 685,
+//                120000 1594 / 1226; four of 8250-16500 610 / 635, 12000-24000 851 / 766
+//   256 rows     one sequence of 12000 497 / 526, 20000 795 / 833, 131072 5761 / 3877; four of 8000-16000 1009 / 869, eight of
+//                4096-32768 6614 / 5099
+//   64 rows      one sequence of 20000 428 / 446
 bool bound_list_supported(const Problem& pb) {
   if (pb.p.pool_mode != SLKV_POOL_MAX || !select_list_supported(pb) || pb.R <= 64) return false;
   if ((int64_t)pb.n_seg * tensor_slot_stride(pb) * pb.R >= (1ll << 31)) return false;        // places of the weights: 32-bit
   const int64_t mean = pb.total_hist / pb.p.n_seqs;
-  return mean >= 32000 || (pb.R > 128 && mean >= 12000 && pb.n_tiles128 >= 3000);
+  return mean >= 32000 || (pb.R > 128 ? mean >= 12000 && pb.n_tiles128 >= 3000 : mean >= 16000);
 }
 
 cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const ScoreLayer* lay, const TailLayer* tail, int n_layers,
@@ -538,11 +538,11 @@ cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const Sco
   for (int i = 0; i < n_layers; ++i) { a.lay[i] = lay[i]; a.lay[i].budgets = tail[i].budgets; a.tail[i] = tail[i]; }
   a.k_stride_tok = pb.p.k_stride_tok;
   a.k_stride_head = pb.p.k_stride_head;
-  int cs = select_list_cluster(pb);
-  const bool small = sh.MT == 1 && pb.max_hist > 8192 && pb.max_hist <= 65536 - 32;
-  if (small) cs = pb.max_hist <= 16384 - 8 ? 2 : pb.max_hist <= 32768 - 16 ? 4 : 8;
+  // One CTA per segment wherever it can hold the segment: in a cluster of four with 512 threads each the two searches for a k-th
+  // largest took 10 and 16 us instead of 3 and 8.
+  const int cs = select_list_cluster(pb);
   const int slice = ((pb.max_hist + 3 + cs - 1) / cs + 3) & ~3;
-  const Variant& var = kVariants[small ? 5 : cs > 1 ? 4 : slice <= 4096 ? 0 : slice <= 8192 ? 1 : slice <= 16384 ? 2 : 3];
+  const Variant& var = kVariants[cs > 1 ? 4 : slice <= 4096 ? 0 : slice <= 8192 ? 1 : slice <= 16384 ? 2 : 3];
   constexpr size_t kStatic = sizeof(SelShared) + sizeof(BoundShared) + 1024;
   const size_t room = var.threads == 512 ? 113 * 1024 - kStatic : kSmemLimit - kStatic;       // two CTAs to an SM
   // two tiles of keys at a time where shared memory and, of two CTAs, TMEM hold them
