@@ -44,9 +44,11 @@ constexpr float kSlack = 1.02f;
 // The first threshold: where T is expected, at the rows' mean error, and a little lower.
 constexpr float kMargin = 0.8f, kFewMargin = 0.45f;
 constexpr int kFew = 64;                     // up to this many positions the lower one: a second round costs more than some keys
-constexpr float kTinyScore = 0x1p-90f;       // a threshold below this proves nothing: the smallest exponentials are 2^-125
 // Logarithms (base 2) of sums, and of errors, with which the bounds hold: see bound_run.
-constexpr float kLowLog = -60.f, kHighLog = 110.f, kMaxError = 60.f;
+constexpr float kLowLog = -48.f, kHighLog = 110.f, kMaxError = 60.f;
+// A threshold below this proves nothing: an estimate takes scores below 2^-126 for zero, which in the vote are up to 2^(-126 - kLowLog)
+// of a row each, 2^-70 over 256 rows.  That is a thousandth of this, well within kSlack; the first threshold lies above 2^-54.
+constexpr float kTinyScore = 0x1p-60f;
 
 struct alignas(16) BoundShared {
   unsigned long long q_full, mma_done;

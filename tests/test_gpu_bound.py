@@ -124,3 +124,23 @@ def test_all_causal_domain_and_strides():
 def test_segments_of_several_ctas(lens, w):
     layers = [inputs("stripes", l, lens, 8, 2, 128, w) for l in range(2)]
     both_ways(layers, lens, w, 7, [[w + 300, w + 2], [w + 1500, w + 9000]])
+
+
+@pytest.mark.parametrize("n", [33000, 66000])           # a CTA per segment, a cluster
+@pytest.mark.parametrize("stripe,rest", [(-59, -90), (-53, -90), (-47, -90), (-53, -74), (-47, -66)])
+def test_keys_whose_exponentials_are_below_fp32(n, stripe, rest):
+    """Rows whose every score is so low that a key's exponential is zero in fp32 though its share of the row is not (2^-126 and
+    2^-75 and the like), and one row that makes the threshold lower still.  Queries along two axes: scores of 1.02 k (log2)."""
+    w, hq, hkv, d = 32, 8, 2, 128
+    q, k = torch.zeros(1, w, hq, d, device=DEV), torch.zeros(n + w, hkv, d, device=DEV)
+    q[..., 0] = 8.0
+    q[0, 5, 1, 0], q[0, 5, 1, 1] = 0.0, 8.0                       # one row of the first segment looks along the other axis
+    k[..., 0], k[..., 1] = -137.0, rest
+    k[::128, :, 0], k[::128, :, 1] = stripe, stripe + 2
+    k[n // 3 + 5, :, 1] = -10.0
+    low = 2 * n // 3 + 9
+    k[low, :, 0], k[low, :, 1] = -124.0, -137.0
+    v = torch.randn(n + w, hkv, d, device=DEV).bfloat16()
+    k = k.bfloat16()
+    keep = n // 128 + 44
+    both_ways([(q.bfloat16(), k, v)] * 2, [n + w], w, 1, [[w + keep, w + 3], [w + 5, w + keep]])
