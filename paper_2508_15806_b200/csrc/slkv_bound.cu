@@ -57,6 +57,7 @@ struct alignas(16) BoundShared {
   alignas(16) float lse[256];                // negated
   float half[2][128];
   float mid[2 * kMaxSplit], reach[2 * kMaxSplit];      // per run and set of weights: expected vote and bound, over the estimate
+  float beside[8];                           // exact votes of the four places on either side of a cluster's slice
 };
 
 template <int T, int IT, int RAD, bool CLUSTER>
@@ -312,6 +313,7 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
     if (!every && safe && b.bin > 0) bound = __uint_as_float(kEstFloor + ((unsigned)(b.bin - 1) << kEstShift)) * (k_keep <= kFew ? kFewMargin : kMargin);
 
     unsigned done = every ? valid : 0, halo_done = 0, kept = 0;
+    float beside = 0.f;                                  // warp 0, a lane each: the bounds of the places beside the slice
     int o_mine = 0, n_mma = 0, n_q = 0;
     for (int round = 0;; ++round) {
       // ---- the places that get their exact vote now; in a cluster also the four on either side of the slice, for the pooling
@@ -344,7 +346,8 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
         bool hit = lane < 8 && own > 0 && (lane < 4 ? rank > 0 : p < n);
         if (hit && bound > 0.f && !(halo_done >> lane & 1u)) {
           const int c = run_of(p);
-          hit = !((round == 0 ? votes[at(place)] / b.mid[c] : __ldcg(vote + p)) * b.reach[c] < bound);
+          if (round == 0) beside = votes[at(place)] * (b.reach[c] / b.mid[c]);
+          hit = !(beside < bound);
         }
         halo = __ballot_sync(kAll, hit);
         if (every) halo_done = halo;
@@ -437,7 +440,9 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
           const int key = i * batch + kt * kTileKeys + (tid & 127);
           if (unit < units && mt == MT - 1 && key < min(total, (i + 1) * batch)) {
             if (MT == 2) acc += b.half[kt][tid & 127];
-            __stcg(vote + base + (int)list[key] - 4, acc * inv_g);
+            const int place = (int)list[key] - 4;
+            if (CLUSTER && (place < 0 || place >= own)) b.beside[place < 0 ? place + 4 : place - own + 4] = acc * inv_g;
+            else __stcg(vote + base + place, acc * inv_g);
           }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -461,7 +466,7 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
       __syncthreads();
       if (wid == 0 && lane < 8) {
         const int place = lane < 4 ? lane - 4 : own + lane - 4;
-        votes[at(place)] = CLUSTER && (halo_done >> lane & 1u) ? __ldcg(vote + base + place) : 0.f;
+        votes[at(place)] = CLUSTER && (halo_done >> lane & 1u) ? (every ? __ldcg(vote + base + place) : b.beside[lane]) : 0.f;
       }
       __syncthreads();
       unsigned key[IT], tau;

@@ -144,3 +144,30 @@ def test_keys_whose_exponentials_are_below_fp32(n, stripe, rest):
     k = k.bfloat16()
     keep = n // 128 + 44
     both_ways([(q.bfloat16(), k, v)] * 2, [n + w], w, 1, [[w + keep, w + 3], [w + 5, w + keep]])
+
+
+@pytest.mark.parametrize("n,hkv", [(40001, 4), (70003, 2), (131000, 2), (262002, 1)])          # clusters of 2, 4, 4 and 8
+def test_borders_between_the_ctas_of_a_cluster_in_a_second_round(n, hkv):
+    """The weightiest key is one that few CTAs saw when they weighed their rows: thresholds come out too high, and are taken again
+    from the votes.  Around every border between slices lie keys on either side of the line."""
+    w, d, hq = 32, 128, 4 * hkv
+    layers = []
+    for l in range(2):
+        q, k, v = inputs("stripes", 7 * l + n % 5, [n + w], hq, hkv, d, w)
+        g = torch.Generator(device=DEV).manual_seed(n + l)
+        u = q[0, 0, ::4].float()
+        u = u / u.norm(dim=1, keepdim=True)
+        cs = 2
+        while (n + 3 + cs - 1) // cs + 3 > 32768:
+            cs *= 2
+        for h in range(hkv):
+            shift = h * n & 3
+            slice_ = ((n + shift + cs - 1) // cs + 3) & ~3
+            for rank in range(1, cs):
+                p = rank * slice_ - shift + torch.arange(-6, 6, device=DEV)
+                amp = 4.0 + 4.0 * torch.rand(12, 1, generator=g, device=DEV)
+                k[p, h] = (0.3 * torch.randn(12, d, generator=g, device=DEV) + amp * u[h] * (d ** 0.5 / 4.0)).bfloat16()
+            k[n // 2 + 11, h] = (16.0 * u[h] * (d ** 0.5 / 4.0)).bfloat16()
+        layers.append((q, k, v))
+    for pool in (3, 7):
+        both_ways(layers, [n + w], w, pool, [[w + 40 + 90 * h for h in range(hkv)], [w + 400 - 30 * h for h in range(hkv)]])
