@@ -147,9 +147,9 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
   const bool every = every_vote(len, budget, window);   // votes, not estimates
   // ---- the rows' log-sum-exps
   const StatView st = stat_view(L.part, n_seg, R, shp.slot_stride);
+  bool far_off = false;                                  // a row with which the bounds do not hold
   if (tid < 256) {
     float l2 = INFINITY;
-    bool bad = false;
     if (tid < R && choose) {
       const size_t row = (size_t)seg * R + tid;
       bool far = false;
@@ -157,14 +157,13 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
       const bool win = L.lse.win_m != nullptr;
       l2 = row_lse(st, __ldcg(st.acc + row), far, seg, tid, R, shp.slot_stride, min(shp.slot_stride, kMaxSplit), win,
                    win ? L.lse.win_m[row] : 0.f, win ? L.lse.win_z[row] : 0.f);
-      bad = far || !(l2 >= kLowLog && l2 <= kHighLog);
+      far_off = far || !(l2 >= kLowLog && l2 <= kHighLog);
     }
     b.lse[tid] = -l2;
-    if (bad) b.bad = 1;
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   tc_fence_before();
-  __syncthreads();
+  const bool rows_off = __syncthreads_or(far_off) != 0;
   tc_fence_after();
   pdl_launch_dependents();
   const uint32_t tmem = b.tmem;
@@ -228,7 +227,7 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
       }
       __syncthreads();
     }
-    const bool safe_rows = b.bad == 0;
+    const bool safe_rows = !rows_off && b.bad == 0;
     auto run_of = [&](int p) {
       const int tile = p >> 7, c = runs.slot(tile), count = runs.count(c), t = tile - runs.begin(c);
       const int nth = MT == 1 ? Spread<1>(count).tile(t) : Spread<2>(count).tile(t);       // its own inverse
