@@ -463,9 +463,11 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
         votes[tid * kPitch + e] = __ldcg(vote + base + i0 + e);
       }
       __syncthreads();
-      if (wid == 0 && lane < 8) {
-        const int place = lane < 4 ? lane - 4 : own + lane - 4;
-        votes[at(place)] = CLUSTER && (halo_done >> lane & 1u) ? (every ? __ldcg(vote + base + place) : b.beside[lane]) : 0.f;
+      // Outside the segment minus infinity, as in k_select_list: it differs from zero where votes are not finite.
+      if (wid == 0 && lane < 11) {
+        const int place = lane < 4 ? lane - 4 : (lane < 8 ? own + lane - 4 : lane - 8), p = base + place;
+        if (p < 0 || p >= n) votes[at(place)] = -INFINITY;
+        else if (lane < 8) votes[at(place)] = CLUSTER && (halo_done >> lane & 1u) ? (every ? __ldcg(vote + p) : b.beside[lane]) : 0.f;
       }
       __syncthreads();
       unsigned key[IT], tau;

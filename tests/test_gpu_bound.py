@@ -171,3 +171,19 @@ def test_borders_between_the_ctas_of_a_cluster_in_a_second_round(n, hkv):
         layers.append((q, k, v))
     for pool in (3, 7):
         both_ways(layers, [n + w], w, pool, [[w + 40 + 90 * h for h in range(hkv)], [w + 400 - 30 * h for h in range(hkv)]])
+
+
+@pytest.mark.parametrize("rows", ["one row", "a segment", "all"])
+@pytest.mark.parametrize("n", [33001, 66003])
+def test_votes_that_are_not_finite(rows, n):
+    """Query rows that are not finite: every vote of the segment is not, and the edges decide what is kept."""
+    w, hq, hkv, d = 32, 8, 2, 128
+    layers = [inputs("stripes", l, [n + w, 700], hq, hkv, d, w) for l in range(2)]
+    for q, _, _ in layers:
+        if rows == "one row":
+            q[0, w - 1, hq - 1, 0] = float("nan")
+        elif rows == "a segment":
+            q[0, :, :hq // hkv, 3] = float("nan")
+        else:
+            q[:] = float("inf")
+    both_ways(layers, [n + w, 700], w, 7, [[w + 60, w + 5], [w + 3, w + 2000]])
