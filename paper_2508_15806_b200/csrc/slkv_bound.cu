@@ -150,7 +150,7 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
   bool far_off = false;                                  // a row with which the bounds do not hold
   if (tid < 256) {
     float l2 = INFINITY;
-    if (tid < R && choose) {
+    if (tid < R && choose && !every) {
       const size_t row = (size_t)seg * R + tid;
       bool far = false;
       for (int w = 0; w < kFarWords; ++w) far |= __ldcg(st.far + (size_t)seg * kFarWords + w) != 0;
@@ -253,6 +253,8 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
     if (mine) {
       const int p0 = base + i0, v_lo = max(-p0, 0), v_hi = min(my_end - p0, IT);
       valid = (v_hi >= 32 ? kAll : (1u << max(v_hi, 0)) - 1u) & (v_lo >= 32 ? 0u : kAll << v_lo);
+    }
+    if (mine && !every) {
       unsigned key[IT];
       pool_places<RAD>(votes + tid * kPitch, votes + at(i0 - 4), true, key);
       int bin = kBins, run = 0;
@@ -271,10 +273,10 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
       atomicAdd(&sh.hist[bin], run);
       if (bad) atomicAdd(&sh.hist[kBins + 1], 1);
     }
-    if (tid == 0) b.bin = 0;
-    sync_all();
-    bool safe;
-    {
+    bool safe = false;
+    if (!every) {
+      if (tid == 0) b.bin = 0;
+      sync_all();
       int c[kPer], sum = 0, bad = sh.hist[kBins + 1];
 #pragma unroll
       for (int i = 0; i < kPer; ++i) c[i] = sh.hist[tid * kPer + i];
@@ -309,165 +311,166 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
       sync_all();                                        // nobody reads the others' bins any more
     }
     float bound = 0.f;                                   // a key whose vote may be this large gets it
-    if (!every && safe && b.bin > 0) bound = __uint_as_float(kEstFloor + ((unsigned)(b.bin - 1) << kEstShift)) * (k_keep <= kFew ? kFewMargin : kMargin);
+    if (safe && b.bin > 0) bound = __uint_as_float(kEstFloor + ((unsigned)(b.bin - 1) << kEstShift)) * (k_keep <= kFew ? kFewMargin : kMargin);
 
-    unsigned done = every ? valid : 0, halo_done = 0, kept = 0;
+    unsigned done = 0, halo_done = 0, kept = 0;
     float beside = 0.f;                                  // warp 0, a lane each: the bounds of the places beside the slice
     int o_mine = 0, n_mma = 0, n_q = 0;
     for (int round = 0;; ++round) {
-      // ---- the places that get their exact vote now; in a cluster also the four on either side of the slice, for the pooling
-      unsigned want = valid, halo = 0;
-      if (bound > 0.f && mine) {
-        // from the expected vote, later from the estimate itself, to the bound
-        const float f_a = round == 0 ? b.reach[run_a] / b.mid[run_a] : b.reach[run_a], f_b = round == 0 ? b.reach[run_b] / b.mid[run_b] : b.reach[run_b];
-        want = 0;
+      if (!every) {
+        // ---- the places that get their exact vote now; in a cluster also the four on either side of the slice, for the pooling
+        unsigned want = valid, halo = 0;
+        if (bound > 0.f && mine) {
+          // from the expected vote, later from the estimate itself, to the bound
+          const float f_a = round == 0 ? b.reach[run_a] / b.mid[run_a] : b.reach[run_a], f_b = round == 0 ? b.reach[run_b] / b.mid[run_b] : b.reach[run_b];
+          want = 0;
 #pragma unroll 2
-        for (int e = 0; e < IT; e += 4) {
-          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (round == 0) {
-            x = *reinterpret_cast<const float4*>(votes + tid * kPitch + e);
-          } else if ((valid >> e & 15u) == 15u) {
-            x = __ldcg(reinterpret_cast<const float4*>(vote + base + i0 + e));
-          } else {
-            const float* f = vote + base + i0 + e;
-            if (valid >> e & 1u) x.x = __ldcg(f);
-            if (valid >> e & 2u) x.y = __ldcg(f + 1);
-            if (valid >> e & 4u) x.z = __ldcg(f + 2);
-            if (valid >> e & 8u) x.w = __ldcg(f + 3);
+          for (int e = 0; e < IT; e += 4) {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (round == 0) {
+              x = *reinterpret_cast<const float4*>(votes + tid * kPitch + e);
+            } else if ((valid >> e & 15u) == 15u) {
+              x = __ldcg(reinterpret_cast<const float4*>(vote + base + i0 + e));
+            } else {
+              const float* f = vote + base + i0 + e;
+              if (valid >> e & 1u) x.x = __ldcg(f);
+              if (valid >> e & 2u) x.y = __ldcg(f + 1);
+              if (valid >> e & 4u) x.z = __ldcg(f + 2);
+              if (valid >> e & 8u) x.w = __ldcg(f + 3);
+            }
+            want |= (!(x.x * (e < cut ? f_a : f_b) < bound) ? 1u : 0u) << e | (!(x.y * (e + 1 < cut ? f_a : f_b) < bound) ? 2u : 0u) << e |
+                    (!(x.z * (e + 2 < cut ? f_a : f_b) < bound) ? 4u : 0u) << e | (!(x.w * (e + 3 < cut ? f_a : f_b) < bound) ? 8u : 0u) << e;
           }
-          want |= (!(x.x * (e < cut ? f_a : f_b) < bound) ? 1u : 0u) << e | (!(x.y * (e + 1 < cut ? f_a : f_b) < bound) ? 2u : 0u) << e |
-                  (!(x.z * (e + 2 < cut ? f_a : f_b) < bound) ? 4u : 0u) << e | (!(x.w * (e + 3 < cut ? f_a : f_b) < bound) ? 8u : 0u) << e;
+          want = (want & valid) | done;
         }
-        want = (want & valid) | done;
-      }
-      if (CLUSTER && wid == 0) {
-        const int place = lane < 4 ? lane - 4 : own + lane - 4, p = base + place;
-        bool hit = lane < 8 && own > 0 && (lane < 4 ? rank > 0 : p < n);
-        if (hit && bound > 0.f && !(halo_done >> lane & 1u)) {
-          const int c = run_of(p);
-          if (round == 0) beside = votes[at(place)] * (b.reach[c] / b.mid[c]);
-          hit = !(beside < bound);
+        if (CLUSTER && wid == 0) {
+          const int place = lane < 4 ? lane - 4 : own + lane - 4, p = base + place;
+          bool hit = lane < 8 && own > 0 && (lane < 4 ? rank > 0 : p < n);
+          if (hit && bound > 0.f && !(halo_done >> lane & 1u)) {
+            const int c = run_of(p);
+            if (round == 0) beside = votes[at(place)] * (b.reach[c] / b.mid[c]);
+            hit = !(beside < bound);
+          }
+          halo = __ballot_sync(kAll, hit);
         }
-        halo = __ballot_sync(kAll, hit);
-        if (every) halo_done = halo;
-      }
-      const unsigned fresh = want & ~done;
-      int inc = __popc(fresh);
+        const unsigned fresh = want & ~done;
+        int inc = __popc(fresh);
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(kAll, inc, o);
-        if (lane >= o) inc += x;
-      }
-      if (lane == 31) sh.wsum[2][wid] = (unsigned)inc;
-      __syncthreads();                                   // also: nobody reads the estimates any more
-      int o = (int)__reduce_add_sync(kAll, lane < wid ? sh.wsum[2][lane] : 0u) + inc - __popc(fresh);
-      int total = (int)__reduce_add_sync(kAll, lane < kWarps ? sh.wsum[2][lane] : 0u);
-      for (unsigned m = fresh; m != 0; m &= m - 1) list[o++] = (unsigned short)(i0 + __ffs(m) - 1 + 4);
-      if (CLUSTER && wid == 0) {
-        const unsigned now = halo & ~halo_done;
-        if (now >> lane & 1u)
-          list[total + __popc(now & ((1u << lane) - 1u))] = (unsigned short)((lane < 4 ? lane - 4 : own + lane - 4) + 4);
-        if (lane == 0) b.halo = (int)now;
-      }
-      // rows of the Q tile that TMA does not write
-      if (R != MT * 128)
-        for (int i = tid; i < q_bytes / 16; i += T) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncthreads();
-      if (CLUSTER) total += __popc(b.halo);
-      // ---- their votes, 128 keys at a time: as in the vote pass, key by key the same
-      if (total > 0) {
-        if (tid == 0) {
-          const uint32_t bar = smem_u32(&b.q_full);
-          mbar_expect_tx(bar, (uint32_t)(halves * R * 128));
-          for (int hf = 0; hf < halves; ++hf)
-            tma_load_4d(q_sh + hf * q_half, &L.tm_q, 64 * hf, shp.q_head_inner ? h * shp.G : 0, shp.q_head_inner ? 0 : h * shp.G, s, bar);
+        for (int o = 1; o < 32; o <<= 1) {
+          const int x = __shfl_up_sync(kAll, inc, o);
+          if (lane >= o) inc += x;
         }
-        const int per_row = 8 * halves, NB = args.k_tiles, batch = NB * kTileKeys, n_batches = (total + batch - 1) / batch;
-        const unsigned char* k_seg = static_cast<const unsigned char*>(a.k) + ((long long)(t0 + base - 4) * args.k_stride_tok + h * args.k_stride_head) * 2;
-        auto load = [&](int i) {
-          const int rows = min(total - i * batch, batch);
-          for (int x = tid; x < rows * per_row; x += T) {
-            const int r = halves == 2 ? x >> 4 : x >> 3, c = x & (per_row - 1);
-            const unsigned char* src = k_seg + (long long)list[i * batch + r] * args.k_stride_tok * 2 + c * 16;
-            const uint32_t dst = k_sh + (uint32_t)((r >> 7) * stage + (c >> 3) * kHalfBytes + (r & 127) * 128 + (((c & 7) ^ (r & 7)) << 4));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-          }
-        };
-        const float scale = shp.scale_log2;
-        const int Rp = shp.Rp, units = NB * MT;          // unit: a tile's rows of one block
-        load(0);
-        bool ok = true;
-        for (int i = 0; i < n_batches; ++i) {
-          asm volatile("cp.async.wait_all;" ::: "memory");
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncthreads();
-          const int tiles_here = (min(total - i * batch, batch) + kTileKeys - 1) / kTileKeys;
+        if (lane == 31) sh.wsum[2][wid] = (unsigned)inc;
+        __syncthreads();                                   // also: nobody reads the estimates any more
+        int o = (int)__reduce_add_sync(kAll, lane < wid ? sh.wsum[2][lane] : 0u) + inc - __popc(fresh);
+        int total = (int)__reduce_add_sync(kAll, lane < kWarps ? sh.wsum[2][lane] : 0u);
+        for (unsigned m = fresh; m != 0; m &= m - 1) list[o++] = (unsigned short)(i0 + __ffs(m) - 1 + 4);
+        if (CLUSTER && wid == 0) {
+          const unsigned now = halo & ~halo_done;
+          if (now >> lane & 1u)
+            list[total + __popc(now & ((1u << lane) - 1u))] = (unsigned short)((lane < 4 ? lane - 4 : own + lane - 4) + 4);
+          if (lane == 0) b.halo = (int)now;
+        }
+        // rows of the Q tile that TMA does not write
+        if (R != MT * 128)
+          for (int i = tid; i < q_bytes / 16; i += T) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (CLUSTER) total += __popc(b.halo);
+        // ---- their votes, 128 keys at a time: as in the vote pass, key by key the same
+        if (total > 0) {
           if (tid == 0) {
-            if (i == 0) ok = mbar_wait(smem_u32(&b.q_full), (uint32_t)n_q & 1u, &b.abort_flag);
-            if (ok) {
-              tc_fence_after();
-              for (int x = 0; x < tiles_here * MT; ++x) {
-                const int kt = x / MT, mt = x - kt * MT;
-                const uint32_t idesc = instr_desc(kTileKeys, min(Rp - mt * 128, 128));
-                const uint64_t kd = smem_desc(k_sh + (uint32_t)(kt * stage)), qd = smem_desc(q_sh + (uint32_t)(mt * 128 * 128));
-                for (int ks = 0; ks < 4 * halves; ++ks)
-                  tc_mma(tmem + (uint32_t)(x * 128), kd + (uint64_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2),
-                         qd + (uint64_t)((ks >> 2) * (q_half >> 4) + (ks & 3) * 2), idesc, ks > 0);
+            const uint32_t bar = smem_u32(&b.q_full);
+            mbar_expect_tx(bar, (uint32_t)(halves * R * 128));
+            for (int hf = 0; hf < halves; ++hf)
+              tma_load_4d(q_sh + hf * q_half, &L.tm_q, 64 * hf, shp.q_head_inner ? h * shp.G : 0, shp.q_head_inner ? 0 : h * shp.G, s, bar);
+          }
+          const int per_row = 8 * halves, NB = args.k_tiles, batch = NB * kTileKeys, n_batches = (total + batch - 1) / batch;
+          const unsigned char* k_seg = static_cast<const unsigned char*>(a.k) + ((long long)(t0 + base - 4) * args.k_stride_tok + h * args.k_stride_head) * 2;
+          auto load = [&](int i) {
+            const int rows = min(total - i * batch, batch);
+            for (int x = tid; x < rows * per_row; x += T) {
+              const int r = halves == 2 ? x >> 4 : x >> 3, c = x & (per_row - 1);
+              const unsigned char* src = k_seg + (long long)list[i * batch + r] * args.k_stride_tok * 2 + c * 16;
+              const uint32_t dst = k_sh + (uint32_t)((r >> 7) * stage + (c >> 3) * kHalfBytes + (r & 127) * 128 + (((c & 7) ^ (r & 7)) << 4));
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+            }
+          };
+          const float scale = shp.scale_log2;
+          const int Rp = shp.Rp, units = NB * MT;          // unit: a tile's rows of one block
+          load(0);
+          bool ok = true;
+          for (int i = 0; i < n_batches; ++i) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            const int tiles_here = (min(total - i * batch, batch) + kTileKeys - 1) / kTileKeys;
+            if (tid == 0) {
+              if (i == 0) ok = mbar_wait(smem_u32(&b.q_full), (uint32_t)n_q & 1u, &b.abort_flag);
+              if (ok) {
+                tc_fence_after();
+                for (int x = 0; x < tiles_here * MT; ++x) {
+                  const int kt = x / MT, mt = x - kt * MT;
+                  const uint32_t idesc = instr_desc(kTileKeys, min(Rp - mt * 128, 128));
+                  const uint64_t kd = smem_desc(k_sh + (uint32_t)(kt * stage)), qd = smem_desc(q_sh + (uint32_t)(mt * 128 * 128));
+                  for (int ks = 0; ks < 4 * halves; ++ks)
+                    tc_mma(tmem + (uint32_t)(x * 128), kd + (uint64_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2),
+                           qd + (uint64_t)((ks >> 2) * (q_half >> 4) + (ks & 3) * 2), idesc, ks > 0);
+                }
+                tc_commit(smem_u32(&b.mma_done));
               }
-              tc_commit(smem_u32(&b.mma_done));
             }
-          }
-          __syncwarp();
-          ok = mbar_wait(smem_u32(&b.mma_done), (uint32_t)n_mma & 1u, &b.abort_flag);
-          ok = __all_sync(kAll, ok);
-          ++n_mma;
-          float acc = 0.f;
-          const int unit = wid >> 2, kt = unit / MT, mt = unit - kt * MT;
-          if (ok) {
-            if (i + 1 < n_batches) load(i + 1);          // the products have read the keys
+            __syncwarp();
+            ok = mbar_wait(smem_u32(&b.mma_done), (uint32_t)n_mma & 1u, &b.abort_flag);
+            ok = __all_sync(kAll, ok);
+            ++n_mma;
+            float acc = 0.f;
+            const int unit = wid >> 2, kt = unit / MT, mt = unit - kt * MT;
+            if (ok) {
+              if (i + 1 < n_batches) load(i + 1);          // the products have read the keys
+              tc_fence_after();
+              if (unit < units && kt < tiles_here) {
+                acc = key_vote(tmem + ((uint32_t)((wid & 3) * 32) << 16) + (uint32_t)(unit * 128), min(Rp - mt * 128, 128), scale, smem_u32(b.lse + mt * 128));
+                if (MT == 2 && mt == 0) b.half[kt][tid & 127] = acc;
+              }
+            }
+            tc_fence_before();
+            __syncthreads();
             tc_fence_after();
-            if (unit < units && kt < tiles_here) {
-              acc = key_vote(tmem + ((uint32_t)((wid & 3) * 32) << 16) + (uint32_t)(unit * 128), min(Rp - mt * 128, 128), scale, smem_u32(b.lse + mt * 128));
-              if (MT == 2 && mt == 0) b.half[kt][tid & 127] = acc;
+            if (b.abort_flag) break;                       // uniform: written before the barrier
+            const int key = i * batch + kt * kTileKeys + (tid & 127);
+            if (unit < units && mt == MT - 1 && key < min(total, (i + 1) * batch)) {
+              if (MT == 2) acc += b.half[kt][tid & 127];
+              const int place = (int)list[key] - 4;
+              if (CLUSTER && (place < 0 || place >= own)) b.beside[place < 0 ? place + 4 : place - own + 4] = acc * inv_g;
+              else __stcg(vote + base + place, acc * inv_g);
             }
           }
-          tc_fence_before();
-          __syncthreads();
-          tc_fence_after();
-          if (b.abort_flag) break;                       // uniform: written before the barrier
-          const int key = i * batch + kt * kTileKeys + (tid & 127);
-          if (unit < units && mt == MT - 1 && key < min(total, (i + 1) * batch)) {
-            if (MT == 2) acc += b.half[kt][tid & 127];
-            const int place = (int)list[key] - 4;
-            if (CLUSTER && (place < 0 || place >= own)) b.beside[place < 0 ? place + 4 : place - own + 4] = acc * inv_g;
-            else __stcg(vote + base + place, acc * inv_g);
+          asm volatile("cp.async.wait_all;" ::: "memory");
+          if (tid == 0 && b.abort_flag) {                  // a load in flight, for a bounded time
+            const unsigned long long w0 = now_ns();
+            while (!mbar_try(smem_u32(&b.q_full), (uint32_t)n_q & 1u) && now_ns() - w0 < kWaitLimitNs) {}
           }
+          ++n_q;
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        if (tid == 0 && b.abort_flag) {                  // a load in flight, for a bounded time
-          const unsigned long long w0 = now_ns();
-          while (!mbar_try(smem_u32(&b.q_full), (uint32_t)n_q & 1u) && now_ns() - w0 < kWaitLimitNs) {}
-        }
-        ++n_q;
-      }
-      done = want;
-      halo_done |= halo;
-      // ---- the votes that are there, none elsewhere; pooled, and the k largest
-      __syncthreads();
-      clear_bins();
+        done = want;
+        halo_done |= halo;
+        // ---- the votes that are there, none elsewhere; pooled, and the k largest
+        __syncthreads();
+        clear_bins();
 #pragma unroll
-      for (int e = 0; e < IT; e += 4) *reinterpret_cast<float4*>(votes + tid * kPitch + e) = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (unsigned m = done; m != 0; m &= m - 1) {
-        const int e = __ffs(m) - 1;
-        votes[tid * kPitch + e] = __ldcg(vote + base + i0 + e);
+        for (int e = 0; e < IT; e += 4) *reinterpret_cast<float4*>(votes + tid * kPitch + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (unsigned m = done; m != 0; m &= m - 1) {
+          const int e = __ffs(m) - 1;
+          votes[tid * kPitch + e] = __ldcg(vote + base + i0 + e);
+        }
       }
       __syncthreads();
       // Outside the segment minus infinity, as in k_select_list: it differs from zero where votes are not finite.
       if (wid == 0 && lane < 11) {
         const int place = lane < 4 ? lane - 4 : (lane < 8 ? own + lane - 4 : lane - 8), p = base + place;
         if (p < 0 || p >= n) votes[at(place)] = -INFINITY;
-        else if (lane < 8) votes[at(place)] = CLUSTER && (halo_done >> lane & 1u) ? (every ? __ldcg(vote + p) : b.beside[lane]) : 0.f;
+        else if (!every && lane < 8) votes[at(place)] = CLUSTER && (halo_done >> lane & 1u) ? b.beside[lane] : 0.f;
       }
       __syncthreads();
       unsigned key[IT], tau;

@@ -187,3 +187,15 @@ def test_votes_that_are_not_finite(rows, n):
         else:
             q[:] = float("inf")
     both_ways(layers, [n + w, 700], w, 7, [[w + 60, w + 5], [w + 3, w + 2000]])
+
+
+@pytest.mark.parametrize("hq,hkv,d,w,lens", [(16, 4, 128, 32, [LONG, 9000, 40, 33000, 1300, 20000, 128 + 32, 60001]), (16, 16, 64, 80, [LONG]),
+                                             (32, 8, 128, 32, [17000] * 3), (8, 2, 128, 64, [2 * LONG, 700]), (6, 1, 64, 40, [200000, 513 + 40])])
+@pytest.mark.parametrize("share", [0.1, 0.5, 0.9])
+def test_heads_that_need_all_votes_among_others(hq, hkv, d, w, lens, share):
+    """Any mixture of heads that keep few positions and many, in all layers and of sequences of any length."""
+    rng = np.random.default_rng(len(lens) * hq + int(10 * share))
+    n_layers = 8 if sum(lens) < 70000 else 5
+    layers = [inputs("stripes", l + w, lens, hq, hkv, d, w) for l in range(n_layers)]
+    budgets = [[int(w + (rng.integers(600, 6000) if rng.random() < share else rng.integers(0, 400))) for _ in range(hkv)] for _ in layers]
+    both_ways(layers, lens, w, 7, budgets)
