@@ -451,9 +451,17 @@ int slkv_trace_set_buffer(void* dev_buf, size_t bytes);
  * there are -- on = 1: where the CTAs of a score launch wait for the statistics, 2: for their clearing, 3: where those of a
  * one-launch layer wait for the row sums, 4: for the votes -- so that exactly this path runs: the call's results are then incomplete
  * and its status word says so; the calls after it are unaffected.  While it is armed with 1 or 2, short layers go the way of the
- * others.  One-shot: the launch that takes it disarms it.
+ * others; a list that goes with one product with every key (slkv_debug_list_way) waits for statistics only where some head needs all
+ * its votes.  One-shot: the launch that takes it disarms it.
  */
 int slkv_debug_expire_next_wait(int on);
+
+/*
+ * Test hook for lists of overlapped calls whose pooled scores nobody asks for (no counterpart in the paper).  Such a list goes with one
+ * product with every key or with two, which keep the same positions, by a rule on its size and its layers' capacities.  way = 1: lists
+ * that the calling thread sends out go with one product wherever the kernels take the shape, 2: with two, 0: by the rule.
+ */
+int slkv_debug_list_way(int way);
 
 /* Library version, major*10000 + minor*100 + patch. */
 int slkv_version(void);

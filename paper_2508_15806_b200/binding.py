@@ -89,6 +89,8 @@ def lib() -> C.CDLL:
         L.slkv_row_lse.argtypes = [pp, vp, vp, vp, i32p, vp, vp, vp, sz, vp]
         L.slkv_debug_expire_next_wait.restype = C.c_int
         L.slkv_debug_expire_next_wait.argtypes = [C.c_int]
+        L.slkv_debug_list_way.restype = C.c_int
+        L.slkv_debug_list_way.argtypes = [C.c_int]
         L.slkv_compress.restype = C.c_int
         L.slkv_compress.argtypes = [pp, vp, vp, vp, vp, i32p, vp, vp, vp, vp, i64, vp, vp, vp, vp, vp, sz, vp]
         L.slkv_compress_overlapped.restype = C.c_int
@@ -278,6 +280,11 @@ def slkv_debug_expire_next_wait(on=True) -> None:
     """False / 0: off; True / 1: the wait for the statistics; 2: the wait for their clearing; of a layer in one launch, 3: the wait
     for the row sums, 4: the wait for the votes."""
     lib().slkv_debug_expire_next_wait(int(on))
+
+
+def slkv_debug_list_way(way=0) -> None:
+    """Lists this thread sends out without pooled scores: 1 one product with every key, 2 two, 0 by the library's rule."""
+    lib().slkv_debug_list_way(int(way))
 
 
 def slkv_score_noalloc(params: SlkvParams, q_win: torch.Tensor, k: torch.Tensor, cu_dev: torch.Tensor,

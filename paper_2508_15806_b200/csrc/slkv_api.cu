@@ -290,7 +290,7 @@ cudaError_t flush_list(ListState* s, cudaStream_t owner, int* launches) {
   s->n = 0;
   s->in_flight = true;
   cudaError_t e;
-  bool bound = !s->with_lse && !next_wait_expires() && bound_list_supported(s->pb);
+  bool bound = !s->with_lse && bound_list_supported(s->pb, s->tail, n);
   for (int i = 0; i < n; ++i) bound = bound && s->tail[i].pooled_out == nullptr;
   if (bound) {
     e = launch_bound_list(s->pb, s->plan.sh, s->score, s->tail, n, owner, launches);
@@ -568,7 +568,7 @@ int take_expire_next_layer_wait(bool sums) {
 LaunchScope::LaunchScope(int kid, cudaStream_t st, int* launches) : kid_(kid), st_(st), slot_(-1) {
   ++*launches;
   if (!g_prof_on) return;
-  const bool score_kid = kid == KID_SCORE_LSE || kid == KID_SCORE_VOTE || kid == KID_SCORE_FUSED || kid == KID_SCORE_LIST;
+  const bool score_kid = kid == KID_SCORE_LSE || kid == KID_SCORE_VOTE || kid == KID_SCORE_FUSED || kid == KID_SCORE_LIST || kid == KID_SCORE_BOUND;
   if (g_prof_on == 2 && !score_kid) return;
   if (!g_prof) g_prof = new std::vector<TimedLaunch>();
   TimedLaunch t{kid, prof_event(), prof_event()};
@@ -631,7 +631,7 @@ int slkv_profile_collect(float* total_ms, int32_t* launches, int32_t n_kernels) 
 const char* slkv_kernel_name(int kernel_id) {
   static const char* names[KID_COUNT] = {"k_setup", "k_score_lse", "k_score_vote", "k_pool", "k_select",
                                          "k_gather", "k_alloc", "k_score_fused", "k_score_list", "k_window_stats",
-                                         "k_merge_lse", "k_behavior", "k_cp", "k_layer"};
+                                         "k_merge_lse", "k_behavior", "k_cp", "k_layer", "k_score_bound"};
   return (kernel_id >= 0 && kernel_id < KID_COUNT) ? names[kernel_id] : "";
 }
 
@@ -645,6 +645,11 @@ int slkv_trace_set_buffer(void* dev_buf, size_t bytes) {
 int slkv_last_cuda_error(void) { return g_last_cuda_error; }
 int slkv_last_launch_count(void) { return g_last_launches; }
 int slkv_version(void) { return 300; }
+
+int slkv_debug_list_way(int way) {
+  set_list_way(way == 1 || way == 2 ? way : 0);
+  return SLKV_OK;
+}
 
 int slkv_debug_expire_next_wait(int on) {
   const int layer = on == 3 || on == 4 ? on - 2 : 0;

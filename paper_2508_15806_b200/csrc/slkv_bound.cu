@@ -528,17 +528,45 @@ size_t select_bytes(const ScoreShape& sh, const Variant& v, int k_tiles) {
 
 }  // namespace
 
-// Where the second product is worth more than the longer selection.  32 layers (16 above 40000 tokens), us, two products / one:
-//   128 rows     one sequence of 8192 203 / 233, 12000 298 / 284, 16384 376 / 327, 24000 567 / 490, 32768 840 / 690, 60000 867 / 685,
-//                120000 1594 / 1226; four of 8250-16500 610 / 635, 12000-24000 851 / 766
-//   256 rows     one sequence of 12000 497 / 526, 20000 795 / 833, 131072 5761 / 3877; four of 8000-16000 1009 / 869, eight of
-//                4096-32768 6614 / 5099
-//   64 rows      one sequence of 20000 428 / 446
-bool bound_list_supported(const Problem& pb) {
-  if (pb.p.pool_mode != SLKV_POOL_MAX || !select_list_supported(pb) || pb.R <= 64) return false;
+namespace {
+thread_local int g_list_way = 0;
+}
+void set_list_way(int way) { g_list_way = way; }
+
+// Where the second product is worth more than the longer selection.  It saves some 3.5 ns for every product of 128 keys x 128 rows; the
+// selection takes 50-90 us longer whatever the list's length, for 256 rows twice that.  With it come the segments that need all their votes
+// (every_vote): both products, the second one from HBM.  The budgets are on the device, but what a layer keeps at most is known
+// here.  Were its budgets even, the share of its segments that need all votes would be 0 or 1, were they as uneven as can be, up to
+// `most`, here the mean over the layers.  Lists, us, two products / one, budgets lognormal with a standard deviation of 1.5:
+//   128 rows  16384 tokens, 20 layers (20480 products): most 0.4 235 / 221, 0.6 259 / 282;  28 (28672): 0.4 323 / 289, 0.6 357 / 360
+//             32768 tokens, 10 (20480): 0.3 227 / 233;  14 (28672): 0.3 310 / 272, 0.6 328 / 342;  16 (32768): 0.6 364 / 342, 0.75 375 / 371, 0.83 385 / 414
+//             65536 tokens, 5 (20480): 0.4 231 / 228, 0.7 252 / 267;  8 (32768): 0.73 385 / 375, 0.82 400 / 417
+//             131072 tokens, 8 (65520): 0.74 856 / 720, even 0.98 774 / 642, 1.00 809 / 867
+//             four of 12000 to 24000, 4 (18016): 0.3 205 / 216;  5 (22520): 0.3 256 / 238, 0.74 277 / 277;  8 (36032): 0.74 435 / 426, 0.83 461 / 468
+//   256 rows  33000 tokens, 5 (20640): 0.35 210 / 207;  7 (28896): 0.35 283 / 268, 0.7 293 / 304;  8 (33024): 0.54 318 / 301, 0.71 328 / 342
+//             in clusters of two, 45000 tokens, 5 (28160): 0.27 281 / 249, 0.74 288 / 294;  60000, 4 (30016): 0.4 295 / 305;  5 (37520): 0.4 361 / 328, 0.7 375 / 404;  48000 tokens, 8 (48000): 0.63 472 / 451,
+//             0.95 510 / 526;  65536 tokens, 8 (65536): 0.81 659 / 650, 0.88 667 / 692
+//             in clusters of four, 100000 tokens, 3 (37488): 0.25 363 / 377;  131072 tokens, 4 (65536): 611 / 521;  8 (131072): 0.67 1270 / 1261
+//             eight of 16384 to 32768, 8 (98304): 0.87 2124 / 1820
+//   64 rows   one sequence of 20000 tokens 428 / 446
+bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers) {
+  if (pb.p.pool_mode != SLKV_POOL_MAX || !select_list_supported(pb) || pb.R <= 64 || g_list_way == 2) return false;
   if ((int64_t)pb.n_seg * tensor_slot_stride(pb) * pb.R >= (1ll << 31)) return false;        // places of the weights: 32-bit
+  if (g_list_way == 1) return true;
   const int64_t mean = pb.total_hist / pb.p.n_seqs;
-  return mean >= 32000 || (pb.R > 128 ? mean >= 12000 && pb.n_tiles128 >= 3000 : mean >= 16000);
+  if (!(mean >= 32000 || (pb.R > 128 ? mean >= 12000 && pb.n_tiles128 >= 3000 : mean >= 16000))) return false;
+  const int64_t line = mean / kEveryVoteShare > kEveryVoteCount ? mean / kEveryVoteShare : kEveryVoteCount;
+  const int64_t window_rows = (int64_t)pb.p.n_kv_heads * (pb.total_tokens - pb.total_hist);
+  double most = 0.0;
+  for (int i = 0; i < n_layers; ++i) {
+    const double share = (double)(tail[i].capacity - window_rows) / (double)(line * pb.n_seg);
+    most += share < 1.0 ? (share > 0.0 ? share : 0.0) : 1.0;
+  }
+  most /= n_layers;
+  const double products = (double)pb.n_tiles128 * n_layers * (pb.R > 128 ? 2 : 1);
+  if (pb.R <= 128) return most < 0.99 && products >= 17000 + 16500 * most + (most > 0.78 ? 24000 : 0);
+  const double clusters = pb.max_hist < 32764 ? 0.0 : 10000 * (pb.max_hist / 32764.0 - 1.0);        // beyond what one CTA holds
+  return most < 0.96 && products >= 17000 + 24000 * most + (most > 0.85 ? 24000 : 0) + (clusters < 14000 ? clusters : 14000);
 }
 
 cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const ScoreLayer* lay, const TailLayer* tail, int n_layers,

@@ -131,7 +131,7 @@ struct Problem {
 };
 
 // kernel ids for launch accounting / per-kernel timing
-enum KernelId { KID_SETUP = 0, KID_SCORE_LSE, KID_SCORE_VOTE, KID_POOL, KID_SELECT, KID_GATHER, KID_ALLOC, KID_SCORE_FUSED, KID_SCORE_LIST, KID_WINDOW_STATS, KID_MERGE_LSE, KID_BEHAVIOR, KID_CP, KID_LAYER, KID_COUNT };
+enum KernelId { KID_SETUP = 0, KID_SCORE_LSE, KID_SCORE_VOTE, KID_POOL, KID_SELECT, KID_GATHER, KID_ALLOC, KID_SCORE_FUSED, KID_SCORE_LIST, KID_WINDOW_STATS, KID_MERGE_LSE, KID_BEHAVIOR, KID_CP, KID_LAYER, KID_SCORE_BOUND, KID_COUNT };
 
 // Brackets one kernel launch: counts it and, when per-kernel timing is on for this thread, records a
 // CUDA event pair around it on the launch stream.
@@ -290,7 +290,8 @@ __device__ __forceinline__ bool every_vote(int len, int budget, int window) {
 cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
                               unsigned long long* sync, cudaStream_t st, int* launches, bool cleared = false);
 // Scores and selection of a list in one product with every key (slkv_bound.cu).  cudaErrorNotSupported: nothing is launched.
-bool bound_list_supported(const Problem& pb);
+bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers);
+void set_list_way(int way);                       // of this thread: 0 by rule, 1 one product wherever it can be, 2 two
 cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const ScoreLayer* lay, const TailLayer* tail, int n_layers,
                               cudaStream_t st, int* launches);
 // lse_out null: into the layer's own statistics area

@@ -1014,7 +1014,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
     e = clear_stats(sh, lay, n_layers, st);
     if (e != cudaSuccess) return e;
   }
-  const int kid = passes == 1 ? KID_SCORE_LSE : (n_layers > 1 ? KID_SCORE_LIST : (passes == 2 ? KID_SCORE_VOTE : KID_SCORE_FUSED));
+  const int kid = bound ? KID_SCORE_BOUND : passes == 1 ? KID_SCORE_LSE : (n_layers > 1 ? KID_SCORE_LIST : (passes == 2 ? KID_SCORE_VOTE : KID_SCORE_FUSED));
   if (!waits_inside) return launch_pdl_scoped(kid, kernel, sh.n_cta, kListThreads, smem, st, launches, a);
   for (int attempt = 0; attempt < 2; ++attempt) {
     cudaLaunchConfig_t cfg = {};

@@ -6,12 +6,22 @@ import pytest
 import torch
 
 from paper_2508_15806_b200 import binding as B
+import parity as P
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
 
 
-LONG = 66000            # a sequence that sends a list this way, whatever else is in it
+@pytest.fixture(autouse=True)
+def hooks_off():
+    yield
+    B.slkv_debug_list_way(0)
+    B.slkv_debug_expire_next_wait(0)
+    B.slkv_profile_enable(0)
+    B.slkv_profile_collect()
+
+
+LONG = 66000            # a sequence whose segments are a cluster's
 
 
 def inputs(kind, seed, lens, hq, hkv, d, w):
@@ -51,28 +61,38 @@ def inputs(kind, seed, lens, hq, hkv, d, w):
     return q.bfloat16(), k.bfloat16(), v
 
 
-def both_ways(layers, lens, w, pool, budgets, **kw):
-    """The list without and with pooled scores."""
+def one_list(layers, lens, w, pool, budgets, way, pooled=False, **kw):
+    """The layers' outputs (k, v, offsets, kept positions, status), and the score kernel they took."""
     cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
     p = B.make_params(*layers[0], w, pool, **kw)
     hkv, d = layers[0][1].shape[1:]
     cu_dev = torch.tensor(cu, dtype=torch.int32, device=DEV)
-    ws = torch.empty(B.slkv_workspace_bytes_overlapped(p, cu), dtype=torch.uint8, device=DEV)
+    ws = torch.full((B.slkv_workspace_bytes_overlapped(p, cu),), 0x5a, dtype=torch.uint8, device=DEV)
+    outs = []
+    B.slkv_debug_list_way(way)
+    B.slkv_profile_enable(2)
+    for (q, k, v), bud in zip(layers, budgets):
+        cap = sum(min(n, max(int(b), w)) for n in lens for b in bud)
+        b = torch.tensor(bud, dtype=torch.int32, device=DEV)
+        o = [torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV), torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV),
+             torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.full((cap,), -1, dtype=torch.int32, device=DEV),
+             torch.zeros(1, dtype=torch.int32, device=DEV)]
+        scores = torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) if pooled else None
+        B.slkv_compress_overlapped(p, q, k, v, cu_dev, cu, b, *o[:4], ws, scores, o[4])
+        outs.append(o + [b, scores])                     # the calls are queued: what they use stays
+    B.slkv_join()
+    torch.cuda.synchronize()
+    B.slkv_profile_enable(0)
+    B.slkv_debug_list_way(0)
+    return outs, set(B.slkv_profile_collect())
+
+
+def both_ways(layers, lens, w, pool, budgets, **kw):
+    """The list without and with pooled scores."""
     got = []
     for pooled in (False, True):
-        ws.fill_(0x5a)
-        outs = []
-        for (q, k, v), bud in zip(layers, budgets):
-            cap = sum(min(n, max(int(b), w)) for n in lens for b in bud)
-            b = torch.tensor(bud, dtype=torch.int32, device=DEV)
-            o = [torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV), torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV),
-                 torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.full((cap,), -1, dtype=torch.int32, device=DEV),
-                 torch.zeros(1, dtype=torch.int32, device=DEV)]
-            scores = torch.zeros(B.slkv_pooled_elems(p, cu), device=DEV) if pooled else None
-            B.slkv_compress_overlapped(p, q, k, v, cu_dev, cu, b, *o[:4], ws, scores, o[4])
-            outs.append(o + [b, scores])                 # the calls are queued: what they use stays
-        B.slkv_join()
-        torch.cuda.synchronize()
+        outs, kernels = one_list(layers, lens, w, pool, budgets, 1, pooled, **kw)
+        assert kernels == {"k_score_list" if pooled else "k_score_bound"}
         got.append(outs)
     for one, all_votes in zip(*got):
         assert int(one[4]) == 0 and int(all_votes[4]) == 0
@@ -198,4 +218,42 @@ def test_heads_that_need_all_votes_among_others(hq, hkv, d, w, lens, share):
     n_layers = 8 if sum(lens) < 70000 else 5
     layers = [inputs("stripes", l + w, lens, hq, hkv, d, w) for l in range(n_layers)]
     budgets = [[int(w + (rng.integers(600, 6000) if rng.random() < share else rng.integers(0, 400))) for _ in range(hkv)] for _ in layers]
+    both_ways(layers, lens, w, 7, budgets)
+
+
+@pytest.mark.parametrize("n", [16300, 32764, 32800])        # 16 and 32 positions a thread, a cluster
+def test_against_the_oracle(n):
+    w, hq, hkv, d = 32, 8, 2, 128
+    lens = [n + w, 9000]
+    layers = [inputs(kind, n + l, lens, hq, hkv, d, w) for l, kind in enumerate(["stripes", "gaussian"])]
+    budgets = [[w + 100, w + 400], [w + 10, w + 700]]
+    outs, kernels = one_list(layers, lens, w, 7, budgets, 1)
+    assert kernels == {"k_score_bound"}
+    cu = [0, lens[0], sum(lens)]
+    for (q, k, v), o, bud in zip(layers, outs, budgets):
+        gpu = {"offsets": o[2].cpu().numpy().astype(np.int64), "kept_idx": o[3].cpu().numpy().astype(np.int64), "k_out": o[0].cpu(), "v_out": o[1].cpu()}
+        assert int(o[4]) == 0
+        P.assert_selection_valid(gpu, P.oracle_pooled(q.cpu(), k.cpu(), cu, w, 7), cu, bud, w, k.cpu(), v.cpu())
+
+
+@pytest.mark.parametrize("n_layers,keep,pooled,kernel", [(31, 100, False, "k_score_bound"), (31, 100, True, "k_score_list"), (31, 512, False, "k_score_list"),
+                                                         (18, 20, False, "k_score_bound"), (18, 400, False, "k_score_list"), (8, 20, False, "k_score_list")])
+def test_which_way_a_list_goes(n_layers, keep, pooled, kernel):
+    """17000 tokens, 8 KV heads, 128 rows: 1064 products a layer.  Few of them, or much to keep, and two products are quicker."""
+    w = 32
+    x = inputs("gaussian", 1, [17000], 32, 8, 128, w)
+    _, kernels = one_list([x] * n_layers, [17000], w, 7, [[w + keep] * 8] * n_layers, 0, pooled)
+    assert kernels == {kernel}
+
+
+@pytest.mark.parametrize("wait", [1, 2])                     # for the statistics, for their clearing
+def test_a_wait_that_runs_out(wait):
+    """Every CTA gives up after its limit, the status words say so, and the next list is right."""
+    w, lens = 32, [33032]
+    layers = [inputs("stripes", l, lens, 8, 2, 128, w) for l in range(3)]
+    budgets = [[w + 50, w + 900]] * 3                        # the second head gets all its votes: those wait for the statistics
+    B.slkv_debug_expire_next_wait(wait)
+    outs, kernels = one_list(layers, lens, w, 7, budgets, 1)
+    assert kernels == {"k_score_bound"}
+    assert all(int(o[4]) == B.ERR["DEVICE_TIMEOUT"] for o in outs)
     both_ways(layers, lens, w, 7, budgets)
