@@ -229,7 +229,7 @@ int enqueue_votes(const Problem& pb, int path, const int32_t* cu_host, int32_t* 
   int rc = enqueue_window_stats(pb, path, st, launches);
   if (rc != SLKV_OK) return rc;
   const int passes = pb.lse_opt ? 2 : 3;
-  cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes, nullptr, false, st, launches)
+  cudaError_t e = path == SLKV_PATH_TENSOR ? launch_score_tensor(pb, cu_host, status, passes == 3 && bound_shape(pb) ? kScoreWide : passes, nullptr, false, st, launches)
                                            : launch_score_simt(pb, status, passes, st, launches);
   if (e != cudaSuccess) return cuda_fail(e);
   return SLKV_OK;
@@ -290,14 +290,15 @@ cudaError_t flush_list(ListState* s, cudaStream_t owner, int* launches) {
   s->n = 0;
   s->in_flight = true;
   cudaError_t e;
-  bool bound = !s->with_lse && bound_list_supported(s->pb, s->tail, n);
-  for (int i = 0; i < n; ++i) bound = bound && s->tail[i].pooled_out == nullptr;
-  if (bound) {
+  const bool bound = !s->with_lse && bound_list_supported(s->pb, s->tail, n);
+  bool pooled = false;
+  for (int i = 0; i < n; ++i) pooled = pooled || s->tail[i].pooled_out != nullptr;
+  if (bound && !pooled) {
     e = launch_bound_list(s->pb, s->plan.sh, s->score, s->tail, n, owner, launches);
     if (e == cudaSuccess) e = launch_gather(s->pb, s->tail, n, owner, launches);
     if (e != cudaErrorNotSupported) return e;
   }
-  e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : 3, s->pb.sync, owner, launches);
+  e = launch_score_list(s->plan.sh, s->score, n, s->with_lse ? 2 : bound || bound_shape(s->pb) ? kScoreWide : 3, s->pb.sync, owner, launches);
   if (e == cudaSuccess)
     e = select_list_supported(s->pb) ? launch_select_list(s->pb, s->tail, n, owner, launches)
                                      : launch_select_cluster(s->pb, s->tail, n, owner, launches);

@@ -533,6 +533,16 @@ thread_local int g_list_way = 0;
 }
 void set_list_way(int way) { g_list_way = way; }
 
+bool bound_possible(const Problem& pb) {
+  if (pb.p.pool_mode != SLKV_POOL_MAX || !select_list_supported(pb) || pb.R <= 64) return false;
+  return (int64_t)pb.n_seg * tensor_slot_stride(pb) * pb.R < (1ll << 31);                    // places of the weights: 32-bit
+}
+bool bound_shape(const Problem& pb) {
+  if (!bound_possible(pb)) return false;
+  const int64_t mean = pb.total_hist / pb.p.n_seqs;
+  return mean >= 32000 || (pb.R > 128 ? mean >= 12000 && pb.n_tiles128 >= 3000 : mean >= 16000);
+}
+
 // Where the second product is worth more than the longer selection.  It saves some 3.5 ns for every product of 128 keys x 128 rows; the
 // selection takes 50-90 us longer whatever the list's length, for 256 rows twice that.  With it come the segments that need all their votes
 // (every_vote): both products, the second one from HBM.  The budgets are on the device, but what a layer keeps at most is known
@@ -550,11 +560,9 @@ void set_list_way(int way) { g_list_way = way; }
 //             eight of 16384 to 32768, 8 (98304): 0.87 2124 / 1820
 //   64 rows   one sequence of 20000 tokens 428 / 446
 bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers) {
-  if (pb.p.pool_mode != SLKV_POOL_MAX || !select_list_supported(pb) || pb.R <= 64 || g_list_way == 2) return false;
-  if ((int64_t)pb.n_seg * tensor_slot_stride(pb) * pb.R >= (1ll << 31)) return false;        // places of the weights: 32-bit
-  if (g_list_way == 1) return true;
+  if (g_list_way != 0) return g_list_way == 1 && bound_possible(pb);
+  if (!bound_shape(pb)) return false;
   const int64_t mean = pb.total_hist / pb.p.n_seqs;
-  if (!(mean >= 32000 || (pb.R > 128 ? mean >= 12000 && pb.n_tiles128 >= 3000 : mean >= 16000))) return false;
   const int64_t line = mean / kEveryVoteShare > kEveryVoteCount ? mean / kEveryVoteShare : kEveryVoteCount;
   const int64_t window_rows = (int64_t)pb.p.n_kv_heads * (pb.total_tokens - pb.total_hist);
   double most = 0.0;

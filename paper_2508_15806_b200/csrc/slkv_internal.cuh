@@ -277,8 +277,9 @@ cudaError_t plan_score_layer(const Problem& pb, int32_t* status, ScoreLayer* lay
 int sm_count();
 int score_list_stages(int MT, int halves);
 // The score kernel over a list of layers of one shape: passes 1 = row statistics, 2 = votes from the callers' row
-// statistics, 3 = both, kScoreBound = row statistics and estimated votes (slkv_bound.cu); sync: Problem's.
-constexpr int kScoreBound = 4;
+// statistics, 3 = both, kScoreBound = row statistics and estimated votes (slkv_bound.cu), kScoreWide = both with the same row sums
+// as those bit for bit; sync: Problem's.
+constexpr int kScoreBound = 4, kScoreWide = 5;
 // A list for bounds computes every vote of a segment that keeps so many positions and that share of them.
 constexpr int kEveryVoteCount = 512, kEveryVoteShare = 64;
 #ifdef __CUDACC__
@@ -290,6 +291,8 @@ __device__ __forceinline__ bool every_vote(int len, int budget, int window) {
 cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n_layers, int passes,
                               unsigned long long* sync, cudaStream_t st, int* launches, bool cleared = false);
 // Scores and selection of a list in one product with every key (slkv_bound.cu).  cudaErrorNotSupported: nothing is launched.
+bool bound_possible(const Problem& pb);
+bool bound_shape(const Problem& pb);              // shapes of which some lists go that way: both passes then take the same row sums
 bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers);
 void set_list_way(int way);                       // of this thread: 0 by rule, 1 one product wherever it can be, 2 two
 cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const ScoreLayer* lay, const TailLayer* tail, int n_layers,

@@ -229,7 +229,7 @@ k_layer_tc(const __grid_constant__ LayerArgs a) {
         }
       double z;
       float far_z, far_m;
-      stats_run(u, 0, a.scale_log2, wg, 4, n_t, x.n - first * kTileKeys, (warp & 3) * 32 < a.R, z, far_z, far_m);
+      stats_run<false>(u, 0, a.scale_log2, wg, 4, n_t, x.n - first * kTileKeys, (warp & 3) * 32 < a.R, z, far_z, far_m);
       f.z_wg[wg][row] = z;
       f.far_wg[wg][row] = make_float2(far_z, far_m);
       if (far_z > 0.f) f.far_here = 1;

@@ -49,6 +49,7 @@ namespace {
 constexpr int kWgs = 4;                              // epilogue warpgroups = TMEM units
 constexpr int kListThreads = 128 + kWgs * 128;
 constexpr int kMaxStages = 6;
+constexpr int kPlain = 0, kWide = 1, kBound = 2;      // kinds of k_score_list
 // Shared memory behind the Q tile and the K ring: mbarriers and flags, far row statistics [2][kWgs][128] (sum, reference),
 // log-sum-exps [2][256], half votes [2][4][128], runs.
 constexpr int kBarBytes = 640;
@@ -695,8 +696,9 @@ __device__ __forceinline__ void fetch_lse(const Smem& c, const ListArgs& a) {
 }
 
 // ---- warps 4-19: the arithmetic ---------------------------------------------------------------------------------------
-template <int MT, bool BOUND>
+template <int MT, int KIND>
 __device__ __forceinline__ void epilogue(const Smem& c) {
+  constexpr bool BOUND = KIND == kBound;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wg = (threadIdx.x - 128) >> 7, row = threadIdx.x & 127;
   Unit u;
@@ -742,7 +744,7 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
         ok = bound_run<MT>(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, wg, b, z, far_z, far_m);
         n_part += n_mine;
       } else {
-        ok = stats_run(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, z, far_z, far_m);
+        ok = stats_run<KIND != kPlain>(u, units, c.sc, i0, every, r.count, r.n_valid, rows_here, z, far_z, far_m);
       }
       const int slot = n_stat & 1;
       ok = ok && mbar_wait(c.stat_empty(slot), ((n_stat >> 1) & 1) ^ 1, c.abort_flag) && mbar_wait(c.cleared(), 0, c.abort_flag);
@@ -777,11 +779,13 @@ __device__ __forceinline__ void epilogue(const Smem& c) {
 // that do the arithmetic is what the instruction caches have to hold, and a row block's constants are folded into it.  With one
 // kernel for all, 32 layers of 4001 / 8000 / 32k tokens, 128 rows: 123.7 / 225 / 838 us, now 121.1 / 220 / 812; 16000 tokens, 64 rows
 // 376 -> 353; four sequences of 5k - 10k 689 -> 658; 256 rows as before.
-// BOUND: statistics and estimated votes in one pass over the list, then the votes of the segments that need them all
-// (slkv_bound.cu); a kernel of its own, so that neither kind's loops grow.
-template <int MT, int HALVES, bool BOUND>
+// kBound: statistics and estimated votes in one pass over the list, then the votes of the segments that need them all
+// (slkv_bound.cu); a kernel of its own, so that neither kind's loops grow.  kWide: both passes with kBound's row sums (TileSum), for
+// every call of a shape that kBound's lists have, so that what is kept depends neither on the list nor on who asks for pooled scores.
+template <int MT, int HALVES, int KIND>
 __global__ void __launch_bounds__(kListThreads, 1)
 k_score_list(const __grid_constant__ ListArgs a) {
+  constexpr bool BOUND = KIND == kBound;
   // Shared memory, all dynamic and 1024-byte aligned (the swizzled tiles need it):
   //   [kQTiles Q tiles: halves x MT x 16 KB][K ring: n_stages x halves x 16 KB][mbarriers, flags][statistics][log-sum-exps][half votes]
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -878,7 +882,7 @@ k_score_list(const __grid_constant__ ListArgs a) {
     pdl_wait();
     fetch_lse(c, a);
   } else {
-    epilogue<MT, BOUND>(c);
+    epilogue<MT, KIND>(c);
   }
 
   tc_fence_before();
@@ -943,13 +947,14 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   if (n_layers < 1 || sh.n_cta == 0) return cudaSuccess;             // no history: nothing to score
   if (n_layers > kListMaxLayers) return cudaErrorInvalidValue;
   const bool bound = passes == kScoreBound;
-  if (bound) passes = 3;
-  const Kern kernel = sh.MT == 1 ? (sh.halves == 1 ? (bound ? k_score_list<1, 1, true> : k_score_list<1, 1, false>)
-                                                   : (bound ? k_score_list<1, 2, true> : k_score_list<1, 2, false>))
-                                 : (sh.halves == 1 ? (bound ? k_score_list<2, 1, true> : k_score_list<2, 1, false>)
-                                                   : (bound ? k_score_list<2, 2, true> : k_score_list<2, 2, false>));
-  static thread_local int configured_on[2][2][2] = {{{-1, -1}, {-1, -1}}, {{-1, -1}, {-1, -1}}};
-  int& configured_dev = configured_on[sh.MT - 1][sh.halves - 1][bound];
+  const int kind = bound ? kBound : passes == kScoreWide ? kWide : kPlain;
+  if (kind != kPlain) passes = 3;
+#define SLKV_LIST(MT, HALVES) {k_score_list<MT, HALVES, kPlain>, k_score_list<MT, HALVES, kWide>, k_score_list<MT, HALVES, kBound>}
+  static const Kern kernels[2][2][3] = {{SLKV_LIST(1, 1), SLKV_LIST(1, 2)}, {SLKV_LIST(2, 1), SLKV_LIST(2, 2)}};
+#undef SLKV_LIST
+  const Kern kernel = kernels[sh.MT - 1][sh.halves - 1][kind];
+  static thread_local int configured_on[2][2][3] = {{{-1, -1, -1}, {-1, -1, -1}}, {{-1, -1, -1}, {-1, -1, -1}}};
+  int& configured_dev = configured_on[sh.MT - 1][sh.halves - 1][kind];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1045,7 +1050,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   }
   cs = -1;
   if (bound) return cudaErrorNotSupported;
-  return launch_score_list(sh, lay, n_layers, passes, sync, st, launches);
+  return launch_score_list(sh, lay, n_layers, kind == kWide ? kScoreWide : passes, sync, st, launches);
 }
 
 }  // namespace slkv

@@ -151,12 +151,18 @@ __device__ __forceinline__ f32x2 ex2_pair(f32x2 x) {
 // both passes (one exponential per query row and key): x = n + f with n = round(x), 2^f by a degree-5 polynomial that
 // is minimax in relative error on [-0.5, 0.5] (Remez exchange; 2.1e-7 evaluated in fp32, ex2.approx has 2^-22 =
 // 2.4e-7), n added into the exponent field.  x is clamped at -125 (the result is then 2^-125: negligible in any sum
-// that holds a term near 1).
+// that holds a term near 1) and, where CLAMP_HI, at 128.5, from where the exponent field overflows to Inf / NaN, which
+// the statistics pass's overflow check catches.
+template <bool CLAMP_HI>
 __device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {
   float a, b;
   unpack2(x, a, b);
   a = fmaxf(a, -125.f);
   b = fmaxf(b, -125.f);
+  if (CLAMP_HI) {
+    a = fminf(a, 128.5f);
+    b = fminf(b, 128.5f);
+  }
   x = pack2(a, b);
   const f32x2 t = add2(x, pack2(12582912.f, 12582912.f));     // 1.5 * 2^23: round(x) lands in the low mantissa bits
   const f32x2 f = fma2(add2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x);
@@ -335,8 +341,8 @@ __device__ __forceinline__ void tile_stats_exact(uint32_t tcol, float sc, int fi
 // Votes: sum_e 2^(v_e * sc + off_e) over 16 accumulator values, in two pair accumulators.  POLY: the first pair's exponentials
 // go to the FMA pipe, where it takes fourteen instructions instead of two.  By cycles alone two pairs of eight would go there;
 // at the power limit the instructions cost more clock than they save cycles (32 layers of 32k / 128k positions, in both
-// passes no pair of a chunk's eight on the FMA pipe 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: none in the
-// statistics, in the votes one in every other chunk.
+// passes no pair of a chunk's eight on the FMA pipe 862 / 5866 us, one 877 / 5806, two 890 / 5905).  Here: in the votes one in
+// every other chunk, in the statistics one in eight (TileSum).
 // The loops around this are kept small, the statistics' one chunk at a time with the last keys of a segment outside: four
 // warps on a scheduler hide a TMEM load's latency, and the epilogue warps are spread over both passes' loops, which have to
 // stay in the instruction cache (4k positions: statistics loop unrolled four times 154 us, twice 144, two chunks with the
@@ -350,22 +356,41 @@ __device__ __forceinline__ void exp_chunk(const uint32_t (&r)[16], f32x2 sc2, ui
     asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(o0), "=l"(o1) : "r"(off_sh + 4u * e));
     const f32x2 x0 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, o0);
     const f32x2 x1 = fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sc2, o1);
-    s0 = add2(s0, POLY && e == 0 ? ex2_pair_poly(x0) : ex2_pair(x0));
+    s0 = add2(s0, POLY && e == 0 ? ex2_pair_poly<false>(x0) : ex2_pair(x0));
     s1 = add2(s1, ex2_pair(x1));
   }
-}
-// Statistics: a row's sum of 2^(v * sc) over a tile goes through eight accumulators, one for each column modulo 8, here four
-// pairs; stats_sum adds those up.  (Eight, because that is how the columns lie in the lanes of bound_run.)
-__device__ __forceinline__ void stats_chunk(const uint32_t (&r)[16], f32x2 sc2, f32x2 (&s)[4]) {
-#pragma unroll
-  for (int e = 0; e < 16; e += 2) s[(e >> 1) & 3] = add2(s[(e >> 1) & 3], ex2_pair(fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, 0)));
 }
 __device__ __forceinline__ float pair_sum(f32x2 v) {
   float a, b;
   unpack2(v, a, b);
   return a + b;
 }
-__device__ __forceinline__ float stats_sum(const f32x2 (&s)[4]) { return (pair_sum(s[0]) + pair_sum(s[1])) + (pair_sum(s[2]) + pair_sum(s[3])); }
+// Statistics: a row's sum of 2^(v * sc) over a tile, in two pair accumulators, one pair of eight on the FMA pipe.  WIDE: the sums of a
+// launch for bounds, where eight accumulators, one for each column modulo 8, lie in the lanes as in bound_run; there a pair of
+// columns is one of four lanes' and none goes to the FMA pipe.  Short lists miss that share (with / without: 32 layers of 4001 tokens, 128 rows
+// 125.0 / 126.5 us, 16 of 24000, 256 rows 495 / 504, a rank's statistics and votes of 32768 111.1 / 112.1), long ones hardly (12000 tokens 302 / 302).  A chunk of
+// sixteen columns on the FMA pipe, the same in both: 131.6, 505, 112.1, and the launch for bounds 623 -> 661.
+template <bool WIDE>
+struct TileSum {
+  f32x2 s[WIDE ? 4 : 2];
+  __device__ __forceinline__ TileSum() {
+#pragma unroll
+    for (int i = 0; i < (WIDE ? 4 : 2); ++i) s[i] = 0;
+  }
+  __device__ __forceinline__ void chunk(const uint32_t (&r)[16], f32x2 sc2) {
+#pragma unroll
+    for (int e = 0; e < 16; e += 2) {
+      const f32x2 x = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, 0);
+      f32x2& to = s[(e >> 1) & (WIDE ? 3 : 1)];
+      to = add2(to, !WIDE && e == 0 ? ex2_pair_poly<true>(x) : ex2_pair(x));
+    }
+  }
+  __device__ __forceinline__ float total() const {
+    const float low = pair_sum(s[0]) + pair_sum(s[1]);
+    if constexpr (WIDE) return low + (pair_sum(s[2]) + pair_sum(s[3]));
+    else return low;
+  }
+};
 
 // An epilogue thread's unit.
 struct Unit {
@@ -389,6 +414,7 @@ __device__ __forceinline__ void unit_release(const Unit& u) {
 // reference; (far_z, far_m): what of it fp64 cannot hold (see StatView).  A tile is summed in fp32, without a reference
 // either as long as nothing overflows and not everything underflows; one whose sum is not finite and above kTinySum is
 // redone exactly.  false: a wait ran out.
+template <bool WIDE>
 __device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i0, int every, int count, int n_valid0,
                                           bool rows_here, double& z, float& far_z, float& far_m) {
   z = 0.0;
@@ -400,15 +426,15 @@ __device__ __forceinline__ bool stats_run(const Unit u, int nth, float sc, int i
     if (rows_here) {
       const int n_valid = n_valid0 - i * kTileKeys;
       const int whole = n_valid < kTileKeys ? n_valid & ~15 : kTileKeys;
-      f32x2 s[4] = {0, 0, 0, 0};
+      TileSum<WIDE> s;
 #pragma unroll 1
       for (int c0 = 0; c0 < whole; c0 += 16) {
         uint32_t v[16];
         tc_ld16_issue(u.tcol + c0, v);
         tc_ld_wait(v);
-        stats_chunk(v, sc2, s);
+        s.chunk(v, sc2);
       }
-      float tile = stats_sum(s);
+      float tile = s.total();
       if (n_valid < kTileKeys) {                               // the segment's last keys; those past its end count nothing
         float tm, tz;
         tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
@@ -461,7 +487,7 @@ __device__ __forceinline__ void tc_ld_quads(uint32_t taddr, uint32_t (&v)[16]) {
 }
 // The row, of the warp's 32, whose sum a thread has in the end.
 __device__ __forceinline__ int quad_row() { return ((threadIdx.x & 31) >> 2) + 8 * (threadIdx.x & 3); }
-// stats_chunk for four rows of two columns in eight, whose sums these are bit for bit (s[q]: row g + 8 q), and the four rows'
+// TileSum<true> for four rows of two columns in eight, whose sums these are bit for bit (s[q]: row g + 8 q), and the four rows'
 // weight * exponential of the two columns in h[b], rounded to bf16.
 __device__ __forceinline__ void bound_chunk(const uint32_t (&v)[16], f32x2 sc2, const f32x2 (&w2)[4], f32x2 (&s)[4], uint32_t* h) {
 #pragma unroll
@@ -477,7 +503,7 @@ __device__ __forceinline__ void bound_chunk(const uint32_t (&v)[16], f32x2 sc2, 
     h[b] = bf16_pair(est);
   }
 }
-// stats_sum of the thread's row: of the four rows that lie in four lanes each, a lane keeps one.
+// The sum of the thread's row: of the four rows that lie in four lanes each, a lane keeps one.
 __device__ __forceinline__ float quad_sum(const f32x2 (&s)[4]) {
   const bool odd = threadIdx.x & 1, high = threadIdx.x & 2;
   float a[4];
@@ -546,7 +572,7 @@ struct BoundRun {
   int rows, n_warps;           // rows per KV head, warps that hold some
 };
 
-// Statistics of one run, as stats_run (the sums are the same bit for bit, but of row quad_row() of the warp's), and with the same exponentials an estimate of every key's
+// Statistics of one run, as stats_run<true> (the sums are the same bit for bit, but of row quad_row() of the warp's), and with the same exponentials an estimate of every key's
 // vote, est[key] = sum_rows weight_r * 2^score.  The rows' sums are not known yet: weight_r is the reciprocal of the row's sum over
 // the run's first tiles in the order of Spread, one per warpgroup (two: per pair), whose accumulators are read twice for it, and from a
 // quarter of the run on over that quarter (the bounds are three to five times as tight in the keys that they let through).  The
@@ -566,15 +592,15 @@ __device__ __forceinline__ bool bound_run(const Unit u, int nth, float sc, int i
     if (!unit_wait(u, nth)) return false;
     if (rows_here) {
       const int n_valid = n_valid0 - order.tile(i0) * kTileKeys, whole = n_valid < kTileKeys ? n_valid & ~15 : kTileKeys;
-      f32x2 s[4] = {0, 0, 0, 0};
+      TileSum<true> s;
 #pragma unroll 1
       for (int c0 = 0; c0 < whole; c0 += 16) {
         uint32_t v[16];
         tc_ld16_issue(u.tcol + c0, v);
         tc_ld_wait(v);
-        stats_chunk(v, sc2, s);
+        s.chunk(v, sc2);
       }
-      first = stats_sum(s);
+      first = s.total();
       if (whole < n_valid && whole < kTileKeys) {
         float tm, tz;
         tile_stats_exact(u.tcol, sc, whole, n_valid, tm, tz);
