@@ -38,7 +38,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     obj_dir = os.path.join(HERE, "build")
     os.makedirs(obj_dir, exist_ok=True)
     flags = ["-Xcompiler", "-fPIC", "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
-             "-I", os.path.join(ROOT, "include"), "-I", CSRC]
+             "-Xfatbin=-compress-all", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if verbose:
         flags += ["-Xptxas", "-v"]
 

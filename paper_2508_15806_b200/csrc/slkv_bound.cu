@@ -60,9 +60,13 @@ struct alignas(16) BoundShared {
   float beside[8];                           // exact votes of the four places on either side of a cluster's slice
 };
 
-template <int T, int IT, int RAD, bool CLUSTER>
-__global__ void __launch_bounds__(T, T == 1024 ? 1 : 2)
+constexpr int kThreads = 1024;
+
+// IT consecutive positions a thread.  CLUSTER: a segment is shared by the CTAs of a cluster.
+template <int IT, int RAD, bool CLUSTER>
+__global__ void __launch_bounds__(kThreads, 1)
 k_select_bound(const __grid_constant__ BoundArgs args) {
+  constexpr int T = kThreads;
   constexpr int kWarps = T / 32, kPitch = IT + 4, kPer = kBins / T;
   // [votes] or [Q][keys][list of places]
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -510,27 +514,25 @@ k_select_bound(const __grid_constant__ BoundArgs args) {
 // ---- host side ----------------------------------------------------------------------------------------------------------
 typedef void (*Kern)(const BoundArgs);
 struct Variant {
-  int threads, items;
+  int items;
   Kern kern[kMaxRadius + 1];
 };
-#define SLKV_SEL(T, IT, C) \
-  {T, IT, {k_select_bound<T, IT, 0, C>, k_select_bound<T, IT, 1, C>, k_select_bound<T, IT, 2, C>, k_select_bound<T, IT, 3, C>, k_select_bound<T, IT, 4, C>}}
-const Variant kVariants[] = {SLKV_SEL(512, 8, false), SLKV_SEL(512, 16, false), SLKV_SEL(1024, 16, false), SLKV_SEL(1024, 32, false),
-                             SLKV_SEL(1024, 32, true)};
+#define SLKV_SEL(IT, C) \
+  {IT, {k_select_bound<IT, 0, C>, k_select_bound<IT, 1, C>, k_select_bound<IT, 2, C>, k_select_bound<IT, 3, C>, k_select_bound<IT, 4, C>}}
+const Variant kVariants[] = {SLKV_SEL(16, false), SLKV_SEL(32, false), SLKV_SEL(32, true)};
 #undef SLKV_SEL
 
 size_t select_bytes(const ScoreShape& sh, const Variant& v, int k_tiles) {
   const size_t product = (size_t)sh.halves * (sh.MT * 128 * 128 + k_tiles * kHalfBytes);
-  const size_t votes = (size_t)vote_floats(v.threads, v.items) * sizeof(float);
-  const size_t list = (size_t)(v.threads * v.items + 16) * sizeof(unsigned short);
+  const size_t votes = (size_t)vote_floats(kThreads, v.items) * sizeof(float);
+  const size_t list = (size_t)(kThreads * v.items + 16) * sizeof(unsigned short);
   return product + list > votes ? product + list : votes;
 }
 
+thread_local int g_list_way = 0;
+
 }  // namespace
 
-namespace {
-thread_local int g_list_way = 0;
-}
 void set_list_way(int way) { g_list_way = way; }
 
 bool bound_possible(const Problem& pb) {
@@ -589,11 +591,10 @@ cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const Sco
   // largest took 10 and 16 us instead of 3 and 8.
   const int cs = select_list_cluster(pb);
   const int slice = ((pb.max_hist + 3 + cs - 1) / cs + 3) & ~3;
-  const Variant& var = kVariants[cs > 1 ? 4 : slice <= 4096 ? 0 : slice <= 8192 ? 1 : slice <= 16384 ? 2 : 3];
+  const Variant& var = kVariants[cs > 1 ? 2 : slice <= 16384 ? 0 : 1];
   constexpr size_t kStatic = sizeof(SelShared) + sizeof(BoundShared) + 1024;
-  const size_t room = var.threads == 512 ? 113 * 1024 - kStatic : kSmemLimit - kStatic;       // two CTAs to an SM
-  // two tiles of keys at a time where shared memory and, of two CTAs, TMEM hold them
-  a.k_tiles = select_bytes(sh, var, 2) <= room && (var.threads > 512 || sh.MT == 1) ? 2 : 1;
+  // two tiles of keys at a time where shared memory holds them
+  a.k_tiles = select_bytes(sh, var, 2) <= kSmemLimit - kStatic ? 2 : 1;
   a.n_layers = n_layers;
   static thread_local int configured_dev = -1;
   int dev = 0;
@@ -610,7 +611,7 @@ cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const Sco
   e = launch_score_list(sh, a.lay, n_layers, kScoreBound, pb.sync, st, launches);
   if (e != cudaSuccess) return e;
   LaunchScope scope(KID_SELECT, st, launches);
-  return launch_pdl(var.kern[pb.p.pool_kernel >> 1], dim3((unsigned)(pb.n_seg * cs), (unsigned)n_layers), dim3((unsigned)var.threads),
+  return launch_pdl(var.kern[pb.p.pool_kernel >> 1], dim3((unsigned)(pb.n_seg * cs), (unsigned)n_layers), dim3(kThreads),
                     select_bytes(sh, var, a.k_tiles), st, cs, a);
 }
 

@@ -55,14 +55,16 @@ constexpr int kPlain = 0, kWide = 1, kBound = 2;      // kinds of k_score_list
 constexpr int kBarBytes = 640;
 constexpr int kStatBytes = 2 * kWgs * 128 * 8;
 constexpr int kLseBytes = 2 * 256 * 4;
-constexpr int kPartBytes = kWgs * 2 * 4 * 128 * 4;      // per warpgroup two slots of its warps' shares, see bound_run; half votes take a quarter
+constexpr int kHalfVoteBytes = 2 * 4 * 128 * 4;
+constexpr int kPartBytes = kWgs * 2 * 4 * 128 * 4;      // bounds: per warpgroup two slots of its warps' shares, see bound_run; half votes there, too
 // Two Q tiles, also where that leaves the ring no more than two K tiles (R > 128, d = 128): the next run's queries are
 // there when its keys are.  One Q tile and four K tiles cost a pause of 1.6 us in every run of about 25: 128k positions
 // 5935 -> 5810 us, eight sequences of 4k - 32k 6830 -> 6690 us (32 layers each).
 constexpr int kQTiles = 2;
 constexpr int kRunSlots = 8;                         // runs handed out ahead
-constexpr int kFirstBytes = 2 * kWgs * 128 * 4;      // [2][kWgs][128]: sums over the first tiles of a run, see bound_run
-constexpr int kTail = kBarBytes + kStatBytes + kLseBytes + kPartBytes + kFirstBytes + kRunSlots * 128;
+constexpr int kFirstBytes = 2 * kWgs * 128 * 4;      // bounds: [2][kWgs][128] sums over the first tiles of a run, see bound_run
+constexpr int kRunsAt = kBarBytes + kStatBytes + kLseBytes + kHalfVoteBytes, kRunsAtBound = kBarBytes + kStatBytes + kLseBytes + kPartBytes + kFirstBytes;
+constexpr int kTail = kRunsAt + kRunSlots * 128, kTailBound = kRunsAtBound + kRunSlots * 128;
 
 // The clearing of the statistics and the groups' counts: one word with the launch's tag (40 bits) above two counts of 12 bits,
 // CTAs that are done and CTAs that have cleared their share.  A CTA that finds another value puts the tag first; the last CTA
@@ -810,8 +812,8 @@ k_score_list(const __grid_constant__ ListArgs a) {
   c.stat_far = reinterpret_cast<unsigned*>(tail + kBarBytes - 8);
   c.lse = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes);
   c.half_vote = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes + kLseBytes);
-  c.first = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes + kLseBytes + kPartBytes);
-  c.runs = reinterpret_cast<RunDesc*>(tail + kBarBytes + kStatBytes + kLseBytes + kPartBytes + kFirstBytes);
+  c.first = reinterpret_cast<float*>(tail + kBarBytes + kStatBytes + kLseBytes + kPartBytes);       // bounds
+  c.runs = reinterpret_cast<RunDesc*>(tail + (BOUND ? kRunsAtBound : kRunsAt));
 
   if (tid == 0) {
     trace_mark(a.trace, 0);
@@ -938,7 +940,7 @@ unsigned long long* tensor_trace_buffer(int n_cta) {
 
 // K tiles of the ring beside the Q tiles.
 int score_list_stages(int MT, int halves) {
-  const int n = (kSmemLimit - kTail - kQTiles * halves * MT * 128 * 128) / (halves * kHalfBytes);
+  const int n = (kSmemLimit - kTailBound - kQTiles * halves * MT * 128 * 128) / (halves * kHalfBytes);
   return n < kMaxStages ? n : kMaxStages;
 }
 
@@ -992,7 +994,7 @@ cudaError_t launch_score_list(const ScoreShape& sh, const ScoreLayer* lay, int n
   a.target = (unsigned)sh.n_cta + (expire == 1);
   a.sync.expect = (unsigned)sh.n_cta + (expire == 2);
   a.trace = tensor_trace_buffer(sh.n_cta);
-  const size_t smem = (size_t)(kQTiles * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + kTail);
+  const size_t smem = (size_t)(kQTiles * sh.halves * sh.MT * 128 * 128 + sh.n_stages * sh.halves * kHalfBytes + (bound ? kTailBound : kTail));
 
   // CTAs that wait for one another must all be resident: cooperative launch, with dependent launch on top where the
   // device takes both.  Where it takes no cooperative launch, or the environment says so (tests), the two passes go out
