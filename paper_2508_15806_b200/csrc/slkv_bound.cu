@@ -567,9 +567,11 @@ bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers
   const int64_t mean = pb.total_hist / pb.p.n_seqs;
   const int64_t line = mean / kEveryVoteShare > kEveryVoteCount ? mean / kEveryVoteShare : kEveryVoteCount;
   const int64_t window_rows = (int64_t)pb.p.n_kv_heads * (pb.total_tokens - pb.total_hist);
+  // Room for every row says nothing of what is kept: few positions, which is what a cache is compressed for.
+  const int64_t all_rows = (int64_t)pb.p.n_kv_heads * pb.total_tokens;
   double most = 0.0;
   for (int i = 0; i < n_layers; ++i) {
-    const double share = (double)(tail[i].capacity - window_rows) / (double)(line * pb.n_seg);
+    const double share = tail[i].capacity >= all_rows ? 0.5 : (double)(tail[i].capacity - window_rows) / (double)(line * pb.n_seg);
     most += share < 1.0 ? (share > 0.0 ? share : 0.0) : 1.0;
   }
   most /= n_layers;

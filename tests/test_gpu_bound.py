@@ -61,7 +61,7 @@ def inputs(kind, seed, lens, hq, hkv, d, w):
     return q.bfloat16(), k.bfloat16(), v
 
 
-def one_list(layers, lens, w, pool, budgets, way, pooled=False, **kw):
+def one_list(layers, lens, w, pool, budgets, way, pooled=False, room=None, **kw):
     """The layers' outputs (k, v, offsets, kept positions, status), and the score kernel they took."""
     cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
     p = B.make_params(*layers[0], w, pool, **kw)
@@ -72,7 +72,7 @@ def one_list(layers, lens, w, pool, budgets, way, pooled=False, **kw):
     B.slkv_debug_list_way(way)
     B.slkv_profile_enable(2)
     for (q, k, v), bud in zip(layers, budgets):
-        cap = sum(min(n, max(int(b), w)) for n in lens for b in bud)
+        cap = room or sum(min(n, max(int(b), w)) for n in lens for b in bud)
         b = torch.tensor(bud, dtype=torch.int32, device=DEV)
         o = [torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV), torch.full((cap, d), 7, dtype=torch.bfloat16, device=DEV),
              torch.zeros(len(lens) * hkv + 1, dtype=torch.int32, device=DEV), torch.full((cap,), -1, dtype=torch.int32, device=DEV),
@@ -236,13 +236,16 @@ def test_against_the_oracle(n):
         P.assert_selection_valid(gpu, P.oracle_pooled(q.cpu(), k.cpu(), cu, w, 7), cu, bud, w, k.cpu(), v.cpu())
 
 
-@pytest.mark.parametrize("n_layers,keep,pooled,kernel", [(31, 100, False, "k_score_bound"), (31, 100, True, "k_score_list"), (31, 512, False, "k_score_list"),
-                                                         (18, 20, False, "k_score_bound"), (18, 400, False, "k_score_list"), (8, 20, False, "k_score_list")])
-def test_which_way_a_list_goes(n_layers, keep, pooled, kernel):
-    """17000 tokens, 8 KV heads, 128 rows: 1064 products a layer.  Few of them, or much to keep, and two products are quicker."""
+@pytest.mark.parametrize("n_layers,keep,room,pooled,kernel", [
+    (31, 100, None, False, "k_score_bound"), (31, 100, None, True, "k_score_list"), (31, 100, 8 * 17000, False, "k_score_bound"),
+    (31, 512, None, False, "k_score_list"), (18, 20, None, False, "k_score_bound"), (18, 400, None, False, "k_score_list"),
+    (8, 20, None, False, "k_score_list")])
+def test_which_way_a_list_goes(n_layers, keep, room, pooled, kernel):
+    """17000 tokens, 8 KV heads, 128 rows: 1064 products a layer.  Few of them, or much to keep, and two products are quicker; room
+    for every row tells nothing of what is kept."""
     w = 32
     x = inputs("gaussian", 1, [17000], 32, 8, 128, w)
-    _, kernels = one_list([x] * n_layers, [17000], w, 7, [[w + keep] * 8] * n_layers, 0, pooled)
+    _, kernels = one_list([x] * n_layers, [17000], w, 7, [[w + keep] * 8] * n_layers, 0, pooled, room)
     assert kernels == {kernel}
 
 

@@ -74,9 +74,9 @@ def test_config5_long_context_split_over_four_ranks():
 
 
 def test_config3_full_layers_through_the_overlapped_entry_point():
-    # the launch configuration bench.py times: layers queued by slkv_compress_overlapped, the score kernel taking
-    # them a list at a time (here 10 layers: a full list of 8, then the rest at the join).  Pooled scores and the
-    # selection of two of the layers against the oracle, every layer against slkv_compress bit for bit.
+    # layers queued by slkv_compress_overlapped with their pooled scores (lists without go with one product:
+    # test_gpu_bound.py), the score kernel taking them a list at a time.  Pooled scores and the selection of two of the
+    # layers against the oracle, every layer against slkv_compress bit for bit.
     from paper_2508_15806_b200 import binding as B
     wl = synth.workloads()[2]
     total = wl.totals[1]
