@@ -34,6 +34,7 @@ WORKLOAD_INDEX = 2          # the 32k-context, 32-layer configuration (third of 
 TOTAL_INDEX = 1             # average budget 512 per KV head
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_per_key_row.txt")
 KERNEL_SOURCES = {"k_score_list": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"],
+                  "k_score_bound": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"],
                   "k_score_fused": ["slkv_score_pipe.cu", "slkv_tc_device.cuh"]}
 
 
@@ -420,7 +421,8 @@ def run_cuda(args):
     q_bytes = len(wl.seq_lens) * w * wl.n_q_heads * d * e
     k_scan = hkv * n_hist * d * e
     rows_avg = sum(L["rows"] for L in layers) / nl
-    alg = {"k_score_fused": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_list": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_lse": k_scan + q_bytes, "k_score_vote": k_scan + q_bytes + 4 * hkv * n_hist,
+    alg = {"k_score_fused": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_list": k_scan + q_bytes + 4 * hkv * n_hist,
+           "k_score_bound": k_scan + q_bytes + 4 * hkv * n_hist, "k_score_lse": k_scan + q_bytes, "k_score_vote": k_scan + q_bytes + 4 * hkv * n_hist,
            "k_pool": 8 * hkv * n_hist, "k_select": 4 * hkv * n_hist + 4 * rows_avg,
            "k_gather": 4 * rows_avg * d * e + 4 * rows_avg, "k_setup": 0,
            "k_layer": k_scan + q_bytes + 4 * rows_avg * d * e}           # a short layer's steps in one launch
@@ -430,12 +432,15 @@ def run_cuda(args):
         kern[name] = {"launches_per_step": cnt / prof_steps, "avg_us": ms * 1e3 / cnt, "share": ms / prof_total}
     top = max(per_kernel, key=lambda n: per_kernel[n][0])
     top_us = kern[top]["avg_us"]
-    # a launch of k_score_list takes a list of layers: its units are those of all its layers
-    layers_per_launch = nl / kern[top]["launches_per_step"] if top == "k_score_list" else 1.0
+    # a launch of k_score_list or k_score_bound takes a list of layers: its units are those of all its layers
+    layers_per_launch = nl / kern[top]["launches_per_step"] if top in ("k_score_list", "k_score_bound") else 1.0
     alg_top = alg[top] * layers_per_launch
     achieved = alg_top / (top_us * 1e-6) / 1e9
     layer_bytes = k_scan + q_bytes + 4 * rows_avg * d * e
-    passes = 1 if args.with_lse else 2                              # row statistics + votes, or votes alone
+    # row statistics + votes, or one product: votes alone, or statistics with estimated votes (k_score_bound; the votes of the heads that
+    # get all of them come on top and are not counted)
+    one_product = "k_score_bound" in per_kernel
+    passes = 1 if args.with_lse or one_product else 2
     flops_layer = passes * 2.0 * wl.n_q_heads * w * n_hist * d
     exps_layer = float(passes) * wl.n_q_heads * w * n_hist
     f_sm = (clocks["sm_mhz"] or 1965.0) * 1e6
@@ -450,15 +455,18 @@ def run_cuda(args):
                           "frac": layer_bytes / (t_layer_us * 1e-6) / 1e9 / peaks["hbm_gbs"],
                           "frac_of_8TBs_nominal": layer_bytes / (t_layer_us * 1e-6) / 8e12},
                 "ceilings": ceilings}
-    # The score kernel's own ceiling is the special-function unit, not HBM: two exponentials per (query row, key)
-    # at 16 ex2.approx per clock per SM need longer than streaming K once.  Reported beside the HBM figures.
+    # The score kernel's own ceiling is the special-function unit, not HBM: an exponential per (query row, key) and pass
+    # at 16 ex2.approx per clock per SM needs longer than streaming K once.  Reported beside the HBM figures.
     if top.startswith("k_score"):
-        n_exp = (exps_layer if top in ("k_score_fused", "k_score_list") else exps_layer / 2) * layers_per_launch
+        n_exp = (exps_layer if top in ("k_score_fused", "k_score_list", "k_score_bound") else exps_layer / 2) * layers_per_launch
         peak_gexp = 148 * 16 * 1965e6 / 1e9
         roofline["alu"] = {"bound": "alu", "unit": "Gexp/s", "achieved": n_exp / (top_us * 1e-6) / 1e9, "peak": peak_gexp,
                            "frac": n_exp / (top_us * 1e-6) / 1e9 / peak_gexp, "exps_per_launch": n_exp,
                            "peak_source": "148 SMs x 16 ex2.approx per clock x 1965 MHz (nominal unit count and maximum clock)"}
-    tr = dram_traffic_per_key_row(top, "lse" if args.with_lse else "two_pass")
+    # with one product the bytes depend on how many heads get all their votes: the captured workload's alone
+    mode = "lse" if args.with_lse else "one_product" if one_product else "two_pass"
+    captured = not one_product or (args.workload or WORKLOAD_INDEX + 1) == WORKLOAD_INDEX + 1
+    tr = dram_traffic_per_key_row(top, mode) if captured else None
     if tr:
         roofline["traffic"] = tr["bytes"] * hkv * n_hist * layers_per_launch
         roofline["traffic_source"] = tr["source"]
@@ -491,7 +499,8 @@ def run_cuda(args):
                "config": {"workload": wl.name, "n_layers": nl, "n_q_heads": wl.n_q_heads, "n_kv_heads": hkv,
                           "head_dim": d, "seq_lens": wl.seq_lens, "window": w, "pool_kernel": wl.pool_kernel,
                           "avg_budget_per_kv_head": total // (nl * hkv), "fixed": wl.fixed,
-                          "row_lse": "supplied by the caller (--with-lse)" if args.with_lse else "computed (two passes over K)",
+                          "row_lse": "supplied by the caller (--with-lse)" if args.with_lse else
+                          "computed (one product with every key, exact votes where they may decide)" if one_product else "computed (two passes over K)",
                           "parallelism":
                           f"dp{world} (one sequence batch per GPU, no collective)",
                           "api": ("slkv_compress_overlapped + slkv_join per step" +

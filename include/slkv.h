@@ -272,6 +272,8 @@ int slkv_compress(const slkv_params* p, const void* q_win, const void* k, const 
  *     captured in a CUDA graph.
  *   - Lists take bf16 and (n_q_heads / n_kv_heads) * window <= 256, at most 64 sequences, segments the one-launch
  *     selections take (up to 262116 history positions with pool_kernel <= 9, up to 131040 with pool_kernel <= 129).  Other shapes run as slkv_compress does, on `stream`, after a join.
+ *   - Long lists with max pooling, without pooled_opt and lse_opt, take one product with every key instead of two where that is quicker, with
+ *     the same results.  out_capacity_rows tells which: as many rows as the budgets make, or room for all, lets the line be drawn best.
  * Arguments, results and error codes otherwise as slkv_compress.
  */
 int slkv_compress_overlapped(const slkv_params* p, const void* q_win, const void* k, const void* v,

@@ -136,12 +136,13 @@ bool list_supported(const Problem& pb) {
 
 // Layers of a list.  A list costs some 23 us beside its layers (pipeline fill and tail, selections and gathers that nothing
 // runs beside), and its layers wait for the last of them to be called: it goes out when it holds about 0.4 ms of work, 32768
-// products of 128 keys x 128 rows in both passes, or eight layers (with log-sum-exps handed in, one pass: half as long).  Steps of 32 layers, us in a row / by themselves from an idle GPU, with 32, 16, 8 and 4
-// layers to a list:
+// products of 128 keys x 128 rows, or eight layers (with two passes over them; with log-sum-exps handed in, one pass, half as long).  Steps
+// of 32 layers, both passes, us in a row / by themselves from an idle GPU, with 32, 16, 8 and 4 layers to a list:
 //   4001 tokens, 128 rows    132 / 197    154 / 191    202 / 228    329 / 348
 //   32768 tokens, 128 rows   734 / 879    756 / 889    804 / 887    946 / 1017
 //   131072 tokens, 256 rows  5175 / 5717  5147 / 5690  5130 / 5697  5101 / 5746
-// At 32768 tokens 32 layers to a list would be 1-3 % quicker than the 16 of the rule, for twice the workspace.
+// At 32768 tokens 32 layers to a list would be 1-3 % quicker than the 16 of the rule, for twice the workspace.  Lists that go with one
+// product (slkv_bound.cu) were not measured at other lengths.
 constexpr int64_t kListProducts = 32768;
 constexpr int kListMinLayers = 8;      // four: eight ragged sequences of 147k tokens, held, 6504 -> 6696 us
 int list_layers(const Problem& pb) {

@@ -2,11 +2,11 @@
 // instead of two.  Max pooling, everything the list score kernel takes, no log-sum-exps handed in.
 //
 // A vote needs its rows' sums over all keys, so a kernel that computes all votes goes over the keys twice.  Few of them decide
-// what is kept.  Here k_score_list (BOUND; slkv_score_pipe.cu, bound_run) adds up the rows' sums as ever and from the same
+// what is kept.  Here k_score_list (kBound; slkv_score_pipe.cu, bound_run) adds up the rows' sums as ever and from the same
 // exponentials, run by run, estimates the keys' votes with the rows' sums over the run's first tiles: est[j] = sum_r w_r 2^s_rj.
 // k_select_bound then knows how far every weight is off.  With rho the largest w_r^-1 / sum_r of the run,
 // vote[j] <= rho * est[j] / G: the keys whose bound is above a threshold get their exact vote, on the tensor cores as in the vote
-// pass and bit for bit the same, the others none.  With T the k-th largest pooled score of what is there, a position whose score is
+// pass and bit for bit the same (kWide's, whose row sums these are), the others none.  With T the k-th largest pooled score of what is there, a position whose score is
 // T or more has it from a key whose vote is T or more; if the threshold is below T, no key without its vote is such a one, so the
 // kept positions are those of all votes, ties included.  If not, every key whose bound is T or more is added, and then it
 // holds: T can only have grown.

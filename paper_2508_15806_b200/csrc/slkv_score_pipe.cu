@@ -24,8 +24,8 @@
 // (the parameters of a list are kilobytes) took 3600 cycles per run and 1000 per tile of the MMA thread.
 //
 // What bounds it and why this shape (one B200, tiles of 128 keys x 128 rows, clock cycles per tile and SM):
-//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; of the votes' one in sixteen goes
-//     to the FMA pipe, and scale / subtract / sum run on packed pairs;
+//   - exponentials: 16384 per tile at 16 per clock on the special-function unit = 1024; one in eight (statistics, but for the
+//     shapes of one product, see TileSum) or sixteen (votes) goes to the FMA pipe, and scale / subtract / sum run on packed pairs;
 //   - shared memory: an MMA with both operands there reads 64 KB per tile at 128 B per clock, the K tile is 32 KB more:
 //     730 measured for loads and MMAs alone;
 //   - two epilogue warpgroups instead of four: 1250; sums over the keys across lanes instead of a lane per row: 1255;
