@@ -561,6 +561,9 @@ bool bound_shape(const Problem& pb) {
 //             in clusters of four, 100000 tokens, 3 (37488): 0.25 363 / 377;  131072 tokens, 4 (65536): 611 / 521;  8 (131072): 0.67 1270 / 1261
 //             eight of 16384 to 32768, 8 (98304): 0.87 2124 / 1820
 //   64 rows   one sequence of 20000 tokens 428 / 446
+// The line lies between the two; shapes differ by some 10 % about it, and a list on the wrong side loses that much.  48 models of 8 to 32 layers with
+// lengths over the range and budgets lognormal or most of them in six heads: 0.58 to 1.04 of the time with two products, 0.87 to 1.07 of that with one
+// wherever the lengths allow it.
 bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers) {
   if (g_list_way != 0) return g_list_way == 1 && bound_possible(pb);
   if (!bound_shape(pb)) return false;
@@ -576,9 +579,13 @@ bool bound_list_supported(const Problem& pb, const TailLayer* tail, int n_layers
   }
   most /= n_layers;
   const double products = (double)pb.n_tiles128 * n_layers * (pb.R > 128 ? 2 : 1);
-  if (pb.R <= 128) return most < 0.99 && products >= 17000 + 16500 * most + (most > 0.78 ? 24000 : 0);
+  auto above = [&](double least, double at0, double slope, double steep) {
+    const double x = at0 + slope * most;
+    return products >= (x > least ? x : least) + (most > steep ? 24000 : 0);
+  };
+  if (pb.R <= 128) return most < 0.99 && above(13000, 6400, 30000, 0.78);
   const double clusters = pb.max_hist < 32764 ? 0.0 : 10000 * (pb.max_hist / 32764.0 - 1.0);        // beyond what one CTA holds
-  return most < 0.96 && products >= 17000 + 24000 * most + (most > 0.85 ? 24000 : 0) + (clusters < 14000 ? clusters : 14000);
+  return most < 0.96 && above(18000, 8500 + (clusters < 16000 ? clusters : 16000), 35000, 0.85);
 }
 
 cudaError_t launch_bound_list(const Problem& pb, const ScoreShape& sh, const ScoreLayer* lay, const TailLayer* tail, int n_layers,
