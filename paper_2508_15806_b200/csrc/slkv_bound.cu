@@ -556,8 +556,8 @@ bool bound_shape(const Problem& pb) {
 //             131072 tokens, 8 (65520): 0.74 856 / 720, even 0.98 774 / 642, 1.00 809 / 867
 //             four of 12000 to 24000, 4 (18016): 0.3 205 / 216;  5 (22520): 0.3 256 / 238, 0.74 277 / 277;  8 (36032): 0.74 435 / 426, 0.83 461 / 468
 //   256 rows  33000 tokens, 5 (20640): 0.35 210 / 207;  7 (28896): 0.35 283 / 268, 0.7 293 / 304;  8 (33024): 0.54 318 / 301, 0.71 328 / 342
-//             in clusters of two, 45000 tokens, 5 (28160): 0.27 281 / 249, 0.74 288 / 294;  60000, 4 (30016): 0.4 295 / 305;  5 (37520): 0.4 361 / 328, 0.7 375 / 404;  48000 tokens, 8 (48000): 0.63 472 / 451,
-//             0.95 510 / 526;  65536 tokens, 8 (65536): 0.81 659 / 650, 0.88 667 / 692
+//             in clusters of two, 45000 tokens, 5 (28160): 0.27 281 / 249;  6 (33792): 0.73 342 / 341;  60000, 4 (30016): 0.4 295 / 305;  5 (37520): 0.4 361 / 328,
+//             0.7 375 / 404;  48000 tokens, 8 (48000): 0.63 472 / 451, 0.95 510 / 526;  65536 tokens, 8 (65536): 0.81 659 / 650, 0.88 667 / 692
 //             in clusters of four, 100000 tokens, 3 (37488): 0.25 363 / 377;  131072 tokens, 4 (65536): 611 / 521;  8 (131072): 0.67 1270 / 1261
 //             eight of 16384 to 32768, 8 (98304): 0.87 2124 / 1820
 //   64 rows   one sequence of 20000 tokens 428 / 446
